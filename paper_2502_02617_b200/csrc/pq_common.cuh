@@ -214,6 +214,19 @@ __device__ inline double polar_quant_block_exact(const double* y, const Tables& 
   return hypot(r3[0], r3[1]);
 }
 
+// Packed float32 arithmetic: one instruction for two IEEE multiply-adds.
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // Host side: remember the CUDA error behind a PQ_ERR_CUDA return (see pq_last_cuda_error).
 void note_cuda_error(cudaError_t e);
 // Test hook (pq_debug_fail_next_wait): returns true once after the hook was armed for `which`
@@ -228,15 +241,15 @@ inline int32_t launch_status() {
 }
 
 // One-time, per-device launch configuration of a kernel that needs more than 48 KB of dynamic shared
-// memory: the attribute belongs to the (kernel, device) pair, so the memo is indexed by the current
-// device. `state` is a zero-initialised array the caller keeps per kernel; an entry holds the device's
+// memory (or, `big_clusters`, clusters of more than 8 blocks): the attribute belongs to the (kernel, device)
+// pair, so the memo is indexed by the current device. `state` is a zero-initialised array the caller keeps per kernel; an entry holds the device's
 // SM count once the kernel is configured there (atomic: host threads may call into the library
 // concurrently; two that race on a device both set the same attribute). Returns the SM count, or 0 with
 // the CUDA error noted.
 constexpr int kMaxDevices = 64;
 using DeviceMemo = std::atomic<int>[kMaxDevices];
 template <typename Kernel>
-inline int configure_for_device(Kernel kernel, int smem_bytes, DeviceMemo& state) {
+inline int configure_for_device(Kernel kernel, int smem_bytes, DeviceMemo& state, bool big_clusters = false) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
@@ -249,6 +262,7 @@ inline int configure_for_device(Kernel kernel, int smem_bytes, DeviceMemo& state
   int n_sm = 0;
   e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e == cudaSuccess && big_clusters) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && n_sm <= 0) e = cudaErrorInvalidDevice;
   if (e != cudaSuccess) {
     note_cuda_error(e);

@@ -74,49 +74,26 @@ __device__ inline float decode_coord(const uint8_t* tb, const Layout& L, int tok
 // ---- workspace -----------------------------------------------------------------------------
 constexpr int kFastMaxGridHost = 160;  // upper bound on the persistent kernel's grid (one CTA per SM)
 
-struct Workspace {
-  float* qrot;       // [B][Hq][d]      rotated queries times scale*log2(e)
-  __half* qrot_h;    // the same rounded to fp16 (tensor-core operand of the fast kernel)
-  __half* qrot_l;    // fp16 residual: qrot - qrot_h
-  int32_t* tickets;  // [B][Hkv]
+struct Workspace {   // of the persistent head_dim-128 kernel; nothing else needs scratch
+  int32_t* tickets;  // [B][Hkv], 8 bytes each: the kernel's tagged tickets
   float* ml;         // [slot][head in group][2]   slot = first slot of the unit + part
   float* o;          // [slot][head in group][d]
-  int n_splits;      // parts per unit of the any-head_dim kernel (the head_dim-128 kernel decides on the device)
-  int n_slots;
   int64_t bytes;
 };
 
-// Token splits per (sequence, kv head) for the any-head_dim kernel.
-__host__ inline int choose_splits(int d, int batch, int n_kv_heads, int max_len) {
-  const int units = batch * n_kv_heads;
-  const int max_blocks = (max_len + kTokenBlock - 1) / kTokenBlock;
-  int splits = (148 * 4 + units - 1) / units;
-  if (splits > max_blocks) splits = max_blocks;
-  if (splits < 1) splits = 1;
-  if (splits > 256) splits = 256;
-  return splits;
-}
-
-__host__ inline Workspace carve_workspace(void* base, int d, int batch, int n_q_heads, int n_kv_heads, int max_len) {
+__host__ inline Workspace carve_workspace(void* base, int d, int batch, int n_q_heads, int n_kv_heads) {
   Workspace w;
-  w.n_splits = choose_splits(d, batch, n_kv_heads, max_len);
   auto align = [](int64_t x) { return (x + 255) & ~(int64_t)255; };
   int64_t off = 0;
   uint8_t* p = reinterpret_cast<uint8_t*>(base);
-  w.qrot = reinterpret_cast<float*>(p + off);
-  off = align(off + (int64_t)batch * n_q_heads * d * 4);
-  w.qrot_h = reinterpret_cast<__half*>(p + off);
-  off = align(off + (int64_t)batch * n_q_heads * d * 2);
-  w.qrot_l = reinterpret_cast<__half*>(p + off);
-  off = align(off + (int64_t)batch * n_q_heads * d * 2);
   w.tickets = reinterpret_cast<int32_t*>(p + off);
-  off = align(off + (int64_t)batch * n_kv_heads * 8);  // 8 bytes per unit (the persistent kernel's tagged tickets)
-  const int g = n_q_heads / n_kv_heads, units = batch * n_kv_heads;
-  w.n_slots = (d == 128 && units <= 2048) ? units + kFastMaxGridHost : units * w.n_splits;
+  off = align(off + (int64_t)batch * n_kv_heads * 8);
+  const int64_t g = n_q_heads / n_kv_heads, units = (int64_t)batch * n_kv_heads;
+  const int64_t n_slots = (d == 128 && units <= 2048) ? units + kFastMaxGridHost : 0;
   w.ml = reinterpret_cast<float*>(p + off);
-  off = align(off + (int64_t)w.n_slots * g * 2 * 4);
+  off = align(off + n_slots * g * 2 * 4);
   w.o = reinterpret_cast<float*>(p + off);
-  off = align(off + (int64_t)w.n_slots * g * d * 4);
+  off = align(off + n_slots * g * d * 4);
   w.bytes = off;
   return w;
 }
@@ -151,27 +128,6 @@ struct DecodeArgs {
     return v > 0 ? v : 0;
   }
 };
-
-// q' = (q . S) * scale * log2(e); also clears the split tickets.
-__global__ void rotate_query_kernel(DecodeArgs a) {
-  extern __shared__ float qs[];
-  const int bh = blockIdx.x, j = threadIdx.x, d = a.d;
-  const int64_t base = (int64_t)bh * d;
-  if (a.io_dtype == PQ_DTYPE_BF16) qs[j] = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[base + j]);
-  else qs[j] = reinterpret_cast<const float*>(a.q)[base + j];
-  __syncthreads();
-  float acc = 0.f;
-#pragma unroll 16
-  for (int k = 0; k < d; ++k) acc = fmaf(qs[k], __ldg(a.S + k * d + j), acc);
-  acc *= a.scale * 1.4426950408889634f;
-  a.ws.qrot[base + j] = acc;
-  const __half qh = __float2half_rn(acc);
-  a.ws.qrot_h[base + j] = qh;
-  a.ws.qrot_l[base + j] = __float2half_rn(acc - __half2float(qh));
-  if (bh < a.batch * a.n_kv_heads && j == 0) a.ws.tickets[bh] = 0;
-}
-
-constexpr int kSimpleThreads = 128;
 
 // Shared memory (floats) that combine_and_store needs.
 __host__ __device__ inline int combine_smem_floats(int g, int d, int n_parts) { return ((2 * g * n_parts + g + 3) & ~3) + g * d; }
@@ -262,157 +218,74 @@ __device__ void combine_and_store(const DecodeArgs& a, int b, int hk, int g, int
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Straightforward float32 kernel: one CTA per (token split, kv head, sequence); per token-block
-// (1) stage the K and V blocks in shared memory, (2) a thread per token decodes the key and
-// forms the scores of the group's query heads, (3) online softmax per head, (4) a thread per
-// coordinate decodes the values and accumulates.  Serves every head_dim and group size.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSimpleThreads) decode_attention_simple_kernel(DecodeArgs a) {
-  extern __shared__ __align__(128) uint8_t smem[];
-  const int d = a.d, g = a.n_q_heads / a.n_kv_heads;
-  const Layout L = make_layout(d, a.pg.page_tokens);
-  const int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  uint8_t* kblk = smem;
-  uint8_t* vblk = smem + L.block_bytes;
-  float* qs = reinterpret_cast<float*>(smem + 2 * L.block_bytes);  // [g][d]
-  float* s_part = qs + g * d;                                      // [2][g][64]
-  float* p_sm = s_part + 2 * g * kTokenBlock;                      // [g][64]
-  float* corr_sm = p_sm + g * kTokenBlock;                         // [g]
-  float* m_run = corr_sm + kMaxGroup;                              // [g]
-  float* l_run = m_run + kMaxGroup;                                // [g]
-  float* cen_cos = l_run + kMaxGroup;                              // [28]
-  float* cen_sin = cen_cos + 32;                                   // [28]
-  __shared__ int is_last;
-
-  for (int i = tid; i < g * d; i += kSimpleThreads) qs[i] = a.ws.qrot[((int64_t)b * a.n_q_heads + hk * g) * d + i];
-  if (tid < PQ_N_CENTROIDS) {
-    cen_cos[tid] = a.tables->cen_cos[tid];
-    cen_sin[tid] = a.tables->cen_sin[tid];
-  }
-  if (tid < g) {
-    m_run[tid] = -CUDART_INF_F;
-    l_run[tid] = 0.f;
-  }
-  float o_acc[kMaxGroup];
-#pragma unroll
-  for (int h = 0; h < kMaxGroup; ++h) o_acc[h] = 0.f;
-
-  const int len = a.visible_len(b);
-  const int nblk_total = len > 0 ? (len + kTokenBlock - 1) / kTokenBlock : 0;
-  const int per = (nblk_total + a.ws.n_splits - 1) / a.ws.n_splits;
-  const int j0 = split * per;
-  const int j1 = min(nblk_total, j0 + per);
-  const int seq = a.seq_of(b);
-  __syncthreads();
-
-  for (int jb = j0; jb < j1; ++jb) {
-    {
-      const uint4* src = reinterpret_cast<const uint4*>(a.cache + kv_block_pair_offset(L, a.pg, a.n_kv_heads, seq, hk, jb, a.status));
-      uint4* dst = reinterpret_cast<uint4*>(smem);
-      for (int i = tid; i < 2 * L.block_bytes / 16; i += kSimpleThreads) dst[i] = src[i];
-    }
-    __syncthreads();
-    {  // scores
-      const int tk = tid & 63, half = tid >> 6;
-      float s[kMaxGroup];
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h) s[h] = 0.f;
-      for (int blk = half; blk < L.nb; blk += 2) {
-        float y[16];
-        decode_block(kblk, L, tk, blk, cen_cos, cen_sin, y);
-#pragma unroll
-        for (int h = 0; h < kMaxGroup; ++h) {
-          if (h < g) {
-            const float* qh = qs + h * d + blk * 16;
-            float acc = s[h];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc = fmaf(qh[i], y[i], acc);
-            s[h] = acc;
-          }
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h)
-        if (h < g) s_part[(half * g + h) * kTokenBlock + tk] = s[h];
-    }
-    __syncthreads();
-    for (int h = warp; h < g; h += kSimpleThreads / 32) {  // online softmax, one warp per head
-      float sv[2], mx = -CUDART_INF_F;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int tk = lane + 32 * t;
-        const bool ok = jb * kTokenBlock + tk < len;
-        sv[t] = ok ? s_part[h * kTokenBlock + tk] + s_part[(g + h) * kTokenBlock + tk] : -CUDART_INF_F;
-        mx = fmaxf(mx, sv[t]);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_old = m_run[h], m_new = fmaxf(m_old, mx);
-      float sum = 0.f;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const float p = sv[t] == -CUDART_INF_F ? 0.f : exp2f(sv[t] - m_new);
-        p_sm[h * kTokenBlock + lane + 32 * t] = p;
-        sum += p;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0) {
-        const float corr = m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
-        corr_sm[h] = corr;
-        m_run[h] = m_new;
-        l_run[h] = l_run[h] * corr + sum;
-      }
-    }
-    __syncthreads();
-    if (tid < d) {  // values
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h)
-        if (h < g) o_acc[h] *= corr_sm[h];
-      const int n_valid = min(kTokenBlock, len - jb * kTokenBlock);  // stale bytes past len may decode to NaN
-      for (int tk = 0; tk < n_valid; ++tk) {
-        const float v = decode_coord(vblk, L, tk, tid, cen_cos, cen_sin);
-#pragma unroll
-        for (int h = 0; h < kMaxGroup; ++h)
-          if (h < g) o_acc[h] = fmaf(p_sm[h * kTokenBlock + tk], v, o_acc[h]);
-      }
-    }
-    __syncthreads();
-  }
-
-  // partials of this split
-  const int slot0 = (b * a.n_kv_heads + hk) * a.ws.n_splits;
-  for (int h = 0; h < g; ++h) {
-    const int64_t idx = (int64_t)(slot0 + split) * g + h;
-    if (tid == 0) {
-      a.ws.ml[2 * idx] = m_run[h];
-      a.ws.ml[2 * idx + 1] = l_run[h];
-    }
-    if (tid < d) a.ws.o[idx * d + tid] = o_acc[h];
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const int t = atomicAdd(a.ws.tickets + b * a.n_kv_heads + hk, 1);
-    is_last = (t == a.ws.n_splits - 1);
-    if (is_last) a.ws.tickets[b * a.n_kv_heads + hk] = 0;  // leave no small counts behind in scratch that other calls reuse
-    if (is_last && len <= 0 && a.lse == nullptr) set_status(a.status, PQ_ERR_EMPTY);
-  }
-  __syncthreads();
-  if (is_last) {
-    __threadfence();
-    combine_and_store(a, b, hk, g, slot0, a.ws.n_splits, reinterpret_cast<float*>(smem));
-  }
-}
-
 }  // namespace pq
 #include "pq_decode_fast.cuh"
 #include "pq_prefill.cuh"
 #include "pq_prefill_tc.cuh"
+#include "pq_split_attention.cuh"
 namespace pq {
+
+// The packed cache for split_attention_kernel: head dims below 128 (and head_dim 128 with more units than the persistent
+// kernel's schedule holds).  A chunk is whole token-blocks, which are contiguous and 16-byte aligned.
+struct PackedSplit {
+  static constexpr bool kEarlyTables = true;
+  SplitCommon c;
+  Layout L;
+  int stage_bytes, n_tab, n_q;
+  const Tables* tables;
+  const uint8_t* cache;
+  const int32_t* lens;
+  Paging pg;
+
+  __device__ __forceinline__ int len(int pair) const {
+    const int b = pair / n_q, v = lens[b] - (n_q - 1 - (pair - b * n_q));
+    return v > 0 ? v : 0;
+  }
+  __device__ __forceinline__ void fill_tables(float2* tab, int tid) const {
+    if (tid < PQ_N_CENTROIDS) tab[tid] = make_float2(tables->cen_cos[tid], tables->cen_sin[tid]);
+  }
+  __device__ __forceinline__ int shift(int, int, int, int) const { return 0; }
+  __device__ __forceinline__ void stage(uint32_t buf, int pair, int hk, int kv, int t0, int n, int tid) const {
+    const int per_block = L.block_bytes >> 4, pieces = ((n + kTokenBlock - 1) / kTokenBlock) * per_block;
+    for (int i = tid; i < pieces; i += kSplitThreads) {
+      const int blk = i / per_block;
+      const int64_t off = kv_block_pair_offset(L, pg, c.n_kv_heads, pair / n_q, hk, t0 / kTokenBlock + blk, c.status);
+      split_cp16(buf + 16 * i, cache + off + (int64_t)kv * L.block_bytes + 16 * (i - blk * per_block));
+    }
+  }
+  // the groups of a token lie side by side in every plane: neighbouring lanes on neighbouring groups read without conflicts
+  __device__ __forceinline__ int lanes_per_token(int ng) const { return ng < 4 ? ng : 4; }
+  __device__ __forceinline__ void decode(uint32_t buf, int t, int grp, uint32_t tab, float* y) const {
+    const uint32_t tb = buf + (t / kTokenBlock) * L.block_bytes;
+    const int tok = t % kTokenBlock;
+    const uint32_t l1 = split_lds32(tb + tok * L.b1 + 4 * grp), l2 = split_lds8(tb + L.o2 + tok * L.b2 + grp);
+    const uint32_t l3 = split_lds8(tb + L.o3 + tok * L.b3 + (grp >> 1)) >> (4 * (grp & 1));
+    const uint32_t l4 = split_lds8(tb + L.o4 + tok * L.b4 + (grp >> 2)) >> (2 * (grp & 3));
+    const float r = __half2float(__ushort_as_half((unsigned short)split_lds16(tb + L.orad + tok * L.br + 2 * grp)));
+    float r3[2], r2[4], r1[8];
+    const float2 e4 = split_lds_f2(tab + (24 + (l4 & 3u)) * 8);
+    r3[0] = r * e4.x;
+    r3[1] = r * e4.y;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float2 e = split_lds_f2(tab + (20 + ((l3 >> (2 * j)) & 3u)) * 8);
+      r2[2 * j] = r3[j] * e.x;
+      r2[2 * j + 1] = r3[j] * e.y;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 e = split_lds_f2(tab + (16 + ((l2 >> (2 * j)) & 3u)) * 8);
+      r1[2 * j] = r2[j] * e.x;
+      r1[2 * j + 1] = r2[j] * e.y;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float2 e = split_lds_f2(tab + ((l1 >> (4 * j)) & 15u) * 8);
+      y[2 * j] = r1[j] * e.x;
+      y[2 * j + 1] = r1[j] * e.y;
+    }
+  }
+};
 
 // ---- partial attentions: merge, and exact attention over an uncompressed window -----------------
 // out = sum_p w_p out_p with w_p = exp(lse_p - lse) and lse = log sum_p exp(lse_p): the attention over the union of
@@ -701,7 +574,7 @@ extern "C" {
 int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t max_len) {
   if (!(head_dim == 16 || head_dim == 32 || head_dim == 64 || head_dim == 128)) return PQ_ERR_UNSUPPORTED;
   if (batch <= 0 || n_q_heads <= 0 || n_kv_heads <= 0 || max_len <= 0 || n_q_heads % n_kv_heads) return PQ_ERR_INVALID_ARG;
-  return pq::carve_workspace(nullptr, head_dim, batch, n_q_heads, n_kv_heads, max_len).bytes;
+  return pq::carve_workspace(nullptr, head_dim, batch, n_q_heads, n_kv_heads).bytes;
 }
 
 static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, const float* S_dev,
@@ -730,7 +603,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.status = status_dev;
   a.lse = lse_dev;
   a.pg = pg;
-  a.ws = pq::carve_workspace(workspace_dev, head_dim, (int)pairs, n_q_heads, n_kv_heads, max_len);
+  a.ws = pq::carve_workspace(workspace_dev, head_dim, (int)pairs, n_q_heads, n_kv_heads);
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
   // Chunks of 32 or more rows (queries x heads of a group), d = 128: the tcgen05 kernel (operands in shared memory,
@@ -840,17 +713,21 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     }
     return pq::launch_status();
   }
-  a.epoch = 0u;
-  a.debug = 0u;
-  pq::rotate_query_kernel<<<(unsigned)pairs * n_q_heads, head_dim, head_dim * sizeof(float), st>>>(a);
-  const pq::Layout L = pq::make_layout(head_dim, pg.page_tokens);
-  size_t smem = 2 * L.block_bytes + sizeof(float) * ((size_t)g * head_dim + 3 * g * pq::kTokenBlock +
-                                                     3 * pq::kMaxGroup + 64);
-  const size_t smem_combine = sizeof(float) * pq::combine_smem_floats(g, head_dim, a.ws.n_splits);
-  if (smem < smem_combine) smem = smem_combine;
-  dim3 grid(a.ws.n_splits, n_kv_heads, (unsigned)pairs);
-  pq::decode_attention_simple_kernel<<<grid, pq::kSimpleThreads, smem, st>>>(a);
-  return pq::launch_status();
+  pq::PackedSplit p;
+  p.c.d = head_dim; p.c.n_q_heads = n_q_heads; p.c.n_kv_heads = n_kv_heads; p.c.io_dtype = io_dtype; p.c.scale = scale;
+  p.c.S = S_dev; p.c.q = q_dev; p.c.out = out_dev; p.c.lse = lse_dev; p.c.status = status_dev;
+  p.L = pq::make_layout(head_dim, pg.page_tokens);
+  p.n_tab = (PQ_N_CENTROIDS + 1) & ~1; p.n_q = n_q; p.tables = a.tables; p.cache = a.cache; p.lens = cache_lens_dev; p.pg = pg;
+  p.c.chunk = 512;   // two tokens per thread
+  p.stage_bytes = p.c.chunk / pq::kTokenBlock * p.L.block_bytes;
+  const int kh = g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : 8;
+  const int smem = pq::split_smem_bytes(head_dim, kh, p.n_tab, p.c.chunk, p.stage_bytes);
+  switch (kh) {
+    case 1: return pq::launch_split_attention<pq::PackedSplit, 1>(p, pairs, max_len, smem, st);
+    case 2: return pq::launch_split_attention<pq::PackedSplit, 2>(p, pairs, max_len, smem, st);
+    case 4: return pq::launch_split_attention<pq::PackedSplit, 4>(p, pairs, max_len, smem, st);
+    default: return pq::launch_split_attention<pq::PackedSplit, 8>(p, pairs, max_len, smem, st);
+  }
 }
 
 int32_t pq_decode_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, const float* S_dev,

@@ -1,7 +1,7 @@
 // KV-cache encoder (Algorithm 1 lines 2 and 4 with fixed codebooks) and the append step.
 #include <math_constants.h>
 
-#include "pq_common.cuh"
+#include "pq_general_common.cuh"
 
 namespace pq {
 
@@ -94,92 +94,6 @@ __device__ inline void store_block(uint8_t* tb_base, const Layout& L, int tok, i
   if (L.nb < 2 || (blk & 1) == 0) tb_base[L.o3 + tok * L.b3 + (blk >> 1)] = (uint8_t)l3;
   if (L.nb < 4 || (blk & 3) == 0) tb_base[L.o4 + tok * L.b4 + (blk >> 2)] = (uint8_t)l4;
   reinterpret_cast<__half*>(tb_base + L.orad + tok * L.br)[blk] = radius;
-}
-
-// ------------------------------------------------------------------------------------------
-// Reference-precision encoder: everything in float64.  One CTA of 128 threads handles
-// 16 * (128 / d) vectors: thread (group, j) forms coordinate j of y = x . S for the 16 vectors
-// of its group, then every thread quantises one 16-coordinate block.
-// A "vector" is (row, kv, head): index v = (row * 2 + kv) * n_kv_heads + head.
-// ------------------------------------------------------------------------------------------
-constexpr int kExactThreads = 128;
-constexpr int kExactVecPerGroup = 16;
-
-__global__ void __launch_bounds__(kExactThreads) encode_exact_kernel(EncodeArgs a) {
-  extern __shared__ double smem_d[];
-  const int d = a.head_dim;
-  const int groups = kExactThreads / d;
-  const int vec_per_cta = kExactVecPerGroup * groups;
-  double* xs = smem_d;                     // [vec_per_cta][d]
-  double* ys = smem_d + vec_per_cta * d;   // [vec_per_cta][d]
-  const int64_t n_vec = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
-  const int64_t v0 = (int64_t)blockIdx.x * vec_per_cta;
-  const int tid = threadIdx.x;
-  const Layout L = make_layout(d, a.pg.page_tokens);
-
-  int bad = 0;
-  for (int i = tid; i < vec_per_cta * d; i += kExactThreads) {
-    const int64_t v = v0 + i / d;
-    double x = 0.0;
-    if (v < n_vec) {
-      const int head = (int)(v % a.n_kv_heads);
-      const int kv = (int)((v / a.n_kv_heads) & 1);
-      const int64_t row = v / (2 * a.n_kv_heads);
-      const float f = load_elem(kv ? a.V : a.K, a.in_dtype, row * a.token_stride + head * a.head_stride + (i % d));
-      if (!isfinite(f)) ++bad;
-      x = (double)f;
-    }
-    xs[i] = x;
-  }
-  if (bad) {
-    atomicAdd(a.status + 1, bad);
-    set_status(a.status, PQ_ERR_NONFINITE);
-  }
-  __syncthreads();
-
-  {
-    const int grp = tid / d, j = tid % d;
-    double acc[kExactVecPerGroup];
-#pragma unroll
-    for (int i = 0; i < kExactVecPerGroup; ++i) acc[i] = 0.0;
-    const double* xg = xs + grp * kExactVecPerGroup * d;
-    for (int k = 0; k < d; ++k) {
-      const double s = (double)a.S[k * d + j];
-#pragma unroll
-      for (int i = 0; i < kExactVecPerGroup; ++i) acc[i] = fma(xg[i * d + k], s, acc[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < kExactVecPerGroup; ++i) ys[(grp * kExactVecPerGroup + i) * d + j] = acc[i];
-  }
-  __syncthreads();
-
-  {
-    const int nb = L.nb;
-    const int lv = tid / nb, blk = tid % nb;  // local vector, block
-    const int64_t v = v0 + lv;
-    bool valid = v < n_vec;
-    BlockCodes c = {0, 0, 0, 0};
-    double radius = 0.0;
-    int seq = 0, pos = -1, head = 0, kv = 0;
-    if (valid) {
-      head = (int)(v % a.n_kv_heads);
-      kv = (int)((v / a.n_kv_heads) & 1);
-      row_destination(a, (int)(v / (2 * a.n_kv_heads)), &seq, &pos);
-      valid = pos >= 0;
-    }
-    if (valid) {
-      double y[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) y[i] = ys[lv * d + blk * 16 + i];
-      radius = polar_quant_block_exact(y, *a.tables, c);
-      if (radius > 65504.0) {
-        radius = 65504.0;
-        atomicAdd(a.status + 2, 1);
-      }
-    }
-    uint8_t* tb_base = a.cache + (valid ? block_offset(L, a.pg, a.n_kv_heads, seq, head, kv, pos) : 0);
-    store_block(tb_base, L, valid ? pos % kTokenBlock : 0, blk, c, __double2half(radius), valid);
-  }
 }
 
 }  // namespace pq
@@ -577,13 +491,13 @@ static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
     encode_ffma_kernel<<<grid, kFfmaThreads, kFfmaSmem, stream>>>(a);
     return launch_advance_lens(a, lens, stream);
   }
-  const int groups = kExactThreads / a.head_dim;
-  const int vec_per_cta = kExactVecPerGroup * groups;
-  const int64_t n_vec = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
-  const int64_t grid = (n_vec + vec_per_cta - 1) / vec_per_cta;
-  const size_t smem = (size_t)2 * vec_per_cta * a.head_dim * sizeof(double);
-  encode_exact_kernel<<<(unsigned)grid, kExactThreads, smem, stream>>>(a);
-  return launch_advance_lens(a, lens, stream);
+  GenEncodeArgs ga;
+  ga.K = a.K; ga.V = a.V; ga.in_dtype = a.in_dtype; ga.token_stride = a.token_stride; ga.head_stride = a.head_stride;
+  ga.cu_seqlens = a.cu_seqlens; ga.batch = a.batch; ga.total_tokens = a.total_tokens; ga.n_kv_heads = a.n_kv_heads;
+  ga.capacity = a.capacity; ga.S = a.S; ga.boundaries = a.tables->bnd; ga.cache = a.cache; ga.lens = a.cache_lens;
+  ga.status = a.status; ga.pg = a.pg;
+  const int32_t st = launch_packed_encode(ga, a.head_dim, stream);
+  return st == PQ_OK ? launch_advance_lens(a, lens, stream) : st;
 }
 
 }  // namespace pq

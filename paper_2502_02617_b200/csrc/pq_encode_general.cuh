@@ -1,0 +1,557 @@
+// Encoder for any head_dim <= 256, recursion depth and bits per level, and for the packed cache at head dims below 128
+// (included by pq_general.cu): float32 rotation and float32 decisions with certified margins, float64
+// for what a margin does not cover, so the codes are those of a float64 evaluation of Algorithm 1.
+//
+// A thread block takes a tile of vectors (consecutive rows of one head, K or V):
+//   * y = x S on the FMA pipe: thread = kVT vectors x 8 columns, S in slices of 32 rows through shared memory.  The sum
+//     over k is formed per slice and the slices are added, so |y - y_exact| <= (32 + d / 32) 2^-24 sum_k |x_k||S_kj|,
+//     which is at most that factor times ||x||_2 (Cauchy-Schwarz; the columns of an orthogonal S have unit norm).
+//   * quantise: thread = (vector, group of 16 coordinates), the four lowest levels in registers.  A code is found by
+//     binary search over the level's boundary lines: psi > beta iff r_b cos(beta) - r_a sin(beta) > 0 (with the
+//     half-plane bookkeeping of level 1), which needs no arc tangent.  The search tests both neighbours of the cell it
+//     ends in, so the smallest |r_b cos - r_a sin| it met bounds the distance to the next boundary.
+//   * levels 5 and up: a thread per vector on the groups' norms.
+//   * a (vector, group) with any decision inside its margin, or a block radius that close to a rounding boundary of
+//     fp16, is taken again by a warp in float64 from the inputs; the same for the upper levels of a vector.
+// Margins: moving every coordinate by at most dy moves the norm of n of them by at most sqrt(n) dy, so a test on the
+// radii of n-coordinate halves moves by at most sqrt(2 n) dy; 1.1 x that, plus 1e-6 (r_a + r_b) for the float32
+// roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
+// A radius is certified by kRadiusSlack: its float32 error is that of a norm, whose coordinate errors average out
+// (2e-8 of the norm on synthetic rows), plus the sum of squares and the square root, at most 5e-7 together.
+#pragma once
+#include <math_constants.h>
+
+#include "pq_general_common.cuh"
+
+namespace pq {
+
+constexpr int kGeThreads = 256;
+constexpr int kGeSlice = 32;              // rows of S per slice
+constexpr float kRadiusSlack = 2e-6f;
+
+struct GeShape {
+  int dc, ng, vecs, x_stride, row_words, floats_xy;
+};
+// dc: columns of the tile (head dims below 16 are padded); x rows are dc + 4 floats apart, the 16-coordinate groups of
+// a y row 20 floats (conflict-free 16-byte reads in both cases).
+__host__ __device__ inline GeShape ge_shape(int d, int row_bytes, int vt) {
+  GeShape s;
+  s.dc = d < 16 ? 16 : d;
+  s.ng = s.dc / 16;
+  s.vecs = kGeThreads / (s.dc / 8) * vt;
+  s.x_stride = s.dc + 4;
+  s.row_words = ((row_bytes + 3) / 4) | 1;
+  const int fx = s.vecs * s.x_stride, fy = s.vecs * s.ng * 20;
+  s.floats_xy = fx > fy ? fx : fy;
+  return s;
+}
+__host__ inline int ge_smem_bytes(const GeShape& s, int n_bnd) {
+  return 4 * (s.floats_xy + kGeSlice * s.dc + s.vecs * s.row_words + s.vecs * s.ng + 2 * s.vecs + 2 * ((n_bnd + 1) & ~1)) +
+         8 * s.vecs + 8 * s.vecs * s.ng + 4 * s.vecs * s.ng + 2 * s.vecs + 64;
+}
+
+__device__ __forceinline__ float ge_load(const void* base, int dtype, int64_t i) {
+  return dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[i])
+                                : reinterpret_cast<const float*>(base)[i];
+}
+// OR `value` (at most 32 bits) into a row at bit `bit`.
+__device__ __forceinline__ void ge_put(uint32_t* row, int bit, uint32_t value) {
+  const int sh = bit & 31;
+  atomicOr(row + (bit >> 5), value << sh);
+  const uint32_t hi = sh ? value >> (32 - sh) : 0u;
+  if (hi) atomicOr(row + (bit >> 5) + 1, hi);
+}
+// Would r round to another fp16 value if it moved by kRadiusSlack?  (NaN and infinite r: yes.)
+__device__ __forceinline__ bool ge_radius_unsure(float r) {
+  const float lo = fminf(r * (1.f - kRadiusSlack), 65504.f), hi = fminf(r * (1.f + kRadiusSlack), 65504.f);
+  return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(lo)) != __half_as_ushort(__float2half_rn(hi)) ||
+         (r > 65000.f);   // saturation is counted from the exact value
+}
+__device__ __forceinline__ float ge_sqrt(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Code of (a, b) at one level: `tab` = (cos, sin) of the level's boundaries, 2^bits - 1 of them; level 1 (kFirst): the first
+// n_upper lie in [0, pi].  `near` becomes the smallest distance met.
+template <bool kFirst>
+__device__ __forceinline__ uint32_t ge_search(float a, float b, const float2* tab, int bits, int n_upper, float& near) {
+  uint32_t pos = 0;
+  const bool neg = kFirst && b < 0.f;
+  near = kFirst ? fabsf(b) : CUDART_INF_F;
+  for (int s = bits - 1; s >= 0; --s) {
+    const int k = (int)pos + (1 << s) - 1;
+    const float2 cs = tab[k];
+    const float cross = fmaf(b, cs.x, -a * cs.y);
+    near = fminf(near, fabsf(cross));
+    bool above = cross > 0.f;
+    if (kFirst) above = k < n_upper ? (neg || above) : (neg && above);
+    pos += above ? 1u << s : 0u;
+  }
+  return pos;
+}
+
+// The exact code of the pair (a, b) at level l (0-based).
+__device__ __forceinline__ uint32_t ge_exact_code(double a, double b, const GenConfig& g, int l, const double* boundaries) {
+  double psi = atan2(b, a);
+  if (l == 0 && psi < 0.0) psi += 6.283185307179586476925286766559;
+  const double* bnd = boundaries + g.bnd_off[l];
+  uint32_t code = 0;
+  for (int k = 0; k < (1 << g.bits[l]) - 1; ++k) code += psi > __ldg(bnd + k);
+  return code;
+}
+
+// One warp: coordinate 16 grp + (lane & 15) of x S in float64 (each half-warp sums half of the terms, in four chains: a
+// float64 multiply-add has several times the latency of a float32 one).
+__device__ __forceinline__ double ge_exact_coord(const GenEncodeArgs& a, const void* xbase, int64_t xoff, int grp, int lane) {
+  const int d = a.g.d, col = 16 * grp + (lane & 15), half = d >> 1, k0 = (lane >> 4) * half;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  if (col < d) {
+    const float* s = a.S + (int64_t)k0 * d + col;
+    const int n4 = half & ~3;
+#pragma unroll 2
+    for (int k = 0; k < n4; k += 4)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        acc[i] = fma((double)ge_load(xbase, a.in_dtype, xoff + k0 + k + i), (double)__ldg(s + (int64_t)(k + i) * d), acc[i]);
+    for (int k = n4; k < half; ++k) acc[0] = fma((double)ge_load(xbase, a.in_dtype, xoff + k0 + k), (double)__ldg(s + (int64_t)k * d), acc[0]);
+  }
+  const double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  return sum + __shfl_xor_sync(0xffffffffu, sum, 16);
+}
+
+// kVT: vectors per thread in the product (4; 1 for few rows).  kSub: levels inside a group, min(L, 4).
+template <int kVT, int kSub>
+__global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_constant__ GenEncodeArgs a) {
+  extern __shared__ __align__(16) uint8_t ge_smem[];
+  const GenConfig& g = a.g;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = g.d, L = g.L;
+  const GeShape s = ge_shape(d, g.row_bytes, kVT);
+  const int V = s.vecs, ng = s.ng, dc = s.dc;
+  float* xy = reinterpret_cast<float*>(ge_smem);                        // x [V][x_stride], then y [V][ng * 20]
+  float* Ss = xy + s.floats_xy;                                         // [kGeSlice][dc]
+  uint32_t* rows = reinterpret_cast<uint32_t*>(Ss + kGeSlice * dc);     // [V][row_words]
+  float* gsum = reinterpret_cast<float*>(rows + V * s.row_words);       // [V][ng] squared norms of the groups
+  float* dy_sm = gsum + V * ng;                                         // [V] bound on the error of a coordinate
+  float2* tab = reinterpret_cast<float2*>(dy_sm + 2 * V);               // boundaries
+  const int n_bnd = g.n_cen - L;
+  int64_t* dest = reinterpret_cast<int64_t*>(tab + ((n_bnd + 1) & ~1)); // [V] where the row goes (-1: nowhere)
+  double* norm_up = reinterpret_cast<double*>(dest + V);                // [V * ng] exact norms of groups, where needed
+  uint16_t* list = reinterpret_cast<uint16_t*>(norm_up + V * ng);       // [V * ng] (vector, group) pairs to take again
+  uint16_t* norms = list + V * ng;                                      // [V * ng] (vector, group) pairs of which the norm is needed
+  uint16_t* list_up = norms + V * ng;                                   // [V] vectors whose upper levels are taken again
+  __shared__ int n_list, n_norms, n_list_up, n_upper;
+  const int head = blockIdx.y, kv = blockIdx.z, row0 = blockIdx.x * V;
+  const void* xbase = kv ? a.V : a.K;
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid == 0) n_list = n_norms = n_list_up = n_upper = 0;
+  for (int i = tid; i < V * s.row_words; i += kGeThreads) rows[i] = 0u;
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the inputs may come from the kernel before this one
+  for (int i = tid; i < n_bnd; i += kGeThreads) {
+    const double beta = a.boundaries[i];
+    tab[i] = cos_sin_table(beta);
+    if (i < (1 << g.bits[0]) - 1 && beta <= 3.14159265358979323846) atomicAdd(&n_upper, 1);
+  }
+
+  // ---- destinations and inputs
+  for (int v = tid; v < V; v += kGeThreads) {
+    const int row = row0 + v;
+    int64_t off = -1;
+    if (row < a.total_tokens) {
+      int b = row, first = row, count = 1;
+      if (a.cu_seqlens != nullptr) {   // the sequence that owns the row: largest b with cu[b] <= row
+        int lo = 0, hi = a.batch - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (a.cu_seqlens[mid] <= row) lo = mid; else hi = mid - 1;
+        }
+        b = lo; first = a.cu_seqlens[lo]; count = a.cu_seqlens[lo + 1] - first;
+      }
+      const int start = a.lens[b];
+      if (start < 0 || start + count > a.capacity) {
+        set_status(a.status, PQ_ERR_CAPACITY);
+      } else {
+        const int pos = start + (row - first);
+        if (a.packed) {
+          const Layout P = make_layout(d, a.pg.page_tokens);
+          off = block_offset(P, a.pg, a.n_kv_heads, b, head, kv, pos);
+          if (off < 0) set_status(a.status, PQ_ERR_INVALID_ARG);   // a page outside the pool
+          else off = off * kTokenBlock + pos % kTokenBlock;        // token-block and token in one number
+        } else {
+          off = ((((int64_t)b * a.n_kv_heads + head) * 2 + kv) * a.capacity + pos) * g.row_bytes;
+        }
+      }
+    }
+    dest[v] = off;
+  }
+  const bool vec8 = a.in_dtype == PQ_DTYPE_BF16 && d >= 16 && ((a.token_stride | a.head_stride) & 7) == 0 &&
+                    ((uintptr_t)xbase & 15) == 0;
+  int bad = 0;
+  if (vec8) {
+    const int per_row = d / 8;
+    for (int i = tid; i < V * per_row; i += kGeThreads) {
+      const int v = i / per_row, p = i - v * per_row, row = row0 + v;
+      uint4 w = make_uint4(0u, 0u, 0u, 0u);
+      if (row < a.total_tokens)
+        w = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(xbase) + (int64_t)row * a.token_stride +
+                                                 (int64_t)head * a.head_stride + 8 * p));
+      const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+      float f[8];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        f[2 * e] = __uint_as_float(u[e] << 16);
+        f[2 * e + 1] = __uint_as_float(u[e] & 0xFFFF0000u);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) bad += !(fabsf(f[e]) < CUDART_INF_F);
+      float4* dst = reinterpret_cast<float4*>(xy + v * s.x_stride + 8 * p);
+      dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+      dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+  } else {
+    for (int i = tid; i < V * dc; i += kGeThreads) {
+      const int v = i / dc, k = i - v * dc, row = row0 + v;
+      float f = 0.f;
+      if (row < a.total_tokens && k < d)
+        f = ge_load(xbase, a.in_dtype, (int64_t)row * a.token_stride + (int64_t)head * a.head_stride + k);
+      bad += !(fabsf(f) < CUDART_INF_F);
+      xy[v * s.x_stride + k] = f;
+    }
+  }
+  if (bad) {
+    atomicAdd(a.status + 1, bad);
+    set_status(a.status, PQ_ERR_NONFINITE);
+  }
+
+  // ---- y = x S: thread = kVT vectors x 8 columns (four packed pairs)
+  const int tx = tid % (dc / 8), ty = tid / (dc / 8);
+  float tot[kVT][8];
+#pragma unroll
+  for (int v = 0; v < kVT; ++v)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) tot[v][j] = 0.f;
+  for (int k0 = 0; k0 < dc; k0 += kGeSlice) {
+    const int nk = min(kGeSlice, dc - k0);
+    __syncthreads();
+    if (d >= 16) {
+      const float4* src = reinterpret_cast<const float4*>(a.S + (int64_t)k0 * d);
+      float4* dst = reinterpret_cast<float4*>(Ss);
+      if (((uintptr_t)a.S & 15) == 0) {
+        for (int i = tid; i < nk * dc / 4; i += kGeThreads) dst[i] = __ldg(src + i);
+      } else {
+        for (int i = tid; i < nk * dc; i += kGeThreads) Ss[i] = __ldg(a.S + (int64_t)k0 * d + i);
+      }
+    } else {
+      for (int i = tid; i < nk * dc; i += kGeThreads) {
+        const int k = k0 + i / dc, j = i % dc;
+        Ss[i] = k < d && j < d ? __ldg(a.S + k * d + j) : 0.f;
+      }
+    }
+    __syncthreads();
+    uint64_t acc[kVT][4];
+#pragma unroll
+    for (int v = 0; v < kVT; ++v)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[v][j] = 0ull;
+#pragma unroll 2
+    for (int k = 0; k < nk; k += 4) {
+      float4 xv[kVT];
+#pragma unroll
+      for (int v = 0; v < kVT; ++v) xv[v] = *reinterpret_cast<const float4*>(xy + (ty * kVT + v) * s.x_stride + k0 + k);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const ulonglong2 sa = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx);
+        const ulonglong2 sb = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx + 4);
+#pragma unroll
+        for (int v = 0; v < kVT; ++v) {
+          const float xk = kk == 0 ? xv[v].x : kk == 1 ? xv[v].y : kk == 2 ? xv[v].z : xv[v].w;
+          const uint64_t xx = f2_pack(xk, xk);
+          acc[v][0] = f2_fma(xx, sa.x, acc[v][0]);
+          acc[v][1] = f2_fma(xx, sa.y, acc[v][1]);
+          acc[v][2] = f2_fma(xx, sb.x, acc[v][2]);
+          acc[v][3] = f2_fma(xx, sb.y, acc[v][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kVT; ++v)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float lo, hi;
+        f2_unpack(acc[v][j], lo, hi);
+        tot[v][2 * j] += lo;
+        tot[v][2 * j + 1] += hi;
+      }
+  }
+  __syncthreads();   // x has been used: y takes its place
+#pragma unroll
+  for (int v = 0; v < kVT; ++v) {
+    float* dst = xy + ((ty * kVT + v) * ng + (tx >> 1)) * 20 + 8 * (tx & 1);
+    *reinterpret_cast<float4*>(dst) = make_float4(tot[v][0], tot[v][1], tot[v][2], tot[v][3]);
+    *reinterpret_cast<float4*>(dst + 4) = make_float4(tot[v][4], tot[v][5], tot[v][6], tot[v][7]);
+  }
+  __syncthreads();
+  for (int i = tid; i < V * ng; i += kGeThreads) {   // squared norms of the groups
+    const float4* src = reinterpret_cast<const float4*>(xy + i * 20);
+    float q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 w = src[j];
+      q[j] = fmaf(w.x, w.x, w.y * w.y) + fmaf(w.z, w.z, w.w * w.w);
+    }
+    gsum[i] = (q[0] + q[1]) + (q[2] + q[3]);
+  }
+  __syncthreads();
+  const float rot_err = 1.1f * (float)(kGeSlice + dc / kGeSlice) * 5.9604644775390625e-08f;
+  for (int v = tid; v < V; v += kGeThreads) {
+    float t = 0.f;
+    for (int i = 0; i < ng; ++i) t += gsum[v * ng + i];
+    dy_sm[v] = rot_err * 1.0001f * sqrtf(t);
+  }
+  __syncthreads();
+
+  // ---- the levels inside a group of 16 coordinates
+  for (int i = tid; i < V * ng; i += kGeThreads) {
+    const int v = i / ng, grp = i - v * ng;
+    if (dest[v] < 0) continue;
+    const float dy = dy_sm[v];
+    float r[16];
+    const float4* src = reinterpret_cast<const float4*>(xy + i * 20);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 w = src[j];
+      r[4 * j] = w.x; r[4 * j + 1] = w.y; r[4 * j + 2] = w.z; r[4 * j + 3] = w.w;
+    }
+    bool sure = true;
+    uint32_t lo[kSub], hi[kSub];   // the level's codes in the group: the first half of them in lo, the second in hi
+    float s2[8];                   // squared radii of the level
+#pragma unroll
+    for (int l = 0; l < kSub; ++l) {
+      const int n = 8 >> l, b = g.bits[l];
+      const float m_dy = 1.1f * (l == 0 ? 1.41421356f : l == 1 ? 2.f : l == 2 ? 2.82842712f : 4.f) * dy;
+      lo[l] = hi[l] = 0u;
+#pragma unroll
+      for (int j = 0; j < n; ++j) {
+        const float p = r[2 * j], q = r[2 * j + 1];
+        float near;
+        const uint32_t code = l == 0 ? ge_search<true>(p, q, tab, b, n_upper, near) : ge_search<false>(p, q, tab + g.bnd_off[l], b, 0, near);
+        if (l == 0 && 16 * grp + 2 * j >= d) near = CUDART_INF_F;   // padding of a head_dim below 16
+        if (l > 0 && 16 * grp + (j << (l + 1)) >= d) near = CUDART_INF_F;
+        sure = sure && near > fmaf(1e-6f, fabsf(p) + fabsf(q), m_dy);
+        if (n == 1 || j < n / 2) lo[l] |= code << (j * b);
+        else hi[l] |= code << ((j - n / 2) * b);
+        s2[j] = l == 0 ? fmaf(p, p, q * q) : s2[2 * j] + s2[2 * j + 1];
+      }
+      // radii of the next level (in place: r[j] is read before r[j] of the next level is needed)
+#pragma unroll
+      for (int j = 0; j < n; ++j) r[j] = ge_sqrt(s2[j]);
+    }
+    const int n_blk = 16 >> kSub;
+    uint32_t rad[n_blk];
+    if (L == kSub) {
+#pragma unroll
+      for (int j = 0; j < n_blk; ++j) {
+        if (grp * n_blk + j < g.nb) sure = sure && !ge_radius_unsure(r[j]);
+        rad[j] = __half_as_ushort(__float2half_rn(r[j]));
+      }
+    }
+    if (!sure) {
+      list[atomicAdd(&n_list, 1)] = (uint16_t)i;
+      continue;
+    }
+    uint32_t* row = rows + v * s.row_words;
+#pragma unroll
+    for (int l = 0; l < kSub; ++l) {
+      const int n = 8 >> l, b = g.bits[l], bit = g.byte_off[l] * 8 + grp * n * b;
+      if (16 * grp >= d) continue;
+      ge_put(row, bit, lo[l]);
+      if (n > 1) ge_put(row, bit + (n / 2) * b, hi[l]);
+    }
+    if (L == kSub) {
+#pragma unroll
+      for (int j = 0; j < n_blk; ++j)
+        if (grp * n_blk + j < g.nb) ge_put(row, g.rad_off * 8 + 16 * (grp * n_blk + j), rad[j]);
+    }
+  }
+  // ---- levels above the groups: a thread per vector, the squared norms halved in place
+  if (L > 4) {
+    __syncthreads();
+    for (int v = tid; v < V; v += kGeThreads) {
+      if (dest[v] < 0) continue;
+      float* q2 = gsum + v * ng;
+      uint32_t* row = rows + v * s.row_words;
+      bool sure = true;
+      const float dy = dy_sm[v];
+      for (int l = 4; l < L; ++l) {
+        const int n = d >> (l + 1), b = g.bits[l];
+        const float m_dy = 1.1f * ge_sqrt((float)(2 << l)) * dy;
+        uint32_t word = 0u;
+        int fill = 0, bit = g.byte_off[l] * 8;
+        for (int j = 0; j < n; ++j) {
+          const float sa = q2[2 * j], sb = q2[2 * j + 1], p = ge_sqrt(sa), q = ge_sqrt(sb);
+          float near;
+          const uint32_t code = ge_search<false>(p, q, tab + g.bnd_off[l], b, 0, near);
+          sure = sure && near > fmaf(1e-6f, p + q, m_dy);
+          word |= code << fill;
+          fill += b;
+          if (fill > 24 || j + 1 == n) {
+            ge_put(row, bit, word);
+            bit += fill;
+            word = 0u;
+            fill = 0;
+          }
+          q2[j] = sa + sb;
+        }
+      }
+      for (int j = 0; j < g.nb; ++j) {
+        const float r = ge_sqrt(q2[j]);
+        sure = sure && !ge_radius_unsure(r);
+        ge_put(row, g.rad_off * 8 + 16 * j, __half_as_ushort(__float2half_rn(r)));
+      }
+      if (!sure) {
+        list_up[atomicAdd(&n_list_up, 1)] = (uint16_t)v;
+        const int at = atomicAdd(&n_norms, ng);
+        for (int i = 0; i < ng; ++i) norms[at + i] = (uint16_t)(v * ng + i);
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- float64 for what the margins do not cover: a warp per (vector, group)
+  for (int e = warp; e < n_list; e += kGeThreads / 32) {
+    const int i = list[e], v = i / ng, grp = i - v * ng;
+    const int64_t xoff = (int64_t)(row0 + v) * a.token_stride + (int64_t)head * a.head_stride;
+    double y = ge_exact_coord(a, xbase, xoff, grp, lane);   // of coordinate 16 grp + (lane & 15)
+    uint32_t* row = rows + v * s.row_words;
+#pragma unroll
+    for (int l = 0; l < kSub; ++l) {
+      const int n = 8 >> l;
+      const double p = __shfl_sync(0xffffffffu, y, (2 * lane) & 31), q = __shfl_sync(0xffffffffu, y, (2 * lane + 1) & 31);
+      if (lane < n && 16 * grp + (lane << (l + 1)) < d)
+        ge_put(row, g.byte_off[l] * 8 + (grp * n + lane) * g.bits[l], ge_exact_code(p, q, g, l, a.boundaries));
+      y = sqrt(p * p + q * q);
+    }
+    const int n_blk = 16 >> kSub;
+    if (L == kSub && lane < n_blk && grp * n_blk + lane < g.nb) {
+      double r = y;
+      if (r > 65504.0) {
+        r = 65504.0;
+        atomicAdd(a.status + 2, 1);
+      }
+      ge_put(row, g.rad_off * 8 + 16 * (grp * n_blk + lane), __half_as_ushort(__double2half(r)));
+    }
+    if (lane == 0) atomicAdd(a.status + 3, 1);
+  }
+  if (L > 4) {
+    // the norms of all groups of the vectors whose upper levels are taken again, then those levels, a warp per vector
+    for (int e = warp; e < n_norms; e += kGeThreads / 32) {
+      const int i = norms[e], v = i / ng;
+      double y = ge_exact_coord(a, xbase, (int64_t)(row0 + v) * a.token_stride + (int64_t)head * a.head_stride, i - v * ng, lane);
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {   // radius of a pair, of four coordinates, ... as the recursion forms them
+        const double p = __shfl_sync(0xffffffffu, y, (2 * lane) & 31), q = __shfl_sync(0xffffffffu, y, (2 * lane + 1) & 31);
+        y = sqrt(p * p + q * q);
+      }
+      if (lane == 0) norm_up[i] = y;
+    }
+    __syncthreads();
+    for (int e = warp; e < n_list_up; e += kGeThreads / 32) {
+      const int v = list_up[e];
+      uint32_t* row = rows + v * s.row_words;
+      double mine = lane < ng ? norm_up[v * ng + lane] : 0.0;
+      for (int t = g.byte_off[4] + lane; t < g.row_bytes; t += 32)   // take the float32 codes and radii out
+        atomicAnd(row + (t >> 2), ~(0xFFu << (8 * (t & 3))));
+      __syncwarp();
+      for (int l = 4; l < L; ++l) {
+        const int n = d >> (l + 1);
+        const double p = __shfl_sync(0xffffffffu, mine, (2 * lane) & 31), q = __shfl_sync(0xffffffffu, mine, (2 * lane + 1) & 31);
+        if (lane < n) ge_put(row, g.byte_off[l] * 8 + lane * g.bits[l], ge_exact_code(p, q, g, l, a.boundaries));
+        mine = sqrt(p * p + q * q);
+      }
+      if (lane < g.nb) {
+        double r = mine;
+        if (r > 65504.0) {
+          r = 65504.0;
+          atomicAdd(a.status + 2, 1);
+        }
+        ge_put(row, g.rad_off * 8 + 16 * lane, __half_as_ushort(__double2half(r)));
+      }
+      if (lane == 0) atomicAdd(a.status + 3, 1);
+    }
+  }
+  __syncthreads();
+
+  // ---- rows out
+  if (a.packed) {
+    const Layout P = make_layout(d, a.pg.page_tokens);
+    for (int i = tid; i < V * g.row_bytes; i += kGeThreads) {
+      const int v = i / g.row_bytes, t = i - v * g.row_bytes;
+      const int64_t at = dest[v];
+      if (at < 0) continue;
+      uint8_t* tb = a.cache + at / kTokenBlock;
+      const int tok = (int)(at % kTokenBlock);
+      const uint8_t byte = reinterpret_cast<const uint8_t*>(rows + v * s.row_words)[t];
+      if (t < P.b1) tb[tok * P.b1 + t] = byte;
+      else if (t < P.b1 + P.b2) tb[P.o2 + tok * P.b2 + t - P.b1] = byte;
+      else if (t < P.b1 + P.b2 + P.b3) tb[P.o3 + tok * P.b3 + t - P.b1 - P.b2] = byte;
+      else if (t < P.b1 + P.b2 + P.b3 + P.b4) tb[P.o4 + tok * P.b4 + t - P.b1 - P.b2 - P.b3] = byte;
+      else if (t >= g.rad_off) tb[P.orad + tok * P.br + t - g.rad_off] = byte;
+    }
+  } else if ((g.row_bytes & 3) == 0 && ((uintptr_t)a.cache & 3) == 0) {
+    const int per = g.row_bytes >> 2;
+    for (int i = tid; i < V * per; i += kGeThreads) {
+      const int v = i / per, t = i - v * per;
+      if (dest[v] >= 0) reinterpret_cast<uint32_t*>(a.cache + dest[v])[t] = rows[v * s.row_words + t];
+    }
+  } else {
+    const int per = g.row_bytes >> 1;
+    for (int i = tid; i < V * per; i += kGeThreads) {
+      const int v = i / per, t = i - v * per;
+      if (dest[v] >= 0)
+        reinterpret_cast<uint16_t*>(a.cache + dest[v])[t] = reinterpret_cast<const uint16_t*>(rows + v * s.row_words)[t];
+    }
+  }
+}
+
+template <int kVT, int kSub>
+static int32_t launch_gen_encode_as(const GenEncodeArgs& a, cudaStream_t stream) {
+  const GeShape s = ge_shape(a.g.d, a.g.row_bytes, kVT);
+  static DeviceMemo configured;
+  auto kernel = gen_encode_kernel<kVT, kSub>;
+  if (configure_for_device(kernel, 113 * 1024, configured) == 0) return PQ_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.total_tokens + s.vecs - 1) / s.vecs, a.n_kv_heads, 2);
+  cfg.blockDim = dim3(kGeThreads);
+  cfg.dynamicSmemBytes = ge_smem_bytes(s, a.g.n_cen - a.g.L);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];   // set up while the kernel before it in the stream finishes (it waits inside)
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+  if (e != cudaSuccess) {
+    note_cuda_error(e);
+    cudaGetLastError();
+    return PQ_ERR_CUDA;
+  }
+  return PQ_OK;
+}
+
+// One vector per thread in the product instead of four as long as that many blocks fit on the device at once: a short
+// chunk then spreads over four times as many SMs.
+static int32_t launch_gen_encode(const GenEncodeArgs& a, cudaStream_t stream) {
+  const GeShape s1 = ge_shape(a.g.d, a.g.row_bytes, 1);
+  const bool few = (int64_t)((a.total_tokens + s1.vecs - 1) / s1.vecs) * 2 * a.n_kv_heads <= 2 * 148;
+  switch (a.g.L < 4 ? a.g.L : 4) {
+    case 1: return few ? launch_gen_encode_as<1, 1>(a, stream) : launch_gen_encode_as<4, 1>(a, stream);
+    case 2: return few ? launch_gen_encode_as<1, 2>(a, stream) : launch_gen_encode_as<4, 2>(a, stream);
+    case 3: return few ? launch_gen_encode_as<1, 3>(a, stream) : launch_gen_encode_as<4, 3>(a, stream);
+    default: return few ? launch_gen_encode_as<1, 4>(a, stream) : launch_gen_encode_as<4, 4>(a, stream);
+  }
+}
+
+}  // namespace pq

@@ -1,32 +1,17 @@
 // General recursion depth and bit tables (Definition 1 and Algorithm 1 with any L <= log2 d levels and any bits per
-// level; Section 4 counts b_FPN + (d - 1) b bits per vector for L = log2 d and b bits everywhere).  Plain kernels:
-// float64 for the encoder (the codes are those of a float64 evaluation of Algorithm 1), float32 for attention; one
-// thread block per vector, or per (sequence, kv head).  The tuned path of the other files is the L = 4, bits (4,2,2,2)
-// case in its own layout; this one covers what the paper describes beyond it, at reference speed.
+// level; Section 4 counts b_FPN + (d - 1) b bits per vector for L = log2 d and b bits everywhere).  The encoder decides
+// in float32 with certified margins and takes the rest in float64 (pq_encode_general.cuh), attention is float32
+// throughout (pq_split_attention.cuh).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <math_constants.h>
 #include <vector>
 
-#include "pq_common.cuh"
+#include "pq_encode_general.cuh"
+#include "pq_split_attention.cuh"
 
 namespace pq {
-
-constexpr int kGenMaxLevels = PQ_GENERAL_MAX_LEVELS;
-constexpr int kGenMaxBits = 6;
-constexpr int kGenMaxDim = 256;
-constexpr int kGenMaxCentroids = kGenMaxLevels << kGenMaxBits;
-
-// A validated configuration with the derived sizes.  A row (one token of one head, K or V) holds, per level, the
-// level's d / 2^l codes as one bit stream (code i at bits [i b, (i + 1) b), least significant first, padded to a
-// byte), then padding to an even offset, then the d / 2^L block radii in fp16.  The cache is
-// [sequence][kv head][K | V][token][row_bytes].
-struct GenConfig {
-  int d, L, nb, n_codes, n_cen, row_bytes, rad_off;
-  int bits[kGenMaxLevels], cen_off[kGenMaxLevels], bnd_off[kGenMaxLevels], code_off[kGenMaxLevels], byte_off[kGenMaxLevels],
-      level_bytes[kGenMaxLevels];
-};
 
 static int32_t make_gen_config(const pq_general_config* c, GenConfig* g) {
   if (c == nullptr) return PQ_ERR_INVALID_ARG;
@@ -73,104 +58,8 @@ __device__ __forceinline__ float gen_decode_coord(const uint8_t* row, const GenC
   return v;
 }
 
-struct GenEncodeArgs {
-  GenConfig g;
-  const void* K;
-  const void* V;
-  int in_dtype;
-  int64_t token_stride, head_stride;
-  const int32_t* cu_seqlens;
-  int batch, total_tokens, n_kv_heads, capacity;
-  const float* S;
-  const double* boundaries;
-  uint8_t* cache;
-  const int32_t* lens;
-  int32_t* status;
-};
-
-// One thread block of max(d, 32) threads per vector (row, K | V, head): y = x . S in float64, the polar tree level by
-// level (thread j forms angle j of the level), codes = number of boundaries below the angle, then the bit streams.
-__global__ void gen_encode_kernel(GenEncodeArgs a) {
-  __shared__ double ra[kGenMaxDim], rb[kGenMaxDim];
-  __shared__ uint8_t codes[kGenMaxDim];
-  __shared__ int dest[2];
-  const GenConfig& g = a.g;
-  const int j = threadIdx.x, d = g.d;
-  const int64_t v = blockIdx.x;
-  const int head = (int)(v % a.n_kv_heads), kv = (int)((v / a.n_kv_heads) & 1);
-  const int row = (int)(v / (2 * a.n_kv_heads));
-  if (j == 0) {   // destination: the sequence that owns the row (largest b with cu[b] <= row) and its position
-    int lo = 0, hi = a.batch - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.cu_seqlens[mid] <= row) lo = mid; else hi = mid - 1;
-    }
-    const int first = a.cu_seqlens[lo], count = a.cu_seqlens[lo + 1] - first, start = a.lens[lo];
-    dest[0] = lo;
-    dest[1] = (start < 0 || start + count > a.capacity) ? -1 : start + (row - first);
-    if (dest[1] < 0) set_status(a.status, PQ_ERR_CAPACITY);
-  }
-  if (j < d) {
-    const int64_t idx = (int64_t)row * a.token_stride + (int64_t)head * a.head_stride + j;
-    const float x = a.in_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(kv ? a.V : a.K)[idx])
-                                                : reinterpret_cast<const float*>(kv ? a.V : a.K)[idx];
-    if (!isfinite(x)) {
-      atomicAdd(a.status + 1, 1);
-      set_status(a.status, PQ_ERR_NONFINITE);
-    }
-    ra[j] = (double)x;
-  }
-  __syncthreads();
-  if (j < d) {
-    double acc = 0.0;
-    for (int k = 0; k < d; ++k) acc = fma(ra[k], (double)__ldg(a.S + (int64_t)k * d + j), acc);
-    rb[j] = acc;
-  }
-  __syncthreads();
-  double* src = rb;
-  double* dst = ra;
-  for (int l = 0; l < g.L; ++l) {
-    const int n = d >> (l + 1);
-    if (j < n) {
-      const double x0 = src[2 * j], x1 = src[2 * j + 1];
-      double psi = atan2(x1, x0);
-      if (l == 0 && psi < 0.0) psi += 6.283185307179586476925286766559;
-      const double* bnd = a.boundaries + g.bnd_off[l];
-      int code = 0;
-      for (int k = 0; k < (1 << g.bits[l]) - 1; ++k) code += psi > bnd[k];
-      codes[g.code_off[l] + j] = (uint8_t)code;
-      dst[j] = sqrt(x0 * x0 + x1 * x1);
-    }
-    __syncthreads();
-    double* t = src; src = dst; dst = t;
-  }
-  const int pos = dest[1];
-  if (pos < 0) return;
-  uint8_t* out = a.cache + gen_row_offset(g, a.n_kv_heads, a.capacity, dest[0], head, kv, pos);
-  for (int t = j; t < g.rad_off; t += blockDim.x) {   // byte t of the row: gather its bits
-    int l = g.L - 1;
-    while (l > 0 && t < g.byte_off[l]) --l;
-    uint32_t byte = 0;
-    if (t < g.byte_off[l] + g.level_bytes[l]) {
-      const int b = g.bits[l], n = d >> (l + 1);
-      for (int bit = 0; bit < 8; ++bit) {
-        const int pos_bit = (t - g.byte_off[l]) * 8 + bit, idx = pos_bit / b;
-        if (idx < n) byte |= (((uint32_t)codes[g.code_off[l] + idx] >> (pos_bit % b)) & 1u) << bit;
-      }
-    }
-    out[t] = (uint8_t)byte;
-  }
-  if (j < g.nb) {
-    double r = src[j];
-    if (r > 65504.0) {
-      r = 65504.0;
-      atomicAdd(a.status + 2, 1);
-    }
-    reinterpret_cast<__half*>(out + g.rad_off)[j] = __double2half(r);
-  }
-}
-
 __global__ void gen_advance_lens_kernel(const int32_t* cu_seqlens, int batch, int capacity, int32_t* lens) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched ahead of time: the encoder reads the lengths
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= batch) return;
   const int count = cu_seqlens[b + 1] - cu_seqlens[b], start = lens[b];
@@ -196,8 +85,9 @@ __global__ void gen_dequant_kernel(GenConfig g, int n_kv_heads, const float* S, 
   __shared__ float cc[kGenMaxCentroids], cs[kGenMaxCentroids], ys[kGenMaxDim];
   const int j = threadIdx.x, d = g.d;
   for (int i = j; i < g.n_cen; i += blockDim.x) {
-    cc[i] = (float)cos(centroids[i]);
-    cs[i] = (float)sin(centroids[i]);
+    const float2 e = cos_sin_table(centroids[i]);
+    cc[i] = e.x;
+    cs[i] = e.y;
   }
   __syncthreads();
   const int64_t v = blockIdx.x;
@@ -213,131 +103,115 @@ __global__ void gen_dequant_kernel(GenConfig g, int n_kv_heads, const float* S, 
   }
 }
 
-struct GenAttnArgs {
+// General rows for split_attention_kernel.  Rows are only 2-byte aligned, so a chunk is copied as the 16-byte pieces that
+// lie inside it, to the same position modulo 16 in the buffer, and two ragged ends in 2-byte steps.
+// kSub = min(L, 4): the levels inside a group of 16 coordinates (the angles above it are walked one by one).
+template <int kSub>
+struct GenSplit {
+  static constexpr bool kEarlyTables = false;
+  SplitCommon c;
   GenConfig g;
-  int n_q_heads, n_kv_heads, capacity, io_dtype;
-  float scale;
-  const float* S;
+  int stage_bytes, n_tab, capacity;
   const double* centroids;
-  const void* q;
   const uint8_t* cache;
   const int32_t* lens;
-  void* out;
-  int32_t* status;
+
+  __device__ __forceinline__ int len(int pair) const { return max(0, min(lens[pair], capacity)); }
+  __device__ __forceinline__ void fill_tables(float2* tab, int tid) const {
+    for (int i = tid; i < g.n_cen; i += kSplitThreads) tab[i] = cos_sin_table(centroids[i]);
+  }
+  __device__ __forceinline__ int64_t row_offset(int pair, int hk, int kv, int t) const {
+    return gen_row_offset(g, c.n_kv_heads, capacity, pair, hk, kv, t);
+  }
+  __device__ __forceinline__ int shift(int pair, int hk, int kv, int t0) const {
+    return (int)((reinterpret_cast<uintptr_t>(cache) + row_offset(pair, hk, kv, t0)) & 15);
+  }
+  __device__ __forceinline__ void stage(uint32_t buf, int pair, int hk, int kv, int t0, int n, int tid) const {
+    const uint8_t* src = cache + row_offset(pair, hk, kv, t0);
+    const int bytes = n * g.row_bytes, sh = (int)(reinterpret_cast<uintptr_t>(src) & 15);
+    const int head = min(bytes, (16 - sh) & 15), pieces = (bytes - head) >> 4, tail = head + 16 * pieces;
+    const uint32_t dst = buf + sh;
+    for (int i = tid; i < pieces; i += kSplitThreads) split_cp16(dst + head + 16 * i, src + head + 16 * i);
+    const int ends = (head + bytes - tail) >> 1;   // at most 14
+    if (tid < ends) {
+      const int at = 2 * tid < head ? 2 * tid : tail + 2 * tid - head;
+      asm volatile("st.shared.u16 [%0], %1;" ::"r"(dst + at), "h"(*reinterpret_cast<const uint16_t*>(src + at)) : "memory");
+    }
+  }
+  __device__ __forceinline__ int lanes_per_token(int) const { return 1; }
+  // 32 bits of a row from bit `bit` on
+  __device__ __forceinline__ static uint32_t window(uint32_t row, int bit) {
+    const uint32_t at = row + (bit >> 3), al = at & ~3u;
+    return __funnelshift_r(split_lds32(al), split_lds32(al + 4), ((at & 3u) << 3) + (bit & 7));
+  }
+  __device__ __forceinline__ void decode(uint32_t buf, int t, int grp, uint32_t tab, float* y) const {
+    const uint32_t row = buf + t * g.row_bytes;
+    constexpr int kBlk = 16 >> kSub;   // blocks whose radius (or subtree root) starts inside the group
+    float v[16];
+    if (kSub == 4) {
+      float r = __half2float(__ushort_as_half((unsigned short)split_lds16(row + g.rad_off + 2 * (grp >> (g.L - 4)))));
+      for (int l = g.L - 1; l >= 4; --l) {   // the angles above the group
+        const int b = g.bits[l];
+        const uint32_t code = window(row, g.byte_off[l] * 8 + (grp >> (l - 3)) * b) & ((1u << b) - 1u);
+        const float2 cs = split_lds_f2(tab + (g.cen_off[l] + code) * 8);
+        r *= (grp >> (l - 4)) & 1 ? cs.y : cs.x;
+      }
+      v[0] = r;
+    } else {
+#pragma unroll
+      for (int j = 0; j < kBlk; ++j) {
+        const int blk = grp * kBlk + j;
+        v[j] = blk < g.nb ? __half2float(__ushort_as_half((unsigned short)split_lds16(row + g.rad_off + 2 * blk))) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int l = kSub - 1; l >= 0; --l) {
+      const int n = 8 >> l, b = g.bits[l], bit = g.byte_off[l] * 8 + grp * n * b;   // n angles of the level in the group
+      const uint32_t mask = (1u << b) - 1u, entry = tab + g.cen_off[l] * 8;
+      uint32_t w = window(row, bit), w2 = 0u;
+      if (n == 8) w2 = b <= 4 ? w >> (4 * b) : window(row, bit + 4 * b);   // 8 codes of up to 6 bits
+#pragma unroll
+      for (int j = n - 1; j >= 0; --j) {
+        const uint32_t code = ((j < 4 ? w : w2) >> ((j & 3) * b)) & mask;
+        const float2 cs = split_lds_f2(entry + code * 8);
+        const float r = v[j];
+        v[2 * j] = r * cs.x;
+        v[2 * j + 1] = r * cs.y;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) y[i] = v[i];
+  }
 };
 
-// Eq. 3, one thread block of 256 threads per (kv head, sequence): q' = q S once, then chunks of 256 tokens: a thread
-// per token decodes the key coordinate by coordinate and forms the scores of the group's heads, a warp per head keeps
-// the running maximum and denominator, a thread per coordinate decodes the values and accumulates P . V; the
-// result is normalised and rotated back by S^T.
-constexpr int kGenAttnThreads = 256;
-__global__ void __launch_bounds__(kGenAttnThreads) gen_attention_kernel(GenAttnArgs a) {
-  extern __shared__ float gsm[];
-  const GenConfig& g = a.g;
-  const int d = g.d, grp = a.n_q_heads / a.n_kv_heads, hk = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  float* cc = gsm;                          // [n_cen]
-  float* cs = cc + g.n_cen;                 // [n_cen]
-  float* qs = cs + g.n_cen;                 // [grp][d]  q' = q S * scale * log2(e); later the normalised output
-  float* sc = qs + grp * d;                 // [grp][kGenAttnThreads]
-  float* m_sm = sc + grp * kGenAttnThreads; // [grp]
-  float* l_sm = m_sm + kMaxGroup;
-  float* corr_sm = l_sm + kMaxGroup;
-  float* qin = corr_sm + kMaxGroup;         // [grp][d] the queries as given
-  for (int i = tid; i < g.n_cen; i += kGenAttnThreads) {
-    cc[i] = (float)cos(a.centroids[i]);
-    cs[i] = (float)sin(a.centroids[i]);
+template <int kSub>
+static int32_t launch_gen_attention(const GenConfig& g, SplitCommon c, int batch, int capacity, const double* centroids,
+                                    const void* cache, const int32_t* lens, cudaStream_t stream) {
+  GenSplit<kSub> p;
+  p.g = g; p.capacity = capacity; p.centroids = centroids; p.cache = reinterpret_cast<const uint8_t*>(cache); p.lens = lens;
+  p.n_tab = (g.n_cen + 1) & ~1;
+  const int grp = c.n_q_heads / c.n_kv_heads, kh = grp <= 1 ? 1 : grp <= 2 ? 2 : grp <= 4 ? 4 : 8;
+  // chunk: two tokens per thread, as long as two staging buffers stay within 64 KB
+  int chunk = 512;
+  while (chunk > 64 && chunk * g.row_bytes > 32 * 1024) chunk >>= 1;
+  c.chunk = chunk;
+  p.c = c;
+  p.stage_bytes = (chunk * g.row_bytes + 16 + 8 + 15) & ~15;   // + the shift, + what a window reads past the last row
+  const int smem = split_smem_bytes(g.d, kh, p.n_tab, chunk, p.stage_bytes);
+  switch (kh) {
+    case 1: return launch_split_attention<GenSplit<kSub>, 1>(p, batch, capacity, smem, stream);
+    case 2: return launch_split_attention<GenSplit<kSub>, 2>(p, batch, capacity, smem, stream);
+    case 4: return launch_split_attention<GenSplit<kSub>, 4>(p, batch, capacity, smem, stream);
+    default: return launch_split_attention<GenSplit<kSub>, 8>(p, batch, capacity, smem, stream);
   }
-  const int64_t q0 = ((int64_t)b * a.n_q_heads + hk * grp) * d;
-  for (int i = tid; i < grp * d; i += kGenAttnThreads)
-    qin[i] = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[q0 + i])
-                                         : reinterpret_cast<const float*>(a.q)[q0 + i];
-  if (tid < grp) {
-    m_sm[tid] = -CUDART_INF_F;
-    l_sm[tid] = 0.f;
-  }
-  __syncthreads();
-  for (int i = tid; i < grp * d; i += kGenAttnThreads) {
-    const int h = i / d, jj = i - h * d;
-    float acc = 0.f;
-    for (int k = 0; k < d; ++k) acc = fmaf(qin[h * d + k], __ldg(a.S + (int64_t)k * d + jj), acc);
-    qs[i] = acc * a.scale * 1.4426950408889634f;
-  }
-  int len = a.lens[b];
-  len = len < 0 ? 0 : (len > a.capacity ? a.capacity : len);
-  float acc[kMaxGroup];
-#pragma unroll
-  for (int h = 0; h < kMaxGroup; ++h) acc[h] = 0.f;
-  __syncthreads();
-  const uint8_t* kbase = a.cache + gen_row_offset(g, a.n_kv_heads, a.capacity, b, hk, 0, 0);
-  const uint8_t* vbase = a.cache + gen_row_offset(g, a.n_kv_heads, a.capacity, b, hk, 1, 0);
-  for (int c0 = 0; c0 < len; c0 += kGenAttnThreads) {
-    const int n = min(kGenAttnThreads, len - c0);
-    if (tid < n) {
-      const uint8_t* row = kbase + (int64_t)(c0 + tid) * g.row_bytes;
-      float s[kMaxGroup];
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h) s[h] = 0.f;
-      for (int i = 0; i < d; ++i) {
-        const float kvv = gen_decode_coord(row, g, i, cc, cs);
-#pragma unroll
-        for (int h = 0; h < kMaxGroup; ++h)
-          if (h < grp) s[h] = fmaf(qs[h * d + i], kvv, s[h]);
-      }
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h)
-        if (h < grp) sc[h * kGenAttnThreads + tid] = s[h];
-    }
-    __syncthreads();
-    for (int h = warp; h < grp; h += kGenAttnThreads / 32) {
-      float mx = -CUDART_INF_F;
-      for (int t = lane; t < n; t += 32) mx = fmaxf(mx, sc[h * kGenAttnThreads + t]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_new = fmaxf(m_sm[h], mx);
-      float sum = 0.f;
-      for (int t = lane; t < n; t += 32) {
-        const float p = exp2f(sc[h * kGenAttnThreads + t] - m_new);
-        sc[h * kGenAttnThreads + t] = p;
-        sum += p;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0) {
-        const float corr = exp2f(m_sm[h] - m_new);
-        corr_sm[h] = corr;
-        l_sm[h] = l_sm[h] * corr + sum;
-        m_sm[h] = m_new;
-      }
-    }
-    __syncthreads();
-    if (tid < d) {
-#pragma unroll
-      for (int h = 0; h < kMaxGroup; ++h)
-        if (h < grp) acc[h] *= corr_sm[h];
-      for (int t = 0; t < n; ++t) {
-        const float vv = gen_decode_coord(vbase + (int64_t)(c0 + t) * g.row_bytes, g, tid, cc, cs);
-#pragma unroll
-        for (int h = 0; h < kMaxGroup; ++h)
-          if (h < grp) acc[h] = fmaf(sc[h * kGenAttnThreads + t], vv, acc[h]);
-      }
-    }
-    __syncthreads();
-  }
-  if (tid < d) {
-#pragma unroll
-    for (int h = 0; h < kMaxGroup; ++h)
-      if (h < grp) qs[h * d + tid] = len > 0 ? acc[h] / l_sm[h] : 0.f;
-  }
-  if (tid == 0 && len <= 0) set_status(a.status, PQ_ERR_EMPTY);
-  __syncthreads();
-  for (int i = tid; i < grp * d; i += kGenAttnThreads) {   // x_hat_j = sum_k y_hat_k S[j][k]
-    const int h = i / d, jj = i - h * d;
-    float o = 0.f;
-    for (int k = 0; k < d; ++k) o = fmaf(qs[h * d + k], __ldg(a.S + (int64_t)jj * d + k), o);
-    if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[q0 + i] = __float2bfloat16(o);
-    else reinterpret_cast<float*>(a.out)[q0 + i] = o;
-  }
+}
+
+int32_t launch_packed_encode(GenEncodeArgs a, int head_dim, cudaStream_t stream) {
+  pq_general_config cfg = {head_dim, 4, {4, 2, 2, 2}};
+  const int32_t st = make_gen_config(&cfg, &a.g);
+  if (st != PQ_OK) return st;
+  a.packed = 1;
+  return launch_gen_encode(a, stream);
 }
 
 }  // namespace pq
@@ -434,10 +308,27 @@ int32_t pq_general_encode_kv(const pq_general_config* cfg, int32_t n_kv_heads, c
   a.cu_seqlens = cu_seqlens_dev; a.batch = batch; a.total_tokens = total_tokens; a.n_kv_heads = n_kv_heads; a.capacity = capacity;
   a.S = S_dev; a.boundaries = boundaries_dev; a.cache = reinterpret_cast<uint8_t*>(cache_dev); a.lens = cache_lens_dev;
   a.status = status_dev;
+  a.packed = 0;
+  a.pg = pq::contiguous_paging(capacity, batch);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const unsigned n_vec = (unsigned)((int64_t)total_tokens * 2 * n_kv_heads);
-  pq::gen_encode_kernel<<<n_vec, a.g.d < 32 ? 32 : a.g.d, 0, s>>>(a);
-  pq::gen_advance_lens_kernel<<<(batch + 127) / 128, 128, 0, s>>>(cu_seqlens_dev, batch, capacity, cache_lens_dev);
+  const int32_t launched = pq::launch_gen_encode(a, s);
+  if (launched != PQ_OK) return launched;
+  // the length update as a programmatic dependent launch of the encode kernel (its launch latency is hidden)
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((batch + 127) / 128);
+  lc.blockDim = dim3(128);
+  lc.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&lc, pq::gen_advance_lens_kernel, cu_seqlens_dev, (int)batch, (int)capacity, cache_lens_dev);
+  if (e != cudaSuccess) {
+    pq::note_cuda_error(e);
+    cudaGetLastError();
+    return PQ_ERR_CUDA;
+  }
   return pq::launch_status();
 }
 
@@ -445,26 +336,24 @@ int32_t pq_general_decode_attention(const pq_general_config* cfg, int32_t n_q_he
                                     const double* centroids_dev, const void* q_dev, int32_t io_dtype, const void* cache_dev,
                                     const int32_t* cache_lens_dev, int32_t batch, int32_t capacity, float scale,
                                     void* out_dev, int32_t* status_dev, void* stream) {
-  pq::GenAttnArgs a;
-  const int32_t st = pq::make_gen_config(cfg, &a.g);
+  pq::GenConfig g;
+  const int32_t st = pq::make_gen_config(cfg, &g);
   if (st != PQ_OK) return st;
   if (!S_dev || !centroids_dev || !q_dev || !cache_dev || !cache_lens_dev || !out_dev || !status_dev) return PQ_ERR_INVALID_ARG;
   if (batch <= 0 || batch > 65535 || n_q_heads <= 0 || n_kv_heads <= 0 || capacity <= 0 || n_q_heads % n_kv_heads) return PQ_ERR_INVALID_ARG;
   if (n_q_heads / n_kv_heads > pq::kMaxGroup) return PQ_ERR_UNSUPPORTED;
   if (io_dtype != PQ_DTYPE_F32 && io_dtype != PQ_DTYPE_BF16) return PQ_ERR_UNSUPPORTED;
-  if ((uintptr_t)centroids_dev & 7) return PQ_ERR_ALIGNMENT;
-  a.n_q_heads = n_q_heads; a.n_kv_heads = n_kv_heads; a.capacity = capacity; a.io_dtype = io_dtype; a.scale = scale;
-  a.S = S_dev; a.centroids = centroids_dev; a.q = q_dev; a.cache = reinterpret_cast<const uint8_t*>(cache_dev);
-  a.lens = cache_lens_dev; a.out = out_dev; a.status = status_dev;
-  const int grp = n_q_heads / n_kv_heads;
-  const size_t smem = sizeof(float) * ((size_t)2 * a.g.n_cen + (size_t)2 * grp * a.g.d + (size_t)grp * pq::kGenAttnThreads +
-                                      3 * pq::kMaxGroup);
-  static pq::DeviceMemo configured;
-  if (pq::configure_for_device(pq::gen_attention_kernel, 64 * 1024, configured) == 0) return PQ_ERR_CUDA;
-  if (smem > 64 * 1024) return PQ_ERR_UNSUPPORTED;
-  dim3 grid(n_kv_heads, batch);
-  pq::gen_attention_kernel<<<grid, pq::kGenAttnThreads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
-  return pq::launch_status();
+  if (((uintptr_t)centroids_dev & 7) || ((uintptr_t)cache_dev & 1)) return PQ_ERR_ALIGNMENT;
+  pq::SplitCommon c;
+  c.d = g.d; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.chunk = 0; c.scale = scale;
+  c.S = S_dev; c.q = q_dev; c.out = out_dev; c.lse = nullptr; c.status = status_dev;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  switch (g.L < 4 ? g.L : 4) {
+    case 1: return pq::launch_gen_attention<1>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
+    case 2: return pq::launch_gen_attention<2>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
+    case 3: return pq::launch_gen_attention<3>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
+    default: return pq::launch_gen_attention<4>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
+  }
 }
 
 int32_t pq_general_unpack_codes(const pq_general_config* cfg, int32_t n_kv_heads, const void* cache_dev, int32_t batch,
