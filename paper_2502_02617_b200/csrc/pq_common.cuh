@@ -34,6 +34,15 @@ __host__ __device__ constexpr int bnd_off(int level) { return level == 1 ? 0 : 1
 constexpr int kL1Cells = 128;            // cells per octant of the level-1 decision table
 constexpr float kL1CellScale = 127.93f;  // cell = floor(t * kL1CellScale + 1/16): t = 1 still falls in the last cell
 
+// Constants of the float32 quantiser (pq_encode_fast.cuh), one word each.
+struct QuantLines {
+  float t2[3][3];            // tan^2 of the three boundaries of levels 2, 3, 4
+  float ua[3][3], ub[3][3];  // their lines scaled to max(|A|, |B|) = 1: D_k = A_k sa + B_k sb
+  uint32_t sym;              // the boundaries of every level >= 2 are b, pi/4, pi/2 - b (kFlagSymmetricUpper)
+  uint32_t analytic;         // sym and the uniform level-1 codebook: every decision is a sign test
+  uint32_t unused;
+};
+
 // Compiled form of the codebooks (built on the host by pq_build_tables, copied verbatim to
 // the device by the caller).
 struct Tables {
@@ -64,7 +73,7 @@ struct Tables {
   //                          so that a half2 of the two pairs' multipliers multiplies element-wise
   uint2 t1p_hi[256];
   uint2 t1p_lo[256];
-  uint32_t reserved[30];
+  QuantLines lines;
   // Level-1 decision table for any codebook (see quant_level1_table_push): octant o = (b < 0) << 2 | (a < 0) << 1 |
   // (|b| > |a|), cell = position of t = min(|a|,|b|) / max(|a|,|b|) in [0, 1].  .x = float bits of tau, the
   // one boundary value of t the cell decides against (NaN: the cell cannot be decided by one comparison);
@@ -213,6 +222,9 @@ __device__ inline double polar_quant_block_exact(const double* y, const Tables& 
   c.l4 = quant_upper_exact(r3[0], r3[1], 4, tb);
   return hypot(r3[0], r3[1]);
 }
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
 // Packed float32 arithmetic: one instruction for two IEEE multiply-adds.
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {

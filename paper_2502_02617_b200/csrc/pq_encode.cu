@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(kFfmaThreads) encode_ffma_kernel(EncodeArgs a)
     atomicAdd(a.status + 1, bad);
     set_status(a.status, PQ_ERR_NONFINITE);
   }
+  if (tid < 32) load_fast_quant(a.tables, fq, tid, &a.tables->l1_cells[0][0]);
   if (tid == 0) {
-    load_fast_quant(a.tables, fq);
     fixq->count[0] = fixq->count[1] = fixq->count[2] = fixq->count[3] = 0;
   }
   __syncthreads();
@@ -273,99 +273,8 @@ __global__ void __launch_bounds__(kFfmaThreads) encode_ffma_kernel(EncodeArgs a)
   fix_rounds(a, fixq, leftbits, xoff, tb, tok, 4 * half, kv, tid, kFfmaThreads, 1);
 }
 
-// ------------------------------------------------------------------------------------------
-// Few vectors (append, short chunks), head_dim 128: one CTA of 128 threads per vector.  Thread j
-// forms y_j in float32; eight threads quantise one block each with the certified sign tests; if
-// any decision of the vector is ambiguous the CTA forms y again in float64 and those blocks are
-// decided exactly.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) encode_vector_kernel(EncodeArgs a) {
-  // a programmatic dependent of the kernel before it (which may have produced the vectors, or still reads the lengths):
-  // nothing of the stream is read before the wait; the length update after this grid may be set up at once
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  __shared__ float xs[128];
-  __shared__ float ys[128];
-  __shared__ double yd[128];
-  __shared__ float red[4];
-  __shared__ uint32_t amb_blocks;   // bit b: block b has a decision that float32 cannot certify
-  __shared__ FastQuant fq;
-  const int j = threadIdx.x;
-  const int64_t v = blockIdx.x;  // vector index: (row * 2 + kv) * n_kv_heads + head
-  const int head = (int)(v % a.n_kv_heads), kv = (int)((v / a.n_kv_heads) & 1);
-  const int row = (int)(v / (2 * a.n_kv_heads));
-  const int64_t xoff = (int64_t)row * a.token_stride + (int64_t)head * a.head_stride;
-  const float xv = load_elem(kv ? a.V : a.K, a.in_dtype, xoff + j);
-  if (!isfinite(xv)) {
-    atomicAdd(a.status + 1, 1);
-    set_status(a.status, PQ_ERR_NONFINITE);
-  }
-  xs[j] = xv;
-  if (j == 0) {
-    load_fast_quant(a.tables, &fq);
-    amb_blocks = 0u;
-  }
-  __syncthreads();
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-  for (int k = 0; k < 128; k += 4) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = fmaf(xs[k + i], __ldg(a.S + (k + i) * 128 + j), acc[i]);
-  }
-  const float y = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-  ys[j] = y;
-  float sq = y * y;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-  if ((j & 31) == 0) red[j >> 5] = sq;
-  __syncthreads();
-  // four independent partial sums instead of one chain: the bound of a 128-term float32 dot product still holds
-  const float norm = 1.0001f * sqrtf((red[0] + red[1]) + (red[2] + red[3]));
-  FastBlock fb = {0u, 0u, 0u, 0u, 0u, 0.f};
-  if (j < 8) {
-    float yb[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) yb[i] = ys[16 * j + i];
-    if (fq.analytic) polar_quant_block_fast<true>(yb, make_row_margins(norm, kRotErr, fq), fq, &fb);
-    else polar_quant_block_fast<false>(yb, make_row_margins(norm, kRotErr, fq), fq, &fb);
-  }
-  if (fb.amb != 0u) atomicOr(&amb_blocks, 1u << j);
-  if (__syncthreads_or(fb.amb != 0u)) {
-    if ((amb_blocks >> (j >> 4)) & 1u) {   // only the coordinates of the blocks in question (half-warps: the float64 pipe is slow)
-      double accd[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int k = 0; k < 128; k += 4) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) accd[i] = fma((double)xs[k + i], (double)__ldg(a.S + (k + i) * 128 + j), accd[i]);
-      }
-      yd[j] = (accd[0] + accd[1]) + (accd[2] + accd[3]);
-    }
-    __syncthreads();
-    if (j < 8 && fb.amb != 0u) {
-      double yb[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) yb[i] = yd[16 * j + i];
-      BlockCodes c;
-      fb.radius = (float)polar_quant_block_exact(yb, *a.tables, c);
-      fb.l1 = c.l1; fb.l2 = c.l2; fb.l3 = c.l3; fb.l4 = c.l4;
-      atomicAdd(a.status + 3, __popc(fb.amb));
-    }
-  }
-  if (j >= 32) return;  // the first warp stores (lanes 0..7 hold the blocks)
-  int seq = 0, pos = -1;
-  if (j < 8) row_destination(a, row, &seq, &pos);
-  const bool valid = j < 8 && pos >= 0;
-  float rv = fb.radius;
-  if (valid && rv > 65504.f) {
-    rv = 65504.f;
-    atomicAdd(a.status + 2, 1);
-  }
-  const Layout L = make_layout(128, a.pg.page_tokens);
-  BlockCodes c = {fb.l1, fb.l2, fb.l3, fb.l4};
-  uint8_t* tb = a.cache + (valid ? block_offset(L, a.pg, a.n_kv_heads, seq, head, kv, pos) : 0);
-  store_block(tb, L, valid ? pos % kTokenBlock : 0, j & 7, c, __float2half_rn(rv), valid);
-}
-
 }  // namespace pq
+#include "pq_append.cuh"
 #include "pq_hist.cuh"
 #include "pq_encode_tc.cuh"
 namespace pq {
@@ -467,24 +376,8 @@ static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
     if (tc < 0) return tc;
     if (tc == 1) return launch_advance_lens(a, lens, stream);
   }
-  if (a.head_dim == 128 && a.total_tokens < 32) {
-    const int64_t n_vec = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)n_vec);
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];   // may be set up while the kernel before it in the stream finishes (it waits inside)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, encode_vector_kernel, a) != cudaSuccess) {
-      cudaGetLastError();
-      return PQ_ERR_CUDA;
-    }
-    return launch_advance_lens(a, lens, stream);
-  }
-  if (a.head_dim == 128 && a.total_tokens >= 32) {
+  if (a.total_tokens < 32 && a.batch <= 65535) return launch_encode_rows(a, lens, stream);
+  if (a.head_dim == 128) {
     static DeviceMemo configured;
     if (configure_for_device(encode_ffma_kernel, kFfmaSmem, configured) == 0) return PQ_ERR_CUDA;
     dim3 grid((a.total_tokens + 127) / 128, a.n_kv_heads, 2);

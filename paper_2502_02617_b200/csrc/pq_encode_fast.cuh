@@ -25,28 +25,18 @@ constexpr float kRotErr = 1.1f * 7.62939453125e-06f;                            
 constexpr float kRotErrTc = 1.1f * (3.f * 9.5367431640625e-07f + 1.4901161193847656e-08f);  // 1.1 * (3 * 2^-20 + 2^-26)
 
 // Per-call constants of the fast quantiser.
-struct FastQuant {
-  float t2[3][3];   // tan^2 of the three boundaries of levels 2, 3, 4
-  uint32_t sym;     // the boundaries of every level >= 2 are b, pi/4, pi/2 - b (kFlagSymmetricUpper)
-  float ua[3][3], ub[3][3];  // the boundary lines of levels 2, 3, 4 scaled to max(|A|, |B|) = 1: D_k = A_k sa + B_k sb
-  uint32_t analytic;       // sym and the uniform level-1 codebook: every decision is a sign test
-  const uint2* l1_cells;   // level-1 decision table of any other codebook (Tables::l1_cells or a copy in shared memory)
+struct FastQuant : QuantLines {
+  const uint2* l1_cells;   // level-1 decision table of a codebook that is not analytic (Tables::l1_cells or a copy in shared memory)
 };
 
 constexpr int kFastQuantBytes = 128;  // what the kernels set aside for a FastQuant in shared memory
 static_assert(sizeof(FastQuant) <= kFastQuantBytes, "shared-memory slot of FastQuant");
 
-__device__ inline void load_fast_quant(const Tables* tb, FastQuant* fq) {
-  for (int l = 0; l < 3; ++l)
-    for (int k = 0; k < 3; ++k) {
-      const double T = tb->bnd_tan2[3 * l + k];
-      fq->t2[l][k] = (float)T;
-      fq->ua[l][k] = (float)(T > 1.0 ? -1.0 : -T);      // sb - T sa, divided by max(1, T)
-      fq->ub[l][k] = (float)(T > 1.0 ? 1.0 / T : 1.0);
-    }
-  fq->sym = (tb->flags & kFlagSymmetricUpper) != 0u;
-  fq->analytic = (tb->flags & (kFlagSymmetricUpper | kFlagUniformL1)) == (kFlagSymmetricUpper | kFlagUniformL1);
-  fq->l1_cells = &tb->l1_cells[0][0];
+// Called by the 32 lanes of a warp.
+__device__ __forceinline__ void load_fast_quant(const Tables* tb, FastQuant* fq, int lane, const uint2* l1_cells) {
+  static_assert(sizeof(QuantLines) == 30 * 4, "one word per lane");
+  if (lane < 30) reinterpret_cast<uint32_t*>(fq)[lane] = __ldg(reinterpret_cast<const uint32_t*>(&tb->lines) + lane);
+  if (lane == 0) fq->l1_cells = l1_cells;
 }
 
 // Per-row constants of the margins (dy = bound on the error of one rotated coordinate of the row).

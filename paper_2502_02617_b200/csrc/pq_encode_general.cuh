@@ -16,8 +16,7 @@
 // Margins: moving every coordinate by at most dy moves the norm of n of them by at most sqrt(n) dy, so a test on the
 // radii of n-coordinate halves moves by at most sqrt(2 n) dy; 1.1 x that, plus 1e-6 (r_a + r_b) for the float32
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
-// A radius is certified by kRadiusSlack: its float32 error is that of a norm, whose coordinate errors average out
-// (2e-8 of the norm on synthetic rows), plus the sum of squares and the square root, at most 5e-7 together.
+// A radius is certified by radius_unsure.
 #pragma once
 #include <math_constants.h>
 
@@ -27,7 +26,6 @@ namespace pq {
 
 constexpr int kGeThreads = 256;
 constexpr int kGeSlice = 32;              // rows of S per slice
-constexpr float kRadiusSlack = 2e-6f;
 
 struct GeShape {
   int dc, ng, vecs, x_stride, row_words, floats_xy;
@@ -60,12 +58,6 @@ __device__ __forceinline__ void ge_put(uint32_t* row, int bit, uint32_t value) {
   atomicOr(row + (bit >> 5), value << sh);
   const uint32_t hi = sh ? value >> (32 - sh) : 0u;
   if (hi) atomicOr(row + (bit >> 5) + 1, hi);
-}
-// Would r round to another fp16 value if it moved by kRadiusSlack?  (NaN and infinite r: yes.)
-__device__ __forceinline__ bool ge_radius_unsure(float r) {
-  const float lo = fminf(r * (1.f - kRadiusSlack), 65504.f), hi = fminf(r * (1.f + kRadiusSlack), 65504.f);
-  return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(lo)) != __half_as_ushort(__float2half_rn(hi)) ||
-         (r > 65000.f);   // saturation is counted from the exact value
 }
 __device__ __forceinline__ float ge_sqrt(float x) {
   float r;
@@ -354,7 +346,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     if (L == kSub) {
 #pragma unroll
       for (int j = 0; j < n_blk; ++j) {
-        if (grp * n_blk + j < g.nb) sure = sure && !ge_radius_unsure(r[j]);
+        if (grp * n_blk + j < g.nb) sure = sure && !radius_unsure(r[j]);
         rad[j] = __half_as_ushort(__float2half_rn(r[j]));
       }
     }
@@ -408,7 +400,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
       }
       for (int j = 0; j < g.nb; ++j) {
         const float r = ge_sqrt(q2[j]);
-        sure = sure && !ge_radius_unsure(r);
+        sure = sure && !radius_unsure(r);
         ge_put(row, g.rad_off * 8 + 16 * j, __half_as_ushort(__float2half_rn(r)));
       }
       if (!sure) {

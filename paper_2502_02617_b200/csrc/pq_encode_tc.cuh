@@ -138,11 +138,8 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     // its results are read only after this wait; the set-up around it overlaps that kernel's tail.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int it = 0; it < kTcStages; ++it) issue_tma(it);  // the first tiles arrive while S is split
-    if (!kHist) {
-      load_fast_quant(a.tables, fq);
-      fq->l1_cells = reinterpret_cast<const uint2*>(smem + kTcSmL1);  // the copy made below
-    }
   }
+  if (!kHist && warp == 2) load_fast_quant(a.tables, fq, lane, reinterpret_cast<const uint2*>(smem + kTcSmL1));  // the copy made below
   uint32_t* hist_s = reinterpret_cast<uint32_t*>(smem + kTcSmFix);
   if (kHist) {
     for (int i = tid; i < 4 * a.n_bins; i += kTcThreads) hist_s[i] = 0u;

@@ -1,5 +1,7 @@
 // The general row layout (any recursion depth and bits per level) and what its encoder and its readers share.
 #pragma once
+#include <math_constants.h>
+
 #include "pq_common.cuh"
 
 namespace pq {
@@ -38,6 +40,16 @@ struct GenEncodeArgs {
 
 // Encode into the packed cache at head dims below 128 (levels and bits of Section 4.1); a.g and a.packed are filled in.
 int32_t launch_packed_encode(GenEncodeArgs a, int head_dim, cudaStream_t stream);
+
+// Would the block radius r round to another fp16 value if it moved by kRadiusSlack?  (NaN and infinite r: yes; near
+// saturation: yes, it is counted from the exact value.)  The float32 error of r is that of a norm, whose coordinate errors
+// average out (2e-8 of the norm on synthetic rows), plus the sum of squares and the square root, at most 5e-7 together.
+constexpr float kRadiusSlack = 2e-6f;
+__device__ __forceinline__ bool radius_unsure(float r) {
+  const float lo = fminf(r * (1.f - kRadiusSlack), 65504.f), hi = fminf(r * (1.f + kRadiusSlack), 65504.f);
+  return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(lo)) != __half_as_ushort(__float2half_rn(hi)) ||
+         r > 65000.f;
+}
 
 // (cos x, sin x) for 0 <= x <= 2 pi, rounded once to float32 from a float64 evaluation: x is reduced by a multiple of
 // pi/2 and both functions of the remainder r (|r| <= pi/4) are summed from their Taylor series; the first terms left

@@ -411,6 +411,14 @@ int32_t pq_build_tables(const double* cen, const double* bnd, void* tables_host)
     if (std::fabs(t.bnd_tan2[3 * l + 1] - 1.0) > 1e-9 || std::fabs(t.bnd_tan2[3 * l] * t.bnd_tan2[3 * l + 2] - 1.0) > 1e-9)
       symmetric = false;
   t.flags = (uniform ? pq::kFlagUniformL1 : 0u) | (symmetric ? pq::kFlagSymmetricUpper : 0u);
+  for (int k = 0; k < 9; ++k) {
+    const double T = t.bnd_tan2[k];
+    (&t.lines.t2[0][0])[k] = (float)T;
+    (&t.lines.ua[0][0])[k] = (float)(T > 1.0 ? -1.0 : -T);   // sb - T sa, divided by max(1, T)
+    (&t.lines.ub[0][0])[k] = (float)(T > 1.0 ? 1.0 / T : 1.0);
+  }
+  t.lines.sym = symmetric ? 1u : 0u;
+  t.lines.analytic = symmetric && uniform ? 1u : 0u;
   for (int k = 0; k < PQ_N_CENTROIDS; ++k) {
     t.cen_cos[k] = (float)std::cos(cen[k]);
     t.cen_sin[k] = (float)std::sin(cen[k]);
