@@ -1,9 +1,10 @@
-"""Thin ctypes binding of the C ABI declared in include/polarquant.h.
+"""Thin binding of the C ABI declared in include/polarquant.h.
 
 Argument marshalling only: every step of the path (rotation, polar transform, quantisation,
 packing, decode attention) runs inside the CUDA library.  PyTorch supplies device memory and
-streams.  There is no CPU fallback: if the shared library is missing the import of any entry
-point raises.
+streams.  The calls of a serving loop go through the extension module _pq_binding (csrc/pq_binding.cpp),
+everything else through ctypes.  There is no CPU fallback: if the shared library or the module is missing
+any entry point raises.
 """
 from __future__ import annotations
 
@@ -127,6 +128,19 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The extension module behind the calls of a serving loop (built in-tree beside the library).  Raises if absent."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _pq_binding
+        _native = _pq_binding
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().pq_status_string(int(status)).decode()
 
@@ -237,43 +251,29 @@ def pq_workspace_bytes(d: int, batch: int, n_q_heads: int, n_kv_heads: int, max_
 
 def pq_encode_kv(S, tables, K, V, cu_seqlens, cache, cache_lens, capacity, status, stream=None):
     """Encode packed ragged K, V [total_tokens, Hkv, d] into `cache`; cache_lens advances."""
-    total, n_kv_heads, d = K.shape
-    assert V.shape == K.shape and V.dtype == K.dtype and K.stride(2) == 1 and V.stride() == K.stride()
-    _check(lib().pq_encode_kv(d, n_kv_heads, _ptr(S), _ptr(tables), _ptr(K), _ptr(V), _dtype_code(K), K.stride(0),
-                              K.stride(1), _ptr(cu_seqlens), cu_seqlens.numel() - 1, total, _ptr(cache),
-                              _ptr(cache_lens), capacity, _ptr(status), _stream(stream)), "pq_encode_kv")
+    _check((_native or native()).encode(S, tables, K, V, cu_seqlens, cache, cache_lens, capacity, status, 0, stream), "pq_encode_kv")
 
 
 def pq_append_kv(S, tables, k_new, v_new, cache, cache_lens, capacity, status, stream=None):
     """Append one token per sequence: k_new, v_new [B, Hkv, d] contiguous."""
-    batch, n_kv_heads, d = k_new.shape
-    assert k_new.is_contiguous() and v_new.is_contiguous() and v_new.shape == k_new.shape
-    _check(lib().pq_append_kv(d, n_kv_heads, _ptr(S), _ptr(tables), _ptr(k_new), _ptr(v_new), _dtype_code(k_new),
-                              batch, _ptr(cache), _ptr(cache_lens), capacity, _ptr(status), _stream(stream)),
-           "pq_append_kv")
+    _check((_native or native()).append(S, tables, k_new, v_new, cache, cache_lens, capacity, status, 0, stream), "pq_append_kv")
 
 
 def pq_decode_attention(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, workspace,
                         status, stream=None):
     """Eq. 3 for one query per sequence: q, out [B, Hq, d] (bf16 or f32)."""
-    batch, n_q_heads, d = q.shape
-    assert q.is_contiguous() and out.is_contiguous() and out.shape == q.shape and out.dtype == q.dtype
-    _check(lib().pq_decode_attention(d, n_q_heads, n_kv_heads, _ptr(S), _ptr(tables), _ptr(q), _dtype_code(q),
-                                     _ptr(cache), _ptr(cache_lens), batch, capacity, max_len, float(scale),
-                                     _ptr(out), _ptr(workspace), _ptr(status), _stream(stream)),
-           "pq_decode_attention")
+    assert q.dim() == 3
+    _check((_native or native()).attend(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, None, workspace, status,
+                                        0, stream), "pq_decode_attention")
 
 
 def pq_multi_query_attention(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, workspace,
                              status, stream=None):
     """Eq. 2 / 3 for the last n_q positions of every sequence: q, out [B, n_q, Hq, d]; query j sees the cached
     tokens before and at its own position.  `workspace` must hold pq_workspace_bytes(d, B * n_q, Hq, Hkv, max_len)."""
-    batch, n_q, n_q_heads, d = q.shape
-    assert q.is_contiguous() and out.is_contiguous() and out.shape == q.shape and out.dtype == q.dtype
-    _check(lib().pq_multi_query_attention(d, n_q_heads, n_kv_heads, _ptr(S), _ptr(tables), _ptr(q), _dtype_code(q),
-                                          _ptr(cache), _ptr(cache_lens), batch, n_q, capacity, max_len, float(scale),
-                                          _ptr(out), _ptr(workspace), _ptr(status), _stream(stream)),
-           "pq_multi_query_attention")
+    assert q.dim() == 4
+    _check((_native or native()).attend(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, None, workspace, status,
+                                        0, stream), "pq_multi_query_attention")
 
 
 def pq_static_scratch_bytes() -> int:
@@ -319,14 +319,8 @@ def pq_decode_attention_lse(S, tables, q, cache, cache_lens, n_kv_heads, capacit
                             status, paging=None, stream=None):
     """pq_decode_attention that also writes lse float32 [B, Hq] (log of the softmax denominator); `paging`: a Paging
     for a paged cache, else the contiguous cache of `capacity` tokens."""
-    batch, n_q_heads, d = q.shape
-    assert q.is_contiguous() and out.is_contiguous() and out.shape == q.shape and out.dtype == q.dtype
-    assert lse.dtype == torch.float32 and lse.is_contiguous() and lse.shape == (batch, n_q_heads)
-    _check(lib().pq_decode_attention_lse(d, n_q_heads, n_kv_heads, _ptr(S), _ptr(tables), _ptr(q), _dtype_code(q),
-                                         _ptr(cache), _ptr(cache_lens), batch, capacity,
-                                         None if paging is None else ctypes.addressof(paging), max_len, float(scale),
-                                         _ptr(out), _ptr(lse), _ptr(workspace), _ptr(status), _stream(stream)),
-           "pq_decode_attention_lse")
+    _check((_native or native()).attend(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, lse, workspace, status,
+                                        0 if paging is None else ctypes.addressof(paging), stream), "pq_decode_attention_lse")
 
 
 def pq_merge_attention(parts_out, parts_lse, out, status, lse_out=None, stream=None):
@@ -442,13 +436,23 @@ class PolarQuantCache:
         """q [B, n_q, Hq, d]: the last n_q positions of every sequence (already in the cache), causal."""
         out = torch.empty_like(q) if out is None else out
         scale = self.d ** -0.5 if scale is None else scale
-        need = pq_workspace_bytes(self.d, self.batch * q.shape[1], self.n_q_heads, self.n_kv_heads, self.capacity)
-        if getattr(self, "_multi_ws", None) is None or self._multi_ws.numel() < need:
-            self._multi_ws = torch.empty(need, dtype=torch.uint8, device=self.device)
         pq_multi_query_attention(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
-                                 self.capacity if max_len is None else max_len, scale, out, self._multi_ws, self.status,
-                                 stream)
+                                 self.capacity if max_len is None else max_len, scale, out, self._multi_workspace(q.shape[1]),
+                                 self.status, stream)
         return out
+
+    _multi_ws = None   # workspace of attend_multi; _multi_need: bytes it takes per number of queries
+    _multi_need = None
+
+    def _multi_workspace(self, n_q):
+        if self._multi_need is None:
+            self._multi_need = {}
+        need = self._multi_need.get(n_q)
+        if need is None:
+            need = self._multi_need[n_q] = pq_workspace_bytes(self.d, self.batch * n_q, self.n_q_heads, self.n_kv_heads, self.capacity)
+        if self._multi_ws is None or self._multi_ws.numel() < need:
+            self._multi_ws = torch.empty(need, dtype=torch.uint8, device=self.device)
+        return self._multi_ws
 
     def unpack(self, n_tokens):
         return pq_unpack_codes(self.d, self.n_kv_heads, self.cache, self.batch, self.capacity, n_tokens)
@@ -486,52 +490,43 @@ class PagedPolarQuantCache(PolarQuantCache):
         self.workspace = torch.empty(pq_workspace_bytes(d, batch, n_q_heads, n_kv_heads, self.capacity), dtype=torch.uint8,
                                      device=self.device)
 
+    _pg = None   # (page table tensor, its address, tokens per page, pages, the struct, the struct's address)
+
+    def _paging_address(self):
+        """Address of the pq_paging struct, made again when the table or the pool it describes has been replaced."""
+        pg, table = self._pg, self.page_table
+        if pg is None or pg[0] is not table or pg[1] != table.data_ptr() or pg[2] != self.page_tokens or pg[3] != self.n_pages:
+            s = Paging.of(table, self.page_tokens, self.n_pages)
+            pg = self._pg = (table, table.data_ptr(), self.page_tokens, self.n_pages, s, ctypes.addressof(s))
+        return pg[5]
+
     def _paging(self):
-        return Paging.of(self.page_table, self.page_tokens, self.n_pages)
+        self._paging_address()
+        return self._pg[4]
 
     def encode(self, K, V, cu_seqlens, stream=None):
-        total, n_kv_heads, d = K.shape
-        assert V.shape == K.shape and V.dtype == K.dtype and K.stride(2) == 1 and V.stride() == K.stride()
-        pg = self._paging()
-        _check(lib().pq_encode_kv_paged(d, n_kv_heads, _ptr(self.S), _ptr(self.tables), _ptr(K), _ptr(V), _dtype_code(K),
-                                        K.stride(0), K.stride(1), _ptr(cu_seqlens), cu_seqlens.numel() - 1, total,
-                                        _ptr(self.cache), _ptr(self.lens), ctypes.addressof(pg), _ptr(self.status),
-                                        _stream(stream)), "pq_encode_kv_paged")
+        _check((_native or native()).encode(self.S, self.tables, K, V, cu_seqlens, self.cache, self.lens, self.capacity, self.status,
+                                            self._paging_address(), stream), "pq_encode_kv_paged")
 
     def append(self, k_new, v_new, stream=None):
-        batch, n_kv_heads, d = k_new.shape
-        assert k_new.is_contiguous() and v_new.is_contiguous() and v_new.shape == k_new.shape
-        pg = self._paging()
-        _check(lib().pq_append_kv_paged(d, n_kv_heads, _ptr(self.S), _ptr(self.tables), _ptr(k_new), _ptr(v_new),
-                                        _dtype_code(k_new), batch, _ptr(self.cache), _ptr(self.lens), ctypes.addressof(pg),
-                                        _ptr(self.status), _stream(stream)), "pq_append_kv_paged")
+        _check((_native or native()).append(self.S, self.tables, k_new, v_new, self.cache, self.lens, self.capacity, self.status,
+                                            self._paging_address(), stream), "pq_append_kv_paged")
 
     def attend(self, q, out=None, scale=None, max_len=None, stream=None):
         out = torch.empty_like(q) if out is None else out
-        batch, n_q_heads, d = q.shape
-        assert q.is_contiguous() and out.is_contiguous() and out.shape == q.shape and out.dtype == q.dtype
-        pg = self._paging()
-        _check(lib().pq_decode_attention_paged(d, n_q_heads, self.n_kv_heads, _ptr(self.S), _ptr(self.tables), _ptr(q),
-                                               _dtype_code(q), _ptr(self.cache), _ptr(self.lens), batch,
-                                               ctypes.addressof(pg), self.capacity if max_len is None else max_len,
-                                               float(self.d ** -0.5 if scale is None else scale), _ptr(out),
-                                               _ptr(self.workspace), _ptr(self.status), _stream(stream)),
+        assert q.dim() == 3
+        _check((_native or native()).attend(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
+                                            self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
+                                            out, None, self.workspace, self.status, self._paging_address(), stream),
                "pq_decode_attention_paged")
         return out
 
     def attend_multi(self, q, out=None, scale=None, max_len=None, stream=None):
         out = torch.empty_like(q) if out is None else out
-        batch, n_q, n_q_heads, d = q.shape
-        assert q.is_contiguous() and out.is_contiguous() and out.shape == q.shape and out.dtype == q.dtype
-        need = pq_workspace_bytes(self.d, self.batch * n_q, self.n_q_heads, self.n_kv_heads, self.capacity)
-        if getattr(self, "_multi_ws", None) is None or self._multi_ws.numel() < need:
-            self._multi_ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-        pg = self._paging()
-        _check(lib().pq_multi_query_attention_paged(d, n_q_heads, self.n_kv_heads, _ptr(self.S), _ptr(self.tables), _ptr(q),
-                                                    _dtype_code(q), _ptr(self.cache), _ptr(self.lens), batch, n_q,
-                                                    ctypes.addressof(pg), self.capacity if max_len is None else max_len,
-                                                    float(self.d ** -0.5 if scale is None else scale), _ptr(out),
-                                                    _ptr(self._multi_ws), _ptr(self.status), _stream(stream)),
+        assert q.dim() == 4
+        _check((_native or native()).attend(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
+                                            self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
+                                            out, None, self._multi_workspace(q.shape[1]), self.status, self._paging_address(), stream),
                "pq_multi_query_attention_paged")
         return out
 
@@ -597,22 +592,14 @@ class GeneralPolarQuantCache:
         self.status = torch.zeros(STATUS_WORDS, dtype=torch.int32, device=self.device)
 
     def encode(self, K, V, cu_seqlens, stream=None):
-        total, n_kv_heads, d = K.shape
-        assert V.shape == K.shape and V.dtype == K.dtype and K.stride(2) == 1 and V.stride() == K.stride() and d == self.d
-        _check(lib().pq_general_encode_kv(ctypes.addressof(self.cfg), n_kv_heads, _ptr(self.S), _ptr(self.boundaries_dev), _ptr(K),
-                                          _ptr(V), _dtype_code(K), K.stride(0), K.stride(1), _ptr(cu_seqlens),
-                                          cu_seqlens.numel() - 1, total, _ptr(self.cache), _ptr(self.lens), self.capacity,
-                                          _ptr(self.status), _stream(stream)), "pq_general_encode_kv")
+        _check((_native or native()).general_encode(ctypes.addressof(self.cfg), self.S, self.boundaries_dev, K, V, cu_seqlens, self.cache,
+                                                    self.lens, self.capacity, self.status, stream), "pq_general_encode_kv")
 
     def attend(self, q, out=None, scale=None, stream=None):
         out = torch.empty_like(q) if out is None else out
-        batch, n_q_heads, d = q.shape
-        assert q.is_contiguous() and out.is_contiguous() and out.dtype == q.dtype and d == self.d
-        _check(lib().pq_general_decode_attention(ctypes.addressof(self.cfg), n_q_heads, self.n_kv_heads, _ptr(self.S),
-                                                 _ptr(self.centroids_dev), _ptr(q), _dtype_code(q), _ptr(self.cache),
-                                                 _ptr(self.lens), batch, self.capacity,
-                                                 float(self.d ** -0.5 if scale is None else scale), _ptr(out),
-                                                 _ptr(self.status), _stream(stream)), "pq_general_decode_attention")
+        _check((_native or native()).general_attend(ctypes.addressof(self.cfg), self.n_kv_heads, self.S, self.centroids_dev, q, self.cache,
+                                                    self.lens, self.capacity, self.d ** -0.5 if scale is None else scale, out,
+                                                    self.status, stream), "pq_general_decode_attention")
         return out
 
     def unpack(self, n_tokens):
