@@ -166,7 +166,7 @@ int32_t pq_fit_codebooks_from_histograms(const uint64_t* hist_host, int32_t n_bi
  * invalid arguments. */
 int64_t pq_cache_bytes(int32_t head_dim, int32_t batch, int32_t n_kv_heads, int32_t capacity);
 
-/* Scratch bytes pq_decode_attention needs (rotated queries, split partials, tickets). */
+/* Scratch bytes pq_decode_attention needs (split partials and their flags). */
 int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, int32_t n_kv_heads,
                            int32_t max_len);
 
@@ -210,8 +210,8 @@ int32_t pq_append_kv(int32_t head_dim, int32_t n_kv_heads, const float* S_dev, c
  *   q_dev          [batch][n_q_heads][head_dim] of `io_dtype` (PQ_DTYPE_BF16 or PQ_DTYPE_F32)
  *   out_dev        same shape and dtype; accumulation is float32
  *   max_len        host-side upper bound on lens[b] (used only to size the token splits)
- *   workspace_dev  pq_workspace_bytes(...) bytes of scratch; it need not be initialised (the split
- *                  counters inside are tagged with a per-call number) and need not be preserved;
+ *   workspace_dev  pq_workspace_bytes(...) bytes of scratch; it need not be initialised (the flags
+ *                  inside are tagged with a per-call number) and need not be preserved;
  *                  two calls that overlap in time must not share it
  * A sequence with lens[b] = 0 yields zeros and records PQ_ERR_EMPTY.
  */
@@ -259,9 +259,8 @@ int32_t pq_multi_query_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_
  *     no allocation); make that first call outside any stream capture.
  *   - Never calls cudaMalloc, cudaFree or any allocating routine.
  *   - All calls on a device share the one array.  It keeps the previous call's contents; nothing in
- *     it has to start at zero: the head_dim-128 kernel tags its split counters with the call's
- *     number and ignores counters of other calls, the other head_dims clear theirs in the call's
- *     first kernel.  Calls that may overlap on the GPU (different streams, no ordering) race on
+ *     it has to start at zero: the head_dim-128 kernel tags its flags with the call's number and
+ *     ignores those of other calls, the other head_dims use none.  Calls that may overlap on the GPU (different streams, no ordering) race on
  *     it: order them.
  */
 #define PQ_STATIC_SCRATCH_BYTES (4 * 1024 * 1024)
@@ -289,6 +288,8 @@ int32_t pq_decode_attention_static(int32_t head_dim, int32_t n_q_heads, int32_t 
  * tcgen05 kernel takes chunks of 128 rows and more, and chunks of 32 to 127 rows when its estimated time
  * -- kv heads x sequences CTA pairs walking max_len / 64 blocks -- is below that of one decode attention
  * per query; everything else runs the decode kernels with one (sequence, query) pair per unit.)
+ * `which` = 5 is of that kind too: the next attention call at head_dim 128 that is decided between the persistent kernel and
+ * the cluster kernel of short contexts runs the persistent one, whatever max_len is (2 implies it).
  */
 int32_t pq_debug_fail_next_wait(int32_t which);
 

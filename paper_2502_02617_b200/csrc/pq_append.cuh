@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
   __shared__ double exact_part[64][17];
   __shared__ BlockCodes exact_codes;
   __shared__ double exact_radius;
-  __shared__ int n_list, row_ok;
+  __shared__ int n_list;
   __shared__ uint16_t list[R::kQuant];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int col = tid % D, slice = (tid / D) % R::kSlices, vgrp = tid / (D * R::kSlices);

@@ -226,6 +226,12 @@ __device__ inline double polar_quant_block_exact(const double* y, const Tables& 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
+// A load of constant data that stays where it is written (the compiler sinks plain loads to their first use).
+__device__ __forceinline__ float ld_const_now(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
 // Packed float32 arithmetic: one instruction for two IEEE multiply-adds.
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
   uint64_t r;
@@ -233,6 +239,11 @@ __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
   return r;
 }
 __device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -275,6 +286,22 @@ inline int configure_for_device(Kernel kernel, int smem_bytes, DeviceMemo& state
   e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e == cudaSuccess && big_clusters) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && n_sm <= 0) e = cudaErrorInvalidDevice;
+  if (e != cudaSuccess) {
+    note_cuda_error(e);
+    return 0;
+  }
+  state[dev].store(n_sm, std::memory_order_release);
+  return n_sm;
+}
+
+// The current device's SM count (0 with the CUDA error noted).
+inline int sm_count_of_device(DeviceMemo& state) {
+  int dev = -1, n_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
+  if (e == cudaSuccess && (n_sm = state[dev].load(std::memory_order_acquire)) > 0) return n_sm;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess && n_sm <= 0) e = cudaErrorInvalidDevice;
   if (e != cudaSuccess) {
     note_cuda_error(e);

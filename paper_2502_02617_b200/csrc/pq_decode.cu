@@ -74,10 +74,11 @@ __device__ inline float decode_coord(const uint8_t* tb, const Layout& L, int tok
 // ---- workspace -----------------------------------------------------------------------------
 constexpr int kFastMaxGridHost = 160;  // upper bound on the persistent kernel's grid (one CTA per SM)
 
-struct Workspace {   // of the persistent head_dim-128 kernel; nothing else needs scratch
-  int32_t* tickets;  // [B][Hkv], 8 bytes each: the kernel's tagged tickets
-  float* ml;         // [slot][head in group][2]   slot = first slot of the unit + part
-  float* o;          // [slot][head in group][d]
+struct Workspace {   // of the persistent head_dim-128 kernel; nothing else needs scratch, and none of it needs clearing
+  uint32_t* elected;  // [B][Hkv]: the epoch of the last call whose parts of the unit were combined
+  uint32_t* flags;    // [slot]: the epoch of the last call whose partial result is in the slot
+  float* ml;          // [slot][head in group][2]   slot = first slot of the unit + part
+  float* o;           // [slot][head in group][d]
   int64_t bytes;
 };
 
@@ -86,10 +87,12 @@ __host__ inline Workspace carve_workspace(void* base, int d, int batch, int n_q_
   auto align = [](int64_t x) { return (x + 255) & ~(int64_t)255; };
   int64_t off = 0;
   uint8_t* p = reinterpret_cast<uint8_t*>(base);
-  w.tickets = reinterpret_cast<int32_t*>(p + off);
-  off = align(off + (int64_t)batch * n_kv_heads * 8);
   const int64_t g = n_q_heads / n_kv_heads, units = (int64_t)batch * n_kv_heads;
   const int64_t n_slots = (d == 128 && units <= 2048) ? units + kFastMaxGridHost : 0;
+  w.elected = reinterpret_cast<uint32_t*>(p + off);
+  off = align(off + units * 4);
+  w.flags = reinterpret_cast<uint32_t*>(p + off);
+  off = align(off + n_slots * 4);
   w.ml = reinterpret_cast<float*>(p + off);
   off = align(off + n_slots * g * 2 * 4);
   w.o = reinterpret_cast<float*>(p + off);
@@ -104,7 +107,7 @@ struct DecodeArgs {
   int n_q;  // queries per sequence (1: decode).  `batch` counts (sequence, query) pairs: q and out are
             // [batch][n_q_heads][d] with pair p = sequence * n_q + query; `lens` and the cache are per sequence.
   float scale;
-  uint32_t epoch;  // differs from call to call (top bit set): tags the split tickets of the persistent kernel
+  uint32_t epoch;  // differs from call to call (top bit set): tags the parts' flags of the persistent kernel
   uint32_t debug;  // test hooks.  bit 0: the first bounded wait of CTA 0 of the persistent kernel reports failure;
                    // bit 1: the MMA thread of CTA (0, 0, 0) of the tcgen05 multi-query kernel reports its wait for the
                    // third decoded block (the last one of a shorter sequence) as failed
@@ -129,95 +132,6 @@ struct DecodeArgs {
   }
 };
 
-// Shared memory (floats) that combine_and_store needs.
-__host__ __device__ inline int combine_smem_floats(int g, int d, int n_parts) { return ((2 * g * n_parts + g + 3) & ~3) + g * d; }
-
-// Merge the `ns` partials (slots slot0 .. slot0 + ns - 1) of the `g` query heads of (b, kv head) in slot
-// order, normalise, rotate back by S^T and store.  Runs in the last CTA that finishes for this
-// (b, kv head); `sm` must hold combine_smem_floats(g, d, ns) floats.  Every phase issues its global
-// loads side by side (the CTA that runs this is the last one still working on the unit).
-__device__ void combine_and_store(const DecodeArgs& a, int b, int hk, int g, int slot0, int ns, float* sm) {
-  const int d = a.d, tid = threadIdx.x, nthr = blockDim.x;
-  float* w_sm = sm;                  // [g][ns] running maximum of split s for head h, then its weight
-  float* l_sm = sm + g * ns;         // [g][ns] denominator of split s for head h
-  float* linv_sm = l_sm + g * ns;    // [g]
-  float* o_sm = sm + ((2 * g * ns + g + 3) & ~3);  // [g][d], 16-byte aligned
-  const int64_t h0 = (int64_t)b * a.n_q_heads + hk * g;
-  for (int idx = tid; idx < g * ns; idx += nthr) {
-    const int h = idx / ns, s = idx - h * ns;
-    const float2 ml = *reinterpret_cast<const float2*>(a.ws.ml + ((int64_t)(slot0 + s) * g + h) * 2);
-    w_sm[idx] = ml.x;
-    l_sm[idx] = ml.y;
-  }
-  __syncthreads();
-  if (tid < g) {
-    float M = -CUDART_INF_F;
-    for (int s = 0; s < ns; ++s) M = fmaxf(M, w_sm[tid * ns + s]);
-    float Lsum = 0.f;
-    for (int s = 0; s < ns; ++s) {  // slot order
-      const float ms = w_sm[tid * ns + s];
-      const float w = ms == -CUDART_INF_F ? 0.f : exp2f(ms - M);
-      w_sm[tid * ns + s] = w;
-      Lsum += l_sm[tid * ns + s] * w;
-    }
-    linv_sm[tid] = Lsum > 0.f ? 1.f / Lsum : 0.f;
-    // scores are kept in the log2 domain: sum_t exp(s_t) = 2^M * Lsum
-    if (a.lse != nullptr) a.lse[h0 + tid] = Lsum > 0.f ? (M + log2f(Lsum)) * 0.693147180559945309f : -CUDART_INF_F;
-  }
-  __syncthreads();
-  for (int idx = tid; idx < g * d; idx += nthr) {
-    const int h = idx / d, j = idx - h * d;
-    const float* op = a.ws.o + ((int64_t)slot0 * g + h) * d + j;
-    float acc = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) acc = fmaf(op[(int64_t)s * g * d], w_sm[h * ns + s], acc);
-    o_sm[idx] = acc * linv_sm[h];
-  }
-  __syncthreads();
-  // x_hat_i = sum_j y_hat_j S[i][j]: a warp takes eight rows i at a time, lanes over j (coalesced), and
-  // has the loads of all eight rows in flight before the first is used.
-  const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
-  constexpr int kRows = 8;
-  for (int i0 = warp * kRows; i0 < d; i0 += nwarps * kRows) {
-    float sv[kRows][4];
-#pragma unroll
-    for (int r = 0; r < kRows; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = lane + 32 * q;
-        sv[r][q] = (i0 + r < d && j < d) ? __ldg(a.S + (int64_t)(i0 + r) * d + j) : 0.f;
-      }
-    for (int h = 0; h < g; ++h) {
-      float ov[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) ov[q] = lane + 32 * q < d ? o_sm[h * d + lane + 32 * q] : 0.f;
-      float v[kRows];
-#pragma unroll
-      for (int r = 0; r < kRows; ++r)
-        v[r] = fmaf(ov[3], sv[r][3], fmaf(ov[2], sv[r][2], fmaf(ov[1], sv[r][1], ov[0] * sv[r][0])));
-      // Sum over the 32 lanes: three halving exchanges leave lane L with row L >> 2 (summed over eight
-      // lanes), two more finish it.  9 shuffles per head instead of 40; the order is fixed.
-      float w4[4], w2[2];
-      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        w4[k] = (b4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, b4 ? v[k] : v[k + 4], 16);
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        w2[k] = (b3 ? w4[k + 2] : w4[k]) + __shfl_xor_sync(0xffffffffu, b3 ? w4[k] : w4[k + 2], 8);
-      float t = (b2 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? w2[0] : w2[1], 4);
-      t += __shfl_xor_sync(0xffffffffu, t, 2);
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      const int row = i0 + (lane >> 2);
-      if ((lane & 3) == 0 && row < d) {
-        const int64_t oidx = (h0 + h) * d + row;
-        if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[oidx] = __float2bfloat16(t);
-        else reinterpret_cast<float*>(a.out)[oidx] = t;
-      }
-    }
-  }
-}
-
 }  // namespace pq
 #include "pq_decode_fast.cuh"
 #include "pq_prefill.cuh"
@@ -225,18 +139,24 @@ __device__ void combine_and_store(const DecodeArgs& a, int b, int hk, int g, int
 #include "pq_split_attention.cuh"
 namespace pq {
 
-// The packed cache for split_attention_kernel: head dims below 128 (and head_dim 128 with more units than the persistent
-// kernel's schedule holds).  A chunk is whole token-blocks, which are contiguous and 16-byte aligned.
+// The packed cache for split_attention_kernel.  A tile is part of a token-block: five pieces, one per plane, each a multiple
+// of 16 bytes long and 16-byte aligned in the cache and in the buffer.
+template <int D>
 struct PackedSplit {
   static constexpr bool kEarlyTables = true;
+  static constexpr int kTabMax = 32, kDim = D;
+  // the planes of a token-block (make_layout for this head_dim)
+  static constexpr int kNb = D / 16, kB1 = 4 * kNb, kB2 = kNb, kB3 = kNb >= 2 ? kNb / 2 : 1, kB4 = kNb >= 4 ? kNb / 4 : 1, kBr = 2 * kNb;
+  static constexpr int kRow = kB1 + kB2 + kB3 + kB4 + kBr, kBlockBytes = kTokenBlock * kRow;
   SplitCommon c;
-  Layout L;
-  int stage_bytes, n_tab, n_q;
+  int n_q;
+  int64_t head_bytes;
   const Tables* tables;
   const uint8_t* cache;
   const int32_t* lens;
   Paging pg;
 
+  static int tile_bytes(int n) { return n * kRow; }
   __device__ __forceinline__ int len(int pair) const {
     const int b = pair / n_q, v = lens[b] - (n_q - 1 - (pair - b * n_q));
     return v > 0 ? v : 0;
@@ -245,47 +165,87 @@ struct PackedSplit {
     if (tid < PQ_N_CENTROIDS) tab[tid] = make_float2(tables->cen_cos[tid], tables->cen_sin[tid]);
   }
   __device__ __forceinline__ int shift(int, int, int, int) const { return 0; }
-  __device__ __forceinline__ void stage(uint32_t buf, int pair, int hk, int kv, int t0, int n, int tid) const {
-    const int per_block = L.block_bytes >> 4, pieces = ((n + kTokenBlock - 1) / kTokenBlock) * per_block;
-    for (int i = tid; i < pieces; i += kSplitThreads) {
-      const int blk = i / per_block;
-      const int64_t off = kv_block_pair_offset(L, pg, c.n_kv_heads, pair / n_q, hk, t0 / kTokenBlock + blk, c.status);
-      split_cp16(buf + 16 * i, cache + off + (int64_t)kv * L.block_bytes + 16 * (i - blk * per_block));
+  __device__ __forceinline__ void stage(uint8_t* buf, int pair, int hk, int kv, int t0, int, int lane) const {
+    Layout L;
+    L.block_bytes = kBlockBytes;
+    L.head_bytes = head_bytes;
+    const uint8_t* src = cache + kv_block_pair_offset(L, pg, c.n_kv_heads, pair / n_q, hk, t0 / kTokenBlock, c.status) +
+                         (int64_t)kv * kBlockBytes;
+    const int tok = t0 % kTokenBlock, tile = c.tile;   // a multiple of 16 at these row lengths
+    // byte i of the tile: plane by plane, [tile][bytes per token] each
+#pragma unroll 1
+    for (int i = 16 * lane; i < tile * kRow; i += 512) {
+      int at = tok * kB1 + i;
+      if (i >= tile * kB1) at = kTokenBlock * kB1 + tok * kB2 + i - tile * kB1;
+      if (i >= tile * (kB1 + kB2)) at = kTokenBlock * (kB1 + kB2) + tok * kB3 + i - tile * (kB1 + kB2);
+      if (i >= tile * (kB1 + kB2 + kB3)) at = kTokenBlock * (kB1 + kB2 + kB3) + tok * kB4 + i - tile * (kB1 + kB2 + kB3);
+      if (i >= tile * (kB1 + kB2 + kB3 + kB4))
+        at = kTokenBlock * (kB1 + kB2 + kB3 + kB4) + tok * kBr + i - tile * (kB1 + kB2 + kB3 + kB4);
+      split_cp16(buf + i, src + at);
     }
   }
-  // the groups of a token lie side by side in every plane: neighbouring lanes on neighbouring groups read without conflicts
-  __device__ __forceinline__ int lanes_per_token(int ng) const { return ng < 4 ? ng : 4; }
-  __device__ __forceinline__ void decode(uint32_t buf, int t, int grp, uint32_t tab, float* y) const {
-    const uint32_t tb = buf + (t / kTokenBlock) * L.block_bytes;
-    const int tok = t % kTokenBlock;
-    const uint32_t l1 = split_lds32(tb + tok * L.b1 + 4 * grp), l2 = split_lds8(tb + L.o2 + tok * L.b2 + grp);
-    const uint32_t l3 = split_lds8(tb + L.o3 + tok * L.b3 + (grp >> 1)) >> (4 * (grp & 1));
-    const uint32_t l4 = split_lds8(tb + L.o4 + tok * L.b4 + (grp >> 2)) >> (2 * (grp & 3));
-    const float r = __half2float(__ushort_as_half((unsigned short)split_lds16(tb + L.orad + tok * L.br + 2 * grp)));
-    float r3[2], r2[4], r1[8];
-    const float2 e4 = split_lds_f2(tab + (24 + (l4 & 3u)) * 8);
-    r3[0] = r * e4.x;
-    r3[1] = r * e4.y;
+  // kU = 16: a block; kU = 8: half of one (the angles above it are the block's)
+  template <int kU>
+  __device__ __forceinline__ void decode(const uint8_t* buf, int, int t, int unit, const float2* tab, float* y) const {
+    const int blk = kU == 16 ? unit : unit >> 1, tile = c.tile;
+    const uint8_t* p2 = buf + tile * kB1;
+    const uint8_t* p3 = p2 + tile * kB2;
+    const uint8_t* p4 = p3 + tile * kB3;
+    const __half* pr = reinterpret_cast<const __half*>(p4 + tile * kB4);
+    uint32_t l2 = p2[t * kB2 + blk], l3 = p3[t * kB3 + (blk >> 1)] >> (4 * (blk & 1));
+    const uint32_t l4 = p4[t * kB4 + (blk >> 2)] >> (2 * (blk & 3));
+    const float r = __half2float(pr[t * kNb + blk]);
+    const float2 e4 = tab[24 + (l4 & 3u)];
+    float r1[kU / 2];
+    uint32_t l1;
+    if (kU == 16) {
+      l1 = *reinterpret_cast<const uint32_t*>(buf + t * kB1 + 4 * blk);
+      const float r3[2] = {r * e4.x, r * e4.y};
+      float r2[4];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float2 e = split_lds_f2(tab + (20 + ((l3 >> (2 * j)) & 3u)) * 8);
-      r2[2 * j] = r3[j] * e.x;
-      r2[2 * j + 1] = r3[j] * e.y;
+      for (int j = 0; j < 2; ++j) {
+        const float2 e = tab[20 + ((l3 >> (2 * j)) & 3u)];
+        r2[2 * j] = r3[j] * e.x;
+        r2[2 * j + 1] = r3[j] * e.y;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 e = tab[16 + ((l2 >> (2 * j)) & 3u)];
+        r1[(2 * j) % (kU / 2)] = r2[j] * e.x;
+        r1[(2 * j + 1) % (kU / 2)] = r2[j] * e.y;
+      }
+    } else {
+      const int hi = unit & 1;
+      l1 = *reinterpret_cast<const uint16_t*>(buf + t * kB1 + 4 * blk + 2 * hi);
+      l2 >>= 4 * hi;
+      l3 >>= 2 * hi;
+      const float r3 = r * (hi ? e4.y : e4.x);
+      const float2 e3 = tab[20 + (l3 & 3u)];
+      const float r2[2] = {r3 * e3.x, r3 * e3.y};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float2 e = tab[16 + ((l2 >> (2 * j)) & 3u)];
+        r1[2 * j] = r2[j] * e.x;
+        r1[2 * j + 1] = r2[j] * e.y;
+      }
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 e = split_lds_f2(tab + (16 + ((l2 >> (2 * j)) & 3u)) * 8);
-      r1[2 * j] = r2[j] * e.x;
-      r1[2 * j + 1] = r2[j] * e.y;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float2 e = split_lds_f2(tab + ((l1 >> (4 * j)) & 15u) * 8);
+    for (int j = 0; j < kU / 2; ++j) {
+      const float2 e = tab[(l1 >> (4 * j)) & 15u];
       y[2 * j] = r1[j] * e.x;
       y[2 * j + 1] = r1[j] * e.y;
     }
   }
 };
+
+template <int D>
+static int32_t launch_packed_attention(const SplitCommon& c, int64_t pairs, int n_q, int max_len, const Tables* tables,
+                                       const uint8_t* cache, const int32_t* lens, const Paging& pg, cudaStream_t stream) {
+  PackedSplit<D> p;
+  p.c = c; p.n_q = n_q; p.tables = tables; p.cache = cache; p.lens = lens; p.pg = pg;
+  p.head_bytes = make_layout(D, pg.page_tokens).head_bytes;
+  return dispatch_split_attention(p, pairs, max_len, stream);
+}
 
 // ---- partial attentions: merge, and exact attention over an uncompressed window -----------------
 // out = sum_p w_p out_p with w_p = exp(lse_p - lse) and lse = log sum_p exp(lse_p): the attention over the union of
@@ -676,9 +636,26 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
     return pq::launch_status();
   }
-  if (head_dim == 128 && pairs * n_kv_heads <= pq::kFastMaxUnits) {
-    // One launch: the persistent kernel rotates the queries itself and needs no cleared tickets.
-    // The tickets in the (uninitialised, possibly shared) scratch are tagged with a per-call number.  It starts
+  bool persistent = head_dim == 128 && pairs * n_kv_heads <= pq::kFastMaxUnits, fail_wait = false;
+  if (persistent) {
+    // Short contexts at head_dim 128 take the cluster kernel too: the persistent kernel needs 14 to 16 us (27 with more
+    // than four heads per kv head) before length matters -- tables, work split, partial results through global memory --
+    // the cluster kernel 9 (10) us and then 0.013 / 0.017 / 0.044 us per token of its busiest SM with up to 2 / 4 / 8
+    // heads, several times the persistent kernel's rate.
+    if (n_sm == 0) {
+      static pq::DeviceMemo sm_count;
+      n_sm = pq::sm_count_of_device(sm_count);
+      if (n_sm == 0) return PQ_ERR_CUDA;
+    }
+    int64_t tokens = 0;
+    pq::split_cluster_size(128, 16, pairs * n_kv_heads, max_len, n_sm, &tokens);
+    const bool forced = pq::take_debug_wait_failure(5);
+    fail_wait = pq::take_debug_wait_failure(2);
+    persistent = forced || fail_wait || tokens > (g <= 2 ? 640 : g <= 4 ? 400 : 320);
+  }
+  if (persistent) {
+    // One launch: the persistent kernel rotates the queries itself and needs no cleared scratch.
+    // The flags in the (uninitialised, possibly shared) scratch are tagged with a per-call number.  It starts
     // at a value drawn from the clock and the address space of this process, advances by an odd constant and
     // always has its top bit set, so it cannot equal a small integer that another kernel left in the same bytes.
     static std::atomic<uint32_t> call_epoch{[] {
@@ -688,7 +665,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
       return (uint32_t)(x ^ (x >> 31));
     }()};
     a.epoch = call_epoch.fetch_add(0x9E3779B1u, std::memory_order_relaxed) | 0x80000000u;
-    a.debug = pq::take_debug_wait_failure(2) ? 1u : 0u;
+    a.debug = fail_wait ? 1u : 0u;
     static pq::DeviceMemo configured[4];
     const bool paged = pg.table != nullptr;
     void (*kernel)(pq::DecodeArgs) =
@@ -713,20 +690,14 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     }
     return pq::launch_status();
   }
-  pq::PackedSplit p;
-  p.c.d = head_dim; p.c.n_q_heads = n_q_heads; p.c.n_kv_heads = n_kv_heads; p.c.io_dtype = io_dtype; p.c.scale = scale;
-  p.c.S = S_dev; p.c.q = q_dev; p.c.out = out_dev; p.c.lse = lse_dev; p.c.status = status_dev;
-  p.L = pq::make_layout(head_dim, pg.page_tokens);
-  p.n_tab = (PQ_N_CENTROIDS + 1) & ~1; p.n_q = n_q; p.tables = a.tables; p.cache = a.cache; p.lens = cache_lens_dev; p.pg = pg;
-  p.c.chunk = 512;   // two tokens per thread
-  p.stage_bytes = p.c.chunk / pq::kTokenBlock * p.L.block_bytes;
-  const int kh = g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : 8;
-  const int smem = pq::split_smem_bytes(head_dim, kh, p.n_tab, p.c.chunk, p.stage_bytes);
-  switch (kh) {
-    case 1: return pq::launch_split_attention<pq::PackedSplit, 1>(p, pairs, max_len, smem, st);
-    case 2: return pq::launch_split_attention<pq::PackedSplit, 2>(p, pairs, max_len, smem, st);
-    case 4: return pq::launch_split_attention<pq::PackedSplit, 4>(p, pairs, max_len, smem, st);
-    default: return pq::launch_split_attention<pq::PackedSplit, 8>(p, pairs, max_len, smem, st);
+  pq::SplitCommon c;
+  c.d = head_dim; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
+  c.S = S_dev; c.q = q_dev; c.out = out_dev; c.lse = lse_dev; c.status = status_dev;
+  switch (head_dim) {
+    case 16: return pq::launch_packed_attention<16>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
+    case 32: return pq::launch_packed_attention<32>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
+    case 64: return pq::launch_packed_attention<64>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
+    default: return pq::launch_packed_attention<128>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
   }
 }
 

@@ -43,11 +43,15 @@ constexpr int kSmU = kSmT1lo + 256 * 16 * 8;          // 4 * 64 * 16 * 8 = 32768
 constexpr int kSmBar = kSmU + 4 * 64 * 16 * 8;        // full[4], empty[4] : 64
 constexpr int kSmFlags = kSmBar + 64;                 // abort flag, is_last, n_segs, first_rank : 16
 constexpr int kSmSegs = kSmFlags + 16;                // Segment[32] : 768
-constexpr int kSmQ = kSmSegs + 768;                   // q (fp32) [8][128], q' fp16 value [8][128], q' fp16 residual [8][128] : 8192
-constexpr int kSmRing = (kSmQ + 8192 + 127) / 128 * 128;
+// q (fp32) [8][128], then q' as fp16 values and as fp16 residuals.  A head's q' takes 288 bytes, its quarters (32 coordinates
+// of a fragment lane c) 72 bytes each, and the residuals start 2312 bytes after the values: the 16 lanes of a half-warp
+// (two heads, value or residual, four quarters) then read 16 different bank pairs.
+constexpr int kQHead = 288, kQQuarter = 72, kQLo = 8 * kQHead + 8;
+constexpr int kSmQ = kSmSegs + 768;
+constexpr int kSmRing = (kSmQ + 4096 + kQLo + 8 * kQHead + 127) / 128 * 128;
 // after the main loop the ring is reused for the cross-warp merge: 16 warps x 8 heads x (kMrgStride + 2) floats
 constexpr int kMrgStride = 136;  // floats per (warp, head) row of the merge buffer (136 = 128 + 8: heads 8 banks apart)
-constexpr int kMergeBytes = 16 * 8 * kMrgStride * 4 + 16 * 8 * 2 * 4;  // also >= combine_smem_floats(8, 128, 160) * 4
+constexpr int kMergeBytes = 16 * 8 * kMrgStride * 4 + 16 * 8 * 2 * 4;
 constexpr int kSmUsed = kSmRing + (kStages * kStageBytes > kMergeBytes ? kStages * kStageBytes : kMergeBytes);
 // The tables start on a 32 KB boundary of the shared window, so that a table address is the OR of
 // disjoint bit fields (base | lane replica | index) and needs no addition; the launch asks for 32 KB
@@ -266,6 +270,106 @@ struct Segment {
   int unit, st0, st1, part, n_parts, slot0;
 };
 
+// Merge the `ns` partials (slots slot0 .. slot0 + ns - 1) of the `g` query heads of (b, kv head) in slot order, normalise,
+// rotate back by S^T and store.  Runs in the last CTA that finishes for this unit, so it is a chain of round trips to L2:
+// the rows of S, the first partial outputs of a thread's coordinates and the (m, l) pairs are all requested before
+// anything waits.  `sm`: kCombineFloats floats.
+constexpr int kCombineFloats = 8 * kFastMaxGrid + 8 + 8 * 128;
+static_assert(kCombineFloats * 4 <= kMergeBytes, "the combine uses the merge buffer");
+template <int kHG>
+__device__ __forceinline__ void combine_and_store(const DecodeArgs& a, int b, int hk, int g, int slot0, int ns, float* sm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* w_sm = sm;                          // [g][ns] weights
+  float* linv_sm = w_sm + 8 * kFastMaxGrid;  // [g]
+  float* o_sm = linv_sm + 8;                 // [g][128]
+  const int64_t h0 = (int64_t)b * a.n_q_heads + hk * g;
+  // x_hat_i = sum_j y_hat_j S[i][j]: a warp takes eight rows i, lanes over j
+  constexpr int kRows = 8;
+  const int i0 = warp * kRows;
+  float sv[kRows][4];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sv[r][q] = __ldg(a.S + (i0 + r) * 128 + lane + 32 * q);
+  constexpr int kAhead = 16 / kHG;
+  float part[kHG][kAhead];
+#pragma unroll
+  for (int r = 0; r < kHG; ++r) {
+    const int h = (tid >> 7) + 4 * r;
+    const float* op = a.ws.o + ((int64_t)slot0 * g + h) * 128 + (tid & 127);
+#pragma unroll
+    for (int s = 0; s < kAhead; ++s) part[r][s] = h < g && s < ns ? __ldcg(op + (int64_t)s * g * 128) : 0.f;
+  }
+  if (warp < g) {   // a warp per head: weights of the parts
+    const float2* mlp = reinterpret_cast<const float2*>(a.ws.ml) + (int64_t)slot0 * g + warp;
+    float2 ml[(kFastMaxGrid + 31) / 32];
+    float M = -CUDART_INF_F;
+#pragma unroll
+    for (int i = 0; i < (kFastMaxGrid + 31) / 32; ++i) {
+      ml[i] = make_float2(-CUDART_INF_F, 0.f);
+      if (lane + 32 * i < ns) ml[i] = __ldcg(mlp + (int64_t)(lane + 32 * i) * g);
+      M = fmaxf(M, ml[i].x);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    float L = 0.f;
+#pragma unroll
+    for (int i = 0; i < (kFastMaxGrid + 31) / 32; ++i) {
+      const float w = ml[i].x == -CUDART_INF_F ? 0.f : fast_exp2(ml[i].x - M);
+      if (lane + 32 * i < ns) w_sm[warp * kFastMaxGrid + lane + 32 * i] = w;
+      L = fmaf(ml[i].y, w, L);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    if (lane == 0) {
+      linv_sm[warp] = L > 0.f ? 1.f / L : 0.f;
+      // scores are kept in the log2 domain: sum_t exp(s_t) = 2^M * L
+      if (a.lse != nullptr) a.lse[h0 + warp] = L > 0.f ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kHG; ++r) {
+    const int h = (tid >> 7) + 4 * r, j = tid & 127;
+    if (h < g) {
+      float acc = 0.f;
+#pragma unroll
+      for (int s = 0; s < kAhead; ++s)
+        if (s < ns) acc = fmaf(part[r][s], w_sm[h * kFastMaxGrid + s], acc);
+      const float* op = a.ws.o + ((int64_t)slot0 * g + h) * 128 + j;
+#pragma unroll 4
+      for (int s = kAhead; s < ns; ++s) acc = fmaf(__ldcg(op + (int64_t)s * g * 128), w_sm[h * kFastMaxGrid + s], acc);
+      o_sm[h * 128 + j] = acc * linv_sm[h];
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int h = 0; h < g; ++h) {
+    float ov[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ov[q] = o_sm[h * 128 + lane + 32 * q];
+    float v[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) v[r] = fmaf(ov[3], sv[r][3], fmaf(ov[2], sv[r][2], fmaf(ov[1], sv[r][1], ov[0] * sv[r][0])));
+    // Sum over the 32 lanes: three halving exchanges leave lane L with row L >> 2 (summed over eight
+    // lanes), two more finish it.  9 shuffles per head instead of 40; the order is fixed.
+    float w4[4], w2[2];
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w4[k] = (b4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, b4 ? v[k] : v[k + 4], 16);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) w2[k] = (b3 ? w4[k + 2] : w4[k]) + __shfl_xor_sync(0xffffffffu, b3 ? w4[k] : w4[k + 2], 8);
+    float t = (b2 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? w2[0] : w2[1], 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    if ((lane & 3) == 0) {
+      const int64_t oidx = (h0 + h) * 128 + i0 + (lane >> 2);
+      if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[oidx] = __float2bfloat16(t);
+      else reinterpret_cast<float*>(a.out)[oidx] = t;
+    }
+  }
+}
+
 // kHG = groups of four query heads per kv head (1: up to 4 heads, 2: up to 8).
 // kPaged: the cache lies behind a block table (the contiguous instantiation carries none of that code: the kernel
 // sits at its register limit).
@@ -293,6 +397,17 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   // The kernel after this one may be set up as soon as this grid has started.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   build_fast_tables(smem, a.tables);   // from the caller's tables, which no kernel writes
+  // What this thread needs of S (constant too) to rotate the queries: column warp * 8 + lane / 4, rows 16 i + 4 (lane & 3)
+  // + 0..3 -- a warp's load covers whole 32-byte sectors, and four lanes share a column's sum.
+  const int rot_j = warp * 8 + (lane >> 2), rot_k = (lane & 3) * 4;
+  float s_col[32];
+  auto load_s_col = [&]() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s_col[4 * i + e] = ld_const_now(a.S + (16 * i + rot_k + e) * 128 + rot_j);
+  };
+  load_s_col();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
 
@@ -300,54 +415,94 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   // gridDim.x contiguous ranges of equal cost; a CTA's range may cover the end of one unit and the
   // start of the next, and a unit may be shared by several CTAs (its "parts").  Starting on another
   // unit costs a CTA about kSegmentCost stages (query rotation, refilling the ring, the merge), so
-  // every unit is preceded by that many empty positions on the line that is cut.  Each thread works
-  // out one unit; the units this CTA takes part in are consecutive among the non-empty ones and are
-  // listed kFastMaxSegs at a time (a ragged batch -- one very long sequence and many short ones --
-  // can give a CTA more than that; the split is then worked out again for the next batch of the list,
-  // because its scratch lies in the ring).
+  // every unit is preceded by that many empty positions on the line that is cut.  A thread works out up to four
+  // consecutive units (positions, ranks and partial slots by block-wide scans); the units this CTA takes
+  // part in are consecutive among the non-empty ones and are listed kFastMaxSegs at a time (a ragged batch -- one very
+  // long sequence and many short ones -- can give a CTA more than that; the split is then worked out again for the next
+  // batch of the list, because its scratch lies in the ring).
   const int n_units = a.batch * a.n_kv_heads, G = gridDim.x, cta = blockIdx.x;
-  int* u_nst = reinterpret_cast<int*>(smem + kSmRing);  // [n_units] stages; the ring is idle while the split is worked out
-  int* u_parts = u_nst + kFastMaxUnits;                 // [n_units] CTAs that share the unit
+  long long* scan_w = reinterpret_cast<long long*>(smem + kSmRing);   // [16 warps]; the ring is idle while the split is worked out
+  int* scan_r = reinterpret_cast<int*>(scan_w + 16);                  // [16]
+  int* scan_p = scan_r + 16;                                          // [16]
   Segment* segs = reinterpret_cast<Segment*>(smem + kSmSegs);
   int* n_segs = reinterpret_cast<int*>(smem + kSmFlags) + 2;   // units of this CTA (all batches of the list)
   int* first_rank = reinterpret_cast<int*>(smem + kSmFlags) + 3;
+  // Stages of unit u (0 past the last one).
+  auto stages_of = [&](int u) -> int {
+    const int len_u = u < n_units ? a.visible_len(u / a.n_kv_heads) : 0;
+    return len_u > 0 ? (len_u + kStageTokens - 1) / kStageTokens : 0;
+  };
   // Fills `segs` with the CTA's units number kFastMaxSegs * batch_no .. (counted among the CTA's own) and returns how many
-  // units the CTA has in all.  Called by all threads.
+  // units the CTA has in all.  Called by all threads.  The loops over a thread's units are kept rolled here and in the other
+  // parts that run once: at the start of a launch every instruction is fetched through cold instruction caches, and a
+  // short call takes longer to fetch straight-line code than to run it.
   auto build_segments = [&](int batch_no) -> int {
     if (tid == 0) {
       *n_segs = 0;
       *first_rank = 0x7fffffff;
     }
-    for (int u = tid; u < n_units; u += kFastThreads) {
-      const int len_u = a.visible_len(u / a.n_kv_heads);
-      u_nst[u] = len_u > 0 ? (len_u + kStageTokens - 1) / kStageTokens : 0;
+    const int per = (n_units + kFastThreads - 1) / kFastThreads, u0 = tid * per;   // this thread's units u0 .. u0 + per - 1
+    long long w_mine = 0;
+    int r_mine = 0;
+#pragma unroll 1
+    for (int i = 0; i < per; ++i) {
+      const int nst = stages_of(u0 + i);
+      w_mine += nst > 0 ? nst + kSegmentCost : 0;
+      r_mine += nst > 0;
+    }
+    long long w_pos = w_mine;   // inclusive scans over the warp, then over the warps
+    int r_pos = r_mine;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long w = __shfl_up_sync(0xffffffffu, w_pos, o);
+      const int r = __shfl_up_sync(0xffffffffu, r_pos, o);
+      if (lane >= o) {
+        w_pos += w;
+        r_pos += r;
+      }
+    }
+    if (lane == 31) {
+      scan_w[warp] = w_pos;
+      scan_r[warp] = r_pos;
     }
     __syncthreads();
     long long w_total = 0;
-    for (int u = 0; u < n_units; ++u) w_total += u_nst[u] > 0 ? u_nst[u] + kSegmentCost : 0;
-    const long long lo = cta * w_total / G, hi = (cta + 1) * w_total / G;
-    // pass 1: parts of every unit; rank (among non-empty units) of the first unit of this CTA
-    for (int u = tid; u < n_units; u += kFastThreads) {
-      int parts = 0;
-      if (u_nst[u] > 0) {
-        long long start = kSegmentCost;  // position of the unit's first stage
-        int rank = 0;
-        for (int v = 0; v < u; ++v) {
-          start += u_nst[v] > 0 ? u_nst[v] + kSegmentCost : 0;
-          rank += u_nst[v] > 0;
-        }
-        const long long end = start + u_nst[u];
-        const int c_first = (int)(((start + 1) * G + w_total - 1) / w_total) - 1;  // CTA whose range holds stage `start`
-        const int c_last = (int)((end * G + w_total - 1) / w_total) - 1;           // ... stage `end - 1`
-        parts = c_last - c_first + 1;
-        if (cta >= c_first && cta <= c_last) {
+    w_pos -= w_mine;   // start of this thread's first unit
+    r_pos -= r_mine;
+#pragma unroll 4
+    for (int w = 0; w < 16; ++w) {
+      w_pos += w < warp ? scan_w[w] : 0;
+      r_pos += w < warp ? scan_r[w] : 0;
+      w_total += scan_w[w];
+    }
+    // positions times G fit 32 bits for all but enormous calls: a 64-bit division costs several times a 32-bit one
+    const bool small = w_total * G < (1ll << 31);
+    auto ratio = [&](long long x, long long y) -> long long { return small ? (long long)((uint32_t)x / (uint32_t)y) : x / y; };
+    // the CTAs c_first .. c_first + parts - 1 share a unit whose first stage has position `start`
+    auto shared_by = [&](long long start, int nst, int* c_first) -> int {
+      *c_first = (int)ratio((start + 1) * G + w_total - 1, w_total) - 1;                 // CTA whose range holds stage `start`
+      return (int)ratio((start + nst) * G + w_total - 1, w_total) - *c_first;            // ... and the one of its last stage
+    };
+    int p_mine = 0, rank = r_pos;
+    long long w_at = w_pos;
+#pragma unroll 1
+    for (int i = 0; i < per; ++i) {
+      const int u = u0 + i, nst = stages_of(u);
+      if (nst > 0) {
+        int c_first;
+        const int parts = shared_by(w_at + kSegmentCost, nst, &c_first);
+        p_mine += parts;
+        if (cta >= c_first && cta < c_first + parts) {
           atomicAdd(n_segs, 1);
           atomicMin(first_rank, rank);
         }
-      } else if (cta == 0 && batch_no == 0) {  // empty sequence: zeros, and the status says so
+        w_at += kSegmentCost + nst;
+        ++rank;
+      } else if (cta == 0 && batch_no == 0 && u < n_units) {  // empty sequence: zeros, and the status says so
         const int b = u / a.n_kv_heads, hk = u - b * a.n_kv_heads;
-        for (int i = 0; i < g_heads * 128; ++i) {
-          const int64_t idx = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128 + i;
+#pragma unroll 1
+        for (int e = 0; e < g_heads * 128; ++e) {
+          const int64_t idx = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128 + e;
           if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
           else reinterpret_cast<float*>(a.out)[idx] = 0.f;
         }
@@ -356,32 +511,41 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
         else
           set_status(a.status, PQ_ERR_EMPTY);
       }
-      u_parts[u] = parts;
     }
+    int p_pos = p_mine;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, p_pos, o);
+      if (lane >= o) p_pos += v;
+    }
+    if (lane == 31) scan_p[warp] = p_pos;
     __syncthreads();
     const int r0 = *first_rank + batch_no * kFastMaxSegs;  // this batch: ranks r0 .. r0 + kFastMaxSegs - 1
-    // pass 2: the units of this batch, in unit order
-    for (int u = tid; u < n_units; u += kFastThreads) {
-      if (u_nst[u] == 0) continue;
-      long long start = kSegmentCost;
-      int rank = 0, slot = 0;
-      for (int v = 0; v < u; ++v) {
-        start += u_nst[v] > 0 ? u_nst[v] + kSegmentCost : 0;
-        rank += u_nst[v] > 0;
-        slot += u_parts[v];
-      }
-      const long long end = start + u_nst[u];
-      const int c_first = (int)(((start + 1) * G + w_total - 1) / w_total) - 1;
-      const int c_last = (int)((end * G + w_total - 1) / w_total) - 1;
-      if (cta >= c_first && cta <= c_last && rank >= r0 && rank < r0 + kFastMaxSegs) {
+    p_pos -= p_mine;
+#pragma unroll 4
+    for (int w = 0; w < 16; ++w) p_pos += w < warp ? scan_p[w] : 0;
+    w_at = w_pos;
+    rank = r_pos;
+#pragma unroll 1
+    for (int i = 0; i < per; ++i) {
+      const int nst = stages_of(u0 + i);
+      if (nst == 0) continue;
+      const long long start = w_at + kSegmentCost, end = start + nst;
+      int c_first;
+      const int parts = shared_by(start, nst, &c_first);
+      if (cta >= c_first && cta < c_first + parts && rank >= r0 && rank < r0 + kFastMaxSegs) {
+        const long long lo = ratio(cta * w_total, G), hi = ratio((cta + 1) * w_total, G);
         Segment& sgm = segs[rank - r0];
-        sgm.unit = u;
+        sgm.unit = u0 + i;
         sgm.st0 = (int)((lo > start ? lo : start) - start);
         sgm.st1 = (int)((hi < end ? hi : end) - start);  // > st0: the CTA's range holds a stage of the unit
         sgm.part = cta - c_first;
-        sgm.n_parts = u_parts[u];
-        sgm.slot0 = slot;  // first partial slot of the unit
+        sgm.n_parts = parts;
+        sgm.slot0 = p_pos;  // first partial slot of the unit
       }
+      p_pos += parts;
+      w_at = end;
+      ++rank;
     }
     __syncthreads();
     return *n_segs;
@@ -459,23 +623,33 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     // The first stages of the segment are already on their way while this runs.
     {
       float* q_in = reinterpret_cast<float*>(smem + kSmQ);
-      __half* q_hi = reinterpret_cast<__half*>(smem + kSmQ + 4096);
-      __half* q_lo = q_hi + 8 * 128;
+      __half* q_hi = reinterpret_cast<__half*>(smem + kSmQ + 4096) + (rot_j >> 5) * (kQQuarter / 2) + (rot_j & 31);
       const int64_t q0 = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128;
       for (int i = tid; i < g_heads * 128; i += kFastThreads)
         q_in[i] = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[q0 + i])
                                               : reinterpret_cast<const float*>(a.q)[q0 + i];
+      if (batch_no + sg > 0) load_s_col();
       __syncthreads();
-      for (int i = tid; i < g_heads * 128; i += kFastThreads) {
-        const float* qrow = q_in + (i & ~127);
-        const float* scol = a.S + (i & 127);
-        float acc = 0.f;
-#pragma unroll 32
-        for (int k = 0; k < 128; ++k) acc = fmaf(qrow[k], __ldg(scol + k * 128), acc);
-        acc *= a.scale * 1.4426950408889634f;
-        const __half qh = __float2half_rn(acc);
-        q_hi[i] = qh;
-        q_lo[i] = __float2half_rn(acc - __half2float(qh));
+#pragma unroll 1
+      for (int h = 0; h < g_heads; ++h) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 qv = *reinterpret_cast<const float4*>(q_in + h * 128 + 16 * i + rot_k);
+          acc[0] = fmaf(qv.x, s_col[4 * i], acc[0]);
+          acc[1] = fmaf(qv.y, s_col[4 * i + 1], acc[1]);
+          acc[2] = fmaf(qv.z, s_col[4 * i + 2], acc[2]);
+          acc[3] = fmaf(qv.w, s_col[4 * i + 3], acc[3]);
+        }
+        float v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v *= a.scale * 1.4426950408889634f;
+        if ((lane & 3) == (h & 3)) {
+          const __half qh = __float2half_rn(v);
+          q_hi[h * (kQHead / 2)] = qh;
+          q_hi[h * (kQHead / 2) + kQLo / 2] = __float2half_rn(v - __half2float(qh));
+        }
       }
       __syncthreads();
     }
@@ -486,7 +660,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
 #pragma unroll
     for (int hg = 0; hg < kHG; ++hg) {
       const int h = (g >> 1) + 4 * hg;
-      const uint2* qsrc = reinterpret_cast<const uint2*>(smem + kSmQ + 4096 + (g & 1) * 2048) + (h * 128 + 32 * c) / 4;
+      const uint2* qsrc = reinterpret_cast<const uint2*>(smem + kSmQ + 4096 + (g & 1) * kQLo + h * kQHead + c * kQQuarter);
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         uint2 v = make_uint2(0u, 0u);
@@ -668,75 +842,82 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     }
     if (g == 0) {
 #pragma unroll
-      for (int hg = 0; hg < kHG; ++hg) {
-        mrg_ml[(warp * 8 + c + 4 * hg) * 2] = m_run[hg];
-        mrg_ml[(warp * 8 + c + 4 * hg) * 2 + 1] = l_run[hg];
-      }
-      if (kHG == 1) {  // heads 4..7 do not exist: neutral entries
-        mrg_ml[(warp * 8 + c + 4) * 2] = -CUDART_INF_F;
-        mrg_ml[(warp * 8 + c + 4) * 2 + 1] = 0.f;
-      }
+      for (int hg = 0; hg < kHG; ++hg)
+        *reinterpret_cast<float2*>(mrg_ml + (warp * 8 + c + 4 * hg) * 2) = make_float2(m_run[hg], l_run[hg]);
     }
+    __syncthreads();
+    // every warp brings its accumulators to the common reference before it hands them over
 #pragma unroll
     for (int hg = 0; hg < kHG; ++hg)
       if (c + 4 * hg < g_heads) {
+        float M = -CUDART_INF_F;
+#pragma unroll
+        for (int w = 0; w < kFastConsumerWarps; ++w) M = fmaxf(M, mrg_ml[(w * 8 + c + 4 * hg) * 2]);
+        const float wgt = m_run[hg] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[hg] - M);
         float* o0 = mrg_o + (warp * 8 + c + 4 * hg) * kMrgStride + g;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          o0[(4 * i) * 8] = o_acc[hg][i][0];
-          o0[(4 * i + 2) * 8] = o_acc[hg][i][1];
-          o0[(4 * i + 1) * 8] = o_acc[hg][i][2];
-          o0[(4 * i + 3) * 8] = o_acc[hg][i][3];
+          o0[(4 * i) * 8] = o_acc[hg][i][0] * wgt;
+          o0[(4 * i + 2) * 8] = o_acc[hg][i][1] * wgt;
+          o0[(4 * i + 1) * 8] = o_acc[hg][i][2] * wgt;
+          o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
         }
       }
-    __syncthreads();
     const int slot = unit_slot + (cta - c_first);
-    for (int idx = tid; idx < g_heads * 128; idx += kFastThreads) {
-      const int h = idx >> 7, j = idx & 127;
-      float M = -CUDART_INF_F;
+    if (tid < g_heads * 16) {   // denominators: 16 lanes per head
+      const int h = tid >> 4;
+      const unsigned half = 0xFFFFu << (lane & 16);
+      const float2 ml = *reinterpret_cast<const float2*>(mrg_ml + ((tid & 15) * 8 + h) * 2);
+      float M = ml.x;
 #pragma unroll
-      for (int w = 0; w < kFastConsumerWarps; ++w) M = fmaxf(M, mrg_ml[(w * 8 + h) * 2]);
-      float lsum = 0.f, acc = 0.f;
+      for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(half, M, o));
+      float l = ml.x == -CUDART_INF_F ? 0.f : ml.y * fast_exp2(ml.x - M);
 #pragma unroll
-      for (int w = 0; w < kFastConsumerWarps; ++w) {
-        const float mw = mrg_ml[(w * 8 + h) * 2];
-        const float wgt = mw == -CUDART_INF_F ? 0.f : exp2f(mw - M);
-        lsum += mrg_ml[(w * 8 + h) * 2 + 1] * wgt;
-        acc += mrg_o[(w * 8 + h) * kMrgStride + (j & 15) * 8 + (j >> 4)] * wgt;
-      }
-      const int64_t pidx = (int64_t)slot * g_heads + h;
-      a.ws.o[pidx * 128 + j] = acc;
-      if (j == 0) {
-        a.ws.ml[2 * pidx] = M;
-        a.ws.ml[2 * pidx + 1] = lsum;
+      for (int o = 8; o > 0; o >>= 1) l += __shfl_xor_sync(half, l, o);
+      if ((tid & 15) == 0) __stcg(reinterpret_cast<float2*>(a.ws.ml) + (int64_t)slot * g_heads + h, make_float2(M, l));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kHG; ++r) {
+      const int idx = tid + r * kFastThreads, h = idx >> 7, j = idx & 127;
+      if (h < g_heads) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int w = 0; w < kFastConsumerWarps; ++w) acc[w & 3] += mrg_o[(w * 8 + h) * kMrgStride + (j & 15) * 8 + (j >> 4)];
+        __stcg(a.ws.o + ((int64_t)slot * g_heads + h) * 128 + j, (acc[0] + acc[1]) + (acc[2] + acc[3]));
       }
     }
-    __threadfence();
     __syncthreads();
-    if (tid == 0) {
-      // Arrival count of the unit's parts.  The workspace is not assumed to start at zero: a ticket
-      // holds (call epoch << 32 | arrivals), and a ticket of another epoch counts as zero arrivals.
+    if (warp == 0) {
+      // Every part raises a flag of its own -- the call's epoch, so nothing in the workspace has to be cleared before the
+      // call -- and then looks at all flags of the unit.  The last one to raise its flag sees them all; if several do, the
+      // first to put the epoch into the unit's election word combines.  (One counter per unit, taken by
+      // compare-and-swap, makes the parts retry on one another: 20 us for the 49 parts of a short two-head call.)  The part
+      // that combines takes flags and election word back, so that a replayed graph, whose calls keep their epochs, starts
+      // without them; a part that meets the word in between combines once more, to the same result.
       bool last = true;
       if (n_parts > 1) {
-        unsigned long long* tk = reinterpret_cast<unsigned long long*>(a.ws.tickets) + u;
-        unsigned long long cur = *reinterpret_cast<volatile unsigned long long*>(tk), want = 0ull;
-        bool done = false;
-        for (int i = 0; i < 4096 && !done; ++i) {  // every failed attempt is another part's success: <= n_parts rounds
-          want = (uint32_t)(cur >> 32) == a.epoch ? cur + 1ull : ((unsigned long long)a.epoch << 32) | 1ull;
-          const unsigned long long prev = atomicCAS(tk, cur, want);
-          done = prev == cur;
-          cur = prev;
-        }
-        if (!done) set_status(a.status, PQ_ERR_TIMEOUT);
-        last = done && (int)(want & 0xffffffffull) == n_parts;
-        if (last) *tk = 0ull;  // no other part of this call touches it any more
+        __threadfence();   // the CTA's partial result (ordered before this by the barrier) before its flag
+        volatile uint32_t* flags = a.ws.flags + unit_slot;
+        if (lane == 0) flags[cta - c_first] = a.epoch;
+        __syncwarp();
+        __threadfence();   // the flag before the look at the others
+        for (int p0 = 0; p0 < n_parts; p0 += 32) last = last && (p0 + lane >= n_parts || flags[p0 + lane] == a.epoch);
+        last = __all_sync(0xffffffffu, last);
+        if (last && lane == 0) last = atomicExch(a.ws.elected + u, a.epoch) != a.epoch;
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last)   // all parts have raised theirs
+          for (int p0 = lane; p0 < n_parts; p0 += 32) flags[p0] = 0u;
       }
-      *is_last = last;
+      if (lane == 0) {
+        __threadfence();
+        *is_last = last;
+      }
     }
     __syncthreads();
     if (*is_last) {
-      __threadfence();
-      combine_and_store(a, b, hk, g_heads, unit_slot, n_parts, reinterpret_cast<float*>(smem + kSmRing));
+      combine_and_store<kHG>(a, b, hk, g_heads, unit_slot, n_parts, reinterpret_cast<float*>(smem + kSmRing));
+      if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
     }
     __syncthreads();  // the ring is free again for the next unit
   }

@@ -103,22 +103,26 @@ __global__ void gen_dequant_kernel(GenConfig g, int n_kv_heads, const float* S, 
   }
 }
 
-// General rows for split_attention_kernel.  Rows are only 2-byte aligned, so a chunk is copied as the 16-byte pieces that
-// lie inside it, to the same position modulo 16 in the buffer, and two ragged ends in 2-byte steps.
-// kSub = min(L, 4): the levels inside a group of 16 coordinates (the angles above it are walked one by one).
-template <int kSub>
+// General rows for split_attention_kernel.  Rows are only 2-byte aligned: a tile is copied as the aligned 16-byte pieces that
+// hold a byte of it, to the same position modulo 16 in the buffer.  (An aligned 16-byte piece never crosses the end of an
+// allocation, so the few bytes beside the tile are readable; they are not used.)
+// kSub = min(L, 4): the levels inside a group of 16 coordinates (the angles above it are walked one by one).  kB: bits per
+// angle where every level has the same number (2, 3 or 4: shifts and masks become constants), 0 for any table.
+template <int kSub, int kB>
 struct GenSplit {
   static constexpr bool kEarlyTables = false;
+  static constexpr int kTabMax = kB ? kGenMaxLevels << kB : kGenMaxCentroids, kDim = 0;
   SplitCommon c;
   GenConfig g;
-  int stage_bytes, n_tab, capacity;
+  int capacity;
   const double* centroids;
   const uint8_t* cache;
   const int32_t* lens;
 
+  int tile_bytes(int n) const { return (n * g.row_bytes + 15 + 8 + 15) & ~15; }   // + the shift, + what a window reads past a row
   __device__ __forceinline__ int len(int pair) const { return max(0, min(lens[pair], capacity)); }
   __device__ __forceinline__ void fill_tables(float2* tab, int tid) const {
-    for (int i = tid; i < g.n_cen; i += kSplitThreads) tab[i] = cos_sin_table(centroids[i]);
+    for (int i = tid; i < g.n_cen; i += blockDim.x) tab[i] = cos_sin_table(centroids[i]);
   }
   __device__ __forceinline__ int64_t row_offset(int pair, int hk, int kv, int t) const {
     return gen_row_offset(g, c.n_kv_heads, capacity, pair, hk, kv, t);
@@ -126,83 +130,86 @@ struct GenSplit {
   __device__ __forceinline__ int shift(int pair, int hk, int kv, int t0) const {
     return (int)((reinterpret_cast<uintptr_t>(cache) + row_offset(pair, hk, kv, t0)) & 15);
   }
-  __device__ __forceinline__ void stage(uint32_t buf, int pair, int hk, int kv, int t0, int n, int tid) const {
+  __device__ __forceinline__ void stage(uint8_t* buf, int pair, int hk, int kv, int t0, int n, int lane) const {
     const uint8_t* src = cache + row_offset(pair, hk, kv, t0);
-    const int bytes = n * g.row_bytes, sh = (int)(reinterpret_cast<uintptr_t>(src) & 15);
-    const int head = min(bytes, (16 - sh) & 15), pieces = (bytes - head) >> 4, tail = head + 16 * pieces;
-    const uint32_t dst = buf + sh;
-    for (int i = tid; i < pieces; i += kSplitThreads) split_cp16(dst + head + 16 * i, src + head + 16 * i);
-    const int ends = (head + bytes - tail) >> 1;   // at most 14
-    if (tid < ends) {
-      const int at = 2 * tid < head ? 2 * tid : tail + 2 * tid - head;
-      asm volatile("st.shared.u16 [%0], %1;" ::"r"(dst + at), "h"(*reinterpret_cast<const uint16_t*>(src + at)) : "memory");
-    }
+    const int sh = (int)(reinterpret_cast<uintptr_t>(src) & 15);
+    src -= sh;
+#pragma unroll 1
+    for (int i = 16 * lane; i < sh + n * g.row_bytes; i += 512) split_cp16(buf + i, src + i);
   }
-  __device__ __forceinline__ int lanes_per_token(int) const { return 1; }
-  // 32 bits of a row from bit `bit` on
-  __device__ __forceinline__ static uint32_t window(uint32_t row, int bit) {
-    const uint32_t at = row + (bit >> 3), al = at & ~3u;
-    return __funnelshift_r(split_lds32(al), split_lds32(al + 4), ((at & 3u) << 3) + (bit & 7));
+  __device__ __forceinline__ int bits(int l) const { return kB ? kB : g.bits[l]; }
+  __device__ __forceinline__ const float2* level(const float2* tab, int l) const { return tab + (kB ? l << kB : g.cen_off[l]); }
+  // 32 bits from bit `bit` of the row at buf + row on
+  __device__ __forceinline__ static uint32_t window(const uint8_t* buf, int row, int bit) {
+    const int at = row + (bit >> 3);
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(buf + (at & ~3));
+    return __funnelshift_r(w[0], w[1], ((at & 3) << 3) + (bit & 7));
   }
-  __device__ __forceinline__ void decode(uint32_t buf, int t, int grp, uint32_t tab, float* y) const {
-    const uint32_t row = buf + t * g.row_bytes;
-    constexpr int kBlk = 16 >> kSub;   // blocks whose radius (or subtree root) starts inside the group
-    float v[16];
-    if (kSub == 4) {
-      float r = __half2float(__ushort_as_half((unsigned short)split_lds16(row + g.rad_off + 2 * (grp >> (g.L - 4)))));
-      for (int l = g.L - 1; l >= 4; --l) {   // the angles above the group
-        const int b = g.bits[l];
-        const uint32_t code = window(row, g.byte_off[l] * 8 + (grp >> (l - 3)) * b) & ((1u << b) - 1u);
-        const float2 cs = split_lds_f2(tab + (g.cen_off[l] + code) * 8);
-        r *= (grp >> (l - 4)) & 1 ? cs.y : cs.x;
+  template <int kU>
+  __device__ __forceinline__ void decode(const uint8_t* buf, int at, int t, int unit, const float2* tab, float* y) const {
+    constexpr int kTop = kU == 16 ? 4 : 3;                 // levels a unit of kU coordinates spans
+    constexpr int kIn = kSub < kTop ? kSub : kTop;         // ... and those of them that exist
+    constexpr int kBlk = kU >> kIn;                        // subtrees whose root starts inside the unit
+    const int row = at + t * g.row_bytes;
+    const __half* radii = reinterpret_cast<const __half*>(buf + row + g.rad_off);
+    float v[kU];
+    if (kIn == kTop) {
+      float r = __half2float(radii[unit >> (g.L - kTop)]);
+      for (int l = g.L - 1; l >= kTop; --l) {   // the angles above the unit
+        const int b = bits(l);
+        const uint32_t code = window(buf, row, g.byte_off[l] * 8 + (unit >> (l + 1 - kTop)) * b) & ((1u << b) - 1u);
+        const float2 cs = level(tab, l)[code];
+        r *= (unit >> (l - kTop)) & 1 ? cs.y : cs.x;
       }
       v[0] = r;
     } else {
 #pragma unroll
       for (int j = 0; j < kBlk; ++j) {
-        const int blk = grp * kBlk + j;
-        v[j] = blk < g.nb ? __half2float(__ushort_as_half((unsigned short)split_lds16(row + g.rad_off + 2 * blk))) : 0.f;
+        const int blk = unit * kBlk + j;
+        v[j] = blk < g.nb ? __half2float(radii[blk]) : 0.f;
       }
     }
 #pragma unroll
-    for (int l = kSub - 1; l >= 0; --l) {
-      const int n = 8 >> l, b = g.bits[l], bit = g.byte_off[l] * 8 + grp * n * b;   // n angles of the level in the group
-      const uint32_t mask = (1u << b) - 1u, entry = tab + g.cen_off[l] * 8;
-      uint32_t w = window(row, bit), w2 = 0u;
-      if (n == 8) w2 = b <= 4 ? w >> (4 * b) : window(row, bit + 4 * b);   // 8 codes of up to 6 bits
+    for (int l = kIn - 1; l >= 0; --l) {
+      constexpr int kAngles = kU / 2;
+      const int n = kAngles >> l, b = bits(l), bit = g.byte_off[l] * 8 + unit * n * b;   // n angles of the level in the unit
+      const uint32_t mask = (1u << b) - 1u;
+      const float2* entry = level(tab, l);
+      const uint32_t w = window(buf, row, bit);
+      uint32_t w2 = 0u;
+      if (n == 8) w2 = b <= 4 ? w >> (4 * b) : window(buf, row, bit + 4 * b);   // 8 codes of up to 6 bits
 #pragma unroll
       for (int j = n - 1; j >= 0; --j) {
-        const uint32_t code = ((j < 4 ? w : w2) >> ((j & 3) * b)) & mask;
-        const float2 cs = split_lds_f2(entry + code * 8);
+        const float2 cs = entry[((j < 4 ? w : w2) >> ((j & 3) * b)) & mask];
         const float r = v[j];
         v[2 * j] = r * cs.x;
         v[2 * j + 1] = r * cs.y;
       }
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) y[i] = v[i];
+    for (int i = 0; i < kU; ++i) y[i] = v[i];
   }
 };
 
-template <int kSub>
-static int32_t launch_gen_attention(const GenConfig& g, SplitCommon c, int batch, int capacity, const double* centroids,
-                                    const void* cache, const int32_t* lens, cudaStream_t stream) {
-  GenSplit<kSub> p;
-  p.g = g; p.capacity = capacity; p.centroids = centroids; p.cache = reinterpret_cast<const uint8_t*>(cache); p.lens = lens;
-  p.n_tab = (g.n_cen + 1) & ~1;
-  const int grp = c.n_q_heads / c.n_kv_heads, kh = grp <= 1 ? 1 : grp <= 2 ? 2 : grp <= 4 ? 4 : 8;
-  // chunk: two tokens per thread, as long as two staging buffers stay within 64 KB
-  int chunk = 512;
-  while (chunk > 64 && chunk * g.row_bytes > 32 * 1024) chunk >>= 1;
-  c.chunk = chunk;
-  p.c = c;
-  p.stage_bytes = (chunk * g.row_bytes + 16 + 8 + 15) & ~15;   // + the shift, + what a window reads past the last row
-  const int smem = split_smem_bytes(g.d, kh, p.n_tab, chunk, p.stage_bytes);
-  switch (kh) {
-    case 1: return launch_split_attention<GenSplit<kSub>, 1>(p, batch, capacity, smem, stream);
-    case 2: return launch_split_attention<GenSplit<kSub>, 2>(p, batch, capacity, smem, stream);
-    case 4: return launch_split_attention<GenSplit<kSub>, 4>(p, batch, capacity, smem, stream);
-    default: return launch_split_attention<GenSplit<kSub>, 8>(p, batch, capacity, smem, stream);
+template <int kSub, int kB>
+static int32_t launch_gen_attention_as(const GenConfig& g, const SplitCommon& c, int batch, int capacity, const double* centroids,
+                                       const void* cache, const int32_t* lens, cudaStream_t stream) {
+  GenSplit<kSub, kB> p;
+  p.c = c; p.g = g; p.capacity = capacity; p.centroids = centroids; p.cache = reinterpret_cast<const uint8_t*>(cache); p.lens = lens;
+  return dispatch_split_attention(p, batch, capacity, stream);
+}
+static int32_t launch_gen_attention(const GenConfig& g, const SplitCommon& c, int batch, int capacity, const double* centroids,
+                                    const void* cache, const int32_t* lens, cudaStream_t s) {
+  bool same = true;
+  for (int l = 1; l < g.L; ++l) same = same && g.bits[l] == g.bits[0];
+  if (g.L >= 4 && same && g.bits[0] == 2) return launch_gen_attention_as<4, 2>(g, c, batch, capacity, centroids, cache, lens, s);
+  if (g.L >= 4 && same && g.bits[0] == 3) return launch_gen_attention_as<4, 3>(g, c, batch, capacity, centroids, cache, lens, s);
+  if (g.L >= 4 && same && g.bits[0] == 4) return launch_gen_attention_as<4, 4>(g, c, batch, capacity, centroids, cache, lens, s);
+  switch (g.L < 4 ? g.L : 4) {
+    case 1: return launch_gen_attention_as<1, 0>(g, c, batch, capacity, centroids, cache, lens, s);
+    case 2: return launch_gen_attention_as<2, 0>(g, c, batch, capacity, centroids, cache, lens, s);
+    case 3: return launch_gen_attention_as<3, 0>(g, c, batch, capacity, centroids, cache, lens, s);
+    default: return launch_gen_attention_as<4, 0>(g, c, batch, capacity, centroids, cache, lens, s);
   }
 }
 
@@ -345,15 +352,10 @@ int32_t pq_general_decode_attention(const pq_general_config* cfg, int32_t n_q_he
   if (io_dtype != PQ_DTYPE_F32 && io_dtype != PQ_DTYPE_BF16) return PQ_ERR_UNSUPPORTED;
   if (((uintptr_t)centroids_dev & 7) || ((uintptr_t)cache_dev & 1)) return PQ_ERR_ALIGNMENT;
   pq::SplitCommon c;
-  c.d = g.d; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.chunk = 0; c.scale = scale;
+  c.d = g.d; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
   c.S = S_dev; c.q = q_dev; c.out = out_dev; c.lse = nullptr; c.status = status_dev;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  switch (g.L < 4 ? g.L : 4) {
-    case 1: return pq::launch_gen_attention<1>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
-    case 2: return pq::launch_gen_attention<2>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
-    case 3: return pq::launch_gen_attention<3>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
-    default: return pq::launch_gen_attention<4>(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev, s);
-  }
+  return pq::launch_gen_attention(g, c, batch, capacity, centroids_dev, cache_dev, cache_lens_dev,
+                                  reinterpret_cast<cudaStream_t>(stream));
 }
 
 int32_t pq_general_unpack_codes(const pq_general_config* cfg, int32_t n_kv_heads, const void* cache_dev, int32_t batch,

@@ -1,31 +1,39 @@
 // Decode attention in float32 over any packed layout (included by pq_decode.cu and pq_general.cu): one cluster of
-// thread blocks per (kv head, sequence), the tokens cut into one contiguous range per block of the cluster.
+// thread blocks per (kv head, sequence), every warp of the cluster an independent stream of small token tiles.
 //
-// A block keeps a chunk of packed keys and values in shared memory (16-byte cp.async, the next chunk's copies in flight
-// while the current one is used) and works on "groups" of 16 coordinates:
-//   * scores: thread = (token, group or several groups); the 16 coordinates are decoded into registers and multiplied
-//     into the group's query heads there (packed float32 multiply-adds), partial scores meet in shuffles;
-//   * softmax: a warp per head, once per chunk (log2 domain);
-//   * values: warp = group, lane = token; every thread accumulates heads x 16 coordinates of its own tokens in registers,
-//     and the 32 lanes are summed once per chunk by halving exchanges.
-// No decoded coordinate is ever stored: per token and kv head the work is the angle lookups (one 8-byte (cos, sin) entry
-// each), two multiplications per angle and 2 x heads x d multiply-adds.
-// The blocks of a cluster share the rotation of the query (each forms d / C coordinates of q' = q S and sends them to
-// the others), merge their partial softmaxes through distributed shared memory, and each un-rotates d / C coordinates
-// of the output.  So a call is one launch and needs no scratch in global memory.
-// Bound by instruction issue (angle decode); the figures are beside the launch code of the two layouts.
+// A lane owns kU consecutive coordinates of the head (its "unit") for the whole call: its share of the rotated queries and
+// of the output accumulators stay in registers, and d / kU neighbouring lanes work on one token.  Per token of a tile a lane
+// decodes its unit of the key (one 8-byte (cos, sin) lookup per angle, two multiplications), multiplies it into the
+// group's query heads (packed float32 multiply-adds), the lanes of the token sum their partial scores, and the decoded
+// unit of the value is accumulated with p = 2^(score - m).  m moves lazily: only when a score exceeds it by more than 8
+// (log2 units) are the accumulators rescaled.  Units lie side by side in the packed rows, so neighbouring lanes read
+// neighbouring bytes.  Tiles of 16 tokens (32 at head_dim 16) go round the warps of the cluster, so a short context
+// spreads over all of them; each warp copies its own tiles (16-byte cp.async, three ahead), and nothing in the loop
+// waits for another warp.
+// The warps of a block merge in shared memory, the blocks of the cluster through distributed shared memory, and each
+// block un-rotates d / C coordinates of the output: one launch, no scratch in global memory.
+// Bound by instruction issue (angle decode) for long sequences and by the chain of phases for short ones, hence: S is copied
+// to shared memory (head dims up to 128) before the kernel ahead in the stream has finished, every block rotates the
+// whole query by itself instead of meeting the others first, and the merge has one cluster barrier.
+// kU = 16 for up to four query heads per kv head, 8 for up to eight (the registers of q' and of the accumulators).
 #pragma once
+#include <cstdint>
 
 namespace pq {
 
-constexpr int kSplitThreads = 256;
-constexpr int kSplitWarps = kSplitThreads / 32;
-constexpr int kGroupStride = 20;  // floats between the 16-coordinate groups of q': eight groups start in eight bank quads
+// Warps of a block.  With four or eight query heads q' and the accumulators take 128 registers and the loop is bound by the
+// latency of a warp's own chain: two warps per scheduler with 255 registers (31.6 us for 64 units of 2048 tokens at
+// head_dim 128, four heads; three warps with 168 and a few spills 39 us, four with half units 32.3 us).  With one or two
+// heads four warps per scheduler fit (19.0 us against 20.0 with three and 22.6 with two; head_dim 64, two heads).
+__host__ __device__ constexpr int split_warps(int kh) { return kh <= 2 ? 16 : 8; }
+constexpr int kSplitStages = 4;            // tiles in flight per warp
+constexpr int kSplitSmemMax = 216 * 1024;
+constexpr int kUnitStride = 20;            // floats between the 16-coordinate groups of q' in shared memory
 
 // What the kernel needs beside the layout.
 struct SplitCommon {
   int d, n_q_heads, n_kv_heads, io_dtype;
-  int chunk;   // tokens staged at a time (a multiple of 64)
+  int tile, stage_bytes;   // tokens of a tile, bytes of its staged keys (or values): set by dispatch_split_attention
   float scale;
   const float* S;
   const void* q;
@@ -34,15 +42,20 @@ struct SplitCommon {
   int32_t* status;
 };
 
-constexpr int kSplitSmemMax = 200 * 1024;
-
-__host__ __device__ inline int split_groups(int d) { return d < 16 ? 1 : d / 16; }
-// Shared memory of a block in bytes: tables, q', scores, partial sums, three [heads][d] vectors, running (m, l, corr),
-// the two staging buffers.
-__host__ __device__ inline int split_smem_bytes(int d, int kh, int n_tab, int chunk, int stage_bytes) {
-  const int ng = split_groups(d);
-  const int floats = 2 * n_tab + kh * ng * kGroupStride + chunk * kh + kSplitThreads * kh + 3 * kh * 16 * ng + 4 * kh;
-  return ((floats * 4 + 15) & ~15) + 2 * stage_bytes;
+__host__ __device__ constexpr int split_heads(int g) { return g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : 8; }   // heads a block is built for
+__host__ __device__ constexpr int split_unit(int kh) { return kh == 8 ? 8 : 16; }
+__host__ __device__ inline int split_lanes(int d, int kh) { return d < split_unit(kh) ? 1 : d / split_unit(kh); }   // per token
+__host__ __device__ inline int split_pad(int d) { return d < 16 ? 16 : d; }
+// Dynamic shared memory: q', the query and partial sums of q', (m, l) of the warps, the block's output, m and l and the merged output, then the
+// tiles in flight, whose place the warps' outputs take at the end.
+__host__ __device__ inline int split_fixed_bytes(int d, int kh) {
+  const int dp = split_pad(d);
+  return (4 * (kh * dp / 16 * kUnitStride + 3 * kh * dp + 34 * split_warps(kh) * kh + 2 * kh) + 15) & ~15;
+}
+__host__ __device__ inline int split_s_bytes(int d) { return d <= 128 ? (d * d * 4 + 15) & ~15 : 0; }   // S, where it fits
+__host__ __device__ inline int split_smem_bytes(int d, int kh, int stage_bytes) {
+  const int ring = split_warps(kh) * kSplitStages * 2 * stage_bytes, merge = split_warps(kh) * kh * split_pad(d) * 4;
+  return split_fixed_bytes(d, kh) + split_s_bytes(d) + (ring > merge ? ring : merge);
 }
 
 __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
@@ -55,102 +68,94 @@ __device__ __forceinline__ float cluster_ld(uint32_t addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
   return v;
 }
-__device__ __forceinline__ void cluster_st(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+__device__ __forceinline__ float4 cluster_ld4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
 }
-__device__ __forceinline__ void split_cp16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+__device__ __forceinline__ void split_cp16(uint8_t* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void split_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int kPending>
 __device__ __forceinline__ void split_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
 }
-__device__ __forceinline__ uint32_t split_lds32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ float2 split_lds_f2(uint32_t addr) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ uint32_t split_lds16(uint32_t addr) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ uint32_t split_lds8(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
+__device__ __forceinline__ float split_exp2(float x) {   // relative error 2^-22, 2^-inf = 0
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// Sum of v[0 .. kN) over the 32 lanes by halving exchanges: lane L ends with the kN / 32 sums from L * kN / 32 on in
-// v[0 ..] (kN = 16: lanes 2 i and 2 i + 1 both with sum i).  The order of the additions is fixed.
-template <int kN>
-__device__ __forceinline__ void lane_sums(float* v, int lane) {
-  int half = kN / 2;
+// Sum of v[0 .. kN) over the lanes that own the same unit (lanes L, L + kLanes, ...): halving exchanges while the count
+// is even, so that such a lane ends with kN / (32 / kLanes) of the sums, from (L / kLanes) * that on; *from is the index
+// of the first.  The order of the additions is fixed.
+template <int kN, int kLanes>
+__device__ __forceinline__ void unit_lane_sums(float* v, int lane, int* from, int* count) {
+  int n = kN, at = 0;
 #pragma unroll
-  for (int mask = 16; mask >= 1; mask >>= 1) {
-    if (half >= 1) {
+  for (int mask = 16; mask >= kLanes; mask >>= 1) {
+    if (n > 1) {
       const bool up = lane & mask;
+      n >>= 1;
 #pragma unroll
       for (int i = 0; i < kN / 2; ++i)
-        if (i < half) v[i] = (up ? v[i + half] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + half], mask);
-      half >>= 1;
+        if (i < n) v[i] = (up ? v[i + n] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + n], mask);
+      at += up ? n : 0;
     } else {
       v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
     }
   }
+  *from = at;
+  *count = n;
 }
 
 // Layout policies (template parameter P, passed by value) provide
 //   SplitCommon c;
-//   int stage_bytes                   size of a staging buffer (keys or values of a chunk)
+//   int tile_bytes(n)                 bytes of n staged tokens of keys (or values)
 //   int len(pair)                     tokens the pair's query sees
-//   int n_tab                         entries of the (cos, sin) table (even)
-//   void fill_tables(tab, tid)        kEarlyTables: before the kernel ahead in the stream has finished (it may not write them)
-//   void stage(buf, pair, hk, kv, t0, n, tid)   issue the copies of the keys (kv = 0) or values (1) of tokens t0 .. t0 + n - 1
-//   int shift(pair, hk, kv, t0)       where in the buffer the chunk that starts at token t0 begins
-//   int lanes_per_token(ng)           least number of lanes that should share a token in the score phase
-//   void decode(buf, t, g, tab, y)    16 rotated coordinates of group g of the chunk's token t
+//   kTabMax, fill_tables(tab, tid)    the (cos, sin) table; kEarlyTables: filled before the kernel ahead in the stream has
+//                                     finished (it may not write them)
+//   kDim                              head_dim where it is a compile-time constant, else 0
+//   void stage(buf, pair, hk, kv, t0, n, lane)  issue a warp's copies of the keys (kv = 0) or values (1) of tokens
+//                                     t0 .. t0 + n - 1 (n = tile size, or less in the last tile)
+//   int shift(pair, hk, kv, t0)       where in the buffer the tile that starts at token t0 begins
+//   void decode<kU>(buf, at, t, unit, tab, y)   the coordinates of a unit of token t of the tile at buf + at
 template <class P, int kH>
-__global__ void __launch_bounds__(kSplitThreads, kH == 8 ? 1 : 2) split_attention_kernel(const __grid_constant__ P p) {
+__global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kernel(const __grid_constant__ P p) {
+  constexpr int kU = split_unit(kH), kSplitWarps = split_warps(kH), kSplitThreads = 32 * kSplitWarps;
   extern __shared__ __align__(16) uint8_t split_smem[];
+  __shared__ float2 tab[P::kTabMax];   // at a fixed address: a lookup's offset needs no addition
   const SplitCommon& c = p.c;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int C = gridDim.x, rank = blockIdx.x, hk = blockIdx.y, pair = blockIdx.z;   // the cluster spans the x dimension
-  const int d = c.d, ng = split_groups(d), dp = 16 * ng, grp = c.n_q_heads / c.n_kv_heads;
-  float2* tab = reinterpret_cast<float2*>(split_smem);
-  float* qg = reinterpret_cast<float*>(tab + p.n_tab);   // [kH][ng * kGroupStride]
-  float* sc = qg + kH * ng * kGroupStride;                 // [chunk][kH]
-  float* part = sc + c.chunk * kH;                         // [kSplitThreads * kH]
-  float* o_sm = part + kSplitThreads * kH;                 // [kH][dp]
-  float* y_sm = o_sm + kH * dp;                            // [kH][dp]
-  float* q_in = y_sm + kH * dp;                            // [kH][dp]
-  float* m_sm = q_in + kH * dp;                            // [kH] running maximum, [kH] denominator, [kH] rescale
-  float* l_sm = m_sm + kH;
-  float* corr_sm = l_sm + kH;
-  const uint32_t tab_s = (uint32_t)__cvta_generic_to_shared(split_smem);
-  const int head_floats = (int)(corr_sm + 2 * kH - reinterpret_cast<float*>(split_smem));
-  const uint32_t kbuf = tab_s + ((head_floats * 4 + 15) & ~15), vbuf = kbuf + p.stage_bytes;
+  const int d = P::kDim ? P::kDim : c.d, dp = split_pad(d), grp = c.n_q_heads / c.n_kv_heads;
+  const int lanes = split_lanes(d, kH), T = c.tile, qs = dp / 16 * kUnitStride;
+  float* qg = reinterpret_cast<float*>(split_smem);   // [kH][dp / 16][kUnitStride]
+  float* q_in = qg + kH * qs;                         // [kH][dp]
+  float* o_sm = q_in + kH * dp;                       // [kH][dp] this block's output (relative to m_sm)
+  float* y_sm = o_sm + kH * dp;                       // [kH][dp] merged output
+  float* rot_sm = y_sm + kH * dp;                     // [kSplitThreads * kH] partial sums of q'
+  float* wm_sm = rot_sm + kSplitThreads * kH;         // [warps][kH]
+  float* wl_sm = wm_sm + kSplitWarps * kH;            // [warps][kH]
+  float* m_sm = wl_sm + kSplitWarps * kH;             // [kH]
+  float* l_sm = m_sm + kH;                            // [kH]
+  float* S_sm = reinterpret_cast<float*>(split_smem + split_fixed_bytes(d, kH));   // [d][d], or nothing
+  uint8_t* ring = split_smem + split_fixed_bytes(d, kH) + split_s_bytes(d);
+  float* w_out = reinterpret_cast<float*>(ring);      // [warps][kH][dp], after the loop
+  uint8_t* mine = ring + warp * (kSplitStages * 2 * c.stage_bytes);
 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool s_staged = d <= 128 && d >= 4 && (reinterpret_cast<uintptr_t>(c.S) & 15) == 0;
+  if (s_staged) {
+#pragma unroll 2
+    for (int i = 4 * tid; i < d * d; i += 4 * kSplitThreads) split_cp16(reinterpret_cast<uint8_t*>(S_sm + i), c.S + i);
+  }
+  split_commit();
   if (P::kEarlyTables) p.fill_tables(tab, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // lengths, cache and queries may come from the kernel before this one
-  const int len = p.len(pair);
-  const int per = ((len + C - 1) / C + 63) & ~63;
-  const int t_first = min(len, rank * per), n_mine = min(len, t_first + per) - t_first;
-  if (n_mine > 0) p.stage(kbuf, pair, hk, 0, t_first, min(n_mine, c.chunk), tid);
-  split_commit();
-  if (n_mine > 0) p.stage(vbuf, pair, hk, 1, t_first, min(n_mine, c.chunk), tid);
-  split_commit();
-  if (!P::kEarlyTables) p.fill_tables(tab, tid);
-
-  // ---- q' = q S * scale * log2(e): this block's d / C columns, sent to every block of the cluster
   const int64_t q0 = ((int64_t)pair * c.n_q_heads + hk * grp) * d;
+  const int len = p.len(pair);
   for (int i = tid; i < kH * dp; i += kSplitThreads) {
     const int h = i / dp, k = i - h * dp;
     float v = 0.f;
@@ -158,256 +163,341 @@ __global__ void __launch_bounds__(kSplitThreads, kH == 8 ? 1 : 2) split_attentio
       v = c.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(c.q)[q0 + h * d + k])
                                       : reinterpret_cast<const float*>(c.q)[q0 + h * d + k];
     q_in[i] = v;
-    o_sm[i] = 0.f;
+    if (d < 16) qg[h * qs + k] = 0.f;   // coordinates past d
   }
-  for (int i = tid; i < kH * ng * kGroupStride; i += kSplitThreads)   // coordinates past d (head dims below 16) stay zero
-    if (d < 16) qg[i] = 0.f;
-  if (tid < kH) {
-    m_sm[tid] = -CUDART_INF_F;
-    l_sm[tid] = 0.f;
-  }
-  cluster_arrive();   // (A) every block of the cluster runs and has cleared its q'; waited for before the first remote store
+  // tiles of this warp: worker, worker + workers, ...; consecutive tiles go to different blocks first.  Where there are
+  // fewer tiles than warps, `share` warps take a tile together, each every share-th pass over it.
+  const int n_tiles = (len + T - 1) / T, per_pass = 32 / lanes;   // tokens side by side in a warp
+  int share = 1;
+  while (2 * share * n_tiles <= C * kSplitWarps && 2 * share * per_pass <= T) share *= 2;
+  const int worker = (warp * C + rank) / share, sub = (warp * C + rank) - worker * share, workers = C * kSplitWarps / share;
+  auto stage = [&](int i) {
+    const int tile = worker + i * workers;
+    if (tile < n_tiles && worker < workers) {
+      uint8_t* buf = mine + (i % kSplitStages) * 2 * c.stage_bytes;
+      p.stage(buf, pair, hk, 0, tile * T, min(T, len - tile * T), lane);
+      p.stage(buf + c.stage_bytes, pair, hk, 1, tile * T, min(T, len - tile * T), lane);
+    }
+    split_commit();
+  };
+#pragma unroll 1
+  for (int i = 0; i < kSplitStages - 1; ++i) stage(i);
+  if (!P::kEarlyTables) p.fill_tables(tab, tid);
+
+  // ---- q' = q S * scale * log2(e): thread = column tid % d of one of `parts` slices of the sum
+  split_wait<kSplitStages - 1>();   // S has landed (the tiles are younger)
   __syncthreads();
-  const int nc = d / C, j0 = rank * nc, kparts = kSplitThreads / nc;   // C divides d
-  {
-    const int cc = tid % nc, kp = tid / nc;
+  const int parts = max(1, kSplitThreads / d), rot_j = tid % d, rot_k = tid / d;   // threads past parts * d idle
+  const int slice = ((d + parts - 1) / parts + 3) & ~3, k_end = min(d, (rot_k + 1) * slice);
+  if (rot_k < parts) {
     float acc[kH];
 #pragma unroll
     for (int h = 0; h < kH; ++h) acc[h] = 0.f;
-    for (int k = kp; k < d; k += kparts) {
-      const float s = __ldg(c.S + (int64_t)k * d + j0 + cc);
+    if (s_staged) {
+#pragma unroll 1
+      for (int k = rot_k * slice; k < k_end; k += 4) {
+        float s[4];
 #pragma unroll
-      for (int h = 0; h < kH; ++h) acc[h] = fmaf(q_in[h * dp + k], s, acc[h]);
+        for (int e = 0; e < 4; ++e) s[e] = S_sm[(k + e) * d + rot_j];
+#pragma unroll
+        for (int h = 0; h < kH; ++h) {
+          const float4 q4 = *reinterpret_cast<const float4*>(q_in + h * dp + k);
+          acc[h] = fmaf(q4.w, s[3], fmaf(q4.z, s[2], fmaf(q4.y, s[1], fmaf(q4.x, s[0], acc[h]))));
+        }
+      }
+    } else {
+#pragma unroll 8
+      for (int k = rot_k * slice; k < k_end; ++k) {
+        const float s = __ldg(c.S + (int64_t)k * d + rot_j);
+#pragma unroll
+        for (int h = 0; h < kH; ++h) acc[h] = fmaf(q_in[h * dp + k], s, acc[h]);
+      }
     }
 #pragma unroll
-    for (int h = 0; h < kH; ++h) part[(kp * nc + cc) * kH + h] = acc[h];
+    for (int h = 0; h < kH; ++h) rot_sm[(rot_k * kH + h) * d + rot_j] = acc[h];
   }
-  cluster_wait();   // (A)
   __syncthreads();
-  for (int i = tid; i < nc * kH; i += kSplitThreads) {
-    const int cc = i / kH, h = i - cc * kH, j = j0 + cc;
-    float v = 0.f;
-    const int n_kp = min(kparts, d);
-    for (int kp = 0; kp < n_kp; ++kp) v += part[(kp * nc + cc) * kH + h];
-    v *= c.scale * 1.4426950408889634f;
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(qg + h * ng * kGroupStride + (j >> 4) * kGroupStride + (j & 15));
-    for (int r = 0; r < C; ++r) cluster_st(cluster_map(dst, r), v);
+#pragma unroll 1
+  for (int i = tid; i < kH * d; i += kSplitThreads) {
+    float v = rot_sm[i];
+#pragma unroll 2
+    for (int r = 1; r < parts; ++r) v += rot_sm[r * kH * d + i];
+    const int h = i / d, j = i - h * d;
+    qg[h * qs + (j >> 4) * kUnitStride + (j & 15)] = v * (c.scale * 1.4426950408889634f);
   }
-  cluster_arrive();   // (B) q' is complete everywhere
-  cluster_wait();
+  __syncthreads();
 
-  // ---- chunks of this block's tokens
-  const int n_slice = ng < kSplitWarps ? kSplitWarps / ng : 1;
-  const uint32_t qg_s = (uint32_t)__cvta_generic_to_shared(qg);
-  for (int c0 = 0; c0 < n_mine; c0 += c.chunk) {
-    const int n = min(c.chunk, n_mine - c0), t0 = t_first + c0, n_next = min(c.chunk, n_mine - c0 - c.chunk);
-    split_wait<1>();   // the keys have landed (the values are the younger group)
-    __syncthreads();
-    {
-      // scores: gs consecutive lanes share a token; more of them when there are few tokens
-      const uint32_t kb = kbuf + p.shift(pair, hk, 0, t0);
-      int gs = p.lanes_per_token(ng);
-      while (gs < ng && n * gs < 2 * kSplitThreads) gs <<= 1;
-      const int gs_log = 31 - __clz(gs);
-      for (int i0 = 0; i0 < (n << gs_log); i0 += kSplitThreads) {
-        const int t = (i0 + tid) >> gs_log, g0 = (i0 + tid) & (gs - 1);
-        uint64_t s2[kH];
+  // ---- the stream of this warp
+  const int unit = lane & (lanes - 1);   // this lane's unit
+  uint64_t q2[kH][kU / 2], acc[kH][kU / 2];
+  float m_run[kH], l_run[kH];   // running reference of every head (the same in all lanes), this lane's share of the denominator
 #pragma unroll
-        for (int h = 0; h < kH; ++h) s2[h] = 0ull;
-        if (t < n)
-          for (int g = g0; g < ng; g += gs) {
-            float y[16];
-            p.decode(kb, t, g, tab_s, y);
+  for (int h = 0; h < kH; ++h) {
+    m_run[h] = -CUDART_INF_F;
+    l_run[h] = 0.f;
+    const float* src = qg + h * qs + (unit * kU >> 4) * kUnitStride + (unit * kU & 15);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint64_t ya = f2_pack(y[4 * i], y[4 * i + 1]), yb = f2_pack(y[4 * i + 2], y[4 * i + 3]);
+    for (int i = 0; i < kU / 4; ++i) {
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(src + 4 * i);
+      q2[h][2 * i] = w.x;
+      q2[h][2 * i + 1] = w.y;
+    }
 #pragma unroll
-              for (int h = 0; h < kH; ++h) {
-                uint64_t qa, qb;
-                asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];"
-                             : "=l"(qa), "=l"(qb)
-                             : "r"(qg_s + ((h * ng + g) * kGroupStride + 4 * i) * 4));
-                s2[h] = f2_fma(ya, qa, s2[h]);
-                s2[h] = f2_fma(yb, qb, s2[h]);
-              }
-            }
-          }
+    for (int i = 0; i < kU / 2; ++i) acc[h][i] = 0ull;
+  }
+  int n_mine = 0;
+#pragma unroll 1
+  for (int tile = worker; tile < n_tiles && worker < workers; tile += workers, ++n_mine) {
+    split_wait<kSplitStages - 2>();
+    __syncwarp();
+    const uint8_t* kbuf = mine + (n_mine % kSplitStages) * 2 * c.stage_bytes;
+    const uint8_t* vbuf = kbuf + c.stage_bytes;
+    const int t0 = tile * T, n = min(T, len - t0);
+    const int at_k = p.shift(pair, hk, 0, t0), at_v = p.shift(pair, hk, 1, t0);
+#pragma unroll 1
+    for (int tb = sub * per_pass; tb < n; tb += share * per_pass) {
+      const int tt = tb + lane / lanes, t = min(tt, n - 1);   // past the end: the last token again, with weight 0
+      float y[kU];
+      p.template decode<kU>(kbuf, at_k, t, unit, tab, y);
+      float s[kH];
+#pragma unroll
+      for (int h = 0; h < kH; ++h) {
+        uint64_t s2 = 0ull;
+#pragma unroll
+        for (int i = 0; i < kU / 2; ++i) s2 = f2_fma(f2_pack(y[2 * i], y[2 * i + 1]), q2[h][i], s2);
+        float a, b;
+        f2_unpack(s2, a, b);
+        s[h] = a + b;
+      }
+      for (int m = 1; m < lanes; m <<= 1)
+#pragma unroll
+        for (int h = 0; h < kH; ++h) s[h] += __shfl_xor_sync(0xffffffffu, s[h], m);
+      bool over = false;
+#pragma unroll
+      for (int h = 0; h < kH; ++h) {
+        if (tt >= n) s[h] = -CUDART_INF_F;
+        over = over || s[h] > m_run[h] + 8.f;
+      }
+      if (__any_sync(0xffffffffu, over)) {
 #pragma unroll
         for (int h = 0; h < kH; ++h) {
-          float a, b;
-          f2_unpack(s2[h], a, b);
-          float s = a + b;
-          for (int m = 1; m < gs; m <<= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-          if (t < n && g0 == 0) sc[t * kH + h] = s;
+          float mx = s[h];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          const float m_new = fmaxf(m_run[h], mx);   // finite: the tile has a token
+          const float k = split_exp2(m_run[h] - m_new);   // 0 at first
+          m_run[h] = m_new;
+          l_run[h] *= k;
+          const uint64_t kk = f2_pack(k, k);
+#pragma unroll
+          for (int i = 0; i < kU / 2; ++i) acc[h][i] = f2_mul(acc[h][i], kk);
         }
       }
-    }
-    __syncthreads();
-    // the keys have been used: the next chunk's keys may arrive
-    if (n_next > 0) p.stage(kbuf, pair, hk, 0, t0 + c.chunk, n_next, tid);
-    split_commit();
-    if (warp < kH) {
-      const int h = warp;
-      float mx = -CUDART_INF_F;
-      for (int t = lane; t < n; t += 32) mx = fmaxf(mx, sc[t * kH + h]);
+      p.template decode<kU>(vbuf, at_v, t, unit, tab, y);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_old = m_sm[h], m_new = fmaxf(m_old, mx);
-      float sum = 0.f;
-      for (int t = lane; t < n; t += 32) {
-        const float e = exp2f(sc[t * kH + h] - m_new);
-        sc[t * kH + h] = e;
-        sum += e;
-      }
+      for (int h = 0; h < kH; ++h) {
+        const float e = split_exp2(s[h] - m_run[h]);
+        l_run[h] += e;
+        const uint64_t ee = f2_pack(e, e);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      __syncwarp();
-      if (lane == 0) {
-        const float corr = exp2f(m_old - m_new);   // 0 on the first chunk
-        corr_sm[h] = corr;
-        l_sm[h] = l_sm[h] * corr + sum;
-        m_sm[h] = m_new;
+        for (int i = 0; i < kU / 2; ++i) acc[h][i] = f2_fma(ee, f2_pack(y[2 * i], y[2 * i + 1]), acc[h][i]);
       }
     }
-    split_wait<1>();   // the values have landed
-    __syncthreads();
-    const uint32_t vb = vbuf + p.shift(pair, hk, 1, t0);
-    for (int g = ng < kSplitWarps ? warp % ng : warp; g < ng; g += kSplitWarps) {
-      const int slice = ng < kSplitWarps ? warp / ng : 0;
-      uint64_t acc[kH][8];
+    __syncwarp();
+    stage(n_mine + kSplitStages - 1);
+  }
+  // ---- merge the warps: bring every warp to the block's reference, then add
+  float mb[kH];
 #pragma unroll
-      for (int h = 0; h < kH; ++h)
+  for (int h = 0; h < kH; ++h)
+    for (int m = lanes; m < 32; m <<= 1) l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], m);
+  if (lane == 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[h][i] = 0ull;
-      for (int t = lane + 32 * slice; t < n; t += 32 * n_slice) {
-        float y[16];
-        p.decode(vb, t, g, tab_s, y);
-        float pr[kH];
-        if (kH >= 4) {
-#pragma unroll
-          for (int h = 0; h < kH / 4; ++h) {
-            const float4 p4 = *reinterpret_cast<const float4*>(sc + t * kH + 4 * h);
-            pr[4 * h] = p4.x; pr[(4 * h + 1) % kH] = p4.y; pr[(4 * h + 2) % kH] = p4.z; pr[(4 * h + 3) % kH] = p4.w;
-          }
-        } else {
-#pragma unroll
-          for (int h = 0; h < kH; ++h) pr[h] = sc[t * kH + h];
-        }
-#pragma unroll
-        for (int h = 0; h < kH; ++h) {
-          const uint64_t pp = f2_pack(pr[h], pr[h]);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) acc[h][i] = f2_fma(pp, f2_pack(y[2 * i], y[2 * i + 1]), acc[h][i]);
-        }
-      }
-      float v[16 * kH];
-#pragma unroll
-      for (int h = 0; h < kH; ++h)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f2_unpack(acc[h][i], v[16 * h + 2 * i], v[16 * h + 2 * i + 1]);
-      lane_sums<16 * kH>(v, lane);
-      float* dst = part + (g * n_slice + slice) * 16 * kH;
-      if (kH == 1) {
-        if ((lane & 1) == 0) dst[lane >> 1] = v[0];
-      } else {
-#pragma unroll
-        for (int i = 0; i < kH / 2; ++i) dst[lane * (kH / 2) + i] = v[i];
-      }
-    }
-    __syncthreads();
-    if (n_next > 0) p.stage(vbuf, pair, hk, 1, t0 + c.chunk, n_next, tid);
-    split_commit();
-    for (int i = tid; i < kH * dp; i += kSplitThreads) {
-      const int h = i / dp, j = i - h * dp;
-      float v = 0.f;
-      for (int s = 0; s < n_slice; ++s) v += part[((j >> 4) * n_slice + s) * 16 * kH + h * 16 + (j & 15)];
-      o_sm[i] = fmaf(o_sm[i], corr_sm[h], v);
+    for (int h = 0; h < kH; ++h) {
+      wm_sm[warp * kH + h] = m_run[h];
+      wl_sm[warp * kH + h] = l_run[h];
     }
   }
-  // ---- merge over the cluster: this block's d / C coordinates of every head, in rank order
-  __syncthreads();
-  cluster_arrive();   // (C) partial results are complete everywhere
-  cluster_wait();
-  for (int i = tid; i < nc * kH; i += kSplitThreads) {
-    const int h = i / nc, j = j0 + (i - h * nc);
-    const uint32_t m_a = (uint32_t)__cvta_generic_to_shared(m_sm + h), l_a = (uint32_t)__cvta_generic_to_shared(l_sm + h);
-    const uint32_t o_a = (uint32_t)__cvta_generic_to_shared(o_sm + h * dp + j);
-    float M = -CUDART_INF_F;
-#pragma unroll 4
-    for (int r = 0; r < C; ++r) M = fmaxf(M, cluster_ld(cluster_map(m_a, r)));
-    float L = 0.f, y = 0.f;
-#pragma unroll 4
-    for (int r = 0; r < C; ++r) {
-      const float m = cluster_ld(cluster_map(m_a, r));
-      const float w = m == -CUDART_INF_F ? 0.f : exp2f(m - M);
-      L = fmaf(cluster_ld(cluster_map(l_a, r)), w, L);
-      y = fmaf(cluster_ld(cluster_map(o_a, r)), w, y);
+  split_wait<0>();
+  __syncthreads();   // the ring is free
+  {
+    float o[kH * kU];
+#pragma unroll
+    for (int h = 0; h < kH; ++h) {
+      mb[h] = -CUDART_INF_F;
+#pragma unroll
+      for (int w = 0; w < kSplitWarps; ++w) mb[h] = fmaxf(mb[h], wm_sm[w * kH + h]);
+      const float k = m_run[h] == -CUDART_INF_F ? 0.f : split_exp2(m_run[h] - mb[h]);
+#pragma unroll
+      for (int i = 0; i < kU / 2; ++i) {
+        f2_unpack(acc[h][i], o[h * kU + 2 * i], o[h * kU + 2 * i + 1]);
+        o[h * kU + 2 * i] *= k;
+        o[h * kU + 2 * i + 1] *= k;
+      }
     }
-    y = len > 0 ? y / L : 0.f;
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(y_sm + h * dp + j);
-    for (int r = 0; r < C; ++r) cluster_st(cluster_map(dst, r), y);
-    if (c.lse != nullptr && j == 0 && h < grp)   // scores are in the log2 domain
+    int from, count;
+    switch (lanes) {
+      case 1: unit_lane_sums<kH * kU, 1>(o, lane, &from, &count); break;
+      case 2: unit_lane_sums<kH * kU, 2>(o, lane, &from, &count); break;
+      case 4: unit_lane_sums<kH * kU, 4>(o, lane, &from, &count); break;
+      case 8: unit_lane_sums<kH * kU, 8>(o, lane, &from, &count); break;
+      case 16: unit_lane_sums<kH * kU, 16>(o, lane, &from, &count); break;
+      default: from = 0; count = kH * kU; break;
+    }
+#pragma unroll
+    for (int i = 0; i < kH * kU; ++i)
+      if (i < count) {   // value from + i: head / coordinate of the unit
+        const int e = from + i;
+        w_out[(warp * kH + e / kU) * dp + unit * kU + e % kU] = o[i];
+      }
+  }
+  __syncthreads();
+  for (int i = tid; i < kH * dp; i += kSplitThreads) {
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < kSplitWarps; ++w) v[w & 3] += w_out[w * kH * dp + i];
+    o_sm[i] = (v[0] + v[1]) + (v[2] + v[3]);
+  }
+  if (warp == 0) {
+#pragma unroll
+    for (int h = 0; h < kH; ++h) {
+      float l = 0.f;
+      if (lane < kSplitWarps) {
+        const float m = wm_sm[lane * kH + h];
+        l = m == -CUDART_INF_F ? 0.f : wl_sm[lane * kH + h] * split_exp2(m - mb[h]);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) {
+        m_sm[h] = mb[h];
+        l_sm[h] = l;
+      }
+    }
+  }
+  // ---- merge the blocks: every block reads all partial outputs (in rank order) and un-rotates d / C coordinates
+  const int nc = d / C, j0 = rank * nc;
+  if (C > 1) {
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    __syncthreads();
+  }
+  for (int i = tid; i < kH * dp / 4; i += kSplitThreads) {
+    const int h = 4 * i / dp;
+    const uint32_t m_a = (uint32_t)__cvta_generic_to_shared(m_sm + h), l_a = (uint32_t)__cvta_generic_to_shared(l_sm + h);
+    const uint32_t o_a = (uint32_t)__cvta_generic_to_shared(o_sm + 4 * i);
+    float M = -CUDART_INF_F, L = 0.f;
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = 0; r0 < C; r0 += 8) {   // eight ranks at a time: their remote loads are all in flight together
+      float m[8], l[8];
+      float4 o[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const uint32_t from = r0 + r < C ? r0 + r : r0;
+        m[r] = cluster_ld(cluster_map(m_a, from));
+        l[r] = cluster_ld(cluster_map(l_a, from));
+        o[r] = cluster_ld4(cluster_map(o_a, from));
+      }
+      float m8 = M;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) m8 = fmaxf(m8, m[r]);
+      if (m8 == -CUDART_INF_F) continue;
+      const float k = split_exp2(M - m8);   // 0 at first
+      L *= k;
+      y.x *= k; y.y *= k; y.z *= k; y.w *= k;
+      M = m8;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float w = r0 + r < C ? split_exp2(m[r] - M) : 0.f;   // 0 for a block without tokens
+        L = fmaf(l[r], w, L);
+        y.x = fmaf(o[r].x, w, y.x);
+        y.y = fmaf(o[r].y, w, y.y);
+        y.z = fmaf(o[r].z, w, y.z);
+        y.w = fmaf(o[r].w, w, y.w);
+      }
+    }
+    const float inv = len > 0 ? 1.f / L : 0.f;
+    *reinterpret_cast<float4*>(y_sm + 4 * i) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+    if (c.lse != nullptr && rank == 0 && 4 * i == h * dp && h < grp)   // scores are in the log2 domain
       c.lse[(int64_t)pair * c.n_q_heads + hk * grp + h] = len > 0 ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
   }
   if (rank == 0 && tid == 0 && len <= 0 && c.lse == nullptr) set_status(c.status, PQ_ERR_EMPTY);
-  cluster_arrive();   // (D) the merged output is complete everywhere; no block reads another's shared memory after this
-  cluster_wait();
-  // ---- x_hat_j = sum_k y_k S[j][k] for this block's coordinates: a warp per row of S
+  __syncthreads();
+  if (C > 1) cluster_arrive();   // this block has read the others' shared memory; waited for before it gives up its own
+  // x_hat_j = sum_k y_k S[j][k]: a warp per row of S
+#pragma unroll 1
   for (int jj = warp; jj < nc; jj += kSplitWarps) {
-    const int j = j0 + jj;
-    float acc[kH];
+    const float* row = (s_staged ? S_sm : c.S) + (j0 + jj) * d;
+    float sum[kH];
 #pragma unroll
-    for (int h = 0; h < kH; ++h) acc[h] = 0.f;
+    for (int h = 0; h < kH; ++h) sum[h] = 0.f;
+#pragma unroll 4
     for (int k = lane; k < d; k += 32) {
-      const float s = __ldg(c.S + (int64_t)j * d + k);
+      const float s = row[k];
 #pragma unroll
-      for (int h = 0; h < kH; ++h) acc[h] = fmaf(y_sm[h * dp + k], s, acc[h]);
+      for (int h = 0; h < kH; ++h) sum[h] = fmaf(y_sm[h * dp + k], s, sum[h]);
     }
 #pragma unroll
-    for (int h = 0; h < kH; ++h) {
-      float v = acc[h];
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0 && h < grp) {
-        const int64_t idx = q0 + h * d + j;
-        if (c.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(c.out)[idx] = __float2bfloat16(v);
-        else reinterpret_cast<float*>(c.out)[idx] = v;
-      }
+      for (int h = 0; h < kH; ++h) sum[h] += __shfl_xor_sync(0xffffffffu, sum[h], o);
+    float mine_h = sum[0];   // lane h stores head h
+#pragma unroll
+    for (int h = 1; h < kH; ++h) mine_h = lane == h ? sum[h] : mine_h;
+    if (lane < grp) {
+      const int64_t idx = q0 + lane * d + j0 + jj;
+      if (c.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(c.out)[idx] = __float2bfloat16(mine_h);
+      else reinterpret_cast<float*>(c.out)[idx] = mine_h;
     }
   }
+  if (C > 1) cluster_wait();
 }
 
-// Blocks per cluster: enough to give every SM two blocks, a power of two that divides d, at least 64 tokens per block,
-// at most 8 (the portable limit) or 16 where the call has so few (kv head, sequence) pairs that 8 leave SMs idle.
-inline int split_cluster_size(int d, int64_t units, int max_len, int n_sm, int smem_bytes) {
-  int C = 1;
-  while (C < 8 && C * 2 <= d && C * 64 < max_len && C * units < 2 * n_sm) C *= 2;
-  if (C == 8 && d >= 16 && C * 64 < max_len && C * units < n_sm && smem_bytes <= 100 * 1024) C = 16;
-  return C;
+// Blocks per cluster: a power of two that divides d, four tiles per block or more, at most 8 (the portable limit; with 16 blocks
+// of this size few clusters find room in a GPC at once).  The choice is the one with the shortest estimated time: waves of
+// resident blocks times (tokens of a block plus what its set-up and merge cost, as long as 25000 / d tokens).  *tokens
+// becomes the former product without the overhead: what the busiest SM goes through.
+inline int split_cluster_size(int d, int tile, int64_t units, int max_len, int n_sm, int64_t* tokens) {
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int C = 1; C <= 8 && C <= d; C *= 2) {
+    if (C > 1 && (int64_t)(C / 2) * tile * 4 >= max_len) break;   // half as many blocks already have no more than four tiles each
+    const int64_t waves = (units * C + n_sm - 1) / n_sm;
+    const int64_t cost = waves * ((max_len + C - 1) / C + 25000 / d);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = C;
+      *tokens = waves * ((max_len + C - 1) / C);
+    }
+  }
+  return best;
 }
 
 // `configured`: one DeviceMemo per instantiation.
 template <class P, int kH>
-int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, int smem, cudaStream_t stream) {
+int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStream_t stream) {
   static DeviceMemo configured;
   auto kernel = split_attention_kernel<P, kH>;
   const int n_sm = configure_for_device(kernel, kSplitSmemMax, configured, true);
   if (n_sm == 0) return PQ_ERR_CUDA;
-  const int C = split_cluster_size(p.c.d, pairs * p.c.n_kv_heads, max_len, n_sm, smem);
+  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
+  if (smem > kSplitSmemMax) return PQ_ERR_UNSUPPORTED;
+  int64_t tokens;
+  const int C = split_cluster_size(p.c.d, p.c.tile, pairs * p.c.n_kv_heads, max_len, n_sm, &tokens);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C, p.c.n_kv_heads, (unsigned)pairs);
-  cfg.blockDim = dim3(kSplitThreads);
+  cfg.blockDim = dim3(32 * split_warps(kH));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set up while the kernel before it finishes (it waits inside)
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set up while the kernel before it finishes (it waits inside)
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = C;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = C > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
   if (e != cudaSuccess) {
     note_cuda_error(e);
@@ -415,6 +505,23 @@ int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, int smem,
     return PQ_ERR_CUDA;
   }
   return launch_status();
+}
+
+// The instantiation for the group size.  Tiles of 16 tokens (32 where a lane takes a whole token), fewer where long rows
+// would take more than 200 KB of shared memory.
+template <class P>
+int32_t dispatch_split_attention(P p, int64_t pairs, int max_len, cudaStream_t stream) {
+  const int kh = split_heads(p.c.n_q_heads / p.c.n_kv_heads), lanes = split_lanes(p.c.d, kh);
+  int T = lanes == 1 ? 32 : 16;
+  while (T > 32 / lanes && split_smem_bytes(p.c.d, kh, p.tile_bytes(T)) > 200 * 1024) T /= 2;
+  p.c.tile = T;
+  p.c.stage_bytes = p.tile_bytes(T);
+  switch (kh) {
+    case 1: return launch_split_attention<P, 1>(p, pairs, max_len, stream);
+    case 2: return launch_split_attention<P, 2>(p, pairs, max_len, stream);
+    case 4: return launch_split_attention<P, 4>(p, pairs, max_len, stream);
+    default: return launch_split_attention<P, 8>(p, pairs, max_len, stream);
+  }
 }
 
 }  // namespace pq
