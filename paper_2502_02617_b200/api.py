@@ -204,12 +204,7 @@ def pq_fit_codebooks(bits=DEFAULT_BITS):
 
 def pq_angle_histograms(S, K, V, hist, status, stream=None):
     """Add the angles of the rows of K and V [total_tokens, Hkv, d] to hist (int64 device tensor [4, n_bins])."""
-    total, n_kv_heads, d = K.shape
-    assert V.shape == K.shape and V.dtype == K.dtype and K.stride(2) == 1 and V.stride() == K.stride()
-    assert hist.dtype == torch.int64 and hist.is_contiguous() and hist.shape[0] == N_LEVELS
-    _check(lib().pq_angle_histograms(d, n_kv_heads, _ptr(S), _ptr(K), _ptr(V), _dtype_code(K), K.stride(0), K.stride(1),
-                                     total, hist.shape[1], _ptr(hist), _ptr(status), _stream(stream)),
-           "pq_angle_histograms")
+    _check((_native or native()).angle_histograms(S, K, V, hist, status, stream), "pq_angle_histograms")
 
 
 def pq_fit_codebooks_from_histograms(hist: torch.Tensor, init_centroids: torch.Tensor = None):
@@ -224,11 +219,11 @@ def pq_fit_codebooks_from_histograms(hist: torch.Tensor, init_centroids: torch.T
     return cen, bnd
 
 
-def pq_build_tables(centroids: torch.Tensor, boundaries: torch.Tensor) -> torch.Tensor:
-    """Compiled device tables as a CPU uint8 tensor; move it to the GPU unchanged."""
+def pq_build_tables(centroids: torch.Tensor, boundaries: torch.Tensor, pinned: bool = False) -> torch.Tensor:
+    """Compiled device tables as a CPU uint8 tensor (in pinned memory on request); move it to the GPU unchanged."""
     centroids = centroids.to(torch.float64).contiguous()
     boundaries = boundaries.to(torch.float64).contiguous()
-    out = torch.zeros(int(lib().pq_tables_bytes()), dtype=torch.uint8)
+    out = torch.empty(int(lib().pq_tables_bytes()), dtype=torch.uint8, pin_memory=pinned)
     _check(lib().pq_build_tables(ctypes.cast(centroids.data_ptr(), POINTER(c_double)),
                                  ctypes.cast(boundaries.data_ptr(), POINTER(c_double)), out.data_ptr()),
            "pq_build_tables")
@@ -325,25 +320,14 @@ def pq_decode_attention_lse(S, tables, q, cache, cache_lens, n_kv_heads, capacit
 
 def pq_merge_attention(parts_out, parts_lse, out, status, lse_out=None, stream=None):
     """Merge partial attentions: parts_out [P, B, Hq, d] (float32 or bf16), parts_lse float32 [P, B, Hq] -> out [B, Hq, d]."""
-    n_parts, batch, n_q_heads, d = parts_out.shape
-    assert parts_out.is_contiguous() and parts_lse.is_contiguous() and out.is_contiguous()
-    assert parts_lse.shape == (n_parts, batch, n_q_heads) and parts_lse.dtype == torch.float32 and out.shape == parts_out.shape[1:]
-    _check(lib().pq_merge_attention(d, n_q_heads, batch, n_parts, _ptr(parts_out), _dtype_code(parts_out), _ptr(parts_lse),
-                                    _ptr(out), _dtype_code(out), _ptr(lse_out), _ptr(status), _stream(stream)),
-           "pq_merge_attention")
+    _check((_native or native()).merge(parts_out, parts_lse, out, lse_out, status, stream), "pq_merge_attention")
     return out
 
 
 def pq_tail_attention(q, k_tail, v_tail, tail_lens, scale, out, lse, status, n_splits=1, stream=None):
     """Exact attention of q [B, Hq, d] over an uncompressed window k_tail, v_tail [B, T, Hkv, d] (first tail_lens[b] rows),
     as n_splits partial attentions: out [n_splits, B, Hq, d] (or [B, Hq, d] for one), lse [n_splits, B, Hq]."""
-    batch, n_q_heads, d = q.shape
-    assert k_tail.is_contiguous() and v_tail.is_contiguous() and k_tail.shape == v_tail.shape and k_tail.dtype == v_tail.dtype
-    assert k_tail.shape[0] == batch and k_tail.shape[3] == d and q.is_contiguous() and out.is_contiguous() and out.dtype == q.dtype
-    assert out.numel() == n_splits * q.numel() and (lse is None or lse.numel() == n_splits * batch * n_q_heads)
-    _check(lib().pq_tail_attention(d, n_q_heads, k_tail.shape[2], _ptr(q), _dtype_code(q), _ptr(k_tail), _ptr(v_tail),
-                                   _dtype_code(k_tail), _ptr(tail_lens), batch, k_tail.shape[1], n_splits, float(scale),
-                                   _ptr(out), _ptr(lse), _ptr(status), _stream(stream)), "pq_tail_attention")
+    _check((_native or native()).tail_attend(q, k_tail, v_tail, tail_lens, scale, out, lse, status, n_splits, stream), "pq_tail_attention")
 
 
 def sharded_decode_attention(cache, q, dist, group=None, scale=None, stream=None):
@@ -383,14 +367,19 @@ class PolarQuantCache:
         """Replace the codebooks of this cache by the ones clustered on the angles of K, V ([tokens, Hkv, d], the
         prompt's keys and values): histogram on the device, clustering on the host, new tables.  To be called
         before anything is encoded (codes already in the cache belong to the previous codebooks)."""
-        hist = torch.zeros((N_LEVELS, n_bins), dtype=torch.int64, device=self.device)
-        pq_angle_histograms(self.S, K, V, hist, self.status, stream)
-        self.set_codebooks(*pq_fit_codebooks_from_histograms(hist.cpu()))
+        with torch.cuda.stream(stream):   # None: the current stream
+            hist = torch.zeros((N_LEVELS, n_bins), dtype=torch.int64, device=self.device)
+            pq_angle_histograms(self.S, K, V, hist, self.status)
+            # the copies go through pinned memory (from a pool that keeps a block until its copy has finished)
+            counts = torch.empty((N_LEVELS, n_bins), dtype=torch.int64, pin_memory=True)
+            counts.copy_(hist, non_blocking=True)
+            torch.cuda.current_stream().synchronize()
+            self.set_codebooks(*pq_fit_codebooks_from_histograms(counts))
         return hist
 
     def set_codebooks(self, centroids, boundaries):
         self.centroids, self.boundaries = centroids, boundaries
-        self.tables = pq_build_tables(centroids, boundaries).to(self.device)
+        self.tables = pq_build_tables(centroids, boundaries, pinned=True).to(self.device, non_blocking=True)
 
     def encode(self, K, V, cu_seqlens, stream=None):
         pq_encode_kv(self.S, self.tables, K, V, cu_seqlens, self.cache, self.lens, self.capacity, self.status, stream)

@@ -191,7 +191,57 @@ PyObject* general_attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
+// angle_histograms(S, K, V, hist, status, stream): hist int64 [levels, bins], counts are added
+PyObject* angle_histograms(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return entry(n, 6, [&]() -> int32_t {
+    const at::Tensor &K = tensor(a[1]), &V = tensor(a[2]), &hist = tensor(a[3]);
+    check_rows(K, V);
+    check(hist.scalar_type() == at::kLong && hist.is_contiguous() && hist.dim() == 2 && hist.size(0) == PQ_N_LEVELS,
+          "hist must be a contiguous int64 tensor [levels, bins]");
+    return pq_angle_histograms((int32_t)K.size(2), (int32_t)K.size(1), ptr<float>(tensor(a[0])), ptr(K), ptr(V), dtype_code(K),
+                               K.stride(0), K.stride(1), (int32_t)K.size(0), (int32_t)hist.size(1), ptr<uint64_t>(hist),
+                               ptr<int32_t>(tensor(a[4])), stream_of(a[5]));
+  });
+}
+
+// tail_attend(q, k_tail, v_tail, tail_lens, scale, out, lse or None, status, n_splits, stream)
+PyObject* tail_attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return entry(n, 10, [&]() -> int32_t {
+    const at::Tensor &q = tensor(a[0]), &k = tensor(a[1]), &v = tensor(a[2]), &out = tensor(a[5]);
+    const at::Tensor* lse = tensor_or_none(a[6]);
+    const int32_t splits = i32(a[8]);
+    check(q.dim() == 3 && q.is_contiguous() && out.is_contiguous() && out.scalar_type() == q.scalar_type(),
+          "q and out must be contiguous tensors of one dtype");
+    check(k.dim() == 4 && k.is_contiguous() && v.is_contiguous() && k.sizes() == v.sizes() && k.scalar_type() == v.scalar_type() &&
+              k.size(0) == q.size(0) && k.size(3) == q.size(2),
+          "the window must be contiguous [batch, tokens, kv heads, head_dim]");
+    check(out.numel() == splits * q.numel() && (lse == nullptr || lse->numel() == splits * q.size(0) * q.size(1)),
+          "out and lse must hold n_splits parts");
+    return pq_tail_attention((int32_t)q.size(2), (int32_t)q.size(1), (int32_t)k.size(2), ptr(q), dtype_code(q), ptr(k), ptr(v),
+                             dtype_code(k), ptr<int32_t>(tensor(a[3])), (int32_t)q.size(0), (int32_t)k.size(1), splits, f32(a[4]),
+                             ptr(out), lse == nullptr ? nullptr : ptr<float>(*lse), ptr<int32_t>(tensor(a[7])), stream_of(a[9]));
+  });
+}
+
+// merge(parts_out, parts_lse, out, lse_out or None, status, stream)
+PyObject* merge(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return entry(n, 6, [&]() -> int32_t {
+    const at::Tensor &parts = tensor(a[0]), &lse = tensor(a[1]), &out = tensor(a[2]);
+    const at::Tensor* lse_out = tensor_or_none(a[3]);
+    check(parts.dim() == 4 && parts.is_contiguous() && lse.is_contiguous() && out.is_contiguous(), "contiguous tensors are taken");
+    check(lse.scalar_type() == at::kFloat && lse.dim() == 3 && lse.sizes() == parts.sizes().slice(0, 3) &&
+              out.sizes() == parts.sizes().slice(1, 3),
+          "parts_out [parts, batch, heads, head_dim], parts_lse float32 [parts, batch, heads], out [batch, heads, head_dim]");
+    return pq_merge_attention((int32_t)parts.size(3), (int32_t)parts.size(2), (int32_t)parts.size(1), (int32_t)parts.size(0), ptr(parts),
+                              dtype_code(parts), ptr<float>(lse), ptr(out), dtype_code(out),
+                              lse_out == nullptr ? nullptr : ptr<float>(*lse_out), ptr<int32_t>(tensor(a[4])), stream_of(a[5]));
+  });
+}
+
 PyMethodDef kMethods[] = {
+    {"angle_histograms", (PyCFunction)(void (*)(void))angle_histograms, METH_FASTCALL, nullptr},
+    {"tail_attend", (PyCFunction)(void (*)(void))tail_attend, METH_FASTCALL, nullptr},
+    {"merge", (PyCFunction)(void (*)(void))merge, METH_FASTCALL, nullptr},
     {"encode", (PyCFunction)(void (*)(void))encode, METH_FASTCALL, nullptr},
     {"append", (PyCFunction)(void (*)(void))append, METH_FASTCALL, nullptr},
     {"attend", (PyCFunction)(void (*)(void))attend, METH_FASTCALL, nullptr},

@@ -67,13 +67,37 @@ struct L1Ray {
   int below, above;  // codes on the sides t_c < t and t_c > t
 };
 
-int l1_code_of_angle(const double* bnd, double psi) {
-  int c = 0;
-  for (int k = 0; k < 15; ++k) c += psi > bnd[k];
-  return c;
+// Number of (ascending) boundaries below psi, found from `near`, the number below a psi close by.
+int l1_code_of_angle(const double* bnd, double psi, int near) {
+  while (near < 15 && psi > bnd[near]) ++near;
+  while (near > 0 && !(psi > bnd[near - 1])) --near;
+  return near;
 }
 
+// What the cells look like whatever the codebook is: their ranges of t and the angles of the points that are looked at.
+// 768 arc tangents, computed once per process (most of the cost of a table that is built for every prompt).
+struct L1Grid {
+  double lo[pq::kL1Cells], hi[pq::kL1Cells], mid_phi[pq::kL1Cells];  // with slack: the decisions
+  double t[pq::kL1Cells][5], phi[pq::kL1Cells][5];                     // the points of the check
+  L1Grid() {
+    // the kernel's cell index is floor(m / 8), m = t * kL1CellScale * 8 rounded to an integer
+    const double scale = (double)pq::kL1CellScale;
+    for (int c = 0; c < pq::kL1Cells; ++c) {
+      const double a = (c - 1.0 / 16.0) / scale, b = (c + 15.0 / 16.0) / scale;
+      lo[c] = std::fmax(0.0, a - 1e-6);
+      hi[c] = std::fmin(1.0, b + 1e-6);
+      mid_phi[c] = std::atan(0.5 * (lo[c] + hi[c]));
+      const double lo0 = std::fmax(0.0, a), hi0 = std::fmin(1.0, b);
+      for (int i = 0; i <= 4; ++i) {
+        t[c][i] = lo0 + (hi0 - lo0) * i / 4.0;
+        phi[c][i] = std::atan(t[c][i]);
+      }
+    }
+  }
+};
+
 bool build_l1_cells(const double* bnd, uint2 (*cells)[pq::kL1Cells]) {
+  static const L1Grid grid;   // thread-safe initialisation
   const double kHalfPi = 0.5 * kPi;
   for (int o = 0; o < 8; ++o) {
     const int sb = (o >> 2) & 1, sa = (o >> 1) & 1, sw = o & 1;
@@ -82,42 +106,43 @@ bool build_l1_cells(const double* bnd, uint2 (*cells)[pq::kL1Cells]) {
     else if (sa && !sb) { B = sw ? kHalfPi : kPi; D = sw ? 1.0 : -1.0; }
     else if (sa && sb) { B = sw ? 3.0 * kHalfPi : kPi; D = sw ? -1.0 : 1.0; }
     else { B = sw ? 3.0 * kHalfPi : 2.0 * kPi; D = sw ? 1.0 : -1.0; }
-    std::vector<L1Ray> rays;
+    L1Ray rays[16];
+    int n_rays = 0;
     for (int j = 0; j < 16; ++j) {
       const double ang = j == 0 ? 0.0 : bnd[j - 1];
-      double phi = std::remainder(D * (ang - B), 2.0 * kPi);  // in [-pi, pi]
+      double phi = D * (ang - B);   // in [-2 pi, 2 pi]: brought to [-pi, pi] (exact)
+      if (phi > kPi) phi -= 2.0 * kPi;
+      else if (phi < -kPi) phi += 2.0 * kPi;
       if (phi < -0.25 * kPi - 0.02 || phi > std::atan(2.0) + 0.02) continue;
       const int below = (j + 15) & 15, above = j;  // codes at smaller / larger psi
-      rays.push_back({std::tan(phi), D > 0 ? below : above, D > 0 ? above : below});
+      rays[n_rays++] = {std::tan(phi), D > 0 ? below : above, D > 0 ? above : below};
     }
+    std::sort(rays, rays + n_rays, [](const L1Ray& x, const L1Ray& y) { return x.t < y.t; });
+    int code_near = 0;
+    int first = 0;   // rays before this one lie below the cell (the cells ascend)
     for (int c = 0; c < pq::kL1Cells; ++c) {
-      // the kernel's cell index is floor(m / 8), m = t * kL1CellScale * 8 rounded to an integer
-      const double scale = (double)pq::kL1CellScale;
-      const double lo = std::fmax(0.0, (c - 1.0 / 16.0) / scale - 1e-6), hi = std::fmin(1.0, (c + 15.0 / 16.0) / scale + 1e-6);
-      const double w = hi - lo;
-      int n_in = 0, in_idx = -1;
-      double dA = 1e30, dB = 1e30;  // distance from the cell to the nearest ray below / above it
-      for (size_t i = 0; i < rays.size(); ++i) {
-        if (rays[i].t >= lo && rays[i].t <= hi) { ++n_in; in_idx = (int)i; }
-        else if (rays[i].t < lo) dA = std::fmin(dA, lo - rays[i].t);
-        else dB = std::fmin(dB, rays[i].t - hi);
-      }
+      const double lo = grid.lo[c], hi = grid.hi[c], w = hi - lo;
+      while (first < n_rays && rays[first].t < lo) ++first;
+      int end = first;   // rays first .. end - 1 lie inside
+      while (end < n_rays && rays[end].t <= hi) ++end;
+      const int n_in = end - first, in_idx = first;
+      // distance from the cell to the nearest ray below / above it
+      const double dA = first > 0 ? lo - rays[first - 1].t : 1e30, dB = end < n_rays ? rays[end].t - hi : 1e30;
       float tau;
       int code_lo, code_hi;
       if (n_in == 0) {
         // no ray inside: a virtual tau outside the cell whose distance stays below both neighbours' for every t
-        const double mA = std::fmin(dA, dB - w), mB = std::fmin(dB, dA - w);
-        const double t = mA >= mB ? lo - std::fmin(mA, 1.0) : hi + std::fmin(mB, 1.0);
-        const double mid = 0.5 * (lo + hi);
-        double psi = B + D * std::atan(mid);
+        const double mA = std::min(dA, dB - w), mB = std::min(dB, dA - w);
+        const double t = mA >= mB ? lo - std::min(mA, 1.0) : hi + std::min(mB, 1.0);
+        double psi = B + D * grid.mid_phi[c];
         if (psi >= 2.0 * kPi) psi -= 2.0 * kPi;
         if (psi < 0.0) psi += 2.0 * kPi;
-        code_lo = code_hi = l1_code_of_angle(bnd, psi);
-        tau = (float)std::fmin(1.0, std::fmax(0.0, t));
+        code_lo = code_hi = code_near = l1_code_of_angle(bnd, psi, code_near);
+        tau = (float)std::min(1.0, std::max(0.0, t));
         if ((mA >= mB ? mA : mB) <= 0.0) tau = std::nanf("");  // a ray touches the cell from both sides
       } else if (n_in == 1) {
         const double tm = rays[in_idx].t;
-        const double far = std::fmax(tm - lo, hi - tm);  // largest distance from a t of the cell to the ray
+        const double far = std::max(tm - lo, hi - tm);  // largest distance from a t of the cell to the ray
         tau = (dA >= far && dB >= far) ? (float)tm : std::nanf("");
         code_lo = rays[in_idx].below;
         code_hi = rays[in_idx].above;
@@ -131,22 +156,24 @@ bool build_l1_cells(const double* bnd, uint2 (*cells)[pq::kL1Cells]) {
     }
     // Check the two properties on a grid of every cell (the table is small; a wrong entry would be a silent
     // wrong code).
+    int next = 0;   // first ray above the point; consecutive points are close, cells overlap by 1/8 of their width
     for (int c = 0; c < pq::kL1Cells; ++c) {
       float tau;
       std::memcpy(&tau, &cells[o][c].x, 4);
       if (tau != tau) continue;
-      const double scale = (double)pq::kL1CellScale;
-      const double lo = std::fmax(0.0, (c - 1.0 / 16.0) / scale), hi = std::fmin(1.0, (c + 15.0 / 16.0) / scale);
       for (int i = 0; i <= 4; ++i) {
-        const double t = lo + (hi - lo) * i / 4.0, dist = std::fabs(t - (double)tau);
+        const double t = grid.t[c][i], dist = std::fabs(t - (double)tau);
+        while (next < n_rays && rays[next].t < t) ++next;
+        while (next > 0 && rays[next - 1].t >= t) --next;
         double nearest = 1e30;
-        for (const L1Ray& r : rays) nearest = std::fmin(nearest, std::fabs(t - r.t));
+        if (next < n_rays) nearest = rays[next].t - t;
+        if (next > 0) nearest = std::min(nearest, t - rays[next - 1].t);
         if (dist > nearest + 1e-7) return false;
         if (dist < 1e-6) continue;
-        double psi = B + D * std::atan(t);
+        double psi = B + D * grid.phi[c][i];
         if (psi >= 2.0 * kPi) psi -= 2.0 * kPi;
         if (psi < 0.0) psi += 2.0 * kPi;
-        const int want = l1_code_of_angle(bnd, psi);
+        const int want = code_near = l1_code_of_angle(bnd, psi, code_near);
         const int got = (int)((cells[o][c].y >> (t > (double)tau ? 24 : 28)) & 15u);
         if (want != got) return false;
       }
@@ -328,7 +355,7 @@ int32_t pq_fit_codebooks_from_histograms(const uint64_t* hist, int32_t n_bins, c
   std::vector<double> centre(n_bins), w0(n_bins + 1), w1(n_bins + 1);
   for (int level = 1; level <= PQ_N_LEVELS; ++level) {
     const int n = level == 1 ? 16 : 4;
-    const double hi = level == 1 ? 2.0 * kPi : 0.5 * kPi, width = hi / n_bins;
+    const double hi = level == 1 ? 2.0 * kPi : 0.5 * kPi, width = hi / n_bins, inv_width = n_bins / hi;
     const uint64_t* h = hist + (size_t)(level - 1) * n_bins;
     double* theta = cen + pq::cen_off(level);
     double* beta = bnd + pq::bnd_off(level);
