@@ -82,30 +82,43 @@ struct Workspace {   // of the persistent head_dim-128 kernel; nothing else need
   int64_t bytes;
 };
 
-__host__ inline Workspace carve_workspace(void* base, int d, int batch, int n_q_heads, int n_kv_heads) {
+// `units` with `rows` (query, head) rows each.
+__host__ inline Workspace carve_workspace(void* base, int d, int64_t units, int64_t rows) {
   Workspace w;
   auto align = [](int64_t x) { return (x + 255) & ~(int64_t)255; };
   int64_t off = 0;
   uint8_t* p = reinterpret_cast<uint8_t*>(base);
-  const int64_t g = n_q_heads / n_kv_heads, units = (int64_t)batch * n_kv_heads;
   const int64_t n_slots = (d == 128 && units <= 2048) ? units + kFastMaxGridHost : 0;
   w.elected = reinterpret_cast<uint32_t*>(p + off);
   off = align(off + units * 4);
   w.flags = reinterpret_cast<uint32_t*>(p + off);
   off = align(off + n_slots * 4);
   w.ml = reinterpret_cast<float*>(p + off);
-  off = align(off + n_slots * g * 2 * 4);
+  off = align(off + n_slots * rows * 2 * 4);
   w.o = reinterpret_cast<float*>(p + off);
-  off = align(off + n_slots * g * d * 4);
+  off = align(off + n_slots * rows * d * 4);
   w.bytes = off;
   return w;
 }
 
+// How rows_attention_kernel cuts the n_q * g rows of a kv head: blocks of equal size of at most 32 rows, whole groups of four.
+struct RowCut {
+  int blocks, rows;
+};
+__host__ inline RowCut cut_rows(int64_t all_rows) {
+  const int64_t groups = (all_rows + 3) / 4, blocks = (groups + 7) / 8;
+  RowCut c;
+  c.rows = (int)(4 * ((groups + blocks - 1) / blocks));
+  c.blocks = (int)((all_rows + c.rows - 1) / c.rows);
+  if (c.blocks == 1) c.rows = (int)all_rows;
+  return c;
+}
 
 struct DecodeArgs {
   int d, n_q_heads, n_kv_heads, batch, capacity, io_dtype;
   int n_q;  // queries per sequence (1: decode).  `batch` counts (sequence, query) pairs: q and out are
             // [batch][n_q_heads][d] with pair p = sequence * n_q + query; `lens` and the cache are per sequence.
+  int rows_per_block, n_row_blocks;   // of rows_attention_kernel: its cut of a kv head's n_q * group rows
   float scale;
   uint32_t epoch;  // differs from call to call (top bit set): tags the parts' flags of the persistent kernel
   uint32_t debug;  // test hooks.  bit 0: the first bounded wait of CTA 0 of the persistent kernel reports failure;
@@ -134,6 +147,7 @@ struct DecodeArgs {
 
 }  // namespace pq
 #include "pq_decode_fast.cuh"
+#include "pq_rows.cuh"
 #include "pq_prefill.cuh"
 #include "pq_prefill_tc.cuh"
 #include "pq_split_attention.cuh"
@@ -529,12 +543,80 @@ __global__ void dequant_kernel(int d, int n_kv_heads, const float* S, const Tabl
 
 }  // namespace pq
 
+namespace pq {
+
+// The flags in the (uninitialised, possibly shared) scratch are tagged with a per-call number.  It starts at a value drawn from
+// the clock and the address space of this process, advances by an odd constant and always has its top bit set, so it
+// cannot equal a small integer that another kernel left in the same bytes.
+static uint32_t next_epoch() {
+  static std::atomic<uint32_t> call_epoch{[] {
+    uint64_t x = (uint64_t)std::chrono::steady_clock::now().time_since_epoch().count() ^ (uint64_t)(uintptr_t)&next_epoch;
+    x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
+    x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
+    return (uint32_t)(x ^ (x >> 31));
+  }()};
+  return call_epoch.fetch_add(0x9E3779B1u, std::memory_order_relaxed) | 0x80000000u;
+}
+
+// A persistent kernel (one CTA per SM) as a programmatic dependent: it may be set up while the kernel before it in the stream
+// finishes (it waits inside).
+static int32_t launch_persistent(void (*kernel)(DecodeArgs), const DecodeArgs& a, int n_sm, int threads, int smem, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_sm < kFastMaxGrid ? n_sm : kFastMaxGrid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+  if (e != cudaSuccess) {
+    note_cuda_error(e);
+    cudaGetLastError();
+    return PQ_ERR_CUDA;
+  }
+  return launch_status();
+}
+
+template <int kHG>
+static int32_t launch_rows_as(const DecodeArgs& a, bool paged, cudaStream_t stream) {
+  static DeviceMemo configured[2];
+  void (*kernel)(DecodeArgs) = paged ? rows_attention_kernel<kHG, true> : rows_attention_kernel<kHG, false>;
+  const int n_sm = configure_for_device(kernel, kRowSmTotal, configured[paged ? 1 : 0]);
+  return n_sm == 0 ? PQ_ERR_CUDA : launch_persistent(kernel, a, n_sm, kRowThreads, kRowSmTotal, stream);
+}
+static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq, bool paged, cudaStream_t stream) {
+  a.rows_per_block = cut.rows;
+  a.n_row_blocks = cut.blocks;
+  a.ws = carve_workspace(a.ws.elected, 128, (int64_t)n_seq * a.n_kv_heads * cut.blocks, cut.rows);
+  a.epoch = next_epoch();
+  a.debug = 0u;
+  if (cut.rows <= 4) return launch_rows_as<1>(a, paged, stream);
+  if (cut.rows <= 8) return launch_rows_as<2>(a, paged, stream);
+  if (cut.rows <= 12) return launch_rows_as<3>(a, paged, stream);
+  if (cut.rows <= 16) return launch_rows_as<4>(a, paged, stream);
+  if (cut.rows <= 20) return launch_rows_as<5>(a, paged, stream);
+  if (cut.rows <= 24) return launch_rows_as<6>(a, paged, stream);
+  return launch_rows_as<8>(a, paged, stream);
+}
+
+}  // namespace pq
+
 extern "C" {
 
 int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t max_len) {
   if (!(head_dim == 16 || head_dim == 32 || head_dim == 64 || head_dim == 128)) return PQ_ERR_UNSUPPORTED;
   if (batch <= 0 || n_q_heads <= 0 || n_kv_heads <= 0 || max_len <= 0 || n_q_heads % n_kv_heads) return PQ_ERR_INVALID_ARG;
-  return pq::carve_workspace(nullptr, head_dim, batch, n_q_heads, n_kv_heads).bytes;
+  // `batch` may be sequences or (sequence, query) pairs: enough for any way the rows of the pairs are cut into units.  A cut into
+  // units of at most 32 rows has no more rows than pairs * (group + 3), and 160 more slots.
+  const int64_t units = (int64_t)batch * n_kv_heads, g = n_q_heads / n_kv_heads;
+  const int64_t one = pq::carve_workspace(nullptr, head_dim, units, g).bytes;
+  if (head_dim != 128) return one;
+  const int64_t rows = units * (g + 3) + 32 * pq::kFastMaxGridHost;
+  const int64_t cut = 4 * 256 + units * 4 + (units + pq::kFastMaxGridHost) * 4 + rows * (2 + 128) * 4;
+  return units <= 2048 * 32 && cut > one ? cut : one;
 }
 
 static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, const float* S_dev,
@@ -563,7 +645,8 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.status = status_dev;
   a.lse = lse_dev;
   a.pg = pg;
-  a.ws = pq::carve_workspace(workspace_dev, head_dim, (int)pairs, n_q_heads, n_kv_heads);
+  a.ws = pq::carve_workspace(workspace_dev, head_dim, pairs * n_kv_heads, n_q_heads / n_kv_heads);
+  a.rows_per_block = a.n_row_blocks = 0;
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
   // Chunks of 32 or more rows (queries x heads of a group), d = 128: the tcgen05 kernel (operands in shared memory,
@@ -636,6 +719,10 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
     return pq::launch_status();
   }
+  static const int force_rows = getenv("PQ_ROWS") ? atoi(getenv("PQ_ROWS")) : -1;
+  const pq::RowCut cut = pq::cut_rows(rows);
+  if (head_dim == 128 && rows > (force_rows == 2 ? 0 : 4) && (int64_t)batch * n_kv_heads * cut.blocks <= pq::kFastMaxUnits && force_rows >= 1)
+    return pq::launch_rows_attention(a, cut, batch, pg.table != nullptr, st);
   bool persistent = head_dim == 128 && pairs * n_kv_heads <= pq::kFastMaxUnits, fail_wait = false;
   if (persistent) {
     // Short contexts at head_dim 128 take the cluster kernel too: the persistent kernel needs 14 to 16 us (27 with more
@@ -655,16 +742,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   }
   if (persistent) {
     // One launch: the persistent kernel rotates the queries itself and needs no cleared scratch.
-    // The flags in the (uninitialised, possibly shared) scratch are tagged with a per-call number.  It starts
-    // at a value drawn from the clock and the address space of this process, advances by an odd constant and
-    // always has its top bit set, so it cannot equal a small integer that another kernel left in the same bytes.
-    static std::atomic<uint32_t> call_epoch{[] {
-      uint64_t x = (uint64_t)std::chrono::steady_clock::now().time_since_epoch().count() ^ (uint64_t)(uintptr_t)&launch_attention;
-      x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
-      x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
-      return (uint32_t)(x ^ (x >> 31));
-    }()};
-    a.epoch = call_epoch.fetch_add(0x9E3779B1u, std::memory_order_relaxed) | 0x80000000u;
+    a.epoch = pq::next_epoch();
     a.debug = fail_wait ? 1u : 0u;
     static pq::DeviceMemo configured[4];
     const bool paged = pg.table != nullptr;
@@ -673,22 +751,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
                : (paged ? pq::decode_attention_fast_kernel<2, true> : pq::decode_attention_fast_kernel<2, false>);
     const int n_sm = pq::configure_for_device(kernel, pq::kSmTotal, configured[(g <= 4 ? 0 : 1) + (paged ? 2 : 0)]);
     if (n_sm == 0) return PQ_ERR_CUDA;
-    const int grid = n_sm < pq::kFastMaxGrid ? n_sm : pq::kFastMaxGrid;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(pq::kFastThreads);
-    cfg.dynamicSmemBytes = pq::kSmTotal;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];   // may be set up while the kernel before it in the stream finishes (it waits inside)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) {
-      cudaGetLastError();
-      return PQ_ERR_CUDA;
-    }
-    return pq::launch_status();
+    return pq::launch_persistent(kernel, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
   }
   pq::SplitCommon c;
   c.d = head_dim; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
@@ -817,8 +880,8 @@ int32_t pq_decode_attention_static(int32_t head_dim, int32_t n_q_heads, int32_t 
                                    const void* cache_dev, const int32_t* cache_lens_dev, int32_t batch,
                                    int32_t capacity, int32_t max_len, float scale, void* out_dev,
                                    int32_t* status_dev, void* stream) {
-  const int64_t need = pq_workspace_bytes(head_dim, batch, n_q_heads, n_kv_heads, max_len);
-  if (need < 0) return (int32_t)need;
+  if (const int64_t st = pq_workspace_bytes(head_dim, batch, n_q_heads, n_kv_heads, max_len); st < 0) return (int32_t)st;
+  const int64_t need = pq::carve_workspace(nullptr, head_dim, (int64_t)batch * n_kv_heads, n_q_heads / n_kv_heads).bytes;
   if (need > PQ_STATIC_SCRATCH_BYTES) return PQ_ERR_SCRATCH;
   static std::atomic<void*> scratch_of_device[pq::kMaxDevices];
   int dev = -1;

@@ -237,26 +237,27 @@ constexpr int kO2 = 32 * kTokenBlock, kO3 = kO2 + 8 * kTokenBlock, kO4 = kO3 + 4
 
 // Build the replicated shared-memory tables from `Tables`: entry e goes to 16 consecutive slots.
 // All loads are issued before the stores so that their latencies overlap.
-__device__ inline void build_fast_tables(uint8_t* smem, const Tables* tb) {
+template <int kThreads>
+__device__ __forceinline__ void build_fast_tables(uint8_t* smem, const Tables* tb) {
   const int tid = threadIdx.x;
-  static_assert(kFastThreads == 512, "table fill assumes 512 threads");
-  uint2 v[24];
+  constexpr int kPer = 256 * 16 / kThreads;
+  uint2 v[3 * kPer];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int e = (tid + r * kFastThreads) >> 4;  // 0..255
+  for (int r = 0; r < kPer; ++r) {
+    const int e = (tid + r * kThreads) >> 4;  // 0..255
     v[r] = tb->t1p_hi[e];
-    v[8 + r] = tb->t1p_lo[e];
-    v[16 + r] = tb->u_tab[e >> 6][e & 63];
+    v[kPer + r] = tb->t1p_lo[e];
+    v[2 * kPer + r] = tb->u_tab[e >> 6][e & 63];
   }
   uint2* t1hi = reinterpret_cast<uint2*>(smem + kSmT1p);
   uint2* t1lo = reinterpret_cast<uint2*>(smem + kSmT1lo);
   uint2* u = reinterpret_cast<uint2*>(smem + kSmU);
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = tid + r * kFastThreads;
+  for (int r = 0; r < kPer; ++r) {
+    const int i = tid + r * kThreads;
     t1hi[i] = v[r];
-    t1lo[i] = v[8 + r];
-    u[i] = v[16 + r];
+    t1lo[i] = v[kPer + r];
+    u[i] = v[2 * kPer + r];
   }
 }
 
@@ -269,6 +270,145 @@ constexpr int kFastMaxSegs = 16;     // units of one CTA that are listed at a ti
 struct Segment {
   int unit, st0, st1, part, n_parts, slot0;
 };
+
+// Persistent work split: the 128-token stages of all units, in unit order, are cut into
+// gridDim.x contiguous ranges of equal cost; a CTA's range may cover the end of one unit and the
+// start of the next, and a unit may be shared by several CTAs (its "parts").  Starting on another
+// unit costs a CTA about kSegmentCost stages (query rotation, refilling the ring, the merge), so
+// every unit is preceded by that many empty positions on the line that is cut.  A thread works out up to four
+// consecutive units (positions, ranks and partial slots by block-wide scans); the units this CTA takes
+// part in are consecutive among the non-empty ones and are listed kFastMaxSegs at a time (a ragged batch -- one very
+// long sequence and many short ones -- can give a CTA more than that; the split is then worked out again for the next
+// batch of the list, because its scratch lies in the ring).
+// Fills `segs` with the CTA's units number kFastMaxSegs * batch_no .. (counted among the CTA's own) and returns how many
+// units the CTA has in all.  Called by all threads; `scratch`: 16 bytes per warp.  stages_of(u): stages of unit u (0 past the last
+// one); empty_unit(u) is called once for every unit without any.  The loops over a thread's units are kept rolled here and
+// in the other parts that run once: at the start of a launch every instruction is fetched through cold instruction
+// caches, and a short call takes longer to fetch straight-line code than to run it.
+template <int kThreads, class StagesOf, class EmptyUnit>
+__device__ __forceinline__ int list_segments(int batch_no, int n_units, uint8_t* scratch, Segment* segs, int* n_segs, int* first_rank,
+                                             StagesOf stages_of, EmptyUnit empty_unit) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x, cta = blockIdx.x;
+  long long* scan_w = reinterpret_cast<long long*>(scratch);   // [warps]
+  int* scan_r = reinterpret_cast<int*>(scan_w + kThreads / 32);
+  int* scan_p = scan_r + kThreads / 32;
+  if (tid == 0) {
+    *n_segs = 0;
+    *first_rank = 0x7fffffff;
+  }
+  const int per = (n_units + kThreads - 1) / kThreads, u0 = tid * per;   // this thread's units u0 .. u0 + per - 1
+  long long w_mine = 0;
+  int r_mine = 0;
+#pragma unroll 1
+  for (int i = 0; i < per; ++i) {
+    const int nst = stages_of(u0 + i);
+    w_mine += nst > 0 ? nst + kSegmentCost : 0;
+    r_mine += nst > 0;
+  }
+  long long w_pos = w_mine;   // inclusive scans over the warp, then over the warps
+  int r_pos = r_mine;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long w = __shfl_up_sync(0xffffffffu, w_pos, o);
+    const int r = __shfl_up_sync(0xffffffffu, r_pos, o);
+    if (lane >= o) {
+      w_pos += w;
+      r_pos += r;
+    }
+  }
+  if (lane == 31) {
+    scan_w[warp] = w_pos;
+    scan_r[warp] = r_pos;
+  }
+  __syncthreads();
+  long long w_total = 0;
+  w_pos -= w_mine;   // start of this thread's first unit
+  r_pos -= r_mine;
+#pragma unroll 4
+  for (int w = 0; w < kThreads / 32; ++w) {
+    w_pos += w < warp ? scan_w[w] : 0;
+    r_pos += w < warp ? scan_r[w] : 0;
+    w_total += scan_w[w];
+  }
+  // positions times G fit 32 bits for all but enormous calls: a 64-bit division costs several times a 32-bit one
+  const bool small = w_total * G < (1ll << 31);
+  auto ratio = [&](long long x, long long y) -> long long { return small ? (long long)((uint32_t)x / (uint32_t)y) : x / y; };
+  // the CTAs c_first .. c_first + parts - 1 share a unit whose first stage has position `start`
+  auto shared_by = [&](long long start, int nst, int* c_first) -> int {
+    *c_first = (int)ratio((start + 1) * G + w_total - 1, w_total) - 1;                 // CTA whose range holds stage `start`
+    return (int)ratio((start + nst) * G + w_total - 1, w_total) - *c_first;            // ... and the one of its last stage
+  };
+  int p_mine = 0, rank = r_pos;
+  long long w_at = w_pos;
+#pragma unroll 1
+  for (int i = 0; i < per; ++i) {
+    const int u = u0 + i, nst = stages_of(u);
+    if (nst > 0) {
+      int c_first;
+      const int parts = shared_by(w_at + kSegmentCost, nst, &c_first);
+      p_mine += parts;
+      if (cta >= c_first && cta < c_first + parts) {
+        atomicAdd(n_segs, 1);
+        atomicMin(first_rank, rank);
+      }
+      w_at += kSegmentCost + nst;
+      ++rank;
+    } else if (cta == 0 && batch_no == 0 && u < n_units) {
+      empty_unit(u);
+    }
+  }
+  int p_pos = p_mine;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, p_pos, o);
+    if (lane >= o) p_pos += v;
+  }
+  if (lane == 31) scan_p[warp] = p_pos;
+  __syncthreads();
+  const int r0 = *first_rank + batch_no * kFastMaxSegs;  // this batch: ranks r0 .. r0 + kFastMaxSegs - 1
+  p_pos -= p_mine;
+#pragma unroll 4
+  for (int w = 0; w < kThreads / 32; ++w) p_pos += w < warp ? scan_p[w] : 0;
+  w_at = w_pos;
+  rank = r_pos;
+#pragma unroll 1
+  for (int i = 0; i < per; ++i) {
+    const int nst = stages_of(u0 + i);
+    if (nst == 0) continue;
+    const long long start = w_at + kSegmentCost, end = start + nst;
+    int c_first;
+    const int parts = shared_by(start, nst, &c_first);
+    if (cta >= c_first && cta < c_first + parts && rank >= r0 && rank < r0 + kFastMaxSegs) {
+      const long long lo = ratio(cta * w_total, G), hi = ratio((cta + 1) * w_total, G);
+      Segment& sgm = segs[rank - r0];
+      sgm.unit = u0 + i;
+      sgm.st0 = (int)((lo > start ? lo : start) - start);
+      sgm.st1 = (int)((hi < end ? hi : end) - start);  // > st0: the CTA's range holds a stage of the unit
+      sgm.part = cta - c_first;
+      sgm.n_parts = parts;
+      sgm.slot0 = p_pos;  // first partial slot of the unit
+    }
+    p_pos += parts;
+    w_at = end;
+    ++rank;
+  }
+  __syncthreads();
+  return *n_segs;
+}
+
+// Sums over the 32 lanes of eight values per lane: three halving exchanges leave lane L with row L >> 2 (summed over eight
+// lanes), two more finish it.  9 shuffles instead of 40; the order is fixed.  The four lanes 4 r .. 4 r + 3 return row r.
+__device__ __forceinline__ float sum_eight_rows(const float* v, int lane) {
+  float w4[4], w2[2];
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w4[k] = (b4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, b4 ? v[k] : v[k + 4], 16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) w2[k] = (b3 ? w4[k + 2] : w4[k]) + __shfl_xor_sync(0xffffffffu, b3 ? w4[k] : w4[k + 2], 8);
+  float t = (b2 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? w2[0] : w2[1], 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  return t + __shfl_xor_sync(0xffffffffu, t, 1);
+}
 
 // Merge the `ns` partials (slots slot0 .. slot0 + ns - 1) of the `g` query heads of (b, kv head) in slot order, normalise,
 // rotate back by S^T and store.  Runs in the last CTA that finishes for this unit, so it is a chain of round trips to L2:
@@ -351,22 +491,41 @@ __device__ __forceinline__ void combine_and_store(const DecodeArgs& a, int b, in
     float v[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) v[r] = fmaf(ov[3], sv[r][3], fmaf(ov[2], sv[r][2], fmaf(ov[1], sv[r][1], ov[0] * sv[r][0])));
-    // Sum over the 32 lanes: three halving exchanges leave lane L with row L >> 2 (summed over eight
-    // lanes), two more finish it.  9 shuffles per head instead of 40; the order is fixed.
-    float w4[4], w2[2];
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w4[k] = (b4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, b4 ? v[k] : v[k + 4], 16);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) w2[k] = (b3 ? w4[k + 2] : w4[k]) + __shfl_xor_sync(0xffffffffu, b3 ? w4[k] : w4[k + 2], 8);
-    float t = (b2 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? w2[0] : w2[1], 4);
-    t += __shfl_xor_sync(0xffffffffu, t, 2);
-    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    const float t = sum_eight_rows(v, lane);
     if ((lane & 3) == 0) {
       const int64_t oidx = (h0 + h) * 128 + i0 + (lane >> 2);
       if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[oidx] = __float2bfloat16(t);
       else reinterpret_cast<float*>(a.out)[oidx] = t;
     }
+  }
+}
+
+// Called by one warp of every part of unit `u` when the part's partial result is written (and a barrier has ordered the
+// block's writes before this).
+// Every part raises a flag of its own -- the call's epoch, so nothing in the workspace has to be cleared before the call -- and
+// then looks at all flags of the unit.  The last one to raise its flag sees them all; if several do, the first to put the
+// epoch into the unit's election word combines.  (One counter per unit, taken by compare-and-swap, makes the parts retry on
+// one another: 20 us for the 49 parts of a short two-head call.)  The part that combines takes flags and election word
+// back, so that a replayed graph, whose calls keep their epochs, starts without them; a part that meets the word in
+// between combines once more, to the same result.
+__device__ __forceinline__ void elect_combiner(const DecodeArgs& a, int u, int unit_slot, int part, int n_parts, int lane, int* is_last) {
+  bool last = true;
+  if (n_parts > 1) {
+    __threadfence();   // the block's partial result before its flag
+    volatile uint32_t* flags = a.ws.flags + unit_slot;
+    if (lane == 0) flags[part] = a.epoch;
+    __syncwarp();
+    __threadfence();   // the flag before the look at the others
+    for (int p0 = 0; p0 < n_parts; p0 += 32) last = last && (p0 + lane >= n_parts || flags[p0 + lane] == a.epoch);
+    last = __all_sync(0xffffffffu, last);
+    if (last && lane == 0) last = atomicExch(a.ws.elected + u, a.epoch) != a.epoch;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (last)   // all parts have raised theirs
+      for (int p0 = lane; p0 < n_parts; p0 += 32) flags[p0] = 0u;
+  }
+  if (lane == 0) {
+    __threadfence();
+    *is_last = last;
   }
 }
 
@@ -396,7 +555,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   // while that kernel finishes; its results (lengths, cache, queries, workspace) are read only after this wait.
   // The kernel after this one may be set up as soon as this grid has started.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  build_fast_tables(smem, a.tables);   // from the caller's tables, which no kernel writes
+  build_fast_tables<kFastThreads>(smem, a.tables);   // from the caller's tables, which no kernel writes
   // What this thread needs of S (constant too) to rotate the queries: column warp * 8 + lane / 4, rows 16 i + 4 (lane & 3)
   // + 0..3 -- a warp's load covers whole 32-byte sectors, and four lanes share a column's sum.
   const int rot_j = warp * 8 + (lane >> 2), rot_k = (lane & 3) * 4;
@@ -411,19 +570,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
 
-  // ---- persistent work split: the 128-token stages of all units, in unit order, are cut into
-  // gridDim.x contiguous ranges of equal cost; a CTA's range may cover the end of one unit and the
-  // start of the next, and a unit may be shared by several CTAs (its "parts").  Starting on another
-  // unit costs a CTA about kSegmentCost stages (query rotation, refilling the ring, the merge), so
-  // every unit is preceded by that many empty positions on the line that is cut.  A thread works out up to four
-  // consecutive units (positions, ranks and partial slots by block-wide scans); the units this CTA takes
-  // part in are consecutive among the non-empty ones and are listed kFastMaxSegs at a time (a ragged batch -- one very
-  // long sequence and many short ones -- can give a CTA more than that; the split is then worked out again for the next
-  // batch of the list, because its scratch lies in the ring).
-  const int n_units = a.batch * a.n_kv_heads, G = gridDim.x, cta = blockIdx.x;
-  long long* scan_w = reinterpret_cast<long long*>(smem + kSmRing);   // [16 warps]; the ring is idle while the split is worked out
-  int* scan_r = reinterpret_cast<int*>(scan_w + 16);                  // [16]
-  int* scan_p = scan_r + 16;                                          // [16]
+  const int n_units = a.batch * a.n_kv_heads, cta = blockIdx.x;   // the work split: see list_segments
   Segment* segs = reinterpret_cast<Segment*>(smem + kSmSegs);
   int* n_segs = reinterpret_cast<int*>(smem + kSmFlags) + 2;   // units of this CTA (all batches of the list)
   int* first_rank = reinterpret_cast<int*>(smem + kSmFlags) + 3;
@@ -432,123 +579,21 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     const int len_u = u < n_units ? a.visible_len(u / a.n_kv_heads) : 0;
     return len_u > 0 ? (len_u + kStageTokens - 1) / kStageTokens : 0;
   };
-  // Fills `segs` with the CTA's units number kFastMaxSegs * batch_no .. (counted among the CTA's own) and returns how many
-  // units the CTA has in all.  Called by all threads.  The loops over a thread's units are kept rolled here and in the other
-  // parts that run once: at the start of a launch every instruction is fetched through cold instruction caches, and a
-  // short call takes longer to fetch straight-line code than to run it.
+  auto empty_unit = [&](int u) {   // empty sequence: zeros, and the status says so
+    const int b = u / a.n_kv_heads, hk = u - b * a.n_kv_heads;
+#pragma unroll 1
+    for (int e = 0; e < g_heads * 128; ++e) {
+      const int64_t idx = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128 + e;
+      if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
+      else reinterpret_cast<float*>(a.out)[idx] = 0.f;
+    }
+    if (a.lse != nullptr)
+      for (int h = 0; h < g_heads; ++h) a.lse[(int64_t)b * a.n_q_heads + hk * g_heads + h] = -CUDART_INF_F;
+    else
+      set_status(a.status, PQ_ERR_EMPTY);
+  };
   auto build_segments = [&](int batch_no) -> int {
-    if (tid == 0) {
-      *n_segs = 0;
-      *first_rank = 0x7fffffff;
-    }
-    const int per = (n_units + kFastThreads - 1) / kFastThreads, u0 = tid * per;   // this thread's units u0 .. u0 + per - 1
-    long long w_mine = 0;
-    int r_mine = 0;
-#pragma unroll 1
-    for (int i = 0; i < per; ++i) {
-      const int nst = stages_of(u0 + i);
-      w_mine += nst > 0 ? nst + kSegmentCost : 0;
-      r_mine += nst > 0;
-    }
-    long long w_pos = w_mine;   // inclusive scans over the warp, then over the warps
-    int r_pos = r_mine;
-#pragma unroll 1
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long w = __shfl_up_sync(0xffffffffu, w_pos, o);
-      const int r = __shfl_up_sync(0xffffffffu, r_pos, o);
-      if (lane >= o) {
-        w_pos += w;
-        r_pos += r;
-      }
-    }
-    if (lane == 31) {
-      scan_w[warp] = w_pos;
-      scan_r[warp] = r_pos;
-    }
-    __syncthreads();
-    long long w_total = 0;
-    w_pos -= w_mine;   // start of this thread's first unit
-    r_pos -= r_mine;
-#pragma unroll 4
-    for (int w = 0; w < 16; ++w) {
-      w_pos += w < warp ? scan_w[w] : 0;
-      r_pos += w < warp ? scan_r[w] : 0;
-      w_total += scan_w[w];
-    }
-    // positions times G fit 32 bits for all but enormous calls: a 64-bit division costs several times a 32-bit one
-    const bool small = w_total * G < (1ll << 31);
-    auto ratio = [&](long long x, long long y) -> long long { return small ? (long long)((uint32_t)x / (uint32_t)y) : x / y; };
-    // the CTAs c_first .. c_first + parts - 1 share a unit whose first stage has position `start`
-    auto shared_by = [&](long long start, int nst, int* c_first) -> int {
-      *c_first = (int)ratio((start + 1) * G + w_total - 1, w_total) - 1;                 // CTA whose range holds stage `start`
-      return (int)ratio((start + nst) * G + w_total - 1, w_total) - *c_first;            // ... and the one of its last stage
-    };
-    int p_mine = 0, rank = r_pos;
-    long long w_at = w_pos;
-#pragma unroll 1
-    for (int i = 0; i < per; ++i) {
-      const int u = u0 + i, nst = stages_of(u);
-      if (nst > 0) {
-        int c_first;
-        const int parts = shared_by(w_at + kSegmentCost, nst, &c_first);
-        p_mine += parts;
-        if (cta >= c_first && cta < c_first + parts) {
-          atomicAdd(n_segs, 1);
-          atomicMin(first_rank, rank);
-        }
-        w_at += kSegmentCost + nst;
-        ++rank;
-      } else if (cta == 0 && batch_no == 0 && u < n_units) {  // empty sequence: zeros, and the status says so
-        const int b = u / a.n_kv_heads, hk = u - b * a.n_kv_heads;
-#pragma unroll 1
-        for (int e = 0; e < g_heads * 128; ++e) {
-          const int64_t idx = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128 + e;
-          if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
-          else reinterpret_cast<float*>(a.out)[idx] = 0.f;
-        }
-        if (a.lse != nullptr)
-          for (int h = 0; h < g_heads; ++h) a.lse[(int64_t)b * a.n_q_heads + hk * g_heads + h] = -CUDART_INF_F;
-        else
-          set_status(a.status, PQ_ERR_EMPTY);
-      }
-    }
-    int p_pos = p_mine;
-#pragma unroll 1
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, p_pos, o);
-      if (lane >= o) p_pos += v;
-    }
-    if (lane == 31) scan_p[warp] = p_pos;
-    __syncthreads();
-    const int r0 = *first_rank + batch_no * kFastMaxSegs;  // this batch: ranks r0 .. r0 + kFastMaxSegs - 1
-    p_pos -= p_mine;
-#pragma unroll 4
-    for (int w = 0; w < 16; ++w) p_pos += w < warp ? scan_p[w] : 0;
-    w_at = w_pos;
-    rank = r_pos;
-#pragma unroll 1
-    for (int i = 0; i < per; ++i) {
-      const int nst = stages_of(u0 + i);
-      if (nst == 0) continue;
-      const long long start = w_at + kSegmentCost, end = start + nst;
-      int c_first;
-      const int parts = shared_by(start, nst, &c_first);
-      if (cta >= c_first && cta < c_first + parts && rank >= r0 && rank < r0 + kFastMaxSegs) {
-        const long long lo = ratio(cta * w_total, G), hi = ratio((cta + 1) * w_total, G);
-        Segment& sgm = segs[rank - r0];
-        sgm.unit = u0 + i;
-        sgm.st0 = (int)((lo > start ? lo : start) - start);
-        sgm.st1 = (int)((hi < end ? hi : end) - start);  // > st0: the CTA's range holds a stage of the unit
-        sgm.part = cta - c_first;
-        sgm.n_parts = parts;
-        sgm.slot0 = p_pos;  // first partial slot of the unit
-      }
-      p_pos += parts;
-      w_at = end;
-      ++rank;
-    }
-    __syncthreads();
-    return *n_segs;
+    return list_segments<kFastThreads>(batch_no, n_units, smem + kSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
   };
   const int g = lane >> 2, c = lane & 3;
   const uint32_t rep = (lane & 15) * 8;
@@ -888,32 +933,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       }
     }
     __syncthreads();
-    if (warp == 0) {
-      // Every part raises a flag of its own -- the call's epoch, so nothing in the workspace has to be cleared before the
-      // call -- and then looks at all flags of the unit.  The last one to raise its flag sees them all; if several do, the
-      // first to put the epoch into the unit's election word combines.  (One counter per unit, taken by
-      // compare-and-swap, makes the parts retry on one another: 20 us for the 49 parts of a short two-head call.)  The part
-      // that combines takes flags and election word back, so that a replayed graph, whose calls keep their epochs, starts
-      // without them; a part that meets the word in between combines once more, to the same result.
-      bool last = true;
-      if (n_parts > 1) {
-        __threadfence();   // the CTA's partial result (ordered before this by the barrier) before its flag
-        volatile uint32_t* flags = a.ws.flags + unit_slot;
-        if (lane == 0) flags[cta - c_first] = a.epoch;
-        __syncwarp();
-        __threadfence();   // the flag before the look at the others
-        for (int p0 = 0; p0 < n_parts; p0 += 32) last = last && (p0 + lane >= n_parts || flags[p0 + lane] == a.epoch);
-        last = __all_sync(0xffffffffu, last);
-        if (last && lane == 0) last = atomicExch(a.ws.elected + u, a.epoch) != a.epoch;
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (last)   // all parts have raised theirs
-          for (int p0 = lane; p0 < n_parts; p0 += 32) flags[p0] = 0u;
-      }
-      if (lane == 0) {
-        __threadfence();
-        *is_last = last;
-      }
-    }
+    if (warp == 0) elect_combiner(a, u, unit_slot, cta - c_first, n_parts, lane, is_last);
     __syncthreads();
     if (*is_last) {
       combine_and_store<kHG>(a, b, hk, g_heads, unit_slot, n_parts, reinterpret_cast<float*>(smem + kSmRing));

@@ -1,0 +1,465 @@
+// Attention of a few queries per sequence (drafted tokens, short chunks) and of one query with more than four heads per kv
+// head, head_dim 128 (included by pq_decode.cu): the persistent kernel of pq_decode_fast.cuh with up to 32 (query, head) rows
+// per decoded key and value.
+//
+// A unit is (sequence, kv head, row block); a row block is 4 kHG rows, row r = query r / g, head r % g of the kv head's
+// group, each with its own causal limit.  Tiles are decoded exactly as in the persistent kernel, then the score and value
+// MMAs run once per group of four rows on the same fragments.  Decoding is three quarters of a four-row tile, so 20 rows
+// cost far less than five calls: it is bound by instruction issue, like the persistent kernel.
+// Eight warps with up to 255 registers (16 accumulators per group of rows, all in registers) instead of sixteen with 128; the
+// query fragments stay in shared memory (one conflict-free 8-byte read per MMA pair).  All four ring slots belong to the one
+// group of eight warps, so copies run three stages ahead.
+#pragma once
+
+namespace pq {
+
+constexpr int kRowWarps = 8, kRowThreads = kRowWarps * 32;
+constexpr int kRowMax = 32;                                // rows of a row block
+constexpr int kRowSmQ = kSmSegs + 768;                     // q' fragments [row group][k-step][lane], 8 bytes
+constexpr int kRowSmRing = (kRowSmQ + 8 * 8 * 32 * 8 + 127) / 128 * 128;
+constexpr int kRowQIn = kStages * kStageBytes;             // behind the ring: 16 rows of q in float32
+constexpr int kRowMergeMl = kRowWarps * 16 * kMrgStride * 4;   // in the merge buffer, behind 16 rows of every warp: (m, l)
+constexpr int kRowMergeBytes = kRowMergeMl + kRowWarps * kRowMax * 8;
+constexpr int kRowCombineFloats = kRowMax * kFastMaxGrid + kRowMax + kRowMax * 128;
+constexpr int kRowRingBytes = kRowQIn + 16 * 512 > kRowMergeBytes ? kRowQIn + 16 * 512 : kRowMergeBytes;
+constexpr int kRowSmTotal = kRowSmRing + kRowRingBytes + kSmAlign;
+static_assert(kRowCombineFloats * 4 <= kRowRingBytes, "the combine uses the ring");
+static_assert(kRowSmTotal <= 227 * 1024, "shared memory of one CTA");
+
+// The last part of a unit: merge the `ns` partials of its rows in slot order, normalise, rotate back by S^T and store.
+__device__ __forceinline__ void combine_rows(const DecodeArgs& a, int seq, int hk, int row0, int n_rows, int slot0, int ns, float* sm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = a.n_q_heads / a.n_kv_heads, R = a.rows_per_block;
+  float* w_sm = sm;                                // [row][ns]
+  float* linv_sm = w_sm + kRowMax * kFastMaxGrid;  // [row]
+  float* o_sm = linv_sm + kRowMax;                 // [row][128]
+#pragma unroll 1
+  for (int r = warp; r < n_rows; r += kRowWarps) {   // a warp per row: weights of the parts
+    const float2* mlp = reinterpret_cast<const float2*>(a.ws.ml) + (int64_t)slot0 * R + r;
+    float M = -CUDART_INF_F;
+    for (int s = lane; s < ns; s += 32) M = fmaxf(M, __ldcg(mlp + (int64_t)s * R).x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    float L = 0.f;
+    for (int s = lane; s < ns; s += 32) {
+      const float2 ml = __ldcg(mlp + (int64_t)s * R);
+      const float w = ml.x == -CUDART_INF_F ? 0.f : fast_exp2(ml.x - M);
+      w_sm[r * kFastMaxGrid + s] = w;
+      L = fmaf(ml.y, w, L);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    if (lane == 0) {
+      linv_sm[r] = L > 0.f ? 1.f / L : 0.f;
+      const int j = (row0 + r) / g;
+      if (a.lse != nullptr)   // scores are in the log2 domain
+        a.lse[((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g + (row0 + r - j * g)] =
+            L > 0.f ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
+      else if (!(L > 0.f)) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int i = tid; i < n_rows * 32; i += kRowThreads) {   // four coordinates of a row
+    const int r = i >> 5;
+    const float4* op = reinterpret_cast<const float4*>(a.ws.o + ((int64_t)slot0 * R + r) * 128) + (i & 31);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int s = 0; s < ns; ++s) {
+      const float4 v = __ldcg(op + (int64_t)s * R * 32);
+      const float w = w_sm[r * kFastMaxGrid + s];
+      acc.x = fmaf(v.x, w, acc.x);
+      acc.y = fmaf(v.y, w, acc.y);
+      acc.z = fmaf(v.z, w, acc.z);
+      acc.w = fmaf(v.w, w, acc.w);
+    }
+    const float k = linv_sm[r];
+    *reinterpret_cast<float4*>(o_sm + 4 * i) = make_float4(acc.x * k, acc.y * k, acc.z * k, acc.w * k);
+  }
+  __syncthreads();
+  // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of eight rows at a time
+  const int i = tid & 127;
+  const float4* srow = reinterpret_cast<const float4*>(a.S + i * 128);
+#pragma unroll 1
+  for (int r0 = (tid >> 7) * 8; r0 < n_rows; r0 += 16) {
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+      const float4 s = __ldg(srow + j);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float4 y = *reinterpret_cast<const float4*>(o_sm + (r0 + r) * 128 + 4 * j);   // rows past n_rows are not stored
+        acc[r] = fmaf(y.w, s.w, fmaf(y.z, s.z, fmaf(y.y, s.y, fmaf(y.x, s.x, acc[r]))));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r0 + r < n_rows) {
+        const int j = (row0 + r0 + r) / g;
+        const int64_t idx = (((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g + (row0 + r0 + r - j * g)) * 128 + i;
+        if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(acc[r]);
+        else reinterpret_cast<float*>(a.out)[idx] = acc[r];
+      }
+  }
+}
+
+template <int kHG, bool kPaged>
+__global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((kSmAlign - (smem_u32(smem_raw) & (kSmAlign - 1))) & (kSmAlign - 1));
+  const int g_heads = a.n_q_heads / a.n_kv_heads, all_rows = a.n_q * g_heads, R = a.rows_per_block, nrb = a.n_row_blocks;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t sm_base = smem_u32(smem);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kSmFlags);
+  int* is_last = reinterpret_cast<int*>(smem + kSmFlags) + 1;
+  int* n_segs = reinterpret_cast<int*>(smem + kSmFlags) + 2;
+  int* first_rank = reinterpret_cast<int*>(smem + kSmFlags) + 3;
+  Segment* segs = reinterpret_cast<Segment*>(smem + kSmSegs);
+  const int64_t head_bytes = make_layout(128, a.pg.page_tokens).head_bytes;
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(sm_base + kSmBar + 8 * s, 1);                          // full: producer + tx bytes
+      mbar_init(sm_base + kSmBar + 8 * (kStages + s), kRowWarps);      // empty: one arrive per warp
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // a programmatic dependent of the kernel before it, like the persistent kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  build_fast_tables<kRowThreads>(smem, a.tables);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncthreads();
+
+  const int n_units = a.batch / a.n_q * a.n_kv_heads * nrb, cta = blockIdx.x;
+  // rows of a unit's block, tokens its last row sees (query j sees the tokens t < len - (n_q - 1 - j))
+  auto unit_rows = [&](int rb) -> int { return min(R, all_rows - rb * R); };
+  auto unit_len = [&](int seq, int rb) -> int {
+    const int v = a.lens[seq] - (a.n_q - 1 - (rb * R + unit_rows(rb) - 1) / g_heads);
+    return v > 0 ? v : 0;
+  };
+  auto stages_of = [&](int u) -> int {
+    const int len_u = u < n_units ? unit_len(u / (a.n_kv_heads * nrb), u % nrb) : 0;
+    return (len_u + kStageTokens - 1) / kStageTokens;
+  };
+  auto empty_unit = [&](int u) {   // no row sees a token: zeros, and the status says so
+    const int seq = u / (a.n_kv_heads * nrb), rb = u % nrb, hk = (u / nrb) % a.n_kv_heads, n_rows = unit_rows(rb);
+#pragma unroll 1
+    for (int e = 0; e < n_rows * 128; ++e) {
+      const int row = rb * R + (e >> 7), j = row / g_heads;
+      const int64_t idx = (((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g_heads + (row - j * g_heads)) * 128 + (e & 127);
+      if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
+      else reinterpret_cast<float*>(a.out)[idx] = 0.f;
+      if (a.lse != nullptr && (e & 127) == 0) a.lse[idx >> 7] = -CUDART_INF_F;
+    }
+    if (a.lse == nullptr) set_status(a.status, PQ_ERR_EMPTY);
+  };
+
+  const int g = lane >> 2, c = lane & 3;
+  const uint32_t rep = (lane & 15) * 8;
+  const uint32_t ua = sm_base + kSmU + rep, t1a = sm_base + kSmT1p + rep;
+  const int tk_k = (warp & 3) * 16 + g, tk_v = (warp & 3) * 16 + c;   // see decode_attention_fast_kernel
+  const uint32_t ok_l1 = tk_k * 32 + c * 8, ok_r = kORad + tk_k * 16 + c * 4;
+  const uint32_t ok_c2 = kO2 + tk_k * 8 + c * 2, ok_c3 = kO3 + tk_k * 4 + c, ok_c4 = kO4 + tk_k * 2;
+  const uint32_t ov_l1 = tk_v * 32 + g * 4, ov_r = kORad + tk_v * 16 + g * 2;
+  const uint32_t ov_c2 = kO2 + tk_v * 8 + g, ov_c3 = kO3 + tk_v * 4 + (lane >> 3), ov_c4 = kO4 + tk_v * 2;
+  const uint32_t qf = sm_base + kRowSmQ + lane * 8;
+  int gl0 = 0;   // stages streamed so far
+
+  int my_units = list_segments<kRowThreads>(0, n_units, smem + kRowSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
+  for (int batch_no = 0; batch_no * kFastMaxSegs < my_units; ++batch_no) {
+    if (batch_no > 0)
+      my_units = list_segments<kRowThreads>(batch_no, n_units, smem + kRowSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
+    const int my_segs = min(kFastMaxSegs, my_units - batch_no * kFastMaxSegs);
+    for (int sg = 0; sg < my_segs; ++sg) {
+      const int u = segs[sg].unit, st0 = segs[sg].st0, st1 = segs[sg].st1;
+      const int n_parts = segs[sg].n_parts, unit_slot = segs[sg].slot0, part = segs[sg].part;
+      const int seq = u / (a.n_kv_heads * nrb), rb = u % nrb, hk = (u / nrb) % a.n_kv_heads;
+      const int row0 = rb * R, n_rows = unit_rows(rb), len = unit_len(seq, rb);
+      const int nblk_total = (len + kTokenBlock - 1) / kTokenBlock;
+      const uint8_t* head_base = a.cache + ((int64_t)seq * a.n_kv_heads + hk) * head_bytes;  // of a contiguous cache
+
+      float o_acc[kHG][4][4];
+      float m_run[kHG], l_run[kHG];   // of row c + 4 hg, as in the persistent kernel
+      int limit[kHG];                 // tokens the row sees
+#pragma unroll
+      for (int hg = 0; hg < kHG; ++hg) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o_acc[hg][i][0] = o_acc[hg][i][1] = o_acc[hg][i][2] = o_acc[hg][i][3] = 0.f;
+        m_run[hg] = -CUDART_INF_F;
+        l_run[hg] = 0.f;
+        const int row = c + 4 * hg;
+        limit[hg] = row < n_rows ? a.lens[seq] - (a.n_q - 1 - (row0 + row) / g_heads) : 0;
+      }
+      const int n_li = st1 - st0;
+      int issued = 0;
+      auto issue_copy = [&](int li) {
+        const int gl = gl0 + li, s = gl % kStages;
+        if (gl >= kStages && !mbar_wait(sm_base + kSmBar + 8 * (kStages + s), (gl / kStages - 1) & 1, abort_flag)) return;
+        const int st = st0 + li;
+        const uint32_t bytes = min(2, nblk_total - 2 * st) * 2 * kBlockBytes128;
+        mbar_expect_tx(sm_base + kSmBar + 8 * s, bytes);
+        const uint8_t* src = head_base + (int64_t)st * kStageBytes;
+        if (kPaged) {
+          Layout Lp;  // the two fields the offset needs
+          Lp.block_bytes = kBlockBytes128;
+          Lp.head_bytes = head_bytes;
+          src = a.cache + kv_block_pair_offset(Lp, a.pg, a.n_kv_heads, seq, hk, 2 * st, a.status);
+        }
+        bulk_load(sm_base + kRowSmRing + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
+        issued = li + 1;
+      };
+      if (tid == 0)
+        for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
+      __syncwarp();
+      // q' = (q S) * scale * log2(e) of the rows, 16 rows at a time, as fp16 value + residual in fragment order: the fragment of
+      // (row group, k-step ks, lane) holds, for column n = lane / 4 (row n / 2 of the group; value or residual), coordinates
+      // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.
+      {
+        float* q_in = reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn);
+        constexpr int kAt = 4 * kHG < 16 ? 4 * kHG : 16, kMine = kAt / 2;   // rows at a time; rows of a thread
+        const int j = tid & 127, r_mine = (tid >> 7) * kMine;               // its rotated coordinate
+        const int blk = j >> 4, ks = (blk & 1) * 4 + ((j >> 2) & 3);
+        uint8_t* dst = smem + kRowSmQ + ks * 256 + (blk >> 1) * 8 + (j & 1) * 4 + ((j >> 1) & 1) * 2;
+#pragma unroll 1
+        for (int r0 = 0; r0 < 4 * kHG; r0 += kAt) {
+          __syncthreads();
+          for (int i = tid; i < kAt * 128; i += kRowThreads) {
+            const int r = r0 + (i >> 7);
+            float v = 0.f;
+            if (r < n_rows) {
+              const int jq = (row0 + r) / g_heads;
+              const int64_t idx = (((int64_t)seq * a.n_q + jq) * a.n_q_heads + hk * g_heads + (row0 + r - jq * g_heads)) * 128 + (i & 127);
+              v = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[idx])
+                                              : reinterpret_cast<const float*>(a.q)[idx];
+            }
+            q_in[i] = v;
+          }
+          __syncthreads();
+          float acc[kMine];
+#pragma unroll
+          for (int r = 0; r < kMine; ++r) acc[r] = 0.f;
+#pragma unroll 4
+          for (int k = 0; k < 128; k += 4) {
+            float s[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = __ldg(a.S + (k + e) * 128 + j);
+#pragma unroll
+            for (int r = 0; r < kMine; ++r) {
+              const float4 q4 = *reinterpret_cast<const float4*>(q_in + (r_mine + r) * 128 + k);
+              acc[r] = fmaf(q4.w, s[3], fmaf(q4.z, s[2], fmaf(q4.y, s[1], fmaf(q4.x, s[0], acc[r]))));
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < kMine; ++r) {
+            const int row = r0 + r_mine + r;
+            const float v = acc[r] * (a.scale * 1.4426950408889634f);
+            const __half qh = __float2half_rn(v);
+            __half* at = reinterpret_cast<__half*>(dst + (row >> 2) * 2048 + 2 * (row & 3) * 32);
+            at[0] = qh;
+            at[16] = __float2half_rn(v - __half2float(qh));
+          }
+        }
+        __syncthreads();
+      }
+#pragma unroll 1
+      for (int li = 0; li < n_li; ++li) {
+        const int gl = gl0 + li, s = gl % kStages, st = st0 + li;
+        if (tid == 0 && li + kStages - 1 < n_li) issue_copy(li + kStages - 1);
+        __syncwarp();
+        if (!mbar_wait(sm_base + kSmBar + 8 * s, (gl / kStages) & 1, abort_flag)) break;
+        const int tile_tok0 = st * kStageTokens + warp * 16;
+        if (tile_tok0 < len) {
+          const uint32_t kblk = sm_base + kRowSmRing + s * kStageBytes + (warp >> 2) * 2 * kBlockBytes128;
+          const uint32_t vblk = kblk + kBlockBytes128;
+          // scores: the residual operand's MMA first, into the same accumulators (small terms first)
+          float sc[kHG][4];
+#pragma unroll
+          for (int hg = 0; hg < kHG; ++hg)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sc[hg][i] = 0.f;
+          {
+            const uint2 l1A = lds64i<0>(kblk + ok_l1), l1B = lds64i<8 * 32>(kblk + ok_l1);
+            const uint32_t rrA = lds32i<0>(kblk + ok_r), rrB = lds32i<8 * 16>(kblk + ok_r);
+            const uint32_t c2A = lds16i<0>(kblk + ok_c2), c2B = lds16i<8 * 8>(kblk + ok_c2);
+            const uint32_t c3A = lds8i<0>(kblk + ok_c3), c3B = lds8i<8 * 4>(kblk + ok_c3);
+            const uint32_t c4A = lds16i<0>(kblk + ok_c4) >> (4 * c), c4B = lds16i<8 * 2>(kblk + ok_c4) >> (4 * c);
+#define PQ_KSTEP(H, S)                                                                                      \
+  {                                                                                                         \
+    __half2 xhA, yhA, xlA, ylA, xhB, yhB, xlB, ylB;                                                         \
+    sub_block_hilo<S>(bA, t1a, xhA, yhA, xlA, ylA);                                                         \
+    sub_block_hilo<S>(bB, t1a, xhB, yhB, xlB, ylB);                                                         \
+    uint2 qv[kHG];                                                                                          \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) qv[hg] = lds64(qf + hg * 2048 + (4 * (H) + (S)) * 256); \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg)                                                      \
+        mma_16816(sc[hg], as_u32(xlA), as_u32(xlB), as_u32(ylA), as_u32(ylB), qv[hg].x, qv[hg].y);          \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg)                                                      \
+        mma_16816(sc[hg], as_u32(xhA), as_u32(xhB), as_u32(yhA), as_u32(yhB), qv[hg].x, qv[hg].y);          \
+  }
+            {
+              const BlockRef bA = make_block_ref(l1A.x, c2A, c3A, c4A & 3u, __low2half2(as_h2(rrA)), ua);
+              const BlockRef bB = make_block_ref(l1B.x, c2B, c3B, c4B & 3u, __low2half2(as_h2(rrB)), ua);
+              PQ_KSTEP(0, 0) PQ_KSTEP(0, 1) PQ_KSTEP(0, 2) PQ_KSTEP(0, 3)
+            }
+            {
+              const BlockRef bA = make_block_ref(l1A.y, c2A >> 8, c3A >> 4, (c4A >> 2) & 3u, __high2half2(as_h2(rrA)), ua);
+              const BlockRef bB = make_block_ref(l1B.y, c2B >> 8, c3B >> 4, (c4B >> 2) & 3u, __high2half2(as_h2(rrB)), ua);
+              PQ_KSTEP(1, 0) PQ_KSTEP(1, 1) PQ_KSTEP(1, 2) PQ_KSTEP(1, 3)
+            }
+#undef PQ_KSTEP
+          }
+          // online softmax, lazily updated reference (see the persistent kernel); a row may see nothing of the tile, or
+          // nothing at all yet: its reference is then -inf and its p are 2^-inf = 0
+          const int t0 = tile_tok0 + g;
+          bool over = false;
+#pragma unroll
+          for (int hg = 0; hg < kHG; ++hg) {
+            sc[hg][0] = t0 < limit[hg] ? sc[hg][0] + sc[hg][1] : -CUDART_INF_F;
+            sc[hg][1] = t0 + 8 < limit[hg] ? sc[hg][2] + sc[hg][3] : -CUDART_INF_F;
+            over = over || fmaxf(sc[hg][0], sc[hg][1]) > m_run[hg] + kLazyMax;
+          }
+          if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+            for (int hg = 0; hg < kHG; ++hg) {
+              float mx = fmaxf(sc[hg][0], sc[hg][1]);
+              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+              const float m_new = fmaxf(m_run[hg], mx);
+              const float corr = m_run[hg] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[hg] - m_new);
+              l_run[hg] *= corr;
+              m_run[hg] = m_new;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                o_acc[hg][i][0] *= corr;
+                o_acc[hg][i][1] *= corr;
+                o_acc[hg][i][2] *= corr;
+                o_acc[hg][i][3] *= corr;
+              }
+            }
+          }
+          uint32_t pb[kHG][2][2];   // B operand of the value MMAs, as in the persistent kernel
+#pragma unroll
+          for (int hg = 0; hg < kHG; ++hg) {
+            const float m = m_run[hg] == -CUDART_INF_F ? 0.f : m_run[hg];
+            const float p0 = fast_exp2(sc[hg][0] - m), p1 = fast_exp2(sc[hg][1] - m);
+            l_run[hg] += p0 + p1;
+            const uint32_t ph = as_u32(__floats2half2_rn(p0, p1));
+            const int srcA = c * 4 + (g >> 1);
+            const uint32_t uA = __shfl_sync(0xffffffffu, ph, srcA), uB = __shfl_sync(0xffffffffu, ph, srcA + 16);
+            const uint32_t sel_lo = (g & 1) ? 0x1044u : 0x4410u, sel_hi = (g & 1) ? 0x3244u : 0x4432u;
+            pb[hg][0][0] = __byte_perm(uA, 0u, sel_lo);
+            pb[hg][0][1] = __byte_perm(uB, 0u, sel_lo);
+            pb[hg][1][0] = __byte_perm(uA, 0u, sel_hi);
+            pb[hg][1][1] = __byte_perm(uB, 0u, sel_hi);
+          }
+          {
+            BlockRef bv[4];
+#define PQ_VLOAD(J)                                                                                          \
+  {                                                                                                          \
+    const uint32_t l1 = lds32i<4 * (J) * 32>(vblk + ov_l1);                                                  \
+    uint32_t rr = lds16i<4 * (J) * 16>(vblk + ov_r);                                                         \
+    const uint32_t c2 = lds8i<4 * (J) * 8>(vblk + ov_c2);                                                    \
+    const uint32_t c3 = lds8i<4 * (J) * 4>(vblk + ov_c3) >> (4 * (g & 1));                                   \
+    const uint32_t c4 = lds16i<4 * (J) * 2>(vblk + ov_c4) >> (2 * g);                                        \
+    if (tile_tok0 + c + 4 * (J) >= len) rr = 0u; /* stale bytes past the sequence end stay out of the sums */ \
+    bv[J] = make_block_ref(l1, c2, c3, c4 & 3u, as_h2(rr | (rr << 16)), ua);                                 \
+  }
+            PQ_VLOAD(0) PQ_VLOAD(1) PQ_VLOAD(2) PQ_VLOAD(3)
+#undef PQ_VLOAD
+#define PQ_VSTEP(S)                                                                                        \
+  {                                                                                                        \
+    __half2 x0, y0, x1, y1, x2, y2, x3, y3;                                                                \
+    sub_block_h2<S>(bv[0], t1a, x0, y0);                                                                   \
+    sub_block_h2<S>(bv[1], t1a, x1, y1);                                                                   \
+    sub_block_h2<S>(bv[2], t1a, x2, y2);                                                                   \
+    sub_block_h2<S>(bv[3], t1a, x3, y3);                                                                   \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg)                                                     \
+        mma_16816(o_acc[hg][S], as_u32(x0), as_u32(y0), as_u32(x1), as_u32(y1), pb[hg][0][0], pb[hg][0][1]); \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg)                                                     \
+        mma_16816(o_acc[hg][S], as_u32(x2), as_u32(y2), as_u32(x3), as_u32(y3), pb[hg][1][0], pb[hg][1][1]); \
+  }
+            PQ_VSTEP(0) PQ_VSTEP(1) PQ_VSTEP(2) PQ_VSTEP(3)
+#undef PQ_VSTEP
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sm_base + kSmBar + 8 * (kStages + s));
+      }
+      gl0 += n_li;
+      __syncthreads();
+      if (*abort_flag) {   // gave up: let the copies still in flight land (bounded) before the ring is reused
+        if (tid == 0)
+          for (int li = max(0, issued - kStages); li < issued; ++li) {
+            const int gl = gl0 - n_li + li;
+            for (int i = 0; i < kSpinLimit && !mbar_try_wait(sm_base + kSmBar + 8 * (gl % kStages), (gl / kStages) & 1); ++i)
+              __nanosleep(64);
+          }
+        __syncthreads();
+      }
+
+      // ---- merge the warps (fixed order), 16 rows at a time; write this part's partial; the last part combines the unit
+      float* mrg_o = reinterpret_cast<float*>(smem + kRowSmRing);                 // [warps][16 rows][kMrgStride]
+      float* mrg_ml = reinterpret_cast<float*>(smem + kRowSmRing + kRowMergeMl);  // [warps][kRowMax][2]
+#pragma unroll
+      for (int hg = 0; hg < kHG; ++hg) {
+        l_run[hg] += __shfl_xor_sync(0xffffffffu, l_run[hg], 4);
+        l_run[hg] += __shfl_xor_sync(0xffffffffu, l_run[hg], 8);
+        l_run[hg] += __shfl_xor_sync(0xffffffffu, l_run[hg], 16);
+        if (g == 0) *reinterpret_cast<float2*>(mrg_ml + (warp * kRowMax + c + 4 * hg) * 2) = make_float2(m_run[hg], l_run[hg]);
+      }
+      __syncthreads();
+      const int slot = unit_slot + part;
+#pragma unroll
+      for (int h0 = 0; h0 < kHG; h0 += 4) {
+        if (4 * h0 >= n_rows) break;
+        if (h0 > 0) __syncthreads();
+#pragma unroll
+        for (int hg = h0; hg < h0 + 4 && hg < kHG; ++hg) {
+          float M = -CUDART_INF_F;
+#pragma unroll
+          for (int w = 0; w < kRowWarps; ++w) M = fmaxf(M, mrg_ml[(w * kRowMax + c + 4 * hg) * 2]);
+          const float wgt = m_run[hg] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[hg] - M);
+          float* o0 = mrg_o + (warp * 16 + c + 4 * (hg - h0)) * kMrgStride + g;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            o0[(4 * i) * 8] = o_acc[hg][i][0] * wgt;
+            o0[(4 * i + 2) * 8] = o_acc[hg][i][1] * wgt;
+            o0[(4 * i + 1) * 8] = o_acc[hg][i][2] * wgt;
+            o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
+          }
+        }
+        __syncthreads();
+        const int n_here = min(16, n_rows - 4 * h0);
+#pragma unroll 1
+        for (int i = tid; i < n_here * 128; i += kRowThreads) {
+          const int r = i >> 7, j = i & 127;
+          float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int w = 0; w < kRowWarps; ++w) acc[w & 3] += mrg_o[(w * 16 + r) * kMrgStride + (j & 15) * 8 + (j >> 4)];
+          __stcg(a.ws.o + ((int64_t)slot * R + 4 * h0 + r) * 128 + j, (acc[0] + acc[1]) + (acc[2] + acc[3]));
+        }
+      }
+      if (tid < n_rows) {
+        float M = -CUDART_INF_F, l = 0.f;
+#pragma unroll
+        for (int w = 0; w < kRowWarps; ++w) M = fmaxf(M, mrg_ml[(w * kRowMax + tid) * 2]);
+#pragma unroll
+        for (int w = 0; w < kRowWarps; ++w) {
+          const float2 ml = *reinterpret_cast<const float2*>(mrg_ml + (w * kRowMax + tid) * 2);
+          l += ml.x == -CUDART_INF_F ? 0.f : ml.y * fast_exp2(ml.x - M);
+        }
+        __stcg(reinterpret_cast<float2*>(a.ws.ml) + (int64_t)slot * R + tid, make_float2(M, l));
+      }
+      __syncthreads();
+      if (warp == 0) elect_combiner(a, u, unit_slot, part, n_parts, lane, is_last);
+      __syncthreads();
+      if (*is_last) {
+        combine_rows(a, seq, hk, row0, n_rows, unit_slot, n_parts, reinterpret_cast<float*>(smem + kRowSmRing));
+        if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
+      }
+      __syncthreads();  // the ring is free again for the next unit
+    }
+  }
+  if (tid == 0 && *abort_flag) set_status(a.status, PQ_ERR_TIMEOUT);
+}
+
+}  // namespace pq
