@@ -17,43 +17,57 @@ constexpr int kRowWarps = 8, kRowThreads = kRowWarps * 32;
 constexpr int kRowMax = 32;                                // rows of a row block
 constexpr int kRowSmQ = kSmSegs + 768;                     // q' fragments [row group][k-step][lane], 8 bytes
 constexpr int kRowSmRing = (kRowSmQ + 8 * 8 * 32 * 8 + 127) / 128 * 128;
-constexpr int kRowQIn = kStages * kStageBytes;             // behind the ring: 16 rows of q in float32
+// S, rows 528 bytes apart (a thread per row reads it without bank conflicts), lies where the ring is: before the first copies
+// of a segment for the rotation of the queries, and after the merge for the last part's un-rotation; behind it 16 rows of q in
+// float32.  Both products are rolled loops over shared memory: straight-line code that runs once per segment takes longer
+// to fetch (5.7 us for 16 rows) than to run.
+constexpr int kRowSStride = 132, kRowQIn = 128 * kRowSStride * 4;
 constexpr int kRowMergeMl = kRowWarps * 16 * kMrgStride * 4;   // in the merge buffer, behind 16 rows of every warp: (m, l)
 constexpr int kRowMergeBytes = kRowMergeMl + kRowWarps * kRowMax * 8;
-constexpr int kRowCombineFloats = kRowMax * kFastMaxGrid + kRowMax + kRowMax * 128;
 constexpr int kRowRingBytes = kRowQIn + 16 * 512 > kRowMergeBytes ? kRowQIn + 16 * 512 : kRowMergeBytes;
 constexpr int kRowSmTotal = kRowSmRing + kRowRingBytes + kSmAlign;
-static_assert(kRowCombineFloats * 4 <= kRowRingBytes, "the combine uses the ring");
+constexpr int kRowSmInfo = kSmSegs + 448;                  // int2 [kRowMax]: the row's index in q and out, tokens it sees
+constexpr int kRowSmBarS = kSmSegs + 752;                  // mbarrier of the copies of S (the segments take 384 bytes)
+static_assert(kStages * kStageBytes <= kRowRingBytes, "ring");
+static_assert(kFastMaxSegs * sizeof(Segment) <= 448 && 448 + kRowMax * 8 <= 752 && kRowSmInfo % 8 == 0, "behind the segments");
 static_assert(kRowSmTotal <= 227 * 1024, "shared memory of one CTA");
 
-// The last part of a unit: merge the `ns` partials of its rows in slot order, normalise, rotate back by S^T and store.
-__device__ __forceinline__ void combine_rows(const DecodeArgs& a, int seq, int hk, int row0, int n_rows, int slot0, int ns, float* sm) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = a.n_q_heads / a.n_kv_heads, R = a.rows_per_block;
-  float* w_sm = sm;                                // [row][ns]
-  float* linv_sm = w_sm + kRowMax * kFastMaxGrid;  // [row]
-  float* o_sm = linv_sm + kRowMax;                 // [row][128]
+// One warp: copy S into the ring's place (nothing in it is in use any more; a barrier has ordered what was).
+__device__ __forceinline__ void fetch_S(const float* S, uint32_t ring, uint32_t bar, int lane) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (lane == 0) mbar_expect_tx(bar, 128 * 512);
+  __syncwarp();
 #pragma unroll 1
-  for (int r = warp; r < n_rows; r += kRowWarps) {   // a warp per row: weights of the parts
-    const float2* mlp = reinterpret_cast<const float2*>(a.ws.ml) + (int64_t)slot0 * R + r;
-    float M = -CUDART_INF_F;
-    for (int s = lane; s < ns; s += 32) M = fmaxf(M, __ldcg(mlp + (int64_t)s * R).x);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    float L = 0.f;
-    for (int s = lane; s < ns; s += 32) {
+  for (int r = lane; r < 128; r += 32) bulk_load(ring + r * kRowSStride * 4, S + r * 128, 512, bar);
+}
+
+// The last part of a unit: merge the `ns` partials of its rows in slot order, normalise, rotate back by S^T and store.
+// `y_sm`: kRowMax * 128 floats, `stat`: 2 * kRowMax; S_sm: see fetch_S (the caller has started it; waited for on `bar`, `phase`).
+__device__ __forceinline__ void combine_rows(const DecodeArgs& a, const int2* info, int n_rows, int slot0, int ns, float* y_sm,
+                                             float* stat, const float* S_sm, uint32_t bar, uint32_t phase, volatile int* abort_flag) {
+  const int tid = threadIdx.x, R = a.rows_per_block;
+  {   // eight lanes per row: common reference and denominator
+    const int r = tid >> 3, l8 = tid & 7;
+    const float2* mlp = reinterpret_cast<const float2*>(a.ws.ml) + (int64_t)slot0 * R + min(r, n_rows - 1);
+    float M = -CUDART_INF_F, L = 0.f;
+#pragma unroll 2
+    for (int s = l8; s < ns; s += 8) {
       const float2 ml = __ldcg(mlp + (int64_t)s * R);
-      const float w = ml.x == -CUDART_INF_F ? 0.f : fast_exp2(ml.x - M);
-      w_sm[r * kFastMaxGrid + s] = w;
-      L = fmaf(ml.y, w, L);
+      const float m_new = fmaxf(M, ml.x);
+      if (m_new > -CUDART_INF_F) L = L * fast_exp2(M - m_new) + ml.y * fast_exp2(ml.x - m_new);
+      M = m_new;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-    if (lane == 0) {
-      linv_sm[r] = L > 0.f ? 1.f / L : 0.f;
-      const int j = (row0 + r) / g;
+    for (int o = 4; o > 0; o >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, M, o), l2 = __shfl_xor_sync(0xffffffffu, L, o), m_new = fmaxf(M, m2);
+      if (m_new > -CUDART_INF_F) L = L * fast_exp2(M - m_new) + l2 * fast_exp2(m2 - m_new);
+      M = m_new;
+    }
+    if (l8 == 0 && r < n_rows) {
+      stat[2 * r] = M;
+      stat[2 * r + 1] = L > 0.f ? 1.f / L : 0.f;
       if (a.lse != nullptr)   // scores are in the log2 domain
-        a.lse[((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g + (row0 + r - j * g)] =
-            L > 0.f ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
+        a.lse[info[r].x] = L > 0.f ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
       else if (!(L > 0.f)) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token
     }
   }
@@ -62,40 +76,42 @@ __device__ __forceinline__ void combine_rows(const DecodeArgs& a, int seq, int h
   for (int i = tid; i < n_rows * 32; i += kRowThreads) {   // four coordinates of a row
     const int r = i >> 5;
     const float4* op = reinterpret_cast<const float4*>(a.ws.o + ((int64_t)slot0 * R + r) * 128) + (i & 31);
+    const float2* mlp = reinterpret_cast<const float2*>(a.ws.ml) + (int64_t)slot0 * R + r;
+    const float M = stat[2 * r], k = stat[2 * r + 1];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
+#pragma unroll 4
     for (int s = 0; s < ns; ++s) {
       const float4 v = __ldcg(op + (int64_t)s * R * 32);
-      const float w = w_sm[r * kFastMaxGrid + s];
+      const float m = __ldcg(mlp + (int64_t)s * R).x;
+      const float w = m == -CUDART_INF_F ? 0.f : fast_exp2(m - M);
       acc.x = fmaf(v.x, w, acc.x);
       acc.y = fmaf(v.y, w, acc.y);
       acc.z = fmaf(v.z, w, acc.z);
       acc.w = fmaf(v.w, w, acc.w);
     }
-    const float k = linv_sm[r];
-    *reinterpret_cast<float4*>(o_sm + 4 * i) = make_float4(acc.x * k, acc.y * k, acc.z * k, acc.w * k);
+    *reinterpret_cast<float4*>(y_sm + 4 * i) = make_float4(acc.x * k, acc.y * k, acc.z * k, acc.w * k);
   }
+  mbar_wait(bar, phase, abort_flag);
   __syncthreads();
-  // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of eight rows at a time
-  const int i = tid & 127;
-  const float4* srow = reinterpret_cast<const float4*>(a.S + i * 128);
+  // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of four rows at a time
+  const int i_out = tid & 127;
+  const float* srow = S_sm + i_out * kRowSStride;
 #pragma unroll 1
-  for (int r0 = (tid >> 7) * 8; r0 < n_rows; r0 += 16) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int r0 = (tid >> 7) * 4; r0 < n_rows; r0 += 8) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-    for (int j = 0; j < 32; ++j) {
-      const float4 s = __ldg(srow + j);
+    for (int j = 0; j < 128; j += 4) {
+      const float4 s = *reinterpret_cast<const float4*>(srow + j);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const float4 y = *reinterpret_cast<const float4*>(o_sm + (r0 + r) * 128 + 4 * j);   // rows past n_rows are not stored
+      for (int r = 0; r < 4; ++r) {
+        const float4 y = *reinterpret_cast<const float4*>(y_sm + (r0 + r) * 128 + j);   // rows past n_rows are not stored
         acc[r] = fmaf(y.w, s.w, fmaf(y.z, s.z, fmaf(y.y, s.y, fmaf(y.x, s.x, acc[r]))));
       }
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 4; ++r)
       if (r0 + r < n_rows) {
-        const int j = (row0 + r0 + r) / g;
-        const int64_t idx = (((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g + (row0 + r0 + r - j * g)) * 128 + i;
+        const int64_t idx = (int64_t)info[r0 + r].x * 128 + i_out;
         if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(acc[r]);
         else reinterpret_cast<float*>(a.out)[idx] = acc[r];
       }
@@ -120,6 +136,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
       mbar_init(sm_base + kSmBar + 8 * s, 1);                          // full: producer + tx bytes
       mbar_init(sm_base + kSmBar + 8 * (kStages + s), kRowWarps);      // empty: one arrive per warp
     }
+    mbar_init(sm_base + kRowSmBarS, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -128,6 +145,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   build_fast_tables<kRowThreads>(smem, a.tables);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
+  const uint32_t ring = sm_base + kRowSmRing, bar_S = sm_base + kRowSmBarS;
+  const float* S_sm = reinterpret_cast<const float*>(smem + kRowSmRing);
+  uint32_t n_S = 0;   // copies of S so far
 
   const int n_units = a.batch / a.n_q * a.n_kv_heads * nrb, cta = blockIdx.x;
   // rows of a unit's block, tokens its last row sees (query j sees the tokens t < len - (n_q - 1 - j))
@@ -177,18 +197,6 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
       const int nblk_total = (len + kTokenBlock - 1) / kTokenBlock;
       const uint8_t* head_base = a.cache + ((int64_t)seq * a.n_kv_heads + hk) * head_bytes;  // of a contiguous cache
 
-      float o_acc[kHG][4][4];
-      float m_run[kHG], l_run[kHG];   // of row c + 4 hg, as in the persistent kernel
-      int limit[kHG];                 // tokens the row sees
-#pragma unroll
-      for (int hg = 0; hg < kHG; ++hg) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) o_acc[hg][i][0] = o_acc[hg][i][1] = o_acc[hg][i][2] = o_acc[hg][i][3] = 0.f;
-        m_run[hg] = -CUDART_INF_F;
-        l_run[hg] = 0.f;
-        const int row = c + 4 * hg;
-        limit[hg] = row < n_rows ? a.lens[seq] - (a.n_q - 1 - (row0 + row) / g_heads) : 0;
-      }
       const int n_li = st1 - st0;
       int issued = 0;
       auto issue_copy = [&](int li) {
@@ -204,12 +212,16 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
           Lp.head_bytes = head_bytes;
           src = a.cache + kv_block_pair_offset(Lp, a.pg, a.n_kv_heads, seq, hk, 2 * st, a.status);
         }
-        bulk_load(sm_base + kRowSmRing + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
+        bulk_load(ring + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
         issued = li + 1;
       };
-      if (tid == 0)
-        for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
-      __syncwarp();
+      if (warp == 0) fetch_S(a.S, ring, bar_S, lane);
+      int2* info = reinterpret_cast<int2*>(smem + kRowSmInfo);
+      if (warp == 1) {
+        const int row = row0 + min(lane, n_rows - 1), j = row / g_heads;
+        info[lane] = make_int2((seq * a.n_q + j) * a.n_q_heads + hk * g_heads + (row - j * g_heads),
+                               lane < n_rows ? a.lens[seq] - (a.n_q - 1 - j) : 0);
+      }
       // q' = (q S) * scale * log2(e) of the rows, 16 rows at a time, as fp16 value + residual in fragment order: the fragment of
       // (row group, k-step ks, lane) holds, for column n = lane / 4 (row n / 2 of the group; value or residual), coordinates
       // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.
@@ -222,30 +234,36 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
 #pragma unroll 1
         for (int r0 = 0; r0 < 4 * kHG; r0 += kAt) {
           __syncthreads();
-          for (int i = tid; i < kAt * 128; i += kRowThreads) {
-            const int r = r0 + (i >> 7);
-            float v = 0.f;
-            if (r < n_rows) {
-              const int jq = (row0 + r) / g_heads;
-              const int64_t idx = (((int64_t)seq * a.n_q + jq) * a.n_q_heads + hk * g_heads + (row0 + r - jq * g_heads)) * 128 + (i & 127);
-              v = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[idx])
-                                              : reinterpret_cast<const float*>(a.q)[idx];
+          for (int i = tid; i < kAt * 16; i += kRowThreads) {   // eight elements of a row (rows past the last repeat it)
+            const int64_t at = (int64_t)info[r0 + (i >> 4)].x * 128 + 8 * (i & 15);
+            float4 lo, hi;
+            if (a.io_dtype == PQ_DTYPE_BF16) {
+              const uint4 w = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.q) + at);
+              lo = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                               __uint_as_float(w.y & 0xFFFF0000u));
+              hi = make_float4(__uint_as_float(w.z << 16), __uint_as_float(w.z & 0xFFFF0000u), __uint_as_float(w.w << 16),
+                               __uint_as_float(w.w & 0xFFFF0000u));
+            } else {
+              lo = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at);
+              hi = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at + 4);
             }
-            q_in[i] = v;
+            *reinterpret_cast<float4*>(q_in + 8 * i) = lo;
+            *reinterpret_cast<float4*>(q_in + 8 * i + 4) = hi;
           }
+          if (r0 == 0) mbar_wait(bar_S, n_S++ & 1, abort_flag);
           __syncthreads();
           float acc[kMine];
 #pragma unroll
           for (int r = 0; r < kMine; ++r) acc[r] = 0.f;
 #pragma unroll 4
           for (int k = 0; k < 128; k += 4) {
-            float s[4];
+            float s_col[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) s[e] = __ldg(a.S + (k + e) * 128 + j);
+            for (int e = 0; e < 4; ++e) s_col[e] = S_sm[(k + e) * kRowSStride + j];
 #pragma unroll
             for (int r = 0; r < kMine; ++r) {
               const float4 q4 = *reinterpret_cast<const float4*>(q_in + (r_mine + r) * 128 + k);
-              acc[r] = fmaf(q4.w, s[3], fmaf(q4.z, s[2], fmaf(q4.y, s[1], fmaf(q4.x, s[0], acc[r]))));
+              acc[r] = fmaf(q4.w, s_col[3], fmaf(q4.z, s_col[2], fmaf(q4.y, s_col[1], fmaf(q4.x, s_col[0], acc[r]))));
             }
           }
 #pragma unroll
@@ -258,7 +276,22 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
             at[16] = __float2half_rn(v - __half2float(qh));
           }
         }
-        __syncthreads();
+        __syncthreads();   // S has been used: the ring takes its place
+      }
+      if (tid == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
+      }
+      float o_acc[kHG][4][4];
+      float m_run[kHG], l_run[kHG];   // of row c + 4 hg, as in the persistent kernel
+      int limit[kHG];                 // tokens the row sees
+#pragma unroll
+      for (int hg = 0; hg < kHG; ++hg) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o_acc[hg][i][0] = o_acc[hg][i][1] = o_acc[hg][i][2] = o_acc[hg][i][3] = 0.f;
+        m_run[hg] = -CUDART_INF_F;
+        l_run[hg] = 0.f;
+        limit[hg] = info[c + 4 * hg].y;
       }
 #pragma unroll 1
       for (int li = 0; li < n_li; ++li) {
@@ -453,7 +486,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
       if (warp == 0) elect_combiner(a, u, unit_slot, part, n_parts, lane, is_last);
       __syncthreads();
       if (*is_last) {
-        combine_rows(a, seq, hk, row0, n_rows, unit_slot, n_parts, reinterpret_cast<float*>(smem + kRowSmRing));
+        if (warp == 0) fetch_S(a.S, ring, bar_S, lane);
+        combine_rows(a, info, n_rows, unit_slot, n_parts, reinterpret_cast<float*>(smem + kRowSmQ),
+                     reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn), S_sm, bar_S, n_S++ & 1, abort_flag);
         if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
       }
       __syncthreads();  // the ring is free again for the next unit
