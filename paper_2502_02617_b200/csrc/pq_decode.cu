@@ -1,4 +1,5 @@
 // Decode attention over the packed cache (Eq. 3) and the inspection kernels.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <chrono>
@@ -118,6 +119,9 @@ struct DecodeArgs {
   int d, n_q_heads, n_kv_heads, batch, capacity, io_dtype;
   int n_q;  // queries per sequence (1: decode).  `batch` counts (sequence, query) pairs: q and out are
             // [batch][n_q_heads][d] with pair p = sequence * n_q + query; `lens` and the cache are per sequence.
+  int n_splits;        // of prefill_tc_kernel: ranges of a sequence's blocks, each with a part of its own in
+  float* part_out;     // [split][batch][n_q_heads][128] and
+  float* part_lse;     // [split][batch][n_q_heads] (natural log), for n_splits > 1
   int rows_per_block, n_row_blocks;   // of rows_attention_kernel: its cut of a kv head's n_q * group rows
   float scale;
   uint32_t epoch;  // differs from call to call (top bit set): tags the parts' flags of the persistent kernel
@@ -264,32 +268,92 @@ static int32_t launch_packed_attention(const SplitCommon& c, int64_t pairs, int 
 // ---- partial attentions: merge, and exact attention over an uncompressed window -----------------
 // out = sum_p w_p out_p with w_p = exp(lse_p - lse) and lse = log sum_p exp(lse_p): the attention over the union of
 // the token sets behind the parts (token shards on several GPUs; the packed cache and a 16-bit tail).
-__global__ void merge_attention_kernel(int d, int64_t n_rows, int n_parts, const void* parts_out, int parts_dtype,
-                                       const float* parts_lse, void* out, int out_dtype, float* lse_out, int32_t* status) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// A thread takes kV neighbouring elements of a row (4: 16-byte loads), every part's loads independent of the others'.
+template <int kV>
+__global__ void __launch_bounds__(256) merge_attention_kernel(int d, int64_t n_rows, int n_parts, const void* parts_out, int parts_dtype,
+                                                              const float* parts_lse, void* out, int out_dtype, float* lse_out,
+                                                              int32_t* status) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the parts come from the kernels before this one
+  const int64_t idx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kV;
   if (idx >= n_rows * d) return;
   const int64_t row = idx / d;
   float mx = -CUDART_INF_F;
+#pragma unroll 8
   for (int p = 0; p < n_parts; ++p) mx = fmaxf(mx, parts_lse[(int64_t)p * n_rows + row]);
-  float acc = 0.f, wsum = 0.f;
+  float acc[kV], wsum = 0.f;
+#pragma unroll
+  for (int e = 0; e < kV; ++e) acc[e] = 0.f;
   if (mx > -CUDART_INF_F) {
+#pragma unroll 4
     for (int p = 0; p < n_parts; ++p) {   // part order: the result does not depend on the launch
       const float l = parts_lse[(int64_t)p * n_rows + row];
+      const int64_t i = (int64_t)p * n_rows * d + idx;
+      float v[kV];
+      if (parts_dtype == PQ_DTYPE_BF16) {
+        if (kV == 4) {
+          const uint2 w = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(parts_out) + i);
+          v[0] = __uint_as_float(w.x << 16);
+          v[1 % kV] = __uint_as_float(w.x & 0xFFFF0000u);
+          v[2 % kV] = __uint_as_float(w.y << 16);
+          v[3 % kV] = __uint_as_float(w.y & 0xFFFF0000u);
+        } else {
+          v[0] = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(parts_out)[i]);
+        }
+      } else if (kV == 4) {
+        const float4 w = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(parts_out) + i);
+        v[0] = w.x; v[1 % kV] = w.y; v[2 % kV] = w.z; v[3 % kV] = w.w;
+      } else {
+        v[0] = reinterpret_cast<const float*>(parts_out)[i];
+      }
       if (l == -CUDART_INF_F) continue;   // a part without tokens (its output may hold anything)
       const float w = __expf(l - mx);
-      const int64_t i = (int64_t)p * n_rows * d + idx;
-      const float v = parts_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(parts_out)[i])
-                                                   : reinterpret_cast<const float*>(parts_out)[i];
-      acc = fmaf(w, v, acc);
+#pragma unroll
+      for (int e = 0; e < kV; ++e) acc[e] = fmaf(w, v[e], acc[e]);
       wsum += w;
     }
-    acc /= wsum;
+#pragma unroll
+    for (int e = 0; e < kV; ++e) acc[e] /= wsum;
   } else if (idx == row * d) {
     set_status(status, PQ_ERR_EMPTY);
   }
-  if (out_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(out)[idx] = __float2bfloat16(acc);
-  else reinterpret_cast<float*>(out)[idx] = acc;
+  if (out_dtype == PQ_DTYPE_BF16) {
+    __nv_bfloat16 o[kV];
+#pragma unroll
+    for (int e = 0; e < kV; ++e) o[e] = __float2bfloat16(acc[e]);
+    if (kV == 4) *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(out) + idx) = *reinterpret_cast<const uint2*>(o);
+    else reinterpret_cast<__nv_bfloat16*>(out)[idx] = o[0];
+  } else if (kV == 4) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + idx) = make_float4(acc[0], acc[1 % kV], acc[2 % kV], acc[3 % kV]);
+  } else {
+    reinterpret_cast<float*>(out)[idx] = acc[0];
+  }
   if (lse_out != nullptr && idx == row * d) lse_out[row] = mx > -CUDART_INF_F ? mx + __logf(wsum) : -CUDART_INF_F;
+}
+
+static int32_t launch_merge(int d, int64_t n_rows, int n_parts, const void* parts_out, int parts_dtype, const float* parts_lse, void* out,
+                            int out_dtype, float* lse_out, int32_t* status, cudaStream_t stream) {
+  const bool wide = d % 4 == 0 && (((uintptr_t)parts_out | (uintptr_t)out) & 15) == 0;
+  const int64_t n = n_rows * d / (wide ? 4 : 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = wide ? cudaLaunchKernelEx(&cfg, merge_attention_kernel<4>, d, n_rows, n_parts, parts_out, parts_dtype, parts_lse, out,
+                                                  out_dtype, lse_out, status)
+                             : cudaLaunchKernelEx(&cfg, merge_attention_kernel<1>, d, n_rows, n_parts, parts_out, parts_dtype, parts_lse, out,
+                                                  out_dtype, lse_out, status);
+  if (e != cudaSuccess) {
+    note_cuda_error(e);
+    cudaGetLastError();
+    return PQ_ERR_CUDA;
+  }
+  return launch_status();
 }
 
 // Exact softmax attention (Eq. 2) of one query per sequence over an uncompressed window of keys and values (the
@@ -592,14 +656,114 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
   a.n_row_blocks = cut.blocks;
   a.ws = carve_workspace(a.ws.elected, 128, (int64_t)n_seq * a.n_kv_heads * cut.blocks, cut.rows);
   a.epoch = next_epoch();
-  a.debug = 0u;
-  if (cut.rows <= 4) return launch_rows_as<1>(a, paged, stream);
   if (cut.rows <= 8) return launch_rows_as<2>(a, paged, stream);
   if (cut.rows <= 12) return launch_rows_as<3>(a, paged, stream);
   if (cut.rows <= 16) return launch_rows_as<4>(a, paged, stream);
   if (cut.rows <= 20) return launch_rows_as<5>(a, paged, stream);
   if (cut.rows <= 24) return launch_rows_as<6>(a, paged, stream);
   return launch_rows_as<8>(a, paged, stream);
+}
+
+// ---- which kernel takes a head_dim-128 call ------------------------------------------------------
+// Four kernels compute the same attention; which is fastest depends on the rows per kv head (queries x heads of the group), on
+// the number of (kv head, sequence) units and on the length.  Each is estimated in us, from measurements on B200 (SM clock
+// 1.9 GHz), and the shortest estimate wins:
+//   * cluster kernel, a unit per (query, kv head, sequence): 9 us (8 with up to two heads), then 0.013 / 0.017 / 0.044 us
+//     per token of its busiest SM with up to 2 / 4 / 8 heads;
+//   * persistent kernel, up to four heads, a unit per (query, kv head, sequence): 15 us, then 280 SM cycles per 16-token tile;
+//   * rows kernel, up to 32 rows decoded together: 24 .. 43 us, then 345 + 61 (groups of four rows - 2) cycles per tile;
+//   * tcgen05 kernel: up to 128 rows (a CTA) or 256 (a pair) per decoded block; 1.25 us (pair) or 2.4 us per 64-token block,
+//     20 us per wave for setting up, rotating and un-rotating, 6 us more where a sequence is split and its parts are merged.
+enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
+struct AttentionPlan {
+  AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
+  bool pair;
+  int n_splits;
+};
+constexpr int kMaxSplits = 16;
+// Room for the parts of split tcgen05 calls in the workspace of pq_workspace_bytes: a call whose parts would not fit is split
+// less.  (148 SMs with 128 rows each, twice over, bound what a useful split can need.)
+__host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
+  return std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128);
+}
+static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm) {
+  AttentionPlan plan = {kClusterKernel, kClusterKernel, false, 1};
+  const int64_t pairs = batch * n_q, rows = (int64_t)n_q * g;
+  const double tiles = std::ceil(max_len / 16.0), sm_hz = n_sm * 1900.0;   // cycles per us of the device
+  int64_t tokens = 0;
+  split_cluster_size(128, 16, pairs * n_kv_heads, max_len, n_sm, &tokens);
+  double best = (g <= 2 ? 8.0 : 9.0) + tokens * (g <= 2 ? 0.013 : g <= 4 ? 0.017 : 0.044);
+  double best_persistent = 1e30;
+  auto consider = [&](double t, AttentionKernel k) {
+    if (k != kTensorKernel && t < best_persistent) {
+      best_persistent = t;
+      plan.persistent = k;
+    }
+    if (t >= best) return false;
+    best = t;
+    plan.kernel = k;
+    return true;
+  };
+  if (g <= 4 && pairs * n_kv_heads <= kFastMaxUnits) consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
+  const RowCut cut = cut_rows(rows);
+  if (rows > 4 && batch * n_kv_heads * cut.blocks <= kFastMaxUnits) {
+    const int groups = (cut.rows + 3) / 4;
+    consider(18.0 + 3.2 * groups + batch * n_kv_heads * cut.blocks * tiles * (345.0 + 61.0 * (groups - 2)) / sm_hz, kRowsKernel);
+  }
+  if (rows >= 32) {
+    const int qb_rows = kPtRows / g;
+    const int64_t q_blocks = (n_q + qb_rows - 1) / qb_rows, blocks = (max_len + kTokenBlock - 1) / kTokenBlock;
+    const int64_t room = part_rows_room(pairs, (int64_t)n_kv_heads * g) / (pairs * n_kv_heads * g);
+    // Two query blocks of one (kv head, sequence) per cluster: one 256-row MMA per step, each CTA decodes half of every
+    // block.  An odd count is completed by a CTA without rows, which then only shares the decoding.
+    for (int pair = 0; pair < 2; ++pair)
+      for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
+        const int64_t ctas = (pair ? (q_blocks + 1) / 2 * 2 : q_blocks) * n_kv_heads * batch * s;
+        const double waves = std::ceil((double)ctas / (pair ? n_sm / 2 * 2 : n_sm));
+        const double t = waves * (std::ceil((double)blocks / s) * (pair ? 1.25 : 2.4) + 20.0) + (s > 1 ? 6.0 : 0.0);
+        if (consider(t, kTensorKernel)) {
+          plan.pair = pair != 0;
+          plan.n_splits = s;
+        }
+      }
+  }
+  return plan;
+}
+
+static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, int n_splits, cudaStream_t stream) {
+  static DeviceMemo configured[2];
+  auto kernel = pair ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
+  if (configure_for_device(kernel, kPtSmTotal, configured[pair]) == 0) return PQ_ERR_CUDA;
+  const int qb_rows = kPtRows / (a.n_q_heads / a.n_kv_heads), q_blocks = (n_q + qb_rows - 1) / qb_rows;
+  a.debug = take_debug_wait_failure(4) ? 2u : 0u;
+  a.n_splits = n_splits;
+  a.part_lse = reinterpret_cast<float*>(a.ws.elected);   // the parts take the whole workspace
+  const int64_t part_rows = (int64_t)n_splits * a.batch * a.n_q_heads;
+  a.part_out = a.part_lse + ((part_rows + 63) & ~(int64_t)63);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pair ? (q_blocks + 1) & ~1 : q_blocks, a.n_kv_heads, batch * n_splits);
+  cfg.blockDim = dim3(kPtThreads);
+  cfg.dynamicSmemBytes = kPtSmTotal;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set up while the kernel before it finishes (it waits inside)
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pair ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a, (int)n_q);
+  if (e != cudaSuccess) {
+    note_cuda_error(e);
+    cudaGetLastError();
+    return PQ_ERR_CUDA;
+  }
+  if (n_splits > 1)
+    return launch_merge(128, (int64_t)a.batch * a.n_q_heads, n_splits, a.part_out, PQ_DTYPE_F32, a.part_lse, a.out, a.io_dtype, nullptr,
+                        a.status, stream);
+  return launch_status();
 }
 
 }  // namespace pq
@@ -616,7 +780,8 @@ int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, i
   if (head_dim != 128) return one;
   const int64_t rows = units * (g + 3) + 32 * pq::kFastMaxGridHost;
   const int64_t cut = 4 * 256 + units * 4 + (units + pq::kFastMaxGridHost) * 4 + rows * (2 + 128) * 4;
-  return units <= 2048 * 32 && cut > one ? cut : one;
+  const int64_t parts = 1024 + pq::part_rows_room(batch, n_q_heads) * (1 + 128) * 4;
+  return std::max(std::max(cut, one), parts);
 }
 
 static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, const float* S_dev,
@@ -646,112 +811,38 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.lse = lse_dev;
   a.pg = pg;
   a.ws = pq::carve_workspace(workspace_dev, head_dim, pairs * n_kv_heads, n_q_heads / n_kv_heads);
-  a.rows_per_block = a.n_row_blocks = 0;
+  a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.epoch = a.debug = 0u;
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
-  // Chunks of 32 or more rows (queries x heads of a group), d = 128: the tcgen05 kernel (operands in shared memory,
-  // accumulators in tensor memory) decodes every block once for all rows; below 128 rows it is taken when that is
-  // estimated to be faster than one decode attention per query, which spreads over all SMs whatever the batch.
-  // The register-fragment kernel is only reached through the test hook (it is the slower of the two at every size).
-  const int rows = n_q * g;
-  bool use_tc = false, use_fragment_kernel = false;
-  int n_sm = 0, q_blocks = 0;
-  bool pair = false;
-  if (head_dim == 128 && rows >= 32) {
-    static pq::DeviceMemo configured_pt, configured_pt2;
-    n_sm = pq::configure_for_device(pq::prefill_tc_kernel<false>, pq::kPtSmTotal, configured_pt);
+  if (head_dim == 128) {
+    const bool paged = pg.table != nullptr;
+    static pq::DeviceMemo sm_count;
+    const int n_sm = pq::sm_count_of_device(sm_count);
     if (n_sm == 0) return PQ_ERR_CUDA;
-    if (pq::configure_for_device(pq::prefill_tc_kernel<true>, pq::kPtSmTotal, configured_pt2) == 0) return PQ_ERR_CUDA;
-    const int qb_rows = pq::kPtRows / g;
-    q_blocks = (n_q + qb_rows - 1) / qb_rows;
-    // Two query blocks of one (kv head, sequence) per cluster: one 256-row MMA per step, each CTA decodes half of
-    // every block.  An odd count is completed by a CTA without rows -- also a single block when the pairs still fit
-    // on the device at once: the second CTA then only shares the decoding (the kernel is bound by it).
-    pair = q_blocks >= 2 || 2 * (int64_t)n_kv_heads * batch <= n_sm;
-    if (rows >= pq::kPfRows && pq::take_debug_wait_failure(3)) {
-      use_fragment_kernel = true;
-    } else if (rows >= pq::kPtRows) {
-      use_tc = true;
-    } else {
-      // measured on B200: 1.25 us (pair) or 2.4 us per 64-token block and CTA; decode attention at 1.7 TB/s of packed bytes
-      const double ctas = (double)n_kv_heads * batch * (pair ? 2.0 : 1.0);
-      const double waves = std::ceil(ctas / n_sm);
-      const double t_tc = waves * std::ceil(max_len / 64.0) * (pair ? 1.25 : 2.4) + 10.0;
-      const double t_decode = (double)pairs * n_kv_heads * max_len * 124.0 / 1.7e6 + 10.0;
-      use_tc = t_tc < t_decode || pairs * n_kv_heads > pq::kFastMaxUnits;
-    }
-  }
-  if (use_tc) {
-    a.epoch = 0u;
-    a.debug = pq::take_debug_wait_failure(4) ? 2u : 0u;
-    if (pair) {
-      // Two query blocks of one (kv head, sequence) per cluster: one 256-row MMA per step, each CTA decodes half of
-      // every block.  An odd count is completed by a CTA without rows -- also a single block when the pairs still fit
-      // on the device at once: the second CTA then only shares the decoding (the kernel is bound by it).
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((q_blocks + 1) & ~1, n_kv_heads, batch);
-      cfg.blockDim = dim3(pq::kPtThreads);
-      cfg.dynamicSmemBytes = pq::kPtSmTotal;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 2;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      if (cudaLaunchKernelEx(&cfg, pq::prefill_tc_kernel<true>, a, (int)n_q) != cudaSuccess) {
-        cudaGetLastError();
-        return PQ_ERR_CUDA;
-      }
+    if (n_q * g >= pq::kPfRows && pq::take_debug_wait_failure(3)) {
+      // the register-fragment kernel: decode each block of the cache once for 64 (query, head) rows; only reached here (it is
+      // slower than the tcgen05 kernel at every size)
+      static pq::DeviceMemo configured_pf;
+      if (pq::configure_for_device(pq::prefill_attention_kernel, pq::kPfTotal, configured_pf) == 0) return PQ_ERR_CUDA;
+      const int qb_rows = pq::kPfRows / g;
+      dim3 grid((n_q + qb_rows - 1) / qb_rows, n_kv_heads, batch);
+      pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
       return pq::launch_status();
     }
-    dim3 grid(q_blocks, n_kv_heads, batch);
-    pq::prefill_tc_kernel<false><<<grid, pq::kPtThreads, pq::kPtSmTotal, st>>>(a, n_q);
-    return pq::launch_status();
-  }
-  if (use_fragment_kernel) {
-    // decode each block of the cache once for 64 (query, head) rows, mma.sync on register fragments
-    static pq::DeviceMemo configured_pf;
-    if (pq::configure_for_device(pq::prefill_attention_kernel, pq::kPfTotal, configured_pf) == 0) return PQ_ERR_CUDA;
-    const int qb_rows = pq::kPfRows / g;
-    dim3 grid((n_q + qb_rows - 1) / qb_rows, n_kv_heads, batch);
-    pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
-    return pq::launch_status();
-  }
-  static const int force_rows = getenv("PQ_ROWS") ? atoi(getenv("PQ_ROWS")) : -1;
-  const pq::RowCut cut = pq::cut_rows(rows);
-  if (head_dim == 128 && rows > (force_rows == 2 ? 0 : 4) && (int64_t)batch * n_kv_heads * cut.blocks <= pq::kFastMaxUnits && force_rows >= 1)
-    return pq::launch_rows_attention(a, cut, batch, pg.table != nullptr, st);
-  bool persistent = head_dim == 128 && pairs * n_kv_heads <= pq::kFastMaxUnits, fail_wait = false;
-  if (persistent) {
-    // Short contexts at head_dim 128 take the cluster kernel too: the persistent kernel needs 14 to 16 us (27 with more
-    // than four heads per kv head) before length matters -- tables, work split, partial results through global memory --
-    // the cluster kernel 9 (10) us and then 0.013 / 0.017 / 0.044 us per token of its busiest SM with up to 2 / 4 / 8
-    // heads, several times the persistent kernel's rate.
-    if (n_sm == 0) {
-      static pq::DeviceMemo sm_count;
-      n_sm = pq::sm_count_of_device(sm_count);
-      if (n_sm == 0) return PQ_ERR_CUDA;
-    }
-    int64_t tokens = 0;
-    pq::split_cluster_size(128, 16, pairs * n_kv_heads, max_len, n_sm, &tokens);
-    const bool forced = pq::take_debug_wait_failure(5);
-    fail_wait = pq::take_debug_wait_failure(2);
-    persistent = forced || fail_wait || tokens > (g <= 2 ? 640 : g <= 4 ? 400 : 320);
-  }
-  if (persistent) {
-    // One launch: the persistent kernel rotates the queries itself and needs no cleared scratch.
-    a.epoch = pq::next_epoch();
+    const pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm);
+    const bool forced = n_q * g <= 32 && pq::take_debug_wait_failure(5), fail_wait = n_q * g <= 32 && pq::take_debug_wait_failure(2);
+    pq::AttentionKernel kernel = plan.kernel;
+    if ((forced || fail_wait) && kernel == pq::kClusterKernel) kernel = plan.persistent;
+    if (kernel == pq::kTensorKernel) return pq::launch_prefill_tc(a, batch, n_q, plan.pair, plan.n_splits, st);
     a.debug = fail_wait ? 1u : 0u;
-    static pq::DeviceMemo configured[4];
-    const bool paged = pg.table != nullptr;
-    void (*kernel)(pq::DecodeArgs) =
-        g <= 4 ? (paged ? pq::decode_attention_fast_kernel<1, true> : pq::decode_attention_fast_kernel<1, false>)
-               : (paged ? pq::decode_attention_fast_kernel<2, true> : pq::decode_attention_fast_kernel<2, false>);
-    const int n_sm = pq::configure_for_device(kernel, pq::kSmTotal, configured[(g <= 4 ? 0 : 1) + (paged ? 2 : 0)]);
-    if (n_sm == 0) return PQ_ERR_CUDA;
-    return pq::launch_persistent(kernel, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
+    if (kernel == pq::kRowsKernel) return pq::launch_rows_attention(a, pq::cut_rows((int64_t)n_q * g), batch, paged, st);
+    if (kernel == pq::kPersistentKernel) {
+      a.epoch = pq::next_epoch();
+      static pq::DeviceMemo configured[2];
+      void (*fast)(pq::DecodeArgs) = paged ? pq::decode_attention_fast_kernel<true> : pq::decode_attention_fast_kernel<false>;
+      if (pq::configure_for_device(fast, pq::kSmTotal, configured[paged]) == 0) return PQ_ERR_CUDA;
+      return pq::launch_persistent(fast, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
+    }
   }
   pq::SplitCommon c;
   c.d = head_dim; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
@@ -833,9 +924,8 @@ int32_t pq_merge_attention(int32_t head_dim, int32_t n_q_heads, int32_t batch, i
     return PQ_ERR_UNSUPPORTED;
   const int64_t n_rows = (int64_t)batch * n_q_heads, n = n_rows * head_dim;
   if (n * n_parts >= (1ll << 40)) return PQ_ERR_UNSUPPORTED;
-  pq::merge_attention_kernel<<<(unsigned)((n + 255) / 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      head_dim, n_rows, n_parts, parts_out_dev, parts_dtype, parts_lse_dev, out_dev, out_dtype, lse_out_dev, status_dev);
-  return pq::launch_status();
+  return pq::launch_merge(head_dim, n_rows, n_parts, parts_out_dev, parts_dtype, parts_lse_dev, out_dev, out_dtype, lse_out_dev, status_dev,
+                          reinterpret_cast<cudaStream_t>(stream));
 }
 
 int32_t pq_tail_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, const void* q_dev, int32_t io_dtype,

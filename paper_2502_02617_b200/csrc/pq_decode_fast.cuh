@@ -529,11 +529,12 @@ __device__ __forceinline__ void elect_combiner(const DecodeArgs& a, int u, int u
   }
 }
 
-// kHG = groups of four query heads per kv head (1: up to 4 heads, 2: up to 8).
+// Up to four query heads per kv head; more are taken by rows_attention_kernel.
 // kPaged: the cache lies behind a block table (the contiguous instantiation carries none of that code: the kernel
 // sits at its register limit).
-template <int kHG, bool kPaged>
+template <bool kPaged>
 __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(DecodeArgs a) {
+  constexpr int kHG = 1;   // groups of four query heads
   extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((kSmAlign - (smem_u32(smem_raw) & (kSmAlign - 1))) & (kSmAlign - 1));
   const int g_heads = a.n_q_heads / a.n_kv_heads;

@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = a.n_q_heads / a.n_kv_heads;
   const int qb_rows = kPtRows / g;                      // queries of a CTA
-  const int q0 = blockIdx.x * qb_rows, hk = blockIdx.y, b = blockIdx.z;
+  const int n_splits = a.n_splits, split = blockIdx.z % n_splits;   // a CTA (pair) takes one of n_splits ranges of the blocks
+  const int q0 = blockIdx.x * qb_rows, hk = blockIdx.y, b = blockIdx.z / n_splits;
   const int n_rows = max(0, min(qb_rows, n_q - q0)) * g;   // rows in use; row r = (query q0 + r / g, head hk * g + r % g);
                                                            // none in the CTA that only completes a pair
   uint32_t crank = 0;
@@ -151,7 +152,6 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   constexpr int kRawBufs = kPair ? 6 : kPtRawBufs;
   constexpr int kSmRaw = kPair ? kPtSmKv + kPtStages * kStage : kPtSmRaw;
   static_assert(!kPair || kSmRaw + kRawBufs * kPfRawBytes <= kPtSmRaw, "a pair's packed buffers fit behind its stages");
-  const int len = a.lens[b];
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPtSmMisc + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPtSmMisc);
   uint2* tab = reinterpret_cast<uint2*>(smem + kPtSmTab);
@@ -185,6 +185,10 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
   }
+  // a programmatic dependent of the kernel before it: its results (lengths, cache, queries) are read only after this wait
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int len = a.lens[b];
   // ---- Q' = (Q S) * scale * log2(e) as fp16 value + residual (threads 0..255: column, half of the rows), staged in shared
   // memory and then written to tensor memory by the row owners (lane = row, two k values per column)
   __half* qhi_s = reinterpret_cast<__half*>(smem + kPtSmKv + 128 * 128 * 4);
@@ -248,18 +252,19 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   // the last query of the CTA (of the pair) sees the most
   const int q_last = min(n_q, ((kPair ? (int)(blockIdx.x | 1u) : (int)blockIdx.x) + 1) * qb_rows) - 1;
   const int vis_cta = max(0, len - (n_q - 1 - q_last));
-  const int n_blocks = (vis_cta + kTokenBlock - 1) / kTokenBlock;
+  const int all_blocks = (vis_cta + kTokenBlock - 1) / kTokenBlock;
+  const int jb0 = (int)((int64_t)all_blocks * split / n_splits);                       // this CTA's blocks are jb0 + jb,
+  const int n_blocks = (int)((int64_t)all_blocks * (split + 1) / n_splits) - jb0;      // 0 <= jb < n_blocks
   // where this CTA's warps announce themselves: the barriers of the even CTA
   const uint32_t to_leader = kPair ? pt_mapa(sb, 0u) - sb : 0u;   // + a local shared address: that place in the even CTA (cluster window)
   const Layout L = make_layout(128, a.pg.page_tokens);
 
-  float l_run = 0.f;   // row owners: denominator of this thread's row
+  float l_run = 0.f, m_run = -CUDART_INF_F;   // row owners: denominator and reference of this thread's row
   if (warp < 4) {
     // ================= row owners: softmax of row `tid` =================
     const int r = tid;
     const int vis = r < n_rows ? max(0, len - (n_q - 1 - (q0 + r / g))) : 0;
     const uint32_t trow = tmem_base + ((uint32_t)(warp * 32) << 16);
-    float m_run = -CUDART_INF_F;
     const int vis_min = __reduce_min_sync(0xffffffffu, vis);
     for (int jb = 0; jb < n_blocks; ++jb) {
       const int t = jb & 1;
@@ -277,9 +282,9 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
         for (int i = 0; i < 32; i += 2) pt_add2(s[32 * c + i], s[32 * c + i + 1], lo[i], lo[i + 1], s[32 * c + i], s[32 * c + i + 1]);
       }
       // the causal mask touches only the last blocks of a row: one uniform test per warp skips it elsewhere
-      if ((jb + 1) * kTokenBlock > vis_min) {
+      if ((jb0 + jb + 1) * kTokenBlock > vis_min) {
 #pragma unroll
-        for (int i = 0; i < 64; ++i) s[i] = jb * kTokenBlock + i < vis ? s[i] : -CUDART_INF_F;
+        for (int i = 0; i < 64; ++i) s[i] = (jb0 + jb) * kTokenBlock + i < vis ? s[i] : -CUDART_INF_F;
       }
       float mx4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};   // four chains: no 64-long dependency
 #pragma unroll
@@ -344,7 +349,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     const int dt = tid - 128;
     auto fetch = [&](int jb) {  // packed K block and V block of token-block jb -> raw buffer jb % kRawBufs (one group per call)
       if (jb < n_blocks) {
-        const uint8_t* src = a.cache + kv_block_pair_offset(L, a.pg, a.n_kv_heads, b, hk, jb, a.status);
+        const uint8_t* src = a.cache + kv_block_pair_offset(L, a.pg, a.n_kv_heads, b, hk, jb0 + jb, a.status);
         const uint32_t dst = sb + kSmRaw + (jb % kRawBufs) * kPfRawBytes;
         for (int i = dt; i < kPfRawBytes / 16; i += kPtDecoders) pf_cp16(dst + 16 * i, src + 16 * i);
       }
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
           kv = iw >> 5; half = (iw >> 4) & 1; sp = (iw >> 3) & 1; tg = iw & 7;
         }
         const int blk = 4 * half + (lane >> 3), tok = 8 * tg + (lane & 7), bi = blk & 3;
-        const bool live = jb * kTokenBlock + tok < len;   // stale bytes past the sequence end must not reach the MMAs
+        const bool live = (jb0 + jb) * kTokenBlock + tok < len;   // stale bytes past the sequence end must not reach the MMAs
         const uint32_t raw = kraw + kv * 62 * kTokenBlock;
         const uint32_t l1 = lds16(raw + tok * 32 + blk * 4 + sp * 2);               // the two level-1 bytes of this half
         const uint32_t c2 = lds8(raw + kO2 + tok * 8 + blk) >> (4 * sp);
@@ -552,7 +557,12 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       for (int i = 0; i < 32; i += 4)
         *reinterpret_cast<float4*>(osm + r * kPtOStride + 32 * c + i) = make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
     }
-    if (r < n_rows && l_run <= 0.f && !aborted) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token: zeros
+    if (r < n_rows && !aborted) {
+      if (n_splits > 1)   // scores are in the log2 domain
+        a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] =
+            l_run > 0.f ? (m_run + log2f(l_run)) * 0.693147180559945309f : -CUDART_INF_F;
+      else if (l_run <= 0.f) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token: zeros
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
@@ -577,7 +587,8 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       const int row = rh * 64 + r;
       if (row < n_rows) {
         const int64_t o = row_index(row) + i;
-        if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[o] = __float2bfloat16(acc[r]);
+        if (n_splits > 1) a.part_out[(int64_t)split * a.batch * a.n_q_heads * 128 + o] = acc[r];
+        else if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[o] = __float2bfloat16(acc[r]);
         else reinterpret_cast<float*>(a.out)[o] = acc[r];
       }
     }

@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   }
   // a programmatic dependent of the kernel before it, like the persistent kernel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __syncthreads();   // the barriers are initialised
+  if (warp == 0) fetch_S(a.S, sm_base + kRowSmRing, sm_base + kRowSmBarS, lane);   // a constant of the caller, like the tables
   build_fast_tables<kRowThreads>(smem, a.tables);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
@@ -184,10 +186,10 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   const uint32_t qf = sm_base + kRowSmQ + lane * 8;
   int gl0 = 0;   // stages streamed so far
 
-  int my_units = list_segments<kRowThreads>(0, n_units, smem + kRowSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
+  int my_units = list_segments<kRowThreads>(0, n_units, smem + kRowSmQ, segs, n_segs, first_rank, stages_of, empty_unit);
   for (int batch_no = 0; batch_no * kFastMaxSegs < my_units; ++batch_no) {
     if (batch_no > 0)
-      my_units = list_segments<kRowThreads>(batch_no, n_units, smem + kRowSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
+      my_units = list_segments<kRowThreads>(batch_no, n_units, smem + kRowSmQ, segs, n_segs, first_rank, stages_of, empty_unit);
     const int my_segs = min(kFastMaxSegs, my_units - batch_no * kFastMaxSegs);
     for (int sg = 0; sg < my_segs; ++sg) {
       const int u = segs[sg].unit, st0 = segs[sg].st0, st1 = segs[sg].st1;
@@ -215,7 +217,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         bulk_load(ring + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
         issued = li + 1;
       };
-      if (warp == 0) fetch_S(a.S, ring, bar_S, lane);
+      if (warp == 0 && batch_no + sg > 0) fetch_S(a.S, ring, bar_S, lane);
       int2* info = reinterpret_cast<int2*>(smem + kRowSmInfo);
       if (warp == 1) {
         const int row = row0 + min(lane, n_rows - 1), j = row / g_heads;
@@ -299,6 +301,10 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         if (tid == 0 && li + kStages - 1 < n_li) issue_copy(li + kStages - 1);
         __syncwarp();
         if (!mbar_wait(sm_base + kSmBar + 8 * s, (gl / kStages) & 1, abort_flag)) break;
+        if ((a.debug & 1u) && unit_slot == 0 && part == 0 && li == 0 && warp == 0) {   // test hook: see the persistent kernel
+          *abort_flag = 1;
+          break;
+        }
         const int tile_tok0 = st * kStageTokens + warp * 16;
         if (tile_tok0 < len) {
           const uint32_t kblk = sm_base + kRowSmRing + s * kStageBytes + (warp >> 2) * 2 * kBlockBytes128;
