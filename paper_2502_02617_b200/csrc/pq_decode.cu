@@ -119,9 +119,10 @@ struct DecodeArgs {
   int d, n_q_heads, n_kv_heads, batch, capacity, io_dtype;
   int n_q;  // queries per sequence (1: decode).  `batch` counts (sequence, query) pairs: q and out are
             // [batch][n_q_heads][d] with pair p = sequence * n_q + query; `lens` and the cache are per sequence.
-  int n_splits;        // of prefill_tc_kernel: ranges of a sequence's blocks, each with a part of its own in
-  float* part_out;     // [split][batch][n_q_heads][128] and
-  float* part_lse;     // [split][batch][n_q_heads] (natural log), for n_splits > 1
+  const __half* qrot;  // of prefill_tc_kernel: the rotated queries [batch][n_q_heads][value | residual][128],
+  int n_splits;        // ranges of a sequence's blocks, each with a part of its own in
+  float* part_out;     // [split][batch][n_q_heads][128] (rotated basis) and
+  float* part_lse;     // [split][batch][n_q_heads] (natural log)
   int rows_per_block, n_row_blocks;   // of rows_attention_kernel: its cut of a kv head's n_q * group rows
   float scale;
   uint32_t epoch;  // differs from call to call (top bit set): tags the parts' flags of the persistent kernel
@@ -152,6 +153,7 @@ struct DecodeArgs {
 }  // namespace pq
 #include "pq_decode_fast.cuh"
 #include "pq_rows.cuh"
+#include "pq_rotate.cuh"
 #include "pq_prefill.cuh"
 #include "pq_prefill_tc.cuh"
 #include "pq_split_attention.cuh"
@@ -334,26 +336,9 @@ __global__ void __launch_bounds__(256) merge_attention_kernel(int d, int64_t n_r
 static int32_t launch_merge(int d, int64_t n_rows, int n_parts, const void* parts_out, int parts_dtype, const float* parts_lse, void* out,
                             int out_dtype, float* lse_out, int32_t* status, cudaStream_t stream) {
   const bool wide = d % 4 == 0 && (((uintptr_t)parts_out | (uintptr_t)out) & 15) == 0;
-  const int64_t n = n_rows * d / (wide ? 4 : 1);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = wide ? cudaLaunchKernelEx(&cfg, merge_attention_kernel<4>, d, n_rows, n_parts, parts_out, parts_dtype, parts_lse, out,
-                                                  out_dtype, lse_out, status)
-                             : cudaLaunchKernelEx(&cfg, merge_attention_kernel<1>, d, n_rows, n_parts, parts_out, parts_dtype, parts_lse, out,
-                                                  out_dtype, lse_out, status);
-  if (e != cudaSuccess) {
-    note_cuda_error(e);
-    cudaGetLastError();
-    return PQ_ERR_CUDA;
-  }
-  return launch_status();
+  const dim3 grid((unsigned)((n_rows * d / (wide ? 4 : 1) + 255) / 256));
+  return launch_dependent(wide ? merge_attention_kernel<4> : merge_attention_kernel<1>, grid, 256, 0, stream, d, n_rows, n_parts, parts_out,
+                          parts_dtype, parts_lse, out, out_dtype, lse_out, status);
 }
 
 // Exact softmax attention (Eq. 2) of one query per sequence over an uncompressed window of keys and values (the
@@ -673,7 +658,7 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
 //   * persistent kernel, up to four heads, a unit per (query, kv head, sequence): 15 us, then 280 SM cycles per 16-token tile;
 //   * rows kernel, up to 32 rows decoded together: 24 .. 43 us, then 345 + 61 (groups of four rows - 2) cycles per tile;
 //   * tcgen05 kernel: up to 128 rows (a CTA) or 256 (a pair) per decoded block; 1.25 us (pair) or 2.4 us per 64-token block,
-//     20 us per wave for setting up, rotating and un-rotating, 6 us more where a sequence is split and its parts are merged.
+//     12 us per wave, 12 us for rotating the queries before and merging and rotating back after.
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
@@ -684,7 +669,7 @@ constexpr int kMaxSplits = 16;
 // Room for the parts of split tcgen05 calls in the workspace of pq_workspace_bytes: a call whose parts would not fit is split
 // less.  (148 SMs with 128 rows each, twice over, bound what a useful split can need.)
 __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
-  return std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128);
+  return std::max(pairs * n_q_heads, std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128));
 }
 static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm) {
   AttentionPlan plan = {kClusterKernel, kClusterKernel, false, 1};
@@ -692,7 +677,8 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
   const double tiles = std::ceil(max_len / 16.0), sm_hz = n_sm * 1900.0;   // cycles per us of the device
   int64_t tokens = 0;
   split_cluster_size(128, 16, pairs * n_kv_heads, max_len, n_sm, &tokens);
-  double best = (g <= 2 ? 8.0 : 9.0) + tokens * (g <= 2 ? 0.013 : g <= 4 ? 0.017 : 0.044);
+  // (From 32 rows on only the kernels that decode a block once for many rows are considered.)
+  double best = rows >= 32 ? 1e30 : (g <= 2 ? 8.0 : 9.0) + tokens * (g <= 2 ? 0.013 : g <= 4 ? 0.017 : 0.044);
   double best_persistent = 1e30;
   auto consider = [&](double t, AttentionKernel k) {
     if (k != kTensorKernel && t < best_persistent) {
@@ -704,7 +690,7 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     plan.kernel = k;
     return true;
   };
-  if (g <= 4 && pairs * n_kv_heads <= kFastMaxUnits) consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
+  if (g <= 4 && rows < 32 && pairs * n_kv_heads <= kFastMaxUnits) consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
   const RowCut cut = cut_rows(rows);
   if (rows > 4 && batch * n_kv_heads * cut.blocks <= kFastMaxUnits) {
     const int groups = (cut.rows + 3) / 4;
@@ -720,7 +706,7 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
       for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
         const int64_t ctas = (pair ? (q_blocks + 1) / 2 * 2 : q_blocks) * n_kv_heads * batch * s;
         const double waves = std::ceil((double)ctas / (pair ? n_sm / 2 * 2 : n_sm));
-        const double t = waves * (std::ceil((double)blocks / s) * (pair ? 1.25 : 2.4) + 20.0) + (s > 1 ? 6.0 : 0.0);
+        const double t = waves * (std::ceil((double)blocks / s) * (pair ? 1.25 : 2.4) + 12.0) + 12.0;
         if (consider(t, kTensorKernel)) {
           plan.pair = pair != 0;
           plan.n_splits = s;
@@ -737,9 +723,13 @@ static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, in
   const int qb_rows = kPtRows / (a.n_q_heads / a.n_kv_heads), q_blocks = (n_q + qb_rows - 1) / qb_rows;
   a.debug = take_debug_wait_failure(4) ? 2u : 0u;
   a.n_splits = n_splits;
-  a.part_lse = reinterpret_cast<float*>(a.ws.elected);   // the parts take the whole workspace
-  const int64_t part_rows = (int64_t)n_splits * a.batch * a.n_q_heads;
-  a.part_out = a.part_lse + ((part_rows + 63) & ~(int64_t)63);
+  const int64_t all_rows = (int64_t)a.batch * a.n_q_heads;   // the workspace: rotated queries, parts, their log-sum-exps
+  __half* qrot = reinterpret_cast<__half*>(a.ws.elected);
+  a.qrot = qrot;
+  a.part_out = reinterpret_cast<float*>(qrot + all_rows * 256);
+  a.part_lse = a.part_out + n_splits * all_rows * 128;
+  const int32_t st = launch_rotate(a.S, a.q, a.io_dtype, all_rows, a.scale * 1.4426950408889634f, qrot, stream);
+  if (st != PQ_OK) return st;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pair ? (q_blocks + 1) & ~1 : q_blocks, a.n_kv_heads, batch * n_splits);
   cfg.blockDim = dim3(kPtThreads);
@@ -760,10 +750,9 @@ static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, in
     cudaGetLastError();
     return PQ_ERR_CUDA;
   }
-  if (n_splits > 1)
-    return launch_merge(128, (int64_t)a.batch * a.n_q_heads, n_splits, a.part_out, PQ_DTYPE_F32, a.part_lse, a.out, a.io_dtype, nullptr,
-                        a.status, stream);
-  return launch_status();
+  const int32_t main_st = launch_status();
+  if (main_st != PQ_OK) return main_st;
+  return launch_unrotate(a.S, a.part_out, a.part_lse, n_splits, all_rows, a.out, a.io_dtype, a.status, stream);
 }
 
 }  // namespace pq
@@ -780,7 +769,7 @@ int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, i
   if (head_dim != 128) return one;
   const int64_t rows = units * (g + 3) + 32 * pq::kFastMaxGridHost;
   const int64_t cut = 4 * 256 + units * 4 + (units + pq::kFastMaxGridHost) * 4 + rows * (2 + 128) * 4;
-  const int64_t parts = 1024 + pq::part_rows_room(batch, n_q_heads) * (1 + 128) * 4;
+  const int64_t parts = 1024 + (int64_t)batch * n_q_heads * 512 + pq::part_rows_room(batch, n_q_heads) * (1 + 128) * 4;
   return std::max(std::max(cut, one), parts);
 }
 
@@ -811,7 +800,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.lse = lse_dev;
   a.pg = pg;
   a.ws = pq::carve_workspace(workspace_dev, head_dim, pairs * n_kv_heads, n_q_heads / n_kv_heads);
-  a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.epoch = a.debug = 0u;
+  a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.qrot = nullptr; a.epoch = a.debug = 0u;
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
   if (head_dim == 128) {

@@ -57,25 +57,12 @@ constexpr int kPtQStride = 136;                     // halves per row of the Q' 
 constexpr uint32_t kPtTmS = 0, kPtTmO = 256, kPtTmQhi = 384, kPtTmQlo = 448;
 static_assert(kPtSmTotal <= 227 * 1024, "shared memory of one CTA");
 static_assert(128 * kPtOStride * 4 <= kPtStages * kPtStageBytes, "float32 output staging fits in the stages");
-static_assert(128 * 128 * 4 + 2 * 128 * kPtQStride * 2 <= kPtStages * kPtStageBytes, "q and Q' staging fit in the stages");
+static_assert(2 * 128 * kPtQStride * 2 <= kPtStages * kPtStageBytes, "Q' staging fits in the stages");
 static_assert(kPtStageBytes % 1024 == 0, "swizzled tiles start on 1024-byte boundaries");
-
-// acc[r] += sum_k x[r][k0 + k] * w[k] for 64 rows of a float32 tile in shared memory (the same address in every thread)
-__device__ __forceinline__ void pt_rank4(float (&acc)[64], const float* x, int ld, int k0, float4 w) {
-#pragma unroll
-  for (int r = 0; r < 64; ++r) {
-    const float4 v = *reinterpret_cast<const float4*>(x + r * ld + k0);
-    acc[r] = fmaf(v.x, w.x, fmaf(v.y, w.y, fmaf(v.z, w.z, fmaf(v.w, w.w, acc[r]))));
-  }
-}
 
 __device__ __forceinline__ void pt_sts128(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
-__device__ __forceinline__ void pt_sts16(uint32_t addr, __half v) {
-  asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(__half_as_ushort(v)) : "memory");
-}
-
 __device__ __forceinline__ uint32_t pt_mapa(uint32_t addr, uint32_t cta_rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta_rank));
@@ -189,44 +176,16 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int len = a.lens[b];
-  // ---- Q' = (Q S) * scale * log2(e) as fp16 value + residual (threads 0..255: column, half of the rows), staged in shared
-  // memory and then written to tensor memory by the row owners (lane = row, two k values per column)
-  __half* qhi_s = reinterpret_cast<__half*>(smem + kPtSmKv + 128 * 128 * 4);
-  __half* qlo_s = qhi_s + 128 * kPtQStride;
-  {
-    float* qs = reinterpret_cast<float*>(smem + kPtSmKv);
-    for (int i = tid; i < kPtRows * 128; i += kPtThreads) {
-      const int r = i >> 7, k = i & 127;
-      float v = 0.f;
-      if (r < n_rows)
-        v = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[row_index(r) + k])
-                                        : reinterpret_cast<const float*>(a.q)[row_index(r) + k];
-      qs[i] = v;
-    }
-    __syncthreads();
-    if (tid < 256) {
-      const int j = tid & 127, rh = tid >> 7;
-      float acc[64];
-#pragma unroll
-      for (int r = 0; r < 64; ++r) acc[r] = 0.f;
-      for (int k0 = 0; k0 < 128; k0 += 4) {
-        const float4 w = make_float4(__ldg(a.S + (k0 + 0) * 128 + j), __ldg(a.S + (k0 + 1) * 128 + j),
-                                     __ldg(a.S + (k0 + 2) * 128 + j), __ldg(a.S + (k0 + 3) * 128 + j));
-        pt_rank4(acc, qs + rh * 64 * 128, 128, k0, w);
-      }
-      const float f = a.scale * 1.4426950408889634f;
-      // coordinate j sits at position (j & ~3) | (0, 2, 1, 3)[j & 3] of the contraction index: the order the decoders write
-      const int jp = (j & ~3) | ((j & 1) << 1) | ((j >> 1) & 1);
-#pragma unroll
-      for (int r = 0; r < 64; ++r) {
-        const int row = rh * 64 + r;
-        const float v = acc[r] * f;
-        const __half h = __float2half_rn(v);
-        qhi_s[row * kPtQStride + jp] = h;
-        qlo_s[row * kPtQStride + jp] = __float2half_rn(v - __half2float(h));
-      }
-    }
+  // ---- Q' (fp16 value | residual, rotate_rows_kernel) of this CTA's rows: staged in shared memory with coalesced copies, then
+  // written to tensor memory by the row owners (lane = row, two k values per column).  Rows that do not exist repeat the
+  // last one (they are not stored).
+  for (int i = tid; i < kPtRows * 32; i += kPtThreads) {
+    const int r = i >> 5, piece = i & 31;
+    const uint32_t dst = sb + kPtSmKv + r * (2 * kPtQStride * 2) + (piece >> 4) * (kPtQStride * 2) + (piece & 15) * 16;
+    if (n_rows > 0) pf_cp16(dst, a.qrot + row_index(min(r, n_rows - 1)) * 2 + 8 * piece);
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();   // Q' is staged, tensor memory is allocated
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -235,7 +194,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     const uint32_t trow = tmem_base + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {   // hi columns 0..31, 32..63, then lo
-      const uint4* src = reinterpret_cast<const uint4*>((c < 2 ? qhi_s : qlo_s) + tid * kPtQStride + 64 * (c & 1));
+      const uint4* src = reinterpret_cast<const uint4*>(smem + kPtSmKv + tid * (2 * kPtQStride * 2) + (c >> 1) * (kPtQStride * 2) + (c & 1) * 128);
       uint32_t v[32];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -538,7 +497,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   __syncthreads();   // all MMAs have completed (the issuer waited for its last commit), the stages are idle
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool aborted = *abort_flag != 0;
-  // ---- normalise, un-rotate by S^T, store
+  // ---- normalise; merge_unrotate_kernel merges the ranges' parts and rotates back
   float* osm = reinterpret_cast<float*>(smem + kPtSmKv);
   if (warp < 4) {
     const int r = tid;
@@ -557,12 +516,9 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       for (int i = 0; i < 32; i += 4)
         *reinterpret_cast<float4*>(osm + r * kPtOStride + 32 * c + i) = make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
     }
-    if (r < n_rows && !aborted) {
-      if (n_splits > 1)   // scores are in the log2 domain
-        a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] =
-            l_run > 0.f ? (m_run + log2f(l_run)) * 0.693147180559945309f : -CUDART_INF_F;
-      else if (l_run <= 0.f) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token: zeros
-    }
+    if (r < n_rows)   // scores are in the log2 domain
+      a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] =
+          l_run > 0.f ? (m_run + log2f(l_run)) * 0.693147180559945309f : -CUDART_INF_F;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
@@ -575,24 +531,9 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
   }
   if (tid == 0 && aborted) set_status(a.status, PQ_ERR_TIMEOUT);
-  if (tid < 256 && !aborted) {
-    const int i = tid & 127, rh = tid >> 7;   // x_hat_i = sum_j y_hat_j S[i][j]: thread = i, half of the rows
-    float acc[64];
-#pragma unroll
-    for (int r = 0; r < 64; ++r) acc[r] = 0.f;
-    const float4* srow = reinterpret_cast<const float4*>(a.S + i * 128);
-    for (int j0 = 0; j0 < 128; j0 += 4) pt_rank4(acc, osm + rh * 64 * kPtOStride, kPtOStride, j0, __ldg(srow + (j0 >> 2)));
-#pragma unroll
-    for (int r = 0; r < 64; ++r) {
-      const int row = rh * 64 + r;
-      if (row < n_rows) {
-        const int64_t o = row_index(row) + i;
-        if (n_splits > 1) a.part_out[(int64_t)split * a.batch * a.n_q_heads * 128 + o] = acc[r];
-        else if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[o] = __float2bfloat16(acc[r]);
-        else reinterpret_cast<float*>(a.out)[o] = acc[r];
-      }
-    }
-  }
+  for (int i = tid; i < n_rows * 32; i += kPtThreads)
+    *reinterpret_cast<float4*>(a.part_out + (int64_t)split * a.batch * a.n_q_heads * 128 + row_index(i >> 5) + 4 * (i & 31)) =
+        *reinterpret_cast<const float4*>(osm + (i >> 5) * kPtOStride + 4 * (i & 31));
 }
 
 }  // namespace pq
