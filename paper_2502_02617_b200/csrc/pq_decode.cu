@@ -662,7 +662,6 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
-  bool pair;
   int n_splits;
 };
 constexpr int kMaxSplits = 16;
@@ -672,7 +671,7 @@ __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
   return std::max(pairs * n_q_heads, std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128));
 }
 static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm) {
-  AttentionPlan plan = {kClusterKernel, kClusterKernel, false, 1};
+  AttentionPlan plan = {kClusterKernel, kClusterKernel, 1};
   const int64_t pairs = batch * n_q, rows = (int64_t)n_q * g;
   const double tiles = std::ceil(max_len / 16.0), sm_hz = n_sm * 1900.0;   // cycles per us of the device
   int64_t tokens = 0;
@@ -700,26 +699,18 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     const int qb_rows = kPtRows / g;
     const int64_t q_blocks = (n_q + qb_rows - 1) / qb_rows, blocks = (max_len + kTokenBlock - 1) / kTokenBlock;
     const int64_t room = part_rows_room(pairs, (int64_t)n_kv_heads * g) / (pairs * n_kv_heads * g);
-    // Two query blocks of one (kv head, sequence) per cluster: one 256-row MMA per step, each CTA decodes half of every
-    // block.  An odd count is completed by a CTA without rows, which then only shares the decoding.
-    for (int pair = 0; pair < 2; ++pair)
-      for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
-        const int64_t ctas = (pair ? (q_blocks + 1) / 2 * 2 : q_blocks) * n_kv_heads * batch * s;
-        const double waves = std::ceil((double)ctas / (pair ? n_sm / 2 * 2 : n_sm));
-        const double t = waves * (std::ceil((double)blocks / s) * (pair ? 1.25 : 2.4) + 12.0) + 12.0;
-        if (consider(t, kTensorKernel)) {
-          plan.pair = pair != 0;
-          plan.n_splits = s;
-        }
-      }
+    for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
+      const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s;   // two query blocks each
+      const double waves = std::ceil((double)clusters / (n_sm / 2));
+      if (consider(waves * (std::ceil((double)blocks / s) * 1.25 + 12.0) + 12.0, kTensorKernel)) plan.n_splits = s;
+    }
   }
   return plan;
 }
 
-static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, int n_splits, cudaStream_t stream) {
-  static DeviceMemo configured[2];
-  auto kernel = pair ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
-  if (configure_for_device(kernel, kPtSmTotal, configured[pair]) == 0) return PQ_ERR_CUDA;
+static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, int n_splits, cudaStream_t stream) {
+  static DeviceMemo configured;
+  if (configure_for_device(prefill_tc_kernel, kPtSmTotal, configured) == 0) return PQ_ERR_CUDA;
   const int qb_rows = kPtRows / (a.n_q_heads / a.n_kv_heads), q_blocks = (n_q + qb_rows - 1) / qb_rows;
   a.debug = take_debug_wait_failure(4) ? 2u : 0u;
   a.n_splits = n_splits;
@@ -731,7 +722,7 @@ static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, in
   const int32_t st = launch_rotate(a.S, a.q, a.io_dtype, all_rows, a.scale * 1.4426950408889634f, qrot, stream);
   if (st != PQ_OK) return st;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(pair ? (q_blocks + 1) & ~1 : q_blocks, a.n_kv_heads, batch * n_splits);
+  cfg.gridDim = dim3((q_blocks + 1) & ~1, a.n_kv_heads, batch * n_splits);
   cfg.blockDim = dim3(kPtThreads);
   cfg.dynamicSmemBytes = kPtSmTotal;
   cfg.stream = stream;
@@ -743,8 +734,8 @@ static int32_t launch_prefill_tc(DecodeArgs a, int batch, int n_q, bool pair, in
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pair ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a, (int)n_q);
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_tc_kernel, a, (int)n_q);
   if (e != cudaSuccess) {
     note_cuda_error(e);
     cudaGetLastError();
@@ -822,7 +813,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     const bool forced = n_q * g <= 32 && pq::take_debug_wait_failure(5), fail_wait = n_q * g <= 32 && pq::take_debug_wait_failure(2);
     pq::AttentionKernel kernel = plan.kernel;
     if ((forced || fail_wait) && kernel == pq::kClusterKernel) kernel = plan.persistent;
-    if (kernel == pq::kTensorKernel) return pq::launch_prefill_tc(a, batch, n_q, plan.pair, plan.n_splits, st);
+    if (kernel == pq::kTensorKernel) return pq::launch_prefill_tc(a, batch, n_q, plan.n_splits, st);
     a.debug = fail_wait ? 1u : 0u;
     if (kernel == pq::kRowsKernel) return pq::launch_rows_attention(a, pq::cut_rows((int64_t)n_q * g), batch, paged, st);
     if (kernel == pq::kPersistentKernel) {

@@ -37,28 +37,38 @@ namespace pq {
 
 
 constexpr int kPtThreads = 512;   // warps 0-3 row owners, 4-14 decoders, 15 the MMA issuer (registers are allocated per four warps)
-constexpr int kPtDecoders = 352;
-constexpr int kPtRawBufs = 3;
+constexpr int kPtDecoderWarps = 11;
 constexpr int kPtRows = 128;
-constexpr int kPtStages = 4;                        // decoded (K_hat hi, K_hat lo, V_hat^T) blocks in flight
-constexpr int kPtKBytes = 64 * 128 * 2;             // K_hat hi or lo of a block: two k-halves of 64 tokens x 128 bytes
-constexpr int kPtVBytes = 64 * 128 * 2;             // V_hat of a block: two coordinate halves of 64 tokens x 128 bytes
-constexpr int kPtStageBytes = 2 * kPtKBytes + kPtVBytes;
-constexpr int kPtSmKv = 0;                          // the stages; also q, Q' at the start and O at the end
-constexpr int kPtSmRaw = kPtSmKv + kPtStages * kPtStageBytes;   // three packed (K block, V block) buffers
-constexpr int kPtSmTab = kPtSmRaw + kPtRawBufs * kPfRawBytes;   // u_tab[4][64], t1p_hi[256], t1p_lo[256] of Tables (8 bytes per entry)
-constexpr int kPtSmBar = kPtSmTab + 6144;           // kv_full[S], pv_done[S], s_full[2], (unused)[2], p_full[2], p_free[2], drain
-constexpr int kPtSmMisc = kPtSmBar + 16 * kPtStages + 80;   // tensor-memory base, abort flag
-constexpr int kPtSmTotal = kPtSmMisc + 32 + 1024;   // + slack for 1024-byte alignment
+// Decoded blocks in flight.  Per CTA: the keys of 32 tokens -- for each of the two halves of the coordinates the fp16 values of
+// the tokens (128-byte rows) followed by their residuals, one B operand of 64 rows -- and 64 coordinates of the values of 64 tokens.
+constexpr int kPtStages = 4;
+constexpr int kPtKLo = 32 * 128, kPtKHalf = 2 * kPtKLo, kPtKTile = 2 * kPtKHalf, kPtStage = kPtKTile + 64 * 128;
+constexpr int kPtRawBytes = 2 * kBlockBytes128;     // a packed K block and V block
+constexpr int kPtRawBufs = 4;                       // of them in flight
+constexpr int kPtGroups = 16;                       // warp-sized pieces of a block's decoding
+// Shared memory, as offsets in the CTA's shared window (whose addresses carry the CTA's rank in the cluster above): dynamic shared memory starts behind the 1 KB that the system keeps, the
+// decode tables (those of the decode kernel: 96 KB, replicated for conflict-free lookups) on a 32 KB boundary, so that a
+// table address is the OR of disjoint bit fields.
+constexpr uint32_t kPtBase = 1024;
+constexpr uint32_t kPtRaw = kPtBase;
+constexpr uint32_t kPtTab = 32768, kPtT1 = kPtTab + kSmT1p, kPtU = kPtTab + kSmU;
+constexpr uint32_t kPtKv = kPtTab + kSmBar;         // the stages; also Q' at the start and O at the end
+constexpr uint32_t kPtBar = kPtKv + kPtStages * kPtStage;
+constexpr uint32_t kPtBarKv = kPtBar, kPtBarPv = kPtBarKv + 8 * kPtStages, kPtBarRawFull = kPtBarPv + 8 * kPtStages,
+                   kPtBarRawEmpty = kPtBarRawFull + 8 * kPtRawBufs, kPtBarS = kPtBarRawEmpty + 8 * kPtRawBufs, kPtBarP = kPtBarS + 16,
+                   kPtBarO = kPtBarP + 16, kPtBarDrain = kPtBarO + 16;
+constexpr uint32_t kPtMisc = kPtBarDrain + 16;      // tensor-memory base, abort flag
+constexpr int kPtSmTotal = (int)(kPtMisc + 16 - kPtBase);
 constexpr int kPtOStride = 132;                     // floats per row of the output staging
 constexpr int kPtQStride = 136;                     // halves per row of the Q' staging (rows 16 bytes apart mod 128)
 // tensor-memory columns: two score accumulators of 128 (64 tokens x key value and residual; P_j, two fp16 per column,
 // later takes the first 32 columns of the accumulator it came from), the output accumulator, Q' hi and lo
 constexpr uint32_t kPtTmS = 0, kPtTmO = 256, kPtTmQhi = 384, kPtTmQlo = 448;
 static_assert(kPtSmTotal <= 227 * 1024, "shared memory of one CTA");
-static_assert(128 * kPtOStride * 4 <= kPtStages * kPtStageBytes, "float32 output staging fits in the stages");
-static_assert(2 * 128 * kPtQStride * 2 <= kPtStages * kPtStageBytes, "Q' staging fits in the stages");
-static_assert(kPtStageBytes % 1024 == 0, "swizzled tiles start on 1024-byte boundaries");
+static_assert(kPtRaw + kPtRawBufs * kPtRawBytes <= kPtTab, "the packed blocks fit below the tables");
+static_assert(128 * kPtOStride * 4 <= kPtStages * kPtStage, "float32 output staging fits in the stages");
+static_assert(2 * 128 * kPtQStride * 2 <= kPtStages * kPtStage, "Q' staging fits in the stages");
+static_assert(kPtKv % 1024 == 0 && kPtStage % 1024 == 0, "swizzled tiles start on 1024-byte boundaries");
 
 __device__ __forceinline__ void pt_sts128(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
@@ -90,87 +100,61 @@ __device__ __forceinline__ void pt_add2(float a0, float a1, float b0, float b1, 
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
 
-// Named-barrier OR over `n_threads` threads (also a barrier).
-__device__ __forceinline__ bool pt_bar_or(int bar_id, int n_threads, bool v) {
-  uint32_t out;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, %2, %3, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(out)
-      : "r"((uint32_t)v), "r"(bar_id), "r"(n_threads)
-      : "memory");
-  return out != 0;
-}
-
-// kPair: the CTAs of two consecutive query blocks of one (kv head, sequence) form a cluster and run ONE 256-row MMA per
+// The CTAs of two consecutive query blocks of one (kv head, sequence) form a cluster and run ONE 256-row MMA per
 // step (cta_group::2, issued by a thread of the even CTA): every CTA keeps its own 128 rows of Q', S, P and O in its own
 // tensor memory and supplies half of each B operand from its own shared memory -- the keys of 32 of the block's 64
 // tokens, the values of 64 of the 128 coordinates -- so a CTA decodes half a block per block and no decoded data
 // crosses between the CTAs.  The even CTA's barriers collect the arrivals of both CTAs' decoder and row-owner warps;
-// its commits are multicast to both CTAs' barriers.
-template <bool kPair>
+// its commits are multicast to both CTAs' barriers.  An odd count of query blocks is completed by a CTA without rows.
 __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a, int n_q) {
-  extern __shared__ uint8_t pt_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pt_smem_raw) + 1023) & ~(uintptr_t)1023);
-  const uint32_t sb = tc_smem_u32(smem);
+  extern __shared__ __align__(1024) uint8_t pt_smem_raw[];
+  uint8_t* smem = pt_smem_raw - kPtBase;
+  const uint32_t sb = tc_smem_u32(pt_smem_raw) - kPtBase;   // the window: rank << 24
+  if (sb & 0xFFFFFFu) {   // not on this architecture: the table addresses count on the place (both CTAs leave alike)
+    set_status(a.status, PQ_ERR_CUDA);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = a.n_q_heads / a.n_kv_heads;
   const int qb_rows = kPtRows / g;                      // queries of a CTA
-  const int n_splits = a.n_splits, split = blockIdx.z % n_splits;   // a CTA (pair) takes one of n_splits ranges of the blocks
+  const int n_splits = a.n_splits, split = blockIdx.z % n_splits;   // a pair takes one of n_splits ranges of the blocks
   const int q0 = blockIdx.x * qb_rows, hk = blockIdx.y, b = blockIdx.z / n_splits;
   const int n_rows = max(0, min(qb_rows, n_q - q0)) * g;   // rows in use; row r = (query q0 + r / g, head hk * g + r % g);
                                                            // none in the CTA that only completes a pair
-  uint32_t crank = 0;
-  if (kPair) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+  uint32_t crank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
   const bool leader = crank == 0;   // the CTA whose thread issues the MMAs and whose barriers collect the arrivals
-  // Per-CTA shapes of the B operands: keys of kKTok tokens (two coordinate halves), values of 64 tokens x kVHalves x 64
-  // coordinates.  A key tile holds, for each half of the coordinates, the fp16 values of the kKTok tokens followed by their residuals:
-  // one B operand of 2 kKTok rows, so one MMA gives the products with both.
-  constexpr int kKTok = kPair ? 32 : 64, kKLo = kKTok * 128, kKHalf = 2 * kKLo, kKTile = 2 * kKHalf, kVHalves = kPair ? 1 : 2;
-  constexpr int kStage = kKTile + kVHalves * 8192;
-  // columns of a score accumulator: tokens [32 c, 32 c + 32) times the values at kColHi(c), times the residuals at kColLo(c)
-  // (a pair's accumulator columns follow the two CTAs' operand rows)
-  auto col_hi = [](int c) -> uint32_t { return kPair ? 64u * c : 32u * c; };
-  auto col_lo = [](int c) -> uint32_t { return kPair ? 64u * c + 32u : 64u + 32u * c; };
-  // packed blocks in flight: the copy of block jb + kRawBufs - 1 starts when block jb is decoded.  A pair's stages are
-  // half as large: its packed buffers follow them inside the stage area.
-  constexpr int kRawBufs = kPair ? 6 : kPtRawBufs;
-  constexpr int kSmRaw = kPair ? kPtSmKv + kPtStages * kStage : kPtSmRaw;
-  static_assert(!kPair || kSmRaw + kRawBufs * kPfRawBytes <= kPtSmRaw, "a pair's packed buffers fit behind its stages");
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPtSmMisc + 4);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPtSmMisc);
-  uint2* tab = reinterpret_cast<uint2*>(smem + kPtSmTab);
-  const uint32_t bar_kv = sb + kPtSmBar, bar_pv = bar_kv + 8 * kPtStages, bar_sfull = bar_pv + 8 * kPtStages,
-                 bar_pfull = bar_sfull + 32, bar_pfree = bar_pfull + 16, bar_drain = bar_pfree + 16;
+  // columns of a score accumulator: tokens [32 c, 32 c + 32) times the values at col_hi(c), times the residuals at col_lo(c)
+  // (they follow the two CTAs' operand rows)
+  auto col_hi = [](int c) -> uint32_t { return 64u * c; };
+  auto col_lo = [](int c) -> uint32_t { return 64u * c + 32u; };
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPtMisc + 4);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPtMisc);
   auto row_index = [&](int r) -> int64_t {               // offset of row r in q / out ([batch][n_q][n_q_heads][128])
     return (((int64_t)b * n_q + q0 + r / g) * a.n_q_heads + hk * g + r % g) * 128;
   };
   if (tid == 0) {
     for (int i = 0; i < kPtStages; ++i) {
-      tc_mbar_init(bar_kv + 8 * i, (kPair ? 2 : 1) * kPtDecoders / 32);   // one arrival per decoder warp (of both CTAs)
-      tc_mbar_init(bar_pv + 8 * i, 1);                  // tcgen05.commit after the value MMA that read the stage
+      tc_mbar_init(sb + kPtBarKv + 8 * i, 2 * kPtGroups);    // one arrival per decoded piece (of both CTAs)
+      tc_mbar_init(sb + kPtBarPv + 8 * i, 1);                // tcgen05.commit after the value MMA that read the stage
+    }
+    for (int i = 0; i < kPtRawBufs; ++i) {
+      tc_mbar_init(sb + kPtBarRawFull + 8 * i, 1);           // the bytes of a bulk copy
+      tc_mbar_init(sb + kPtBarRawEmpty + 8 * i, kPtGroups);  // one arrival per decoded piece
     }
     for (int i = 0; i < 2; ++i) {
-      tc_mbar_init(bar_sfull + 8 * i, 1);   // tcgen05.commit
-      tc_mbar_init(bar_pfull + 8 * i, kPair ? 8 : 4);
-      tc_mbar_init(bar_pfree + 8 * i, 1);   // tcgen05.commit after the value MMA: the output accumulator holds the block
+      tc_mbar_init(sb + kPtBarS + 8 * i, 1);   // tcgen05.commit
+      tc_mbar_init(sb + kPtBarP + 8 * i, 8);   // one arrival per row-owner warp (of both CTAs)
+      tc_mbar_init(sb + kPtBarO + 8 * i, 1);   // tcgen05.commit after the value MMA: the output accumulator holds the block
     }
-    tc_mbar_init(bar_drain, 1);
+    tc_mbar_init(sb + kPtBarDrain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int i = tid; i < 768; i += kPtThreads)
-    tab[i] = i < 256 ? a.tables->u_tab[i >> 6][i & 63] : (i < 512 ? a.tables->t1p_hi[i - 256] : a.tables->t1p_lo[i - 512]);
-  if (warp == 15) {   // in a pair: the same warp of both CTAs, the same destination offset
-    if (kPair) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sb + kPtSmMisc) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sb + kPtSmMisc) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+  build_fast_tables<kPtThreads>(smem + kPtTab, a.tables);   // from the caller's tables, which no kernel writes
+  if (warp == 15) {   // the same warp of both CTAs, the same destination offset
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sb + kPtMisc) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   // a programmatic dependent of the kernel before it: its results (lengths, cache, queries) are read only after this wait
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -181,7 +165,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   // last one (they are not stored).
   for (int i = tid; i < kPtRows * 32; i += kPtThreads) {
     const int r = i >> 5, piece = i & 31;
-    const uint32_t dst = sb + kPtSmKv + r * (2 * kPtQStride * 2) + (piece >> 4) * (kPtQStride * 2) + (piece & 15) * 16;
+    const uint32_t dst = sb + kPtKv + r * (2 * kPtQStride * 2) + (piece >> 4) * (kPtQStride * 2) + (piece & 15) * 16;
     if (n_rows > 0) pf_cp16(dst, a.qrot + row_index(min(r, n_rows - 1)) * 2 + 8 * piece);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
@@ -194,7 +178,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     const uint32_t trow = tmem_base + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {   // hi columns 0..31, 32..63, then lo
-      const uint4* src = reinterpret_cast<const uint4*>(smem + kPtSmKv + tid * (2 * kPtQStride * 2) + (c >> 1) * (kPtQStride * 2) + (c & 1) * 128);
+      const uint4* src = reinterpret_cast<const uint4*>(smem + kPtKv + tid * (2 * kPtQStride * 2) + (c >> 1) * (kPtQStride * 2) + (c & 1) * 128);
       uint32_t v[32];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -206,16 +190,16 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();   // Q' is in tensor memory; the staging is dead: the stages may be written
-  if (kPair) pt_cluster_sync();   // both CTAs' barriers are initialised and both halves of Q' are in place
+  pt_cluster_sync();   // both CTAs' barriers are initialised and both halves of Q' are in place
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // the last query of the CTA (of the pair) sees the most
-  const int q_last = min(n_q, ((kPair ? (int)(blockIdx.x | 1u) : (int)blockIdx.x) + 1) * qb_rows) - 1;
+  // the last query of the pair sees the most
+  const int q_last = min(n_q, ((int)(blockIdx.x | 1u) + 1) * qb_rows) - 1;
   const int vis_cta = max(0, len - (n_q - 1 - q_last));
   const int all_blocks = (vis_cta + kTokenBlock - 1) / kTokenBlock;
-  const int jb0 = (int)((int64_t)all_blocks * split / n_splits);                       // this CTA's blocks are jb0 + jb,
+  const int jb0 = (int)((int64_t)all_blocks * split / n_splits);                       // this pair's blocks are jb0 + jb,
   const int n_blocks = (int)((int64_t)all_blocks * (split + 1) / n_splits) - jb0;      // 0 <= jb < n_blocks
   // where this CTA's warps announce themselves: the barriers of the even CTA
-  const uint32_t to_leader = kPair ? pt_mapa(sb, 0u) - sb : 0u;   // + a local shared address: that place in the even CTA (cluster window)
+  const uint32_t to_leader = pt_mapa(sb + kPtBase, 0u) - (sb + kPtBase);   // + a local shared address: that place in the even CTA (cluster window)
   const Layout L = make_layout(128, a.pg.page_tokens);
 
   float l_run = 0.f, m_run = -CUDART_INF_F;   // row owners: denominator and reference of this thread's row
@@ -228,7 +212,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     for (int jb = 0; jb < n_blocks; ++jb) {
       const int t = jb & 1;
       const uint32_t ph = (uint32_t)(jb >> 1) & 1u;
-      bool ok = __all_sync(0xffffffffu, tc_mbar_wait(bar_sfull + 8 * t, ph, abort_flag));
+      bool ok = __all_sync(0xffffffffu, tc_mbar_wait(sb + kPtBarS + 8 * t, ph, abort_flag));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float s[64];
@@ -259,7 +243,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
         const float corr = m_run == -CUDART_INF_F ? 1.f : fast_exp2(m_run - m_new);   // nothing accumulated yet: nothing to scale
         if (jb > 0) {
           // the value MMAs up to block jb - 1 must have completed before the accumulator is touched
-          ok = __all_sync(0xffffffffu, tc_mbar_wait(bar_pfree + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u, abort_flag));
+          ok = __all_sync(0xffffffffu, tc_mbar_wait(sb + kPtBarO + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u, abort_flag));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
@@ -299,122 +283,104 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
-        if (kPair) pt_arrive_cluster(bar_pfull + 8 * t + to_leader);
-        else tc_mbar_arrive(bar_pfull + 8 * t);
+        pt_arrive_cluster(sb + kPtBarP + 8 * t + to_leader);
       }
     }
   } else if (warp < 15) {
     // ================= decoders: packed block -> K_hat hi / lo, V_hat^T =================
-    const int dt = tid - 128;
-    auto fetch = [&](int jb) {  // packed K block and V block of token-block jb -> raw buffer jb % kRawBufs (one group per call)
-      if (jb < n_blocks) {
-        const uint8_t* src = a.cache + kv_block_pair_offset(L, a.pg, a.n_kv_heads, b, hk, jb0 + jb, a.status);
-        const uint32_t dst = sb + kSmRaw + (jb % kRawBufs) * kPfRawBytes;
-        for (int i = dt; i < kPfRawBytes / 16; i += kPtDecoders) pf_cp16(dst + 16 * i, src + 16 * i);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    for (int i = 0; i < kRawBufs - 1; ++i) fetch(i);
-    for (int jb = 0; jb < n_blocks; ++jb) {
-      const int st = jb % kPtStages;
-      asm volatile("cp.async.wait_group %0;" ::"n"(kRawBufs - 2) : "memory");   // this thread's part of block jb has landed
-      // stage st is free once the value MMA of block jb - kPtStages has completed (it also covers that block's score MMAs)
+    // Pieces of 1 / kPtGroups of this CTA's half of a block, counted through all blocks, go to the decoder warps in turn (eleven
+    // warps share sixteen pieces evenly only across blocks).  A piece is 16 coordinates of 32 lanes: 8 tokens x the 4
+    // 16-blocks of one coordinate half (the code words of a warp then sit in few shared-memory rows, and the 8 lanes with one
+    // 16-block store to 8 distinct swizzled positions).  Pieces 0-7: the keys of tokens 32 rank .. + 31; pieces 8-15: the
+    // values of coordinates 64 rank .. + 63 of all 64 tokens.
+    const int dw = warp - 4, bi = lane >> 3, t8 = lane & 7;
+    const uint32_t rep = (uint32_t)(lane & 15) * 8u, t1 = (sb + kPtT1) | rep, ub = (sb + kPtU) | rep;
+    const uint32_t swz = (uint32_t)(t8 * 128 + (((2 * bi) ^ t8) << 4));   // chunk 2 bi of a row's 64-coordinate half, swizzled by the row
+    int fetched = 0, ready = -1;   // blocks requested (decoder warp 0, lane 0); the last block known to have landed and to have a stage
+    for (int n = dw; n < kPtGroups * n_blocks; n += kPtDecoderWarps) {
+      const int jb = n / kPtGroups, i = n % kPtGroups, st = jb % kPtStages, buf = jb % kPtRawBufs;
       bool ok = true;
-      if (jb >= kPtStages) ok = tc_mbar_wait(bar_pv + 8 * st, (uint32_t)(jb / kPtStages - 1) & 1u, abort_flag);
-      // The raw block has landed for all decoder threads, and all of them have finished the previous block (the copy
-      // that the next iteration starts goes into the buffer that block was read from); the decision to go on is
-      // taken together.
-      if (pt_bar_or(1, kPtDecoders, !ok)) break;
-      fetch(jb + kRawBufs - 1);   // into the buffer of block jb - 1
-      // all accesses below are shared-memory instructions on 32-bit addresses
-      const uint32_t kraw = sb + kSmRaw + (jb % kRawBufs) * kPfRawBytes;
-      const uint32_t stage = sb + kPtSmKv + st * kStage;
-      const uint32_t utab = sb + kPtSmTab, t1hi = utab + 2048, t1lo = utab + 4096;
-      // An item is one 16-byte chunk of an operand row: (K | V, 16-block, half of the block, token).  The 32 items of a
-      // warp are 8 tokens x the 4 blocks of one coordinate half: the code words of a warp then sit in few shared-
-      // memory rows (the level-1 plane is 32 bytes per token: 32 tokens with one block would be an 8-way bank
-      // conflict, this is 2-way), and 8 lanes with one block and 8 tokens still store to 8 distinct swizzled
-      // positions.  A CTA of a pair takes the keys of tokens 32 rank .. 32 rank + 31 and the values of blocks
-      // 4 rank .. 4 rank + 3 (coordinates 64 rank .. 64 rank + 63) of all 64 tokens.
-      constexpr int kItems = kPair ? 1024 : 2048;
-#pragma unroll
-      for (int item = dt; item < kItems; item += kPtDecoders) {
-        const int iw = item >> 5;   // the warp's item group
-        int kv, half, sp, tg;
-        if (kPair) {
-          kv = iw >> 4;
-          if (kv == 0) { half = (iw >> 3) & 1; sp = (iw >> 2) & 1; tg = (iw & 3) + 4 * (int)crank; }
-          else { half = (int)crank; sp = (iw >> 3) & 1; tg = iw & 7; }
-        } else {
-          kv = iw >> 5; half = (iw >> 4) & 1; sp = (iw >> 3) & 1; tg = iw & 7;
-        }
-        const int blk = 4 * half + (lane >> 3), tok = 8 * tg + (lane & 7), bi = blk & 3;
-        const bool live = (jb0 + jb) * kTokenBlock + tok < len;   // stale bytes past the sequence end must not reach the MMAs
-        const uint32_t raw = kraw + kv * 62 * kTokenBlock;
-        const uint32_t l1 = lds16(raw + tok * 32 + blk * 4 + sp * 2);               // the two level-1 bytes of this half
-        const uint32_t c2 = lds8(raw + kO2 + tok * 8 + blk) >> (4 * sp);
-        const uint32_t c3 = lds8(raw + kO3 + tok * 4 + (blk >> 1)) >> (4 * (blk & 1) + 2 * sp);
-        const uint32_t c4 = (lds16(raw + kO4 + tok * 2) >> (2 * blk)) & 3u;
-        const uint32_t rbits = live ? lds16(raw + kORad + tok * 16 + blk * 2) : 0u;
-        const __half2 r2 = as_h2(rbits | (rbits << 16));
-        const uint32_t c34 = ((c3 & 3u) << 2) | (c4 << 4);
-        uint32_t hw[4], lw[4];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {   // sub-block 2 sp + q: coordinates 4 (2 sp + q) .. + 3 of the block
-          const uint32_t iu = ((c2 >> (2 * q)) & 3u) | c34;
-          const uint2 uu = lds64(utab + (uint32_t)(2 * sp + q) * 512u + iu * 8u);
-          const uint32_t e = ((l1 >> (8 * q)) & 0xFFu) * 8u;
-          const uint2 th = lds64(t1hi + e);
-          const __half2 u_hi = __hmul2(r2, as_h2(uu.x));
-          const __half2 xh = __hmul2(u_hi, as_h2(th.x)), yh = __hmul2(u_hi, as_h2(th.y));   // coordinates (4s, 4s+2), (4s+1, 4s+3)
-          if (kv == 0) {
-            // the key as an unevaluated sum hi + lo (fp16 fused multiply-adds return the exact residual of a product)
-            const uint2 tl = lds64(t1lo + e);
-            const __half2 u_lo = __hfma2(r2, as_h2(uu.y), __hfma2(r2, as_h2(uu.x), __hneg2(u_hi)));
-            hw[2 * q] = as_u32(xh);
-            hw[2 * q + 1] = as_u32(yh);
-            lw[2 * q] = as_u32(__hfma2(u_hi, as_h2(tl.x), __hfma2(u_lo, as_h2(th.x), __hfma2(u_hi, as_h2(th.x), __hneg2(xh)))));
-            lw[2 * q + 1] = as_u32(__hfma2(u_hi, as_h2(tl.y), __hfma2(u_lo, as_h2(th.y), __hfma2(u_hi, as_h2(th.y), __hneg2(yh)))));
-          } else {
-            // coordinates in natural order: (4s, 4s+1) = (x.lo, y.lo), (4s+2, 4s+3) = (x.hi, y.hi)
-            hw[2 * q] = __byte_perm(as_u32(xh), as_u32(yh), 0x5410);
-            hw[2 * q + 1] = __byte_perm(as_u32(xh), as_u32(yh), 0x7632);
+      if (dw == 0) {   // keep up to kPtRawBufs packed blocks in flight; wait only for the one needed now
+        if (lane == 0)
+          while (ok && fetched < n_blocks && fetched < jb + kPtRawBufs) {
+            const int f = fetched % kPtRawBufs;
+            if (fetched >= kPtRawBufs) {
+              const uint32_t ph = (uint32_t)(fetched / kPtRawBufs - 1) & 1u;
+              if (fetched <= jb) ok = tc_mbar_wait(sb + kPtBarRawEmpty + 8 * f, ph, abort_flag);
+              else if (!tc_mbar_test(sb + kPtBarRawEmpty + 8 * f, ph)) break;
+            }
+            if (ok) {
+              tc_mbar_expect_tx(sb + kPtBarRawFull + 8 * f, kPtRawBytes);
+              bulk_load(sb + kPtRaw + f * kPtRawBytes, a.cache + kv_block_pair_offset(L, a.pg, a.n_kv_heads, b, hk, jb0 + fetched, a.status),
+                        kPtRawBytes, sb + kPtBarRawFull + 8 * f);
+              ++fetched;
+            }
           }
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      if (jb != ready) {
+        // stage st is free once the value MMA of block jb - kPtStages has completed (it also covers that block's score MMAs)
+        if (ok && jb >= kPtStages) ok = tc_mbar_wait(sb + kPtBarPv + 8 * st, (uint32_t)(jb / kPtStages - 1) & 1u, abort_flag);
+        if (ok) ok = tc_mbar_wait(sb + kPtBarRawFull + 8 * buf, (uint32_t)(jb / kPtRawBufs) & 1u, abort_flag);
+        ready = jb;
+      }
+      if (!__all_sync(0xffffffffu, ok)) break;
+      const bool is_v = i >= 8;
+      const int half = is_v ? (int)crank : (i >> 2) & 1, tok = 8 * (is_v ? i & 7 : (i & 3) + 4 * (int)crank) + t8, blk = 4 * half + bi;
+      const bool live = (jb0 + jb) * kTokenBlock + tok < len;   // stale bytes past the sequence end must not reach the MMAs
+      const uint32_t raw = sb + kPtRaw + buf * kPtRawBytes + (is_v ? kBlockBytes128 : 0);
+      const uint32_t l1 = lds32(raw + tok * 32 + blk * 4);
+      const uint32_t c2 = lds8(raw + kO2 + tok * 8 + blk);
+      const uint32_t c3 = lds8(raw + kO3 + tok * 4 + (blk >> 1)) >> (4 * (blk & 1));
+      const uint32_t c4 = (lds16(raw + kO4 + tok * 2) >> (2 * blk)) & 3u;
+      const uint32_t rbits = lds16(raw + kORad + tok * 16 + blk * 2);
+      const uint32_t rr = live ? rbits | (rbits << 16) : 0u;
+      const BlockRef ref = make_block_ref(l1, c2, c3, c4, as_h2(rr), ub);
+      if (!is_v) {
+        // the key as an unevaluated sum hi + lo, coordinates in the order of the lookups: (4s, 4s+2), (4s+1, 4s+3)
+        __half2 h[8], l[8];
+        sub_block_hilo<0>(ref, t1, h[0], h[1], l[0], l[1]);
+        sub_block_hilo<1>(ref, t1, h[2], h[3], l[2], l[3]);
+        sub_block_hilo<2>(ref, t1, h[4], h[5], l[4], l[5]);
+        sub_block_hilo<3>(ref, t1, h[6], h[7], l[6], l[7]);
+        const uint32_t dst = sb + kPtKv + st * kPtStage + half * kPtKHalf + (i & 3) * 1024 + swz;
+        pt_sts128(dst, as_u32(h[0]), as_u32(h[1]), as_u32(h[2]), as_u32(h[3]));
+        pt_sts128(dst ^ 16u, as_u32(h[4]), as_u32(h[5]), as_u32(h[6]), as_u32(h[7]));
+        pt_sts128(dst + kPtKLo, as_u32(l[0]), as_u32(l[1]), as_u32(l[2]), as_u32(l[3]));
+        pt_sts128((dst + kPtKLo) ^ 16u, as_u32(l[4]), as_u32(l[5]), as_u32(l[6]), as_u32(l[7]));
+      } else {
+        __half2 x[4], y[4];
+        sub_block_h2<0>(ref, t1, x[0], y[0]);
+        sub_block_h2<1>(ref, t1, x[1], y[1]);
+        sub_block_h2<2>(ref, t1, x[2], y[2]);
+        sub_block_h2<3>(ref, t1, x[3], y[3]);
+        // coordinates in natural order: (4s, 4s+1) = (x.lo, y.lo), (4s+2, 4s+3) = (x.hi, y.hi)
+        uint32_t w[8];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          w[2 * s] = __byte_perm(as_u32(x[s]), as_u32(y[s]), 0x5410);
+          w[2 * s + 1] = __byte_perm(as_u32(x[s]), as_u32(y[s]), 0x7632);
         }
-        // chunk 2 bi + sp of the row's 64-coordinate half, swizzled by the row
-        if (kv == 0) {
-          const int row = tok & (kKTok - 1);
-          const uint32_t dst = stage + half * kKHalf + row * 128 + (((2 * bi + sp) ^ (row & 7)) << 4);
-          pt_sts128(dst, hw[0], hw[1], hw[2], hw[3]);
-          pt_sts128(dst + kKLo, lw[0], lw[1], lw[2], lw[3]);
-        } else {
-          const uint32_t dst = stage + kKTile + (kPair ? 0 : half * 8192) + tok * 128 + (((2 * bi + sp) ^ (tok & 7)) << 4);
-          pt_sts128(dst, hw[0], hw[1], hw[2], hw[3]);
-        }
+        const uint32_t dst = sb + kPtKv + st * kPtStage + kPtKTile + (i & 7) * 1024 + swz;
+        pt_sts128(dst, w[0], w[1], w[2], w[3]);
+        pt_sts128(dst ^ 16u, w[4], w[5], w[6], w[7]);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
-        if (kPair) pt_arrive_cluster(bar_kv + 8 * st + to_leader);
-        else tc_mbar_arrive(bar_kv + 8 * st);
+        pt_arrive_cluster(sb + kPtBarKv + 8 * st + to_leader);
+        tc_mbar_arrive(sb + kPtBarRawEmpty + 8 * buf);
       }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (dw == 0 && lane == 0)   // no copy may be in flight when the CTA ends (they are, where a wait gave up)
+      for (int f = max(0, fetched - kPtRawBufs); f < fetched; ++f)
+        for (int i = 0; i < (1 << 20) && !tc_mbar_try(sb + kPtBarRawFull + 8 * (f % kPtRawBufs), (uint32_t)(f / kPtRawBufs) & 1u); ++i)
+          __nanosleep(32);
   } else if (tid == 480 && leader) {
     // ================= MMA issuer =================
-    // the value operand is MN-major: [token][coordinate] rows of 64 coordinates, the two coordinate halves 8192 bytes apart
-    // (in a pair: one half per CTA)
-    constexpr uint32_t kM = kPair ? 256 : 128;
-    constexpr uint32_t idesc_qk = tc_idesc(false, kM, 128);   // 64 tokens x (value, residual)
-    constexpr uint32_t idesc_pv = tc_idesc(false, kM, 128) | (1u << 16);
-    auto mma = [&](uint32_t d, uint32_t a_t, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-      if (kPair) tc_mma_ts_pair(d, a_t, bdesc, idesc, acc);
-      else tc_mma_ts(d, a_t, bdesc, idesc, acc);
-    };
-    auto commit = [&](uint32_t bar) {   // in a pair: arrives on both CTAs' barriers
-      if (kPair) tc_commit_pair(bar);
-      else tc_commit(bar);
-    };
+    // the value operand is MN-major: [token][coordinate] rows of 64 coordinates, one half per CTA
+    constexpr uint32_t idesc_qk = tc_idesc(false, 256, 128);   // 64 tokens x (value, residual)
+    constexpr uint32_t idesc_pv = tc_idesc(false, 256, 128) | (1u << 16);
     uint64_t vdesc_hi = (uint64_t)(1024 >> 4) << 32;   // stride between groups of 8 tokens
     vdesc_hi |= (uint64_t)1 << 46;
     vdesc_hi |= (uint64_t)2 << 61;
@@ -422,14 +388,14 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     const uint64_t desc_hi = tc_smem_desc(0u) & 0xFFFFFFFF00000000ull;
     auto issue_pv = [&](int jb) -> bool {   // O (+)= P_jb V_hat_jb
       const int t = jb & 1, st = jb % kPtStages;
-      if (!tc_mbar_wait(bar_pfull + 8 * t, (uint32_t)(jb >> 1) & 1u, abort_flag)) return false;
+      if (!tc_mbar_wait(sb + kPtBarP + 8 * t, (uint32_t)(jb >> 1) & 1u, abort_flag)) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t v_lo = (((sb + kPtSmKv + st * kStage + kKTile) & 0x3FFFFu) >> 4) | vdesc_lbo;
+      const uint32_t v_lo = ((kPtKv + st * kPtStage + kPtKTile) >> 4) | vdesc_lbo;
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)   // 16 tokens = 8 columns of P = 16 rows of 128 bytes of V_hat per step
-        mma(tmem_base + kPtTmO, tmem_base + kPtTmS + 128 * t + 8 * kk, vdesc_hi | (v_lo + 128 * kk), idesc_pv, (jb > 0 || kk > 0) ? 1u : 0u);
-      commit(bar_pv + 8 * st);     // the stage is free
-      commit(bar_pfree + 8 * t);   // the output accumulator holds block jb
+        tc_mma_ts_pair(tmem_base + kPtTmO, tmem_base + kPtTmS + 128 * t + 8 * kk, vdesc_hi | (v_lo + 128 * kk), idesc_pv, (jb > 0 || kk > 0) ? 1u : 0u);
+      tc_commit_pair(sb + kPtBarPv + 8 * st);     // the stage is free
+      tc_commit_pair(sb + kPtBarO + 8 * t);   // the output accumulator holds block jb
       return true;
     };
     bool ok = true;
@@ -439,13 +405,13 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       // it does not queue behind this block's score MMAs; otherwise the score MMAs go first and keep the tensor
       // core busy while the softmax of the previous block finishes.
       bool pv_issued = jb == 0;
-      if (!pv_issued && tc_mbar_test(bar_pfull + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u)) {
+      if (!pv_issued && tc_mbar_test(sb + kPtBarP + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u)) {
         ok = issue_pv(jb - 1);
         pv_issued = true;
         if (!ok) break;
       }
       const int st = jb % kPtStages;
-      ok = tc_mbar_wait(bar_kv + 8 * st, (uint32_t)(jb / kPtStages) & 1u, abort_flag);
+      ok = tc_mbar_wait(sb + kPtBarKv + 8 * st, (uint32_t)(jb / kPtStages) & 1u, abort_flag);
       // accumulator t is free: its scores were read before P_{jb-2} was announced, and the value MMA that read
       // P_{jb-2} from its columns was issued in the previous iteration (MMAs of one thread execute in order)
       if (ok && (a.debug & 2u) && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && jb == min(2, n_blocks - 1)) {
@@ -454,7 +420,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       }
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t kb = (uint32_t)tc_smem_desc(sb + kPtSmKv + st * kStage);
+      const uint32_t kb = (uint32_t)tc_smem_desc(kPtKv + st * kPtStage);
       // [Q' K_hi^T | Q' K_lo^T] = (Q'lo + Q'hi) [K_hi | K_lo]^T, the small term first (its product with K_lo is
       // below float32 resolution and rides along); k-step ks: half ks >> 2, 32 bytes per step
 #pragma unroll
@@ -462,32 +428,32 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
         const uint32_t qa = tmem_base + (term == 0 ? kPtTmQlo : kPtTmQhi);
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {   // 16 k values = 8 columns of Q' per step
-          const uint32_t koff = (uint32_t)((ks >> 2) * kKHalf + (ks & 3) * 32) >> 4;
-          mma(tmem_base + kPtTmS + t * 128, qa + 8 * ks, desc_hi | (kb + koff), idesc_qk, (term | ks) ? 1u : 0u);
+          const uint32_t koff = (uint32_t)((ks >> 2) * kPtKHalf + (ks & 3) * 32) >> 4;
+          tc_mma_ts_pair(tmem_base + kPtTmS + t * 128, qa + 8 * ks, desc_hi | (kb + koff), idesc_qk, (term | ks) ? 1u : 0u);
         }
       }
-      commit(bar_sfull + 8 * t);
+      tc_commit_pair(sb + kPtBarS + 8 * t);
       if (!pv_issued) ok = issue_pv(jb - 1);
     }
     if (ok && n_blocks > 0) ok = issue_pv(n_blocks - 1);
     if (n_blocks > 0) {
       // every MMA issued above has completed when this commit arrives (nothing was issued without blocks: no commit)
-      commit(bar_drain);
+      tc_commit_pair(sb + kPtBarDrain);
       bool drained = false;
       for (int i = 0; i < (1 << 20) && !drained; ++i) {
-        drained = tc_mbar_try(bar_drain, 0);
+        drained = tc_mbar_try(sb + kPtBarDrain, 0);
         if (!drained) __nanosleep(32);
       }
       if (!drained) *abort_flag = 1;
     }
-    if (kPair && *abort_flag)   // tell the other CTA, whose warps wait for commits that will not come
-      asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(sb + kPtSmMisc + 4 + (pt_mapa(sb, 1u) - sb)), "r"(1u) : "memory");
-  } else if (kPair && tid == 480) {
+    if (*abort_flag)   // tell the other CTA, whose warps wait for commits that will not come
+      asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(kPtMisc + 4 - kPtBase + pt_mapa(sb + kPtBase, 1u)), "r"(1u) : "memory");
+  } else if (tid == 480) {
     // the odd CTA of a pair: its operands are read until the even CTA's last commit arrives here too
     if (n_blocks > 0) {
       bool drained = false;
       for (int i = 0; i < kTcSpin && !drained && !*abort_flag; ++i) {
-        drained = tc_mbar_try(bar_drain, 0);
+        drained = tc_mbar_try(sb + kPtBarDrain, 0);
         if (!drained) __nanosleep(64);
       }
       if (!drained) *abort_flag = 1;
@@ -498,7 +464,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool aborted = *abort_flag != 0;
   // ---- normalise; merge_unrotate_kernel merges the ranges' parts and rotates back
-  float* osm = reinterpret_cast<float*>(smem + kPtSmKv);
+  float* osm = reinterpret_cast<float*>(smem + kPtKv);
   if (warp < 4) {
     const int r = tid;
     const float inv = (!aborted && l_run > 0.f) ? 1.f / l_run : 0.f;
@@ -522,13 +488,12 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
-  // In a pair neither CTA may release tensor memory or leave while the other may still arrive on its barriers or
+  // Neither CTA may release tensor memory or leave while the other may still arrive on its barriers or
   // have its operands read: both have drained here.
-  if (kPair) pt_cluster_sync();
+  pt_cluster_sync();
   if (warp == 15) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
-    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
   }
   if (tid == 0 && aborted) set_status(a.status, PQ_ERR_TIMEOUT);
   for (int i = tid; i < n_rows * 32; i += kPtThreads)
