@@ -45,6 +45,7 @@ constexpr int kPtStages = 4;
 constexpr int kPtKLo = 32 * 128, kPtKHalf = 2 * kPtKLo, kPtKTile = 2 * kPtKHalf, kPtStage = kPtKTile + 64 * 128;
 constexpr int kPtRawBytes = 2 * kBlockBytes128;     // a packed K block and V block
 constexpr int kPtRawBufs = 4;                       // of them in flight
+constexpr int kPtScores = 4;                        // score accumulators: the score MMAs run ahead of the softmax
 constexpr int kPtGroups = 16;                       // warp-sized pieces of a block's decoding
 // Shared memory, as offsets in the CTA's shared window (whose addresses carry the CTA's rank in the cluster above): dynamic shared memory starts behind the 1 KB that the system keeps, the
 // decode tables (those of the decode kernel: 96 KB, replicated for conflict-free lookups) on a 32 KB boundary, so that a
@@ -55,14 +56,14 @@ constexpr uint32_t kPtTab = 32768, kPtT1 = kPtTab + kSmT1p, kPtU = kPtTab + kSmU
 constexpr uint32_t kPtKv = kPtTab + kSmBar;         // the stages; also Q' at the start and O at the end
 constexpr uint32_t kPtBar = kPtKv + kPtStages * kPtStage;
 constexpr uint32_t kPtBarKv = kPtBar, kPtBarPv = kPtBarKv + 8 * kPtStages, kPtBarRawFull = kPtBarPv + 8 * kPtStages,
-                   kPtBarRawEmpty = kPtBarRawFull + 8 * kPtRawBufs, kPtBarS = kPtBarRawEmpty + 8 * kPtRawBufs, kPtBarP = kPtBarS + 16,
-                   kPtBarO = kPtBarP + 16, kPtBarDrain = kPtBarO + 16;
+                   kPtBarRawEmpty = kPtBarRawFull + 8 * kPtRawBufs, kPtBarS = kPtBarRawEmpty + 8 * kPtRawBufs, kPtBarP = kPtBarS + 8 * kPtScores,
+                   kPtBarDrain = kPtBarP + 8 * kPtScores;
 constexpr uint32_t kPtMisc = kPtBarDrain + 16;      // tensor-memory base, abort flag
 constexpr int kPtSmTotal = (int)(kPtMisc + 16 - kPtBase);
 constexpr int kPtOStride = 132;                     // floats per row of the output staging
 constexpr int kPtQStride = 136;                     // halves per row of the Q' staging (rows 16 bytes apart mod 128)
-// tensor-memory columns: two score accumulators of 128 (64 tokens x key value and residual; P_j, two fp16 per column,
-// later takes the first 32 columns of the accumulator it came from), the output accumulator, Q' hi and lo
+// tensor-memory columns: four score accumulators of 64 tokens (P_j, two fp16 per column, later takes the first 32 columns of
+// the accumulator it came from), the output accumulator, Q' hi and lo
 constexpr uint32_t kPtTmS = 0, kPtTmO = 256, kPtTmQhi = 384, kPtTmQlo = 448;
 static_assert(kPtSmTotal <= 227 * 1024, "shared memory of one CTA");
 static_assert(kPtRaw + kPtRawBufs * kPtRawBytes <= kPtTab, "the packed blocks fit below the tables");
@@ -100,6 +101,16 @@ __device__ __forceinline__ void pt_add2(float a0, float a1, float b0, float b1, 
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
 
+// c += both halves of p, in float32
+__device__ __forceinline__ void pt_add_halves(float& c, uint32_t p) {
+  asm("{\n\t.reg .b16 lo, hi;\n\t"
+      "mov.b32 {lo, hi}, %1;\n\t"
+      "add.rn.f32.f16 %0, lo, %0;\n\t"
+      "add.rn.f32.f16 %0, hi, %0;\n\t}"
+      : "+f"(c)
+      : "r"(p));
+}
+
 // The CTAs of two consecutive query blocks of one (kv head, sequence) form a cluster and run ONE 256-row MMA per
 // step (cta_group::2, issued by a thread of the even CTA): every CTA keeps its own 128 rows of Q', S, P and O in its own
 // tensor memory and supplies half of each B operand from its own shared memory -- the keys of 32 of the block's 64
@@ -114,7 +125,8 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     set_status(a.status, PQ_ERR_CUDA);
     return;
   }
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform
   const int g = a.n_q_heads / a.n_kv_heads;
   const int qb_rows = kPtRows / g;                      // queries of a CTA
   const int n_splits = a.n_splits, split = blockIdx.z % n_splits;   // a pair takes one of n_splits ranges of the blocks
@@ -124,10 +136,6 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   uint32_t crank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
   const bool leader = crank == 0;   // the CTA whose thread issues the MMAs and whose barriers collect the arrivals
-  // columns of a score accumulator: tokens [32 c, 32 c + 32) times the values at col_hi(c), times the residuals at col_lo(c)
-  // (they follow the two CTAs' operand rows)
-  auto col_hi = [](int c) -> uint32_t { return 64u * c; };
-  auto col_lo = [](int c) -> uint32_t { return 64u * c + 32u; };
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPtMisc + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPtMisc);
   auto row_index = [&](int r) -> int64_t {               // offset of row r in q / out ([batch][n_q][n_q_heads][128])
@@ -142,10 +150,9 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       tc_mbar_init(sb + kPtBarRawFull + 8 * i, 1);           // the bytes of a bulk copy
       tc_mbar_init(sb + kPtBarRawEmpty + 8 * i, kPtGroups);  // one arrival per decoded piece
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kPtScores; ++i) {
       tc_mbar_init(sb + kPtBarS + 8 * i, 1);   // tcgen05.commit
       tc_mbar_init(sb + kPtBarP + 8 * i, 8);   // one arrival per row-owner warp (of both CTAs)
-      tc_mbar_init(sb + kPtBarO + 8 * i, 1);   // tcgen05.commit after the value MMA: the output accumulator holds the block
     }
     tc_mbar_init(sb + kPtBarDrain, 1);
     *abort_flag = 0;
@@ -210,20 +217,14 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     const uint32_t trow = tmem_base + ((uint32_t)(warp * 32) << 16);
     const int vis_min = __reduce_min_sync(0xffffffffu, vis);
     for (int jb = 0; jb < n_blocks; ++jb) {
-      const int t = jb & 1;
-      const uint32_t ph = (uint32_t)(jb >> 1) & 1u;
+      const int t = jb % kPtScores;
+      const uint32_t ph = (uint32_t)(jb / kPtScores) & 1u;
       bool ok = __all_sync(0xffffffffu, tc_mbar_wait(sb + kPtBarS + 8 * t, ph, abort_flag));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float s[64];
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {   // Q' K_hi^T + Q' K_lo^T
-        float lo[32];
-        tc_ld32(trow + t * 128 + col_hi(c), s + 32 * c);
-        tc_ld32(trow + t * 128 + col_lo(c), lo);
-#pragma unroll
-        for (int i = 0; i < 32; i += 2) pt_add2(s[32 * c + i], s[32 * c + i + 1], lo[i], lo[i + 1], s[32 * c + i], s[32 * c + i + 1]);
-      }
+      for (int c = 0; c < 2; ++c) tc_ld32(trow + kPtTmS + 64 * t + 32 * c, s + 32 * c);
       // the causal mask touches only the last blocks of a row: one uniform test per warp skips it elsewhere
       if ((jb0 + jb + 1) * kTokenBlock > vis_min) {
 #pragma unroll
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
         const float corr = m_run == -CUDART_INF_F ? 1.f : fast_exp2(m_run - m_new);   // nothing accumulated yet: nothing to scale
         if (jb > 0) {
           // the value MMAs up to block jb - 1 must have completed before the accumulator is touched
-          ok = __all_sync(0xffffffffu, tc_mbar_wait(sb + kPtBarO + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u, abort_flag));
+          ok = __all_sync(0xffffffffu, tc_mbar_wait(sb + kPtBarPv + 8 * ((jb - 1) % kPtStages), (uint32_t)((jb - 1) / kPtStages) & 1u, abort_flag));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
@@ -261,8 +262,8 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       }
       const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;   // nothing visible yet: every p is 0
       // P_jb takes the first 32 columns of the accumulator it was computed from (all of it is in registers): the value
-      // MMA of block jb - 2, which read them last, was issued before the score MMAs that s_full reported
-      float sum8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      // MMA of block jb - kPtScores, which read them last, was issued before the score MMAs that were waited for
+      float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {   // the store of the first half runs while the second half is computed
         uint32_t pw[16];
@@ -272,13 +273,12 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
           float x0, x1;
           pt_add2(s[i], s[i + 1], -m_use, -m_use, x0, x1);
           const __half2 p2 = __floats2half2_rn(fast_exp2(x0), fast_exp2(x1));
-          const float2 pf = __half22float2(p2);   // the denominator of what the MMA will see
-          pt_add2(sum8[2 * (e & 3)], sum8[2 * (e & 3) + 1], pf.x, pf.y, sum8[2 * (e & 3)], sum8[2 * (e & 3) + 1]);
           pw[e] = as_u32(p2);
+          pt_add_halves(sum4[e & 3], pw[e]);   // the denominator of what the MMA will see
         }
-        tc_st16u_nowait(trow + kPtTmS + 128 * t + 16 * hf, pw);
+        tc_st16u_nowait(trow + kPtTmS + 64 * t + 16 * hf, pw);
       }
-      l_run += ((sum8[0] + sum8[1]) + (sum8[2] + sum8[3])) + ((sum8[4] + sum8[5]) + (sum8[6] + sum8[7]));
+      l_run += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -376,69 +376,77 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       for (int f = max(0, fetched - kPtRawBufs); f < fetched; ++f)
         for (int i = 0; i < (1 << 20) && !tc_mbar_try(sb + kPtBarRawFull + 8 * (f % kPtRawBufs), (uint32_t)(f / kPtRawBufs) & 1u); ++i)
           __nanosleep(32);
-  } else if (tid == 480 && leader) {
+  } else if (leader) {
     // ================= MMA issuer =================
+    // The whole warp goes through the loop and one elected lane issues: the operands of the MMAs are then warp-uniform values.
+    // From a single thread's registers every MMA took 60 cycles to issue, more than it runs.
     // the value operand is MN-major: [token][coordinate] rows of 64 coordinates, one half per CTA
-    constexpr uint32_t idesc_qk = tc_idesc(false, 256, 128);   // 64 tokens x (value, residual)
+    constexpr uint32_t idesc_qk = tc_idesc(false, 256, 64);   // 64 tokens
     constexpr uint32_t idesc_pv = tc_idesc(false, 256, 128) | (1u << 16);
     uint64_t vdesc_hi = (uint64_t)(1024 >> 4) << 32;   // stride between groups of 8 tokens
     vdesc_hi |= (uint64_t)1 << 46;
     vdesc_hi |= (uint64_t)2 << 61;
     const uint32_t vdesc_lbo = (8192u >> 4) << 16;     // leading-dimension offset: the next 64 coordinates
     const uint64_t desc_hi = tc_smem_desc(0u) & 0xFFFFFFFF00000000ull;
-    auto issue_pv = [&](int jb) -> bool {   // O (+)= P_jb V_hat_jb
-      const int t = jb & 1, st = jb % kPtStages;
-      if (!tc_mbar_wait(sb + kPtBarP + 8 * t, (uint32_t)(jb >> 1) & 1u, abort_flag)) return false;
+    const int blocks = __shfl_sync(0xffffffffu, n_blocks, 0);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    auto issue_pv = [&](int jb) {   // O (+)= P_jb V_hat_jb
+      const int t = jb % kPtScores, st = jb % kPtStages;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t v_lo = ((kPtKv + st * kPtStage + kPtKTile) >> 4) | vdesc_lbo;
+      if (tc_elect()) {
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk)   // 16 tokens = 8 columns of P = 16 rows of 128 bytes of V_hat per step
-        tc_mma_ts_pair(tmem_base + kPtTmO, tmem_base + kPtTmS + 128 * t + 8 * kk, vdesc_hi | (v_lo + 128 * kk), idesc_pv, (jb > 0 || kk > 0) ? 1u : 0u);
-      tc_commit_pair(sb + kPtBarPv + 8 * st);     // the stage is free
-      tc_commit_pair(sb + kPtBarO + 8 * t);   // the output accumulator holds block jb
-      return true;
+        for (int kk = 0; kk < 4; ++kk)   // 16 tokens = 8 columns of P = 16 rows of 128 bytes of V_hat per step
+          tc_mma_ts_pair(tm + kPtTmO, tm + kPtTmS + 64 * t + 8 * kk, vdesc_hi | (v_lo + 128 * kk), idesc_pv, (jb > 0 || kk > 0) ? 1u : 0u);
+        tc_commit_pair(sb + kPtBarPv + 8 * st);   // the stage is free, the output accumulator holds block jb
+      }
     };
-    bool ok = true;
-    for (int jb = 0; jb < n_blocks && ok; ++jb) {
-      const int t = jb & 1;
-      // The value MMA of the previous block frees its stage for the decoders: it goes first if its P is ready, so that
-      // it does not queue behind this block's score MMAs; otherwise the score MMAs go first and keep the tensor
-      // core busy while the softmax of the previous block finishes.
-      bool pv_issued = jb == 0;
-      if (!pv_issued && tc_mbar_test(sb + kPtBarP + 8 * ((jb - 1) & 1), (uint32_t)((jb - 1) >> 1) & 1u)) {
-        ok = issue_pv(jb - 1);
-        pv_issued = true;
-        if (!ok) break;
-      }
-      const int st = jb % kPtStages;
-      ok = tc_mbar_wait(sb + kPtBarKv + 8 * st, (uint32_t)(jb / kPtStages) & 1u, abort_flag);
-      // accumulator t is free: its scores were read before P_{jb-2} was announced, and the value MMA that read
-      // P_{jb-2} from its columns was issued in the previous iteration (MMAs of one thread execute in order)
-      if (ok && (a.debug & 2u) && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && jb == min(2, n_blocks - 1)) {
-        *abort_flag = 1;   // test hook: this wait counts as failed (what it waited for has arrived)
-        ok = false;
-      }
-      if (!ok) break;
+    auto issue_qk = [&](int jb) {   // S_jb = Q'lo K_hi^T + Q'hi K_lo^T + Q'hi K_hi^T, the small terms first
+      const int t = jb % kPtScores, st = jb % kPtStages;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t kb = (uint32_t)tc_smem_desc(kPtKv + st * kPtStage);
-      // [Q' K_hi^T | Q' K_lo^T] = (Q'lo + Q'hi) [K_hi | K_lo]^T, the small term first (its product with K_lo is
-      // below float32 resolution and rides along); k-step ks: half ks >> 2, 32 bytes per step
+      if (tc_elect()) {
 #pragma unroll
-      for (int term = 0; term < 2; ++term) {
-        const uint32_t qa = tmem_base + (term == 0 ? kPtTmQlo : kPtTmQhi);
+        for (int term = 0; term < 3; ++term) {
+          const uint32_t qa = tm + (term == 0 ? kPtTmQlo : kPtTmQhi);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {   // 16 k values = 8 columns of Q' per step
-          const uint32_t koff = (uint32_t)((ks >> 2) * kPtKHalf + (ks & 3) * 32) >> 4;
-          tc_mma_ts_pair(tmem_base + kPtTmS + t * 128, qa + 8 * ks, desc_hi | (kb + koff), idesc_qk, (term | ks) ? 1u : 0u);
+          for (int ks = 0; ks < 8; ++ks) {   // 16 k values = 8 columns of Q' per step; step ks: half ks >> 2, 32 bytes per step
+            const uint32_t koff = (uint32_t)((ks >> 2) * kPtKHalf + (ks & 3) * 32 + (term == 1 ? kPtKLo : 0)) >> 4;
+            tc_mma_ts_pair(tm + kPtTmS + 64 * t, qa + 8 * ks, desc_hi | (kb + koff), idesc_qk, (term | ks) ? 1u : 0u);
+          }
+        }
+        tc_commit_pair(sb + kPtBarS + 8 * t);
+      }
+    };
+    // Value MMAs go first when their P is ready (they free a stage for the decoders); the score MMAs run up to kPtScores - 1
+    // blocks ahead of them and keep the tensor core and the row owners busy.  Accumulator t is free for block jb once the
+    // value MMA of block jb - kPtScores, which reads P from its columns, has been issued (MMAs of one thread execute in order).
+    bool ok = true;
+    int qk = 0, pv = 0, idle = 0;
+    while (pv < blocks && ok) {
+      if (pv < qk && __all_sync(0xffffffffu, tc_mbar_test(sb + kPtBarP + 8 * (pv % kPtScores), (uint32_t)(pv / kPtScores) & 1u))) {
+        issue_pv(pv++);
+        idle = 0;
+      } else if (qk < blocks && qk < pv + kPtScores &&
+                 __all_sync(0xffffffffu, tc_mbar_test(sb + kPtBarKv + 8 * (qk % kPtStages), (uint32_t)(qk / kPtStages) & 1u))) {
+        if ((a.debug & 2u) && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && qk == min(2, blocks - 1)) {
+          *abort_flag = 1;   // test hook: this wait counts as failed (what it waited for has arrived)
+          ok = false;
+        } else {
+          issue_qk(qk++);
+          idle = 0;
+        }
+      } else if (++idle > 32) {   // bounded like every wait
+        __nanosleep(32);
+        if (__any_sync(0xffffffffu, *abort_flag != 0) || idle > kTcSpin) {
+          *abort_flag = 1;
+          ok = false;
         }
       }
-      tc_commit_pair(sb + kPtBarS + 8 * t);
-      if (!pv_issued) ok = issue_pv(jb - 1);
     }
-    if (ok && n_blocks > 0) ok = issue_pv(n_blocks - 1);
-    if (n_blocks > 0) {
+    if (blocks > 0) {
       // every MMA issued above has completed when this commit arrives (nothing was issued without blocks: no commit)
-      tc_commit_pair(sb + kPtBarDrain);
+      if (tc_elect()) tc_commit_pair(sb + kPtBarDrain);
       bool drained = false;
       for (int i = 0; i < (1 << 20) && !drained; ++i) {
         drained = tc_mbar_try(sb + kPtBarDrain, 0);
@@ -446,9 +454,10 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       }
       if (!drained) *abort_flag = 1;
     }
-    if (*abort_flag)   // tell the other CTA, whose warps wait for commits that will not come
+    __syncwarp();
+    if (lane == 0 && *abort_flag)   // tell the other CTA, whose warps wait for commits that will not come
       asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(kPtMisc + 4 - kPtBase + pt_mapa(sb + kPtBase, 1u)), "r"(1u) : "memory");
-  } else if (tid == 480) {
+  } else if (lane == 0) {
     // the odd CTA of a pair: its operands are read until the even CTA's last commit arrives here too
     if (n_blocks > 0) {
       bool drained = false;
@@ -459,6 +468,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
       if (!drained) *abort_flag = 1;
     }
   }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();   // all MMAs have completed (the issuer waited for its last commit), the stages are idle
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

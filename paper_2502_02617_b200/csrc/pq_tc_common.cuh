@@ -90,6 +90,16 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint
       ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
 // The 2-CTA form (issued by one thread of the even CTA of a pair): D and A are 256 rows, 128 in each CTA's tensor
 // memory at the same columns; each CTA supplies half of B (N / 2 rows) from its own shared memory at the same offset.
 __device__ __forceinline__ void tc_mma_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
