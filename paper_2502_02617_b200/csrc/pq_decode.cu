@@ -657,8 +657,8 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
 //     per token of its busiest SM with up to 2 / 4 / 8 heads;
 //   * persistent kernel, up to four heads, a unit per (query, kv head, sequence): 15 us, then 280 SM cycles per 16-token tile;
 //   * rows kernel, up to 32 rows decoded together: 24 .. 43 us, then 345 + 61 (groups of four rows - 2) cycles per tile;
-//   * tcgen05 kernel: up to 128 rows (a CTA) or 256 (a pair) per decoded block; 1.25 us (pair) or 2.4 us per 64-token block,
-//     12 us per wave, 12 us for rotating the queries before and merging and rotating back after.
+//   * tcgen05 kernel, up to 256 rows per decoded block: 1.1 us per 64-token block of a pair of CTAs, 26 us per wave, 12 us for
+//     rotating the queries before and merging and rotating back after.
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
@@ -702,7 +702,7 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
       const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s;   // two query blocks each
       const double waves = std::ceil((double)clusters / (n_sm / 2));
-      if (consider(waves * (std::ceil((double)blocks / s) * 1.25 + 12.0) + 12.0, kTensorKernel)) plan.n_splits = s;
+      if (consider(waves * (std::ceil((double)blocks / s) * 1.1 + 26.0) + 12.0, kTensorKernel)) plan.n_splits = s;
     }
   }
   return plan;
