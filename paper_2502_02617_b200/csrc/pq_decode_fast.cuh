@@ -662,6 +662,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       issued = li + 1;
       return true;
     };
+    const bool hook = (a.debug & 1u) && unit_slot == 0 && cta == c_first;
     const bool producer = (tid & 255) == 0;
     if (producer && n_li > 0) issue_copy(0);
     __syncwarp();
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       if (producer && li + 1 < n_li) issue_copy(li + 1);
       __syncwarp();
       if (!mbar_wait(sm_base + kSmBar + 8 * s, (gl >> 1) & 1, abort_flag)) break;
-      if ((a.debug & 1u) && unit_slot == 0 && cta == c_first && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
+      if (hook && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
         // that starts the first non-empty unit is reported as failed
         *abort_flag = 1;
         break;
@@ -909,7 +910,11 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
           o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
         }
       }
-    const int slot = unit_slot + (cta - c_first);
+    // The segment is read again (and through volatile, so that it really is): the registers that its fields would hold through
+    // the tile loop cost that loop 2 % (8 x 131072 tokens: 516 -> 507 us).
+    const volatile Segment* done = segs + sg;
+    const int d_unit = done->unit, d_part = done->part, d_parts = done->n_parts, d_slot = done->slot0;
+    const int slot = d_slot + d_part;
     if (tid < g_heads * 16) {   // denominators: 16 lanes per head
       const int h = tid >> 4;
       const unsigned half = 0xFFFFu << (lane & 16);
@@ -934,11 +939,11 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       }
     }
     __syncthreads();
-    if (warp == 0) elect_combiner(a, u, unit_slot, cta - c_first, n_parts, lane, is_last);
+    if (warp == 0) elect_combiner(a, d_unit, d_slot, d_part, d_parts, lane, is_last);
     __syncthreads();
     if (*is_last) {
-      combine_and_store<kHG>(a, b, hk, g_heads, unit_slot, n_parts, reinterpret_cast<float*>(smem + kSmRing));
-      if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
+      combine_and_store<kHG>(a, d_unit / a.n_kv_heads, d_unit % a.n_kv_heads, g_heads, d_slot, d_parts, reinterpret_cast<float*>(smem + kSmRing));
+      if (tid == 0 && d_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + d_unit) = 0u;
     }
     __syncthreads();  // the ring is free again for the next unit
   }
