@@ -1,0 +1,125 @@
+"""The kernels that a dispatch chooses among, at the sizes where each can go wrong: edges of tiles and of row groups, remainders,
+the smallest and largest of its range.  Attention in float32 I/O against the float64 oracle (the tolerance of one kernel's
+arithmetic, see parity_utils); encoders against the codes of the same tokens encoded in other pieces, because every decision is
+exact whatever kernel takes it."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2502_02617_b200 as pq
+from paper_2502_02617_b200 import synthetic
+from oracle import polarquant_oracle as orc
+from parity_utils import TOL_ATTENTION_F32_IO, rel_l2, to_f64
+from test_gpu_parity import _encode_and_compare, _oracle_cache
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _filled(lens, Hq, Hkv, d, seed, dtype=torch.bfloat16):
+    cache = pq.PolarQuantCache(len(lens), Hq, Hkv, d, capacity=max(lens), seed=seed, device=DEV)
+    K, V = synthetic.kv_like(seed + 1, sum(lens), Hkv, d, dtype, DEV, n_outliers=4 if d >= 64 else 0)
+    cache.encode(K, V, torch.tensor(np.concatenate(([0], np.cumsum(lens))), dtype=torch.int32, device=DEV))
+    return cache, _oracle_cache(cache, K, V, lens)
+
+
+# Rows of a kv head (queries x heads of the group) on both sides of every group of four that the rows kernel is built for
+# (8, 12, 16, 20, 24, 32), odd groups whose rows do not end with a query; lengths around its 16-token tiles and 128-token stages.
+@pytest.mark.parametrize("g,n_q", [(1, 5), (1, 8), (1, 9), (4, 3), (1, 13), (8, 2), (1, 17), (5, 4), (7, 3), (6, 4), (1, 25), (7, 4), (4, 8),
+                                   (8, 4), (1, 32)])
+def test_rows_kernel(g, n_q):
+    lens, Hkv = [16, 129, 397, 2, 128], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 60 + g)
+    q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
+    pq.pq_debug_fail_next_wait(5)   # a call this small would go to the cluster kernel
+    out = to_f64(cache.attend_multi(q))
+    want = orc.multi_query_attention(to_f64(q), ref.k_codes, ref.k_radii, ref.v_codes, ref.v_radii, ref.lens, ref.cb, ref.S, 128 ** -0.5)
+    for b in range(len(lens)):
+        for j in range(n_q):
+            if lens[b] - (n_q - 1 - j) <= 0:
+                assert np.all(out[b, j] == 0)
+            else:
+                assert rel_l2(out[b, j], want[b, j]) < TOL_ATTENTION_F32_IO, (b, j)
+
+
+# The tcgen05 kernel: an odd count of 64-token blocks (half of a tile pair), fewer blocks than ranges (empty parts), more rows than
+# one pair of CTAs holds, a group size that leaves rows of the 128 unused, and 64-row tiles in the rotation kernels.
+@pytest.mark.parametrize("g,Hkv,n_q,lens", [(8, 1, 16, [1, 64, 65, 700]), (7, 2, 19, [1473, 40]), (4, 1, 70, [1000, 71, 64]),
+                                            (8, 8, 75, [90, 75, 300, 65, 76, 80, 91, 99])])
+def test_tcgen05_multi_query_kernel_parts(g, Hkv, n_q, lens):
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 70 + g)
+    q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
+    out = to_f64(cache.attend_multi(q))
+    want = orc.multi_query_attention(to_f64(q), ref.k_codes, ref.k_radii, ref.v_codes, ref.v_radii, ref.lens, ref.cb, ref.S, 128 ** -0.5)
+    for b in range(len(lens)):
+        for j in range(n_q):
+            if lens[b] - (n_q - 1 - j) <= 0:
+                assert np.all(out[b, j] == 0)
+            else:
+                assert rel_l2(out[b, j], want[b, j]) < TOL_ATTENTION_F32_IO, (b, j)
+
+
+# The cluster kernel: lengths around its 16-token tiles, a warp without tokens, one head and every padding of the heads of a group;
+# the persistent kernel and the rows kernel (hook 5) on the same.
+@pytest.mark.parametrize("d,g", [(128, 1), (128, 3), (128, 5), (128, 8), (64, 2), (64, 7), (32, 4), (16, 1), (16, 8)])
+def test_single_query_kernels(d, g):
+    lens, Hkv = [1, 15, 16, 17, 63, 64, 65, 255, 257, 1025], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, d, 80 + g, torch.float32)
+    q = synthetic.queries(5, len(lens), g * Hkv, d, torch.float32, DEV)
+    want = ref.attend(to_f64(q), d ** -0.5)
+    for hook in (0, 5) if d == 128 else (0,):
+        if hook:
+            pq.pq_debug_fail_next_wait(hook)
+        out = to_f64(cache.attend(q))
+        for b in range(len(lens)):
+            assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (hook, lens[b])
+
+
+# Calls below 32 tokens have a kernel of their own (one block per sequence), larger ones tiles of 64 rows (float32 or d < 128)
+# or of 128 (bf16, d = 128): the same codes whatever pieces the tokens come in, and the first piece against the oracle.  The radii
+# are float32 sums in another order before they are rounded to fp16: neighbours at most, 2^-10 apart.
+@pytest.mark.parametrize("d,dtype", [(128, torch.bfloat16), (128, torch.float32), (64, torch.bfloat16), (32, torch.float32), (16, torch.bfloat16)])
+def test_encoders_give_the_same_codes_in_any_pieces(d, dtype):
+    Hkv, pieces = 3, [31, 1, 32, 2, 17, 63, 65, 16, 15, 129, 3]
+    n = sum(pieces)
+    K, V = synthetic.kv_like(90 + d, n, Hkv, d, dtype, DEV, n_outliers=4 if d >= 64 else 0)
+    V[7] = 0                                                    # a zero vector
+    whole, cut = (pq.PolarQuantCache(1, Hkv, Hkv, d, capacity=n, seed=6, device=DEV) for _ in range(2))
+    whole.encode(K, V, torch.tensor([0, n], dtype=torch.int32, device=DEV))
+    at = 0
+    for m in pieces:
+        cut.encode(K[at:at + m], V[at:at + m], torch.tensor([0, m], dtype=torch.int32, device=DEV))
+        at += m
+    (codes, radii), (codes_cut, radii_cut) = whole.unpack(n), cut.unpack(n)
+    assert torch.equal(codes, codes_cut) and cut.lens.tolist() == [n]
+    assert torch.all((radii.float() - radii_cut.float()).abs() <= 2.0 ** -10 * radii.float())
+    few = pq.PolarQuantCache(2, Hkv, Hkv, d, capacity=32, seed=6, device=DEV)
+    _encode_and_compare(few, K[:31], V[:31], [17, 14])          # one launch, odd counts
+
+
+@pytest.mark.parametrize("d,bits", [(128, (3,) * 7), (64, (4, 2)), (16, (2,) * 4)])
+def test_general_encoder_writes_the_same_bytes_in_any_pieces(d, bits):
+    Hkv, pieces = 3, [1, 20, 21, 22, 43, 64, 2]                 # rows = tokens x heads: around the tiles of 64
+    n = sum(pieces)
+    K, V = synthetic.kv_like(95 + d, n, Hkv, d, torch.float32, DEV, n_outliers=4 if d >= 64 else 0)
+    whole, cut = (pq.GeneralPolarQuantCache(1, Hkv, Hkv, d, bits, n, seed=6, device=DEV) for _ in range(2))
+    whole.encode(K, V, torch.tensor([0, n], dtype=torch.int32, device=DEV))
+    at = 0
+    for m in pieces:
+        cut.encode(K[at:at + m], V[at:at + m], torch.tensor([0, m], dtype=torch.int32, device=DEV))
+        at += m
+    assert torch.equal(whole.cache, cut.cache)
+
+
+# Four coordinates per thread where the pointers allow it, else one.  A weighted mean of three float32 values: 1e-6 is eight
+# roundings of 2^-23.
+@pytest.mark.parametrize("d,shift", [(16, 0), (16, 1), (128, 0), (128, 3)])
+def test_merge_of_parts(d, shift):
+    gen = torch.Generator(device=DEV).manual_seed(d + shift)
+    parts = torch.randn(3 * 5 * 7 * d + shift, generator=gen, device=DEV)[shift:].view(3, 5, 7, d)
+    lse = torch.randn((3, 5, 7), generator=gen, device=DEV)
+    lse[1, 2, 3] = -float("inf")                                # a part without tokens
+    out, status = torch.empty((5, 7, d), device=DEV), torch.zeros(4, dtype=torch.int32, device=DEV)
+    pq.pq_merge_attention(parts, lse, out, status)
+    w = torch.softmax(lse.double(), 0)[..., None]
+    assert rel_l2(to_f64(out), (w * parts.double()).sum(0).cpu().numpy()) < 1e-6
