@@ -9,7 +9,8 @@
 // coordinate is at most (16 + D / 16) 2^-24 sum_k |x_k||S_kj| <= that factor times ||x||_2.  Then a thread per
 // 16-coordinate block runs the certified quantiser; a block with an uncertified decision is rotated again in float64 by
 // the whole thread block (two or fewer terms per thread) and decided by one warp.
-// Measured (16 vectors of 128 coordinates, one sequence): see the table of cases.
+// Measured (append with 8 kv heads, a block per vector and a second launch for the lengths before): one sequence, head_dim 128
+// 11.0 -> 7.0 us, sixteen sequences 11.6 -> 10.1 us; eight sequences at head_dim 64 (float64 throughout before) 20.4 -> 8.7 us.
 #pragma once
 
 namespace pq {

@@ -232,11 +232,6 @@ __device__ __forceinline__ float ld_const_now(const float* p) {
   asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
-__device__ __forceinline__ float4 ld_const_now4(const float* p) {   // 16-byte aligned
-  float4 v;
-  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-  return v;
-}
 // Packed float32 arithmetic: one instruction for two IEEE multiply-adds.
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
   uint64_t r;

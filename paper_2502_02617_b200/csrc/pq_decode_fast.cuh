@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       issued = li + 1;
       return true;
     };
-    const bool hook = (a.debug & 1u) && unit_slot == 0 && cta == c_first;
+    const bool hook = !kPaged && (a.debug & 1u) && unit_slot == 0 && cta == c_first;
     const bool producer = (tid & 255) == 0;
     if (producer && n_li > 0) issue_copy(0);
     __syncwarp();
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       if (producer && li + 1 < n_li) issue_copy(li + 1);
       __syncwarp();
       if (!mbar_wait(sm_base + kSmBar + 8 * s, (gl >> 1) & 1, abort_flag)) break;
-      if (hook && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
+      if ((kPaged ? (a.debug & 1u) && unit_slot == 0 && cta == c_first : hook) && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
         // that starts the first non-empty unit is reported as failed
         *abort_flag = 1;
         break;
@@ -910,11 +910,20 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
           o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
         }
       }
-    // The segment is read again (and through volatile, so that it really is): the registers that its fields would hold through
-    // the tile loop cost that loop 2 % (8 x 131072 tokens: 516 -> 507 us).
-    const volatile Segment* done = segs + sg;
-    const int d_unit = done->unit, d_part = done->part, d_parts = done->n_parts, d_slot = done->slot0;
-    const int slot = d_slot + d_part;
+    // In the contiguous instantiation the segment is read again (and through volatile, so that it really is): the registers that its
+    // fields would hold through the tile loop cost that loop 2 % (8 x 131072 tokens: 516 -> 507 us).  In the paged one it is
+    // the other way round (16 ragged sequences of up to 65536 tokens, four steps: 1313 us, 1365 with the fields read again).
+    struct {
+      int unit, b, hk, part, n_parts, slot0;
+    } done;
+    if constexpr (kPaged) {
+      done = {u, b, hk, cta - c_first, n_parts, unit_slot};
+    } else {
+      const volatile Segment* sv = segs + sg;
+      const int du = sv->unit;
+      done = {du, du / a.n_kv_heads, du % a.n_kv_heads, sv->part, sv->n_parts, sv->slot0};
+    }
+    const int slot = done.slot0 + done.part;
     if (tid < g_heads * 16) {   // denominators: 16 lanes per head
       const int h = tid >> 4;
       const unsigned half = 0xFFFFu << (lane & 16);
@@ -939,11 +948,11 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       }
     }
     __syncthreads();
-    if (warp == 0) elect_combiner(a, d_unit, d_slot, d_part, d_parts, lane, is_last);
+    if (warp == 0) elect_combiner(a, done.unit, done.slot0, done.part, done.n_parts, lane, is_last);
     __syncthreads();
     if (*is_last) {
-      combine_and_store<kHG>(a, d_unit / a.n_kv_heads, d_unit % a.n_kv_heads, g_heads, d_slot, d_parts, reinterpret_cast<float*>(smem + kSmRing));
-      if (tid == 0 && d_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + d_unit) = 0u;
+      combine_and_store<kHG>(a, done.b, done.hk, g_heads, done.slot0, done.n_parts, reinterpret_cast<float*>(smem + kSmRing));
+      if (tid == 0 && done.n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + done.unit) = 0u;
     }
     __syncthreads();  // the ring is free again for the next unit
   }

@@ -17,6 +17,9 @@
 // radii of n-coordinate halves moves by at most sqrt(2 n) dy; 1.1 x that, plus 1e-6 (r_a + r_b) for the float32
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
 // A radius is certified by radius_unsure.
+// Bound by the product on the FMA pipe (18 of a block's 47 us) and by the latency of the float64 re-decisions (13).  Measured (8 heads;
+// a block per vector in float64 before): 512 tokens, seven levels of three bits 89.7 -> 43.4 us; packed cache, 2048 tokens at
+// head_dim 64 67 -> 40 us.
 #pragma once
 #include <math_constants.h>
 

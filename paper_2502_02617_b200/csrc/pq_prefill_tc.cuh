@@ -2,33 +2,34 @@
 // pq_decode.cu).  Same computation as pq_prefill.cuh -- the last n_q positions of a sequence attend causally to the
 // cached tokens (Eq. 2 / Eq. 3) -- for chunks that fill 128 rows = (128 / g) queries x the g query heads of a kv head.
 //
-// A CTA of sixteen warps owns 128 rows of one (kv head, sequence) and loops over the 64-token blocks its queries may
-// see; two CTAs with consecutive query blocks run as a pair on one 256-row MMA (see prefill_tc_kernel):
-//   * warps 4-14 ("decoders") copy the packed K and V block with cp.async, DeQuant it (Algorithm 1 by the table
-//     lookups of the decode kernel: per 4-coordinate sub-block one entry for levels 4-2 and one for the two level-1
-//     pairs, fp16 with error-free residuals) and write the tensor-core operands into shared memory as
-//     128-byte-swizzled tiles of 64-coordinate rows: per coordinate half the fp16 values of the tokens followed by
-//     their fp16 residuals (ONE K-major B operand: the contraction runs over the coordinates, the rows are
-//     (value | residual, token)), and V_hat as fp16 values [token][64 coordinates] x two halves (an MN-major B
-//     operand: the contraction runs over the tokens); four stages, so the decoders run ahead of the MMAs.
-//     The lookups deliver coordinates (4s, 4s+2 | 4s+1, 4s+3); K_hat keeps that order and Q' is stored in the same
-//     one (the contraction does not care), V_hat is put back in natural order by two byte permutes per sub-block;
-//   * one thread of warp 15 issues the MMAs: [Q' K_hi^T | Q' K_lo^T] = (Q'lo + Q'hi) [K_hi | K_lo]^T (N = 128, eight
-//     k-steps per term) into one of two 128-column accumulators in tensor memory, and O += P_j V_hat (N = 128, four
-//     k-steps) into a 128-column accumulator.  The A operands live in tensor memory too (Q' hi and lo, written
-//     once; P_j, written by the row owners), the B operands are read from shared memory by the tensor core itself:
-//     no warp re-reads a tile (the register-fragment kernel spends 70 % of the shared-memory pipe on exactly that);
-//   * warps 0-3 ("row owners": tensor-memory lane = row = thread) read the scores with tcgen05.ld, add the value and
-//     residual halves, apply the causal mask and the online softmax in the log2 domain without any shuffle (a thread
-//     owns its whole row), and write P_j in fp16 over the first columns of the accumulator the scores came from, as
-//     the A operand of the value MMA.  The running maximum is updated lazily: only when a score exceeds it by more
-//     than 8 is the output accumulator rescaled (tcgen05.ld / multiply / tcgen05.st by the row's owner, after the
-//     previous value MMA has completed); otherwise p <= 2^8 stays well inside fp16.
-// Q' = (Q S) * scale * log2(e) is formed once per CTA in float32 and kept as fp16 value + residual; the output is
-// normalised and rotated back by S^T in float32 when the CTA ends.  All hand-offs are mbarriers (decoded stage
-// full, scores full, P full, value MMA done = stage free); every wait is bounded, and a wait that gives up makes
-// every role leave its loop, after which the CTA (the pair) drains its copies and MMAs, releases tensor memory and
-// records PQ_ERR_TIMEOUT.
+// Two CTAs of sixteen warps form a cluster; each owns 128 rows of one (kv head, sequence), and both loop together over a range of
+// the 64-token blocks the queries may see, on one 256-row MMA (see prefill_tc_kernel).  Where rows and sequences leave SMs idle
+// the blocks are cut into several ranges, whose parts merge_unrotate_kernel (pq_rotate.cuh) merges; rotate_rows_kernel rotates the
+// queries before.  In a CTA
+//   * warps 4-14 ("decoders") DeQuant the packed blocks, which bulk copies bring in four ahead (Algorithm 1 by the table lookups of
+//     the decode kernel on its replicated, conflict-free tables: fp16 with error-free residuals) and write the tensor-core
+//     operands into shared memory as 128-byte-swizzled tiles of 64-coordinate rows: per coordinate half the fp16 values of the
+//     tokens followed by their fp16 residuals (K-major: the contraction runs over the coordinates), and V_hat as fp16 values
+//     [token][64 coordinates] (MN-major: the contraction runs over the tokens); four stages, so they run ahead of the MMAs.
+//     The lookups deliver coordinates (4s, 4s+2 | 4s+1, 4s+3); K_hat keeps that order and Q' is stored in the same one (the
+//     contraction does not care), V_hat is put back in natural order by two byte permutes per sub-block;
+//   * warp 15 issues the MMAs: S = Q'lo K_hi^T + Q'hi K_lo^T + Q'hi K_hi^T (N = 64, eight k-steps per term) into one of four
+//     64-column accumulators in tensor memory, up to three blocks ahead of the softmax, and O += P_j V_hat (N = 128, four
+//     k-steps) into a 128-column accumulator.  The A operands live in tensor memory too (Q' hi and lo, written once; P_j,
+//     written by the row owners), the B operands are read from shared memory by the tensor core itself;
+//   * warps 0-3 ("row owners": tensor-memory lane = row = thread) read the scores with tcgen05.ld, apply the causal mask and the
+//     online softmax in the log2 domain without any shuffle (a thread owns its whole row), and write P_j in fp16 over the
+//     first columns of the accumulator the scores came from, as the A operand of the value MMA.  The running maximum is
+//     updated lazily: only when a score exceeds it by more than 8 is the output accumulator rescaled (tcgen05.ld / multiply /
+//     tcgen05.st by the row's owner, after the previous value MMA has completed); otherwise p <= 2^8 stays well inside fp16.
+// All hand-offs are mbarriers (packed block full / free, decoded stage full, scores full, P full, value MMA done = stage free);
+// every wait is bounded, and a wait that gives up makes every role leave its loop, after which the pair drains its copies
+// and MMAs, releases tensor memory and records PQ_ERR_TIMEOUT.
+// Measured (32/8 heads, 64 queries, 8 sequences of 32768 tokens): 757 us with the rotations inside, per-lane tables, the score
+// terms in two accumulators and MMAs issued from one thread's registers (60 cycles each); 710 with the rotations outside; 582 now:
+// 1.1 us per block of a pair.  Decoding and MMAs share the bound: 420 us with the tables left unread and no softmax, 558 without the
+// softmax, 469 without the decoding.  Score MMAs of two blocks with N = 128 (24 per two blocks instead of 48) took 675: such an MMA
+// runs for 110 cycles, one with N = 64 for 40.  Keys and values in one piece of decoding: 599.
 #pragma once
 
 #include "pq_tc_common.cuh"

@@ -9,6 +9,7 @@
 // Eight warps with up to 255 registers (16 accumulators per group of rows, all in registers) instead of sixteen with 128; the
 // query fragments stay in shared memory (one conflict-free 8-byte read per MMA pair).  All four ring slots belong to the one
 // group of eight warps, so copies run three stages ahead.
+// Measured (32/8 heads, 4 sequences of 8192 tokens; one decode per query before): 2 queries 52 -> 44 us, 5 107 -> 66, 8 162 -> 84.
 #pragma once
 
 namespace pq {
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   const float* S_sm = reinterpret_cast<const float*>(smem + kRowSmRing);
   uint32_t n_S = 0;   // copies of S so far
 
-  const int n_units = a.batch / a.n_q * a.n_kv_heads * nrb, cta = blockIdx.x;
+  const int n_units = a.batch / a.n_q * a.n_kv_heads * nrb;
   // rows of a unit's block, tokens its last row sees (query j sees the tokens t < len - (n_q - 1 - j))
   auto unit_rows = [&](int rb) -> int { return min(R, all_rows - rb * R); };
   auto unit_len = [&](int seq, int rb) -> int {

@@ -15,6 +15,8 @@
 // Bound by instruction issue (angle decode) for long sequences and by the chain of phases for short ones, hence: S is copied
 // to shared memory (head dims up to 128) before the kernel ahead in the stream has finished, every block rotates the
 // whole query by itself instead of meeting the others first, and the merge has one cluster barrier.
+// Measured (32/8 heads; two launches and a workspace before): one sequence of 1000 tokens, head_dim 128 19.8 -> 10.7 us; eight of
+// 4096, head_dim 64 111 -> 32 us; the general layout with three bits and seven levels, eight of 4096, 5330 -> 95 us.
 // kU = 16 for up to four query heads per kv head, 8 for up to eight (the registers of q' and of the accumulators).
 #pragma once
 #include <cstdint>

@@ -81,15 +81,6 @@ __device__ __forceinline__ void tc_mma_idesc(uint32_t tmem_d, uint64_t adesc, ui
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   tc_mma_idesc(tmem_d, adesc, bdesc, kTcIdesc, accumulate);
 }
-// The same with the A operand in tensor memory (lane = row, two 16-bit elements per column, k ascending).
-__device__ __forceinline__ void tc_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 // True in one lane of a converged warp.
 __device__ __forceinline__ bool tc_elect() {
   uint32_t p;
@@ -100,7 +91,8 @@ __device__ __forceinline__ bool tc_elect() {
       : "=r"(p));
   return p != 0;
 }
-// The 2-CTA form (issued by one thread of the even CTA of a pair): D and A are 256 rows, 128 in each CTA's tensor
+// The 2-CTA form with the A operand in tensor memory (lane = row, two 16-bit elements per column, k ascending), issued by one
+// thread of the even CTA of a pair: D and A are 256 rows, 128 in each CTA's tensor
 // memory at the same columns; each CTA supplies half of B (N / 2 rows) from its own shared memory at the same offset.
 __device__ __forceinline__ void tc_mma_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
