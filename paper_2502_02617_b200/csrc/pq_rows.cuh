@@ -33,13 +33,24 @@ static_assert(kStages * kStageBytes <= kRowRingBytes, "ring");
 static_assert(kFastMaxSegs * sizeof(Segment) <= 448 && 448 + kRowMax * 8 <= 752 && kRowSmInfo % 8 == 0, "behind the segments");
 static_assert(kRowSmTotal <= 227 * 1024, "shared memory of one CTA");
 
-// One warp: copy S into the ring's place (nothing in it is in use any more; a barrier has ordered what was).
+// One warp: copy S into the ring's place (nothing in it is in use any more; a barrier has ordered what was).  Every copy is waited
+// for with wait_S before the block reuses the place or ends.
 __device__ __forceinline__ void fetch_S(const float* S, uint32_t ring, uint32_t bar, int lane) {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (lane == 0) mbar_expect_tx(bar, 128 * 512);
   __syncwarp();
 #pragma unroll 1
   for (int r = lane; r < 128; r += 32) bulk_load(ring + r * kRowSStride * 4, S + r * 128, 512, bar);
+}
+
+// Waits for copy `phase` of S.  Bounded, but a wait that gave up elsewhere does not cut it short: the copy is the block's own,
+// and it must not be in flight when its place is reused or the block ends.
+__device__ __forceinline__ void wait_S(uint32_t bar, uint32_t phase, volatile int* abort_flag) {
+  for (int i = 0; i < kSpinLimit; ++i) {
+    if (mbar_try_wait(bar, phase)) return;
+    if (i > 64) __nanosleep(64);
+  }
+  *abort_flag = 1;
 }
 
 // The last part of a unit: merge the `ns` partials of its rows in slot order, normalise, rotate back by S^T and store.
@@ -92,7 +103,7 @@ __device__ __forceinline__ void combine_rows(const DecodeArgs& a, const int2* in
     }
     *reinterpret_cast<float4*>(y_sm + 4 * i) = make_float4(acc.x * k, acc.y * k, acc.z * k, acc.w * k);
   }
-  mbar_wait(bar, phase, abort_flag);
+  wait_S(bar, phase, abort_flag);
   __syncthreads();
   // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of four rows at a time
   const int i_out = tid & 127;
@@ -150,7 +161,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   __syncthreads();
   const uint32_t ring = sm_base + kRowSmRing, bar_S = sm_base + kRowSmBarS;
   const float* S_sm = reinterpret_cast<const float*>(smem + kRowSmRing);
-  uint32_t n_S = 0;   // copies of S so far
+  uint32_t n_S = 0;   // copies of S waited for so far
 
   const int n_units = a.batch / a.n_q * a.n_kv_heads * nrb;
   // rows of a unit's block, tokens its last row sees (query j sees the tokens t < len - (n_q - 1 - j))
@@ -253,7 +264,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
             *reinterpret_cast<float4*>(q_in + 8 * i) = lo;
             *reinterpret_cast<float4*>(q_in + 8 * i + 4) = hi;
           }
-          if (r0 == 0) mbar_wait(bar_S, n_S++ & 1, abort_flag);
+          if (r0 == 0) wait_S(bar_S, n_S++ & 1, abort_flag);
           __syncthreads();
           float acc[kMine];
 #pragma unroll
@@ -501,6 +512,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
       __syncthreads();  // the ring is free again for the next unit
     }
   }
+  // A block whose range of the work lies between two units has no segment: the copy of S that it started ahead of the split lands
+  // before the block ends.
+  if (n_S == 0) wait_S(bar_S, 0u, abort_flag);
   if (tid == 0 && *abort_flag) set_status(a.status, PQ_ERR_TIMEOUT);
 }
 

@@ -123,3 +123,24 @@ def test_merge_of_parts(d, shift):
     pq.pq_merge_attention(parts, lse, out, status)
     w = torch.softmax(lse.double(), 0)[..., None]
     assert rel_l2(to_f64(out), (w * parts.double()).sum(0).cpu().numpy()) < 1e-6
+
+
+# Fewer stages of work than SMs: two units of 32 stages (and 7 empty positions each) over 148 blocks leave more than half of the
+# blocks without a segment.  They have started the copy of S all the same; the calls in between put other kernels' shared
+# memory where it lands.
+def test_rows_kernel_with_blocks_that_own_nothing():
+    lens, g, Hkv = [4096], 8, 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 31)
+    other, _ = _filled([4096], 4, 2, 128, 32)
+    q, q4 = synthetic.queries(6, 1, g * Hkv, 128, torch.float32, DEV), synthetic.queries(7, 1, 4, 128, torch.float32, DEV)
+    pq.pq_debug_fail_next_wait(5)
+    first4 = other.attend(q4)
+    outs, outs4 = [], []
+    for _ in range(20):
+        pq.pq_debug_fail_next_wait(5)
+        outs.append(cache.attend(q))
+        pq.pq_debug_fail_next_wait(5)
+        outs4.append(other.attend(q4))
+    assert rel_l2(to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)) < TOL_ATTENTION_F32_IO
+    assert all(torch.equal(o, outs[0]) for o in outs) and all(torch.equal(o, first4) for o in outs4)
+    cache.check_status()
