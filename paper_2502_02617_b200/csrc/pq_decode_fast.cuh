@@ -664,7 +664,12 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     };
     const bool hook = !kPaged && (a.debug & 1u) && unit_slot == 0 && cta == c_first;
     const bool producer = (tid & 255) == 0;
-    if (producer && n_li > 0) issue_copy(0);
+    if (producer && n_li > 0) {
+      // what list_segments, the merge or the combine left in the ring by ordinary accesses (a barrier has ordered them before this)
+      // comes before the copies into it
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue_copy(0);
+    }
     __syncwarp();
     // q' = (q S) * scale * log2(e) for the unit's query heads, as an fp16 value plus an fp16 residual.
     // The first stages of the segment are already on their way while this runs.

@@ -144,3 +144,20 @@ def test_rows_kernel_with_blocks_that_own_nothing():
     assert rel_l2(to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)) < TOL_ATTENTION_F32_IO
     assert all(torch.equal(o, outs[0]) for o in outs) and all(torch.equal(o, first4) for o in outs4)
     cache.check_status()
+
+
+# The persistent kernel's ring holds the scratch of the work split and the merge of the segment before when a segment's first copies
+# go into it: more units than blocks (several segments per block), some of one stage, repeated on changing neighbours.
+def test_persistent_kernel_reuses_its_ring_between_segments():
+    rng = np.random.default_rng(5)
+    lens, Hkv = [int(x) for x in rng.integers(1, 400, size=60)] + [2000], 8
+    cache, ref = _filled(lens, 4 * Hkv, Hkv, 128, 33)
+    q = synthetic.queries(8, len(lens), 4 * Hkv, 128, torch.float32, DEV)
+    outs = []
+    for _ in range(10):
+        pq.pq_debug_fail_next_wait(5)
+        outs.append(cache.attend(q))
+    assert all(torch.equal(o, outs[0]) for o in outs)
+    out, want = to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)
+    for b in range(len(lens)):
+        assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, lens[b]
