@@ -255,6 +255,7 @@ void note_cuda_error(cudaError_t e);
 // Test hook (pq_debug_fail_next_wait): returns true once after the hook was armed for `which`
 // (1 = tensor-core encoder, 2 = head_dim-128 decode attention) and disarms it.
 bool take_debug_wait_failure(int which);
+int take_debug_hook(int first, int last);   // the hook armed in first .. last, disarmed; 0 if there is none
 int32_t paging_from(const pq_paging* p, int head_dim, Paging* out);
 inline int32_t launch_status() {
   const cudaError_t e = cudaGetLastError();

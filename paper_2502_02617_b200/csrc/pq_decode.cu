@@ -676,6 +676,12 @@ struct AttentionPlan {
   int n_splits;
 };
 constexpr int kMaxSplits = 16;
+// Whether a kernel takes a call at all.
+static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_kv_heads, int g) {
+  if (kernel == kPersistentKernel) return g <= 4 && batch * n_q * n_kv_heads <= kFastMaxUnits;
+  if (kernel == kRowsKernel) return batch * n_kv_heads * cut_rows((int64_t)n_q * g).blocks <= kFastMaxUnits;
+  return true;
+}
 // Room for the parts of split tcgen05 calls in the workspace of pq_workspace_bytes: a call whose parts would not fit is split
 // less.  (148 SMs with 128 rows each, twice over, bound what a useful split can need.)
 __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
@@ -700,9 +706,10 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     plan.kernel = k;
     return true;
   };
-  if (g <= 4 && rows < 32 && pairs * n_kv_heads <= kFastMaxUnits) consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
+  if (rows < 32 && kernel_takes(kPersistentKernel, batch, n_q, n_kv_heads, g))
+    consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
   const RowCut cut = cut_rows(rows);
-  if (rows > 4 && batch * n_kv_heads * cut.blocks <= kFastMaxUnits) {
+  if (rows > 4 && kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
     const int groups = (cut.rows + 3) / 4;
     consider(18.0 + 3.2 * groups + batch * n_kv_heads * cut.blocks * tiles * (345.0 + 61.0 * (groups - 2)) / sm_hz, kRowsKernel);
   }
@@ -820,7 +827,12 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
       pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
       return pq::launch_status();
     }
-    const pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm);
+    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm);
+    if (const int named = pq::take_debug_hook(6, 9)) {   // test hook: the kernel is named
+      plan.kernel = named == 6 ? pq::kClusterKernel : named == 7 ? pq::kPersistentKernel : named == 8 ? pq::kRowsKernel : pq::kTensorKernel;
+      if (!pq::kernel_takes(plan.kernel, batch, n_q, n_kv_heads, g) || (plan.kernel == pq::kTensorKernel && lse_dev != nullptr))
+        return PQ_ERR_UNSUPPORTED;
+    }
     const bool forced = n_q * g <= 32 && pq::take_debug_wait_failure(5), fail_wait = n_q * g <= 32 && pq::take_debug_wait_failure(2);
     pq::AttentionKernel kernel = plan.kernel;
     if ((forced || fail_wait) && kernel == pq::kClusterKernel) kernel = plan.persistent;

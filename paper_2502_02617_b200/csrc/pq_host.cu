@@ -204,6 +204,10 @@ bool take_debug_wait_failure(int which) {
   int armed = which;
   return g_debug_wait_failure.compare_exchange_strong(armed, 0);
 }
+int take_debug_hook(int first, int last) {
+  int armed = g_debug_wait_failure.load(std::memory_order_relaxed);
+  return armed >= first && armed <= last && g_debug_wait_failure.compare_exchange_strong(armed, 0) ? armed : 0;
+}
 }  // namespace pq
 
 extern "C" {
@@ -231,7 +235,7 @@ const char* pq_status_string(int32_t status) {
 int32_t pq_token_block(void) { return pq::kTokenBlock; }
 
 int32_t pq_debug_fail_next_wait(int32_t which) {
-  if (which < 0 || which > 5) return PQ_ERR_INVALID_ARG;
+  if (which < 0 || which > 9) return PQ_ERR_INVALID_ARG;
   pq::g_debug_wait_failure.store(which);
   return PQ_OK;
 }

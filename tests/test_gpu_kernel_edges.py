@@ -16,63 +16,79 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _filled(lens, Hq, Hkv, d, seed, dtype=torch.bfloat16):
-    cache = pq.PolarQuantCache(len(lens), Hq, Hkv, d, capacity=max(lens), seed=seed, device=DEV)
+def _filled(lens, Hq, Hkv, d, seed, dtype=torch.bfloat16, paged=False):
+    if paged:
+        pages = -(-max(lens) // 128)
+        table = torch.randperm(len(lens) * pages, generator=torch.Generator().manual_seed(seed)).view(len(lens), pages)
+        cache = pq.PagedPolarQuantCache(len(lens), Hq, Hkv, d, 128, len(lens) * pages, table, seed=seed, device=DEV)
+    else:
+        cache = pq.PolarQuantCache(len(lens), Hq, Hkv, d, capacity=max(lens), seed=seed, device=DEV)
     K, V = synthetic.kv_like(seed + 1, sum(lens), Hkv, d, dtype, DEV, n_outliers=4 if d >= 64 else 0)
     cache.encode(K, V, torch.tensor(np.concatenate(([0], np.cumsum(lens))), dtype=torch.int32, device=DEV))
     return cache, _oracle_cache(cache, K, V, lens)
 
 
-# Rows of a kv head (queries x heads of the group) on both sides of every group of four that the rows kernel is built for
-# (8, 12, 16, 20, 24, 32), odd groups whose rows do not end with a query; lengths around its 16-token tiles and 128-token stages.
-@pytest.mark.parametrize("g,n_q", [(1, 5), (1, 8), (1, 9), (4, 3), (1, 13), (8, 2), (1, 17), (5, 4), (7, 3), (6, 4), (1, 25), (7, 4), (4, 8),
-                                   (8, 4), (1, 32)])
-def test_rows_kernel(g, n_q):
-    lens, Hkv = [16, 129, 397, 2, 128], 2
-    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 60 + g)
-    q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
-    pq.pq_debug_fail_next_wait(5)   # a call this small would go to the cluster kernel
+CLUSTER, PERSISTENT, ROWS, TCGEN05 = 6, 7, 8, 9    # pq_debug_fail_next_wait: the next attention call runs this kernel
+
+
+def _check_multi(cache, ref, q, lens, kernel):
+    pq.pq_debug_fail_next_wait(kernel)
     out = to_f64(cache.attend_multi(q))
+    n_q = q.shape[1]
     want = orc.multi_query_attention(to_f64(q), ref.k_codes, ref.k_radii, ref.v_codes, ref.v_radii, ref.lens, ref.cb, ref.S, 128 ** -0.5)
     for b in range(len(lens)):
         for j in range(n_q):
             if lens[b] - (n_q - 1 - j) <= 0:
                 assert np.all(out[b, j] == 0)
             else:
-                assert rel_l2(out[b, j], want[b, j]) < TOL_ATTENTION_F32_IO, (b, j)
+                assert rel_l2(out[b, j], want[b, j]) < TOL_ATTENTION_F32_IO, (kernel, b, j)
+
+
+# Rows of a kv head (queries x heads of the group) on both sides of every group of four that the rows kernel is built for
+# (8, 12, 16, 20, 24, 32) and beyond one row block, odd groups whose rows do not end with a query; lengths around its 16-token
+# tiles and 128-token stages; contiguous and behind a block table.
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("g,n_q", [(1, 1), (1, 5), (1, 8), (1, 9), (4, 3), (1, 13), (8, 2), (1, 17), (5, 4), (7, 3), (6, 4), (1, 25), (7, 4),
+                                   (4, 8), (8, 4), (1, 32), (8, 5), (3, 23)])
+def test_rows_kernel(g, n_q, paged):
+    lens, Hkv = [16, 129, 397, 2, 128], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 60 + g, paged=paged)
+    q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
+    _check_multi(cache, ref, q, lens, ROWS)
+
+
+def test_a_named_kernel_that_does_not_take_the_call_is_refused():
+    cache, _ = _filled([40], 16, 2, 128, 1)
+    q = synthetic.queries(1, 1, 16, 128, torch.float32, DEV)
+    pq.pq_debug_fail_next_wait(PERSISTENT)                      # eight heads per kv head
+    with pytest.raises(pq.PolarQuantError) as e:
+        cache.attend(q)
+    assert e.value.status == pq.ERR_UNSUPPORTED
 
 
 # The tcgen05 kernel: an odd count of 64-token blocks (half of a tile pair), fewer blocks than ranges (empty parts), more rows than
 # one pair of CTAs holds, a group size that leaves rows of the 128 unused, and 64-row tiles in the rotation kernels.
 @pytest.mark.parametrize("g,Hkv,n_q,lens", [(8, 1, 16, [1, 64, 65, 700]), (7, 2, 19, [1473, 40]), (4, 1, 70, [1000, 71, 64]),
-                                            (8, 8, 75, [90, 75, 300, 65, 76, 80, 91, 99])])
+                                            (8, 8, 75, [90, 75, 300, 65, 76, 80, 91, 99]), (4, 2, 8, [130] * 64), (1, 1, 32, [64, 3])])
 def test_tcgen05_multi_query_kernel_parts(g, Hkv, n_q, lens):
     cache, ref = _filled(lens, g * Hkv, Hkv, 128, 70 + g)
     q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
-    out = to_f64(cache.attend_multi(q))
-    want = orc.multi_query_attention(to_f64(q), ref.k_codes, ref.k_radii, ref.v_codes, ref.v_radii, ref.lens, ref.cb, ref.S, 128 ** -0.5)
-    for b in range(len(lens)):
-        for j in range(n_q):
-            if lens[b] - (n_q - 1 - j) <= 0:
-                assert np.all(out[b, j] == 0)
-            else:
-                assert rel_l2(out[b, j], want[b, j]) < TOL_ATTENTION_F32_IO, (b, j)
+    _check_multi(cache, ref, q, lens, TCGEN05)
 
 
 # The cluster kernel: lengths around its 16-token tiles, a warp without tokens, one head and every padding of the heads of a group;
-# the persistent kernel and the rows kernel (hook 5) on the same.
+# at head_dim 128 the persistent kernel (up to four heads) and the rows kernel on the same.
 @pytest.mark.parametrize("d,g", [(128, 1), (128, 3), (128, 5), (128, 8), (64, 2), (64, 7), (32, 4), (16, 1), (16, 8)])
 def test_single_query_kernels(d, g):
     lens, Hkv = [1, 15, 16, 17, 63, 64, 65, 255, 257, 1025], 2
     cache, ref = _filled(lens, g * Hkv, Hkv, d, 80 + g, torch.float32)
     q = synthetic.queries(5, len(lens), g * Hkv, d, torch.float32, DEV)
     want = ref.attend(to_f64(q), d ** -0.5)
-    for hook in (0, 5) if d == 128 else (0,):
-        if hook:
-            pq.pq_debug_fail_next_wait(hook)
+    for kernel in (0,) if d < 128 else (CLUSTER, PERSISTENT, ROWS) if g <= 4 else (CLUSTER, ROWS):
+        pq.pq_debug_fail_next_wait(kernel)
         out = to_f64(cache.attend(q))
         for b in range(len(lens)):
-            assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (hook, lens[b])
+            assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (kernel, lens[b])
 
 
 # Calls below 32 tokens have a kernel of their own (one block per sequence), larger ones tiles of 64 rows (float32 or d < 128)
@@ -133,13 +149,13 @@ def test_rows_kernel_with_blocks_that_own_nothing():
     cache, ref = _filled(lens, g * Hkv, Hkv, 128, 31)
     other, _ = _filled([4096], 4, 2, 128, 32)
     q, q4 = synthetic.queries(6, 1, g * Hkv, 128, torch.float32, DEV), synthetic.queries(7, 1, 4, 128, torch.float32, DEV)
-    pq.pq_debug_fail_next_wait(5)
+    pq.pq_debug_fail_next_wait(PERSISTENT)
     first4 = other.attend(q4)
     outs, outs4 = [], []
     for _ in range(20):
-        pq.pq_debug_fail_next_wait(5)
+        pq.pq_debug_fail_next_wait(ROWS)
         outs.append(cache.attend(q))
-        pq.pq_debug_fail_next_wait(5)
+        pq.pq_debug_fail_next_wait(PERSISTENT)
         outs4.append(other.attend(q4))
     assert rel_l2(to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)) < TOL_ATTENTION_F32_IO
     assert all(torch.equal(o, outs[0]) for o in outs) and all(torch.equal(o, first4) for o in outs4)
@@ -155,7 +171,7 @@ def test_persistent_kernel_reuses_its_ring_between_segments():
     q = synthetic.queries(8, len(lens), 4 * Hkv, 128, torch.float32, DEV)
     outs = []
     for _ in range(10):
-        pq.pq_debug_fail_next_wait(5)
+        pq.pq_debug_fail_next_wait(PERSISTENT)
         outs.append(cache.attend(q))
     assert all(torch.equal(o, outs[0]) for o in outs)
     out, want = to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)

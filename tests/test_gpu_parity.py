@@ -226,10 +226,9 @@ def test_multi_query_attention_is_causal_over_the_last_positions(d, Hq, Hkv, n_q
 
 @pytest.mark.parametrize("n_q,B", [(32, 80), (16, 80), (16, 32), (8, 64)])
 def test_multi_query_single_block_on_a_full_device(n_q, B):
-    """One query block per (kv head, sequence).  With more units than half the SMs the tcgen05 kernel runs one CTA per
-    unit, each decoding whole blocks; with fewer, a second CTA without rows shares the decoding.  Chunks of 32 to 127
-    rows take the kernel when the batch is large enough for it to beat one decode attention per query (here: all four
-    cases).  Against the oracle on the first and last sequence, against the register-fragment kernel everywhere."""
+    """The tcgen05 kernel (named to the dispatch) with one query block per (kv head, sequence), a second CTA without rows sharing
+    the decoding, and more pairs of CTAs than the device holds at once in three of the four cases.  Against the oracle on the
+    first and last sequence, against the register-fragment kernel and one decode attention everywhere."""
     d, Hq, Hkv, n = 128, 8, 2, 130
     lens_list = [n - (b % 3) for b in range(B)]
     cache = pq.PolarQuantCache(B, Hq, Hkv, d, capacity=n, seed=31, device=DEV)
@@ -239,6 +238,7 @@ def test_multi_query_single_block_on_a_full_device(n_q, B):
     g = torch.Generator(device=DEV)
     g.manual_seed(33)
     q = torch.randn((B, n_q, Hq, d), generator=g, device=DEV, dtype=torch.float32)
+    pq.pq_debug_fail_next_wait(9)
     out = cache.attend_multi(q)
     torch.cuda.synchronize()
     cache.check_status()
