@@ -259,12 +259,12 @@ struct PackedSplit {
 };
 
 template <int D>
-static int32_t launch_packed_attention(const SplitCommon& c, int64_t pairs, int n_q, int max_len, const Tables* tables,
-                                       const uint8_t* cache, const int32_t* lens, const Paging& pg, cudaStream_t stream) {
+static PackedSplit<D> packed_split(const SplitCommon& c, int n_q, const Tables* tables, const uint8_t* cache, const int32_t* lens,
+                                   const Paging& pg) {
   PackedSplit<D> p;
   p.c = c; p.n_q = n_q; p.tables = tables; p.cache = cache; p.lens = lens; p.pg = pg;
   p.head_bytes = make_layout(D, pg.page_tokens).head_bytes;
-  return dispatch_split_attention(p, pairs, max_len, stream);
+  return p;
 }
 
 // ---- partial attentions: merge, and exact attention over an uncompressed window -----------------
@@ -687,12 +687,11 @@ static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_k
 __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
   return std::max(pairs * n_q_heads, std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128));
 }
-static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm) {
+// `tokens`: what the busiest SM of the cluster kernel goes through (plan_split).
+static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm, int64_t tokens) {
   AttentionPlan plan = {kClusterKernel, kClusterKernel, 1};
   const int64_t pairs = batch * n_q, rows = (int64_t)n_q * g;
   const double tiles = std::ceil(max_len / 16.0), sm_hz = n_sm * 1900.0;   // cycles per us of the device
-  int64_t tokens = 0;
-  split_cluster_size(128, 16, pairs * n_kv_heads, max_len, n_sm, &tokens);
   // (From 32 rows on only the kernels that decode a block once for many rows are considered.)
   double best = rows >= 32 ? 1e30 : (g <= 2 ? 8.0 : 9.0) + tokens * (g <= 2 ? 0.013 : g <= 4 ? 0.017 : 0.044);
   double best_persistent = 1e30;
@@ -812,6 +811,9 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.qrot = nullptr; a.epoch = a.debug = 0u;
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
+  pq::SplitCommon c;
+  c.d = head_dim; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
+  c.S = S_dev; c.q = q_dev; c.out = out_dev; c.lse = lse_dev; c.status = status_dev;
   if (head_dim == 128) {
     const bool paged = pg.table != nullptr;
     static pq::DeviceMemo sm_count;
@@ -827,7 +829,11 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
       pq::prefill_attention_kernel<<<grid, pq::kPfThreads, pq::kPfTotal, st>>>(a, n_q);
       return pq::launch_status();
     }
-    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm);
+    pq::PackedSplit<128> split = pq::packed_split<128>(c, n_q, a.tables, a.cache, cache_lens_dev, pg);
+    pq::size_split(split);
+    int64_t tokens = 0;
+    if (pq::plan_split(split, pairs, max_len, &tokens) == 0) return PQ_ERR_CUDA;
+    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, tokens);
     if (const int named = pq::take_debug_hook(6, 9)) {   // test hook: the kernel is named
       plan.kernel = named == 6 ? pq::kClusterKernel : named == 7 ? pq::kPersistentKernel : named == 8 ? pq::kRowsKernel : pq::kTensorKernel;
       if (!pq::kernel_takes(plan.kernel, batch, n_q, n_kv_heads, g) || (plan.kernel == pq::kTensorKernel && lse_dev != nullptr))
@@ -847,14 +853,11 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
       return pq::launch_persistent(fast, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
     }
   }
-  pq::SplitCommon c;
-  c.d = head_dim; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.io_dtype = io_dtype; c.scale = scale;
-  c.S = S_dev; c.q = q_dev; c.out = out_dev; c.lse = lse_dev; c.status = status_dev;
   switch (head_dim) {
-    case 16: return pq::launch_packed_attention<16>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
-    case 32: return pq::launch_packed_attention<32>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
-    case 64: return pq::launch_packed_attention<64>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
-    default: return pq::launch_packed_attention<128>(c, pairs, n_q, max_len, a.tables, a.cache, cache_lens_dev, pg, st);
+    case 16: return pq::dispatch_split_attention(pq::packed_split<16>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
+    case 32: return pq::dispatch_split_attention(pq::packed_split<32>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
+    case 64: return pq::dispatch_split_attention(pq::packed_split<64>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
+    default: return pq::dispatch_split_attention(pq::packed_split<128>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
   }
 }
 

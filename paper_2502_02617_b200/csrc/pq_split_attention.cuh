@@ -455,16 +455,52 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
   if (C > 1) cluster_wait();
 }
 
-// Blocks per cluster: a power of two that divides d, four tiles per block or more, at most 8 (the portable limit; with 16 blocks
-// of this size few clusters find room in a GPC at once).  The choice is the one with the shortest estimated time: waves of
-// resident blocks times (tokens of a block plus what its set-up and merge cost, as long as 25000 / d tokens).  *tokens
-// becomes the former product without the overhead: what the busiest SM goes through.
-inline int split_cluster_size(int d, int tile, int64_t units, int max_len, int n_sm, int64_t* tokens) {
+// Clusters of 2^log2c blocks that the device holds at once, one block per SM: a cluster lies inside a GPC, whose SMs need not be
+// a multiple of its size (measured: 148 SMs hold 33 clusters of four, 15 of eight, 7 of sixteen).  The runtime is asked once per
+// kernel, device and amount of shared memory; `memo` keeps (bytes + 1) << 32 | answer.
+constexpr int kClusterSizes = 5;
+using ClusterMemo = std::atomic<int64_t>[kMaxDevices][kClusterSizes];
+template <typename Kernel>
+inline int clusters_at_once(Kernel kernel, int threads, int smem, int log2c, int n_sm, ClusterMemo& memo) {
+  if (log2c == 0) return n_sm;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return n_sm >> log2c;
+  const int64_t known = memo[dev][log2c].load(std::memory_order_relaxed);
+  if (known >> 32 == smem + 1) return (int)(known & 0x7fffffff);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1 << log2c, (unsigned)n_sm);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1u << log2c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  n = n < (n_sm >> log2c) ? n : n_sm >> log2c;
+  memo[dev][log2c].store((int64_t)(smem + 1) << 32 | n, std::memory_order_relaxed);
+  return n;
+}
+
+// Blocks per cluster: a power of two that divides d, four tiles per block or more, at most 16 (above the portable limit of 8: for
+// a few units of a long context).  The choice is the one with the shortest estimated time: waves of clusters that
+// are resident together times (tokens of a block plus what its set-up and merge cost, as long as 25000 / d tokens).  *tokens
+// becomes the former product without the overhead: what the busiest SM goes through.  room(i): clusters of 2^i blocks at once.
+template <class Room>
+inline int split_cluster_size(int d, int tile, int64_t units, int max_len, Room room, int64_t* tokens) {
   int best = 1;
   int64_t best_cost = INT64_MAX;
-  for (int C = 1; C <= 8 && C <= d; C *= 2) {
+  for (int i = 0, C = 1; i < kClusterSizes && C <= d; ++i, C *= 2) {
     if (C > 1 && (int64_t)(C / 2) * tile * 4 >= max_len) break;   // half as many blocks already have no more than four tiles each
-    const int64_t waves = (units * C + n_sm - 1) / n_sm;
+    const int at_once = room(i);
+    if (at_once <= 0) continue;
+    const int64_t waves = (units + at_once - 1) / at_once;
     const int64_t cost = waves * ((max_len + C - 1) / C + 25000 / d);
     if (cost < best_cost) {
       best_cost = cost;
@@ -475,17 +511,27 @@ inline int split_cluster_size(int d, int tile, int64_t units, int max_len, int n
   return best;
 }
 
-// `configured`: one DeviceMemo per instantiation.
+// The kernel's cluster size for a call, 0 with the CUDA error noted; P sized by size_split.
 template <class P, int kH>
-int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStream_t stream) {
+int plan_split_as(const P& p, int64_t pairs, int max_len, int64_t* tokens) {
   static DeviceMemo configured;
+  static ClusterMemo memo;
   auto kernel = split_attention_kernel<P, kH>;
   const int n_sm = configure_for_device(kernel, kSplitSmemMax, configured, true);
-  if (n_sm == 0) return PQ_ERR_CUDA;
+  if (n_sm == 0) return 0;
+  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
+  return split_cluster_size(p.c.d, p.c.tile, pairs * p.c.n_kv_heads, max_len,
+                            [&](int i) { return clusters_at_once(kernel, 32 * split_warps(kH), smem, i, n_sm, memo); }, tokens);
+}
+
+template <class P, int kH>
+int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStream_t stream) {
+  auto kernel = split_attention_kernel<P, kH>;
   const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
   if (smem > kSplitSmemMax) return PQ_ERR_UNSUPPORTED;
   int64_t tokens;
-  const int C = split_cluster_size(p.c.d, p.c.tile, pairs * p.c.n_kv_heads, max_len, n_sm, &tokens);
+  const int C = plan_split_as<P, kH>(p, pairs, max_len, &tokens);
+  if (C == 0) return PQ_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C, p.c.n_kv_heads, (unsigned)pairs);
   cfg.blockDim = dim3(32 * split_warps(kH));
@@ -509,16 +555,29 @@ int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStrea
   return launch_status();
 }
 
-// The instantiation for the group size.  Tiles of 16 tokens (32 where a lane takes a whole token), fewer where long rows
-// would take more than 200 KB of shared memory.
+// Tiles of 16 tokens (32 where a lane takes a whole token), fewer where long rows would take more than 200 KB of shared memory.
 template <class P>
-int32_t dispatch_split_attention(P p, int64_t pairs, int max_len, cudaStream_t stream) {
+void size_split(P& p) {
   const int kh = split_heads(p.c.n_q_heads / p.c.n_kv_heads), lanes = split_lanes(p.c.d, kh);
   int T = lanes == 1 ? 32 : 16;
   while (T > 32 / lanes && split_smem_bytes(p.c.d, kh, p.tile_bytes(T)) > 200 * 1024) T /= 2;
   p.c.tile = T;
   p.c.stage_bytes = p.tile_bytes(T);
-  switch (kh) {
+}
+// The instantiation for the group size.
+template <class P>
+int plan_split(const P& p, int64_t pairs, int max_len, int64_t* tokens) {
+  switch (split_heads(p.c.n_q_heads / p.c.n_kv_heads)) {
+    case 1: return plan_split_as<P, 1>(p, pairs, max_len, tokens);
+    case 2: return plan_split_as<P, 2>(p, pairs, max_len, tokens);
+    case 4: return plan_split_as<P, 4>(p, pairs, max_len, tokens);
+    default: return plan_split_as<P, 8>(p, pairs, max_len, tokens);
+  }
+}
+template <class P>
+int32_t dispatch_split_attention(P p, int64_t pairs, int max_len, cudaStream_t stream) {
+  size_split(p);
+  switch (split_heads(p.c.n_q_heads / p.c.n_kv_heads)) {
     case 1: return launch_split_attention<P, 1>(p, pairs, max_len, stream);
     case 2: return launch_split_attention<P, 2>(p, pairs, max_len, stream);
     case 4: return launch_split_attention<P, 4>(p, pairs, max_len, stream);

@@ -91,6 +91,17 @@ def test_single_query_kernels(d, g):
             assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (kernel, lens[b])
 
 
+# One or two units of a longer sequence: clusters of sixteen blocks (the limit), also where a block un-rotates one coordinate.
+@pytest.mark.parametrize("d,g,Hkv", [(128, 1, 1), (128, 8, 2), (64, 4, 1), (32, 2, 2), (16, 1, 1), (16, 8, 1)])
+def test_cluster_kernel_with_sixteen_blocks(d, g, Hkv):
+    lens = [4101]
+    cache, ref = _filled(lens, g * Hkv, Hkv, d, 90 + g, torch.float32)
+    q = synthetic.queries(5, 1, g * Hkv, d, torch.float32, DEV)
+    if d == 128:
+        pq.pq_debug_fail_next_wait(CLUSTER)
+    assert rel_l2(to_f64(cache.attend(q)), ref.attend(to_f64(q), d ** -0.5)) < TOL_ATTENTION_F32_IO
+
+
 # Calls below 32 tokens have a kernel of their own (one block per sequence), larger ones tiles of 64 rows (float32 or d < 128)
 # or of 128 (bf16, d = 128): the same codes whatever pieces the tokens come in, and the first piece against the oracle.  The radii
 # are float32 sums in another order before they are rounded to fp16: neighbours at most, 2^-10 apart.
