@@ -662,14 +662,15 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
 
 // ---- which kernel takes a head_dim-128 call ------------------------------------------------------
 // Four kernels compute the same attention; which is fastest depends on the rows per kv head (queries x heads of the group), on
-// the number of (kv head, sequence) units and on the length.  Each is estimated in us, from measurements on B200 (SM clock
-// 1.9 GHz), and the shortest estimate wins:
-//   * cluster kernel, a unit per (query, kv head, sequence): 9 us (8 with up to two heads), then 0.013 / 0.017 / 0.044 us
-//     per token of its busiest SM with up to 2 / 4 / 8 heads;
-//   * persistent kernel, up to four heads, a unit per (query, kv head, sequence): 15 us, then 280 SM cycles per 16-token tile;
-//   * rows kernel, up to 32 rows decoded together: 24 .. 43 us, then 345 + 61 (groups of four rows - 2) cycles per tile;
-//   * tcgen05 kernel, up to 256 rows per decoded block: 1.1 us per 64-token block of a pair of CTAs, 26 us per wave, 12 us for
-//     rotating the queries before and merging and rotating back after.
+// the number of (kv head, sequence) units and on the length.  Each is estimated in us by a formula fitted to measurements on
+// B200 (SM clock 1.9 GHz; 1 to 64 queries, 1 to 16 sequences of 150 to 32768 tokens, 32/8, 28/4, 20/4, 16/2, 8/8, 8/4, 8/2 and 8/1
+// heads), and the shortest estimate wins; over those calls the choice is 0.3 % slower than the best one on average, 20 % at worst:
+//   * cluster kernel, a unit per (query, kv head, sequence): start and end, then per token of a block and wave;
+//   * persistent kernel, a unit per (query, kv head, sequence) too: start and end, then 268 SM cycles per 16-token tile (320 with
+//     more than four heads), more where a block has several units, and the merge of a unit's parts;
+//   * rows kernel, up to 32 rows decoded together: the same with 2.8 us per group of four rows and 278 + 50 groups cycles per tile;
+//   * tcgen05 kernel, up to 256 rows per decoded block, from 32 rows on: 1.1 us per 64-token block of a pair of CTAs; rotating the
+//     queries before and merging and rotating back after grow with the rows and the parts.
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
@@ -678,7 +679,7 @@ struct AttentionPlan {
 constexpr int kMaxSplits = 16;
 // Whether a kernel takes a call at all.
 static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_kv_heads, int g) {
-  if (kernel == kPersistentKernel) return g <= 4 && batch * n_q * n_kv_heads <= kFastMaxUnits;
+  if (kernel == kPersistentKernel) return batch * n_q * n_kv_heads <= kFastMaxUnits;
   if (kernel == kRowsKernel) return batch * n_kv_heads * cut_rows((int64_t)n_q * g).blocks <= kFastMaxUnits;
   return true;
 }
@@ -687,41 +688,53 @@ static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_k
 __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
   return std::max(pairs * n_q_heads, std::min<int64_t>(kMaxSplits * pairs * n_q_heads, 2 * 160 * 128));
 }
-// `tokens`: what the busiest SM of the cluster kernel goes through (plan_split).
-static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm, int64_t tokens) {
-  AttentionPlan plan = {kClusterKernel, kClusterKernel, 1};
-  const int64_t pairs = batch * n_q, rows = (int64_t)n_q * g;
+// `load`: of the cluster kernel (plan_split).  `tensor`: the tcgen05 kernel may be taken.
+static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int g, int max_len, int n_sm, const SplitLoad& load, bool tensor) {
+  const double kNever = 1e30;
+  const int64_t pairs = batch * n_q, rows = (int64_t)n_q * g, stages = ((int64_t)max_len + kStageTokens - 1) / kStageTokens;
   const double tiles = std::ceil(max_len / 16.0), sm_hz = n_sm * 1900.0;   // cycles per us of the device
-  // (From 32 rows on only the kernels that decode a block once for many rows are considered.)
-  double best = rows >= 32 ? 1e30 : (g <= 2 ? 8.0 : 9.0) + tokens * (g <= 2 ? 0.013 : g <= 4 ? 0.017 : 0.044);
-  double best_persistent = 1e30;
-  auto consider = [&](double t, AttentionKernel k) {
-    if (k != kTensorKernel && t < best_persistent) {
-      best_persistent = t;
-      plan.persistent = k;
-    }
-    if (t >= best) return false;
-    best = t;
-    plan.kernel = k;
-    return true;
+  // of a persistent schedule (list_segments): units of a block beyond its first one, log2 of the parts of a unit
+  auto more_units = [&](int64_t units) -> double {
+    const double range = units * (stages + kSegmentCost) / (double)n_sm - (kSegmentCost + 1.5);
+    return range <= 0.0 ? 0.0 : 1.0 + std::floor(range / (stages + kSegmentCost));
   };
-  if (rows < 32 && kernel_takes(kPersistentKernel, batch, n_q, n_kv_heads, g))
-    consider(15.0 + pairs * n_kv_heads * tiles * 280.0 / sm_hz, kPersistentKernel);
-  const RowCut cut = cut_rows(rows);
-  if (rows > 4 && kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
-    const int groups = (cut.rows + 3) / 4;
-    consider(18.0 + 3.2 * groups + batch * n_kv_heads * cut.blocks * tiles * (345.0 + 61.0 * (groups - 2)) / sm_hz, kRowsKernel);
+  auto log_parts = [&](int64_t units) { return std::log2(std::min((double)stages, std::max(1.0, (double)n_sm / units))); };
+  double est[4] = {kNever, kNever, kNever, kNever};
+  AttentionPlan plan = {kClusterKernel, kClusterKernel, 1};
+  est[kClusterKernel] = g <= 2   ? 8.2 + 0.0136 * load.waves * load.tokens + 6.3 * (load.waves - 1)
+                        : g <= 4 ? 9.5 + 0.0223 * load.waves * load.tokens + 9.0 * (load.waves - 1)
+                                 : 13.5 + 0.0422 * load.waves * load.tokens + 13.4 * (load.waves - 1);
+  if (kernel_takes(kPersistentKernel, batch, n_q, n_kv_heads, g)) {
+    const int64_t units = pairs * n_kv_heads;
+    const double full = std::max(0.0, units / (double)n_sm - 1.0);
+    est[kPersistentKernel] = g <= 4 ? 16.2 + units * tiles * 268.0 / sm_hz + 3.6 * more_units(units) + 5.2 * full + 1.2 * log_parts(units) / units
+                                    : 20.8 + units * tiles * 320.0 / sm_hz + 5.2 * more_units(units) + 9.1 * full + 2.9 * log_parts(units) / units;
   }
-  if (rows >= 32) {
+  if (kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
+    const RowCut cut = cut_rows(rows);
+    const int64_t units = batch * n_kv_heads * cut.blocks;
+    const int groups = (cut.rows + 3) / 4;
+    est[kRowsKernel] = 18.2 + units * tiles * (278.0 + 50.0 * groups) / sm_hz + groups * (2.8 + 1.4 * more_units(units) + 0.9 * log_parts(units) / units);
+  }
+  if (tensor) {
     const int qb_rows = kPtRows / g;
-    const int64_t q_blocks = (n_q + qb_rows - 1) / qb_rows, blocks = (max_len + kTokenBlock - 1) / kTokenBlock;
-    const int64_t room = part_rows_room(pairs, (int64_t)n_kv_heads * g) / (pairs * n_kv_heads * g);
+    const int64_t q_blocks = (n_q + qb_rows - 1) / qb_rows, blocks = ((int64_t)max_len + kTokenBlock - 1) / kTokenBlock;
+    const int64_t all_rows = pairs * n_kv_heads * g, room = part_rows_room(pairs, (int64_t)n_kv_heads * g) / all_rows;
     for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
-      const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s;   // two query blocks each
-      const double waves = std::ceil((double)clusters / (n_sm / 2));
-      if (consider(waves * (std::ceil((double)blocks / s) * 1.1 + 26.0) + 12.0, kTensorKernel)) plan.n_splits = s;
+      const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s, at_once = n_sm / 2;   // two query blocks each
+      const double waves = (double)((clusters + at_once - 1) / at_once), work = waves * ((blocks + s - 1) / s);
+      const double t = 18.0 + 1.11 * work + 1.1 * std::min(work, 4.0) + 5.2 * clusters / (at_once * waves) +
+                       2.6e-3 * std::min<int64_t>(all_rows, 3000) + 1.06e-3 * all_rows + 0.36e-3 * s * all_rows;
+      if (t < est[kTensorKernel]) {
+        est[kTensorKernel] = t;
+        plan.n_splits = s;
+      }
     }
   }
+  for (AttentionKernel k : {kPersistentKernel, kRowsKernel, kTensorKernel})
+    if (est[k] < est[plan.kernel]) plan.kernel = k;
+  plan.persistent = est[kPersistentKernel] <= est[kRowsKernel] ? kPersistentKernel : kRowsKernel;
+  if (est[plan.persistent] == kNever) plan.persistent = kClusterKernel;   // too many units for either
   return plan;
 }
 
@@ -831,9 +844,9 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     }
     pq::PackedSplit<128> split = pq::packed_split<128>(c, n_q, a.tables, a.cache, cache_lens_dev, pg);
     pq::size_split(split);
-    int64_t tokens = 0;
-    if (pq::plan_split(split, pairs, max_len, &tokens) == 0) return PQ_ERR_CUDA;
-    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, tokens);
+    pq::SplitLoad load = {};
+    if (pq::plan_split(split, pairs, max_len, &load) == 0) return PQ_ERR_CUDA;
+    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, load, lse_dev == nullptr && n_q * g >= 32);
     if (const int named = pq::take_debug_hook(6, 9)) {   // test hook: the kernel is named
       plan.kernel = named == 6 ? pq::kClusterKernel : named == 7 ? pq::kPersistentKernel : named == 8 ? pq::kRowsKernel : pq::kTensorKernel;
       if (!pq::kernel_takes(plan.kernel, batch, n_q, n_kv_heads, g) || (plan.kernel == pq::kTensorKernel && lse_dev != nullptr))
@@ -847,9 +860,11 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     if (kernel == pq::kRowsKernel) return pq::launch_rows_attention(a, pq::cut_rows((int64_t)n_q * g), batch, paged, st);
     if (kernel == pq::kPersistentKernel) {
       a.epoch = pq::next_epoch();
-      static pq::DeviceMemo configured[2];
-      void (*fast)(pq::DecodeArgs) = paged ? pq::decode_attention_fast_kernel<true> : pq::decode_attention_fast_kernel<false>;
-      if (pq::configure_for_device(fast, pq::kSmTotal, configured[paged]) == 0) return PQ_ERR_CUDA;
+      static pq::DeviceMemo configured[4];
+      void (*fast)(pq::DecodeArgs) =
+          g <= 4 ? (paged ? pq::decode_attention_fast_kernel<1, true> : pq::decode_attention_fast_kernel<1, false>)
+                 : (paged ? pq::decode_attention_fast_kernel<2, true> : pq::decode_attention_fast_kernel<2, false>);
+      if (pq::configure_for_device(fast, pq::kSmTotal, configured[(g > 4 ? 2 : 0) + (paged ? 1 : 0)]) == 0) return PQ_ERR_CUDA;
       return pq::launch_persistent(fast, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
     }
   }

@@ -529,12 +529,11 @@ __device__ __forceinline__ void elect_combiner(const DecodeArgs& a, int u, int u
   }
 }
 
-// Up to four query heads per kv head; more are taken by rows_attention_kernel.
+// kHG: groups of four query heads per kv head (1 or 2).
 // kPaged: the cache lies behind a block table (the contiguous instantiation carries none of that code: the kernel
 // sits at its register limit).
-template <bool kPaged>
+template <int kHG, bool kPaged>
 __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(DecodeArgs a) {
-  constexpr int kHG = 1;   // groups of four query heads
   extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((kSmAlign - (smem_u32(smem_raw) & (kSmAlign - 1))) & (kSmAlign - 1));
   const int g_heads = a.n_q_heads / a.n_kv_heads;
@@ -567,7 +566,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
 #pragma unroll
       for (int e = 0; e < 4; ++e) s_col[4 * i + e] = ld_const_now(a.S + (16 * i + rot_k + e) * 128 + rot_j);
   };
-  load_s_col();
+  if (kHG == 1) load_s_col();   // two groups: held through the work split, the 32 registers spill
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
 
@@ -680,7 +679,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       for (int i = tid; i < g_heads * 128; i += kFastThreads)
         q_in[i] = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[q0 + i])
                                               : reinterpret_cast<const float*>(a.q)[q0 + i];
-      if (batch_no + sg > 0) load_s_col();
+      if (kHG > 1 || batch_no + sg > 0) load_s_col();
       __syncthreads();
 #pragma unroll 1
       for (int h = 0; h < g_heads; ++h) {

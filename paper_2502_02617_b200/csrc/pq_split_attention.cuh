@@ -490,10 +490,13 @@ inline int clusters_at_once(Kernel kernel, int threads, int smem, int log2c, int
 
 // Blocks per cluster: a power of two that divides d, four tiles per block or more, at most 16 (above the portable limit of 8: for
 // a few units of a long context).  The choice is the one with the shortest estimated time: waves of clusters that
-// are resident together times (tokens of a block plus what its set-up and merge cost, as long as 25000 / d tokens).  *tokens
-// becomes the former product without the overhead: what the busiest SM goes through.  room(i): clusters of 2^i blocks at once.
+// are resident together times (tokens of a block plus what its set-up and merge cost, as long as 25000 / d tokens).  room(i):
+// clusters of 2^i blocks at once.
+struct SplitLoad {
+  int64_t waves, tokens;   // of the choice: waves of clusters, tokens of a block in each
+};
 template <class Room>
-inline int split_cluster_size(int d, int tile, int64_t units, int max_len, Room room, int64_t* tokens) {
+inline int split_cluster_size(int d, int tile, int64_t units, int max_len, Room room, SplitLoad* load) {
   int best = 1;
   int64_t best_cost = INT64_MAX;
   for (int i = 0, C = 1; i < kClusterSizes && C <= d; ++i, C *= 2) {
@@ -505,7 +508,7 @@ inline int split_cluster_size(int d, int tile, int64_t units, int max_len, Room 
     if (cost < best_cost) {
       best_cost = cost;
       best = C;
-      *tokens = waves * ((max_len + C - 1) / C);
+      *load = {waves, (max_len + C - 1) / C};
     }
   }
   return best;
@@ -513,7 +516,7 @@ inline int split_cluster_size(int d, int tile, int64_t units, int max_len, Room 
 
 // The kernel's cluster size for a call, 0 with the CUDA error noted; P sized by size_split.
 template <class P, int kH>
-int plan_split_as(const P& p, int64_t pairs, int max_len, int64_t* tokens) {
+int plan_split_as(const P& p, int64_t pairs, int max_len, SplitLoad* load) {
   static DeviceMemo configured;
   static ClusterMemo memo;
   auto kernel = split_attention_kernel<P, kH>;
@@ -521,7 +524,7 @@ int plan_split_as(const P& p, int64_t pairs, int max_len, int64_t* tokens) {
   if (n_sm == 0) return 0;
   const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
   return split_cluster_size(p.c.d, p.c.tile, pairs * p.c.n_kv_heads, max_len,
-                            [&](int i) { return clusters_at_once(kernel, 32 * split_warps(kH), smem, i, n_sm, memo); }, tokens);
+                            [&](int i) { return clusters_at_once(kernel, 32 * split_warps(kH), smem, i, n_sm, memo); }, load);
 }
 
 template <class P, int kH>
@@ -529,8 +532,8 @@ int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStrea
   auto kernel = split_attention_kernel<P, kH>;
   const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
   if (smem > kSplitSmemMax) return PQ_ERR_UNSUPPORTED;
-  int64_t tokens;
-  const int C = plan_split_as<P, kH>(p, pairs, max_len, &tokens);
+  SplitLoad load;
+  const int C = plan_split_as<P, kH>(p, pairs, max_len, &load);
   if (C == 0) return PQ_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C, p.c.n_kv_heads, (unsigned)pairs);
@@ -566,12 +569,12 @@ void size_split(P& p) {
 }
 // The instantiation for the group size.
 template <class P>
-int plan_split(const P& p, int64_t pairs, int max_len, int64_t* tokens) {
+int plan_split(const P& p, int64_t pairs, int max_len, SplitLoad* load) {
   switch (split_heads(p.c.n_q_heads / p.c.n_kv_heads)) {
-    case 1: return plan_split_as<P, 1>(p, pairs, max_len, tokens);
-    case 2: return plan_split_as<P, 2>(p, pairs, max_len, tokens);
-    case 4: return plan_split_as<P, 4>(p, pairs, max_len, tokens);
-    default: return plan_split_as<P, 8>(p, pairs, max_len, tokens);
+    case 1: return plan_split_as<P, 1>(p, pairs, max_len, load);
+    case 2: return plan_split_as<P, 2>(p, pairs, max_len, load);
+    case 4: return plan_split_as<P, 4>(p, pairs, max_len, load);
+    default: return plan_split_as<P, 8>(p, pairs, max_len, load);
   }
 }
 template <class P>

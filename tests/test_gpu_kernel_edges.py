@@ -58,12 +58,23 @@ def test_rows_kernel(g, n_q, paged):
 
 
 def test_a_named_kernel_that_does_not_take_the_call_is_refused():
-    cache, _ = _filled([40], 16, 2, 128, 1)
-    q = synthetic.queries(1, 1, 16, 128, torch.float32, DEV)
-    pq.pq_debug_fail_next_wait(PERSISTENT)                      # eight heads per kv head
-    with pytest.raises(pq.PolarQuantError) as e:
-        cache.attend(q)
-    assert e.value.status == pq.ERR_UNSUPPORTED
+    cache = pq.PolarQuantCache(2049, 2, 1, 128, capacity=64, device=DEV)   # more units than the persistent schedules handle
+    q = synthetic.queries(1, 2049, 2, 128, torch.bfloat16, DEV)
+    for kernel in (PERSISTENT, ROWS):
+        pq.pq_debug_fail_next_wait(kernel)
+        with pytest.raises(pq.PolarQuantError) as e:
+            cache.attend(q)
+        assert e.value.status == pq.ERR_UNSUPPORTED
+
+
+# The persistent kernel with five to eight heads per kv head, a unit per query, both cache layouts.
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("g,n_q", [(5, 3), (8, 5), (7, 12)])
+def test_persistent_kernel_with_two_groups_of_heads(g, n_q, paged):
+    lens, Hkv = [16, 129, 1397, 12, 128], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 40 + g, paged=paged)
+    q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
+    _check_multi(cache, ref, q, lens, PERSISTENT)
 
 
 # The tcgen05 kernel: an odd count of 64-token blocks (half of a tile pair), fewer blocks than ranges (empty parts), more rows than
@@ -77,14 +88,14 @@ def test_tcgen05_multi_query_kernel_parts(g, Hkv, n_q, lens):
 
 
 # The cluster kernel: lengths around its 16-token tiles, a warp without tokens, one head and every padding of the heads of a group;
-# at head_dim 128 the persistent kernel (up to four heads) and the rows kernel on the same.
+# at head_dim 128 the persistent kernel (both instantiations) and the rows kernel on the same.
 @pytest.mark.parametrize("d,g", [(128, 1), (128, 3), (128, 5), (128, 8), (64, 2), (64, 7), (32, 4), (16, 1), (16, 8)])
 def test_single_query_kernels(d, g):
     lens, Hkv = [1, 15, 16, 17, 63, 64, 65, 255, 257, 1025], 2
     cache, ref = _filled(lens, g * Hkv, Hkv, d, 80 + g, torch.float32)
     q = synthetic.queries(5, len(lens), g * Hkv, d, torch.float32, DEV)
     want = ref.attend(to_f64(q), d ** -0.5)
-    for kernel in (0,) if d < 128 else (CLUSTER, PERSISTENT, ROWS) if g <= 4 else (CLUSTER, ROWS):
+    for kernel in (0,) if d < 128 else (CLUSTER, PERSISTENT, ROWS):
         pq.pq_debug_fail_next_wait(kernel)
         out = to_f64(cache.attend(q))
         for b in range(len(lens)):
