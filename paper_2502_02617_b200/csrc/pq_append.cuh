@@ -15,6 +15,8 @@
 
 namespace pq {
 
+static int32_t launch_advance_lens(const EncodeArgs& a, int32_t* lens, cudaStream_t stream);
+
 constexpr int kRowsThreads = 1024;
 template <int D>
 struct RowsShape {
@@ -50,7 +52,8 @@ __device__ __forceinline__ double warp_quant_exact(double y, const Tables& tb, i
   return __shfl_sync(0xffffffffu, y, 0);
 }
 
-template <int D>
+// kFlat: the blocks share all rows evenly, whatever sequences they belong to, and another launch advances the lengths.
+template <int D, bool kFlat>
 __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __grid_constant__ EncodeArgs a, int32_t* lens) {
   using R = RowsShape<D>;
   extern __shared__ __align__(16) float rows_smem[];
@@ -74,15 +77,21 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   const int b = blockIdx.y, rank = blockIdx.x, C = gridDim.x;   // the cluster spans x
-  int first = b, count = 1;
-  if (a.cu_seqlens != nullptr) {
-    first = a.cu_seqlens[b];
-    count = a.cu_seqlens[b + 1] - first;
+  int first = 0, count = 0, rows = a.total_tokens, start = 0;
+  bool fits = false;
+  if (!kFlat) {
+    first = b;
+    count = 1;
+    if (a.cu_seqlens != nullptr) {
+      first = a.cu_seqlens[b];
+      count = a.cu_seqlens[b + 1] - first;
+    }
+    rows = first < 0 ? 0 : min(count, a.total_tokens - first);   // no row outside the inputs, whatever cu_seqlens says
+    start = a.cache_lens[b];
+    fits = start >= 0 && start + count <= a.capacity;
+    if (!fits && count > 0 && tid == 0) set_status(a.status, PQ_ERR_CAPACITY);
   }
-  const int start = a.cache_lens[b];
-  const bool fits = start >= 0 && start + count <= a.capacity;
-  if (!fits && count > 0 && tid == 0) set_status(a.status, PQ_ERR_CAPACITY);
-  const int per_row = 2 * a.n_kv_heads, n_vec = count > 0 ? count * per_row : 0;
+  const int per_row = 2 * a.n_kv_heads, n_vec = rows > 0 ? rows * per_row : 0;
   const Layout L = make_layout(D, a.pg.page_tokens);
   int bad_page = 0;
   for (int v0 = rank * R::kVec; v0 < n_vec; v0 += C * R::kVec) {
@@ -101,11 +110,19 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
       atomicAdd(a.status + 1, bad);
       set_status(a.status, PQ_ERR_NONFINITE);
     }
+    // a thread per (vector, block) quantises; the blocks of a vector are neighbouring lanes
+    const int v = v0 + tid / R::kBlocks, blk = tid % R::kBlocks;
+    int seq = b, pos = start + v / per_row;
+    bool goes = fits;
+    if (kFlat && tid < R::kQuant && v < n_vec) {
+      row_destination(a, v / per_row, &seq, &pos);
+      goes = pos >= 0;
+    }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < R::kPer; ++j) {
-      const int v = vgrp + j * R::kGroups;
-      const float4* xv = reinterpret_cast<const float4*>(xs + v * D + slice * 16);
+      const int w = vgrp + j * R::kGroups;
+      const float4* xv = reinterpret_cast<const float4*>(xs + w * D + slice * 16);
       float acc = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -115,7 +132,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
         acc = fmaf(x4.z, s[4 * i + 2], acc);
         acc = fmaf(x4.w, s[4 * i + 3], acc);
       }
-      part[(slice * R::kVec + v) * D + col] = acc;
+      part[(slice * R::kVec + w) * D + col] = acc;
     }
     __syncthreads();
     for (int i = tid; i < R::kVec * D; i += kRowsThreads) {
@@ -125,8 +142,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
       ys[(i >> 4) * 20 + (i & 15)] = y;
     }
     __syncthreads();
-    // a thread per (vector, block); the blocks of a vector are neighbouring lanes
-    const int v = v0 + tid / R::kBlocks, blk = tid % R::kBlocks;
     FastBlock fb = {0u, 0u, 0u, 0u, 0u, 0.f};
     bool mine = false, unsure = false;
     uint8_t* tb = nullptr;
@@ -148,13 +163,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
       if (fq.analytic) polar_quant_block_fast<true>(yb, rm, fq, &fb);
       else polar_quant_block_fast<false>(yb, rm, fq, &fb);
       if (v < n_vec) {
-        const int r = v / per_row, w = v - r * per_row, kv = w / a.n_kv_heads, head = w - kv * a.n_kv_heads;
-        if (fits) {
-          const int64_t off = block_offset(L, a.pg, a.n_kv_heads, b, head, kv, start + r);
+        const int w = v % per_row, kv = w / a.n_kv_heads, head = w - kv * a.n_kv_heads;
+        if (goes) {
+          const int64_t off = block_offset(L, a.pg, a.n_kv_heads, seq, head, kv, pos);
           if (off < 0) bad_page = 1;   // a page outside the pool: nothing of the row is written
           else {
             tb = a.cache + off;
-            tok = (start + r) % kTokenBlock;
+            tok = pos % kTokenBlock;
             mine = true;
           }
         }
@@ -210,6 +225,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
     __syncthreads();
     if (tid == 0) n_list = 0;
   }
+  if (kFlat) return;   // row_destination has looked at the pages
   // ---- the sequence's length (every block of the cluster has read it and written its vectors)
   bad_page = __syncthreads_or(bad_page);
   if (bad_page && tid == 0) set_status(a.status, PQ_ERR_INVALID_ARG);
@@ -226,17 +242,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
   }
 }
 
-template <int D>
-static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, cudaStream_t stream) {
+template <int D, bool kFlat>
+static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, dim3 grid, cudaStream_t stream) {
   using R = RowsShape<D>;
   static DeviceMemo configured;
-  if (configure_for_device(encode_rows_kernel<D>, R::kSmem, configured) == 0) return PQ_ERR_CUDA;
-  // blocks per sequence: one pass each for an even split of the rows, eight at most (the portable cluster size)
-  const int64_t vec = ((int64_t)a.total_tokens * 2 * a.n_kv_heads + a.batch - 1) / a.batch;
-  int C = 1;
-  while (C < 8 && (int64_t)C * R::kVec < vec) C *= 2;
+  if (configure_for_device(encode_rows_kernel<D, kFlat>, R::kSmem, configured) == 0) return PQ_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(C, a.batch);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(kRowsThreads);
   cfg.dynamicSmemBytes = R::kSmem;
   cfg.stream = stream;
@@ -244,26 +256,41 @@ static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, cudaStr
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set up while the kernel before it finishes (it waits inside)
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = C;
+  attr[1].val.clusterDim.x = grid.x;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = C > 1 ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, encode_rows_kernel<D>, a, lens);
+  cfg.numAttrs = !kFlat && grid.x > 1 ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, encode_rows_kernel<D, kFlat>, a, lens);
   if (e != cudaSuccess) {
     note_cuda_error(e);
     cudaGetLastError();
     return PQ_ERR_CUDA;
   }
-  return PQ_OK;
+  return kFlat ? launch_advance_lens(a, lens, stream) : PQ_OK;
+}
+
+// A block or cluster per sequence where that is a single pass whatever the rows are: an append, or all rows in one sequence,
+// of at most eight blocks' vectors (the portable cluster size).  Otherwise -- the host does not know how the rows of an encode
+// are spread over its sequences -- the rows evenly over all blocks, and a second launch for the lengths.
+template <int D>
+static int32_t launch_encode_rows_of(const EncodeArgs& a, int32_t* lens, cudaStream_t stream) {
+  constexpr int kVec = RowsShape<D>::kVec;
+  const int64_t all = (int64_t)a.total_tokens * 2 * a.n_kv_heads, per_seq = a.cu_seqlens == nullptr ? 2 * (int64_t)a.n_kv_heads : all;
+  if ((a.cu_seqlens == nullptr || a.batch == 1) && per_seq <= 8 * kVec) {
+    int C = 1;
+    while (C * kVec < per_seq) C *= 2;
+    return launch_encode_rows_as<D, false>(a, lens, dim3(C, a.batch), stream);
+  }
+  return launch_encode_rows_as<D, true>(a, lens, dim3((unsigned)((all + kVec - 1) / kVec)), stream);
 }
 
 static int32_t launch_encode_rows(const EncodeArgs& a, int32_t* lens, cudaStream_t stream) {
   switch (a.head_dim) {
-    case 16: return launch_encode_rows_as<16>(a, lens, stream);
-    case 32: return launch_encode_rows_as<32>(a, lens, stream);
-    case 64: return launch_encode_rows_as<64>(a, lens, stream);
-    default: return launch_encode_rows_as<128>(a, lens, stream);
+    case 16: return launch_encode_rows_of<16>(a, lens, stream);
+    case 32: return launch_encode_rows_of<32>(a, lens, stream);
+    case 64: return launch_encode_rows_of<64>(a, lens, stream);
+    default: return launch_encode_rows_of<128>(a, lens, stream);
   }
 }
 

@@ -376,7 +376,7 @@ static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
     if (tc < 0) return tc;
     if (tc == 1) return launch_advance_lens(a, lens, stream);
   }
-  if (a.total_tokens < 32 && a.batch <= 65535) return launch_encode_rows(a, lens, stream);
+  if (a.total_tokens < 32) return launch_encode_rows(a, lens, stream);
   if (a.head_dim == 128) {
     static DeviceMemo configured;
     if (configure_for_device(encode_ffma_kernel, kFfmaSmem, configured) == 0) return PQ_ERR_CUDA;

@@ -9,7 +9,8 @@ import torch
 import paper_2502_02617_b200 as pq
 from paper_2502_02617_b200 import synthetic
 from oracle import polarquant_oracle as orc
-from parity_utils import TOL_ATTENTION_F32_IO, rel_l2, to_f64
+from parity_utils import (TOL_ATTENTION_F32_IO, assert_codes_match, assert_radii_match, code_mismatch_report, oracle_codebooks,
+                          radii_ulp_report, rel_l2, to_f64)
 from test_gpu_parity import _encode_and_compare, _oracle_cache
 
 pytestmark = pytest.mark.gpu
@@ -199,3 +200,42 @@ def test_persistent_kernel_reuses_its_ring_between_segments():
     out, want = to_f64(outs[0]), ref.attend(to_f64(q), 128 ** -0.5)
     for b in range(len(lens)):
         assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, lens[b]
+
+
+# Fewer than 32 tokens, spread unevenly over the sequences: all in one of them, most of them without any, more vectors than a
+# cluster's single pass.
+@pytest.mark.parametrize("d,Hkv", [(128, 3), (128, 32), (64, 8), (32, 5), (16, 8)])
+@pytest.mark.parametrize("lens", [[0] * 7 + [31] + [0] * 8, [3, 0, 0, 11, 1, 0, 14], [31], [0] * 299 + [2]])
+def test_few_tokens_spread_unevenly(d, Hkv, lens):
+    n = sum(lens)
+    cache = pq.PolarQuantCache(len(lens), Hkv, Hkv, d, capacity=64, seed=7, device=DEV)
+    K, V = synthetic.kv_like(50 + d, n, Hkv, d, torch.bfloat16, DEV, n_outliers=4 if d >= 64 else 0)
+    cache.encode(K, V, torch.tensor(np.concatenate(([0], np.cumsum(lens))), dtype=torch.int32, device=DEV))
+    assert cache.lens.tolist() == lens
+    cache.check_status()
+    codes, radii = (x.cpu().numpy() for x in cache.unpack(max(lens)))
+    cb, S, row, off = oracle_codebooks(cache), cache.S_host.double().numpy(), 0, [0, 0]
+    for b, m in enumerate(lens):
+        for kv, X in ((0, to_f64(K)), (1, to_f64(V))):
+            for h in range(Hkv if m else 0):
+                rep = code_mismatch_report(codes[b, h, kv, :m], X[row:row + m, h], S, cb)
+                assert_codes_match(rep)
+                off = [x + y for x, y in zip(off, radii_ulp_report(radii[b, h, kv, :m], rep["radii16"]))]
+        row += m
+    assert_radii_match(counts=off)
+
+
+# cu_seqlens that names more rows than K and V have: the missing rows are neither read (the inputs are the front of a larger
+# tensor here) nor written.
+@pytest.mark.parametrize("lens", [[5], [3, 4]])
+def test_rows_past_the_inputs_are_not_touched(lens):
+    n, Hkv, d = 3, 2, 64
+    cache = pq.PolarQuantCache(len(lens), Hkv, Hkv, d, capacity=64, seed=7, device=DEV)
+    cache.cache.fill_(0xA5)
+    K, V = synthetic.kv_like(51, 40, Hkv, d, torch.bfloat16, DEV)
+    K[n:], V[n:] = float("nan"), float("nan")
+    cache.encode(K[:n], V[:n], torch.tensor([0] + list(np.cumsum(lens)), dtype=torch.int32, device=DEV))
+    assert cache.status.tolist()[:2] == [pq.OK, 0]              # no non-finite input was seen
+    codes, radii = cache.unpack(max(lens))
+    untouched = torch.full((), 0xA5A5 - 0x10000, dtype=torch.int16).view(torch.float16).to(DEV)
+    assert torch.all(radii[0, :, :, n:] == untouched) and not torch.any(radii[0, :, :, :n] == untouched)
