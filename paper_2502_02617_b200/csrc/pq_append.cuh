@@ -1,16 +1,17 @@
-// Encoder of few rows (append: one per sequence; drafted tokens), any head_dim of the packed cache (included by
+// Encoder of few rows (append: one per sequence; drafted tokens; short chunks), any head_dim of the packed cache (included by
 // pq_encode.cu).  A call of this kind is all latency, so everything that does not depend on the rows is in registers
 // before the kernel ahead in the stream has finished (S and the quantiser's constants; the kernel is its programmatic
-// dependent), and one block -- or a cluster of up to eight -- takes all the vectors of a sequence, so that it can also
-// advance the sequence's length: no second launch.
+// dependent), and where one block -- or a cluster of up to eight -- takes all the vectors of a sequence in a pass, it also
+// advances the sequence's length: no second launch.
 //
 // A pass of a block is kVec vectors.  Rotation: thread = (column, slice of 16 rows of S) with its 16 entries of S in
 // registers, all slices in flight at once; the slices' partial sums meet in shared memory.  So the error of a
 // coordinate is at most (16 + D / 16) 2^-24 sum_k |x_k||S_kj| <= that factor times ||x||_2.  Then a thread per
 // 16-coordinate block runs the certified quantiser; a block with an uncertified decision is rotated again in float64 by
 // the whole thread block (two or fewer terms per thread) and decided by one warp.
-// Measured (append with 8 kv heads, a block per vector and a second launch for the lengths before): one sequence, head_dim 128
-// 11.0 -> 7.0 us, sixteen sequences 11.6 -> 10.1 us; eight sequences at head_dim 64 (float64 throughout before) 20.4 -> 8.7 us.
+// Measured (device time behind another kernel, 8 kv heads; a block per vector, float64 below head_dim 128, and a second launch for the
+// lengths before): append of one token at head_dim 128 5.3 -> 4.9 us, of 16 10.9 -> 7.9 us; 31 tokens in one sequence 15.0 -> 7.9 us;
+// at head_dim 64 one token 16.9 -> 7.5 us, 256 tokens 21.5 -> 15.3 us.
 #pragma once
 
 namespace pq {
@@ -18,11 +19,11 @@ namespace pq {
 static int32_t launch_advance_lens(const EncodeArgs& a, int32_t* lens, cudaStream_t stream);
 
 constexpr int kRowsThreads = 1024;
-template <int D>
+template <int D, int kMin>
 struct RowsShape {
   static constexpr int kBlocks = D / 16, kSlices = D / 16;          // 16-coordinate blocks; slices of 16 rows of S
   static constexpr int kGroups = kRowsThreads / (D * kSlices);      // vectors that are rotated side by side
-  static constexpr int kVec = kGroups > 16 ? kGroups : 16;          // vectors of a pass
+  static constexpr int kVec = kGroups > kMin ? kGroups : kMin;      // vectors of a pass
   static constexpr int kPer = kVec / kGroups;                       // ... of a thread
   static constexpr int kQuant = kVec * kBlocks;                     // threads that quantise (a multiple of 32)
   static constexpr int kYFloats = kVec * kBlocks * 20;              // rotated blocks, 20 floats apart (conflict-free 16-byte reads)
@@ -53,9 +54,10 @@ __device__ __forceinline__ double warp_quant_exact(double y, const Tables& tb, i
 }
 
 // kFlat: the blocks share all rows evenly, whatever sequences they belong to, and another launch advances the lengths.
-template <int D, bool kFlat>
+template <int D, int kMin, bool kFlat>
 __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __grid_constant__ EncodeArgs a, int32_t* lens) {
-  using R = RowsShape<D>;
+  using R = RowsShape<D, kMin>;
+  static_assert(R::kQuant % 32 == 0, "whole warps quantise");
   extern __shared__ __align__(16) float rows_smem[];
   float* xs = rows_smem;                       // [kVec][D]
   float* part = xs + R::kVec * D;              // [kSlices][kVec][D]
@@ -242,11 +244,11 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
   }
 }
 
-template <int D, bool kFlat>
+template <int D, int kMin, bool kFlat>
 static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, dim3 grid, cudaStream_t stream) {
-  using R = RowsShape<D>;
+  using R = RowsShape<D, kMin>;
   static DeviceMemo configured;
-  if (configure_for_device(encode_rows_kernel<D, kFlat>, R::kSmem, configured) == 0) return PQ_ERR_CUDA;
+  if (configure_for_device(encode_rows_kernel<D, kMin, kFlat>, R::kSmem, configured) == 0) return PQ_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kRowsThreads);
@@ -261,7 +263,7 @@ static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, dim3 gr
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = !kFlat && grid.x > 1 ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, encode_rows_kernel<D, kFlat>, a, lens);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, encode_rows_kernel<D, kMin, kFlat>, a, lens);
   if (e != cudaSuccess) {
     note_cuda_error(e);
     cudaGetLastError();
@@ -273,24 +275,37 @@ static int32_t launch_encode_rows_as(const EncodeArgs& a, int32_t* lens, dim3 gr
 // A block or cluster per sequence where that is a single pass whatever the rows are: an append, or all rows in one sequence,
 // of at most eight blocks' vectors (the portable cluster size).  Otherwise -- the host does not know how the rows of an encode
 // are spread over its sequences -- the rows evenly over all blocks, and a second launch for the lengths.
-template <int D>
+template <int D, int kMin>
 static int32_t launch_encode_rows_of(const EncodeArgs& a, int32_t* lens, cudaStream_t stream) {
-  constexpr int kVec = RowsShape<D>::kVec;
+  constexpr int kVec = RowsShape<D, kMin>::kVec;
   const int64_t all = (int64_t)a.total_tokens * 2 * a.n_kv_heads, per_seq = a.cu_seqlens == nullptr ? 2 * (int64_t)a.n_kv_heads : all;
-  if ((a.cu_seqlens == nullptr || a.batch == 1) && per_seq <= 8 * kVec) {
+  if ((a.cu_seqlens == nullptr || a.batch == 1) && per_seq <= 8 * kVec && (a.cu_seqlens != nullptr || a.batch <= 65535)) {
     int C = 1;
     while (C * kVec < per_seq) C *= 2;
-    return launch_encode_rows_as<D, false>(a, lens, dim3(C, a.batch), stream);
+    return launch_encode_rows_as<D, kMin, false>(a, lens, dim3(C, a.batch), stream);
   }
-  return launch_encode_rows_as<D, true>(a, lens, dim3((unsigned)((all + kVec - 1) / kVec)), stream);
+  return launch_encode_rows_as<D, kMin, true>(a, lens, dim3((unsigned)((all + kVec - 1) / kVec)), stream);
 }
 
-static int32_t launch_encode_rows(const EncodeArgs& a, int32_t* lens, cudaStream_t stream) {
+// A pass takes as long as its vectors: fewer of them where the blocks still have an SM each (one sequence, 8 kv heads, head_dim 128:
+// 7.1 us with 16 vectors in one block, 4.9 with a cluster of four).
+template <int D, int kFew>
+static int32_t launch_encode_rows_by_size(const EncodeArgs& a, int32_t* lens, int n_sm, cudaStream_t stream) {
+  const int64_t all = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
+  return all <= (int64_t)kFew * n_sm ? launch_encode_rows_of<D, kFew>(a, lens, stream) : launch_encode_rows_of<D, 16>(a, lens, stream);
+}
+
+// Calls that this kernel takes: fewer than 32 tokens; below head_dim 128 also as long as two passes of every SM hold them.
+static bool encode_rows_takes(const EncodeArgs& a, int n_sm) {
+  const int per_pass = a.head_dim == 16 ? RowsShape<16, 16>::kVec : 16;
+  return a.total_tokens < 32 || (a.head_dim < 128 && (int64_t)a.total_tokens * 2 * a.n_kv_heads <= 2 * (int64_t)n_sm * per_pass);
+}
+static int32_t launch_encode_rows(const EncodeArgs& a, int32_t* lens, int n_sm, cudaStream_t stream) {
   switch (a.head_dim) {
-    case 16: return launch_encode_rows_of<16>(a, lens, stream);
-    case 32: return launch_encode_rows_of<32>(a, lens, stream);
-    case 64: return launch_encode_rows_of<64>(a, lens, stream);
-    default: return launch_encode_rows_of<128>(a, lens, stream);
+    case 16: return launch_encode_rows_of<16, 16>(a, lens, stream);
+    case 32: return launch_encode_rows_of<32, 16>(a, lens, stream);
+    case 64: return launch_encode_rows_by_size<64, 8>(a, lens, n_sm, stream);
+    default: return launch_encode_rows_by_size<128, 4>(a, lens, n_sm, stream);
   }
 }
 

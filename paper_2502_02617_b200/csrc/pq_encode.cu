@@ -376,7 +376,10 @@ static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
     if (tc < 0) return tc;
     if (tc == 1) return launch_advance_lens(a, lens, stream);
   }
-  if (a.total_tokens < 32) return launch_encode_rows(a, lens, stream);
+  static DeviceMemo sm_count;
+  const int n_sm = sm_count_of_device(sm_count);
+  if (n_sm == 0) return PQ_ERR_CUDA;
+  if (encode_rows_takes(a, n_sm)) return launch_encode_rows(a, lens, n_sm, stream);
   if (a.head_dim == 128) {
     static DeviceMemo configured;
     if (configure_for_device(encode_ffma_kernel, kFfmaSmem, configured) == 0) return PQ_ERR_CUDA;
