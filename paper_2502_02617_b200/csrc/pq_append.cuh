@@ -161,9 +161,11 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
       float n2 = (sq[0] + sq[1]) + (sq[2] + sq[3]);
 #pragma unroll
       for (int m = 1; m < R::kBlocks; m <<= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, m);
-      const RowMargins rm = make_row_margins(1.0001f * sqrtf(n2), 1.1f * (16 + R::kSlices) * 5.9604644775390625e-08f, fq);
+      const float norm = 1.0001f * sqrtf(n2);
+      const RowMargins rm = make_row_margins(norm, 1.1f * (16 + R::kSlices) * 5.9604644775390625e-08f, fq);
       if (fq.analytic) polar_quant_block_fast<true>(yb, rm, fq, &fb);
       else polar_quant_block_fast<false>(yb, rm, fq, &fb);
+      const float block_err = rotation_block_error(16, R::kSlices) * norm;
       if (v < n_vec) {
         const int w = v % per_row, kv = w / a.n_kv_heads, head = w - kv * a.n_kv_heads;
         if (goes) {
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
           }
         }
         // head dims below 128: radii as rounded once from float64; at 128 as the tensor-core encoder forms them
-        unsure = fb.amb != 0u || (D < 128 && radius_unsure(fb.radius));
+        unsure = fb.amb != 0u || (D < 128 && radius_unsure(fb.radius, block_err));
         if (mine && unsure) list[atomicAdd(&n_list, 1)] = (uint16_t)tid;
       }
     }

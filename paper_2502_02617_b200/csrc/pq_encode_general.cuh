@@ -16,7 +16,8 @@
 // Margins: moving every coordinate by at most dy moves the norm of n of them by at most sqrt(n) dy, so a test on the
 // radii of n-coordinate halves moves by at most sqrt(2 n) dy; 1.1 x that, plus 1e-6 (r_a + r_b) for the float32
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
-// A radius is certified by radius_unsure.
+// A radius is certified by radius_unsure, with the bound of rotation_block_error: 1.4 to 5 % of them are not, according to the slices
+// of S and the blocks of a vector.
 // Bound by the product on the FMA pipe (18 of a block's 47 us) and by the latency of the float64 re-decisions (13).  Measured (8 heads;
 // a block per vector in float64 before): 512 tokens, seven levels of three bits 89.7 -> 43.4 us; packed cache, 2048 tokens at
 // head_dim 64 67 -> 40 us.
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   float* Ss = xy + s.floats_xy;                                         // [kGeSlice][dc]
   uint32_t* rows = reinterpret_cast<uint32_t*>(Ss + kGeSlice * dc);     // [V][row_words]
   float* gsum = reinterpret_cast<float*>(rows + V * s.row_words);       // [V][ng] squared norms of the groups
-  float* dy_sm = gsum + V * ng;                                         // [V] bound on the error of a coordinate
+  float* dy_sm = gsum + V * ng;                                         // [V] bound on the error of a coordinate, [V] on that of a block
   float2* tab = reinterpret_cast<float2*>(dy_sm + 2 * V);               // boundaries
   const int n_bnd = g.n_cen - L;
   int64_t* dest = reinterpret_cast<int64_t*>(tab + ((n_bnd + 1) & ~1)); // [V] where the row goes (-1: nowhere)
@@ -305,6 +306,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     float t = 0.f;
     for (int i = 0; i < ng; ++i) t += gsum[v * ng + i];
     dy_sm[v] = rot_err * 1.0001f * sqrtf(t);
+    dy_sm[V + v] = rotation_block_error(kGeSlice, (dc + kGeSlice - 1) / kGeSlice) * 1.0001f * sqrtf(t);
   }
   __syncthreads();
 
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     if (L == kSub) {
 #pragma unroll
       for (int j = 0; j < n_blk; ++j) {
-        if (grp * n_blk + j < g.nb) sure = sure && !radius_unsure(r[j]);
+        if (grp * n_blk + j < g.nb) sure = sure && !radius_unsure(r[j], dy_sm[V + v]);
         rad[j] = __half_as_ushort(__float2half_rn(r[j]));
       }
     }
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
       }
       for (int j = 0; j < g.nb; ++j) {
         const float r = ge_sqrt(q2[j]);
-        sure = sure && !radius_unsure(r);
+        sure = sure && !radius_unsure(r, dy_sm[V + v]);
         ge_put(row, g.rad_off * 8 + 16 * j, __half_as_ushort(__float2half_rn(r)));
       }
       if (!sure) {

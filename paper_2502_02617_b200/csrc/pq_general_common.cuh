@@ -41,14 +41,23 @@ struct GenEncodeArgs {
 // Encode into the packed cache at head dims below 128 (levels and bits of Section 4.1); a.g and a.packed are filled in.
 int32_t launch_packed_encode(GenEncodeArgs a, int head_dim, cudaStream_t stream);
 
-// Would the block radius r round to another fp16 value if it moved by kRadiusSlack?  (NaN and infinite r: yes; near
-// saturation: yes, it is counted from the exact value.)  The float32 error of r is that of a norm, whose coordinate errors
-// average out (2e-8 of the norm on synthetic rows), plus the sum of squares and the square root, at most 5e-7 together.
-constexpr float kRadiusSlack = 2e-6f;
-__device__ __forceinline__ bool radius_unsure(float r) {
-  const float lo = fminf(r * (1.f - kRadiusSlack), 65504.f), hi = fminf(r * (1.f + kRadiusSlack), 65504.f);
-  return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(lo)) != __half_as_ushort(__float2half_rn(hi)) ||
-         r > 65000.f;
+// Would the block radius r round to another fp16 value if it moved by its error?  (NaN and infinite r: yes; near saturation: yes, it
+// is counted from the exact value.)  `err` bounds the 2-norm of the error of the block's rotated coordinates, and so the error that
+// their rotation brings into r; the sums of squares and the square root add less than 8 roundings of 2^-24, below 1e-6 r.
+__device__ __forceinline__ bool radius_unsure(float r, float err) {
+  const float slack = fmaf(1e-6f, r, err), lo = fminf(r - slack, 65504.f), hi = fminf(r + slack, 65504.f);
+  return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(fmaxf(lo, 0.f))) != __half_as_ushort(__float2half_rn(hi)) || !(r <= 65000.f);
+}
+// That bound for y = x S summed in `slices` chains of `chain` fused multiply-adds whose results are added one by one, relative to
+// ||x||_2: the rounding of step m of a chain moves the coordinates of any block by at most 2^-24 times the norm of the partial sums,
+// which is at most that of the slice of x (the rows and columns of an orthogonal S that meet there have spectral norm 1 or less);
+// the slices' norms add up to sqrt(slices) ||x|| at most, and each of the additions moves the block by 2^-24 ||x||.  2 % for the
+// rounding of S and second order.
+__host__ __device__ constexpr float const_sqrt(int n) {   // of 1, 2, 4, 8 exactly enough, rounded up
+  return n <= 1 ? 1.f : n <= 2 ? 1.4143f : n <= 4 ? 2.f : 2.8285f;
+}
+__host__ __device__ constexpr float rotation_block_error(int chain, int slices) {
+  return 1.02f * (chain * const_sqrt(slices) + slices) * 5.9604644775390625e-08f;
 }
 
 // (cos x, sin x) for 0 <= x <= 2 pi, rounded once to float32 from a float64 evaluation: x is reduced by a multiple of

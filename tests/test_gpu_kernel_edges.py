@@ -239,3 +239,43 @@ def test_rows_past_the_inputs_are_not_touched(lens):
     codes, radii = cache.unpack(max(lens))
     untouched = torch.full((), 0xA5A5 - 0x10000, dtype=torch.int16).view(torch.float16).to(DEV)
     assert torch.all(radii[0, :, :, n:] == untouched) and not torch.any(radii[0, :, :, :n] == untouched)
+
+
+def _codes_and_radii(cache, K, V, pieces):
+    """Encodes the pieces one after the other; (codes, radii) of the cache and of the oracle, [vectors, ...]."""
+    at = 0
+    for m in pieces:
+        cache.encode(K[at:at + m], V[at:at + m], torch.tensor([0, m], dtype=torch.int32, device=DEV))
+        at += m
+    bits = (4, 2, 2, 2) if not hasattr(cache, "bits") else tuple(cache.bits)
+    cb = orc.codebooks_from_arrays(bits, cache.centroids.numpy(), cache.boundaries.numpy())
+    codes, radii = (x.cpu().numpy()[0].transpose(1, 2, 0, 3).reshape(2 * at * cache.n_kv_heads, -1) for x in cache.unpack(at))
+    X = np.stack([to_f64(K[:at]), to_f64(V[:at])]).reshape(2 * at * cache.n_kv_heads, -1)
+    rep = code_mismatch_report(codes, X, cache.S_host.double().numpy(), cb)
+    return rep, radii, rep["radii16"]
+
+
+def _cache_of(d, bits, Hkv, n):
+    if bits is None:
+        return pq.PolarQuantCache(1, Hkv, Hkv, d, capacity=n, seed=6, device=DEV)
+    cache = pq.GeneralPolarQuantCache(1, Hkv, Hkv, d, bits, n, seed=6, device=DEV)
+    cache.bits = bits
+    return cache
+
+
+# Vectors whose norm lies in one rotated block: the float32 rotation's error follows the norm of the vector, not that of a block, and
+# the radii of the small blocks are the one rounding of the exact norm all the same.
+@pytest.mark.parametrize("d,bits", [(64, None), (32, None), (128, (4, 2, 2, 2)), (64, (4, 3, 2)), (256, (3,) * 5)])
+def test_radii_of_vectors_concentrated_in_a_block(d, bits):
+    Hkv, pieces = 2, [20, 700]
+    n = sum(pieces)
+    cache = _cache_of(d, bits, Hkv, n)
+    gen = torch.Generator(device=DEV).manual_seed(d)
+    Y = torch.randn((2, n, Hkv, d // 16, 16), generator=gen, device=DEV, dtype=torch.float64)
+    small = 10.0 ** (-1.5 - 2.5 * torch.rand((2, n, Hkv, d // 16, 1), generator=gen, device=DEV, dtype=torch.float64))
+    big = torch.randint(0, d // 16, (2, n, Hkv, 1, 1), generator=gen, device=DEV)
+    Y *= small.scatter(3, big, 1.0)
+    K, V = (Y.view(2, n, Hkv, d) @ cache.S_host.double().to(DEV).T).float()
+    rep, radii, want = _codes_and_radii(cache, K, V, pieces)
+    assert_codes_match(rep)
+    assert np.array_equal(radii.view(np.uint16), want.astype(np.float16).view(np.uint16))
