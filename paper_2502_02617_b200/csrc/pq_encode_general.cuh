@@ -12,7 +12,7 @@
 //     ends in, so the smallest |r_b cos - r_a sin| it met bounds the distance to the next boundary.
 //   * levels 5 and up: a thread per vector on the groups' norms.
 //   * a (vector, group) with any decision inside its margin, or a block radius that close to a rounding boundary of
-//     fp16, is taken again by a warp in float64 from the inputs; the same for the upper levels of a vector.
+//     fp16, is taken again by a warp in float64 from the inputs; the same for the upper levels of a (vector, block).
 // Margins: moving every coordinate by at most dy moves the norm of n of them by at most sqrt(n) dy, so a test on the
 // radii of n-coordinate halves moves by at most sqrt(2 n) dy; 1.1 x that, plus 1e-6 (r_a + r_b) for the float32
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
@@ -49,7 +49,7 @@ __host__ __device__ inline GeShape ge_shape(int d, int row_bytes, int vt) {
 }
 __host__ inline int ge_smem_bytes(const GeShape& s, int n_bnd) {
   return 4 * (s.floats_xy + kGeSlice * s.dc + s.vecs * s.row_words + s.vecs * s.ng + 2 * s.vecs + 2 * ((n_bnd + 1) & ~1)) +
-         8 * s.vecs + 8 * s.vecs * s.ng + 4 * s.vecs * s.ng + 2 * s.vecs + 64;
+         8 * s.vecs + 8 * s.vecs * s.ng + 6 * s.vecs * s.ng + 64;
 }
 
 __device__ __forceinline__ float ge_load(const void* base, int dtype, int64_t i) {
@@ -62,6 +62,14 @@ __device__ __forceinline__ void ge_put(uint32_t* row, int bit, uint32_t value) {
   atomicOr(row + (bit >> 5), value << sh);
   const uint32_t hi = sh ? value >> (32 - sh) : 0u;
   if (hi) atomicOr(row + (bit >> 5) + 1, hi);
+}
+// Put `value` in the place of the `width` (at most 16) bits from bit `bit` on.
+__device__ __forceinline__ void ge_replace(uint32_t* row, int bit, int width, uint32_t value) {
+  const int sh = bit & 31;
+  const uint32_t mask = (1u << width) - 1u;
+  atomicAnd(row + (bit >> 5), ~(mask << sh));
+  if (sh + width > 32) atomicAnd(row + (bit >> 5) + 1, ~(mask >> (32 - sh)));
+  ge_put(row, bit, value);
 }
 __device__ __forceinline__ float ge_sqrt(float x) {
   float r;
@@ -106,7 +114,7 @@ __device__ __forceinline__ double ge_exact_coord(const GenEncodeArgs& a, const v
   if (col < d) {
     const float* s = a.S + (int64_t)k0 * d + col;
     const int n4 = half & ~3;
-#pragma unroll 2
+#pragma unroll 8   // the loads of 32 terms in flight together: an item is a chain of round trips to L2
     for (int k = 0; k < n4; k += 4)
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -136,7 +144,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   double* norm_up = reinterpret_cast<double*>(dest + V);                // [V * ng] exact norms of groups, where needed
   uint16_t* list = reinterpret_cast<uint16_t*>(norm_up + V * ng);       // [V * ng] (vector, group) pairs to take again
   uint16_t* norms = list + V * ng;                                      // [V * ng] (vector, group) pairs of which the norm is needed
-  uint16_t* list_up = norms + V * ng;                                   // [V] vectors whose upper levels are taken again
+  uint16_t* list_up = norms + V * ng;                                   // [V * ng] (vector, block) pairs whose upper levels are taken again
   __shared__ int n_list, n_norms, n_list_up, n_upper;
   const int head = blockIdx.y, kv = blockIdx.z, row0 = blockIdx.x * V;
   const void* xbase = kv ? a.V : a.K;
@@ -374,13 +382,14 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     }
   }
   // ---- levels above the groups: a thread per vector, the squared norms halved in place
+  const int gpb = L > 4 ? 1 << (L - 4) : 1;   // groups of a block
   if (L > 4) {
     __syncthreads();
     for (int v = tid; v < V; v += kGeThreads) {
       if (dest[v] < 0) continue;
       float* q2 = gsum + v * ng;
       uint32_t* row = rows + v * s.row_words;
-      bool sure = true;
+      uint32_t unsure = 0u;   // blocks with a decision or a radius that is not certified
       const float dy = dy_sm[v];
       for (int l = 4; l < L; ++l) {
         const int n = d >> (l + 1), b = g.bits[l];
@@ -391,7 +400,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
           const float sa = q2[2 * j], sb = q2[2 * j + 1], p = ge_sqrt(sa), q = ge_sqrt(sb);
           float near;
           const uint32_t code = ge_search<false>(p, q, tab + g.bnd_off[l], b, 0, near);
-          sure = sure && near > fmaf(1e-6f, p + q, m_dy);
+          if (!(near > fmaf(1e-6f, p + q, m_dy))) unsure |= 1u << (j >> (L - 1 - l));
           word |= code << fill;
           fill += b;
           if (fill > 24 || j + 1 == n) {
@@ -405,13 +414,14 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
       }
       for (int j = 0; j < g.nb; ++j) {
         const float r = ge_sqrt(q2[j]);
-        sure = sure && !radius_unsure(r, dy_sm[V + v]);
+        if (radius_unsure(r, dy_sm[V + v])) unsure |= 1u << j;
         ge_put(row, g.rad_off * 8 + 16 * j, __half_as_ushort(__float2half_rn(r)));
       }
-      if (!sure) {
-        list_up[atomicAdd(&n_list_up, 1)] = (uint16_t)v;
-        const int at = atomicAdd(&n_norms, ng);
-        for (int i = 0; i < ng; ++i) norms[at + i] = (uint16_t)(v * ng + i);
+      for (; unsure; unsure &= unsure - 1) {
+        const int j = __ffs(unsure) - 1;
+        list_up[atomicAdd(&n_list_up, 1)] = (uint16_t)(v * g.nb + j);
+        const int at = atomicAdd(&n_norms, gpb);
+        for (int i = 0; i < gpb; ++i) norms[at + i] = (uint16_t)(v * ng + j * gpb + i);
       }
     }
   }
@@ -456,27 +466,24 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     }
     __syncthreads();
     for (int e = warp; e < n_list_up; e += kGeThreads / 32) {
-      const int v = list_up[e];
+      const int v = list_up[e] / g.nb, blk = list_up[e] - v * g.nb;
       uint32_t* row = rows + v * s.row_words;
-      double mine = lane < ng ? norm_up[v * ng + lane] : 0.0;
-      for (int t = g.byte_off[4] + lane; t < g.row_bytes; t += 32)   // take the float32 codes and radii out
-        atomicAnd(row + (t >> 2), ~(0xFFu << (8 * (t & 3))));
-      __syncwarp();
+      double mine = lane < gpb ? norm_up[v * ng + blk * gpb + lane] : 0.0;
       for (int l = 4; l < L; ++l) {
-        const int n = d >> (l + 1);
+        const int n = gpb >> (l - 3);   // the block's angles at this level
         const double p = __shfl_sync(0xffffffffu, mine, (2 * lane) & 31), q = __shfl_sync(0xffffffffu, mine, (2 * lane + 1) & 31);
-        if (lane < n) ge_put(row, g.byte_off[l] * 8 + lane * g.bits[l], ge_exact_code(p, q, g, l, a.boundaries));
+        if (lane < n) ge_replace(row, g.byte_off[l] * 8 + (blk * n + lane) * g.bits[l], g.bits[l], ge_exact_code(p, q, g, l, a.boundaries));
         mine = sqrt(p * p + q * q);
       }
-      if (lane < g.nb) {
+      if (lane == 0) {
         double r = mine;
         if (r > 65504.0) {
           r = 65504.0;
           atomicAdd(a.status + 2, 1);
         }
-        ge_put(row, g.rad_off * 8 + 16 * lane, __half_as_ushort(__double2half(r)));
+        ge_replace(row, g.rad_off * 8 + 16 * blk, 16, __half_as_ushort(__double2half(r)));
+        atomicAdd(a.status + 3, 1);
       }
-      if (lane == 0) atomicAdd(a.status + 3, 1);
     }
   }
   __syncthreads();
