@@ -125,6 +125,34 @@ __device__ __forceinline__ double ge_exact_coord(const GenEncodeArgs& a, const v
   return sum + __shfl_xor_sync(0xffffffffu, sum, 16);
 }
 
+// Where packed row `row` goes, head `head`, K (kv = 0) or V: the byte offset of its general row in the cache; in the packed cache
+// token-block and token in one number; -1 if it is not written.
+__device__ __forceinline__ int64_t ge_destination(const GenEncodeArgs& a, int row, int head, int kv) {
+  int b = row, first = row, count = 1;
+  if (a.cu_seqlens != nullptr) {   // the sequence that owns the row: largest b with cu[b] <= row
+    int lo = 0, hi = a.batch - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (a.cu_seqlens[mid] <= row) lo = mid; else hi = mid - 1;
+    }
+    b = lo; first = a.cu_seqlens[lo]; count = a.cu_seqlens[lo + 1] - first;
+  }
+  const int start = a.lens[b];
+  if (start < 0 || start + count > a.capacity) {
+    set_status(a.status, PQ_ERR_CAPACITY);
+    return -1;
+  }
+  const int pos = start + (row - first);
+  if (!a.packed) return ((((int64_t)b * a.n_kv_heads + head) * 2 + kv) * a.capacity + pos) * a.g.row_bytes;
+  const Layout P = make_layout(a.g.d, a.pg.page_tokens);
+  const int64_t off = block_offset(P, a.pg, a.n_kv_heads, b, head, kv, pos);
+  if (off < 0) {
+    set_status(a.status, PQ_ERR_INVALID_ARG);   // a page outside the pool
+    return -1;
+  }
+  return off * kTokenBlock + pos % kTokenBlock;
+}
+
 // kVT: vectors per thread in the product (4; 1 for few rows).  kSub: levels inside a group, min(L, 4).
 template <int kVT, int kSub>
 __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_constant__ GenEncodeArgs a) {
@@ -163,33 +191,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   // ---- destinations and inputs
   for (int v = tid; v < V; v += kGeThreads) {
     const int row = row0 + v;
-    int64_t off = -1;
-    if (row < a.total_tokens) {
-      int b = row, first = row, count = 1;
-      if (a.cu_seqlens != nullptr) {   // the sequence that owns the row: largest b with cu[b] <= row
-        int lo = 0, hi = a.batch - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (a.cu_seqlens[mid] <= row) lo = mid; else hi = mid - 1;
-        }
-        b = lo; first = a.cu_seqlens[lo]; count = a.cu_seqlens[lo + 1] - first;
-      }
-      const int start = a.lens[b];
-      if (start < 0 || start + count > a.capacity) {
-        set_status(a.status, PQ_ERR_CAPACITY);
-      } else {
-        const int pos = start + (row - first);
-        if (a.packed) {
-          const Layout P = make_layout(d, a.pg.page_tokens);
-          off = block_offset(P, a.pg, a.n_kv_heads, b, head, kv, pos);
-          if (off < 0) set_status(a.status, PQ_ERR_INVALID_ARG);   // a page outside the pool
-          else off = off * kTokenBlock + pos % kTokenBlock;        // token-block and token in one number
-        } else {
-          off = ((((int64_t)b * a.n_kv_heads + head) * 2 + kv) * a.capacity + pos) * g.row_bytes;
-        }
-      }
-    }
-    dest[v] = off;
+    dest[v] = row < a.total_tokens ? ge_destination(a, row, head, kv) : -1;
   }
   const bool vec8 = a.in_dtype == PQ_DTYPE_BF16 && d >= 16 && ((a.token_stride | a.head_stride) & 7) == 0 &&
                     ((uintptr_t)xbase & 15) == 0;
@@ -520,18 +522,80 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   }
 }
 
-template <int kVT, int kSub>
-static int32_t launch_gen_encode_as(const GenEncodeArgs& a, cudaStream_t stream) {
-  const GeShape s = ge_shape(a.g.d, a.g.row_bytes, kVT);
-  static DeviceMemo configured;
-  auto kernel = gen_encode_kernel<kVT, kSub>;
-  if (configure_for_device(kernel, 113 * 1024, configured) == 0) return PQ_ERR_CUDA;
+// Few vectors, general rows: one thread block of max(d, 32) threads per vector (row, K | V, head), float64 throughout: y = x S, then
+// the polar tree level by level (thread j forms angle j of the level, code = number of boundaries below it), then the bit streams.
+// A chain of d float64 multiply-adds and log2 d levels, hardly longer for a thousand vectors than for one: see launch_gen_encode.
+__global__ void gen_encode_vector_kernel(const __grid_constant__ GenEncodeArgs a) {
+  __shared__ double ra[kGenMaxDim], rb[kGenMaxDim];
+  __shared__ uint8_t codes[kGenMaxDim];
+  __shared__ int64_t dest;
+  const GenConfig& g = a.g;
+  const int j = threadIdx.x, d = g.d;
+  const int64_t v = blockIdx.x;
+  const int head = (int)(v % a.n_kv_heads), kv = (int)((v / a.n_kv_heads) & 1);
+  const int row = (int)(v / (2 * a.n_kv_heads));
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the inputs may come from the kernel before this one
+  if (j == 0) dest = ge_destination(a, row, head, kv);
+  if (j < d) {
+    const float x = ge_load(kv ? a.V : a.K, a.in_dtype, (int64_t)row * a.token_stride + (int64_t)head * a.head_stride + j);
+    if (!(fabsf(x) < CUDART_INF_F)) {
+      atomicAdd(a.status + 1, 1);
+      set_status(a.status, PQ_ERR_NONFINITE);
+    }
+    ra[j] = (double)x;
+  }
+  __syncthreads();
+  if (j < d) {
+    double acc = 0.0;
+    for (int k = 0; k < d; ++k) acc = fma(ra[k], (double)__ldg(a.S + (int64_t)k * d + j), acc);
+    rb[j] = acc;
+  }
+  __syncthreads();
+  double* src = rb;
+  double* dst = ra;
+  for (int l = 0; l < g.L; ++l) {
+    if (j < (d >> (l + 1))) {
+      const double p = src[2 * j], q = src[2 * j + 1];
+      codes[g.code_off[l] + j] = (uint8_t)ge_exact_code(p, q, g, l, a.boundaries);
+      dst[j] = sqrt(p * p + q * q);
+    }
+    __syncthreads();
+    double* t = src; src = dst; dst = t;
+  }
+  if (dest < 0) return;
+  uint8_t* out = a.cache + dest;
+  for (int t = j; t < g.rad_off; t += blockDim.x) {   // byte t of the row: gather its bits
+    int l = g.L - 1;
+    while (l > 0 && t < g.byte_off[l]) --l;
+    uint32_t byte = 0;
+    if (t < g.byte_off[l] + g.level_bytes[l]) {
+      const int b = g.bits[l], n = d >> (l + 1);
+      for (int bit = 0; bit < 8; ++bit) {
+        const int at = (t - g.byte_off[l]) * 8 + bit, idx = at / b;
+        if (idx < n) byte |= (((uint32_t)codes[g.code_off[l] + idx] >> (at % b)) & 1u) << bit;
+      }
+    }
+    out[t] = (uint8_t)byte;
+  }
+  if (j < g.nb) {
+    double r = src[j];
+    if (r > 65504.0) {
+      r = 65504.0;
+      atomicAdd(a.status + 2, 1);
+    }
+    reinterpret_cast<__half*>(out + g.rad_off)[j] = __double2half(r);
+  }
+}
+
+// A kernel as a programmatic dependent launch: set up while the kernel before it in the stream finishes (it waits inside).
+static int32_t launch_gen_kernel(void (*kernel)(GenEncodeArgs), dim3 grid, int threads, int smem, const GenEncodeArgs& a, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((a.total_tokens + s.vecs - 1) / s.vecs, a.n_kv_heads, 2);
-  cfg.blockDim = dim3(kGeThreads);
-  cfg.dynamicSmemBytes = ge_smem_bytes(s, a.g.n_cen - a.g.L);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];   // set up while the kernel before it in the stream finishes (it waits inside)
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
@@ -545,9 +609,24 @@ static int32_t launch_gen_encode_as(const GenEncodeArgs& a, cudaStream_t stream)
   return PQ_OK;
 }
 
-// One vector per thread in the product instead of four as long as that many blocks fit on the device at once: a short
-// chunk then spreads over four times as many SMs.
+template <int kVT, int kSub>
+static int32_t launch_gen_encode_as(const GenEncodeArgs& a, cudaStream_t stream) {
+  const GeShape s = ge_shape(a.g.d, a.g.row_bytes, kVT);
+  static DeviceMemo configured;
+  if (configure_for_device(gen_encode_kernel<kVT, kSub>, 113 * 1024, configured) == 0) return PQ_ERR_CUDA;
+  return launch_gen_kernel(gen_encode_kernel<kVT, kSub>, dim3((a.total_tokens + s.vecs - 1) / s.vecs, a.n_kv_heads, 2), kGeThreads,
+                           ge_smem_bytes(s, a.g.n_cen - a.g.L), a, stream);
+}
+
+// A block per vector until the tiled kernel, which starts at 14 to 60 us, is faster.  Measured (vector against tiled kernel): head_dim
+// 256, bits 4,2,2,2,2 128 vectors 18.6 / 53 us, 2048 72 / 78, 4096 135 / 88; 128, seven levels of three bits 128 vectors 16.2 / 35 us,
+// 2048 30 / 40, 4096 50 / 46; 64, bits 4,3,2 4096 vectors 23 / 25 us, 8192 41 / 29; 16 4096 10 / 14 us, 8192 16 / 14.
+// In the tiled kernel one vector per thread in the product instead of four as long as that many blocks fit on the device at
+// once: a short chunk then spreads over four times as many SMs.
 static int32_t launch_gen_encode(const GenEncodeArgs& a, cudaStream_t stream) {
+  const int64_t n_vec = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
+  if (!a.packed && n_vec <= (a.g.d > 128 ? 2048 : a.g.d > 64 ? 3072 : 4096))
+    return launch_gen_kernel(gen_encode_vector_kernel, dim3((unsigned)n_vec), a.g.d < 32 ? 32 : a.g.d, 0, a, stream);
   const GeShape s1 = ge_shape(a.g.d, a.g.row_bytes, 1);
   const bool few = (int64_t)((a.total_tokens + s1.vecs - 1) / s1.vecs) * 2 * a.n_kv_heads <= 2 * 148;
   switch (a.g.L < 4 ? a.g.L : 4) {

@@ -138,7 +138,8 @@ def test_encoders_give_the_same_codes_in_any_pieces(d, dtype):
 
 @pytest.mark.parametrize("d,bits", [(128, (3,) * 7), (64, (4, 2)), (16, (2,) * 4)])
 def test_general_encoder_writes_the_same_bytes_in_any_pieces(d, bits):
-    Hkv, pieces = 3, [1, 20, 21, 22, 43, 64, 2]                 # rows = tokens x heads: around the tiles of 64
+    # up to 3072 or 4096 vectors a block each, in float64; above them tiles of 16 to 256 vectors
+    Hkv, pieces = 3, [1, 20, 21, 22, 43, 64, 2, 700, 701]
     n = sum(pieces)
     K, V = synthetic.kv_like(95 + d, n, Hkv, d, torch.float32, DEV, n_outliers=4 if d >= 64 else 0)
     whole, cut = (pq.GeneralPolarQuantCache(1, Hkv, Hkv, d, bits, n, seed=6, device=DEV) for _ in range(2))
@@ -267,7 +268,7 @@ def _cache_of(d, bits, Hkv, n):
 # the radii of the small blocks are the one rounding of the exact norm all the same.
 @pytest.mark.parametrize("d,bits", [(64, None), (32, None), (128, (4, 2, 2, 2)), (64, (4, 3, 2)), (256, (3,) * 5)])
 def test_radii_of_vectors_concentrated_in_a_block(d, bits):
-    Hkv, pieces = 2, [20, 700]
+    Hkv, pieces = 2, [20, 1400]                                 # few vectors and tiles have kernels of their own
     n = sum(pieces)
     cache = _cache_of(d, bits, Hkv, n)
     gen = torch.Generator(device=DEV).manual_seed(d)
