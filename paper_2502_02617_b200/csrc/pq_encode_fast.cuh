@@ -47,7 +47,7 @@ struct RowMargins {
   float c[3];     // 8.4 E^2 for levels 2, 3, 4 (E^2 = 2, 4, 8 dy^2)
   float cs[3];    // the same plus the float32-rounding term of the folded (symmetric) test
   float csg[3];   // the same for the scaled-line test of any codebook (quant_upper_lines_push)
-  float base[3];  // 42 E^4 * 4: every tested line has coefficients of at most 1
+  float base[3];  // 42 E^4 * 4: every tested line has coefficients of at most 1; at least 1e-36
 };
 // `norm` >= ||y||_2 of the row, `rot_err` = bound on the error of one rotated coordinate relative to it.
 // The float32 roundings of the tests themselves are folded into the constants, using u <= norm and w <= norm^2
@@ -58,6 +58,7 @@ struct RowMargins {
 //     and 42 rho^2 w^2 <= 6.8e-12 norm^2 w.
 __device__ __forceinline__ RowMargins make_row_margins(float norm, float rot_err, const FastQuant& fq) {
   RowMargins m;
+  norm = fmaxf(norm, 1e-18f);   // below, the sum of squares behind it has left the float32 range
   m.dy = rot_err * norm;
   m.dy1 = fmaf(1.8e-7f, norm, m.dy);
   m.dy3 = fmaxf(3.02f * m.dy, 1e-30f);  // the floor keeps a certified u in the range where the reciprocal is accurate
@@ -68,7 +69,7 @@ __device__ __forceinline__ RowMargins make_row_margins(float norm, float rot_err
     m.c[l] = 8.4f * el;
     m.cs[l] = m.c[l] + rr;
     m.csg[l] = fmaf(1.05e-11f * norm, norm, m.c[l]);
-    m.base[l] = 168.f * el * el;
+    m.base[l] = fmaf(168.f * el, el, 1e-36f);   // with a floor far above what squares of squared radii lose to underflow
   }
   return m;
 }

@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   for (int v = tid; v < V; v += kGeThreads) {
     float t = 0.f;
     for (int i = 0; i < ng; ++i) t += gsum[v * ng + i];
-    dy_sm[v] = rot_err * 1.0001f * sqrtf(t);
+    // the floor: where squares leave the float32 range (below 4e-20), nothing is certified
+    dy_sm[v] = fmaf(rot_err * 1.0001f, sqrtf(t), 1e-19f);
     dy_sm[V + v] = rotation_block_error(kGeSlice, (dc + kGeSlice - 1) / kGeSlice) * 1.0001f * sqrtf(t);
   }
   __syncthreads();

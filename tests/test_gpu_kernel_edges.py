@@ -280,3 +280,18 @@ def test_radii_of_vectors_concentrated_in_a_block(d, bits):
     rep, radii, want = _codes_and_radii(cache, K, V, pieces)
     assert_codes_match(rep)
     assert np.array_equal(radii.view(np.uint16), want.astype(np.float16).view(np.uint16))
+
+
+# Rows so small that squares, or the squares of squares that the sign tests compare, leave the float32 range.
+@pytest.mark.parametrize("scale", [3e-21, 2e-10, 1.0])
+@pytest.mark.parametrize("d,bits", [(128, None), (64, None), (16, None), (128, (3,) * 7), (64, (4, 3, 2)), (32, (5,)), (128, (6, 5, 4, 3, 2, 1, 1))])
+def test_codes_of_tiny_rows(d, bits, scale):
+    Hkv, pieces = 2, [20, 1400]
+    cache = _cache_of(d, bits, Hkv, sum(pieces))
+    K, V = (x * scale for x in synthetic.kv_like(52, sum(pieces), Hkv, d, torch.float32, DEV, n_outliers=0))
+    rep, radii, want = _codes_and_radii(cache, K, V, pieces)
+    assert_codes_match(rep)
+    if d < 128 or bits is not None:
+        assert np.array_equal(radii, want)
+    else:
+        assert_radii_match(radii, want)
