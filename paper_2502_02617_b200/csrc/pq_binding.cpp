@@ -66,6 +66,18 @@ int32_t dtype_code(const at::Tensor& t) {
   fail(PyExc_TypeError, "unsupported dtype (float32 and bfloat16 are taken)");
 }
 
+// Calls the library without the interpreter lock, as ctypes does: a launch may block on a full queue, and the first call of a kernel loads
+// it.  The arguments have been evaluated by then; the caller's frame holds the tensors.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <class... Params, class... Args>
+int32_t call(int32_t (*fn)(Params...), Args... args) {
+  const Unlocked unlocked;
+  return fn(args...);
+}
+
 // Runs `body` with `n` arguments checked and every exception turned into a Python one.
 template <class Body>
 PyObject* entry(Py_ssize_t got, Py_ssize_t want, Body body) {
@@ -100,10 +112,10 @@ PyObject* encode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const auto* pg = address<pq_paging>(a[9]);
     const int32_t d = (int32_t)K.size(2), h = (int32_t)K.size(1), total = (int32_t)K.size(0), batch = (int32_t)cu.numel() - 1;
     if (pg != nullptr)
-      return pq_encode_kv_paged(d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(K), ptr(V), dtype_code(K), K.stride(0),
+      return call(pq_encode_kv_paged, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(K), ptr(V), dtype_code(K), K.stride(0),
                                 K.stride(1), ptr<int32_t>(cu), batch, total, ptr(tensor(a[5])), ptr<int32_t>(tensor(a[6])), pg,
                                 ptr<int32_t>(tensor(a[8])), stream_of(a[10]));
-    return pq_encode_kv(d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(K), ptr(V), dtype_code(K), K.stride(0), K.stride(1),
+    return call(pq_encode_kv, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(K), ptr(V), dtype_code(K), K.stride(0), K.stride(1),
                         ptr<int32_t>(cu), batch, total, ptr(tensor(a[5])), ptr<int32_t>(tensor(a[6])), i32(a[7]),
                         ptr<int32_t>(tensor(a[8])), stream_of(a[10]));
   });
@@ -118,9 +130,9 @@ PyObject* append(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const auto* pg = address<pq_paging>(a[8]);
     const int32_t d = (int32_t)k.size(2), h = (int32_t)k.size(1), batch = (int32_t)k.size(0);
     if (pg != nullptr)
-      return pq_append_kv_paged(d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(k), ptr(v), dtype_code(k), batch,
+      return call(pq_append_kv_paged, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(k), ptr(v), dtype_code(k), batch,
                                 ptr(tensor(a[4])), ptr<int32_t>(tensor(a[5])), pg, ptr<int32_t>(tensor(a[7])), stream_of(a[9]));
-    return pq_append_kv(d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(k), ptr(v), dtype_code(k), batch, ptr(tensor(a[4])),
+    return call(pq_append_kv, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(k), ptr(v), dtype_code(k), batch, ptr(tensor(a[4])),
                         ptr<int32_t>(tensor(a[5])), i32(a[6]), ptr<int32_t>(tensor(a[7])), stream_of(a[9]));
   });
 }
@@ -145,21 +157,21 @@ PyObject* attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (lse != nullptr) {
       check(!multi && lse->scalar_type() == at::kFloat && lse->is_contiguous() && lse->dim() == 2 && lse->size(0) == batch && lse->size(1) == hq,
             "lse must be a contiguous float32 tensor [batch, query heads]");
-      return pq_decode_attention_lse(d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, cap, pg, most, scale, ptr(out),
+      return call(pq_decode_attention_lse, d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, cap, pg, most, scale, ptr(out),
                                      ptr<float>(*lse), ws, status, stream);
     }
     if (multi) {
       const int32_t nq = (int32_t)q.size(1);
       if (pg != nullptr)
-        return pq_multi_query_attention_paged(d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, nq, pg, most, scale,
+        return call(pq_multi_query_attention_paged, d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, nq, pg, most, scale,
                                               ptr(out), ws, status, stream);
-      return pq_multi_query_attention(d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, nq, cap, most, scale, ptr(out),
+      return call(pq_multi_query_attention, d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, nq, cap, most, scale, ptr(out),
                                       ws, status, stream);
     }
     if (pg != nullptr)
-      return pq_decode_attention_paged(d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, pg, most, scale, ptr(out), ws,
+      return call(pq_decode_attention_paged, d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, pg, most, scale, ptr(out), ws,
                                        status, stream);
-    return pq_decode_attention(d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, cap, most, scale, ptr(out), ws, status,
+    return call(pq_decode_attention, d, hq, hkv, S, tables, ptr(q), dtype_code(q), cache, lens, batch, cap, most, scale, ptr(out), ws, status,
                                stream);
   });
 }
@@ -171,7 +183,7 @@ PyObject* general_encode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_rows(K, V);
     const auto* cfg = address<pq_general_config>(a[0]);
     check(cfg != nullptr && K.size(2) == cfg->head_dim, "K and V must have the configuration's head_dim");
-    return pq_general_encode_kv(cfg, (int32_t)K.size(1), ptr<float>(tensor(a[1])), ptr<double>(tensor(a[2])), ptr(K), ptr(V),
+    return call(pq_general_encode_kv, cfg, (int32_t)K.size(1), ptr<float>(tensor(a[1])), ptr<double>(tensor(a[2])), ptr(K), ptr(V),
                                 dtype_code(K), K.stride(0), K.stride(1), ptr<int32_t>(cu), (int32_t)cu.numel() - 1,
                                 (int32_t)K.size(0), ptr(tensor(a[6])), ptr<int32_t>(tensor(a[7])), i32(a[8]),
                                 ptr<int32_t>(tensor(a[9])), stream_of(a[10]));
@@ -185,7 +197,7 @@ PyObject* general_attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_query(q, out, 3);
     const auto* cfg = address<pq_general_config>(a[0]);
     check(cfg != nullptr && q.size(2) == cfg->head_dim, "q must have the configuration's head_dim");
-    return pq_general_decode_attention(cfg, (int32_t)q.size(1), i32(a[1]), ptr<float>(tensor(a[2])), ptr<double>(tensor(a[3])), ptr(q),
+    return call(pq_general_decode_attention, cfg, (int32_t)q.size(1), i32(a[1]), ptr<float>(tensor(a[2])), ptr<double>(tensor(a[3])), ptr(q),
                                        dtype_code(q), ptr(tensor(a[5])), ptr<int32_t>(tensor(a[6])), (int32_t)q.size(0), i32(a[7]),
                                        f32(a[8]), ptr(out), ptr<int32_t>(tensor(a[10])), stream_of(a[11]));
   });
@@ -198,7 +210,7 @@ PyObject* angle_histograms(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_rows(K, V);
     check(hist.scalar_type() == at::kLong && hist.is_contiguous() && hist.dim() == 2 && hist.size(0) == PQ_N_LEVELS,
           "hist must be a contiguous int64 tensor [levels, bins]");
-    return pq_angle_histograms((int32_t)K.size(2), (int32_t)K.size(1), ptr<float>(tensor(a[0])), ptr(K), ptr(V), dtype_code(K),
+    return call(pq_angle_histograms, (int32_t)K.size(2), (int32_t)K.size(1), ptr<float>(tensor(a[0])), ptr(K), ptr(V), dtype_code(K),
                                K.stride(0), K.stride(1), (int32_t)K.size(0), (int32_t)hist.size(1), ptr<uint64_t>(hist),
                                ptr<int32_t>(tensor(a[4])), stream_of(a[5]));
   });
@@ -217,7 +229,7 @@ PyObject* tail_attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
           "the window must be contiguous [batch, tokens, kv heads, head_dim]");
     check(out.numel() == splits * q.numel() && (lse == nullptr || lse->numel() == splits * q.size(0) * q.size(1)),
           "out and lse must hold n_splits parts");
-    return pq_tail_attention((int32_t)q.size(2), (int32_t)q.size(1), (int32_t)k.size(2), ptr(q), dtype_code(q), ptr(k), ptr(v),
+    return call(pq_tail_attention, (int32_t)q.size(2), (int32_t)q.size(1), (int32_t)k.size(2), ptr(q), dtype_code(q), ptr(k), ptr(v),
                              dtype_code(k), ptr<int32_t>(tensor(a[3])), (int32_t)q.size(0), (int32_t)k.size(1), splits, f32(a[4]),
                              ptr(out), lse == nullptr ? nullptr : ptr<float>(*lse), ptr<int32_t>(tensor(a[7])), stream_of(a[9]));
   });
@@ -232,7 +244,7 @@ PyObject* merge(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check(lse.scalar_type() == at::kFloat && lse.dim() == 3 && lse.sizes() == parts.sizes().slice(0, 3) &&
               out.sizes() == parts.sizes().slice(1, 3),
           "parts_out [parts, batch, heads, head_dim], parts_lse float32 [parts, batch, heads], out [batch, heads, head_dim]");
-    return pq_merge_attention((int32_t)parts.size(3), (int32_t)parts.size(2), (int32_t)parts.size(1), (int32_t)parts.size(0), ptr(parts),
+    return call(pq_merge_attention, (int32_t)parts.size(3), (int32_t)parts.size(2), (int32_t)parts.size(1), (int32_t)parts.size(0), ptr(parts),
                               dtype_code(parts), ptr<float>(lse), ptr(out), dtype_code(out),
                               lse_out == nullptr ? nullptr : ptr<float>(*lse_out), ptr<int32_t>(tensor(a[4])), stream_of(a[5]));
   });
