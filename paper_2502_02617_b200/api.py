@@ -160,6 +160,13 @@ def _stream(stream) -> int:
     return stream.cuda_stream
 
 
+def _torch_stream(stream, device):
+    """`stream` (None, or an object with a cuda_stream attribute) as one that PyTorch can make the current one."""
+    if stream is None or isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(stream.cuda_stream, device=device)
+
+
 def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.float32:
         return DTYPE_F32
@@ -368,19 +375,22 @@ class PolarQuantCache:
         """Replace the codebooks of this cache by the ones clustered on the angles of K, V ([tokens, Hkv, d], the
         prompt's keys and values): histogram on the device, clustering on the host, new tables.  To be called
         before anything is encoded (codes already in the cache belong to the previous codebooks)."""
-        with torch.cuda.stream(stream):   # None: the current stream
+        with torch.cuda.stream(_torch_stream(stream, self.device)):   # None: the current stream
             hist = torch.zeros((N_LEVELS, n_bins), dtype=torch.int64, device=self.device)
             pq_angle_histograms(self.S, K, V, hist, self.status)
-            # the copies go through pinned memory (from a pool that keeps a block until its copy has finished)
+            # through pinned memory (from a pool that keeps a block until its copy has finished)
             counts = torch.empty((N_LEVELS, n_bins), dtype=torch.int64, pin_memory=True)
             counts.copy_(hist, non_blocking=True)
-            torch.cuda.current_stream().synchronize()
-            self.set_codebooks(*pq_fit_codebooks_from_histograms(counts))
+            torch.cuda.current_stream(self.device).synchronize()
+        if stream is not None:
+            hist.record_stream(torch.cuda.current_stream(self.device))   # it belongs to `stream`, and the caller uses it here
+        self.set_codebooks(*pq_fit_codebooks_from_histograms(counts))
         return hist
 
     def set_codebooks(self, centroids, boundaries):
+        """The new tables are on the device when this returns: calls on any stream may use them."""
         self.centroids, self.boundaries = centroids, boundaries
-        self.tables = pq_build_tables(centroids, boundaries, pinned=True).to(self.device, non_blocking=True)
+        self.tables = pq_build_tables(centroids, boundaries, pinned=self.device.type == "cuda").to(self.device)
 
     def encode(self, K, V, cu_seqlens, stream=None):
         pq_encode_kv(self.S, self.tables, K, V, cu_seqlens, self.cache, self.lens, self.capacity, self.status, stream)

@@ -216,3 +216,14 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(api, "LIB_PATH", str(ROOT / "no_such_library.so"))
     with pytest.raises(ImportError):
         pq.pq_fit_codebooks()
+
+
+def test_codebooks_of_a_cache_in_host_memory_can_be_replaced():
+    cache = pq.PolarQuantCache(1, 1, 1, 16, 64, device="cpu")
+    before = cache.tables.clone()
+    cen, bnd = pq.pq_fit_codebooks()
+    cen, bnd = cen.clone(), bnd.clone()
+    cen[:16] += 0.1
+    bnd[:15] += 0.1
+    cache.set_codebooks(cen, bnd)
+    assert cache.tables.device.type == "cpu" and not torch.equal(cache.tables, before)

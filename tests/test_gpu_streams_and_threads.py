@@ -39,3 +39,39 @@ def test_a_launch_that_blocks_does_not_hold_the_interpreter_lock():
     torch.cuda.synchronize()
     assert blocked > 0.4                      # the queue was full
     assert max(b - a for a, b in zip(ticks, ticks[1:])) < 0.2
+
+
+def _codebooks():
+    """Level 1 shifted: not the analytic codebook."""
+    cen, bnd = pq.pq_fit_codebooks()
+    cen, bnd = cen.clone(), bnd.clone()
+    cen[:16] += 0.1
+    bnd[:15] += 0.1
+    return cen, bnd
+
+
+@pytest.mark.parametrize("n", [20, 300])
+def test_new_codebooks_are_complete_on_every_stream(n):
+    cache, want = pq.PolarQuantCache(1, 2, 2, 128, capacity=n, device=DEV), pq.PolarQuantCache(1, 2, 2, 128, n, device=DEV, codebooks=_codebooks())
+    K, V = synthetic.kv_like(3, n, 2, 128, torch.bfloat16, DEV)
+    cu, side = torch.tensor([0, n], dtype=torch.int32, device=DEV), torch.cuda.Stream()
+    want.encode(K, V, cu)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(400_000_000)            # the current stream is busy
+    cache.set_codebooks(*_codebooks())
+    cache.encode(K, V, cu, stream=side)
+    torch.cuda.synchronize()
+    assert torch.equal(cache.unpack(n)[0], want.unpack(n)[0])
+
+
+def test_codebooks_fitted_on_one_stream_serve_another():
+    n = 300
+    cache, want = (pq.PolarQuantCache(1, 2, 2, 128, capacity=n, device=DEV) for _ in range(2))
+    K, V = synthetic.kv_like(4, n, 2, 128, torch.bfloat16, DEV)
+    cu, side = torch.tensor([0, n], dtype=torch.int32, device=DEV), torch.cuda.Stream()
+    hist = want.fit_online_codebooks(K, V)
+    want.encode(K, V, cu)
+    torch.cuda.synchronize()
+    assert torch.equal(cache.fit_online_codebooks(K, V, stream=side), hist)
+    cache.encode(K, V, cu)
+    assert torch.equal(cache.centroids, want.centroids) and torch.equal(cache.unpack(n)[0], want.unpack(n)[0])
