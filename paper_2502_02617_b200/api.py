@@ -321,9 +321,10 @@ def pq_dequant_kv(d, n_kv_heads, S, tables, cache, batch, capacity, n_tokens, st
 def pq_decode_attention_lse(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, lse, workspace,
                             status, paging=None, stream=None):
     """pq_decode_attention that also writes lse float32 [B, Hq] (log of the softmax denominator); `paging`: a Paging
-    for a paged cache, else the contiguous cache of `capacity` tokens."""
+    or (page table, tokens per page, pages) for a paged cache, else the contiguous cache of `capacity` tokens."""
     _check((_native or native()).attend(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, lse, workspace, status,
-                                        0 if paging is None else ctypes.addressof(paging), stream), "pq_decode_attention_lse")
+                                        0 if paging is None else ctypes.addressof(paging) if isinstance(paging, Paging) else paging, stream),
+           "pq_decode_attention_lse")
 
 
 def pq_merge_attention(parts_out, parts_lse, out, status, lse_out=None, stream=None):
@@ -406,7 +407,7 @@ class PolarQuantCache:
                             stream)
         return out
 
-    def _paging(self):
+    def _paging_args(self):
         return None
 
     def attend_lse(self, q, scale=None, max_len=None, stream=None):
@@ -415,7 +416,7 @@ class PolarQuantCache:
         lse = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device)
         pq_decode_attention_lse(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
                                 self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
-                                out, lse, self.workspace, self.status, paging=self._paging(), stream=stream)
+                                out, lse, self.workspace, self.status, paging=self._paging_args(), stream=stream)
         return out, lse
 
     def attend_with_tail(self, q, k_tail, v_tail, tail_lens, scale=None, stream=None):
@@ -427,7 +428,7 @@ class PolarQuantCache:
         parts_out = torch.empty((1 + n_splits,) + q32.shape, dtype=torch.float32, device=q.device)
         parts_lse = torch.empty((1 + n_splits,) + q32.shape[:2], dtype=torch.float32, device=q.device)
         pq_decode_attention_lse(self.S, self.tables, q32, self.cache, self.lens, self.n_kv_heads, self.capacity, self.capacity,
-                                scale, parts_out[0], parts_lse[0], self.workspace, self.status, paging=self._paging(),
+                                scale, parts_out[0], parts_lse[0], self.workspace, self.status, paging=self._paging_args(),
                                 stream=stream)
         pq_tail_attention(q32, k_tail, v_tail, tail_lens, scale, parts_out[1:], parts_lse[1:], self.status, n_splits, stream)
         return pq_merge_attention(parts_out, parts_lse, torch.empty_like(q), self.status, stream=stream)
@@ -490,34 +491,26 @@ class PagedPolarQuantCache(PolarQuantCache):
         self.workspace = torch.empty(pq_workspace_bytes(d, batch, n_q_heads, n_kv_heads, self.capacity), dtype=torch.uint8,
                                      device=self.device)
 
-    _pg = None   # (page table tensor, its address, tokens per page, pages, the struct, the struct's address)
-
-    def _paging_address(self):
-        """Address of the pq_paging struct, made again when the table or the pool it describes has been replaced."""
-        pg, table = self._pg, self.page_table
-        if pg is None or pg[0] is not table or pg[1] != table.data_ptr() or pg[2] != self.page_tokens or pg[3] != self.n_pages:
-            s = Paging.of(table, self.page_tokens, self.n_pages)
-            pg = self._pg = (table, table.data_ptr(), self.page_tokens, self.n_pages, s, ctypes.addressof(s))
-        return pg[5]
-
     def _paging(self):
-        self._paging_address()
-        return self._pg[4]
+        return Paging.of(self.page_table, self.page_tokens, self.n_pages)
+
+    def _paging_args(self):   # the same for the extension module, which checks the table as it is now
+        return self.page_table, self.page_tokens, self.n_pages
 
     def encode(self, K, V, cu_seqlens, stream=None):
         _check((_native or native()).encode(self.S, self.tables, K, V, cu_seqlens, self.cache, self.lens, self.capacity, self.status,
-                                            self._paging_address(), stream), "pq_encode_kv_paged")
+                                            self._paging_args(), stream), "pq_encode_kv_paged")
 
     def append(self, k_new, v_new, stream=None):
         _check((_native or native()).append(self.S, self.tables, k_new, v_new, self.cache, self.lens, self.capacity, self.status,
-                                            self._paging_address(), stream), "pq_append_kv_paged")
+                                            self._paging_args(), stream), "pq_append_kv_paged")
 
     def attend(self, q, out=None, scale=None, max_len=None, stream=None):
         out = torch.empty_like(q) if out is None else out
         assert q.dim() == 3
         _check((_native or native()).attend(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
                                             self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
-                                            out, None, self.workspace, self.status, self._paging_address(), stream),
+                                            out, None, self.workspace, self.status, self._paging_args(), stream),
                "pq_decode_attention_paged")
         return out
 
@@ -526,7 +519,7 @@ class PagedPolarQuantCache(PolarQuantCache):
         assert q.dim() == 4
         _check((_native or native()).attend(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
                                             self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
-                                            out, None, self._multi_workspace(q.shape[1]), self.status, self._paging_address(), stream),
+                                            out, None, self._multi_workspace(q.shape[1]), self.status, self._paging_args(), stream),
                "pq_multi_query_attention_paged")
         return out
 

@@ -4,7 +4,7 @@
 // than the kernels of a short step; this path costs below 1 us.  Every function returns the library's status code.
 //
 // Arguments common to all: `stream` is None (PyTorch's current stream) or an object with a cuda_stream attribute,
-// `paging` the address of a struct pq_paging or 0.
+// `paging` 0, the address of a struct pq_paging, or a tuple (page table tensor, tokens per page, pages of the pool).
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -51,6 +51,27 @@ const T* address(PyObject* o) {
   if (p == nullptr && PyErr_Occurred()) throw PyError();
   return static_cast<const T*>(p);
 }
+// The paging of a call, read before the interpreter lock is released.
+class PagingArg {
+ public:
+  explicit PagingArg(PyObject* o) {
+    if (PyTuple_Check(o)) {
+      check(PyTuple_GET_SIZE(o) == 3, "paging is (page table, tokens per page, pages)");
+      const at::Tensor& table = tensor(PyTuple_GET_ITEM(o, 0));
+      check(table.scalar_type() == at::kInt && table.is_contiguous() && table.dim() == 2, "the page table must be a contiguous int32 tensor [batch, pages]");
+      paging_ = {ptr<int32_t>(table), i32(PyTuple_GET_ITEM(o, 1)), (int32_t)table.size(1), i32(PyTuple_GET_ITEM(o, 2))};
+      paged_ = true;
+    } else if (const auto* p = address<pq_paging>(o)) {
+      paging_ = *p;
+      paged_ = true;
+    }
+  }
+  const pq_paging* get() const { return paged_ ? &paging_ : nullptr; }
+
+ private:
+  pq_paging paging_ = {};
+  bool paged_ = false;
+};
 void* stream_of(PyObject* o) {
   if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
   PyObject* v = PyObject_GetAttrString(o, "cuda_stream");
@@ -109,7 +130,8 @@ PyObject* encode(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return entry(n, 11, [&]() -> int32_t {
     const at::Tensor &K = tensor(a[2]), &V = tensor(a[3]), &cu = tensor(a[4]);
     check_rows(K, V);
-    const auto* pg = address<pq_paging>(a[9]);
+    const PagingArg paging(a[9]);
+    const pq_paging* pg = paging.get();
     const int32_t d = (int32_t)K.size(2), h = (int32_t)K.size(1), total = (int32_t)K.size(0), batch = (int32_t)cu.numel() - 1;
     if (pg != nullptr)
       return call(pq_encode_kv_paged, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(K), ptr(V), dtype_code(K), K.stride(0),
@@ -127,7 +149,8 @@ PyObject* append(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor &k = tensor(a[2]), &v = tensor(a[3]);
     check(k.dim() == 3 && k.is_contiguous() && v.is_contiguous() && v.sizes() == k.sizes() && v.scalar_type() == k.scalar_type(),
           "k_new and v_new must be contiguous [batch, kv heads, head_dim] of one dtype");
-    const auto* pg = address<pq_paging>(a[8]);
+    const PagingArg paging(a[8]);
+    const pq_paging* pg = paging.get();
     const int32_t d = (int32_t)k.size(2), h = (int32_t)k.size(1), batch = (int32_t)k.size(0);
     if (pg != nullptr)
       return call(pq_append_kv_paged, d, h, ptr<float>(tensor(a[0])), ptr(tensor(a[1])), ptr(k), ptr(v), dtype_code(k), batch,
@@ -145,7 +168,8 @@ PyObject* attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const bool multi = q.dim() == 4;
     check_query(q, out, multi ? 4 : 3);
     const at::Tensor* lse = tensor_or_none(a[10]);
-    const auto* pg = address<pq_paging>(a[13]);
+    const PagingArg paging(a[13]);
+    const pq_paging* pg = paging.get();
     const int32_t d = (int32_t)q.size(-1), hq = (int32_t)q.size(-2), batch = (int32_t)q.size(0), hkv = i32(a[5]), cap = i32(a[6]),
                   most = i32(a[7]);
     const float scale = f32(a[8]);

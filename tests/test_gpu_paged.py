@@ -121,3 +121,21 @@ def test_a_page_outside_the_pool_is_reported_and_nothing_is_written():
     assert cache.status.cpu().tolist()[0] == pq.ERR_INVALID_ARG and out.shape == (2, Hq, d)
     with pytest.raises(pq.PolarQuantError):
         pq.PagedPolarQuantCache(2, Hq, Hkv, d, 64, 3, table, seed=2, device=DEV)   # 64-token pages at d = 128
+
+
+def test_a_table_that_grows_in_place_is_read_as_it_is():
+    """The same tensor object, and the same memory, with more pages per sequence than at the call before."""
+    cache = pq.PagedPolarQuantCache(1, 2, 1, 128, 128, 4, torch.tensor([[2, 0, 3, 1]]), device=DEV)
+    K, V = synthetic.kv_like(9, 450, 1, 128, torch.bfloat16, DEV)
+    cache.page_table.resize_(1, 2)
+    cache.encode(K[:200], V[:200], torch.tensor([0, 200], dtype=torch.int32, device=DEV))
+    cache.page_table.resize_(1, 4)
+    cache.encode(K[200:], V[200:], torch.tensor([0, 250], dtype=torch.int32, device=DEV))
+    cache.check_status()
+    assert cache.lens.tolist() == [450]
+    flat = pq.PolarQuantCache(1, 2, 1, 128, capacity=512, device=DEV)
+    flat.encode(K, V, torch.tensor([0, 450], dtype=torch.int32, device=DEV))
+    assert torch.equal(cache.unpack(450)[0], flat.unpack(450)[0])
+    cache.page_table = cache.page_table.repeat(1, 2)[:, ::2]
+    with pytest.raises(AssertionError):                    # not contiguous
+        cache.attend(synthetic.queries(1, 1, 2, 128, torch.bfloat16, DEV))
