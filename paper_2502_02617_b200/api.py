@@ -438,22 +438,27 @@ class PolarQuantCache:
         out = torch.empty_like(q) if out is None else out
         scale = self.d ** -0.5 if scale is None else scale
         pq_multi_query_attention(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
-                                 self.capacity if max_len is None else max_len, scale, out, self._multi_workspace(q.shape[1]),
+                                 self.capacity if max_len is None else max_len, scale, out, self._multi_workspace(q.shape[1], stream),
                                  self.status, stream)
         return out
 
-    _multi_ws = None   # workspace of attend_multi; _multi_need: bytes it takes per number of queries
-    _multi_need = None
+    _multi_ws = None     # workspaces of attend_multi, one per stream: calls on different streams may overlap
+    _multi_need = None   # bytes they take per number of queries
 
-    def _multi_workspace(self, n_q):
+    def _multi_workspace(self, n_q, stream):
         if self._multi_need is None:
-            self._multi_need = {}
+            self._multi_need, self._multi_ws = {}, {}
         need = self._multi_need.get(n_q)
         if need is None:
             need = self._multi_need[n_q] = pq_workspace_bytes(self.d, self.batch * n_q, self.n_q_heads, self.n_kv_heads, self.capacity)
-        if self._multi_ws is None or self._multi_ws.numel() < need:
-            self._multi_ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-        return self._multi_ws
+        key = _stream(stream)
+        ws = self._multi_ws.get(key)
+        if ws is None or ws.numel() < need:
+            while len(self._multi_ws) >= 8 and key not in self._multi_ws:   # of streams that are no longer used
+                self._multi_ws.pop(next(iter(self._multi_ws)))
+            with torch.cuda.stream(_torch_stream(stream, self.device)):     # its memory goes back to the stream that used it
+                ws = self._multi_ws[key] = torch.empty(need, dtype=torch.uint8, device=self.device)
+        return ws
 
     def unpack(self, n_tokens):
         return pq_unpack_codes(self.d, self.n_kv_heads, self.cache, self.batch, self.capacity, n_tokens)
@@ -519,7 +524,7 @@ class PagedPolarQuantCache(PolarQuantCache):
         assert q.dim() == 4
         _check((_native or native()).attend(self.S, self.tables, q, self.cache, self.lens, self.n_kv_heads, self.capacity,
                                             self.capacity if max_len is None else max_len, self.d ** -0.5 if scale is None else scale,
-                                            out, None, self._multi_workspace(q.shape[1]), self.status, self._paging_args(), stream),
+                                            out, None, self._multi_workspace(q.shape[1], stream), self.status, self._paging_args(), stream),
                "pq_multi_query_attention_paged")
         return out
 

@@ -75,3 +75,20 @@ def test_codebooks_fitted_on_one_stream_serve_another():
     assert torch.equal(cache.fit_online_codebooks(K, V, stream=side), hist)
     cache.encode(K, V, cu)
     assert torch.equal(cache.centroids, want.centroids) and torch.equal(cache.unpack(n)[0], want.unpack(n)[0])
+
+
+def test_chunks_on_several_streams_do_not_share_scratch():
+    n, n_q = 4000, 64
+    cache = pq.PolarQuantCache(2, 16, 4, 128, capacity=n, device=DEV)
+    K, V = synthetic.kv_like(5, 2 * n, 4, 128, torch.bfloat16, DEV)
+    cache.encode(K, V, torch.tensor([0, n, 2 * n], dtype=torch.int32, device=DEV))
+    qs = [synthetic.queries(6 + i, 2 * n_q, 16, 128, torch.bfloat16, DEV).view(2, n_q, 16, 128) for i in range(10)]
+    want = [cache.attend_multi(q) for q in qs]
+    streams = [torch.cuda.Stream() for _ in qs]              # more than workspaces are kept for
+    outs = [torch.empty_like(q) for q in qs]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for q, out, s in zip(qs, outs, streams):
+            cache.attend_multi(q, out=out, stream=s)
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
