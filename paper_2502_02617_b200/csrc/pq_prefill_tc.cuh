@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
     }
     if (r < n_rows)   // scores are in the log2 domain
       a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] =
-          l_run > 0.f ? (m_run + log2f(l_run)) * 0.693147180559945309f : -CUDART_INF_F;
+          l_run > 0.f ? (m_run + log2f(l_run)) * 0.693147180559945309f : l_run == 0.f ? -CUDART_INF_F : l_run;   // NaN stays NaN
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kRotThreads) merge_unrotate_kernel(const float
       float mx = mine;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (mx > -CUDART_INF_F) {
+      if (mx > -CUDART_INF_F || __any_sync(0xffffffffu, mine != mine)) {   // a NaN part makes the row NaN
         const float w_mine = __expf(mine - mx);
         float wsum = w_mine;
 #pragma unroll

@@ -80,7 +80,7 @@ __device__ __forceinline__ void combine_rows(const DecodeArgs& a, const int2* in
       stat[2 * r + 1] = L > 0.f ? 1.f / L : 0.f;
       if (a.lse != nullptr)   // scores are in the log2 domain
         a.lse[info[r].x] = L > 0.f ? (M + log2f(L)) * 0.693147180559945309f : -CUDART_INF_F;
-      else if (!(L > 0.f)) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token
+      else if (info[r].y <= 0) set_status(a.status, PQ_ERR_EMPTY);   // a query that sees no token
     }
   }
   __syncthreads();

@@ -295,3 +295,23 @@ def test_codes_of_tiny_rows(d, bits, scale):
         assert np.array_equal(radii, want)
     else:
         assert_radii_match(radii, want)
+
+
+# A query that is not finite gives a row that is not finite -- not zeros, and not an empty sequence -- and leaves the others alone.
+@pytest.mark.parametrize("kernel", [CLUSTER, PERSISTENT, ROWS, TCGEN05])
+def test_a_nan_query_gives_a_nan_row(kernel):
+    lens, n_q, Hq = [700, 40], 8, 8
+    cache, ref = _filled(lens, Hq, 2, 128, 77)
+    q = torch.randn((2, n_q, Hq, 128), generator=torch.Generator(device=DEV).manual_seed(3), device=DEV)
+    bad = q.clone()
+    bad[0, 3, 5, 17] = float("nan")
+    bad[1, 7, 0, 0] = float("inf")
+    outs = []
+    for x in (q, bad):
+        pq.pq_debug_fail_next_wait(kernel)
+        outs.append(cache.attend_multi(x))
+    cache.check_status()
+    for b, j, h in ((0, 3, 5), (1, 7, 0)):
+        assert bool(torch.isnan(outs[1][b, j, h]).all())
+        outs[1][b, j, h] = outs[0][b, j, h]
+    assert torch.equal(outs[0], outs[1])
