@@ -96,13 +96,14 @@ __device__ __forceinline__ uint32_t ge_search(float a, float b, const float2* ta
   return pos;
 }
 
-// The exact code of the pair (a, b) at level l (0-based).
+// The exact code of the pair (a, b) at level l (0-based); kShared: the boundaries lie in shared memory.
+template <bool kShared = false>
 __device__ __forceinline__ uint32_t ge_exact_code(double a, double b, const GenConfig& g, int l, const double* boundaries) {
   double psi = atan2(b, a);
   if (l == 0 && psi < 0.0) psi += 6.283185307179586476925286766559;
   const double* bnd = boundaries + g.bnd_off[l];
   uint32_t code = 0;
-  for (int k = 0; k < (1 << g.bits[l]) - 1; ++k) code += psi > __ldg(bnd + k);
+  for (int k = 0; k < (1 << g.bits[l]) - 1; ++k) code += psi > (kShared ? bnd[k] : __ldg(bnd + k));
   return code;
 }
 
@@ -527,7 +528,7 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
 // the polar tree level by level (thread j forms angle j of the level, code = number of boundaries below it), then the bit streams.
 // A chain of d float64 multiply-adds and log2 d levels, hardly longer for a thousand vectors than for one: see launch_gen_encode.
 __global__ void gen_encode_vector_kernel(const __grid_constant__ GenEncodeArgs a) {
-  __shared__ double ra[kGenMaxDim], rb[kGenMaxDim];
+  __shared__ double ra[kGenMaxDim], rb[kGenMaxDim], bnd[kGenMaxCentroids];
   __shared__ uint8_t codes[kGenMaxDim];
   __shared__ int64_t dest;
   const GenConfig& g = a.g;
@@ -538,6 +539,7 @@ __global__ void gen_encode_vector_kernel(const __grid_constant__ GenEncodeArgs a
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the inputs may come from the kernel before this one
   if (j == 0) dest = ge_destination(a, row, head, kv);
+  for (int i = j; i < g.n_cen - g.L; i += blockDim.x) bnd[i] = a.boundaries[i];
   if (j < d) {
     const float x = ge_load(kv ? a.V : a.K, a.in_dtype, (int64_t)row * a.token_stride + (int64_t)head * a.head_stride + j);
     if (!(fabsf(x) < CUDART_INF_F)) {
@@ -558,7 +560,7 @@ __global__ void gen_encode_vector_kernel(const __grid_constant__ GenEncodeArgs a
   for (int l = 0; l < g.L; ++l) {
     if (j < (d >> (l + 1))) {
       const double p = src[2 * j], q = src[2 * j + 1];
-      codes[g.code_off[l] + j] = (uint8_t)ge_exact_code(p, q, g, l, a.boundaries);
+      codes[g.code_off[l] + j] = (uint8_t)ge_exact_code<true>(p, q, g, l, bnd);
       dst[j] = sqrt(p * p + q * q);
     }
     __syncthreads();
