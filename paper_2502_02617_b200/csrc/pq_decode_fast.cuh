@@ -517,16 +517,14 @@ __device__ __forceinline__ void elect_combiner(const DecodeArgs& a, int u, int u
     __syncwarp();
     __threadfence();   // the flag before the look at the others
     for (int p0 = 0; p0 < n_parts; p0 += 32) last = last && (p0 + lane >= n_parts || flags[p0 + lane] == a.epoch);
+    __threadfence();   // every lane: the flags that it has seen before the partial results that the block then reads
     last = __all_sync(0xffffffffu, last);
     if (last && lane == 0) last = atomicExch(a.ws.elected + u, a.epoch) != a.epoch;
     last = __shfl_sync(0xffffffffu, last, 0);
     if (last)   // all parts have raised theirs
       for (int p0 = lane; p0 < n_parts; p0 += 32) flags[p0] = 0u;
   }
-  if (lane == 0) {
-    __threadfence();
-    *is_last = last;
-  }
+  if (lane == 0) *is_last = last;
 }
 
 // kHG: groups of four query heads per kv head (1 or 2).
