@@ -322,6 +322,7 @@ def pq_decode_attention_lse(S, tables, q, cache, cache_lens, n_kv_heads, capacit
                             status, paging=None, stream=None):
     """pq_decode_attention that also writes lse float32 [B, Hq] (log of the softmax denominator); `paging`: a Paging
     or (page table, tokens per page, pages) for a paged cache, else the contiguous cache of `capacity` tokens."""
+    assert q.dim() == 3 and lse.dtype == torch.float32
     _check((_native or native()).attend(S, tables, q, cache, cache_lens, n_kv_heads, capacity, max_len, scale, out, lse, workspace, status,
                                         0 if paging is None else ctypes.addressof(paging) if isinstance(paging, Paging) else paging, stream),
            "pq_decode_attention_lse")

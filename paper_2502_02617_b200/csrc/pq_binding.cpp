@@ -218,7 +218,8 @@ PyObject* general_encode(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* general_attend(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return entry(n, 12, [&]() -> int32_t {
     const at::Tensor &q = tensor(a[4]), &out = tensor(a[9]);
-    check_query(q, out, 3);
+    check(q.dim() == 3 && q.is_contiguous() && out.is_contiguous() && out.numel() >= q.numel() && out.scalar_type() == q.scalar_type(),
+          "q must be [batch, heads, head_dim], out of its dtype with room for as many values, both contiguous");
     const auto* cfg = address<pq_general_config>(a[0]);
     check(cfg != nullptr && q.size(2) == cfg->head_dim, "q must have the configuration's head_dim");
     return call(pq_general_decode_attention, cfg, (int32_t)q.size(1), i32(a[1]), ptr<float>(tensor(a[2])), ptr<double>(tensor(a[3])), ptr(q),

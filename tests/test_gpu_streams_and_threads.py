@@ -92,3 +92,19 @@ def test_chunks_on_several_streams_do_not_share_scratch():
             cache.attend_multi(q, out=out, stream=s)
         torch.cuda.synchronize()
         assert all(torch.equal(o, w) for o, w in zip(outs, want))
+
+
+def test_arguments_that_the_entry_points_take_and_refuse():
+    cache = pq.PolarQuantCache(2, 4, 2, 128, capacity=64, device=DEV)
+    K, V = synthetic.kv_like(7, 20, 2, 128, torch.bfloat16, DEV)
+    cache.encode(K, V, torch.tensor([0, 10, 20], dtype=torch.int32, device=DEV))
+    q = synthetic.queries(8, 2, 4, 128, torch.bfloat16, DEV)
+    with pytest.raises((AssertionError, AttributeError)):    # the log-sum-exp has nowhere to go
+        pq.pq_decode_attention_lse(cache.S, cache.tables, q, cache.cache, cache.lens, 2, 64, 64, 0.1, torch.empty_like(q), None,
+                                   cache.workspace, cache.status)
+    general = pq.GeneralPolarQuantCache(2, 4, 2, 64, (3, 3), 64, device=DEV)
+    Kg, Vg = synthetic.kv_like(9, 20, 2, 64, torch.float32, DEV)
+    general.encode(Kg, Vg, torch.tensor([0, 10, 20], dtype=torch.int32, device=DEV))
+    qg = synthetic.queries(10, 2, 4, 64, torch.float32, DEV)
+    flat = torch.empty(2 * 4 * 64, device=DEV)               # an output of another shape
+    assert torch.equal(general.attend(qg, out=flat).view(2, 4, 64), general.attend(qg))
