@@ -287,7 +287,8 @@ int32_t pq_decode_attention_static(int32_t head_dim, int32_t n_q_heads, int32_t 
  * `which` = 5 is of that kind too: the next attention call at head_dim 128 with up to 32 rows that would run the cluster
  * kernel of short contexts runs one of the persistent kernels instead, whatever max_len is (2 implies it).
  * `which` = 6, 7, 8, 9: the next attention call at head_dim 128 runs the cluster kernel, the persistent kernel, the rows
- * kernel or the tcgen05 kernel whatever the estimates say, or returns PQ_ERR_UNSUPPORTED if that kernel does not take it.
+ * kernel or the tcgen05 kernel whatever the estimates say, or returns PQ_ERR_UNSUPPORTED if that kernel does not take it;
+ * `which` = 10: the next one runs as on a device that the tcgen05 kernel does not fit.
  */
 int32_t pq_debug_fail_next_wait(int32_t which);
 

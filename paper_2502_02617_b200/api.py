@@ -296,7 +296,7 @@ def pq_decode_attention_static(S, tables, q, cache, cache_lens, n_kv_heads, capa
 
 def pq_debug_fail_next_wait(which: int) -> None:
     """Test support: 1 = the next tensor-core encode launch, 2 = the next head_dim-128 decode-attention
-    launch, 4 = the next tcgen05 multi-query launch runs its give-up path (PQ_ERR_TIMEOUT in status word 0); 3, 5 .. 9 choose
+    launch, 4 = the next tcgen05 multi-query launch runs its give-up path (PQ_ERR_TIMEOUT in status word 0); 3, 5 .. 10 choose
     the kernel of the next head_dim-128 attention call (see polarquant.h); 0 disarms."""
     _check(lib().pq_debug_fail_next_wait(int(which)), "pq_debug_fail_next_wait")
 

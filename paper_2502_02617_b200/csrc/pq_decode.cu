@@ -683,6 +683,23 @@ static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_k
   if (kernel == kRowsKernel) return batch * n_kv_heads * cut_rows((int64_t)n_q * g).blocks <= kFastMaxUnits;
   return true;
 }
+// Whether the tcgen05 kernel's map of shared memory holds on the current device: it counts on the place where dynamic shared memory
+// starts.
+static bool tensor_kernel_fits() {
+  static DeviceMemo reserved;   // bytes + 1
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+  int known = reserved[dev].load(std::memory_order_relaxed);
+  if (known == 0) {
+    int bytes = 0;
+    if (cudaDeviceGetAttribute(&bytes, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    reserved[dev].store(known = bytes + 1, std::memory_order_relaxed);
+  }
+  return known - 1 == (int)kPtBase;
+}
 // Room for the parts of split tcgen05 calls in the workspace of pq_workspace_bytes: a call whose parts would not fit is split
 // less.  (148 SMs with 128 rows each, twice over, bound what a useful split can need.)
 __host__ inline int64_t part_rows_room(int64_t pairs, int64_t n_q_heads) {
@@ -846,10 +863,11 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     pq::size_split(split);
     pq::SplitLoad load = {};
     if (pq::plan_split(split, pairs, max_len, &load) == 0) return PQ_ERR_CUDA;
-    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, load, lse_dev == nullptr && n_q * g >= 32);
+    const bool tensor = lse_dev == nullptr && pq::tensor_kernel_fits() && !pq::take_debug_wait_failure(10);
+    pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, load, tensor && n_q * g >= 32);
     if (const int named = pq::take_debug_hook(6, 9)) {   // test hook: the kernel is named
       plan.kernel = named == 6 ? pq::kClusterKernel : named == 7 ? pq::kPersistentKernel : named == 8 ? pq::kRowsKernel : pq::kTensorKernel;
-      if (!pq::kernel_takes(plan.kernel, batch, n_q, n_kv_heads, g) || (plan.kernel == pq::kTensorKernel && lse_dev != nullptr))
+      if (!pq::kernel_takes(plan.kernel, batch, n_q, n_kv_heads, g) || (plan.kernel == pq::kTensorKernel && !tensor))
         return PQ_ERR_UNSUPPORTED;
     }
     const bool forced = n_q * g <= 32 && pq::take_debug_wait_failure(5), fail_wait = n_q * g <= 32 && pq::take_debug_wait_failure(2);

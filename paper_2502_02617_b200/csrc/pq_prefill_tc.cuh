@@ -48,7 +48,8 @@ constexpr int kPtRawBytes = 2 * kBlockBytes128;     // a packed K block and V bl
 constexpr int kPtRawBufs = 4;                       // of them in flight
 constexpr int kPtScores = 4;                        // score accumulators: the score MMAs run ahead of the softmax
 constexpr int kPtGroups = 16;                       // warp-sized pieces of a block's decoding
-// Shared memory, as offsets in the CTA's shared window (whose addresses carry the CTA's rank in the cluster above): dynamic shared memory starts behind the 1 KB that the system keeps, the
+// Shared memory, as offsets in the CTA's shared window (whose addresses carry the CTA's rank in the cluster above): dynamic shared
+// memory starts behind what the system keeps (1 KB; where it is not, the kernel is not taken: tensor_kernel_fits), the
 // decode tables (those of the decode kernel: 96 KB, replicated for conflict-free lookups) on a 32 KB boundary, so that a
 // table address is the OR of disjoint bit fields.
 constexpr uint32_t kPtBase = 1024;
@@ -122,10 +123,6 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   extern __shared__ __align__(1024) uint8_t pt_smem_raw[];
   uint8_t* smem = pt_smem_raw - kPtBase;
   const uint32_t sb = tc_smem_u32(pt_smem_raw) - kPtBase;   // the window: rank << 24
-  if (sb & 0xFFFFFFu) {   // not on this architecture: the table addresses count on the place (both CTAs leave alike)
-    set_status(a.status, PQ_ERR_CUDA);
-    return;
-  }
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform
   const int g = a.n_q_heads / a.n_kv_heads;
@@ -142,6 +139,12 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   auto row_index = [&](int r) -> int64_t {               // offset of row r in q / out ([batch][n_q][n_q_heads][128])
     return (((int64_t)b * n_q + q0 + r / g) * a.n_q_heads + hk * g + r % g) * 128;
   };
+  if (sb & 0xFFFFFFu) {   // the host asks for the place (tensor_kernel_fits): never, and then NaN rather than anything (both CTAs leave alike)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int r = tid; r < n_rows; r += kPtThreads) a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] = CUDART_NAN_F;
+    set_status(a.status, PQ_ERR_CUDA);
+    return;
+  }
   if (tid == 0) {
     for (int i = 0; i < kPtStages; ++i) {
       tc_mbar_init(sb + kPtBarKv + 8 * i, 2 * kPtGroups);    // one arrival per decoded piece (of both CTAs)

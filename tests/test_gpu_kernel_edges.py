@@ -315,3 +315,15 @@ def test_a_nan_query_gives_a_nan_row(kernel):
         assert bool(torch.isnan(outs[1][b, j, h]).all())
         outs[1][b, j, h] = outs[0][b, j, h]
     assert torch.equal(outs[0], outs[1])
+
+
+# Where the tcgen05 kernel does not fit, a long chunk runs on the others.
+def test_long_chunk_without_the_tcgen05_kernel():
+    lens, n_q = [700, 300], 64
+    cache, ref = _filled(lens, 8, 2, 128, 78)
+    q = torch.randn((2, n_q, 8, 128), generator=torch.Generator(device=DEV).manual_seed(4), device=DEV)
+    _check_multi(cache, ref, q, lens, 10)
+    pq.pq_debug_fail_next_wait(TCGEN05)
+    other = cache.attend_multi(q)
+    pq.pq_debug_fail_next_wait(10)
+    assert not torch.equal(cache.attend_multi(q), other)
