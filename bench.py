@@ -767,8 +767,7 @@ def reduce_and_format(local, steps, warmup, rank, world, dist=None, device="cpu"
                               "pq_decode_attention, D2H of the output]; the byte counts are the copies inside that region.  "
                               "The prefill chunk's own H2D (e2e_h2d_bytes_per_chunk) and encode are timed as encode.e2e_tokens_per_s",
                 "ms_per_pass_with_prefill_h2d": e2e_total_ms / (steps * head["e2e_inner"])},
-        "gpu_launches": 5 * n_pass,  # steps of a pass: encode, its lengths, append, its lengths, decode attention
-        "gpu_launches_note": "an append advances its lengths in the same launch: 4 launches carry the 5 steps of a pass",
+        "gpu_launches": 4 * n_pass,  # encode, its lengths, append (which advances its own), decode attention
         "clocks": clocks,
         "oracle_match": head["match"],
         "configs": {},

@@ -8,6 +8,7 @@ any entry point raises.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from ctypes import c_char_p, c_double, c_float, c_int32, c_int64, c_uint64, c_void_p, POINTER
@@ -457,8 +458,8 @@ class PolarQuantCache:
         if ws is None or ws.numel() < need:
             while len(self._multi_ws) >= 8 and key not in self._multi_ws:   # of streams that are no longer used
                 self._multi_ws.pop(next(iter(self._multi_ws)))
-            with torch.cuda.stream(_torch_stream(stream, self.device)):     # its memory goes back to the stream that used it
-                ws = self._multi_ws[key] = torch.empty(need, dtype=torch.uint8, device=self.device)
+            with contextlib.nullcontext() if stream is None else torch.cuda.stream(_torch_stream(stream, self.device)):
+                ws = self._multi_ws[key] = torch.empty(need, dtype=torch.uint8, device=self.device)   # goes back to the stream that used it
         return ws
 
     def unpack(self, n_tokens):

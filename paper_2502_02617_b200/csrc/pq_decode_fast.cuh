@@ -166,13 +166,6 @@ __device__ __forceinline__ void mma_16816(float* d, uint32_t a0, uint32_t a1, ui
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// D(16x8, f32) += A(16x8, f16, row) * B(8x8, f16, col)
-__device__ __forceinline__ void mma_1688(float* d, uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a0), "r"(a1), "r"(b0));
-}
-
 // Codes of one 16-coordinate block of one token, prepared for the table lookups.  Entry idx of the
 // replicated u table of sub-block s sits at s * 8192 + idx * 128 with idx = c2_s | c3 << 2 | c4 << 4, i.e.
 // c2_s -> address bits 7..8, c3 -> bits 9..10, c4 -> bits 11..12; `ub` = table base | lane replica has

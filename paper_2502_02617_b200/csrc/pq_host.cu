@@ -359,7 +359,7 @@ int32_t pq_fit_codebooks_from_histograms(const uint64_t* hist, int32_t n_bins, c
   std::vector<double> centre(n_bins), w0(n_bins + 1), w1(n_bins + 1);
   for (int level = 1; level <= PQ_N_LEVELS; ++level) {
     const int n = level == 1 ? 16 : 4;
-    const double hi = level == 1 ? 2.0 * kPi : 0.5 * kPi, width = hi / n_bins, inv_width = n_bins / hi;
+    const double hi = level == 1 ? 2.0 * kPi : 0.5 * kPi, width = hi / n_bins;
     const uint64_t* h = hist + (size_t)(level - 1) * n_bins;
     double* theta = cen + pq::cen_off(level);
     double* beta = bnd + pq::bnd_off(level);

@@ -15,7 +15,8 @@ from parity_utils import (TOL_ATTENTION, TOL_DECODED, assert_codes_match, assert
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 CASES = [(128, (3,) * 7, 8, 2), (64, (4, 3, 2), 4, 2), (256, (4, 2, 2, 2, 2), 2, 1), (16, (2, 2, 2, 2), 2, 1),
-         (128, (4, 2, 2, 2), 8, 2), (32, (5,), 3, 3), (128, (6, 5, 4, 3, 2, 1, 1), 4, 1)]
+         (128, (4, 2, 2, 2), 8, 2), (32, (5,), 3, 3), (128, (6, 5, 4, 3, 2, 1, 1), 4, 1),
+         (64, (2,) * 6, 4, 2), (128, (4,) * 7, 8, 1)]      # every angle with two or with four bits: instances of their own
 
 
 @pytest.mark.parametrize("d,bits,Hq,Hkv", CASES)
