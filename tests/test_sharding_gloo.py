@@ -96,7 +96,7 @@ def test_bench_rank_logic_takes_the_slowest_rank_and_sums_the_job():
     assert abs(line["value"] - 2 * comp / (0.15 * 1.5 * 1e-3) / 1e9) < 1e-6  # both ranks' bytes over that time
     assert abs(line["ms_per_step"] - 60.0 * 1.5 / 20) < 1e-9
     assert abs(line["e2e"]["region_ms"] - (0.03 + 0.2) * 1.5) < 1e-12
-    assert line["e2e"]["h2d_bytes_per_step"] == 98304 and line["gpu_launches"] == 5 * 20 * 3
+    assert line["e2e"]["h2d_bytes_per_step"] == 98304 and line["gpu_launches"] == 4 * 20 * 3
     assert abs(line["configs"]["cfg4"]["decode_step_ms"] - 4.5) < 1e-12 and abs(line["configs"]["cfg5"]["decode_ms"] - 0.45) < 1e-12
     assert line["roofline"]["bound"] == "hbm" and abs(line["roofline"]["frac"] * line["roofline"]["peak"] - line["roofline"]["achieved"]) < 1e-6
 
