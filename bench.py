@@ -620,8 +620,7 @@ def measure_tail_window(args, pq, synthetic, dev, rank):
 
 def measure_general(args, pq, synthetic, dev, rank):
     """The general entry points on the full recursion of Section 4 (d = 128, log2 d = 7 levels, 3 bits per angle:
-    16 + 127 x 3 bits per vector): encode of 4096 tokens x 8 kv heads and decode attention over batch 8 x 4096 tokens.
-    Reference-speed kernels (float64 encoder, one thread block per sequence and kv head in attention)."""
+    16 + 127 x 3 bits per vector): encode of 4096 tokens x 8 kv heads and decode attention over batch 8 x 4096 tokens."""
     n, bits = 4096, (3,) * 7
     cache = pq.GeneralPolarQuantCache(BATCH, HQ, HKV, D, bits, n, seed=0, device=dev)
     K, V = synthetic.kv_like(1000 * rank + 5, n, HKV, D, torch.bfloat16, dev)

@@ -13,7 +13,8 @@
  *     the current device.  The library allocates no device memory; every buffer belongs to
  *     the caller.  Device pointers must be 16-byte aligned.
  *   - State the library keeps, all of it per process: a call counter that tags the scratch of
- *     pq_decode_attention, a per-device note of which kernels have been configured (and, for
+ *     pq_decode_attention, a per-device note of which kernels have been configured and of what the device answered about
+ *     them (and, for
  *     pq_decode_attention_static, the device address of its built-in array, which every GPU
  *     that loads the library carries), the last CUDA error of each host thread, the analytic
  *     codebook pq_fit_codebooks_from_histograms starts from (computed at its first use), and the
@@ -252,8 +253,8 @@ int32_t pq_multi_query_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_
  * device array of PQ_STATIC_SCRATCH_BYTES bytes that every GPU which loads the library keeps
  * until the process exits.  Arguments and results are those of pq_decode_attention without
  * `workspace_dev`.
- *   - Returns PQ_ERR_SCRATCH, and launches nothing, if pq_workspace_bytes(...) for these arguments
- *     exceeds PQ_STATIC_SCRATCH_BYTES (compare pq_static_scratch_bytes()).
+ *   - Returns PQ_ERR_SCRATCH, and launches nothing, if the partial results of a single-query call with these arguments
+ *     exceed PQ_STATIC_SCRATCH_BYTES (pq_workspace_bytes() is an upper bound: it covers multi-query calls too).
  *   - The first call on each device looks up the device address of the array (a host-side query,
  *     no allocation); make that first call outside any stream capture.
  *   - Never calls cudaMalloc, cudaFree or any allocating routine.

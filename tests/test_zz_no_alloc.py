@@ -40,8 +40,8 @@ def test_static_scratch_entry_matches_workspace_entry_twice_in_a_row(d, Hq, Hkv,
 
 
 def test_static_scratch_entry_after_a_call_of_the_other_kernel_family():
-    """The head_dim-16 path counts its splits with small integers in the shared array; the head_dim-128 path that
-    runs next on the same bytes (units shared by several CTAs) must not take them for arrivals of its own call.  Device
+    """Calls of the two families in turn on the shared array: the head_dim-128 path (units shared by several CTAs) must not take
+    what it finds there for arrivals of its own call.  Device
     memory in use is the same before and after: the entry allocates nothing."""
     small = _filled_cache(16, 2, 1, [100, 37], seed=62)
     big = _filled_cache(128, 8, 2, [9000, 5000], seed=63)   # few units, many CTAs per unit
