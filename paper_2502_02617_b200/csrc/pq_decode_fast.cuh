@@ -905,9 +905,10 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
           o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
         }
       }
-    // Register allocation of nvcc 12.9, not a property of paging: in the contiguous instantiation the segment is read again (and through volatile, so that it really is): the registers that its
+    // In the contiguous instantiation the segment is read again (and through volatile, so that it really is): the registers that its
     // fields would hold through the tile loop cost that loop 2 % (8 x 131072 tokens: 516 -> 507 us).  In the paged one it is
-    // the other way round (16 ragged sequences of up to 65536 tokens, four steps: 1313 us, 1365 with the fields read again).
+    // the other way round (16 ragged sequences of up to 65536 tokens, four steps: 1313 us, 1365 with the fields read again).  That is
+    // the register allocation of nvcc 12.9, not a property of paging.
     struct {
       int unit, b, hk, part, n_parts, slot0;
     } done;
