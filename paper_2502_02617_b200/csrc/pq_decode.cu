@@ -740,7 +740,7 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
       const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s, at_once = n_sm / 2;   // two query blocks each
       const double waves = (double)((clusters + at_once - 1) / at_once), work = waves * ((blocks + s - 1) / s);
-      const double t = 18.0 + 1.11 * work + 1.1 * std::min(work, 4.0) + 5.2 * clusters / (at_once * waves) +
+      const double t = 18.0 + 1.11 * work + 1.1 * std::min(work, 4.0) + 5.2 * clusters / (at_once * waves) + 20.0 * (waves - 1.0) +
                        2.6e-3 * std::min<int64_t>(all_rows, 3000) + 1.06e-3 * all_rows + 0.36e-3 * s * all_rows;
       if (t < est[kTensorKernel]) {
         est[kTensorKernel] = t;
