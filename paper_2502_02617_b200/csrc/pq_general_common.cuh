@@ -43,9 +43,9 @@ int32_t launch_packed_encode(GenEncodeArgs a, int head_dim, cudaStream_t stream)
 
 // Would the block radius r round to another fp16 value if it moved by its error?  (NaN and infinite r: yes; near saturation: yes, it
 // is counted from the exact value.)  `err` bounds the 2-norm of the error of the block's rotated coordinates, and so the error that
-// their rotation brings into r; the sums of squares and the square root add less than 8 roundings of 2^-24, below 1e-6 r.
+// their rotation brings into r; the sums of squares and the square root add less than 8 roundings of 2^-24, below 5e-7 r.
 __device__ __forceinline__ bool radius_unsure(float r, float err) {
-  const float slack = fmaf(1e-6f, r, err), lo = fminf(r - slack, 65504.f), hi = fminf(r + slack, 65504.f);
+  const float slack = fmaf(5e-7f, r, err), lo = fminf(r - slack, 65504.f), hi = fminf(r + slack, 65504.f);
   return !(r < CUDART_INF_F) || __half_as_ushort(__float2half_rn(fmaxf(lo, 0.f))) != __half_as_ushort(__float2half_rn(hi)) || !(r <= 65000.f);
 }
 // That bound for y = x S summed in `slices` chains of `chain` fused multiply-adds whose results are added one by one, relative to
