@@ -4,6 +4,7 @@
 #include <cmath>
 #include <chrono>
 #include <math_constants.h>
+#include <type_traits>
 
 #include "pq_common.cuh"
 
@@ -677,15 +678,9 @@ struct AttentionPlan {
   int n_splits;
 };
 constexpr int kMaxSplits = 16;
-// Whether a kernel takes a call at all.
-static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_kv_heads, int g) {
-  if (kernel == kPersistentKernel) return batch * n_q * n_kv_heads <= kFastMaxUnits;
-  if (kernel == kRowsKernel) return batch * n_kv_heads * cut_rows((int64_t)n_q * g).blocks <= kFastMaxUnits;
-  return true;
-}
-// Whether the tcgen05 kernel's map of shared memory holds on the current device: it counts on the place where dynamic shared memory
-// starts.
-static bool tensor_kernel_fits() {
+// Whether the persistent and the tcgen05 kernel's maps of shared memory hold on the current device: they count on the place where
+// dynamic shared memory starts.
+static bool window_as_mapped() {
   static DeviceMemo reserved;   // bytes + 1
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
@@ -698,7 +693,13 @@ static bool tensor_kernel_fits() {
     }
     reserved[dev].store(known = bytes + 1, std::memory_order_relaxed);
   }
-  return known - 1 == (int)kPtBase;
+  return known - 1 == (int)kWindowBase;
+}
+// Whether a kernel takes a call at all.
+static bool kernel_takes(AttentionKernel kernel, int64_t batch, int n_q, int n_kv_heads, int g) {
+  if (kernel == kPersistentKernel) return batch * n_q * n_kv_heads <= kFastMaxUnits && window_as_mapped();
+  if (kernel == kRowsKernel) return batch * n_kv_heads * cut_rows((int64_t)n_q * g).blocks <= kFastMaxUnits;
+  return true;
 }
 // Room for the parts of split tcgen05 calls in the workspace of pq_workspace_bytes: a call whose parts would not fit is split
 // less.  (148 SMs with 128 rows each, twice over, bound what a useful split can need.)
@@ -863,7 +864,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
     pq::size_split(split);
     pq::SplitLoad load = {};
     if (pq::plan_split(split, pairs, max_len, &load) == 0) return PQ_ERR_CUDA;
-    const bool tensor = lse_dev == nullptr && pq::tensor_kernel_fits() && !pq::take_debug_wait_failure(10);
+    const bool tensor = lse_dev == nullptr && pq::window_as_mapped() && !pq::take_debug_wait_failure(10);
     pq::AttentionPlan plan = pq::plan_attention(batch, n_q, n_kv_heads, g, max_len, n_sm, load, tensor && n_q * g >= 32);
     if (const int named = pq::take_debug_hook(6, 9)) {   // test hook: the kernel is named
       plan.kernel = named == 6 ? pq::kClusterKernel : named == 7 ? pq::kPersistentKernel : named == 8 ? pq::kRowsKernel : pq::kTensorKernel;
@@ -882,8 +883,8 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
       void (*fast)(pq::DecodeArgs) =
           g <= 4 ? (paged ? pq::decode_attention_fast_kernel<1, true> : pq::decode_attention_fast_kernel<1, false>)
                  : (paged ? pq::decode_attention_fast_kernel<2, true> : pq::decode_attention_fast_kernel<2, false>);
-      if (pq::configure_for_device(fast, pq::kSmTotal, configured[(g > 4 ? 2 : 0) + (paged ? 1 : 0)]) == 0) return PQ_ERR_CUDA;
-      return pq::launch_persistent(fast, a, n_sm, pq::kFastThreads, pq::kSmTotal, st);
+      if (pq::configure_for_device(fast, pq::kFsTotal, configured[(g > 4 ? 2 : 0) + (paged ? 1 : 0)]) == 0) return PQ_ERR_CUDA;
+      return pq::launch_persistent(fast, a, n_sm, pq::kFastThreads, pq::kFsTotal, st);
     }
   }
   switch (head_dim) {

@@ -14,13 +14,20 @@
 //   * decodes the values into A fragments (coordinates x (token, element of a decoded pair)) and
 //     accumulates O^T += V_hat^T P on tensor cores (fp32 accumulators in registers).
 // DeQuant (Algorithm 1) of one 16-coordinate block is a product tree r * t4 * t3 * t2 * t1.
-// Levels 4..2 are folded into one table per 4-coordinate sub-block, level 1 is a half2 multiply:
-//   u    [4][64][16] sub-block s, index c2_s | c3_(s>>1) << 2 | c4 << 4 -> the multipliers of the
-//                    sub-block's two level-1 pairs as (half2 values, half2 rounding residuals)
-//   t1hi [256][16]   index = one byte of level-1 codes (pair a = 2s | pair b = 2s+1 << 4) -> (cos a, cos b), (sin a, sin b)
-//                    in fp16: the half2 (u_a, u_b) of the table above multiplies them element-wise
-//   t1lo [256][16]   the fp16 rounding residuals of the same entries
-// All are replicated 16 times so that every lane of a half-warp reads its own banks.
+// Levels 4..2 are folded into one lookup per half block (8 coordinates), level 1 is one lookup per byte of codes and a half2
+// multiply by it:
+//   U  index = the half's level-2 codes (4 bits) | level-3 code << 4 | level-4 code << 6 -> the multipliers of its four level-1
+//      pairs as (half2 values, half2 rounding residuals)
+//   T  index = one byte of level-1 codes (pair a = 2s | pair b = 2s+1 << 4) -> (cos a, cos b), (sin a, sin b) in fp16: a half2
+//      (u_a, u_b) of the table above multiplies them element-wise; where they are not exact enough, the fp16 rounding residuals too
+// replicated so that the lanes that read together read their own banks (16 copies of 8-byte entries, 8 of 16-byte ones).  Bound by
+// the shared-memory pipe and by instruction issue together, so a lookup's work is what counts: index bytes are put together four
+// at a time, a row of both tables is 256 bytes, so that one byte permute makes an address, and the analytic codebook needs no
+// residuals at level 1 and one half's multipliers (kFlagExactDecode).  One lookup per 4-coordinate sub-block at level 2..4, residuals
+// at level 1 and shift-and-mask addresses took 770 instructions and 210 shared-memory wavefronts per tile (8 x 32768 tokens,
+// 32/8 heads: 141.4 us); this 119.5 us, one sequence of 131072 78.4 -> 67.5.  The rows and tcgen05 kernels keep a table
+// per sub-block (u [4][64][16], t1hi and t1lo [256][16]): the first is bound by its start and end and the MMAs of its rows, the second
+// has no room for rows of 256 bytes; leaving out the residuals there gave 0.2 and 0.5 %.
 // Values use the fp16 parts only.  Keys feed the softmax exponent, where an fp16-rounded operand
 // costs ~3x its relative error in the output, so they are decoded as an unevaluated sum hi + lo
 // (error-free fp16 transformations with fused multiply-adds) and contracted with two MMAs.
@@ -36,30 +43,42 @@ constexpr int kStageBytes = 4 * kBlockBytes128;     // 15872
 constexpr int kStages = 4;                          // two per group of 8 warps
 constexpr int kSpinLimit = 1 << 22;
 
-// shared-memory map (bytes)
+// Tables per sub-block, of the rows and the tcgen05 kernels, and what lies behind them (bytes from a 32 KB boundary of the shared window,
+// so that a table address is the OR of disjoint bit fields, base | lane replica | index, and needs no addition; a launch without
+// a fixed map asks for 32 KB of slack to place them)
 constexpr int kSmT1p = 0;                             // 256 * 16 * 8 = 32768
 constexpr int kSmT1lo = kSmT1p + 256 * 16 * 8;        // 32768
 constexpr int kSmU = kSmT1lo + 256 * 16 * 8;          // 4 * 64 * 16 * 8 = 32768
 constexpr int kSmBar = kSmU + 4 * 64 * 16 * 8;        // full[4], empty[4] : 64
 constexpr int kSmFlags = kSmBar + 64;                 // abort flag, is_last, n_segs, first_rank : 16
 constexpr int kSmSegs = kSmFlags + 16;                // Segment[32] : 768
+constexpr int kSmAlign = 32768;
+static_assert(kSmT1p == 0 && kSmT1lo == 32768 && kSmU == 65536, "table addresses are formed with OR");
+
 // q (fp32) [8][128], then q' as fp16 values and as fp16 residuals.  A head's q' takes 288 bytes, its quarters (32 coordinates
 // of a fragment lane c) 72 bytes each, and the residuals start 2312 bytes after the values: the 16 lanes of a half-warp
 // (two heads, value or residual, four quarters) then read 16 different bank pairs.
 constexpr int kQHead = 288, kQQuarter = 72, kQLo = 8 * kQHead + 8;
-constexpr int kSmQ = kSmSegs + 768;
-constexpr int kSmRing = (kSmQ + 4096 + kQLo + 8 * kQHead + 127) / 128 * 128;
-// after the main loop the ring is reused for the cross-warp merge: 16 warps x 8 heads x (kMrgStride + 2) floats
 constexpr int kMrgStride = 136;  // floats per (warp, head) row of the merge buffer (136 = 128 + 8: heads 8 banks apart)
-constexpr int kMergeBytes = 16 * 8 * kMrgStride * 4 + 16 * 8 * 2 * 4;
-constexpr int kSmUsed = kSmRing + (kStages * kStageBytes > kMergeBytes ? kStages * kStageBytes : kMergeBytes);
-// The tables start on a 32 KB boundary of the shared window, so that a table address is the OR of
-// disjoint bit fields (base | lane replica | index) and needs no addition; the launch asks for 32 KB
-// of slack to place them.
-constexpr int kSmAlign = 32768;
-constexpr int kSmTotal = kSmUsed + kSmAlign;
-static_assert(kSmT1p == 0 && kSmT1lo == 32768 && kSmU == 65536, "table addresses are formed with OR");
-static_assert(kSmRing % 128 == 0, "ring must be 128-byte aligned");
+
+// ---- shared-memory map of the persistent kernel -------------------------------------------------
+// Its tables have rows of 256 bytes on 64 KB boundaries of the shared window, so that one byte permute of (index bytes, table base)
+// forms a lookup's address: the index byte becomes address byte 1, the base gives the others (byte 0: the lane's replica).  What
+// else the kernel keeps lies around them, at fixed places of the window (dynamic shared memory starts at kWindowBase, which the
+// host asks the device for):
+//   ring | T [256 bytes of level-1 codes]    16 x (cos a, cos b | sin a, sin b) in fp16, then 16 x the residuals of the same
+//        | U [256 half-block codes]          kFlagExactDecode: 8 x (values, residuals) for the keys, then 16 x values for the values;
+//                                            otherwise 8 x (values, residuals) of half 0, then 8 x of half 1
+//        | barriers, segments, q'
+constexpr uint32_t kWindowBase = 1024;
+constexpr uint32_t kFsRing = kWindowBase, kFsT = 0x10000, kFsU = 0x20000, kFsBar = 0x30000;
+constexpr uint32_t kFsFlags = kFsBar + 64, kFsSegs = kFsFlags + 16, kFsQ = kFsSegs + 768;
+constexpr uint32_t kFsEnd = kFsQ + 4096 + kQLo + 8 * kQHead;
+constexpr int kFsTotal = (int)(kFsEnd - kWindowBase);
+// after the main loop the ring is reused for the merge across the warps, four heads at a time: their accumulators, then (m, l)
+constexpr int kFsMergeMl = kFastConsumerWarps * 4 * kMrgStride * 4;
+static_assert(kFsRing + kStages * kStageBytes <= kFsT && kFsMergeMl + kFastConsumerWarps * 8 * 8 <= kStages * kStageBytes, "ring");
+static_assert(kFsTotal <= 227 * 1024, "shared memory of one CTA");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -122,6 +141,12 @@ template <int kOff>
 __device__ __forceinline__ uint2 lds64i(uint32_t addr) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(addr), "n"(kOff));
+  return v;
+}
+template <int kOff>
+__device__ __forceinline__ uint4 lds128i(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr), "n"(kOff));
   return v;
 }
 template <int kOff>
@@ -224,6 +249,83 @@ __device__ __forceinline__ void sub_block_hilo(const BlockRef& b, uint32_t t1, _
   yl = __hfma2(u_hi, as_h2(tl.y), __hfma2(u_lo, as_h2(th.y), __hfma2(u_hi, as_h2(th.y), __hneg2(yh))));
 }
 
+// ---- lookups in tables with 256-byte rows (the persistent kernel's map) --------------------------
+// Byte kByte of `index` as the row of the table with base `base` (a multiple of 64 KB | offset inside a row).
+template <int kByte>
+__device__ __forceinline__ uint32_t row_address(uint32_t index, uint32_t base) {
+  return __byte_perm(index, base, 0x7604 | (kByte << 4));
+}
+// Half-block indices, four to a word: byte = the half's two level-2 codes | level-3 code << 4 | level-4 code << 6; the level-4 code
+// of a second half mirrored (3 - c4) in the exact tables, which hold a first half's entries only.  Each field of a byte is spread by a
+// shift or a multiplication that leaves garbage in the other fields only, and two bitwise selects put the three together.
+// Two blocks of one token -> (block 0: half 0, half 1; block 1: half 0, half 1).  c2: the blocks' level-2 bytes; n3: their level-3
+// nibbles; c4: their level-4 codes in bits 0..3 (garbage above).
+template <bool kExact>
+__device__ __forceinline__ uint32_t half_indices_of_blocks(uint32_t c2, uint32_t n3, uint32_t c4) {
+  const uint32_t f2 = __byte_perm(c2, c2 >> 4, 0x5140);
+  // even fields to bytes 0 and 2, odd ones to bytes 1 and 3; bits 6, 7 of a byte stay clear but for the mirror
+  const uint32_t f3 = (n3 & 0x33u) * 0x10010u + ((n3 & 0xCCu) * 0x400400u + (kExact ? 0xC000C000u : 0u));
+  const uint32_t f4 = (c4 & 0xFu) * 0x10104040u;
+  const uint32_t w = (f2 & 0x0F0F0F0Fu) | (f3 & 0xF0F0F0F0u);
+  return w ^ (f4 & 0xC0C0C0C0u);
+}
+// One block of two tokens -> (token A: half 0, half 1; token B: half 0, half 1).  Bits 0..15 of each argument belong to token A, the
+// others to token B; c2: level-2 byte, n3: level-3 nibble, c4: level-4 code in bits 0..1 (garbage above, but n3 and c4 may be garbage).
+template <bool kExact>
+__device__ __forceinline__ uint32_t half_indices_of_tokens(uint32_t c2, uint32_t n3, uint32_t c4) {
+  const uint32_t f2 = (c2 & 0x000F000Fu) | ((c2 << 4) & 0x0F000F00u);
+  const uint32_t f3 = (n3 & 0x000F000Fu) * 0x410u;
+  const uint32_t f4 = kExact ? (c4 & 0x00030003u) * (64u - 16384u) + 0xC000C000u : (c4 & 0x00030003u) * (64u + 16384u);
+  const uint32_t w = f2 | (f3 & 0x30303030u);
+  return w | f4;
+}
+// Half kByte & 1 of a key block (byte kByte of `index`; level-1 bytes kL1, kL1 + 1 of `l1`) as unevaluated sums hi + lo, see
+// sub_block_hilo.  With the exact tables the level-1 factors have no residual.
+struct KeyHalf {
+  __half2 xh[2], yh[2], xl[2], yl[2];
+};
+template <bool kExact, int kByte, int kL1>
+__device__ __forceinline__ void decode_key_half(uint32_t index, uint32_t l1, __half2 r2, uint32_t uk, uint32_t t, KeyHalf& k) {
+  const uint4 uu = lds128i<!kExact && (kByte & 1) ? 128 : 0>(row_address<kByte>(index, uk));
+  const uint32_t ta[2] = {row_address<kL1>(l1, t), row_address<kL1 + 1>(l1, t)};
+  const uint32_t uh[2] = {uu.x, uu.y}, ul[2] = {uu.z, uu.w};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint2 th = lds64i<0>(ta[i]);
+    const __half2 u_hi = __hmul2(r2, as_h2(uh[i]));
+    const __half2 u_lo = __hfma2(r2, as_h2(ul[i]), __hfma2(r2, as_h2(uh[i]), __hneg2(u_hi)));
+    k.xh[i] = __hmul2(u_hi, as_h2(th.x));
+    k.yh[i] = __hmul2(u_hi, as_h2(th.y));
+    k.xl[i] = __hfma2(u_lo, as_h2(th.x), __hfma2(u_hi, as_h2(th.x), __hneg2(k.xh[i])));
+    k.yl[i] = __hfma2(u_lo, as_h2(th.y), __hfma2(u_hi, as_h2(th.y), __hneg2(k.yh[i])));
+    if (!kExact) {
+      const uint2 tl = lds64i<128>(ta[i]);
+      k.xl[i] = __hfma2(u_hi, as_h2(tl.x), k.xl[i]);
+      k.yl[i] = __hfma2(u_hi, as_h2(tl.y), k.yl[i]);
+    }
+  }
+}
+// The multipliers u = r U of half kByte & 1 of a value block.
+template <bool kExact, int kByte>
+__device__ __forceinline__ void value_half(uint32_t index, __half2 r2, uint32_t uv, __half2* u) {
+  const uint2 uu = lds64i<!kExact && (kByte & 1) ? 128 : 0>(row_address<kByte>(index, uv));
+  u[0] = __hmul2(r2, as_h2(uu.x));
+  u[1] = __hmul2(r2, as_h2(uu.y));
+}
+template <int kByte>
+__device__ __forceinline__ void value_sub_block(__half2 u, uint32_t l1, uint32_t t, __half2& x, __half2& y) {
+  const uint2 e = lds64i<0>(row_address<kByte>(l1, t));
+  x = __hmul2(u, as_h2(e.x));
+  y = __hmul2(u, as_h2(e.y));
+}
+// Two 8 x 8 matrices of 16-bit elements, transposed: lane (g, c) gets element g of rows 2c and 2c + 1 of each; lanes 0..7
+// and 8..15 give the rows' addresses.
+__device__ __forceinline__ uint2 ldmatrix2_trans(uint32_t row) {
+  uint2 v;
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(row));
+  return v;
+}
+
 // plane offsets of a d = 128 token-block
 constexpr int kO2 = 32 * kTokenBlock, kO3 = kO2 + 8 * kTokenBlock, kO4 = kO3 + 4 * kTokenBlock,
               kORad = kO4 + 2 * kTokenBlock;
@@ -252,6 +354,41 @@ __device__ __forceinline__ void build_fast_tables(uint8_t* smem, const Tables* t
     t1lo[i] = v[kPer + r];
     u[i] = v[2 * kPer + r];
   }
+}
+
+// The same for the map with 256-byte rows (`window`: start of the shared window).  Returns whether the tables are exact ones.
+template <int kThreads>
+__device__ __forceinline__ bool build_row_tables(uint8_t* window, const Tables* tb) {
+  const int row0 = threadIdx.x >> 4, rep = threadIdx.x & 15;   // 16 threads per row
+  constexpr int kPer = 256 * 16 / kThreads, kStep = kThreads / 16;
+  const bool exact = (tb->flags & kFlagExactDecode) != 0;
+  // entry i of half h: sub-blocks 2h and 2h + 1 at their level-2 codes (bits 0..1 and 2..3 of i) and the codes above, common to both
+  auto pair = [&](int h, int i) {
+    const uint2 lo = tb->u_tab[2 * h][(i & 3) | (i >> 2 & ~3)], hi = tb->u_tab[2 * h + 1][i >> 2];
+    return make_uint4(lo.x, hi.x, lo.y, hi.y);
+  };
+  uint2 th[kPer];
+  uint4 up[kPer];
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    th[r] = tb->t1p_hi[row0 + r * kStep];
+    up[r] = pair(0, row0 + r * kStep);
+  }
+  uint8_t* t = window + kFsT + row0 * 256;
+  uint8_t* u = window + kFsU + row0 * 256;
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    *reinterpret_cast<uint2*>(t + r * kStep * 256 + rep * 8) = th[r];
+    if (rep < 8) *reinterpret_cast<uint4*>(u + r * kStep * 256 + rep * 16) = up[r];
+    if (exact) *reinterpret_cast<uint2*>(u + r * kStep * 256 + 128 + rep * 8) = make_uint2(up[r].x, up[r].y);
+  }
+  if (!exact)
+#pragma unroll 1
+    for (int r = 0; r < kPer; ++r) {
+      *reinterpret_cast<uint2*>(t + r * kStep * 256 + 128 + rep * 8) = tb->t1p_lo[row0 + r * kStep];
+      if (rep < 8) *reinterpret_cast<uint4*>(u + r * kStep * 256 + 128 + rep * 16) = pair(1, row0 + r * kStep);
+    }
+  return exact;
 }
 
 // Slots of split partials for the persistent kernel: every unit (sequence, kv head) has one slot
@@ -408,7 +545,7 @@ __device__ __forceinline__ float sum_eight_rows(const float* v, int lane) {
 // the rows of S, the first partial outputs of a thread's coordinates and the (m, l) pairs are all requested before
 // anything waits.  `sm`: kCombineFloats floats.
 constexpr int kCombineFloats = 8 * kFastMaxGrid + 8 + 8 * 128;
-static_assert(kCombineFloats * 4 <= kMergeBytes, "the combine uses the merge buffer");
+static_assert(kCombineFloats * 4 <= kStages * kStageBytes, "the combine uses the ring");
 template <int kHG>
 __device__ __forceinline__ void combine_and_store(const DecodeArgs& a, int b, int hk, int g, int slot0, int ns, float* sm) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -526,18 +663,18 @@ __device__ __forceinline__ void elect_combiner(const DecodeArgs& a, int u, int u
 template <int kHG, bool kPaged>
 __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + ((kSmAlign - (smem_u32(smem_raw) & (kSmAlign - 1))) & (kSmAlign - 1));
+  uint8_t* smem = smem_raw - kWindowBase;   // the shared window; see the map
   const int g_heads = a.n_q_heads / a.n_kv_heads;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t sm_base = smem_u32(smem);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kSmFlags);
-  int* is_last = reinterpret_cast<int*>(smem + kSmFlags) + 1;
+  const uint32_t sm_base = smem_u32(smem_raw) - kWindowBase;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kFsFlags);
+  int* is_last = reinterpret_cast<int*>(smem + kFsFlags) + 1;
   const int64_t head_bytes = make_layout(128, a.pg.page_tokens).head_bytes;
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(sm_base + kSmBar + 8 * s, 1);                                  // full: producer + tx bytes
-      mbar_init(sm_base + kSmBar + 8 * (kStages + s), kFastConsumerWarps / 2);  // empty: one arrive per warp of the group
+      mbar_init(sm_base + kFsBar + 8 * s, 1);                                  // full: producer + tx bytes
+      mbar_init(sm_base + kFsBar + 8 * (kStages + s), kFastConsumerWarps / 2);  // empty: one arrive per warp of the group
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -546,7 +683,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   // while that kernel finishes; its results (lengths, cache, queries, workspace) are read only after this wait.
   // The kernel after this one may be set up as soon as this grid has started.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  build_fast_tables<kFastThreads>(smem, a.tables);   // from the caller's tables, which no kernel writes
+  const bool exact = build_row_tables<kFastThreads>(smem, a.tables);   // from the caller's tables, which no kernel writes
   // What this thread needs of S (constant too) to rotate the queries: column warp * 8 + lane / 4, rows 16 i + 4 (lane & 3)
   // + 0..3 -- a warp's load covers whole 32-byte sectors, and four lanes share a column's sum.
   const int rot_j = warp * 8 + (lane >> 2), rot_k = (lane & 3) * 4;
@@ -562,9 +699,9 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   __syncthreads();
 
   const int n_units = a.batch * a.n_kv_heads, cta = blockIdx.x;   // the work split: see list_segments
-  Segment* segs = reinterpret_cast<Segment*>(smem + kSmSegs);
-  int* n_segs = reinterpret_cast<int*>(smem + kSmFlags) + 2;   // units of this CTA (all batches of the list)
-  int* first_rank = reinterpret_cast<int*>(smem + kSmFlags) + 3;
+  Segment* segs = reinterpret_cast<Segment*>(smem + kFsSegs);
+  int* n_segs = reinterpret_cast<int*>(smem + kFsFlags) + 2;   // units of this CTA (all batches of the list)
+  int* first_rank = reinterpret_cast<int*>(smem + kFsFlags) + 3;
   // Stages of unit u (0 past the last one).
   auto stages_of = [&](int u) -> int {
     const int len_u = u < n_units ? a.visible_len(u / a.n_kv_heads) : 0;
@@ -584,11 +721,12 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       set_status(a.status, PQ_ERR_EMPTY);
   };
   auto build_segments = [&](int batch_no) -> int {
-    return list_segments<kFastThreads>(batch_no, n_units, smem + kSmRing, segs, n_segs, first_rank, stages_of, empty_unit);
+    return list_segments<kFastThreads>(batch_no, n_units, smem + kFsRing, segs, n_segs, first_rank, stages_of, empty_unit);
   };
   const int g = lane >> 2, c = lane & 3;
-  const uint32_t rep = (lane & 15) * 8;
-  const uint32_t ua = sm_base + kSmU + rep, t1a = sm_base + kSmT1p + rep;  // table base | lane replica
+  // table base | lane replica; the value multipliers are the high parts of the keys' entries where the tables are not exact
+  const uint32_t t1a = sm_base + kFsT + (lane & 15) * 8, uk = sm_base + kFsU + (lane & 7) * 16;
+  const uint32_t uv = exact ? sm_base + kFsU + 128 + (lane & 15) * 8 : uk;
   const int wg = warp >> 3;  // group of 8 warps
   // Offsets, inside a token-block, of what this thread reads of its tile (16 tokens from token (warp & 3) * 16).
   // Keys: tokens g and g + 8, blocks 2c and 2c + 1.  Values: block g of tokens c, c + 4, c + 8, c + 12 (these are
@@ -597,7 +735,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   const int tk_k = (warp & 3) * 16 + (lane >> 2), tk_v = (warp & 3) * 16 + (lane & 3);
   const uint32_t ok_l1 = tk_k * 32 + (lane & 3) * 8, ok_r = kORad + tk_k * 16 + (lane & 3) * 4;
   const uint32_t ok_c2 = kO2 + tk_k * 8 + (lane & 3) * 2, ok_c3 = kO3 + tk_k * 4 + (lane & 3), ok_c4 = kO4 + tk_k * 2;
-  const uint32_t ov_l1 = tk_v * 32 + (lane >> 2) * 4, ov_r = kORad + tk_v * 16 + (lane >> 2) * 2;
+  const uint32_t ov_l1 = tk_v * 32 + (lane >> 2) * 4, ov_r = kORad + ((warp & 3) * 16 + ((lane >> 1) & 3) + 4 * (lane & 1) + (lane & 8)) * 16;   // rows for ldmatrix2_trans
   const uint32_t ov_c2 = kO2 + tk_v * 8 + (lane >> 2), ov_c3 = kO3 + tk_v * 4 + (lane >> 3), ov_c4 = kO4 + tk_v * 2;
   int gl0 = 0;               // stages this group has streamed so far (ring slot and barrier phase bookkeeping)
 
@@ -635,11 +773,11 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     int issued = 0;
     auto issue_copy = [&](int li) -> bool {
       const int gl = gl0 + li, s = 2 * wg + (gl & 1);
-      if (gl >= 2 && !mbar_wait(sm_base + kSmBar + 8 * (kStages + s), ((gl >> 1) - 1) & 1, abort_flag)) return false;
+      if (gl >= 2 && !mbar_wait(sm_base + kFsBar + 8 * (kStages + s), ((gl >> 1) - 1) & 1, abort_flag)) return false;
       const int st = st0 + wg + 2 * li;
       const int nblk = min(2, nblk_total - 2 * st);
       const uint32_t bytes = nblk * 2 * kBlockBytes128;
-      mbar_expect_tx(sm_base + kSmBar + 8 * s, bytes);
+      mbar_expect_tx(sm_base + kFsBar + 8 * s, bytes);
       // a stage is two token-blocks, K | V | K | V, of one page (page_tokens is a multiple of 128)
       const uint8_t* src = head_base + (int64_t)st * kStageBytes;
       if (kPaged) {
@@ -648,7 +786,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
         Lp.head_bytes = head_bytes;
         src = a.cache + kv_block_pair_offset(Lp, a.pg, a.n_kv_heads, seq, hk, 2 * st, a.status);
       }
-      bulk_load(sm_base + kSmRing + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
+      bulk_load(sm_base + kFsRing + s * kStageBytes, src, bytes, sm_base + kFsBar + 8 * s);
       issued = li + 1;
       return true;
     };
@@ -664,8 +802,8 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     // q' = (q S) * scale * log2(e) for the unit's query heads, as an fp16 value plus an fp16 residual.
     // The first stages of the segment are already on their way while this runs.
     {
-      float* q_in = reinterpret_cast<float*>(smem + kSmQ);
-      __half* q_hi = reinterpret_cast<__half*>(smem + kSmQ + 4096) + (rot_j >> 5) * (kQQuarter / 2) + (rot_j & 31);
+      float* q_in = reinterpret_cast<float*>(smem + kFsQ);
+      __half* q_hi = reinterpret_cast<__half*>(smem + kFsQ + 4096) + (rot_j >> 5) * (kQQuarter / 2) + (rot_j & 31);
       const int64_t q0 = ((int64_t)b * a.n_q_heads + hk * g_heads) * 128;
       for (int i = tid; i < g_heads * 128; i += kFastThreads)
         q_in[i] = a.io_dtype == PQ_DTYPE_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.q)[q0 + i])
@@ -702,7 +840,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
 #pragma unroll
     for (int hg = 0; hg < kHG; ++hg) {
       const int h = (g >> 1) + 4 * hg;
-      const uint2* qsrc = reinterpret_cast<const uint2*>(smem + kSmQ + 4096 + (g & 1) * kQLo + h * kQHead + c * kQQuarter);
+      const uint2* qsrc = reinterpret_cast<const uint2*>(smem + kFsQ + 4096 + (g & 1) * kQLo + h * kQHead + c * kQQuarter);
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         uint2 v = make_uint2(0u, 0u);
@@ -712,12 +850,14 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
         qb[hg][ks][1] = __byte_perm(v.x, v.y, 0x7632);
       }
     }
+    auto stream = [&](auto exact_tables) {
+    constexpr bool kExact = decltype(exact_tables)::value;
     for (int li = 0; li < n_li; ++li) {
       const int gl = gl0 + li, s = 2 * wg + (gl & 1);
       const int st = st0 + wg + 2 * li;
       if (producer && li + 1 < n_li) issue_copy(li + 1);
       __syncwarp();
-      if (!mbar_wait(sm_base + kSmBar + 8 * s, (gl >> 1) & 1, abort_flag)) break;
+      if (!mbar_wait(sm_base + kFsBar + 8 * s, (gl >> 1) & 1, abort_flag)) break;
       if ((kPaged ? (a.debug & 1u) && unit_slot == 0 && cta == c_first : hook) && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
         // that starts the first non-empty unit is reported as failed
         *abort_flag = 1;
@@ -725,7 +865,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       }
       const int tile_tok0 = st * kStageTokens + (warp & 7) * 16;  // first token of this warp's 16-token tile
       if (tile_tok0 < len) {
-        const uint32_t kblk = sm_base + kSmRing + s * kStageBytes + ((warp >> 2) & 1) * 2 * kBlockBytes128;
+        const uint32_t kblk = sm_base + kFsRing + s * kStageBytes + ((warp >> 2) & 1) * 2 * kBlockBytes128;
         const uint32_t vblk = kblk + kBlockBytes128;
         // ---- scores S (tokens x columns): A operand = keys of tokens g (rows 0..7) and g + 8 (rows 8..15),
         // decoded as hi + lo; one MMA with the hi parts and one with the lo parts per k-step.  Column 2c is
@@ -736,47 +876,46 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
 #pragma unroll
           for (int i = 0; i < 4; ++i) sc[hg][i] = scl[hg][i] = 0.f;
         {
-          const uint2 l1A = lds64i<0>(kblk + ok_l1), l1B = lds64i<8 * 32>(kblk + ok_l1);
+          const uint2 l1pA = lds64i<0>(kblk + ok_l1), l1pB = lds64i<8 * 32>(kblk + ok_l1);
           const uint32_t rrA = lds32i<0>(kblk + ok_r), rrB = lds32i<8 * 16>(kblk + ok_r);
           const uint32_t c2A = lds16i<0>(kblk + ok_c2), c2B = lds16i<8 * 8>(kblk + ok_c2);
           const uint32_t c3A = lds8i<0>(kblk + ok_c3), c3B = lds8i<8 * 4>(kblk + ok_c3);
           const uint32_t c4A = lds16i<0>(kblk + ok_c4) >> (4 * c), c4B = lds16i<8 * 2>(kblk + ok_c4) >> (4 * c);
-#define PQ_KSTEP(H, S)                                                                                    \
-  {                                                                                                       \
-    __half2 xhA, yhA, xlA, ylA, xhB, yhB, xlB, ylB;                                                       \
-    sub_block_hilo<S>(bA, t1a, xhA, yhA, xlA, ylA);                                                       \
-    sub_block_hilo<S>(bB, t1a, xhB, yhB, xlB, ylB);                                                       \
-    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                                                  \
-      mma_16816(scl[hg], as_u32(xlA), as_u32(xlB), as_u32(ylA), as_u32(ylB), qb[hg][4 * (H) + (S)][0],    \
-                qb[hg][4 * (H) + (S)][1]);                                                                \
-      mma_16816(sc[hg], as_u32(xhA), as_u32(xhB), as_u32(yhA), as_u32(yhB), qb[hg][4 * (H) + (S)][0],     \
-                qb[hg][4 * (H) + (S)][1]);                                                                \
-    }                                                                                                     \
+#define PQ_KHALF(INDEX, L1, R2, H, HALF)                                                                                \
+  {                                                                                                                     \
+    KeyHalf kA, kB;                                                                                                     \
+    decode_key_half<kExact, 2 * (H) + (HALF), 2 * (HALF)>(INDEX##A, L1##A, R2(as_h2(rrA)), uk, t1a, kA);                \
+    decode_key_half<kExact, 2 * (H) + (HALF), 2 * (HALF)>(INDEX##B, L1##B, R2(as_h2(rrB)), uk, t1a, kB);                \
+    _Pragma("unroll") for (int i = 0; i < 2; ++i) _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                  \
+      const uint32_t* qv = qb[hg][4 * (H) + 2 * (HALF) + i];                                                            \
+      mma_16816(scl[hg], as_u32(kA.xl[i]), as_u32(kB.xl[i]), as_u32(kA.yl[i]), as_u32(kB.yl[i]), qv[0], qv[1]);         \
+      mma_16816(sc[hg], as_u32(kA.xh[i]), as_u32(kB.xh[i]), as_u32(kA.yh[i]), as_u32(kB.yh[i]), qv[0], qv[1]);          \
+    }                                                                                                                   \
   }
-          {
-            const BlockRef bA = make_block_ref(l1A.x, c2A, c3A, c4A & 3u, __low2half2(as_h2(rrA)), ua);
-            const BlockRef bB = make_block_ref(l1B.x, c2B, c3B, c4B & 3u, __low2half2(as_h2(rrB)), ua);
-            PQ_KSTEP(0, 0) PQ_KSTEP(0, 1) PQ_KSTEP(0, 2) PQ_KSTEP(0, 3)
-          }
-          {
-            const BlockRef bA = make_block_ref(l1A.y, c2A >> 8, c3A >> 4, (c4A >> 2) & 3u, __high2half2(as_h2(rrA)), ua);
-            const BlockRef bB = make_block_ref(l1B.y, c2B >> 8, c3B >> 4, (c4B >> 2) & 3u, __high2half2(as_h2(rrB)), ua);
-            PQ_KSTEP(1, 0) PQ_KSTEP(1, 1) PQ_KSTEP(1, 2) PQ_KSTEP(1, 3)
-          }
-#undef PQ_KSTEP
+          const uint32_t ixA = half_indices_of_blocks<kExact>(c2A, c3A, c4A), ixB = half_indices_of_blocks<kExact>(c2B, c3B, c4B);
+          const uint32_t l1A = l1pA.x, l1B = l1pB.x, l1hA = l1pA.y, l1hB = l1pB.y;
+          PQ_KHALF(ix, l1, __low2half2, 0, 0)
+          PQ_KHALF(ix, l1, __low2half2, 0, 1)
+          PQ_KHALF(ix, l1h, __high2half2, 1, 0)
+          PQ_KHALF(ix, l1h, __high2half2, 1, 1)
+#undef PQ_KHALF
         }
         // ---- online softmax: this thread holds head c (+ 4 hg) of tokens g and g + 8.  The reference m_run of a
         // head moves only when a score exceeds it by more than kLazyMax (log2 units), so p = 2^(s - m_run) stays
         // below 2^kLazyMax (fp16 holds it with its full relative precision) and the common tile needs neither
         // the reductions over tokens nor a rescaling; l_run is this thread's share of the denominator (its own
         // tokens), summed over the eight lanes of the head when the segment ends.
-        const bool ok0 = tile_tok0 + g < len, ok1 = tile_tok0 + g + 8 < len;
+        const bool whole = tile_tok0 + 16 <= len;
         float s0[kHG], s1[kHG];
         bool over = false;
 #pragma unroll
         for (int hg = 0; hg < kHG; ++hg) {
-          s0[hg] = ok0 ? (scl[hg][0] + scl[hg][1]) + sc[hg][1] + sc[hg][0] : -CUDART_INF_F;  // small terms first
-          s1[hg] = ok1 ? (scl[hg][2] + scl[hg][3]) + sc[hg][3] + sc[hg][2] : -CUDART_INF_F;
+          s0[hg] = (scl[hg][0] + scl[hg][1]) + sc[hg][1] + sc[hg][0];  // small terms first
+          s1[hg] = (scl[hg][2] + scl[hg][3]) + sc[hg][3] + sc[hg][2];
+          if (!whole) {   // the last tile of the sequence: what lies past its end may be anything
+            if (tile_tok0 + g >= len) s0[hg] = -CUDART_INF_F;
+            if (tile_tok0 + g + 8 >= len) s1[hg] = -CUDART_INF_F;
+          }
           over = over || fmaxf(s0[hg], s1[hg]) > m_run[hg] + kLazyMax;  // always on the first tile (m_run = -inf)
         }
         if (__any_sync(0xffffffffu, over)) {
@@ -826,38 +965,52 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
         }
         // ---- values: block g of tokens c, c+4, c+8, c+12 -> O^T (coordinates x (head, element)) += V_hat^T P
         {
-          BlockRef bv[4];
-#define PQ_VLOAD(J)                                                                                          \
-  {                                                                                                          \
-    const uint32_t l1 = lds32i<4 * (J) * 32>(vblk + ov_l1);                                                  \
-    uint32_t rr = lds16i<4 * (J) * 16>(vblk + ov_r);                                                         \
-    const uint32_t c2 = lds8i<4 * (J) * 8>(vblk + ov_c2);                                                    \
-    const uint32_t c3 = lds8i<4 * (J) * 4>(vblk + ov_c3) >> (4 * (g & 1));                                   \
-    const uint32_t c4 = lds16i<4 * (J) * 2>(vblk + ov_c4) >> (2 * g);                                        \
-    if (tile_tok0 + c + 4 * (J) >= len) rr = 0u; /* stale bytes past the sequence end stay out of the sums */ \
-    bv[J] = make_block_ref(l1, c2, c3, c4 & 3u, as_h2(rr | (rr << 16)), ua);                                 \
+          const uint32_t l1v[4] = {lds32i<0>(vblk + ov_l1), lds32i<4 * 32>(vblk + ov_l1), lds32i<8 * 32>(vblk + ov_l1), lds32i<12 * 32>(vblk + ov_l1)};
+          uint2 rr = ldmatrix2_trans(vblk + ov_r);   // radii of tokens c | c + 4 and c + 8 | c + 12
+          // codes of two tokens in one word
+          const uint32_t c2v[2] = {lds8i<0>(vblk + ov_c2) | lds8i<4 * 8>(vblk + ov_c2) << 16, lds8i<8 * 8>(vblk + ov_c2) | lds8i<12 * 8>(vblk + ov_c2) << 16};
+          const uint32_t c3v[2] = {lds8i<0>(vblk + ov_c3) | lds8i<4 * 4>(vblk + ov_c3) << 16, lds8i<8 * 4>(vblk + ov_c3) | lds8i<12 * 4>(vblk + ov_c3) << 16};
+          const uint32_t c4v[2] = {lds16i<0>(vblk + ov_c4) | lds16i<4 * 2>(vblk + ov_c4) << 16, lds16i<8 * 2>(vblk + ov_c4) | lds16i<12 * 2>(vblk + ov_c4) << 16};
+          if (!whole) {   // stale bytes past the sequence end stay out of the sums
+            const int left = len - tile_tok0 - c;   // token c + 4 j is inside if 4 j < left
+            rr.x = left > 4 ? rr.x : left > 0 ? rr.x & 0xFFFFu : 0u;
+            rr.y = left > 12 ? rr.y : left > 8 ? rr.y & 0xFFFFu : 0u;
+          }
+          uint32_t ixv[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) ixv[j] = half_indices_of_tokens<kExact>(c2v[j], c3v[j] >> (4 * (g & 1)), c4v[j] >> (2 * g));
+#define PQ_VHALF(HALF)                                                                                   \
+  {                                                                                                      \
+    __half2 u0[2], u1[2], u2[2], u3[2];                                                                  \
+    value_half<kExact, (HALF)>(ixv[0], __low2half2(as_h2(rr.x)), uv, u0);                                \
+    value_half<kExact, 2 + (HALF)>(ixv[0], __high2half2(as_h2(rr.x)), uv, u1);                           \
+    value_half<kExact, (HALF)>(ixv[1], __low2half2(as_h2(rr.y)), uv, u2);                                \
+    value_half<kExact, 2 + (HALF)>(ixv[1], __high2half2(as_h2(rr.y)), uv, u3);                           \
+    PQ_VSTEP(2 * (HALF), 0) PQ_VSTEP(2 * (HALF) + 1, 1)                                                  \
   }
-          PQ_VLOAD(0) PQ_VLOAD(1) PQ_VLOAD(2) PQ_VLOAD(3)
-#undef PQ_VLOAD
-#define PQ_VSTEP(S)                                                                                      \
+#define PQ_VSTEP(S, I)                                                                                   \
   {                                                                                                      \
     __half2 x0, y0, x1, y1, x2, y2, x3, y3;                                                              \
-    sub_block_h2<S>(bv[0], t1a, x0, y0);                                                                 \
-    sub_block_h2<S>(bv[1], t1a, x1, y1);                                                                 \
-    sub_block_h2<S>(bv[2], t1a, x2, y2);                                                                 \
-    sub_block_h2<S>(bv[3], t1a, x3, y3);                                                                 \
+    value_sub_block<S>(u0[I], l1v[0], t1a, x0, y0);                                                      \
+    value_sub_block<S>(u1[I], l1v[1], t1a, x1, y1);                                                      \
+    value_sub_block<S>(u2[I], l1v[2], t1a, x2, y2);                                                      \
+    value_sub_block<S>(u3[I], l1v[3], t1a, x3, y3);                                                      \
     _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                                                 \
       mma_16816(o_acc[hg][S], as_u32(x0), as_u32(y0), as_u32(x1), as_u32(y1), pb[hg][0][0], pb[hg][0][1]); \
       mma_16816(o_acc[hg][S], as_u32(x2), as_u32(y2), as_u32(x3), as_u32(y3), pb[hg][1][0], pb[hg][1][1]); \
     }                                                                                                    \
   }
-          PQ_VSTEP(0) PQ_VSTEP(1) PQ_VSTEP(2) PQ_VSTEP(3)
+          PQ_VHALF(0) PQ_VHALF(1)
+#undef PQ_VHALF
 #undef PQ_VSTEP
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(sm_base + kSmBar + 8 * (kStages + s));
+      if (lane == 0) mbar_arrive(sm_base + kFsBar + 8 * (kStages + s));
     }
+    };
+    if (exact) stream(std::true_type{});
+    else stream(std::false_type{});
     gl0 += n_li;
     __syncthreads();  // every copy that was consumed is done with; the rest is waited for below
     if (*abort_flag) {
@@ -865,17 +1018,17 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       if (producer)
         for (int li = max(0, issued - 2); li < issued; ++li) {
           const int gl = gl0 - n_li + li;
-          for (int i = 0; i < kSpinLimit && !mbar_try_wait(sm_base + kSmBar + 8 * (2 * wg + (gl & 1)), (gl >> 1) & 1); ++i)
+          for (int i = 0; i < kSpinLimit && !mbar_try_wait(sm_base + kFsBar + 8 * (2 * wg + (gl & 1)), (gl >> 1) & 1); ++i)
             __nanosleep(64);
         }
       __syncthreads();
     }
 
     // ---- merge the 16 warps (fixed order), write this part's partial, last part combines the unit
-    // Coordinate j of head h of warp w sits at (w * 8 + h) * kMrgStride + (j & 15) * 8 + (j >> 4): for a fixed
+    // Coordinate j of head h (of four) of warp w sits at (w * 4 + h) * kMrgStride + (j & 15) * 8 + (j >> 4): for a fixed
     // accumulator register the 32 lanes (block g, head c) then hit 32 different banks.
-    float* mrg_o = reinterpret_cast<float*>(smem + kSmRing);          // [16 warps][8 heads][kMrgStride]
-    float* mrg_ml = mrg_o + kFastConsumerWarps * 8 * kMrgStride;      // [16 warps][8 heads][2]
+    float* mrg_o = reinterpret_cast<float*>(smem + kFsRing);                  // [16 warps][4 heads][kMrgStride]
+    float* mrg_ml = reinterpret_cast<float*>(smem + kFsRing + kFsMergeMl);    // [16 warps][8 heads][2]
 #pragma unroll
     for (int hg = 0; hg < kHG; ++hg) {  // the head's denominator: sum of the shares of its eight lanes
       l_run[hg] += __shfl_xor_sync(0xffffffffu, l_run[hg], 4);
@@ -888,23 +1041,6 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
         *reinterpret_cast<float2*>(mrg_ml + (warp * 8 + c + 4 * hg) * 2) = make_float2(m_run[hg], l_run[hg]);
     }
     __syncthreads();
-    // every warp brings its accumulators to the common reference before it hands them over
-#pragma unroll
-    for (int hg = 0; hg < kHG; ++hg)
-      if (c + 4 * hg < g_heads) {
-        float M = -CUDART_INF_F;
-#pragma unroll
-        for (int w = 0; w < kFastConsumerWarps; ++w) M = fmaxf(M, mrg_ml[(w * 8 + c + 4 * hg) * 2]);
-        const float wgt = m_run[hg] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[hg] - M);
-        float* o0 = mrg_o + (warp * 8 + c + 4 * hg) * kMrgStride + g;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          o0[(4 * i) * 8] = o_acc[hg][i][0] * wgt;
-          o0[(4 * i + 2) * 8] = o_acc[hg][i][1] * wgt;
-          o0[(4 * i + 1) * 8] = o_acc[hg][i][2] * wgt;
-          o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
-        }
-      }
     // In the contiguous instantiation the segment is read again (and through volatile, so that it really is): the registers that its
     // fields would hold through the tile loop cost that loop 2 % (8 x 131072 tokens: 516 -> 507 us).  In the paged one it is
     // the other way round (16 ragged sequences of up to 65536 tokens, four steps: 1313 us, 1365 with the fields read again).  That is
@@ -932,14 +1068,30 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       for (int o = 8; o > 0; o >>= 1) l += __shfl_xor_sync(half, l, o);
       if ((tid & 15) == 0) __stcg(reinterpret_cast<float2*>(a.ws.ml) + (int64_t)slot * g_heads + h, make_float2(M, l));
     }
-    __syncthreads();
+    // every warp brings its accumulators to the common reference before it hands them over
 #pragma unroll
-    for (int r = 0; r < kHG; ++r) {
-      const int idx = tid + r * kFastThreads, h = idx >> 7, j = idx & 127;
+    for (int hg = 0; hg < kHG; ++hg) {
+      if (hg > 0) __syncthreads();   // the four heads before these have been read
+      if (c + 4 * hg < g_heads) {
+        float M = -CUDART_INF_F;
+#pragma unroll
+        for (int w = 0; w < kFastConsumerWarps; ++w) M = fmaxf(M, mrg_ml[(w * 8 + c + 4 * hg) * 2]);
+        const float wgt = m_run[hg] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[hg] - M);
+        float* o0 = mrg_o + (warp * 4 + c) * kMrgStride + g;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          o0[(4 * i) * 8] = o_acc[hg][i][0] * wgt;
+          o0[(4 * i + 2) * 8] = o_acc[hg][i][1] * wgt;
+          o0[(4 * i + 1) * 8] = o_acc[hg][i][2] * wgt;
+          o0[(4 * i + 3) * 8] = o_acc[hg][i][3] * wgt;
+        }
+      }
+      __syncthreads();
+      const int h = (tid >> 7) + 4 * hg, j = tid & 127;
       if (h < g_heads) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int w = 0; w < kFastConsumerWarps; ++w) acc[w & 3] += mrg_o[(w * 8 + h) * kMrgStride + (j & 15) * 8 + (j >> 4)];
+        for (int w = 0; w < kFastConsumerWarps; ++w) acc[w & 3] += mrg_o[(w * 4 + (tid >> 7)) * kMrgStride + (j & 15) * 8 + (j >> 4)];
         __stcg(a.ws.o + ((int64_t)slot * g_heads + h) * 128 + j, (acc[0] + acc[1]) + (acc[2] + acc[3]));
       }
     }
@@ -947,7 +1099,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     if (warp == 0) elect_combiner(a, done.unit, done.slot0, done.part, done.n_parts, lane, is_last);
     __syncthreads();
     if (*is_last) {
-      combine_and_store<kHG>(a, done.b, done.hk, g_heads, done.slot0, done.n_parts, reinterpret_cast<float*>(smem + kSmRing));
+      combine_and_store<kHG>(a, done.b, done.hk, g_heads, done.slot0, done.n_parts, reinterpret_cast<float*>(smem + kFsRing));
       if (tid == 0 && done.n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + done.unit) = 0u;
     }
     __syncthreads();  // the ring is free again for the next unit

@@ -466,7 +466,13 @@ int32_t pq_build_tables(const double* cen, const double* bnd, void* tables_host)
     *hi = h2(va, vb);
     *lo = h2(va - ha, vb - hb);
   };
-  for (int c = 0; c < 16; ++c) split(std::cos(cen[c]), std::sin(cen[c]), &t.l1_hi[c], &t.l1_lo[c]);
+  double l1_scale = pq::kL1Scale;   // 1 if it does not bring every level-1 factor close to an fp16 value
+  for (int c = 0; c < 16; ++c)
+    for (const double f : {std::cos(cen[c]), std::sin(cen[c])}) {
+      const double v = f * pq::kL1Scale;
+      if (!(std::fabs((double)__half2float(__double2half(v)) - v) <= std::ldexp(std::fabs(v), -16))) l1_scale = 1.0;
+    }
+  for (int c = 0; c < 16; ++c) split(l1_scale * std::cos(cen[c]), l1_scale * std::sin(cen[c]), &t.l1_hi[c], &t.l1_lo[c]);
   for (int e = 0; e < 256; ++e) {
     const uint32_t ha = t.l1_hi[e & 15], hb = t.l1_hi[e >> 4], la = t.l1_lo[e & 15], lb = t.l1_lo[e >> 4];
     t.t1p_hi[e] = make_uint2((ha & 0xFFFFu) | (hb << 16), (ha >> 16) | (hb & 0xFFFF0000u));
@@ -482,8 +488,12 @@ int32_t pq_build_tables(const double* cen, const double* bnd, void* tables_host)
       const int k2 = i & 3, k3 = 4 + ((i >> 2) & 3), k4 = 8 + (i >> 4);
       const double t4 = (s >> 1) ? us[k4] : uc[k4];
       const double t3 = (s & 1) ? us[k3] : uc[k3];
-      split(t4 * t3 * uc[k2], t4 * t3 * us[k2], &t.u_tab[s][i].x, &t.u_tab[s][i].y);
+      split(t4 * t3 * uc[k2] / l1_scale, t4 * t3 * us[k2] / l1_scale, &t.u_tab[s][i].x, &t.u_tab[s][i].y);
     }
+  bool mirrored = true;   // cos of a level-4 centroid = sin of its mirror image, to what the tables hold (22 bits)
+  for (int k = 0; k < 4; ++k)
+    if (std::fabs(uc[8 + k] - us[11 - k]) > 1e-8) mirrored = false;
+  if (l1_scale != 1.0 && mirrored) t.flags |= pq::kFlagExactDecode;
   if (!build_l1_cells(bnd, t.l1_cells)) return PQ_ERR_INVALID_ARG;
   std::memcpy(tables_host, &t, sizeof(t));
   return PQ_OK;

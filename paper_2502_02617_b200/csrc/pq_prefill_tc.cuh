@@ -49,10 +49,10 @@ constexpr int kPtRawBufs = 4;                       // of them in flight
 constexpr int kPtScores = 4;                        // score accumulators: the score MMAs run ahead of the softmax
 constexpr int kPtGroups = 16;                       // warp-sized pieces of a block's decoding
 // Shared memory, as offsets in the CTA's shared window (whose addresses carry the CTA's rank in the cluster above): dynamic shared
-// memory starts behind what the system keeps (1 KB; where it is not, the kernel is not taken: tensor_kernel_fits), the
+// memory starts behind what the system keeps (1 KB; where it is not, the kernel is not taken: window_as_mapped), the
 // decode tables (those of the decode kernel: 96 KB, replicated for conflict-free lookups) on a 32 KB boundary, so that a
 // table address is the OR of disjoint bit fields.
-constexpr uint32_t kPtBase = 1024;
+constexpr uint32_t kPtBase = kWindowBase;
 constexpr uint32_t kPtRaw = kPtBase;
 constexpr uint32_t kPtTab = 32768, kPtT1 = kPtTab + kSmT1p, kPtU = kPtTab + kSmU;
 constexpr uint32_t kPtKv = kPtTab + kSmBar;         // the stages; also Q' at the start and O at the end
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) prefill_tc_kernel(DecodeArgs a,
   auto row_index = [&](int r) -> int64_t {               // offset of row r in q / out ([batch][n_q][n_q_heads][128])
     return (((int64_t)b * n_q + q0 + r / g) * a.n_q_heads + hk * g + r % g) * 128;
   };
-  if (sb & 0xFFFFFFu) {   // the host asks for the place (tensor_kernel_fits): never, and then NaN rather than anything (both CTAs leave alike)
+  if (sb & 0xFFFFFFu) {   // the host asks for the place (window_as_mapped): never, and then NaN rather than anything (both CTAs leave alike)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int r = tid; r < n_rows; r += kPtThreads) a.part_lse[(int64_t)split * a.batch * a.n_q_heads + row_index(r) / 128] = CUDART_NAN_F;
     set_status(a.status, PQ_ERR_CUDA);

@@ -17,13 +17,13 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _filled(lens, Hq, Hkv, d, seed, dtype=torch.bfloat16, paged=False):
+def _filled(lens, Hq, Hkv, d, seed, dtype=torch.bfloat16, paged=False, codebooks=None):
     if paged:
         pages = -(-max(lens) // 128)
         table = torch.randperm(len(lens) * pages, generator=torch.Generator().manual_seed(seed)).view(len(lens), pages)
-        cache = pq.PagedPolarQuantCache(len(lens), Hq, Hkv, d, 128, len(lens) * pages, table, seed=seed, device=DEV)
+        cache = pq.PagedPolarQuantCache(len(lens), Hq, Hkv, d, 128, len(lens) * pages, table, seed=seed, device=DEV, codebooks=codebooks)
     else:
-        cache = pq.PolarQuantCache(len(lens), Hq, Hkv, d, capacity=max(lens), seed=seed, device=DEV)
+        cache = pq.PolarQuantCache(len(lens), Hq, Hkv, d, capacity=max(lens), seed=seed, device=DEV, codebooks=codebooks)
     K, V = synthetic.kv_like(seed + 1, sum(lens), Hkv, d, dtype, DEV, n_outliers=4 if d >= 64 else 0)
     cache.encode(K, V, torch.tensor(np.concatenate(([0], np.cumsum(lens))), dtype=torch.int32, device=DEV))
     return cache, _oracle_cache(cache, K, V, lens)
@@ -101,6 +101,23 @@ def test_single_query_kernels(d, g):
         out = to_f64(cache.attend(q))
         for b in range(len(lens)):
             assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (kernel, lens[b])
+
+
+# Codebooks whose decode tables need the residuals of the level-1 factors and both halves of the level-4 factors (the analytic one
+# needs neither): every level moved, or the top level alone, in the three kernels that read those tables.
+@pytest.mark.parametrize("moved", [slice(0, 28), slice(24, 28)])
+@pytest.mark.parametrize("g,paged", [(4, False), (4, True), (7, False)])
+def test_attention_with_codebooks_that_are_not_analytic(g, paged, moved):
+    cen, bnd = (t.clone() for t in pq.pq_fit_codebooks())
+    cen[moved] += 0.01 * torch.cos(torch.arange(28, dtype=torch.float64))[moved]
+    for c0, b0, n in ((0, 0, 16), (16, 15, 4), (20, 18, 4), (24, 21, 4)):
+        bnd[b0:b0 + n - 1] = 0.5 * (cen[c0:c0 + n - 1] + cen[c0 + 1:c0 + n])
+    lens, Hkv = [1, 15, 16, 17, 127, 129, 1025], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 30 + g, paged=paged, codebooks=(cen, bnd))
+    for n_q, kernels in ((1, (PERSISTENT, ROWS)), (16, (TCGEN05,))):
+        q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(g), device=DEV)
+        for kernel in kernels:
+            _check_multi(cache, ref, q, lens, kernel)
 
 
 # One or two units of a longer sequence: clusters of sixteen blocks (the limit), also where a block un-rotates one coordinate.
