@@ -3,9 +3,10 @@
 // for what a margin does not cover, so the codes are those of a float64 evaluation of Algorithm 1.
 //
 // A thread block takes a tile of vectors (consecutive rows of one head, K or V):
-//   * y = x S on the FMA pipe: thread = kVT vectors x 8 columns, S in slices of 32 rows through shared memory.  The sum
-//     over k is formed per slice and the slices are added, so |y - y_exact| <= (32 + d / 32) 2^-24 sum_k |x_k||S_kj|,
-//     which is at most that factor times ||x||_2 (Cauchy-Schwarz; the columns of an orthogonal S have unit norm).
+//   * y = x S.  bf16 rows, where there are enough for four vectors a thread: on tensor cores (mma.sync), S split into three bf16 terms
+//     as its slices of 32 rows arrive in shared memory (ge_product_mma; its error bound there).  Otherwise on the FMA pipe: thread =
+//     kVT vectors x 8 columns, the sum over k formed per slice and the slices added, so |y - y_exact| <= (32 + d / 32) 2^-24
+//     sum_k |x_k||S_kj|, which is at most that factor times ||x||_2 (Cauchy-Schwarz; the columns of an orthogonal S have unit norm).
 //   * quantise: thread = (vector, group of 16 coordinates), the four lowest levels in registers.  A code is found by
 //     binary search over the level's boundary lines: psi > beta iff r_b cos(beta) - r_a sin(beta) > 0 (with the
 //     half-plane bookkeeping of level 1), which needs no arc tangent.  The search tests both neighbours of the cell it
@@ -18,9 +19,10 @@
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
 // A radius is certified by radius_unsure, with the bound of rotation_block_error: 1.4 to 5 % of them are not, according to the slices
 // of S and the blocks of a vector.
-// Bound by the product on the FMA pipe (18 of a block's 47 us) and by the latency of the float64 re-decisions (13).  Measured (8 heads;
-// a block per vector in float64 before): 512 tokens, seven levels of three bits 89.7 -> 43.4 us; packed cache, 2048 tokens at
-// head_dim 64 67 -> 40 us.
+// Bound by the latency of its phases and of the float64 re-decisions (13 of a block's 47 us before the product moved to tensor cores, of
+// which the product on the FMA pipe was 18).  Measured (8 heads; a block per vector in float64 before): 512 tokens, seven
+// levels of three bits 89.7 -> 43.4 us; packed cache, 2048 tokens at head_dim 64 67 -> 40 us.  Product on tensor cores: 8 x 512 tokens,
+// seven levels of three bits, and an attention over 8 x 4096 of 95 us 312 -> 273 us.
 #pragma once
 #include <math_constants.h>
 
@@ -30,6 +32,9 @@ namespace pq {
 
 constexpr int kGeThreads = 256;
 constexpr int kGeSlice = 32;              // rows of S per slice
+
+// A slice in shared memory: float32, or its three bf16 terms with rows of dc + 8.
+__host__ __device__ constexpr int ge_slice_floats(int dc) { return 3 * kGeSlice * (dc + 8) / 2; }
 
 struct GeShape {
   int dc, ng, vecs, x_stride, row_words, floats_xy;
@@ -48,7 +53,7 @@ __host__ __device__ inline GeShape ge_shape(int d, int row_bytes, int vt) {
   return s;
 }
 __host__ inline int ge_smem_bytes(const GeShape& s, int n_bnd) {
-  return 4 * (s.floats_xy + kGeSlice * s.dc + s.vecs * s.row_words + s.vecs * s.ng + 2 * s.vecs + 2 * ((n_bnd + 1) & ~1)) +
+  return 4 * (s.floats_xy + ge_slice_floats(s.dc) + s.vecs * s.row_words + s.vecs * s.ng + 2 * s.vecs + 2 * ((n_bnd + 1) & ~1)) +
          8 * s.vecs + 8 * s.vecs * s.ng + 6 * s.vecs * s.ng + 64;
 }
 
@@ -154,6 +159,116 @@ __device__ __forceinline__ int64_t ge_destination(const GenEncodeArgs& a, int ro
   return off * kTokenBlock + pos % kTokenBlock;
 }
 
+// Bounds on the error of the product on tensor cores relative to ||x||_2, as rot_err in the kernel and rotation_block_error: products
+// of bf16 values are exact in float32, the three terms represent S to 2^-26, and each of the six accumulating MMAs of a slice is
+// taken to add at most 2 * 2^-24 of its running sum, which is at most the norm of the slice of x (twice that for the norm of a
+// block's errors); the slices' norms add up to sqrt(slices) ||x|| at most and their sums are added one by one.  Measured against
+// float64 over 2^20 vectors per head dim of 16 to 256 (normal, outlier channels, log-normal, concentrated, positive): at most 0.37
+// of the first bound (head_dim 32; 0.09 at 128) and 0.22 of the second.
+__host__ __device__ constexpr float ge_mma_error(int dc) {
+  return 1.1f * (12.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
+}
+__host__ __device__ constexpr float ge_mma_block_error(int dc) {
+  return 1.02f * (24.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
+}
+
+// Three bf16 terms of a pair of float32 values (round to nearest each: together within 2^-26 of the values).
+__device__ __forceinline__ void ge_split(float a, float b, uint32_t* t) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat162 w = __floats2bfloat162_rn(a, b);
+    t[i] = *reinterpret_cast<const uint32_t*>(&w);
+    a -= __uint_as_float(t[i] << 16);
+    b -= __uint_as_float(t[i] & 0xFFFF0000u);
+  }
+}
+template <bool kTrans>
+__device__ __forceinline__ void ge_ldmatrix(const __nv_bfloat16* row, uint32_t (&v)[4]) {
+  const uint32_t at = (uint32_t)__cvta_generic_to_shared(row);
+  if (kTrans)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
+}
+__device__ __forceinline__ void ge_mma(float* d, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// y = x S of a tile of V bf16 vectors (xh [V][dc + 8]) on tensor cores, into y [V][dc / 16][20] over the same memory.  S goes through
+// shared memory in slices of 32 rows, split into three bf16 terms as it arrives; a warp owns eight 16 x 8 tiles of y, smallest terms
+// first, a fresh accumulator per slice.
+__device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, int dc, float* xy, float* Ss, int tid) {
+  const int lane = tid & 31, warp = tid >> 5, stride = dc + 8;
+  const __nv_bfloat16* xh = reinterpret_cast<const __nv_bfloat16*>(xy);
+  uint32_t* Sw = reinterpret_cast<uint32_t*>(Ss);   // [term][32][stride / 2] pairs
+  const int m_tiles = V >> 4, per_m = m_tiles >= 8 ? 1 : 8 / m_tiles;      // warps that share 16 vectors
+  const int pairs = m_tiles >= 8 ? 32 / m_tiles : 4;                       // pairs of 8-column tiles per 16 vectors of a warp
+  const int m0 = m_tiles >= 8 ? warp * (m_tiles >> 3) : warp / per_m, n0 = m_tiles >= 8 ? 0 : (warp % per_m) * 64;
+  const int lr = (lane & 7) + (lane & 8), lc = (lane >> 4) * 8;            // this lane's row and column of a 16 x 16 ldmatrix
+  const bool aligned = ((uintptr_t)a.S & 15) == 0;
+  float tot[8][4];
+#pragma unroll
+  for (int t = 0; t < 8; ++t)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tot[t][e] = 0.f;
+#pragma unroll 1
+  for (int k0 = 0; k0 < dc; k0 += kGeSlice) {
+    const int nk = min(kGeSlice, dc - k0);
+    __syncthreads();   // x is complete; the slice before has been used
+#pragma unroll 4
+    for (int i = 4 * tid; i < nk * dc; i += 4 * kGeThreads) {
+      const int k = i / dc, n = i - k * dc;   // four columns of a row
+      const float* src = a.S + (int64_t)k0 * dc + i;
+      float4 v;
+      if (aligned) v = __ldg(reinterpret_cast<const float4*>(src));
+      else v = make_float4(__ldg(src), __ldg(src + 1), __ldg(src + 2), __ldg(src + 3));
+      uint32_t lo[3], hi[3];
+      ge_split(v.x, v.y, lo);
+      ge_split(v.z, v.w, hi);
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+        *reinterpret_cast<uint2*>(Sw + ((t * kGeSlice + k) * stride + n) / 2) = make_uint2(lo[t], hi[t]);
+    }
+    __syncthreads();
+    float acc[8][4];
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[t][e] = 0.f;
+#pragma unroll 1
+    for (int ks = 0; ks < nk; ks += 16) {
+      uint32_t A[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int m = m0 + p / pairs, n = n0 + (p % pairs) * 16;
+        if (p % pairs == 0) ge_ldmatrix<false>(xh + (m * 16 + lr) * stride + k0 + ks + lc, A);
+#pragma unroll
+        for (int t = 2; t >= 0; --t) {
+          uint32_t B[4];
+          ge_ldmatrix<true>(reinterpret_cast<const __nv_bfloat16*>(Sw) + (t * kGeSlice + ks + lr) * stride + n + lc, B);
+          ge_mma(acc[2 * p], A, B[0], B[1]);
+          ge_mma(acc[2 * p + 1], A, B[2], B[3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) tot[t][e] += acc[t][e];
+  }
+  __syncthreads();   // x has been used: y takes its place
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int p = t >> 1, row = (m0 + p / pairs) * 16 + (lane >> 2), col = n0 + (p % pairs) * 16 + 8 * (t & 1) + 2 * (lane & 3);
+    float* y = xy + (row * (dc >> 4) + (col >> 4)) * 20 + (col & 15);
+    *reinterpret_cast<float2*>(y) = make_float2(tot[t][0], tot[t][1]);
+    *reinterpret_cast<float2*>(y + 8 * (dc >> 4) * 20) = make_float2(tot[t][2], tot[t][3]);
+  }
+}
+
 // kVT: vectors per thread in the product (4; 1 for few rows).  kSub: levels inside a group, min(L, 4).
 template <int kVT, int kSub>
 __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_constant__ GenEncodeArgs a) {
@@ -163,8 +278,8 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   const GeShape s = ge_shape(d, g.row_bytes, kVT);
   const int V = s.vecs, ng = s.ng, dc = s.dc;
   float* xy = reinterpret_cast<float*>(ge_smem);                        // x [V][x_stride], then y [V][ng * 20]
-  float* Ss = xy + s.floats_xy;                                         // [kGeSlice][dc]
-  uint32_t* rows = reinterpret_cast<uint32_t*>(Ss + kGeSlice * dc);     // [V][row_words]
+  float* Ss = xy + s.floats_xy;                                         // a slice of S
+  uint32_t* rows = reinterpret_cast<uint32_t*>(Ss + ge_slice_floats(dc)); // [V][row_words]
   float* gsum = reinterpret_cast<float*>(rows + V * s.row_words);       // [V][ng] squared norms of the groups
   float* dy_sm = gsum + V * ng;                                         // [V] bound on the error of a coordinate, [V] on that of a block
   float2* tab = reinterpret_cast<float2*>(dy_sm + 2 * V);               // boundaries
@@ -196,6 +311,8 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
   }
   const bool vec8 = a.in_dtype == PQ_DTYPE_BF16 && d >= 16 && ((a.token_stride | a.head_stride) & 7) == 0 &&
                     ((uintptr_t)xbase & 15) == 0;
+  const bool tc = kVT == 4 && a.in_dtype == PQ_DTYPE_BF16 && d >= 16;   // the product on tensor cores: x stays bf16
+  __nv_bfloat16* xh = reinterpret_cast<__nv_bfloat16*>(xy);
   int bad = 0;
   if (vec8) {
     const int per_row = d / 8;
@@ -214,6 +331,10 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
       }
 #pragma unroll
       for (int e = 0; e < 8; ++e) bad += !(fabsf(f[e]) < CUDART_INF_F);
+      if (tc) {
+        *reinterpret_cast<uint4*>(xh + v * (dc + 8) + 8 * p) = w;
+        continue;
+      }
       float4* dst = reinterpret_cast<float4*>(xy + v * s.x_stride + 8 * p);
       dst[0] = make_float4(f[0], f[1], f[2], f[3]);
       dst[1] = make_float4(f[4], f[5], f[6], f[7]);
@@ -225,7 +346,8 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
       if (row < a.total_tokens && k < d)
         f = ge_load(xbase, a.in_dtype, (int64_t)row * a.token_stride + (int64_t)head * a.head_stride + k);
       bad += !(fabsf(f) < CUDART_INF_F);
-      xy[v * s.x_stride + k] = f;
+      if (tc) xh[v * (dc + 8) + k] = __float2bfloat16(f);
+      else xy[v * s.x_stride + k] = f;
     }
   }
   if (bad) {
@@ -233,72 +355,76 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     set_status(a.status, PQ_ERR_NONFINITE);
   }
 
-  // ---- y = x S: thread = kVT vectors x 8 columns (four packed pairs)
-  const int tx = tid % (dc / 8), ty = tid / (dc / 8);
-  float tot[kVT][8];
-#pragma unroll
-  for (int v = 0; v < kVT; ++v)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) tot[v][j] = 0.f;
-  for (int k0 = 0; k0 < dc; k0 += kGeSlice) {
-    const int nk = min(kGeSlice, dc - k0);
-    __syncthreads();
-    if (d >= 16) {
-      const float4* src = reinterpret_cast<const float4*>(a.S + (int64_t)k0 * d);
-      float4* dst = reinterpret_cast<float4*>(Ss);
-      if (((uintptr_t)a.S & 15) == 0) {
-        for (int i = tid; i < nk * dc / 4; i += kGeThreads) dst[i] = __ldg(src + i);
-      } else {
-        for (int i = tid; i < nk * dc; i += kGeThreads) Ss[i] = __ldg(a.S + (int64_t)k0 * d + i);
-      }
-    } else {
-      for (int i = tid; i < nk * dc; i += kGeThreads) {
-        const int k = k0 + i / dc, j = i % dc;
-        Ss[i] = k < d && j < d ? __ldg(a.S + k * d + j) : 0.f;
-      }
-    }
-    __syncthreads();
-    uint64_t acc[kVT][4];
+  if (tc) {
+    ge_product_mma(a, V, dc, xy, Ss, tid);
+  } else {
+    // ---- y = x S: thread = kVT vectors x 8 columns (four packed pairs)
+    const int tx = tid % (dc / 8), ty = tid / (dc / 8);
+    float tot[kVT][8];
 #pragma unroll
     for (int v = 0; v < kVT; ++v)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[v][j] = 0ull;
-#pragma unroll 2
-    for (int k = 0; k < nk; k += 4) {
-      float4 xv[kVT];
-#pragma unroll
-      for (int v = 0; v < kVT; ++v) xv[v] = *reinterpret_cast<const float4*>(xy + (ty * kVT + v) * s.x_stride + k0 + k);
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const ulonglong2 sa = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx);
-        const ulonglong2 sb = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx + 4);
-#pragma unroll
-        for (int v = 0; v < kVT; ++v) {
-          const float xk = kk == 0 ? xv[v].x : kk == 1 ? xv[v].y : kk == 2 ? xv[v].z : xv[v].w;
-          const uint64_t xx = f2_pack(xk, xk);
-          acc[v][0] = f2_fma(xx, sa.x, acc[v][0]);
-          acc[v][1] = f2_fma(xx, sa.y, acc[v][1]);
-          acc[v][2] = f2_fma(xx, sb.x, acc[v][2]);
-          acc[v][3] = f2_fma(xx, sb.y, acc[v][3]);
+      for (int j = 0; j < 8; ++j) tot[v][j] = 0.f;
+    for (int k0 = 0; k0 < dc; k0 += kGeSlice) {
+      const int nk = min(kGeSlice, dc - k0);
+      __syncthreads();
+      if (d >= 16) {
+        const float4* src = reinterpret_cast<const float4*>(a.S + (int64_t)k0 * d);
+        float4* dst = reinterpret_cast<float4*>(Ss);
+        if (((uintptr_t)a.S & 15) == 0) {
+          for (int i = tid; i < nk * dc / 4; i += kGeThreads) dst[i] = __ldg(src + i);
+        } else {
+          for (int i = tid; i < nk * dc; i += kGeThreads) Ss[i] = __ldg(a.S + (int64_t)k0 * d + i);
+        }
+      } else {
+        for (int i = tid; i < nk * dc; i += kGeThreads) {
+          const int k = k0 + i / dc, j = i % dc;
+          Ss[i] = k < d && j < d ? __ldg(a.S + k * d + j) : 0.f;
         }
       }
-    }
+      __syncthreads();
+      uint64_t acc[kVT][4];
 #pragma unroll
-    for (int v = 0; v < kVT; ++v)
+      for (int v = 0; v < kVT; ++v)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float lo, hi;
-        f2_unpack(acc[v][j], lo, hi);
-        tot[v][2 * j] += lo;
-        tot[v][2 * j + 1] += hi;
+        for (int j = 0; j < 4; ++j) acc[v][j] = 0ull;
+#pragma unroll 2
+      for (int k = 0; k < nk; k += 4) {
+        float4 xv[kVT];
+#pragma unroll
+        for (int v = 0; v < kVT; ++v) xv[v] = *reinterpret_cast<const float4*>(xy + (ty * kVT + v) * s.x_stride + k0 + k);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const ulonglong2 sa = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx);
+          const ulonglong2 sb = *reinterpret_cast<const ulonglong2*>(Ss + (k + kk) * dc + 8 * tx + 4);
+#pragma unroll
+          for (int v = 0; v < kVT; ++v) {
+            const float xk = kk == 0 ? xv[v].x : kk == 1 ? xv[v].y : kk == 2 ? xv[v].z : xv[v].w;
+            const uint64_t xx = f2_pack(xk, xk);
+            acc[v][0] = f2_fma(xx, sa.x, acc[v][0]);
+            acc[v][1] = f2_fma(xx, sa.y, acc[v][1]);
+            acc[v][2] = f2_fma(xx, sb.x, acc[v][2]);
+            acc[v][3] = f2_fma(xx, sb.y, acc[v][3]);
+          }
+        }
       }
-  }
-  __syncthreads();   // x has been used: y takes its place
 #pragma unroll
-  for (int v = 0; v < kVT; ++v) {
-    float* dst = xy + ((ty * kVT + v) * ng + (tx >> 1)) * 20 + 8 * (tx & 1);
-    *reinterpret_cast<float4*>(dst) = make_float4(tot[v][0], tot[v][1], tot[v][2], tot[v][3]);
-    *reinterpret_cast<float4*>(dst + 4) = make_float4(tot[v][4], tot[v][5], tot[v][6], tot[v][7]);
+      for (int v = 0; v < kVT; ++v)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float lo, hi;
+          f2_unpack(acc[v][j], lo, hi);
+          tot[v][2 * j] += lo;
+          tot[v][2 * j + 1] += hi;
+        }
+    }
+    __syncthreads();   // x has been used: y takes its place
+#pragma unroll
+    for (int v = 0; v < kVT; ++v) {
+      float* dst = xy + ((ty * kVT + v) * ng + (tx >> 1)) * 20 + 8 * (tx & 1);
+      *reinterpret_cast<float4*>(dst) = make_float4(tot[v][0], tot[v][1], tot[v][2], tot[v][3]);
+      *reinterpret_cast<float4*>(dst + 4) = make_float4(tot[v][4], tot[v][5], tot[v][6], tot[v][7]);
+    }
   }
   __syncthreads();
   for (int i = tid; i < V * ng; i += kGeThreads) {   // squared norms of the groups
@@ -312,13 +438,14 @@ __global__ void __launch_bounds__(kGeThreads, 2) gen_encode_kernel(const __grid_
     gsum[i] = (q[0] + q[1]) + (q[2] + q[3]);
   }
   __syncthreads();
-  const float rot_err = 1.1f * (float)(kGeSlice + dc / kGeSlice) * 5.9604644775390625e-08f;
+  const float rot_err = tc ? ge_mma_error(dc) : 1.1f * (float)(kGeSlice + dc / kGeSlice) * 5.9604644775390625e-08f;
+  const float blk_err = tc ? ge_mma_block_error(dc) : rotation_block_error(kGeSlice, (dc + kGeSlice - 1) / kGeSlice);
   for (int v = tid; v < V; v += kGeThreads) {
     float t = 0.f;
     for (int i = 0; i < ng; ++i) t += gsum[v * ng + i];
     // the floor: where squares leave the float32 range (below 4e-20), nothing is certified
     dy_sm[v] = fmaf(rot_err * 1.0001f, sqrtf(t), 1e-19f);
-    dy_sm[V + v] = rotation_block_error(kGeSlice, (dc + kGeSlice - 1) / kGeSlice) * 1.0001f * sqrtf(t);
+    dy_sm[V + v] = blk_err * 1.0001f * sqrtf(t);
   }
   __syncthreads();
 

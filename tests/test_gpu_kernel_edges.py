@@ -168,6 +168,30 @@ def test_general_encoder_writes_the_same_bytes_in_any_pieces(d, bits):
     assert torch.equal(whole.cache, cut.cache)
 
 
+# Rows in bf16 are rotated on tensor cores where there are enough of them, the same values in float32 by multiply-adds: every decision
+# and every radius is exact, so the bytes are the same.  Head dims of every warp layout of the product, a remainder of its tiles, rows
+# that cannot be read 16 bytes at a time, outlier channels, a zero vector and rows near the ends of the float32 range.
+@pytest.mark.parametrize("strided", [False, True])
+@pytest.mark.parametrize("d,bits,n", [(16, None, 2500), (32, None, 1301), (64, None, 645), (128, (3,) * 7, 333), (256, (4, 2, 2, 2, 2), 167)])
+def test_the_encoder_on_tensor_cores_writes_the_bytes_of_the_float32_one(d, bits, n, strided):
+    Hkv = 8
+    K, V = synthetic.kv_like(d + n, n, Hkv, d, torch.bfloat16, DEV, n_outliers=4 if d >= 64 else 0)
+    V[7] = 0
+    K[3::17] *= 1e-18
+    K[5::19] *= 1e15
+    if strided:
+        K, V = (torch.nn.functional.pad(t, (0, 1))[..., :d] for t in (K, V))
+    cu = torch.tensor([0, n], dtype=torch.int32, device=DEV)
+    caches = []
+    for dtype in (torch.bfloat16, torch.float32):
+        c = (pq.PolarQuantCache(1, Hkv, Hkv, d, capacity=n, seed=6, device=DEV) if bits is None else
+             pq.GeneralPolarQuantCache(1, Hkv, Hkv, d, bits, n, seed=6, device=DEV))
+        c.cache.zero_()
+        c.encode(*((K, V) if dtype == torch.bfloat16 else (K.float(), V.float())), cu)
+        caches.append(c)
+    assert torch.equal(caches[0].cache, caches[1].cache) and caches[0].status[:3].tolist() == caches[1].status[:3].tolist()
+
+
 # Four coordinates per thread where the pointers allow it, else one.  A weighted mean of three float32 values: 1e-6 is eight
 # roundings of 2^-23.
 @pytest.mark.parametrize("d,shift", [(16, 0), (16, 1), (128, 0), (128, 3)])
