@@ -75,10 +75,10 @@ int l1_code_of_angle(const double* bnd, double psi, int near) {
 }
 
 // What the cells look like whatever the codebook is: their ranges of t and the angles of the points that are looked at.
-// 768 arc tangents, computed once per process (most of the cost of a table that is built for every prompt).
+// 384 arc tangents, computed once per process (most of the cost of a table that is built for every prompt).
 struct L1Grid {
   double lo[pq::kL1Cells], hi[pq::kL1Cells], mid_phi[pq::kL1Cells];  // with slack: the decisions
-  double t[pq::kL1Cells][5], phi[pq::kL1Cells][5];                     // the points of the check
+  double t[pq::kL1Cells][2], phi[pq::kL1Cells][2];                   // the points of the check: a cell's ends
   L1Grid() {
     // the kernel's cell index is floor(m / 8), m = t * kL1CellScale * 8 rounded to an integer
     const double scale = (double)pq::kL1CellScale;
@@ -87,11 +87,9 @@ struct L1Grid {
       lo[c] = std::fmax(0.0, a - 1e-6);
       hi[c] = std::fmin(1.0, b + 1e-6);
       mid_phi[c] = std::atan(0.5 * (lo[c] + hi[c]));
-      const double lo0 = std::fmax(0.0, a), hi0 = std::fmin(1.0, b);
-      for (int i = 0; i <= 4; ++i) {
-        t[c][i] = lo0 + (hi0 - lo0) * i / 4.0;
-        phi[c][i] = std::atan(t[c][i]);
-      }
+      t[c][0] = std::fmax(0.0, a);
+      t[c][1] = std::fmin(1.0, b);
+      for (int i = 0; i < 2; ++i) phi[c][i] = std::atan(t[c][i]);
     }
   }
 };
@@ -154,14 +152,15 @@ bool build_l1_cells(const double* bnd, uint2 (*cells)[pq::kL1Cells]) {
       std::memcpy(&bits, &tau, 4);
       cells[o][c] = make_uint2(bits, ((uint32_t)code_lo << 28) | ((uint32_t)code_hi << 24));
     }
-    // Check the two properties on a grid of every cell (the table is small; a wrong entry would be a silent
-    // wrong code).
+    // Check the two properties at both ends of every cell (a wrong entry would be a silent wrong code).  That covers the cell: between
+    // neighbouring rays the code does not change, |t - tau| is convex and the distance to the nearest ray concave in t, so the
+    // first exceeds the second at an end of the stretch if anywhere, and the only ray inside a decided cell is tau itself.
     int next = 0;   // first ray above the point; consecutive points are close, cells overlap by 1/8 of their width
     for (int c = 0; c < pq::kL1Cells; ++c) {
       float tau;
       std::memcpy(&tau, &cells[o][c].x, 4);
       if (tau != tau) continue;
-      for (int i = 0; i <= 4; ++i) {
+      for (int i = 0; i < 2; ++i) {
         const double t = grid.t[c][i], dist = std::fabs(t - (double)tau);
         while (next < n_rays && rays[next].t < t) ++next;
         while (next > 0 && rays[next - 1].t >= t) --next;
@@ -454,17 +453,16 @@ int32_t pq_build_tables(const double* cen, const double* bnd, void* tables_host)
     t.cen_cos[k] = (float)std::cos(cen[k]);
     t.cen_sin[k] = (float)std::sin(cen[k]);
   }
-  auto h2 = [](double lo, double hi) -> uint32_t {
-    const __half a = __double2half(lo), b = __double2half(hi);
+  auto h2 = [](__half a, __half b) -> uint32_t {
     uint16_t ua, ub;
     std::memcpy(&ua, &a, 2);
     std::memcpy(&ub, &b, 2);
     return (uint32_t)ua | ((uint32_t)ub << 16);
   };
   auto split = [&](double va, double vb, uint32_t* hi, uint32_t* lo) {
-    const double ha = (double)__half2float(__double2half(va)), hb = (double)__half2float(__double2half(vb));
-    *hi = h2(va, vb);
-    *lo = h2(va - ha, vb - hb);
+    const __half ha = __double2half(va), hb = __double2half(vb);
+    *hi = h2(ha, hb);
+    *lo = h2(__double2half(va - (double)__half2float(ha)), __double2half(vb - (double)__half2float(hb)));
   };
   double l1_scale = pq::kL1Scale;   // 1 if it does not bring every level-1 factor close to an fp16 value
   for (int c = 0; c < 16; ++c)
