@@ -164,7 +164,9 @@ namespace pq {
 // of 16 bytes long and 16-byte aligned in the cache and in the buffer.
 template <int D>
 struct PackedSplit {
-  static constexpr bool kEarlyTables = true;
+  // pairs of level-1 codes where the loop over the tokens is what takes the time: at head_dim 128 the kernel has short contexts only, and
+  // at 16 a call is mostly its start (256 tokens, one head: 12.2 -> 12.5 us with them)
+  static constexpr bool kEarlyTables = true, kPairs = D == 64 || D == 32;
   static constexpr int kTabMax = 32, kDim = D;
   // the planes of a token-block (make_layout for this head_dim)
   static constexpr int kNb = D / 16, kB1 = 4 * kNb, kB2 = kNb, kB3 = kNb >= 2 ? kNb / 2 : 1, kB4 = kNb >= 4 ? kNb / 4 : 1, kBr = 2 * kNb;
@@ -178,6 +180,10 @@ struct PackedSplit {
   Paging pg;
 
   static int tile_bytes(int n) { return n * kRow; }
+  // Tokens of a tile, as size_split chooses them (packed rows are short): a constant, so that the planes of a staged tile are at
+  // constant distances.
+  template <int kU>
+  __host__ __device__ static constexpr int tile_tokens() { return D <= kU ? 32 : 16; }
   __device__ __forceinline__ int len(int pair) const {
     const int b = pair / n_q, v = lens[b] - (n_q - 1 - (pair - b * n_q));
     return v > 0 ? v : 0;
@@ -186,6 +192,13 @@ struct PackedSplit {
     if (tid < PQ_N_CENTROIDS) tab[tid] = make_float2(tables->cen_cos[tid], tables->cen_sin[tid]);
   }
   __device__ __forceinline__ int shift(int, int, int, int) const { return 0; }
+  __device__ __forceinline__ void fill_pairs(float4* pairs, int tid, int n_threads) const {
+#pragma unroll 4
+    for (int i = tid; i < 256 * 8; i += n_threads) {
+      const int a = i >> 3 & 15, b = i >> 7;
+      pairs[i] = make_float4(tables->cen_cos[a], tables->cen_sin[a], tables->cen_cos[b], tables->cen_sin[b]);
+    }
+  }
   __device__ __forceinline__ void stage(uint8_t* buf, int pair, int hk, int kv, int t0, int, int lane) const {
     Layout L;
     L.block_bytes = kBlockBytes;
@@ -207,8 +220,9 @@ struct PackedSplit {
   }
   // kU = 16: a block; kU = 8: half of one (the angles above it are the block's)
   template <int kU>
-  __device__ __forceinline__ void decode(const uint8_t* buf, int, int t, int unit, const float2* tab, float* y) const {
-    const int blk = kU == 16 ? unit : unit >> 1, tile = c.tile;
+  __device__ __forceinline__ void decode(const uint8_t* buf, int, int t, int unit, const float2* tab, const float4* pairs, float* y) const {
+    constexpr int tile = tile_tokens<kU>();
+    const int blk = kU == 16 ? unit : unit >> 1;
     const uint8_t* p2 = buf + tile * kB1;
     const uint8_t* p3 = p2 + tile * kB2;
     const uint8_t* p4 = p3 + tile * kB3;
@@ -251,6 +265,17 @@ struct PackedSplit {
       }
     }
 #pragma unroll
+    if (kPairs) {
+#pragma unroll
+      for (int j = 0; j < kU / 4; ++j) {   // byte j of the codes: 128 bytes per entry of the table
+        const uint32_t row = (j == 0 ? l1 << 7 : l1 >> (8 * j - 7)) & 0x7F80u;
+        const float4 e = *reinterpret_cast<const float4*>(reinterpret_cast<const uint8_t*>(pairs) + row);
+        y[4 * j] = r1[2 * j] * e.x;
+        y[4 * j + 1] = r1[2 * j] * e.y;
+        y[4 * j + 2] = r1[2 * j + 1] * e.z;
+        y[4 * j + 3] = r1[2 * j + 1] * e.w;
+      }
+    } else {
     for (int j = 0; j < kU / 2; ++j) {
       const float2 e = tab[(l1 >> (4 * j)) & 15u];
       y[2 * j] = r1[j] * e.x;

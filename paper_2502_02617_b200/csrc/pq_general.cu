@@ -111,7 +111,7 @@ __global__ void gen_dequant_kernel(GenConfig g, int n_kv_heads, const float* S, 
 // 128: 102.6 -> 92.5, 102.6 -> 93.6 and 103.5 -> 92.4 us), 0 for any table.
 template <int kSub, int kB>
 struct GenSplit {
-  static constexpr bool kEarlyTables = false;
+  static constexpr bool kEarlyTables = false, kPairs = false;
   static constexpr int kTabMax = kB ? kGenMaxLevels << kB : kGenMaxCentroids, kDim = 0;
   SplitCommon c;
   GenConfig g;
@@ -147,7 +147,7 @@ struct GenSplit {
     return __funnelshift_r(w[0], w[1], ((at & 3) << 3) + (bit & 7));
   }
   template <int kU>
-  __device__ __forceinline__ void decode(const uint8_t* buf, int at, int t, int unit, const float2* tab, float* y) const {
+  __device__ __forceinline__ void decode(const uint8_t* buf, int at, int t, int unit, const float2* tab, const float4*, float* y) const {
     constexpr int kTop = kU == 16 ? 4 : 3;                 // levels a unit of kU coordinates spans
     constexpr int kIn = kSub < kTop ? kSub : kTop;         // ... and those of them that exist
     constexpr int kBlk = kU >> kIn;                        // subtrees whose root starts inside the unit

@@ -17,6 +17,8 @@
 // whole query by itself instead of meeting the others first, and the merge has one cluster barrier.
 // Measured (32/8 heads; two launches and a workspace before): one sequence of 1000 tokens, head_dim 128 19.8 -> 10.7 us; eight of
 // 4096, head_dim 64 111 -> 32 us; the general layout with three bits and seven levels, eight of 4096, 5330 -> 95 us.
+// Level 1 of the packed layout, head dims 32 and 64: one 16-byte lookup per byte of codes instead of two of 8 bytes, and planes of a staged
+// tile at constant distances: 8 sequences of up to 4096 tokens at head_dim 64, four steps with their appends 127.2 -> 123.4 us.
 // kU = 16 for up to four query heads per kv head, 8 for up to eight (the registers of q' and of the accumulators).
 #pragma once
 #include <cstdint>
@@ -30,6 +32,7 @@ namespace pq {
 __host__ __device__ constexpr int split_warps(int kh) { return kh <= 2 ? 16 : 8; }
 constexpr int kSplitStages = 4;            // tiles in flight per warp
 constexpr int kSplitSmemMax = 216 * 1024;
+constexpr int kSplitPairBytes = 256 * 8 * 16;   // (cos, sin) of both level-1 codes of a byte, eight copies for conflict-free 16-byte reads
 constexpr int kUnitStride = 20;            // floats between the 16-coordinate groups of q' in shared memory
 
 // What the kernel needs beside the layout.
@@ -55,9 +58,9 @@ __host__ __device__ inline int split_fixed_bytes(int d, int kh) {
   return (4 * (kh * dp / 16 * kUnitStride + 3 * kh * dp + 34 * split_warps(kh) * kh + 2 * kh) + 15) & ~15;
 }
 __host__ __device__ inline int split_s_bytes(int d) { return d <= 128 ? (d * d * 4 + 15) & ~15 : 0; }   // S, where it fits
-__host__ __device__ inline int split_smem_bytes(int d, int kh, int stage_bytes) {
+__host__ __device__ inline int split_smem_bytes(int d, int kh, int stage_bytes, bool pairs) {
   const int ring = split_warps(kh) * kSplitStages * 2 * stage_bytes, merge = split_warps(kh) * kh * split_pad(d) * 4;
-  return split_fixed_bytes(d, kh) + split_s_bytes(d) + (ring > merge ? ring : merge);
+  return (pairs ? kSplitPairBytes : 0) + split_fixed_bytes(d, kh) + split_s_bytes(d) + (ring > merge ? ring : merge);
 }
 
 __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
@@ -118,11 +121,12 @@ __device__ __forceinline__ void unit_lane_sums(float* v, int lane, int* from, in
 //   int len(pair)                     tokens the pair's query sees
 //   kTabMax, fill_tables(tab, tid)    the (cos, sin) table; kEarlyTables: filled before the kernel ahead in the stream has
 //                                     finished (it may not write them)
+//   kPairs, fill_pairs(pairs, tid, n) with kPairs also a table of pairs of level-1 codes (kSplitPairBytes)
 //   kDim                              head_dim where it is a compile-time constant, else 0
 //   void stage(buf, pair, hk, kv, t0, n, lane)  issue a warp's copies of the keys (kv = 0) or values (1) of tokens
 //                                     t0 .. t0 + n - 1 (n = tile size, or less in the last tile)
 //   int shift(pair, hk, kv, t0)       where in the buffer the tile that starts at token t0 begins
-//   void decode<kU>(buf, at, t, unit, tab, y)   the coordinates of a unit of token t of the tile at buf + at
+//   void decode<kU>(buf, at, t, unit, tab, pairs, y)   the coordinates of a unit of token t of the tile at buf + at
 template <class P, int kH>
 __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kernel(const __grid_constant__ P p) {
   constexpr int kU = split_unit(kH), kSplitWarps = split_warps(kH), kSplitThreads = 32 * kSplitWarps;
@@ -133,7 +137,8 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
   const int C = gridDim.x, rank = blockIdx.x, hk = blockIdx.y, pair = blockIdx.z;   // the cluster spans the x dimension
   const int d = P::kDim ? P::kDim : c.d, dp = split_pad(d), grp = c.n_q_heads / c.n_kv_heads;
   const int lanes = split_lanes(d, kH), T = c.tile, qs = dp / 16 * kUnitStride;
-  float* qg = reinterpret_cast<float*>(split_smem);   // [kH][dp / 16][kUnitStride]
+  float4* pairs = reinterpret_cast<float4*>(split_smem);   // [256][8] where the layout has them
+  float* qg = reinterpret_cast<float*>(split_smem + (P::kPairs ? kSplitPairBytes : 0));   // [kH][dp / 16][kUnitStride]
   float* q_in = qg + kH * qs;                         // [kH][dp]
   float* o_sm = q_in + kH * dp;                       // [kH][dp] this block's output (relative to m_sm)
   float* y_sm = o_sm + kH * dp;                       // [kH][dp] merged output
@@ -142,8 +147,8 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
   float* wl_sm = wm_sm + kSplitWarps * kH;            // [warps][kH]
   float* m_sm = wl_sm + kSplitWarps * kH;             // [kH]
   float* l_sm = m_sm + kH;                            // [kH]
-  float* S_sm = reinterpret_cast<float*>(split_smem + split_fixed_bytes(d, kH));   // [d][d], or nothing
-  uint8_t* ring = split_smem + split_fixed_bytes(d, kH) + split_s_bytes(d);
+  float* S_sm = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(qg) + split_fixed_bytes(d, kH));   // [d][d], or nothing
+  uint8_t* ring = reinterpret_cast<uint8_t*>(S_sm) + split_s_bytes(d);
   float* w_out = reinterpret_cast<float*>(ring);      // [warps][kH][dp], after the loop
   uint8_t* mine = ring + warp * (kSplitStages * 2 * c.stage_bytes);
 
@@ -155,6 +160,7 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
   }
   split_commit();
   if (P::kEarlyTables) p.fill_tables(tab, tid);
+  if constexpr (P::kPairs) p.fill_pairs(pairs, tid, kSplitThreads);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // lengths, cache and queries may come from the kernel before this one
   const int64_t q0 = ((int64_t)pair * c.n_q_heads + hk * grp) * d;
   const int len = p.len(pair);
@@ -230,6 +236,7 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
   __syncthreads();
 
   // ---- the stream of this warp
+  pairs += lane & 7;   // this lane's copy
   const int unit = lane & (lanes - 1);   // this lane's unit
   uint64_t q2[kH][kU / 2], acc[kH][kU / 2];
   float m_run[kH], l_run[kH];   // running reference of every head (the same in all lanes), this lane's share of the denominator
@@ -260,7 +267,7 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
     for (int tb = sub * per_pass; tb < n; tb += share * per_pass) {
       const int tt = tb + lane / lanes, t = min(tt, n - 1);   // past the end: the last token again, with weight 0
       float y[kU];
-      p.template decode<kU>(kbuf, at_k, t, unit, tab, y);
+      p.template decode<kU>(kbuf, at_k, t, unit, tab, pairs, y);
       float s[kH];
 #pragma unroll
       for (int h = 0; h < kH; ++h) {
@@ -295,7 +302,7 @@ __global__ void __launch_bounds__(32 * split_warps(kH), 1) split_attention_kerne
           for (int i = 0; i < kU / 2; ++i) acc[h][i] = f2_mul(acc[h][i], kk);
         }
       }
-      p.template decode<kU>(vbuf, at_v, t, unit, tab, y);
+      p.template decode<kU>(vbuf, at_v, t, unit, tab, pairs, y);
 #pragma unroll
       for (int h = 0; h < kH; ++h) {
         const float e = split_exp2(s[h] - m_run[h]);
@@ -522,7 +529,7 @@ int plan_split_as(const P& p, int64_t pairs, int max_len, SplitLoad* load) {
   auto kernel = split_attention_kernel<P, kH>;
   const int n_sm = configure_for_device(kernel, kSplitSmemMax, configured, true);
   if (n_sm == 0) return 0;
-  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
+  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes, P::kPairs);
   return split_cluster_size(p.c.d, p.c.tile, pairs * p.c.n_kv_heads, max_len,
                             [&](int i) { return clusters_at_once(kernel, 32 * split_warps(kH), smem, i, n_sm, memo); }, load);
 }
@@ -530,7 +537,7 @@ int plan_split_as(const P& p, int64_t pairs, int max_len, SplitLoad* load) {
 template <class P, int kH>
 int32_t launch_split_attention(const P& p, int64_t pairs, int max_len, cudaStream_t stream) {
   auto kernel = split_attention_kernel<P, kH>;
-  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes);
+  const int smem = split_smem_bytes(p.c.d, kH, p.c.stage_bytes, P::kPairs);
   if (smem > kSplitSmemMax) return PQ_ERR_UNSUPPORTED;
   SplitLoad load;
   const int C = plan_split_as<P, kH>(p, pairs, max_len, &load);
@@ -563,9 +570,10 @@ template <class P>
 void size_split(P& p) {
   const int kh = split_heads(p.c.n_q_heads / p.c.n_kv_heads), lanes = split_lanes(p.c.d, kh);
   int T = lanes == 1 ? 32 : 16;
-  while (T > 32 / lanes && split_smem_bytes(p.c.d, kh, p.tile_bytes(T)) > 200 * 1024) T /= 2;
+  while (T > 32 / lanes && split_smem_bytes(p.c.d, kh, p.tile_bytes(T), P::kPairs) > 200 * 1024) T /= 2;
   p.c.tile = T;
   p.c.stage_bytes = p.tile_bytes(T);
+  if constexpr (P::kDim != 0) p.c.tile = kh == 8 ? P::template tile_tokens<8>() : P::template tile_tokens<16>();   // the same
 }
 // The instantiation for the group size.
 template <class P>
