@@ -161,15 +161,15 @@ __device__ __forceinline__ int64_t ge_destination(const GenEncodeArgs& a, int ro
 
 // Bounds on the error of the product on tensor cores relative to ||x||_2, as rot_err in the kernel and rotation_block_error: products
 // of bf16 values are exact in float32, the three terms represent S to 2^-26, and each of the six accumulating MMAs of a slice is
-// taken to add at most 2 * 2^-24 of its running sum, which is at most the norm of the slice of x (twice that for the norm of a
-// block's errors); the slices' norms add up to sqrt(slices) ||x|| at most and their sums are added one by one.  Measured against
+// taken to add at most 2 * 2^-24 of the largest of its terms (16 products and the running sum); over the coordinates of a block the
+// squares of those add up to at most the squared norm of the slice of x, as they do for one coordinate; the slices' norms add up to sqrt(slices) ||x|| at most and their sums are added one by one.  Measured against
 // float64 over 2^20 vectors per head dim of 16 to 256 (normal, outlier channels, log-normal, concentrated, positive): at most 0.37
-// of the first bound (head_dim 32; 0.09 at 128) and 0.22 of the second.
+// of the first bound and 0.42 of the second (head_dim 32; 0.09 and 0.10 at 128).
 __host__ __device__ constexpr float ge_mma_error(int dc) {
   return 1.1f * (12.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
 }
 __host__ __device__ constexpr float ge_mma_block_error(int dc) {
-  return 1.02f * (24.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
+  return 1.02f * (12.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
 }
 
 // Three bf16 terms of a pair of float32 values (round to nearest each: together within 2^-26 of the values).
