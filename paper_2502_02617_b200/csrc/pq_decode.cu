@@ -120,11 +120,12 @@ struct DecodeArgs {
   int d, n_q_heads, n_kv_heads, batch, capacity, io_dtype;
   int n_q;  // queries per sequence (1: decode).  `batch` counts (sequence, query) pairs: q and out are
             // [batch][n_q_heads][d] with pair p = sequence * n_q + query; `lens` and the cache are per sequence.
-  const __half* qrot;  // of prefill_tc_kernel: the rotated queries [batch][n_q_heads][value | residual][128],
-  int n_splits;        // ranges of a sequence's blocks, each with a part of its own in
+  const __half* qrot;  // of prefill_tc_kernel and rows_attention_kernel: the rotated queries [batch][n_q_heads][value | residual][128]
+  int n_splits;        // of prefill_tc_kernel: ranges of a sequence's blocks, each with a part of its own in
   float* part_out;     // [split][batch][n_q_heads][128] (rotated basis) and
   float* part_lse;     // [split][batch][n_q_heads] (natural log)
-  int rows_per_block, n_row_blocks;   // of rows_attention_kernel: its cut of a kv head's n_q * group rows
+  int rows_per_block, n_row_blocks;   // of rows_attention_kernel: its cut of a kv head's n_q * group rows and, with qrot, where
+  int2* unit_parts;                   // it says which slots a unit's parts are in (first, number)
   float scale;
   uint32_t epoch;  // differs from call to call (top bit set): tags the parts' flags of the persistent kernel
   uint32_t debug;  // test hooks.  bit 0: the first bounded wait of CTA 0 of the persistent kernel reports failure;
@@ -674,16 +675,36 @@ static int32_t launch_rows_as(const DecodeArgs& a, bool paged, cudaStream_t stre
   return n_sm == 0 ? PQ_ERR_CUDA : launch_persistent(kernel, a, n_sm, kRowThreads, kRowSmTotal, stream);
 }
 static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq, bool paged, cudaStream_t stream) {
+// Groups of four rows that the instance for a row block of `rows` rows is built for.
+static int rows_groups(int rows) { return rows <= 8 ? 2 : rows <= 24 ? (rows + 3) / 4 : 8; }
   a.rows_per_block = cut.rows;
   a.n_row_blocks = cut.blocks;
-  a.ws = carve_workspace(a.ws.elected, 128, (int64_t)n_seq * a.n_kv_heads * cut.blocks, cut.rows);
+  const int64_t units = (int64_t)n_seq * a.n_kv_heads * cut.blocks;
+  a.ws = carve_workspace(a.ws.elected, 128, units, cut.rows);
   a.epoch = next_epoch();
-  if (cut.rows <= 8) return launch_rows_as<2>(a, paged, stream);
-  if (cut.rows <= 12) return launch_rows_as<3>(a, paged, stream);
-  if (cut.rows <= 16) return launch_rows_as<4>(a, paged, stream);
-  if (cut.rows <= 20) return launch_rows_as<5>(a, paged, stream);
-  if (cut.rows <= 24) return launch_rows_as<6>(a, paged, stream);
-  return launch_rows_as<8>(a, paged, stream);
+  // Several queries: their rotation, and the merge of the parts with the rotation back, are kernels before and after, whose set-up
+  // overlaps this one's.  Inside, a part's rotation of 20 rows takes 7 us and the last part of a unit 12 us for the merge and the
+  // rotation back, and a block that works on two units pays twice (draft of 5 tokens in four sequences of up to 8192 tokens, encode included: 73.9 -> 58.4 us).
+  // One query has at most eight rows, and its workspace may be the static scratch, which has no room for rotated queries.
+  if (a.n_q > 1) {
+    const int64_t all_rows = (int64_t)a.batch * a.n_q_heads;
+    uint8_t* behind = reinterpret_cast<uint8_t*>(a.ws.elected) + a.ws.bytes;
+    __half* qrot = reinterpret_cast<__half*>(behind);
+    a.qrot = qrot;
+    a.unit_parts = reinterpret_cast<int2*>(qrot + all_rows * 256);
+    const int32_t st = launch_rotate(a.S, a.q, a.io_dtype, all_rows, a.scale * 1.4426950408889634f, qrot, stream);
+    if (st != PQ_OK) return st;
+  }
+  int32_t st;
+  switch (rows_groups(cut.rows)) {
+    case 2: st = launch_rows_as<2>(a, paged, stream); break;
+    case 3: st = launch_rows_as<3>(a, paged, stream); break;
+    case 4: st = launch_rows_as<4>(a, paged, stream); break;
+    case 5: st = launch_rows_as<5>(a, paged, stream); break;
+    case 6: st = launch_rows_as<6>(a, paged, stream); break;
+    default: st = launch_rows_as<8>(a, paged, stream); break;
+  }
+  return st != PQ_OK || a.n_q == 1 ? st : launch_merge_rows(a, stream);
 }
 
 // ---- which kernel takes a head_dim-128 call ------------------------------------------------------
@@ -756,8 +777,15 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
   if (kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
     const RowCut cut = cut_rows(rows);
     const int64_t units = batch * n_kv_heads * cut.blocks;
-    const int groups = (cut.rows + 3) / 4;
-    est[kRowsKernel] = 18.2 + units * tiles * (278.0 + 50.0 * groups) / sm_hz + groups * (2.8 + 1.4 * more_units(units) + 0.9 * log_parts(units) / units);
+    if (n_q == 1) {
+      const int groups = (cut.rows + 3) / 4;
+      est[kRowsKernel] = 18.2 + units * tiles * (278.0 + 50.0 * groups) / sm_hz + groups * (2.8 + 1.4 * more_units(units) + 0.9 * log_parts(units) / units);
+    } else {
+      const int groups = rows_groups(cut.rows);
+      const double full = std::max(0.0, units / (double)n_sm - 1.0), all_rows = (double)pairs * n_kv_heads * g;
+      est[kRowsKernel] = 13.7 + units * tiles * (231.0 + 58.5 * groups) / sm_hz + groups * (0.7 + 0.28 * more_units(units)) + 3.7 * log_parts(units) / units -
+                         1.3 * full + 3.6e-3 * all_rows + 2.9e-3 * std::min(all_rows, 2368.0);
+    }
   }
   if (tensor) {
     const int qb_rows = kPtRows / g;
@@ -832,7 +860,8 @@ int64_t pq_workspace_bytes(int32_t head_dim, int32_t batch, int32_t n_q_heads, i
   const int64_t one = pq::carve_workspace(nullptr, head_dim, units, g).bytes;
   if (head_dim != 128) return one;
   const int64_t rows = units * (g + 3) + 32 * pq::kFastMaxGridHost;
-  const int64_t cut = 4 * 256 + units * 4 + (units + pq::kFastMaxGridHost) * 4 + rows * (2 + 128) * 4;
+  // ... and, for several queries, the rotated queries and a record per unit
+  const int64_t cut = 6 * 256 + units * 4 + (units + pq::kFastMaxGridHost) * 4 + rows * (2 + 128) * 4 + (int64_t)batch * n_q_heads * 512 + units * 8;
   const int64_t parts = 1024 + (int64_t)batch * n_q_heads * 512 + pq::part_rows_room(batch, n_q_heads) * (1 + 128) * 4;
   return std::max(std::max(cut, one), parts);
 }
@@ -864,7 +893,7 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   a.lse = lse_dev;
   a.pg = pg;
   a.ws = pq::carve_workspace(workspace_dev, head_dim, pairs * n_kv_heads, n_q_heads / n_kv_heads);
-  a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.qrot = nullptr; a.epoch = a.debug = 0u;
+  a.rows_per_block = a.n_row_blocks = 0; a.n_splits = 1; a.part_out = a.part_lse = nullptr; a.qrot = nullptr; a.unit_parts = nullptr; a.epoch = a.debug = 0u;
   const int g = n_q_heads / n_kv_heads;
   if (lse_dev != nullptr && n_q != 1) return PQ_ERR_UNSUPPORTED;
   pq::SplitCommon c;

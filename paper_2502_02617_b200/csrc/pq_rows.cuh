@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   // a programmatic dependent of the kernel before it, like the persistent kernel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();   // the barriers are initialised
-  if (warp == 0) fetch_S(a.S, sm_base + kRowSmRing, sm_base + kRowSmBarS, lane);   // a constant of the caller, like the tables
+  const bool around = a.qrot != nullptr;   // the rotations are kernels of their own, see launch_rows_attention
+  if (warp == 0 && !around) fetch_S(a.S, sm_base + kRowSmRing, sm_base + kRowSmBarS, lane);   // a constant of the caller, like the tables
   build_fast_tables<kRowThreads>(smem, a.tables);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
@@ -175,6 +176,10 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
     return (len_u + kStageTokens - 1) / kStageTokens;
   };
   auto empty_unit = [&](int u) {   // no row sees a token: zeros, and the status says so
+    if (around) {
+      a.unit_parts[u] = make_int2(0, 0);
+      return;
+    }
     const int seq = u / (a.n_kv_heads * nrb), rb = u % nrb, hk = (u / nrb) % a.n_kv_heads, n_rows = unit_rows(rb);
 #pragma unroll 1
     for (int e = 0; e < n_rows * 128; ++e) {
@@ -229,17 +234,37 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         bulk_load(ring + s * kStageBytes, src, bytes, sm_base + kSmBar + 8 * s);
         issued = li + 1;
       };
-      if (warp == 0 && batch_no + sg > 0) fetch_S(a.S, ring, bar_S, lane);
+      auto first_copies = [&]() {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
+      };
+      if (around) {
+        if (tid == 0) first_copies();
+      } else if (warp == 0 && batch_no + sg > 0) {
+        fetch_S(a.S, ring, bar_S, lane);
+      }
       int2* info = reinterpret_cast<int2*>(smem + kRowSmInfo);
       if (warp == 1) {
         const int row = row0 + min(lane, n_rows - 1), j = row / g_heads;
         info[lane] = make_int2((seq * a.n_q + j) * a.n_q_heads + hk * g_heads + (row - j * g_heads),
                                lane < n_rows ? a.lens[seq] - (a.n_q - 1 - j) : 0);
       }
-      // q' = (q S) * scale * log2(e) of the rows, 16 rows at a time, as fp16 value + residual in fragment order: the fragment of
+      // q' = (q S) * scale * log2(e) of the rows as fp16 value + residual in fragment order: the fragment of
       // (row group, k-step ks, lane) holds, for column n = lane / 4 (row n / 2 of the group; value or residual), coordinates
-      // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.
-      {
+      // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.  Read as it is where it was formed before, else formed 16 rows
+      // at a time.
+      if (around) {
+        __syncthreads();   // info
+        static_assert(kRowThreads == 8 * 32, "a thread per fragment of a row group");
+        const int ks = tid >> 5, at = (lane >> 2 & 1) * 128 + (2 * (lane & 3) + (ks >> 2)) * 16 + (ks & 3) * 4;
+        uint2 frag[kHG];
+#pragma unroll
+        for (int hg = 0; hg < kHG; ++hg)   // rows past the last repeat it
+          frag[hg] = __ldcg(reinterpret_cast<const uint2*>(a.qrot + (int64_t)info[4 * hg + (lane >> 3)].x * 256 + at));
+#pragma unroll
+        for (int hg = 0; hg < kHG; ++hg) *reinterpret_cast<uint2*>(smem + kRowSmQ + hg * 2048 + tid * 8) = frag[hg];
+        __syncthreads();
+      } else {
         float* q_in = reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn);
         constexpr int kAt = 4 * kHG < 16 ? 4 * kHG : 16, kMine = kAt / 2;   // rows at a time; rows of a thread
         const int j = tid & 127, r_mine = (tid >> 7) * kMine;               // its rotated coordinate
@@ -292,10 +317,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         }
         __syncthreads();   // S has been used: the ring takes its place
       }
-      if (tid == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
-      }
+      if (tid == 0 && !around) first_copies();
       float o_acc[kHG][4][4];
       float m_run[kHG], l_run[kHG];   // of row c + 4 hg, as in the persistent kernel
       int limit[kHG];                 // tokens the row sees
@@ -500,6 +522,11 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         }
         __stcg(reinterpret_cast<float2*>(a.ws.ml) + (int64_t)slot * R + tid, make_float2(M, l));
       }
+      if (around) {   // merge_rows_kernel does the rest
+        if (part == 0 && tid == 0) a.unit_parts[u] = make_int2(unit_slot, n_parts);
+        __syncthreads();   // the ring is free again for the next unit
+        continue;
+      }
       __syncthreads();
       if (warp == 0) elect_combiner(a, u, unit_slot, part, n_parts, lane, is_last);
       __syncthreads();
@@ -514,7 +541,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   }
   // A block whose range of the work lies between two units has no segment: the copy of S that it started ahead of the split lands
   // before the block ends.
-  if (n_S == 0) wait_S(bar_S, 0u, abort_flag);
+  if (n_S == 0 && !around) wait_S(bar_S, 0u, abort_flag);
   if (tid == 0 && *abort_flag) set_status(a.status, PQ_ERR_TIMEOUT);
 }
 
