@@ -180,11 +180,11 @@ struct PackedSplit {
   const int32_t* lens;
   Paging pg;
 
-  static int tile_bytes(int n) { return n * kRow; }
   // Tokens of a tile, as size_split chooses them (packed rows are short): a constant, so that the planes of a staged tile are at
   // constant distances.
   template <int kU>
   __host__ __device__ static constexpr int tile_tokens() { return D <= kU ? 32 : 16; }
+  static int tile_bytes(int n) { return n * kRow; }
   __device__ __forceinline__ int len(int pair) const {
     const int b = pair / n_q, v = lens[b] - (n_q - 1 - (pair - b * n_q));
     return v > 0 ? v : 0;
@@ -192,7 +192,6 @@ struct PackedSplit {
   __device__ __forceinline__ void fill_tables(float2* tab, int tid) const {
     if (tid < PQ_N_CENTROIDS) tab[tid] = make_float2(tables->cen_cos[tid], tables->cen_sin[tid]);
   }
-  __device__ __forceinline__ int shift(int, int, int, int) const { return 0; }
   __device__ __forceinline__ void fill_pairs(float4* pairs, int tid, int n_threads) const {
 #pragma unroll 4
     for (int i = tid; i < 256 * 8; i += n_threads) {
@@ -200,6 +199,7 @@ struct PackedSplit {
       pairs[i] = make_float4(tables->cen_cos[a], tables->cen_sin[a], tables->cen_cos[b], tables->cen_sin[b]);
     }
   }
+  __device__ __forceinline__ int shift(int, int, int, int) const { return 0; }
   __device__ __forceinline__ void stage(uint8_t* buf, int pair, int hk, int kv, int t0, int, int lane) const {
     Layout L;
     L.block_bytes = kBlockBytes;
@@ -265,7 +265,6 @@ struct PackedSplit {
         r1[2 * j + 1] = r2[j] * e.y;
       }
     }
-#pragma unroll
     if (kPairs) {
 #pragma unroll
       for (int j = 0; j < kU / 4; ++j) {   // byte j of the codes: 128 bytes per entry of the table
@@ -277,10 +276,12 @@ struct PackedSplit {
         y[4 * j + 3] = r1[2 * j + 1] * e.w;
       }
     } else {
-    for (int j = 0; j < kU / 2; ++j) {
-      const float2 e = tab[(l1 >> (4 * j)) & 15u];
-      y[2 * j] = r1[j] * e.x;
-      y[2 * j + 1] = r1[j] * e.y;
+#pragma unroll
+      for (int j = 0; j < kU / 2; ++j) {
+        const float2 e = tab[(l1 >> (4 * j)) & 15u];
+        y[2 * j] = r1[j] * e.x;
+        y[2 * j + 1] = r1[j] * e.y;
+      }
     }
   }
 };
@@ -674,9 +675,9 @@ static int32_t launch_rows_as(const DecodeArgs& a, bool paged, cudaStream_t stre
   const int n_sm = configure_for_device(kernel, kRowSmTotal, configured[paged ? 1 : 0]);
   return n_sm == 0 ? PQ_ERR_CUDA : launch_persistent(kernel, a, n_sm, kRowThreads, kRowSmTotal, stream);
 }
-static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq, bool paged, cudaStream_t stream) {
 // Groups of four rows that the instance for a row block of `rows` rows is built for.
 static int rows_groups(int rows) { return rows <= 8 ? 2 : rows <= 24 ? (rows + 3) / 4 : 8; }
+static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq, bool paged, cudaStream_t stream) {
   a.rows_per_block = cut.rows;
   a.n_row_blocks = cut.blocks;
   const int64_t units = (int64_t)n_seq * a.n_kv_heads * cut.blocks;
@@ -684,8 +685,9 @@ static int rows_groups(int rows) { return rows <= 8 ? 2 : rows <= 24 ? (rows + 3
   a.epoch = next_epoch();
   // Several queries: their rotation, and the merge of the parts with the rotation back, are kernels before and after, whose set-up
   // overlaps this one's.  Inside, a part's rotation of 20 rows takes 7 us and the last part of a unit 12 us for the merge and the
-  // rotation back, and a block that works on two units pays twice (draft of 5 tokens in four sequences of up to 8192 tokens, encode included: 73.9 -> 58.4 us).
-  // One query has at most eight rows, and its workspace may be the static scratch, which has no room for rotated queries.
+  // rotation back, and a block that works on two units pays twice (five drafted tokens in four sequences of up to 8192 tokens, encode
+  // included: 73.9 -> 58.4 us).  One query has at most eight rows, and its workspace may be the static scratch, which has no room for
+  // rotated queries.
   if (a.n_q > 1) {
     const int64_t all_rows = (int64_t)a.batch * a.n_q_heads;
     uint8_t* behind = reinterpret_cast<uint8_t*>(a.ws.elected) + a.ws.bytes;
@@ -710,14 +712,16 @@ static int rows_groups(int rows) { return rows <= 8 ? 2 : rows <= 24 ? (rows + 3
 // ---- which kernel takes a head_dim-128 call ------------------------------------------------------
 // Four kernels compute the same attention; which is fastest depends on the rows per kv head (queries x heads of the group), on
 // the number of (kv head, sequence) units and on the length.  Each is estimated in us by a formula fitted to measurements on
-// B200 (SM clock 1.9 GHz; 1 to 64 queries, 1 to 16 sequences of 150 to 32768 tokens, 32/8, 28/4, 20/4, 16/2, 8/8, 8/4, 8/2 and 8/1
-// heads), and the shortest estimate wins; over those calls the choice is 0.3 % slower than the best one on average, 20 % at worst:
+// B200 (SM clock 1.9 GHz; 1 to 64 queries, 1 to 32 sequences of 150 to 65536 tokens, 32/8, 28/4, 16/2, 8/8 and 8/1 heads: 2986
+// calls, up to four kernels each), and the shortest estimate wins; over those calls the choice is 0.3 % slower than the best
+// one on average, 28 % at worst (2.5 % and 55 % with the estimates of the kernels before their tables and rotations changed):
 //   * cluster kernel, a unit per (query, kv head, sequence): start and end, then per token of a block and wave;
-//   * persistent kernel, a unit per (query, kv head, sequence) too: start and end, then 268 SM cycles per 16-token tile (320 with
+//   * persistent kernel, a unit per (query, kv head, sequence) too: start and end, then 215 SM cycles per 16-token tile (256 with
 //     more than four heads), more where a block has several units, and the merge of a unit's parts;
-//   * rows kernel, up to 32 rows decoded together: the same with 2.8 us per group of four rows and 278 + 50 groups cycles per tile;
-//   * tcgen05 kernel, up to 256 rows per decoded block, from 32 rows on: 1.1 us per 64-token block of a pair of CTAs; rotating the
-//     queries before and merging and rotating back after grow with the rows and the parts.
+//   * rows kernel, up to 32 rows decoded together: 231 + 58 groups cycles per tile; several queries: start, end and per row the
+//     rotations before and after, which are kernels of their own; one query: 2.8 us per group of four rows inside;
+//   * tcgen05 kernel, up to 256 rows per decoded block, from 32 rows on: 1.09 us per 64-token block of a pair of CTAs; rotating the
+//     queries before and merging and rotating back after grow with the rows and the parts; never below 19.5 us.
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
@@ -771,8 +775,8 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
   if (kernel_takes(kPersistentKernel, batch, n_q, n_kv_heads, g)) {
     const int64_t units = pairs * n_kv_heads;
     const double full = std::max(0.0, units / (double)n_sm - 1.0);
-    est[kPersistentKernel] = g <= 4 ? 16.2 + units * tiles * 268.0 / sm_hz + 3.6 * more_units(units) + 5.2 * full + 1.2 * log_parts(units) / units
-                                    : 20.8 + units * tiles * 320.0 / sm_hz + 5.2 * more_units(units) + 9.1 * full + 2.9 * log_parts(units) / units;
+    est[kPersistentKernel] = g <= 4 ? 15.3 + units * tiles * 215.0 / sm_hz + 4.2 * more_units(units) + 3.8 * full + 0.5 * log_parts(units) / units
+                                    : 20.0 + units * tiles * 256.0 / sm_hz + 6.0 * more_units(units) + 7.8 * full + 2.8 * log_parts(units) / units;
   }
   if (kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
     const RowCut cut = cut_rows(rows);
@@ -794,8 +798,8 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
       const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s, at_once = n_sm / 2;   // two query blocks each
       const double waves = (double)((clusters + at_once - 1) / at_once), work = waves * ((blocks + s - 1) / s);
-      const double t = 18.0 + 1.11 * work + 1.1 * std::min(work, 4.0) + 5.2 * clusters / (at_once * waves) + 20.0 * (waves - 1.0) +
-                       2.6e-3 * std::min<int64_t>(all_rows, 3000) + 1.06e-3 * all_rows + 0.36e-3 * s * all_rows;
+      const double t = std::max(19.5, 15.1 + 1.086 * work + 0.72 * std::min(work, 4.0) + 8.8 * (waves - 1.0) +
+                                          2.3e-3 * std::min<int64_t>(all_rows, 2368) + 1.98e-3 * all_rows + 0.08e-3 * s * all_rows);
       if (t < est[kTensorKernel]) {
         est[kTensorKernel] = t;
         plan.n_splits = s;
