@@ -1,26 +1,27 @@
 // Tensor-core encoder for head_dim 128, bf16 inputs (included by pq_encode.cu).
 //
-// Persistent CTAs (one per SM, 16 warps) loop over tiles of 128 rows x one (K|V, head).  The 16 warps form
-// four groups ("slots") of four warps; a slot owns one of four 128-column accumulators in tensor memory
-// and takes every fourth tile of the CTA.  Per tile
+// Persistent CTAs (one per SM, 16 warps) loop over tiles of 128 rows x one (K|V, head).  One warp feeds the tensor core, twelve warps
+// quantise: three groups of four, each with every third tile of the CTA.  Four 128-column accumulators in tensor memory go round
+// the tiles, so the next tile is multiplied while the groups work on theirs.  Per tile
 //   * TMA loads of the x tile (two 64-column boxes, 128-byte swizzle) into a 3-deep ring; the copy of
 //     tile i+3 is issued as soon as the MMAs of tile i, which read the same ring stage, have completed;
 //   * y = x . S on the 5th-generation tensor cores: S is split once per CTA into three bf16 terms (exact
 //     for a float32 S) kept in shared memory as the K-major B operand; 3 terms x 8 k-steps of tcgen05.mma
-//     (M = 128 rows, N = 128, K = 16) accumulate in float32 in the slot's accumulator.  One thread of the
-//     slot issues them for the slot's next tile as soon as the current tile's last coordinates have been
-//     read into registers, so the tensor work runs under the quantiser of the last two blocks (and the
-//     other three slots are in their epilogues anyway);
-//   * epilogue on the slot's four warps.  Tensor-memory lane = row and a warp may read its own quarter of
+//     (M = 128 rows, N = 128, K = 16) accumulate in float32;
+//   * epilogue on the group's four warps.  Tensor-memory lane = row and a warp may read its own quarter of
 //     the lanes, so a thread owns one whole row (8 blocks): one pass over the accumulator for the row norm
 //     (the certified margins need it), a second pass of tcgen05.ld of 32 coordinates at a time through the
 //     sign-test quantiser, packed stores of whole plane entries of the token, queued float64 re-decision of
-//     the ambiguous angles (one queue per slot; all 16 warps take them together after the CTA's last tile,
-//     a slot drains alone only when its queue fills up).
+//     the ambiguous angles (one queue per group; all 16 warps take them together after the CTA's last tile,
+//     a group drains alone only when its queue fills up).
 // Per-row work (norm, margins, cache destination, stores) is paid once per 8 blocks, and the only
-// synchronisation in the loop is two named barriers of the slot's 128 threads per tile.
-// There are no dedicated producer / MMA warps: the register file is split over four schedulers, and
-// a 17th warp would cap every thread at 96 registers (the quantiser then spills).
+// synchronisation in the loop is one named barrier of the group's 128 threads per tile.
+// Sixteen quantising warps in four groups, whose warps issued copies and MMAs themselves, quantised for two thirds of the time: issuing 24
+// MMAs takes 1700 to 2700 of a tile's 17000 cycles, the wait for their inputs up to 4000, and the group's other warps waited at the
+// end of the tile for that one.  Twelve that only quantise take a tile in 12200 (three at a time instead of four).  (A 17th warp
+// instead of twelve and four would cap every thread at 96 registers.)  Back to back, 8 heads: 32768 tokens 90.4 -> 86.0 us, 16384
+// 52.0 -> 48.8, 5400 29.6 -> 26.7, but 4000 24.0 -> 24.6: four tiles per CTA are two rounds.  A queue per warp instead of the group's
+// barrier: 16384 tokens 50.2 us.
 // Every mbarrier wait is bounded; a wait that gives up raises the CTA's abort flag, the remaining
 // tiles are skipped (the loops keep their shape, so the named barriers stay consistent), copies in
 // flight are drained, tensor memory is released and PQ_ERR_TIMEOUT is recorded.
@@ -32,8 +33,9 @@
 namespace pq {
 
 constexpr int kTcThreads = 512;
-constexpr int kTcSlots = 4;                // accumulators in tensor memory = groups of four warps
-constexpr int kTcSlotThreads = kTcThreads / kTcSlots;
+constexpr int kTcGroups = 3;               // groups of four quantising warps; the fourth four: one warp for copies and MMAs
+constexpr int kTcGroupThreads = 128;
+constexpr int kTcAccs = 4;                 // accumulators in tensor memory
 constexpr int kTcStages = 3;               // x tiles in flight
 constexpr int kTcTerms = 3;                // bf16 terms of S (exact for a float32 S)
 constexpr int kTcXBytes = 128 * 128 * 2;   // one x tile: 128 rows x 128 bf16
@@ -42,15 +44,16 @@ using TcFixQueue = FixQueueT<256>;
 constexpr int kTcSmS = 0;
 constexpr int kTcSmX = kTcSmS + kTcTerms * kTcSBytes;
 constexpr int kTcSmFq = kTcSmX + kTcStages * kTcXBytes;      // FastQuant
-constexpr int kTcSmBar = kTcSmFq + kFastQuantBytes;                       // x_full[kTcStages], acc_full[kTcSlots]
-constexpr int kTcSmMisc = kTcSmBar + 64;                     // tmem base, abort flag, copies issued per stage
-constexpr int kTcSmFix = kTcSmMisc + 64;                     // one TcFixQueue per slot
-constexpr int kTcSmL1 = kTcSmFix + kTcSlots * (int)sizeof(TcFixQueue);  // copy of Tables::l1_cells (codebooks other than the analytic ones)
+constexpr int kTcSmBar = kTcSmFq + kFastQuantBytes;                       // x_full[kTcStages], acc_full[kTcAccs], acc_empty[kTcAccs]
+constexpr int kTcSmMisc = kTcSmBar + 128;                    // tmem base, abort flag, copies issued per stage
+constexpr int kTcSmFix = kTcSmMisc + 64;                     // one TcFixQueue per group, or the histogram
+constexpr int kTcFixBytes = kTcGroups * (int)sizeof(TcFixQueue) > 4 * PQ_HIST_MAX_BINS * 4 ? kTcGroups * (int)sizeof(TcFixQueue) : 4 * PQ_HIST_MAX_BINS * 4;
+constexpr int kTcSmL1 = kTcSmFix + kTcFixBytes;              // copy of Tables::l1_cells (codebooks other than the analytic ones)
 constexpr int kTcSmTotal = kTcSmL1 + 8 * kL1Cells * 8 + 1024;             // + slack for 1024-byte alignment
 static_assert(kTcTerms == 3, "kRotErrTc is the bound for three terms");
 static_assert(sizeof(TcFixQueue) % 16 == 0, "queues are laid out back to back");
 static_assert(kTcSmTotal <= 227 * 1024, "shared memory of one CTA");
-static_assert(4 * PQ_HIST_MAX_BINS * 4 <= kTcSlots * (int)sizeof(TcFixQueue), "the histogram takes the queues' place");
+static_assert(8 * (kTcStages + 2 * kTcAccs) <= 128, "barriers");
 static_assert(kFixSdBytes <= kTcSmFq, "the float64 copy of S must fit in the operand buffers");
 
 struct TcMaps {
@@ -89,22 +92,18 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
   // completed and its writes are visible, so only its launch latency is hidden.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int quarter = warp & 3;            // tensor-memory lanes this warp may read: rows 32 * quarter ..
-  const int slot = warp >> 2;              // accumulator and tile sequence of this group of four warps
-  const int st = quarter * 32 + lane;      // thread index inside the slot = row of the tile
-  // The slot's issuing thread (TMA, MMAs).  The four warps of a slot sit on the four schedulers; the issuing threads
-  // of the four slots are spread over them too, so that no scheduler carries all of that extra work (the other
-  // warps of a slot would wait for the slow one at every barrier).
-  const bool leader = quarter == slot && lane == 0;
+  const int group = warp >> 2;             // of quantising warps; kTcGroups: the warp that feeds the tensor core and three idle ones
+  const int st = quarter * 32 + lane;      // thread index inside the group = row of the tile
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kTcSmMisc + 4);
   volatile int* copies_issued = reinterpret_cast<volatile int*>(smem + kTcSmMisc + 8);  // [kTcStages]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kTcSmMisc);
   FastQuant* fq = reinterpret_cast<FastQuant*>(smem + kTcSmFq);
-  TcFixQueue* fixq = reinterpret_cast<TcFixQueue*>(smem + kTcSmFix) + slot;
-  const uint32_t bar_xfull = sb + kTcSmBar, bar_acc = bar_xfull + 8 * kTcStages;
+  TcFixQueue* fixq = reinterpret_cast<TcFixQueue*>(smem + kTcSmFix) + min(group, kTcGroups - 1);
+  const uint32_t bar_xfull = sb + kTcSmBar, bar_acc = bar_xfull + 8 * kTcStages, bar_free = bar_acc + 8 * kTcAccs;
   const int n_tiles = n_row_tiles * 2 * a.n_kv_heads;
 
   // Local tile `it` of this CTA is tile blockIdx.x + it * gridDim.x = head + n_kv_heads * (2 * row tile + kv); it
-  // uses ring stage it % kTcStages and belongs to slot it % kTcSlots.
+  // uses ring stage it % kTcStages and accumulator it % kTcAccs and belongs to group it % kTcGroups.
   // One thread issues the TMA loads of local tile `it`.  The caller knows that the stage is free: the MMAs of
   // local tile it - kTcStages, which read it, have completed.
   auto issue_tma = [&](int it) {
@@ -131,7 +130,10 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
       tc_mbar_init(bar_xfull + 8 * s, 1);
       copies_issued[s] = 0;
     }
-    for (int i = 0; i < kTcSlots; ++i) tc_mbar_init(bar_acc + 8 * i, 1);   // one commit by the slot's issuing thread
+    for (int i = 0; i < kTcAccs; ++i) {
+      tc_mbar_init(bar_acc + 8 * i, 1);    // one commit by the issuing thread
+      tc_mbar_init(bar_free + 8 * i, 4);   // the four warps that have read the accumulator
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Launched as a programmatic dependent of the kernel before it in the stream (which may have produced K and V):
@@ -144,7 +146,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
   if (kHist) {
     for (int i = tid; i < 4 * a.n_bins; i += kTcThreads) hist_s[i] = 0u;
   } else {
-    if (st < 4) fixq->count[st] = 0;
+    if (group < kTcGroups && st < 4) fixq->count[st] = 0;
     if ((a.tables->flags & (kFlagSymmetricUpper | kFlagUniformL1)) != (kFlagSymmetricUpper | kFlagUniformL1)) {
       const uint2* src = &a.tables->l1_cells[0][0];
       uint2* dst = reinterpret_cast<uint2*>(smem + kTcSmL1);
@@ -196,62 +198,74 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
 
-  // The slot's issuing thread multiplies local tile `it` into the slot's accumulator.  The accumulator is free:
-  // the slot's four warps have read the previous tile out of it before the barrier that precedes this call.
-  // All MMAs of the tile come from this thread, in order: the first overwrites, the others accumulate.
   const uint64_t desc_hi = tc_smem_desc(0u) & 0xFFFFFFFF00000000ull;  // the address field is in the low word
   const uint32_t bdesc_lo = (uint32_t)tc_smem_desc(sb + kTcSmS);
-  auto issue_mmas = [&](int it) {
-    if (blockIdx.x + it * (int)gridDim.x >= n_tiles) return;
-    const int s = it % kTcStages;
-    // The copy of the tile is issued by another slot's thread (when the tile kTcStages back has been
-    // multiplied).  A parity wait taken before that would be satisfied by the stage's previous phase, so
-    // first wait (bounded) until the copy has been issued: the previous phase is complete by then.
-    bool ok = false;
-    for (int i = 0; i < kTcSpin && !ok; ++i) {
-      ok = copies_issued[s] > it / kTcStages;
-      if (!ok && i > 32) {
-        __nanosleep(64);
-        if (*abort_flag) break;
+
+  // ---- the warp that feeds the tensor core.  It goes through its loop as a whole and one elected lane issues, so that the operands
+  // of the MMAs are warp-uniform values.  All MMAs of a tile come from one thread, in order: the first overwrites, the others accumulate.
+  if (warp == 4 * kTcGroups) {
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+    int n_local = ((int)n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, issued = 0;
+    n_local = __shfl_sync(0xffffffffu, n_local, 0);
+    for (int it = 0; it < n_local; ++it) {
+      const int s = it % kTcStages, acc = it % kTcAccs;
+      bool ok = tc_mbar_wait(bar_xfull + 8 * s, (it / kTcStages) & 1, abort_flag);
+      if (ok && it >= kTcAccs) ok = tc_mbar_wait(bar_free + 8 * acc, (it / kTcAccs - 1) & 1, abort_flag);
+      if (ok && (a.debug & 1u) && blockIdx.x == 0 && it == 0) {  // test hook: report this wait as failed
+        *abort_flag = 1;
+        ok = false;
+      }
+      if (!__all_sync(0xffffffffu, ok)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t adesc_lo = (uint32_t)tc_smem_desc(sb + kTcSmX + s * kTcXBytes);
+      if (tc_elect()) {
+#pragma unroll
+        for (int q = 0; q < 8 * kTcTerms; ++q) {
+          const uint32_t off = ((q >> 2) & 1) * 16384 + (q & 3) * 32;  // k-half, k-step inside the 128-byte swizzled row
+          tc_mma(tmem_u + acc * 128, desc_hi | (adesc_lo + (off >> 4)), desc_hi | (bdesc_lo + (((q >> 3) * kTcSBytes + off) >> 4)),
+                 q ? 1u : 0u);
+        }
+        tc_commit(bar_acc + 8 * acc);  // the accumulator is complete and the x stage has been read
+      }
+      __syncwarp();
+      issued = it + 1;
+      if (it >= 1 && it - 1 + kTcStages < n_local) {   // the stage of the tile before this one is free when its MMAs have completed
+        if (!__all_sync(0xffffffffu, tc_mbar_wait(bar_acc + 8 * ((it - 1) % kTcAccs), ((it - 1) / kTcAccs) & 1, abort_flag))) break;
+        if (lane == 0) issue_tma(it - 1 + kTcStages);
+        __syncwarp();
       }
     }
-    if (!ok) *abort_flag = 1;
-    ok = ok && tc_mbar_wait(bar_xfull + 8 * s, (it / kTcStages) & 1, abort_flag);
-    if (ok && (a.debug & 1u) && blockIdx.x == 0 && it == 0) {  // test hook: report this wait as failed
-      *abort_flag = 1;
-      ok = false;
+    // No MMA may be in flight when tensor memory is released, also where a wait gave up.
+    for (int it = max(0, issued - 2); it < issued; ++it) {
+      bool done = false;
+      for (int i = 0; i < (1 << 16) && !done; ++i) done = tc_mbar_try(bar_acc + 8 * (it % kTcAccs), (it / kTcAccs) & 1);
+      if (!done) *abort_flag = 1;
     }
-    if (!ok) return;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t adesc_lo = (uint32_t)tc_smem_desc(sb + kTcSmX + s * kTcXBytes);
-#pragma unroll
-    for (int q = 0; q < 8 * kTcTerms; ++q) {
-      const uint32_t off = ((q >> 2) & 1) * 16384 + (q & 3) * 32;  // k-half, k-step inside the 128-byte swizzled row
-      tc_mma(tmem_base + slot * 128, desc_hi | (adesc_lo + (off >> 4)),
-             desc_hi | (bdesc_lo + (((q >> 3) * kTcSBytes + off) >> 4)), q ? 1u : 0u);
-    }
-    tc_commit(bar_acc + 8 * slot);  // the accumulator is complete and the x stage has been read
-  };
+  }
 
-  // ---- tile loop of this slot
+  // ---- tile loop of this group
   constexpr int o2 = 32 * kTokenBlock, o3 = o2 + 8 * kTokenBlock, o4 = o3 + 4 * kTokenBlock, orad = o4 + 2 * kTokenBlock;
   const bool analytic = kHist || fq->analytic != 0u;  // uniform over the grid
   const float hist_scale1 = (float)a.n_bins * 0.159154943091895336f, hist_scale_up = (float)a.n_bins * 0.636619772367581343f;
   int hist_bad = 0;
   const Layout L = make_layout(128, a.pg.page_tokens);
-  const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + slot * 128;
-  const int slot_bar = 1 + slot;
+  const int group_bar = 1 + group;
   int rd_seq = 0, rd_first = 0, rd_count = 0, rd_start = -1;   // destination of the last row looked up
-  if (leader) issue_mmas(slot);
-  __syncwarp();
-  for (int it = slot; blockIdx.x + it * (int)gridDim.x < n_tiles; it += kTcSlots) {
+  for (int it = group; group < kTcGroups && blockIdx.x + it * (int)gridDim.x < n_tiles; it += kTcGroups) {
+    const int acc = it % kTcAccs;
+    const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * 128;
     const int tile = blockIdx.x + it * gridDim.x;
     const int head = tile % a.n_kv_heads, hq = tile / a.n_kv_heads;
     const int kv = hq & 1, rt = hq >> 1;
-    // A wait that gives up must not leave the loop: the other warps of the slot would wait for this one at the
-    // slot's barriers.  The tile is skipped instead (warp-uniform): it is quantised as zeros and not stored.
-    const bool ready = __all_sync(0xffffffffu, tc_mbar_wait(bar_acc + 8 * slot, (it / kTcSlots) & 1, abort_flag));
-    if (leader && ready) issue_tma(it + kTcStages);  // the stage of this tile is free again
+    // A wait that gives up must not leave the loop: the other warps of the group would wait for this one at the
+    // group's barrier.  The tile is skipped instead (warp-uniform): it is quantised as zeros and not stored.
+    const bool ready = __all_sync(0xffffffffu, tc_mbar_wait(bar_acc + 8 * acc, (it / kTcAccs) & 1, abort_flag));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    auto accumulator_read = [&]() {   // this warp's last coordinates are in registers
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0 && ready) tc_mbar_arrive(bar_free + 8 * acc);
+    };
     const int row = rt * 128 + st;
     const int64_t xoff = (int64_t)row * a.token_stride + (int64_t)head * a.head_stride;
     uint8_t* tb = nullptr;
@@ -264,12 +278,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
         if (ready) tc_ld32(taddr + 32 * c, y);
-        if (c == 3) {  // as below: the accumulator is free for the slot's next tile
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          asm volatile("bar.sync %0, %1;" ::"r"(slot_bar), "n"(kTcSlotThreads) : "memory");
-          if (leader) issue_mmas(it + kTcSlots);
-          __syncwarp();
-        }
+        if (c == 3) accumulator_read();
         if (ready && row < a.total_tokens) {
           hist_bad += !hist_block(y, hist_s, a.n_bins, hist_scale1, hist_scale_up);
           hist_bad += !hist_block(y + 16, hist_s, a.n_bins, hist_scale1, hist_scale_up);
@@ -280,7 +289,6 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     // pass 1: squared norm of the row (four partial sums)
     float sq[4] = {0.f, 0.f, 0.f, 0.f};
     if (ready) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
         tc_ld32(taddr + 32 * c, y);
@@ -323,14 +331,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
       if (ready) tc_ld32(taddr + 32 * c, y);
-      if (c == 3) {
-        // The last coordinates are in registers: the accumulator is free.  The slot's next tile is multiplied
-        // while this one's last two blocks are quantised.
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        asm volatile("bar.sync %0, %1;" ::"r"(slot_bar), "n"(kTcSlotThreads) : "memory");
-        if (leader) issue_mmas(it + kTcSlots);
-        __syncwarp();
-      }
+      if (c == 3) accumulator_read();
       FastBlock fb0, fb1;
       if (analytic) {
         polar_quant_block_fast<true>(y, rm, *fq, &fb0);
@@ -370,12 +371,12 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
       *reinterpret_cast<uint16_t*>(tb + o4 + tok * 2) = (uint16_t)l4acc;
       if (sat) atomicAdd(a.status + 2, (int)sat);
     }
-    // End of the tile for the slot.  The barrier decides, for all 128 threads alike, whether the slot has to take
+    // End of the tile for the group.  The barrier decides, for all 128 threads alike, whether the group has to take
     // its queued exact re-decisions now: when a push did not fit or a region is 3/4 full.  Otherwise they wait
-    // for the end of the CTA's work, where all 16 warps take them together (the float64 pipe is slow, and a slot
+    // for the end of the CTA's work, where all 16 warps take them together (the float64 pipe is slow, and a group
     // that drains alone holds up its own tiles for as long).
-    const bool drain = bar_or(slot_bar, kTcSlotThreads, (left[0] | left[1]) != 0ull || fix_should_drain(fixq));
-    if (drain) fix_rounds(a, fixq, left, xoff, tb, tok, 0, kv, st, kTcSlotThreads, slot_bar);
+    const bool drain = bar_or(group_bar, kTcGroupThreads, (left[0] | left[1]) != 0ull || fix_should_drain(fixq));
+    if (drain) fix_rounds(a, fixq, left, xoff, tb, tok, 0, kv, st, kTcGroupThreads, group_bar);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -386,7 +387,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     }
     hist_flush(hist_s, 4 * a.n_bins, a.hist, tid, kTcThreads);
   }
-  // Every MMA and copy of this CTA has completed (each was waited for by its slot), so the operand buffers are
+  // Every MMA and copy of this CTA has completed (each was waited for), so the operand buffers are
   // idle: put a float64 copy of S there (rows permuted, see fix_sd_row) for the queued exact re-decisions.
   double* Sd = reinterpret_cast<double*>(smem + kTcSmS);
   if (!kHist && !*abort_flag) {
@@ -402,7 +403,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     __syncthreads();
   }
   if (!kHist)
-    fix_process(fixq - slot, kTcSlots, tid, kTcThreads, a.K, a.V, a.in_dtype, a.S, *abort_flag ? (const double*)nullptr : Sd,
+    fix_process(reinterpret_cast<TcFixQueue*>(smem + kTcSmFix), kTcGroups, tid, kTcThreads, a.K, a.V, a.in_dtype, a.S, *abort_flag ? (const double*)nullptr : Sd,
                 *a.tables, a.status);
   if (*abort_flag && tid < kTcStages && copies_issued[tid] > 0) {
     // gave up somewhere: let the copies that are still in flight land (bounded) before the CTA and its

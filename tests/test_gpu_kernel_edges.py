@@ -103,6 +103,30 @@ def test_single_query_kernels(d, g):
             assert rel_l2(out[b], want[b]) < TOL_ATTENTION_F32_IO, (kernel, lens[b])
 
 
+# The tensor-core encoder where a group's queue of uncertified decisions fills up again and again (zero rows, rows on the boundaries of an
+# unrotated codebook), at every number of tiles that its three groups of warps can be left with, against the float32 encoder: the same
+# codes and status counts, radii that are neighbours at most.
+@pytest.mark.parametrize("n", [128, 129, 640, 1700, 2500])
+@pytest.mark.parametrize("analytic", [True, False])
+def test_tensor_core_encoder_with_many_uncertified_decisions(n, analytic):
+    Hkv = 8
+    K, V = synthetic.kv_like(n, n, Hkv, 128, torch.bfloat16, DEV)
+    K[::3] = 0
+    V[5:90] = 1.0
+    cen, bnd = (t.clone() for t in pq.pq_fit_codebooks())
+    if not analytic:
+        cen[:16] += 0.01 * torch.cos(torch.arange(16, dtype=torch.float64))
+        bnd[:15] = 0.5 * (cen[:15] + cen[1:16])
+    cu = torch.tensor([0, n], dtype=torch.int32, device=DEV)
+    got = []
+    for dtype in (torch.bfloat16, torch.float32):
+        c = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=n, S=torch.eye(128), device=DEV, codebooks=(cen, bnd))
+        c.encode(K.to(dtype), V.to(dtype), cu)
+        got.append((*c.unpack(n), c.status[:3].tolist()))
+    assert torch.equal(got[0][0], got[1][0]) and got[0][2] == got[1][2]
+    assert torch.all((got[0][1].float() - got[1][1].float()).abs() <= 2.0 ** -10 * got[1][1].float())
+
+
 # Codebooks whose decode tables need the residuals of the level-1 factors and both halves of the level-4 factors (the analytic one
 # needs neither): every level moved, or the top level alone, in the three kernels that read those tables.
 @pytest.mark.parametrize("moved", [slice(0, 28), slice(24, 28)])
