@@ -370,7 +370,8 @@ static int32_t launch_merge(int d, int64_t n_rows, int n_parts, const void* part
 }
 
 // Exact softmax attention (Eq. 2) of one query per sequence over an uncompressed window of keys and values (the
-// tokens a serving loop keeps in 16 bits, Section 5.3's protocol for generated tokens).  One CTA per (kv head,
+// tokens a serving loop keeps in 16 bits, Section 5.3's protocol for generated tokens), whatever the head dim, the rows' type and the group;
+// bf16 rows of 128 with up to four heads go to tail_mma_kernel.  One CTA per (kv head,
 // sequence, split of the window's tokens); a CTA writes the partial attention of its tokens (part blockIdx.z of the
 // output), to be merged by merge_attention_kernel.  Steps of kTailStage tokens (half as many for a float32 window): the
 // key and value rows are copied to shared memory with coalesced 16-byte cp.async (all of a step's loads in flight at
@@ -405,9 +406,8 @@ __device__ __forceinline__ float tail_elem(const void* p, int dtype, int64_t i) 
 }
 // kHG = groups of four query heads per kv head (heads past the group read q' = 0 and are not stored).
 template <int kHG>
-__global__ void __launch_bounds__(kTailThreads) tail_attention_kernel(TailArgs a) {
+__device__ __forceinline__ void tail_attention(const TailArgs& a, float* tsm) {
   constexpr int kH = 4 * kHG;
-  extern __shared__ float tsm[];
   const int d = a.d, g = a.n_q_heads / a.n_kv_heads, hk = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   float* qs = tsm;                       // [d][kH]: q' = q * scale * log2(e), the heads of a coordinate side by side
@@ -559,6 +559,15 @@ __global__ void __launch_bounds__(kTailThreads) tail_attention_kernel(TailArgs a
     else if (len <= 0) set_status(a.status, PQ_ERR_EMPTY);
   }
 }
+template <int kHG>
+__global__ void __launch_bounds__(kTailThreads) tail_attention_kernel(const __grid_constant__ TailArgs a) {
+  extern __shared__ __align__(16) float tsm[];
+  tail_attention<kHG>(a, tsm);
+}
+
+}  // namespace pq
+#include "pq_tail_mma.cuh"
+namespace pq {
 
 // ---- inspection kernels ----------------------------------------------------------------------
 __global__ void unpack_codes_kernel(int d, int n_kv_heads, const uint8_t* cache, int batch, Paging pg,
@@ -1050,7 +1059,12 @@ int32_t pq_tail_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_kv_head
   if (pq::configure_for_device(pq::tail_attention_kernel<1>, pq::kTailSmemMax, configured1) == 0) return PQ_ERR_CUDA;
   if (pq::configure_for_device(pq::tail_attention_kernel<2>, pq::kTailSmemMax, configured2) == 0) return PQ_ERR_CUDA;
   dim3 grid(n_kv_heads, batch, n_splits);
-  if (g <= 4) pq::tail_attention_kernel<1><<<grid, pq::kTailThreads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+  if (head_dim == 128 && g <= 4 && kv_dtype == PQ_DTYPE_BF16) {
+    static pq::DeviceMemo configured_mma;
+    const int need = std::max((int)smem, pq::kTmSmTotal);   // a block may fall back on tail_attention
+    if (pq::configure_for_device(pq::tail_mma_kernel, pq::kTailSmemMax, configured_mma) == 0) return PQ_ERR_CUDA;
+    pq::tail_mma_kernel<<<grid, pq::kTailThreads, need, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+  } else if (g <= 4) pq::tail_attention_kernel<1><<<grid, pq::kTailThreads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
   else pq::tail_attention_kernel<2><<<grid, pq::kTailThreads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
   return pq::launch_status();
 }

@@ -392,3 +392,27 @@ def test_long_chunk_without_the_tcgen05_kernel():
     other = cache.attend_multi(q)
     pq.pq_debug_fail_next_wait(10)
     assert not torch.equal(cache.attend_multi(q), other)
+
+
+# The window on tensor cores (bf16 rows of 128, up to four heads per kv head) against the float32 kernel on the same rows: windows that end
+# around its 16-token tiles and its warps' shares, empty ones, more splits than tokens.  Exact products, float32 sums in another order:
+# 1e-5 is 2^-24 times the 128 terms of a score in the exponent.  Infinite and NaN rows give what the float32 kernel gives.
+@pytest.mark.parametrize("io", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("g,n_splits", [(1, 1), (2, 3), (3, 1), (4, 7)])
+def test_window_on_tensor_cores(g, n_splits, io):
+    lens, T, Hkv = [0, 1, 15, 16, 17, 63, 64, 65, 129, 300, 300, 300], 300, 2
+    B = len(lens)
+    K, V = (t.view(B, T, Hkv, 128) for t in synthetic.kv_like(g, B * T, Hkv, 128, torch.bfloat16, DEV))
+    K[10, 7, 0, 3], V[10, 200, 1, 5], V[11, 3, 0, 9], K[11, 250, 1, 0] = -float("inf"), float("inf"), float("nan"), float("nan")
+    q = synthetic.queries(3, B, g * Hkv, 128, io, DEV)
+    n = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    got = []
+    for kv in ((K, V), (K.float(), V.float())):
+        out, lse = torch.empty((n_splits, *q.shape), dtype=io, device=DEV), torch.empty((n_splits, *q.shape[:2]), device=DEV)
+        pq.pq_tail_attention(q, *kv, n, 128 ** -0.5, out, lse, torch.zeros(4, dtype=torch.int32, device=DEV), n_splits)
+        got.append((out.float(), lse))
+    tol = 1e-5 if io == torch.float32 else 2.0 ** -8
+    for a, b in zip(*got):
+        assert torch.equal(a.isnan(), b.isnan()) and torch.equal(a.isinf(), b.isinf())
+        ok = a.isfinite() & b.isfinite()
+        assert torch.all((a - b)[ok].abs() <= tol * b[ok].abs().clamp(min=1.0))
