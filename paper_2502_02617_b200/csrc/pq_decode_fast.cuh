@@ -69,15 +69,19 @@ constexpr int kMrgStride = 136;  // floats per (warp, head) row of the merge buf
 //   ring | T [256 bytes of level-1 codes]    16 x (cos a, cos b | sin a, sin b) in fp16, then 16 x the residuals of the same
 //        | U [256 half-block codes]          kFlagExactDecode: 8 x (values, residuals) for the keys, then 16 x values for the values;
 //                                            otherwise 8 x (values, residuals) of half 0, then 8 x of half 1
-//        | barriers, segments, q'
+//        | barriers, segments, q', places of a paged segment's stages
 constexpr uint32_t kWindowBase = 1024;
 constexpr uint32_t kFsRing = kWindowBase, kFsT = 0x10000, kFsU = 0x20000, kFsBar = 0x30000;
 constexpr uint32_t kFsFlags = kFsBar + 64, kFsSegs = kFsFlags + 16, kFsQ = kFsSegs + 768;
-constexpr uint32_t kFsEnd = kFsQ + 4096 + kQLo + 8 * kQHead;
+constexpr uint32_t kFsPlaces = kFsQ + 4096 + kQLo + 8 * kQHead;
+constexpr int kFsPlaceCap = 1024;                   // stages that are listed at a time
+constexpr uint32_t kFsEnd = kFsPlaces + 4 * kFsPlaceCap;
+constexpr int kPlaceUnit = 256;                     // a token-block's keys and values are 31 of them
 constexpr int kFsTotal = (int)(kFsEnd - kWindowBase);
 // after the main loop the ring is reused for the merge across the warps, four heads at a time: their accumulators, then (m, l)
 constexpr int kFsMergeMl = kFastConsumerWarps * 4 * kMrgStride * 4;
 static_assert(kFsRing + kStages * kStageBytes <= kFsT && kFsMergeMl + kFastConsumerWarps * 8 * 8 <= kStages * kStageBytes, "ring");
+static_assert(2 * kBlockBytes128 % kPlaceUnit == 0, "places of stages");
 static_assert(kFsTotal <= 227 * 1024, "shared memory of one CTA");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -771,7 +775,13 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     // stage of its own ahead; it waits (bounded) until the group's 8 warps have released the slot.
     const int n_li = st1 - st0 > wg ? (st1 - st0 - wg + 1) >> 1 : 0;
     int issued = 0;
-    auto issue_copy = [&](int li) -> bool {
+    auto stage_place = [&](int st) -> int64_t {
+      Layout Lp;  // the two fields the offset needs
+      Lp.block_bytes = kBlockBytes128;
+      Lp.head_bytes = head_bytes;
+      return kv_block_pair_offset(Lp, a.pg, a.n_kv_heads, seq, hk, 2 * st, a.status);
+    };
+    auto issue_copy = [&](int li, auto listed, uint32_t at) -> bool {   // at: where the place of a paged cache's stage stands, if it is listed
       const int gl = gl0 + li, s = 2 * wg + (gl & 1);
       if (gl >= 2 && !mbar_wait(sm_base + kFsBar + 8 * (kStages + s), ((gl >> 1) - 1) & 1, abort_flag)) return false;
       const int st = st0 + wg + 2 * li;
@@ -780,23 +790,32 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       mbar_expect_tx(sm_base + kFsBar + 8 * s, bytes);
       // a stage is two token-blocks, K | V | K | V, of one page (page_tokens is a multiple of 128)
       const uint8_t* src = head_base + (int64_t)st * kStageBytes;
-      if (kPaged) {
-        Layout Lp;  // the two fields the offset needs
-        Lp.block_bytes = kBlockBytes128;
-        Lp.head_bytes = head_bytes;
-        src = a.cache + kv_block_pair_offset(Lp, a.pg, a.n_kv_heads, seq, hk, 2 * st, a.status);
+      if constexpr (kPaged) {
+        if constexpr (decltype(listed)::value) src = a.cache + lds32i<0>(at) * (int64_t)kPlaceUnit;
+        else src = a.cache + stage_place(st);
       }
       bulk_load(sm_base + kFsRing + s * kStageBytes, src, bytes, sm_base + kFsBar + 8 * s);
       issued = li + 1;
       return true;
     };
+    // Where a paged segment's stages begin is listed in shared memory, kFsPlaceCap of them at a time and the first ones before the second
+    // copy is requested (a barrier of the rotation below lies between), so that the copying thread, whose warp has a tile of its own to
+    // work on, needs no division and waits for no table.  Looked up per stage they cost the whole kernel a tenth: 8 x 32768 tokens,
+    // 32/8 heads, pages of 256 131.9 us against 122.6 (contiguous 119.4); 16 x 20000 160.6 -> 148.0, 28/4 heads 88.1 -> 84.5.  Looked up
+    // inside the loop for stages beyond a longer list, the unused branch alone took 125.2: a list is made again instead.
+    auto list_places = [&](int first) {
+      for (int i = tid; i < min(kFsPlaceCap, st1 - st0 - first); i += kFastThreads)
+        reinterpret_cast<uint32_t*>(smem + kFsPlaces)[i] = (uint32_t)(stage_place(st0 + first + i) / kPlaceUnit);
+    };
+    constexpr int kWindow = kFsPlaceCap / 2 - 1;   // steps of the groups that a list is enough for, with the copies one step ahead
+    if (kPaged) list_places(0);
     const bool hook = !kPaged && (a.debug & 1u) && unit_slot == 0 && cta == c_first;
     const bool producer = (tid & 255) == 0;
     if (producer && n_li > 0) {
       // what list_segments, the merge or the combine left in the ring by ordinary accesses (a barrier has ordered them before this)
       // comes before the copies into it
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue_copy(0);
+      issue_copy(0, std::false_type{}, 0);
     }
     __syncwarp();
     // q' = (q S) * scale * log2(e) for the unit's query heads, as an fp16 value plus an fp16 residual.
@@ -856,12 +875,12 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       *reinterpret_cast<uint2*>(smem + kFsQ + hg * 2048 + ks * 256 + lane * 8) = q_fragment(hg, ks);
       __syncthreads();
     }
-    auto stream = [&](auto exact_tables) {
+    auto stream = [&](auto exact_tables, int first, int last) {
     constexpr bool kExact = decltype(exact_tables)::value;
-    for (int li = 0; li < n_li; ++li) {
+    for (int li = first; li < last; ++li) {
       const int gl = gl0 + li, s = 2 * wg + (gl & 1);
       const int st = st0 + wg + 2 * li;
-      if (producer && li + 1 < n_li) issue_copy(li + 1);
+      if (producer && li + 1 < n_li) issue_copy(li + 1, std::true_type{}, kPaged ? sm_base + kFsPlaces + 4 * wg + 8 * (li + 1 - first) : 0);
       __syncwarp();
       if (!mbar_wait(sm_base + kFsBar + 8 * s, (gl >> 1) & 1, abort_flag)) break;
       if ((kPaged ? (a.debug & 1u) && unit_slot == 0 && cta == c_first : hook) && li == 0 && warp == 0) {  // test hook: the first wait of the CTA
@@ -1016,8 +1035,17 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       if (lane == 0) mbar_arrive(sm_base + kFsBar + 8 * (kStages + s));
     }
     };
-    if (exact) stream(std::true_type{});
-    else stream(std::false_type{});
+    for (int first = 0;;) {
+      const int last = kPaged ? min(n_li, first + kWindow) : n_li;
+      if (exact) stream(std::true_type{}, first, last);
+      else stream(std::false_type{}, first, last);
+      first += kWindow;
+      if (!kPaged || 2 * first >= st1 - st0) break;
+      __syncthreads();   // nothing reads the list any more
+      if (*abort_flag) break;
+      list_places(2 * first);
+      __syncthreads();
+    }
     gl0 += n_li;
     __syncthreads();  // every copy that was consumed is done with; the rest is waited for below
     if (*abort_flag) {

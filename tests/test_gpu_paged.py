@@ -65,6 +65,29 @@ def test_paged_cache_equals_the_contiguous_one(d, Hq, Hkv, page_tokens):
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize("Hq,Hkv,B,tokens", [(32, 8, 8, 340_000), (28, 4, 16, 331_111)])
+def test_paged_decode_over_segments_of_more_than_a_thousand_stages(Hq, Hkv, B, tokens):
+    """The decode kernel's CTAs list where 1024 stages of 128 tokens begin at a time, and these calls give each CTA more: the
+    same bytes in a pool of shuffled pages and in one piece, split alike over the CTAs, give the same bits."""
+    page_tokens = 512
+    pages = -(-tokens // page_tokens)
+    paged, flat = _caches(B, Hq, Hkv, 128, page_tokens, pages, seed=9, extra_pages=1)
+    chunk = page_tokens // 64 * 7936
+    flat.cache.random_(0, 256)
+    radii = flat.cache.view(-1, 3968)[:, 2944:].view(torch.float16)
+    radii.copy_(torch.rand(radii.shape, device=DEV) + 0.5)
+    pool, rows = paged.cache.view(-1, Hkv, chunk), flat.cache.view(B, Hkv, pages, chunk)
+    pool[paged.page_table.long().flatten()] = rows.permute(0, 2, 1, 3).reshape(B * pages, Hkv, chunk)
+    for c in (paged, flat):
+        c.lens.fill_(tokens)
+    assert B * Hkv * (tokens // 128) > 1024 * torch.cuda.get_device_properties(0).multi_processor_count
+    q = synthetic.queries(3, B, Hq, 128, torch.bfloat16, DEV)
+    out_paged, out_flat = paged.attend(q), flat.attend(q)
+    for c in (paged, flat):
+        c.check_status()
+    assert torch.equal(out_paged, out_flat) and torch.isfinite(out_flat.float()).all()
+
+
 def test_paged_encode_against_the_oracle_and_pool_sharing():
     """Codes through the paged entry points against the oracle; two caches' worth of sequences share one pool
     without touching each other's pages (the pool's unused pages keep their fill)."""
