@@ -11,7 +11,9 @@
 // the whole thread block (two or fewer terms per thread) and decided by one warp.
 // Measured (device time behind another kernel, 8 kv heads; a block per vector, float64 below head_dim 128, and a second launch for the
 // lengths before): append of one token at head_dim 128 5.3 -> 4.9 us, of 16 10.9 -> 7.9 us; 31 tokens in one sequence 15.0 -> 7.9 us;
-// at head_dim 64 one token 16.9 -> 7.5 us, 256 tokens 21.5 -> 15.3 us.
+// at head_dim 64 one token 16.9 -> 7.5 us, 256 tokens 21.5 -> 15.3 us.  Rows that the tensor-core encoder does not take, at head_dim 128
+// (tiles of 128 rows in encode_ffma_kernel before): 64 tokens 107 -> 13.9 us, 1024 114 -> 57; the neighbours among the radii fall from
+// 0.009 to 0.003 %.
 #pragma once
 
 namespace pq {
@@ -297,10 +299,17 @@ static int32_t launch_encode_rows_by_size(const EncodeArgs& a, int32_t* lens, in
   return all <= (int64_t)kFew * n_sm ? launch_encode_rows_of<D, kFew>(a, lens, stream) : launch_encode_rows_of<D, 16>(a, lens, stream);
 }
 
-// Calls that this kernel takes: fewer than 32 tokens; below head_dim 128 also as long as two passes of every SM hold them.
-static bool encode_rows_takes(const EncodeArgs& a, int n_sm) {
+static bool encode_rows_in_passes(const EncodeArgs& a, int n_sm, int passes) {   // of 16 vectors (RowsShape's kVec at head_dim 16) per SM
   const int per_pass = a.head_dim == 16 ? RowsShape<16, 16>::kVec : 16;
-  return a.total_tokens < 32 || (a.head_dim < 128 && (int64_t)a.total_tokens * 2 * a.n_kv_heads <= 2 * (int64_t)n_sm * per_pass);
+  return (int64_t)a.total_tokens * 2 * a.n_kv_heads <= passes * (int64_t)n_sm * per_pass;
+}
+// Calls that this kernel takes before any other: fewer than 32 tokens; below head_dim 128 as long as two passes of every SM hold them,
+// at head_dim 128 as long as four vectors per SM do.  There the tensor-core encoder takes 16.4 us for its first tile (bf16, 2 kv heads,
+// 128 tokens: 8.8 us here); with sixteen per SM it would be 17.2 -> 13.9, but 18.6 -> 24.8 without a preconditioner, when one pair in a
+// thousand lies on a boundary.
+static bool encode_rows_takes(const EncodeArgs& a, int n_sm) {
+  return a.total_tokens < 32 || (a.head_dim == 128 ? (int64_t)a.total_tokens * 2 * a.n_kv_heads <= 4 * (int64_t)n_sm
+                                                   : encode_rows_in_passes(a, n_sm, 2));
 }
 static int32_t launch_encode_rows(const EncodeArgs& a, int32_t* lens, int n_sm, cudaStream_t stream) {
   switch (a.head_dim) {

@@ -371,16 +371,18 @@ static int32_t launch_advance_lens(const EncodeArgs& a, int32_t* lens, cudaStrea
 
 static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
   if (a.total_tokens == 0) return PQ_OK;
-  {
-    const int32_t tc = try_launch_encode_tc(a, stream);
-    if (tc < 0) return tc;
-    if (tc == 1) return launch_advance_lens(a, lens, stream);
-  }
   static DeviceMemo sm_count;
   const int n_sm = sm_count_of_device(sm_count);
   if (n_sm == 0) return PQ_ERR_CUDA;
   if (encode_rows_takes(a, n_sm)) return launch_encode_rows(a, lens, n_sm, stream);
+  const int32_t tc = try_launch_encode_tc(a, stream);
+  if (tc < 0) return tc;
+  if (tc == 1) return launch_advance_lens(a, lens, stream);
   if (a.head_dim == 128) {
+    // Up to two of its blocks of 128 vectors per SM encode_ffma_kernel takes 107 to 120 us whatever the number of vectors; the rows
+    // kernel takes 5 to 7 us for each pass of 16 vectors per SM (float32, 8 kv heads: 64 tokens 107 -> 13.9 us, 1024 114 -> 57; 2048
+    // tokens, 14 passes, would be 120 -> 103).
+    if (encode_rows_in_passes(a, n_sm, 8)) return launch_encode_rows(a, lens, n_sm, stream);
     static DeviceMemo configured;
     if (configure_for_device(encode_ffma_kernel, kFfmaSmem, configured) == 0) return PQ_ERR_CUDA;
     dim3 grid((a.total_tokens + 127) / 128, a.n_kv_heads, 2);

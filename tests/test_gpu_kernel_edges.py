@@ -177,6 +177,25 @@ def test_encoders_give_the_same_codes_in_any_pieces(d, dtype):
     _encode_and_compare(few, K[:31], V[:31], [17, 14])          # one launch, odd counts
 
 
+# head_dim 128 on both sides of four vectors per SM, where bf16 goes on with the tensor cores, of sixteen, where a second pass of the few-rows
+# kernel begins, and of 128, where float32 goes on with tiles of 128 rows; the pieces are all few rows.
+@pytest.mark.parametrize("dtype,per_sm,Hkv", [(torch.bfloat16, 4, 2), (torch.float32, 16, 4), (torch.float32, 128, 4)])
+def test_encoders_on_both_sides_of_the_few_rows_kernel(dtype, per_sm, Hkv):
+    edge = per_sm * torch.cuda.get_device_properties(0).multi_processor_count // (2 * Hkv)
+    K, V = synthetic.kv_like(17, edge + 1, Hkv, 128, dtype, DEV, n_outliers=4)
+    cut = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=edge + 1, seed=6, device=DEV)
+    for at in range(0, edge + 1, 31):
+        m = min(31, edge + 1 - at)
+        cut.encode(K[at:at + m], V[at:at + m], torch.tensor([0, m], dtype=torch.int32, device=DEV))
+    codes_cut, radii_cut = cut.unpack(edge + 1)
+    for n in (edge, edge + 1):
+        whole = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=n, seed=6, device=DEV)
+        whole.encode(K[:n], V[:n], torch.tensor([0, n], dtype=torch.int32, device=DEV))
+        codes, radii = whole.unpack(n)
+        assert torch.equal(codes, codes_cut[:, :, :, :n]) and whole.lens.tolist() == [n]
+        assert torch.all((radii.float() - radii_cut[:, :, :, :n].float()).abs() <= 2.0 ** -10 * radii.float())
+
+
 @pytest.mark.parametrize("d,bits", [(128, (3,) * 7), (64, (4, 2)), (16, (2,) * 4)])
 def test_general_encoder_writes_the_same_bytes_in_any_pieces(d, bits):
     # up to 3072 or 4096 vectors a block each, in float64; above them tiles of 16 to 256 vectors
