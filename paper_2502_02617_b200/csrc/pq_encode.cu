@@ -174,13 +174,13 @@ __device__ __forceinline__ bool bar_or(int bar_id, int n_threads, bool v) {
 // not fit before).  All `n_threads` threads of named barrier `bar_id` call this together.
 // `left` holds this thread's decisions that found the queue full: 15 bits per block, four blocks per
 // word, starting at block `blk0`; it is all zero on return.
-template <class Q, int kWords>
+template <bool kAligned, class Q, int kWords>
 __device__ inline void fix_rounds(const EncodeArgs& a, Q* q, unsigned long long (&left)[kWords], int64_t xoff, uint8_t* tb,
                                   int tok, int blk0, int kv, int t, int n_threads, int bar_id,
                                   const double* Sd = nullptr) {
   for (int round = 0; round < 4096; ++round) {
     asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(n_threads) : "memory");
-    fix_process(q, 1, t, n_threads, a.K, a.V, a.in_dtype, a.S, Sd, *a.tables, a.status);
+    fix_process<kAligned>(q, 1, t, n_threads, a.K, a.V, a.in_dtype, a.S, Sd, *a.tables, a.status);
     asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(n_threads) : "memory");
     if (t < 4) q->count[t] = 0;
     bool mine = false;
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kFfmaThreads) encode_ffma_kernel(EncodeArgs a)
       leftbits[0] |= (unsigned long long)rest << (15 * i);
     }
   }
-  fix_rounds(a, fixq, leftbits, xoff, tb, tok, 4 * half, kv, tid, kFfmaThreads, 1);
+  fix_rounds<false>(a, fixq, leftbits, xoff, tb, tok, 4 * half, kv, tid, kFfmaThreads, 1);
 }
 
 }  // namespace pq

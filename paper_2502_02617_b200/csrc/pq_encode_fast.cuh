@@ -398,8 +398,9 @@ __device__ __forceinline__ uint32_t exact_code(const double* y, int level, const
 
 // Process everything queued, in level order: called by `n_threads` threads (a multiple of 32) with linear index `t`.
 // `q` points to `n_queues` queues laid out back to back; their entries are taken level by level.
-// `Sd` (may be null) is the float64 copy of S in shared memory for exact_coords_sm.
-template <class Q>
+// `Sd` (may be null) is the float64 copy of S in shared memory for exact_coords_sm.  kAligned: bf16 rows begin on 16-byte boundaries
+// (the tensor-core encoder takes no others); encode_ffma_kernel takes rows of any stride from any address.
+template <bool kAligned, class Q>
 __device__ inline void fix_process(const Q* q, int n_queues, int t, int n_threads, const void* kbase, const void* vbase,
                                    int in_dtype, const float* S, const double* Sd, const Tables& tb, int32_t* status) {
   constexpr int o2 = 32 * kTokenBlock, o3 = o2 + 8 * kTokenBlock, o4 = o3 + 4 * kTokenBlock;
@@ -430,9 +431,16 @@ __device__ inline void fix_process(const Q* q, int n_queues, int t, int n_thread
     const Q* qe;
     const int e = entry_of(i, &qe);
     const void* xbase = (qe->meta[e] >> 15) & 1 ? vbase : kbase;
-    const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(xbase) + qe->xoff[e] + 16 * sub);
-    raw[0] = __ldg(p);
-    raw[1] = __ldg(p + 1);
+    const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(xbase) + qe->xoff[e] + 16 * sub;
+    if (kAligned || ((uintptr_t)x & 15) == 0) {
+      raw[0] = __ldg(reinterpret_cast<const uint4*>(x));
+      raw[1] = __ldg(reinterpret_cast<const uint4*>(x) + 1);
+    } else {
+      const unsigned short* h = reinterpret_cast<const unsigned short*>(x);
+      auto two = [&](int k) { return (uint32_t)__ldg(h + k) | (uint32_t)__ldg(h + k + 1) << 16; };
+      raw[0] = make_uint4(two(0), two(2), two(4), two(6));
+      raw[1] = make_uint4(two(8), two(10), two(12), two(14));
+    }
   };
   uint4 raw[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
   fetch(t >> 3, raw);

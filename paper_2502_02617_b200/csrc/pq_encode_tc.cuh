@@ -376,7 +376,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     // for the end of the CTA's work, where all 16 warps take them together (the float64 pipe is slow, and a group
     // that drains alone holds up its own tiles for as long).
     const bool drain = bar_or(group_bar, kTcGroupThreads, (left[0] | left[1]) != 0ull || fix_should_drain(fixq));
-    if (drain) fix_rounds(a, fixq, left, xoff, tb, tok, 0, kv, st, kTcGroupThreads, group_bar);
+    if (drain) fix_rounds<true>(a, fixq, left, xoff, tb, tok, 0, kv, st, kTcGroupThreads, group_bar);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -403,7 +403,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     __syncthreads();
   }
   if (!kHist)
-    fix_process(reinterpret_cast<TcFixQueue*>(smem + kTcSmFix), kTcGroups, tid, kTcThreads, a.K, a.V, a.in_dtype, a.S, *abort_flag ? (const double*)nullptr : Sd,
+    fix_process<true>(reinterpret_cast<TcFixQueue*>(smem + kTcSmFix), kTcGroups, tid, kTcThreads, a.K, a.V, a.in_dtype, a.S, *abort_flag ? (const double*)nullptr : Sd,
                 *a.tables, a.status);
   if (*abort_flag && tid < kTcStages && copies_issued[tid] > 0) {
     // gave up somewhere: let the copies that are still in flight land (bounded) before the CTA and its

@@ -196,6 +196,28 @@ def test_encoders_on_both_sides_of_the_few_rows_kernel(dtype, per_sm, Hkv):
         assert torch.all((radii.float() - radii_cut[:, :, :, :n].float()).abs() <= 2.0 ** -10 * radii.float())
 
 
+# bf16 rows that do not begin on 16-byte boundaries, in more passes than the few-rows kernel takes: tiles of 128 rows, whose float64
+# decisions read the rows again.  The same codes as from the same rows in one piece, radii that are neighbours at most.
+@pytest.mark.parametrize("pad,shift", [(1, 0), (4, 0), (0, 1), (0, 4)])
+def test_encode_of_many_rows_that_are_not_aligned(pad, shift):
+    Hkv, n = 8, 1300
+    K, V = synthetic.kv_like(23, n, Hkv, 128, torch.bfloat16, DEV, n_outliers=4)
+    K[::5], V[3::7] = 1.0, 0.0
+    moved = []
+    for t in (K, V):
+        t = torch.nn.functional.pad(t, (0, pad))
+        whole = torch.empty(t.numel() + shift, dtype=t.dtype, device=DEV)
+        moved.append(whole[shift:].view(t.shape).copy_(t)[..., :128])
+    got = []
+    for k, v in ((K, V), moved):
+        c = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=n, seed=6, device=DEV)
+        c.encode(k, v, torch.tensor([0, n], dtype=torch.int32, device=DEV))
+        got.append((*c.unpack(n), c.status[:3].tolist()))
+    assert n * 2 * Hkv > 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert torch.equal(got[0][0], got[1][0]) and got[0][2] == got[1][2]
+    assert torch.all((got[0][1].float() - got[1][1].float()).abs() <= 2.0 ** -10 * got[1][1].float())
+
+
 @pytest.mark.parametrize("d,bits", [(128, (3,) * 7), (64, (4, 2)), (16, (2,) * 4)])
 def test_general_encoder_writes_the_same_bytes_in_any_pieces(d, bits):
     # up to 3072 or 4096 vectors a block each, in float64; above them tiles of 16 to 256 vectors
