@@ -168,6 +168,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
       if (fq.analytic) polar_quant_block_fast<true>(yb, rm, fq, &fb);
       else polar_quant_block_fast<false>(yb, rm, fq, &fb);
       const float block_err = rotation_block_error(16, R::kSlices) * norm;
+      bool zero = false;   // EncodeArgs::zero_bad_rows; the eight lanes of a vector look at its inputs together
+      if (D == 128 && a.zero_bad_rows && !(n2 < CUDART_INF_F)) {
+        const unsigned of_vector = 0xFFu << (lane & 24);
+        for (int i = 0; i < 16; ++i) zero = zero || !(fabsf(xs[16 * tid + i]) < CUDART_INF_F);
+        zero = __any_sync(of_vector, zero);
+        if (zero) fb = {0u, 0u, 0u, 0u, 0u, 0.f};
+      }
       if (v < n_vec) {
         const int w = v % per_row, kv = w / a.n_kv_heads, head = w - kv * a.n_kv_heads;
         if (goes) {
@@ -181,7 +188,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) encode_rows_kernel(const __gr
         }
         // head dims below 128: radii as rounded once from float64; at 128 as the tensor-core encoder forms them
         unsure = fb.amb != 0u || (D < 128 && radius_unsure(fb.radius, block_err));
-        if (mine && unsure) list[atomicAdd(&n_list, 1)] = (uint16_t)tid;
+        if (mine && unsure && !zero) list[atomicAdd(&n_list, 1)] = (uint16_t)tid;
       }
     }
     __syncthreads();

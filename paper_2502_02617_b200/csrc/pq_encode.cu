@@ -27,6 +27,9 @@ struct EncodeArgs {
   unsigned long long* hist;
   int n_bins;
   Paging pg;  // where the cache's token-blocks live; `capacity` = pg.pages_per_seq * pg.page_tokens
+  // A row with non-finite inputs is stored as the zero vector.  So the tensor-core encoder does it, and so does the few-rows kernel in
+  // calls that are the former's by type, layout and number of tokens: what is stored does not depend on the heads and the SMs.
+  bool zero_bad_rows = false;
 };
 
 __device__ inline float load_elem(const void* base, int dtype, int64_t idx) {
@@ -374,6 +377,7 @@ static int32_t launch_encode(EncodeArgs a, int32_t* lens, cudaStream_t stream) {
   static DeviceMemo sm_count;
   const int n_sm = sm_count_of_device(sm_count);
   if (n_sm == 0) return PQ_ERR_CUDA;
+  a.zero_bad_rows = tc_takes(a);
   if (encode_rows_takes(a, n_sm)) return launch_encode_rows(a, lens, n_sm, stream);
   const int32_t tc = try_launch_encode_tc(a, stream);
   if (tc < 0) return tc;

@@ -446,14 +446,19 @@ static bool make_x_map(EncodeTiledFn fn, CUtensorMap* map, const void* base, int
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Rows that the kernel can read: type, strides and alignment of TMA, a tile of them at least.
+static bool tc_takes(const EncodeArgs& a) {
+  if (a.head_dim != 128 || a.in_dtype != PQ_DTYPE_BF16 || a.total_tokens < 128) return false;
+  if ((a.token_stride & 7) || (a.head_stride & 7) || a.head_stride < 128 || a.token_stride < 128) return false;
+  if (((uintptr_t)a.K | (uintptr_t)a.V) & 15) return false;
+  return a.n_kv_heads <= 1 || a.head_stride * 2 < ((int64_t)1 << 40);
+}
+
 // Launch the tensor-core encoder (or its histogram form) if the inputs allow it.  Returns 1 if launched, 0 if not
 // applicable, or a negative status.
 template <bool kHist, bool kPaged>
 static int32_t try_launch_tc(const EncodeArgs& a, cudaStream_t stream) {
-  if (a.head_dim != 128 || a.in_dtype != PQ_DTYPE_BF16 || a.total_tokens < 128) return 0;
-  if ((a.token_stride & 7) || (a.head_stride & 7) || a.head_stride < 128 || a.token_stride < 128) return 0;
-  if (((uintptr_t)a.K | (uintptr_t)a.V) & 15) return 0;
-  if (a.n_kv_heads > 1 && a.head_stride * 2 >= ((int64_t)1 << 40)) return 0;
+  if (!tc_takes(a)) return 0;
   EncodeTiledFn fn = get_encode_tiled();
   if (fn == nullptr) return 0;
   TcMaps maps;

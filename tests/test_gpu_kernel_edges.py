@@ -196,6 +196,34 @@ def test_encoders_on_both_sides_of_the_few_rows_kernel(dtype, per_sm, Hkv):
         assert torch.all((radii.float() - radii_cut[:, :, :, :n].float()).abs() <= 2.0 ** -10 * radii.float())
 
 
+# What is stored for a row with a non-finite input does not depend on which kernel takes the call: bf16 calls of 128 tokens and more are the
+# tensor-core encoder's or, up to four vectors per SM, the few-rows kernel's, and store the zero vector; tiles of 128 rows (float32, or
+# bf16 rows that are not aligned, above 128 vectors per SM) store what the arithmetic gives, as fewer tokens do.  The other rows are the
+# ones of a clean call, the elements are counted.
+@pytest.mark.parametrize("dtype,per_sm,Hkv,pad", [(torch.bfloat16, 4, 2, 0), (torch.float32, 128, 8, 0), (torch.bfloat16, 128, 8, 1)])
+def test_rows_that_are_not_finite_on_both_sides_of_the_few_rows_kernel(dtype, per_sm, Hkv, pad):
+    edge = per_sm * torch.cuda.get_device_properties(0).multi_processor_count // (2 * Hkv)
+    for n in (edge, edge + 1):
+        K, V = synthetic.kv_like(19, n, Hkv, 128, dtype, DEV)
+        got = []
+        for spoilt in (False, True):
+            if spoilt:
+                K[3, 0, 5], V[n - 4, 1, 6], V[n - 4, 1, 7] = float("nan"), float("inf"), float("-inf")
+            k, v = (torch.nn.functional.pad(t, (0, pad))[..., :128] for t in (K, V))
+            c = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=n, seed=6, device=DEV)
+            c.encode(k, v, torch.tensor([0, n], dtype=torch.int32, device=DEV))
+            got.append((*(t.movedim(3, 0) for t in c.unpack(n)), c.status.tolist()))
+        (codes, radii, status), (codes_bad, radii_bad, status_bad) = got
+        assert status[:2] == [0, 0] and status_bad[:2] == [pq.ERR_NONFINITE, 3]
+        if dtype == torch.bfloat16 and pad == 0:
+            assert status_bad[2] == 0
+            for bad in ((3, 0, 0, 0), (n - 4, 0, 1, 1)):
+                assert not codes_bad[bad].any() and not radii_bad[bad].any()
+        keep = torch.ones(codes.shape[:4], dtype=torch.bool, device=DEV)
+        keep[3, 0, 0, 0] = keep[n - 4, 0, 1, 1] = False
+        assert torch.equal(codes[keep], codes_bad[keep]) and torch.equal(radii[keep], radii_bad[keep])
+
+
 # bf16 rows that do not begin on 16-byte boundaries, in more passes than the few-rows kernel takes: tiles of 128 rows, whose float64
 # decisions read the rows again.  The same codes as from the same rows in one piece, radii that are neighbours at most.
 @pytest.mark.parametrize("pad,shift", [(1, 0), (4, 0), (0, 1), (0, 4)])

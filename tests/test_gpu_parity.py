@@ -362,8 +362,7 @@ def test_capacity_overflow_and_empty_sequence_are_reported_not_faulted():
 
 @pytest.mark.parametrize("n", [8, 40, 300])
 def test_nonfinite_inputs_are_counted(n):
-    """8 rows go through the per-vector kernel, 40 through the float32-FMA kernel, 300 through the tensor-core
-    kernel: each records the error and counts the non-finite input elements; the other rows are encoded as usual."""
+    """8 and 40 rows go through the few-rows kernel, 300 through the tensor-core kernel: each records the error and counts the non-finite input elements; the other rows are encoded as usual."""
     d = 128
     cache = pq.PolarQuantCache(1, 2, 2, d, capacity=n, seed=8, device=DEV)
     K, V = synthetic.kv_like(51, n, 2, d, torch.bfloat16, DEV)
