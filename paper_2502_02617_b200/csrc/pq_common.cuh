@@ -60,7 +60,7 @@ struct Tables {
   float cen_cos[PQ_N_CENTROIDS];
   float cen_sin[PQ_N_CENTROIDS];
   // fp16 decode tables of the attention kernels.  A level-1 entry is kept times l1_scale and the products above it divided by
-  // it, which changes no decoded value; see kFlagExactDecode.
+  // it, which changes no decoded value; see kL1Scale.
   //   l1_hi[c], l1_lo[c] : l1_scale (cos, sin) of level-1 centroid c as half2, split into the fp16 value and
   //                        the fp16 rounding residual (hi + lo carries ~22 bits)
   //   u_tab[s][i]        : sub-block s (0..3) of a block, i = c2 | c3 << 2 | c4 << 4: the product of
@@ -86,12 +86,11 @@ constexpr uint32_t kFlagUniformL1 = 1u;
 // bit 1: at every level >= 2 the boundaries are b, pi/4, pi/2 - b (tan^2: T, 1, 1/T to 1e-9 relative), as for
 // every Lloyd-Max codebook of the symmetric densities of Lemma 2
 constexpr uint32_t kFlagSymmetricUpper = 2u;
-// bit 2: l1_hi alone is within 2^-16 of the level-1 factors (their residuals are left out: the fp16 value of a key carries a residual
-// for an error of 2^-12, and the values have none at all), and u_tab[2], u_tab[3] are u_tab[0], u_tab[1] at the mirrored level-4 code 3 - c4.  Both
-// hold for the codebook of Lemma 2: its sixteen level-1 centroids have four magnitudes, and kL1Scale brings all four within
-// 1.4e-5 = 2^-16.2 of fp16 values (a plain rounding: 1.8e-4).
-constexpr uint32_t kFlagExactDecode = 4u;
-constexpr double kL1Scale = 1.70066175;   // the best of a grid of 4 million factors in [1, 2]
+// The level-1 factors are kept times l1_scale, which brings them closer to fp16 values: the sixteen level-1 centroids of Lemma 2's codebook
+// have four magnitudes, and this factor, the best of a grid of 4 million in [1, 2], brings all four within 1.4e-5 = 2^-16.2 of fp16
+// values (a plain rounding: 1.8e-4).  The values are decoded from those alone (error of an output against float64 4.0e-4 -> 3.8e-4),
+// the keys with the residuals as well.  1 where it would not bring every factor that close.
+constexpr double kL1Scale = 1.70066175;
 
 // ------------------------------------------------------------------------------------------
 // Packed cache layout.

@@ -19,15 +19,16 @@
 //   U  index = the half's level-2 codes (4 bits) | level-3 code << 4 | level-4 code << 6 -> the multipliers of its four level-1
 //      pairs as (half2 values, half2 rounding residuals)
 //   T  index = one byte of level-1 codes (pair a = 2s | pair b = 2s+1 << 4) -> (cos a, cos b), (sin a, sin b) in fp16: a half2
-//      (u_a, u_b) of the table above multiplies them element-wise; where they are not exact enough, the fp16 rounding residuals too
+//      (u_a, u_b) of the table above multiplies them element-wise; for the keys the fp16 rounding residuals of the same stand beside them
 // replicated so that the lanes that read together read their own banks (16 copies of 8-byte entries, 8 of 16-byte ones).  Bound by
 // the shared-memory pipe and by instruction issue together, so a lookup's work is what counts: index bytes are put together four
-// at a time, a row of both tables is 256 bytes, so that one byte permute makes an address, and the analytic codebook needs no
-// residuals at level 1 and one half's multipliers (kFlagExactDecode).  One lookup per 4-coordinate sub-block at level 2..4, residuals
-// at level 1 and shift-and-mask addresses took 770 instructions and 210 shared-memory wavefronts per tile (8 x 32768 tokens,
-// 32/8 heads: 141.4 us); this 119.5 us, one sequence of 131072 78.4 -> 67.5.  The rows and tcgen05 kernels keep a table
+// at a time, and a row of both tables is 256 bytes, so that one byte permute makes an address.  One lookup per 4-coordinate sub-block at level 2..4, values and residuals of level
+// 1 in tables of their own and shift-and-mask addresses took 770 instructions and 210 shared-memory wavefronts per tile (8 x 32768
+// tokens, 32/8 heads: 141.4 us; now 129.4).  Without the residuals of level 1 it is 119.5 us, but the scores are then off by 1e-5 of
+// their terms: the log-sum-exp by 4e-5 where it is off by 2e-6 now (2 x 4096 tokens, scores up to 16), and outputs of scores in the
+// thousands by 4.5e-4 instead of 3.8e-4.  The rows and tcgen05 kernels keep a table
 // per sub-block (u [4][64][16], t1hi and t1lo [256][16]): the first is bound by its start and end and the MMAs of its rows, the second
-// has no room for rows of 256 bytes; leaving out the residuals there gave 0.2 and 0.5 %.
+// has no room for rows of 256 bytes.
 // Values use the fp16 parts only.  Keys feed the softmax exponent, where an fp16-rounded operand
 // costs ~3x its relative error in the output, so they are decoded as an unevaluated sum hi + lo
 // (error-free fp16 transformations with fused multiply-adds) and contracted with two MMAs.
@@ -66,9 +67,9 @@ constexpr int kMrgStride = 136;  // floats per (warp, head) row of the merge buf
 // forms a lookup's address: the index byte becomes address byte 1, the base gives the others (byte 0: the lane's replica).  What
 // else the kernel keeps lies around them, at fixed places of the window (dynamic shared memory starts at kWindowBase, which the
 // host asks the device for):
-//   ring | T [256 bytes of level-1 codes]    16 x (cos a, cos b | sin a, sin b) in fp16, then 16 x the residuals of the same
-//        | U [256 half-block codes]          kFlagExactDecode: 8 x (values, residuals) for the keys, then 16 x values for the values;
-//                                            otherwise 8 x (values, residuals) of half 0, then 8 x of half 1
+//   ring | T [256 bytes of level-1 codes]    8 x (cos a, cos b | sin a, sin b | their residuals) in fp16 for the keys, then 16 x
+//        |                                   (cos a, cos b | sin a, sin b) for the values
+//        | U [256 half-block codes]          8 x (values, residuals) of half 0, then 8 x of half 1
 //        | barriers, segments, q', places of a paged segment's stages
 constexpr uint32_t kWindowBase = 1024;
 constexpr uint32_t kFsRing = kWindowBase, kFsT = 0x10000, kFsU = 0x20000, kFsBar = 0x30000;
@@ -259,60 +260,53 @@ template <int kByte>
 __device__ __forceinline__ uint32_t row_address(uint32_t index, uint32_t base) {
   return __byte_perm(index, base, 0x7604 | (kByte << 4));
 }
-// Half-block indices, four to a word: byte = the half's two level-2 codes | level-3 code << 4 | level-4 code << 6; the level-4 code
-// of a second half mirrored (3 - c4) in the exact tables, which hold a first half's entries only.  Each field of a byte is spread by a
+// Half-block indices, four to a word: byte = the half's two level-2 codes | level-3 code << 4 | level-4 code << 6.  Each field of a byte is spread by a
 // shift or a multiplication that leaves garbage in the other fields only, and two bitwise selects put the three together.
 // Two blocks of one token -> (block 0: half 0, half 1; block 1: half 0, half 1).  c2: the blocks' level-2 bytes; n3: their level-3
 // nibbles; c4: their level-4 codes in bits 0..3 (garbage above).
-template <bool kExact>
 __device__ __forceinline__ uint32_t half_indices_of_blocks(uint32_t c2, uint32_t n3, uint32_t c4) {
   const uint32_t f2 = __byte_perm(c2, c2 >> 4, 0x5140);
-  // even fields to bytes 0 and 2, odd ones to bytes 1 and 3; bits 6, 7 of a byte stay clear but for the mirror
-  const uint32_t f3 = (n3 & 0x33u) * 0x10010u + ((n3 & 0xCCu) * 0x400400u + (kExact ? 0xC000C000u : 0u));
+  // even fields to bytes 0 and 2, odd ones to bytes 1 and 3; bits 6, 7 of a byte stay clear
+  const uint32_t f3 = (n3 & 0x33u) * 0x10010u + (n3 & 0xCCu) * 0x400400u;
   const uint32_t f4 = (c4 & 0xFu) * 0x10104040u;
   const uint32_t w = (f2 & 0x0F0F0F0Fu) | (f3 & 0xF0F0F0F0u);
   return w ^ (f4 & 0xC0C0C0C0u);
 }
 // One block of two tokens -> (token A: half 0, half 1; token B: half 0, half 1).  Bits 0..15 of each argument belong to token A, the
 // others to token B; c2: level-2 byte, n3: level-3 nibble, c4: level-4 code in bits 0..1 (garbage above, but n3 and c4 may be garbage).
-template <bool kExact>
 __device__ __forceinline__ uint32_t half_indices_of_tokens(uint32_t c2, uint32_t n3, uint32_t c4) {
   const uint32_t f2 = (c2 & 0x000F000Fu) | ((c2 << 4) & 0x0F000F00u);
   const uint32_t f3 = (n3 & 0x000F000Fu) * 0x410u;
-  const uint32_t f4 = kExact ? (c4 & 0x00030003u) * (64u - 16384u) + 0xC000C000u : (c4 & 0x00030003u) * (64u + 16384u);
+  const uint32_t f4 = (c4 & 0x00030003u) * (64u + 16384u);
   const uint32_t w = f2 | (f3 & 0x30303030u);
   return w | f4;
 }
 // Half kByte & 1 of a key block (byte kByte of `index`; level-1 bytes kL1, kL1 + 1 of `l1`) as unevaluated sums hi + lo, see
-// sub_block_hilo.  With the exact tables the level-1 factors have no residual.
+// sub_block_hilo.
 struct KeyHalf {
   __half2 xh[2], yh[2], xl[2], yl[2];
 };
-template <bool kExact, int kByte, int kL1>
+template <int kByte, int kL1>
 __device__ __forceinline__ void decode_key_half(uint32_t index, uint32_t l1, __half2 r2, uint32_t uk, uint32_t t, KeyHalf& k) {
-  const uint4 uu = lds128i<!kExact && (kByte & 1) ? 128 : 0>(row_address<kByte>(index, uk));
+  const uint4 uu = lds128i<(kByte & 1) * 128>(row_address<kByte>(index, uk));
   const uint32_t ta[2] = {row_address<kL1>(l1, t), row_address<kL1 + 1>(l1, t)};
   const uint32_t uh[2] = {uu.x, uu.y}, ul[2] = {uu.z, uu.w};
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    const uint2 th = lds64i<0>(ta[i]);
+    const uint4 e = lds128i<0>(ta[i]);
+    const uint2 th = make_uint2(e.x, e.y), tl = make_uint2(e.z, e.w);
     const __half2 u_hi = __hmul2(r2, as_h2(uh[i]));
     const __half2 u_lo = __hfma2(r2, as_h2(ul[i]), __hfma2(r2, as_h2(uh[i]), __hneg2(u_hi)));
     k.xh[i] = __hmul2(u_hi, as_h2(th.x));
     k.yh[i] = __hmul2(u_hi, as_h2(th.y));
-    k.xl[i] = __hfma2(u_lo, as_h2(th.x), __hfma2(u_hi, as_h2(th.x), __hneg2(k.xh[i])));
-    k.yl[i] = __hfma2(u_lo, as_h2(th.y), __hfma2(u_hi, as_h2(th.y), __hneg2(k.yh[i])));
-    if (!kExact) {
-      const uint2 tl = lds64i<128>(ta[i]);
-      k.xl[i] = __hfma2(u_hi, as_h2(tl.x), k.xl[i]);
-      k.yl[i] = __hfma2(u_hi, as_h2(tl.y), k.yl[i]);
-    }
+    k.xl[i] = __hfma2(u_hi, as_h2(tl.x), __hfma2(u_lo, as_h2(th.x), __hfma2(u_hi, as_h2(th.x), __hneg2(k.xh[i]))));
+    k.yl[i] = __hfma2(u_hi, as_h2(tl.y), __hfma2(u_lo, as_h2(th.y), __hfma2(u_hi, as_h2(th.y), __hneg2(k.yh[i]))));
   }
 }
 // The multipliers u = r U of half kByte & 1 of a value block.
-template <bool kExact, int kByte>
+template <int kByte>
 __device__ __forceinline__ void value_half(uint32_t index, __half2 r2, uint32_t uv, __half2* u) {
-  const uint2 uu = lds64i<!kExact && (kByte & 1) ? 128 : 0>(row_address<kByte>(index, uv));
+  const uint2 uu = lds64i<(kByte & 1) * 128>(row_address<kByte>(index, uv));
   u[0] = __hmul2(r2, as_h2(uu.x));
   u[1] = __hmul2(r2, as_h2(uu.y));
 }
@@ -360,39 +354,32 @@ __device__ __forceinline__ void build_fast_tables(uint8_t* smem, const Tables* t
   }
 }
 
-// The same for the map with 256-byte rows (`window`: start of the shared window).  Returns whether the tables are exact ones.
+// The same for the map with 256-byte rows (`window`: start of the shared window).  All that a thread reads is on its way before it writes:
+// with one table after the other a call took 1.5 us longer.
 template <int kThreads>
-__device__ __forceinline__ bool build_row_tables(uint8_t* window, const Tables* tb) {
+__device__ __forceinline__ void build_row_tables(uint8_t* window, const Tables* tb) {
   const int row0 = threadIdx.x >> 4, rep = threadIdx.x & 15;   // 16 threads per row
   constexpr int kPer = 256 * 16 / kThreads, kStep = kThreads / 16;
-  const bool exact = (tb->flags & kFlagExactDecode) != 0;
   // entry i of half h: sub-blocks 2h and 2h + 1 at their level-2 codes (bits 0..1 and 2..3 of i) and the codes above, common to both
-  auto pair = [&](int h, int i) {
-    const uint2 lo = tb->u_tab[2 * h][(i & 3) | (i >> 2 & ~3)], hi = tb->u_tab[2 * h + 1][i >> 2];
-    return make_uint4(lo.x, hi.x, lo.y, hi.y);
-  };
-  uint2 th[kPer];
-  uint4 up[kPer];
+  const int h = rep >> 3;
+  uint2 th[kPer], tl[kPer], ul[kPer], uh[kPer];
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
-    th[r] = tb->t1p_hi[row0 + r * kStep];
-    up[r] = pair(0, row0 + r * kStep);
+    const int i = row0 + r * kStep;
+    th[r] = tb->t1p_hi[i];
+    tl[r] = tb->t1p_lo[i];
+    ul[r] = tb->u_tab[2 * h][(i & 3) | (i >> 2 & ~3)];
+    uh[r] = tb->u_tab[2 * h + 1][i >> 2];
   }
   uint8_t* t = window + kFsT + row0 * 256;
   uint8_t* u = window + kFsU + row0 * 256;
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
-    *reinterpret_cast<uint2*>(t + r * kStep * 256 + rep * 8) = th[r];
-    if (rep < 8) *reinterpret_cast<uint4*>(u + r * kStep * 256 + rep * 16) = up[r];
-    if (exact) *reinterpret_cast<uint2*>(u + r * kStep * 256 + 128 + rep * 8) = make_uint2(up[r].x, up[r].y);
+    uint8_t* tr = t + r * kStep * 256;
+    *reinterpret_cast<uint2*>(tr + 128 + rep * 8) = th[r];
+    if (rep < 8) *reinterpret_cast<uint4*>(tr + rep * 16) = make_uint4(th[r].x, th[r].y, tl[r].x, tl[r].y);
+    *reinterpret_cast<uint4*>(u + r * kStep * 256 + rep * 16) = make_uint4(ul[r].x, uh[r].x, ul[r].y, uh[r].y);
   }
-  if (!exact)
-#pragma unroll 1
-    for (int r = 0; r < kPer; ++r) {
-      *reinterpret_cast<uint2*>(t + r * kStep * 256 + 128 + rep * 8) = tb->t1p_lo[row0 + r * kStep];
-      if (rep < 8) *reinterpret_cast<uint4*>(u + r * kStep * 256 + 128 + rep * 16) = pair(1, row0 + r * kStep);
-    }
-  return exact;
 }
 
 // Slots of split partials for the persistent kernel: every unit (sequence, kv head) has one slot
@@ -687,7 +674,7 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
   // while that kernel finishes; its results (lengths, cache, queries, workspace) are read only after this wait.
   // The kernel after this one may be set up as soon as this grid has started.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const bool exact = build_row_tables<kFastThreads>(smem, a.tables);   // from the caller's tables, which no kernel writes
+  build_row_tables<kFastThreads>(smem, a.tables);   // from the caller's tables, which no kernel writes
   // What this thread needs of S (constant too) to rotate the queries: column warp * 8 + lane / 4, rows 16 i + 4 (lane & 3)
   // + 0..3 -- a warp's load covers whole 32-byte sectors, and four lanes share a column's sum.
   const int rot_j = warp * 8 + (lane >> 2), rot_k = (lane & 3) * 4;
@@ -728,9 +715,8 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     return list_segments<kFastThreads>(batch_no, n_units, smem + kFsRing, segs, n_segs, first_rank, stages_of, empty_unit);
   };
   const int g = lane >> 2, c = lane & 3;
-  // table base | lane replica; the value multipliers are the high parts of the keys' entries where the tables are not exact
-  const uint32_t t1a = sm_base + kFsT + (lane & 15) * 8, uk = sm_base + kFsU + (lane & 7) * 16;
-  const uint32_t uv = exact ? sm_base + kFsU + 128 + (lane & 15) * 8 : uk;
+  // table base | lane replica; the value multipliers are the high parts of the keys' entries
+  const uint32_t tk = sm_base + kFsT + (lane & 7) * 16, tv = sm_base + kFsT + 128 + (lane & 15) * 8, tu = sm_base + kFsU + (lane & 7) * 16;
   const int wg = warp >> 3;  // group of 8 warps
   // Offsets, inside a token-block, of what this thread reads of its tile (16 tokens from token (warp & 3) * 16).
   // Keys: tokens g and g + 8, blocks 2c and 2c + 1.  Values: block g of tokens c, c + 4, c + 8, c + 12 (these are
@@ -875,8 +861,8 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       *reinterpret_cast<uint2*>(smem + kFsQ + hg * 2048 + ks * 256 + lane * 8) = q_fragment(hg, ks);
       __syncthreads();
     }
-    auto stream = [&](auto exact_tables, int first, int last) {
-    constexpr bool kExact = decltype(exact_tables)::value;
+    for (int first = 0;;) {
+    const int last = kPaged ? min(n_li, first + kWindow) : n_li;
     for (int li = first; li < last; ++li) {
       const int gl = gl0 + li, s = 2 * wg + (gl & 1);
       const int st = st0 + wg + 2 * li;
@@ -906,19 +892,19 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
           const uint32_t c2A = lds16i<0>(kblk + ok_c2), c2B = lds16i<8 * 8>(kblk + ok_c2);
           const uint32_t c3A = lds8i<0>(kblk + ok_c3), c3B = lds8i<8 * 4>(kblk + ok_c3);
           const uint32_t c4A = lds16i<0>(kblk + ok_c4) >> (4 * c), c4B = lds16i<8 * 2>(kblk + ok_c4) >> (4 * c);
-#define PQ_KHALF(INDEX, L1, R2, H, HALF)                                                                                \
-  {                                                                                                                     \
-    KeyHalf kA, kB;                                                                                                     \
-    decode_key_half<kExact, 2 * (H) + (HALF), 2 * (HALF)>(INDEX##A, L1##A, R2(as_h2(rrA)), uk, t1a, kA);                \
-    decode_key_half<kExact, 2 * (H) + (HALF), 2 * (HALF)>(INDEX##B, L1##B, R2(as_h2(rrB)), uk, t1a, kB);                \
-    _Pragma("unroll") for (int i = 0; i < 2; ++i) _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                  \
-      constexpr int kKs0 = 4 * (H) + 2 * (HALF);                                                                        \
-      const uint2 qv = kQInRegs ? qb[kQInRegs ? kKs0 + i : 0] : lds64(qf + hg * 2048 + (kKs0 + i) * 256);               \
-      mma_16816(scl[hg], as_u32(kA.xl[i]), as_u32(kB.xl[i]), as_u32(kA.yl[i]), as_u32(kB.yl[i]), qv.x, qv.y);           \
-      mma_16816(sc[hg], as_u32(kA.xh[i]), as_u32(kB.xh[i]), as_u32(kA.yh[i]), as_u32(kB.yh[i]), qv.x, qv.y);            \
-    }                                                                                                                   \
+#define PQ_KHALF(INDEX, L1, R2, H, HALF)                                                                      \
+  {                                                                                                           \
+    KeyHalf kA, kB;                                                                                           \
+    decode_key_half<2 * (H) + (HALF), 2 * (HALF)>(INDEX##A, L1##A, R2(as_h2(rrA)), tu, tk, kA);               \
+    decode_key_half<2 * (H) + (HALF), 2 * (HALF)>(INDEX##B, L1##B, R2(as_h2(rrB)), tu, tk, kB);               \
+    _Pragma("unroll") for (int i = 0; i < 2; ++i) _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {        \
+      constexpr int kKs0 = 4 * (H) + 2 * (HALF);                                                              \
+      const uint2 qv = kQInRegs ? qb[kQInRegs ? kKs0 + i : 0] : lds64(qf + hg * 2048 + (kKs0 + i) * 256);     \
+      mma_16816(scl[hg], as_u32(kA.xl[i]), as_u32(kB.xl[i]), as_u32(kA.yl[i]), as_u32(kB.yl[i]), qv.x, qv.y); \
+      mma_16816(sc[hg], as_u32(kA.xh[i]), as_u32(kB.xh[i]), as_u32(kA.yh[i]), as_u32(kB.yh[i]), qv.x, qv.y);  \
+    }                                                                                                         \
   }
-          const uint32_t ixA = half_indices_of_blocks<kExact>(c2A, c3A, c4A), ixB = half_indices_of_blocks<kExact>(c2B, c3B, c4B);
+          const uint32_t ixA = half_indices_of_blocks(c2A, c3A, c4A), ixB = half_indices_of_blocks(c2B, c3B, c4B);
           const uint32_t l1A = l1pA.x, l1B = l1pB.x, l1hA = l1pA.y, l1hB = l1pB.y;
           PQ_KHALF(ix, l1, __low2half2, 0, 0)
           PQ_KHALF(ix, l1, __low2half2, 0, 1)
@@ -1004,27 +990,27 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
           }
           uint32_t ixv[2];
 #pragma unroll
-          for (int j = 0; j < 2; ++j) ixv[j] = half_indices_of_tokens<kExact>(c2v[j], c3v[j] >> (4 * (g & 1)), c4v[j] >> (2 * g));
-#define PQ_VHALF(HALF)                                                                                   \
-  {                                                                                                      \
-    __half2 u0[2], u1[2], u2[2], u3[2];                                                                  \
-    value_half<kExact, (HALF)>(ixv[0], __low2half2(as_h2(rr.x)), uv, u0);                                \
-    value_half<kExact, 2 + (HALF)>(ixv[0], __high2half2(as_h2(rr.x)), uv, u1);                           \
-    value_half<kExact, (HALF)>(ixv[1], __low2half2(as_h2(rr.y)), uv, u2);                                \
-    value_half<kExact, 2 + (HALF)>(ixv[1], __high2half2(as_h2(rr.y)), uv, u3);                           \
-    PQ_VSTEP(2 * (HALF), 0) PQ_VSTEP(2 * (HALF) + 1, 1)                                                  \
+          for (int j = 0; j < 2; ++j) ixv[j] = half_indices_of_tokens(c2v[j], c3v[j] >> (4 * (g & 1)), c4v[j] >> (2 * g));
+#define PQ_VHALF(HALF)                                                 \
+  {                                                                    \
+    __half2 u0[2], u1[2], u2[2], u3[2];                                \
+    value_half<(HALF)>(ixv[0], __low2half2(as_h2(rr.x)), tu, u0);      \
+    value_half<2 + (HALF)>(ixv[0], __high2half2(as_h2(rr.x)), tu, u1); \
+    value_half<(HALF)>(ixv[1], __low2half2(as_h2(rr.y)), tu, u2);      \
+    value_half<2 + (HALF)>(ixv[1], __high2half2(as_h2(rr.y)), tu, u3); \
+    PQ_VSTEP(2 * (HALF), 0) PQ_VSTEP(2 * (HALF) + 1, 1)                \
   }
-#define PQ_VSTEP(S, I)                                                                                   \
-  {                                                                                                      \
-    __half2 x0, y0, x1, y1, x2, y2, x3, y3;                                                              \
-    value_sub_block<S>(u0[I], l1v[0], t1a, x0, y0);                                                      \
-    value_sub_block<S>(u1[I], l1v[1], t1a, x1, y1);                                                      \
-    value_sub_block<S>(u2[I], l1v[2], t1a, x2, y2);                                                      \
-    value_sub_block<S>(u3[I], l1v[3], t1a, x3, y3);                                                      \
-    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                                                 \
+#define PQ_VSTEP(S, I)                                                                                     \
+  {                                                                                                        \
+    __half2 x0, y0, x1, y1, x2, y2, x3, y3;                                                                \
+    value_sub_block<S>(u0[I], l1v[0], tv, x0, y0);                                                         \
+    value_sub_block<S>(u1[I], l1v[1], tv, x1, y1);                                                         \
+    value_sub_block<S>(u2[I], l1v[2], tv, x2, y2);                                                         \
+    value_sub_block<S>(u3[I], l1v[3], tv, x3, y3);                                                         \
+    _Pragma("unroll") for (int hg = 0; hg < kHG; ++hg) {                                                   \
       mma_16816(o_acc[hg][S], as_u32(x0), as_u32(y0), as_u32(x1), as_u32(y1), pb[hg][0][0], pb[hg][0][1]); \
       mma_16816(o_acc[hg][S], as_u32(x2), as_u32(y2), as_u32(x3), as_u32(y3), pb[hg][1][0], pb[hg][1][1]); \
-    }                                                                                                    \
+    }                                                                                                      \
   }
           PQ_VHALF(0) PQ_VHALF(1)
 #undef PQ_VHALF
@@ -1034,11 +1020,6 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
       __syncwarp();
       if (lane == 0) mbar_arrive(sm_base + kFsBar + 8 * (kStages + s));
     }
-    };
-    for (int first = 0;;) {
-      const int last = kPaged ? min(n_li, first + kWindow) : n_li;
-      if (exact) stream(std::true_type{}, first, last);
-      else stream(std::false_type{}, first, last);
       first += kWindow;
       if (!kPaged || 2 * first >= st1 - st0) break;
       __syncthreads();   // nothing reads the list any more

@@ -488,10 +488,6 @@ int32_t pq_build_tables(const double* cen, const double* bnd, void* tables_host)
       const double t3 = (s & 1) ? us[k3] : uc[k3];
       split(t4 * t3 * uc[k2] / l1_scale, t4 * t3 * us[k2] / l1_scale, &t.u_tab[s][i].x, &t.u_tab[s][i].y);
     }
-  bool mirrored = true;   // cos of a level-4 centroid = sin of its mirror image, to what the tables hold (22 bits)
-  for (int k = 0; k < 4; ++k)
-    if (std::fabs(uc[8 + k] - us[11 - k]) > 1e-8) mirrored = false;
-  if (l1_scale != 1.0 && mirrored) t.flags |= pq::kFlagExactDecode;
   if (!build_l1_cells(bnd, t.l1_cells)) return PQ_ERR_INVALID_ARG;
   std::memcpy(tables_host, &t, sizeof(t));
   return PQ_OK;

@@ -127,8 +127,8 @@ def test_tensor_core_encoder_with_many_uncertified_decisions(n, analytic):
     assert torch.all((got[0][1].float() - got[1][1].float()).abs() <= 2.0 ** -10 * got[1][1].float())
 
 
-# Codebooks whose decode tables need the residuals of the level-1 factors and both halves of the level-4 factors (the analytic one
-# needs neither): every level moved, or the top level alone, in the three kernels that read those tables.
+# Codebooks without the symmetries of the analytic one: every level moved, or the top level alone, in the three kernels that read the decode
+# tables.
 @pytest.mark.parametrize("moved", [slice(0, 28), slice(24, 28)])
 @pytest.mark.parametrize("g,paged", [(4, False), (4, True), (7, False)])
 def test_attention_with_codebooks_that_are_not_analytic(g, paged, moved):
@@ -142,6 +142,29 @@ def test_attention_with_codebooks_that_are_not_analytic(g, paged, moved):
         q = torch.randn((len(lens), n_q, g * Hkv, 128), generator=torch.Generator(device=DEV).manual_seed(g), device=DEV)
         for kernel in kernels:
             _check_multi(cache, ref, q, lens, kernel)
+
+
+# Scores of a few hundred: an error of the keys' factors that a softmax over small scores hides moves the log-sum-exp by its share of them.
+# Keys and queries are fp16 values with fp16 residuals, 22 bits of each coordinate: 2^-22 of sum |q_i||k_i| <= |q||k| for each of the
+# two, and the float32 sums of the score take as much again.
+@pytest.mark.parametrize("g", [4, 8])
+@pytest.mark.parametrize("fitted", [False, True])
+def test_large_scores_keep_the_precision_of_keys_and_queries(g, fitted):
+    cen, bnd = (t.clone() for t in pq.pq_fit_codebooks())
+    if fitted:
+        cen[:16] += 0.01 * torch.cos(torch.arange(16, dtype=torch.float64))
+        bnd[:15] = 0.5 * (cen[:15] + cen[1:16])
+    lens, Hkv = [600, 33], 2
+    cache, ref = _filled(lens, g * Hkv, Hkv, 128, 70 + g, codebooks=(cen, bnd))
+    q = 16 * synthetic.queries(5, len(lens), g * Hkv, 128, torch.float32, DEV)
+    for kernel in (PERSISTENT, ROWS):
+        pq.pq_debug_fail_next_wait(kernel)
+        _, lse = cache.attend_lse(q)
+        for b in range(len(lens)):
+            for h in range(g * Hkv):
+                K, qh = orc.dequant(ref.k_codes[b, h // g, :lens[b]], ref.k_radii[b, h // g, :lens[b]], ref.cb, ref.S), to_f64(q[b, h])
+                bound = 2.0 ** -20 * np.linalg.norm(qh) * np.linalg.norm(K, axis=1).max() * 128 ** -0.5
+                assert abs(float(lse[b, h]) - orc.log_sum_exp_scores(qh, K, 128 ** -0.5)) < bound, (kernel, b, h)
 
 
 # One or two units of a longer sequence: clusters of sixteen blocks (the limit), also where a block un-rotates one coordinate.
