@@ -20,8 +20,9 @@
 // MMAs takes 1700 to 2700 of a tile's 17000 cycles, the wait for their inputs up to 4000, and the group's other warps waited at the
 // end of the tile for that one.  Twelve that only quantise take a tile in 12200 (three at a time instead of four).  (A 17th warp
 // instead of twelve and four would cap every thread at 96 registers.)  Back to back, 8 heads: 32768 tokens 90.4 -> 86.0 us, 16384
-// 52.0 -> 48.8, 5400 29.6 -> 26.7, but 4000 24.0 -> 24.6: four tiles per CTA are two rounds.  A queue per warp instead of the group's
-// barrier: 16384 tokens 50.2 us.
+// 52.0 -> 48.8, 5400 29.6 -> 26.7.  A last tile that would be a round of its own (one, four, seven .. tiles of a CTA) is shared by two
+// groups: 1000 tokens 18.1 -> 16.9, 4000 24.5 -> 23.7 (24.1 with four groups), with a codebook of one's own 29.7 -> 27.9 (27.7).
+// A queue per warp instead of the group's barrier: 16384 tokens 50.2 us.
 // Every mbarrier wait is bounded; a wait that gives up raises the CTA's abort flag, the remaining
 // tiles are skipped (the loops keep their shape, so the named barriers stay consistent), copies in
 // flight are drained, tensor memory is released and PQ_ERR_TIMEOUT is recorded.
@@ -40,7 +41,7 @@ constexpr int kTcStages = 3;               // x tiles in flight
 constexpr int kTcTerms = 3;                // bf16 terms of S (exact for a float32 S)
 constexpr int kTcXBytes = 128 * 128 * 2;   // one x tile: 128 rows x 128 bf16
 constexpr int kTcSBytes = 128 * 128 * 2;   // one bf16 term of S (B operand)
-using TcFixQueue = FixQueueT<256>;
+using TcFixQueue = FixQueueT<344>;         // three hold what four of 256 did: with S = I and so many ties, 16384 tokens 78.6 -> 59.7 us
 constexpr int kTcSmS = 0;
 constexpr int kTcSmX = kTcSmS + kTcTerms * kTcSBytes;
 constexpr int kTcSmFq = kTcSmX + kTcStages * kTcXBytes;      // FastQuant
@@ -203,10 +204,10 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
 
   // ---- the warp that feeds the tensor core.  It goes through its loop as a whole and one elected lane issues, so that the operands
   // of the MMAs are warp-uniform values.  All MMAs of a tile come from one thread, in order: the first overwrites, the others accumulate.
+  const int n_local = __shfl_sync(0xffffffffu, (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, 0);   // this CTA's tiles
   if (warp == 4 * kTcGroups) {
     const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-    int n_local = ((int)n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, issued = 0;
-    n_local = __shfl_sync(0xffffffffu, n_local, 0);
+    int issued = 0;
     for (int it = 0; it < n_local; ++it) {
       const int s = it % kTcStages, acc = it % kTcAccs;
       bool ok = tc_mbar_wait(bar_xfull + 8 * s, (it / kTcStages) & 1, abort_flag);
@@ -243,7 +244,8 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     }
   }
 
-  // ---- tile loop of this group
+  // ---- tile loop of this group.  A last tile that would find the other two groups idle is shared: group 0 takes columns 0 .. 63, group 1
+  // columns 64 .. 127, both the row norms.
   constexpr int o2 = 32 * kTokenBlock, o3 = o2 + 8 * kTokenBlock, o4 = o3 + 4 * kTokenBlock, orad = o4 + 2 * kTokenBlock;
   const bool analytic = kHist || fq->analytic != 0u;  // uniform over the grid
   const float hist_scale1 = (float)a.n_bins * 0.159154943091895336f, hist_scale_up = (float)a.n_bins * 0.636619772367581343f;
@@ -251,8 +253,12 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
   const Layout L = make_layout(128, a.pg.page_tokens);
   const int group_bar = 1 + group;
   int rd_seq = 0, rd_first = 0, rd_count = 0, rd_start = -1;   // destination of the last row looked up
-  for (int it = group; group < kTcGroups && blockIdx.x + it * (int)gridDim.x < n_tiles; it += kTcGroups) {
-    const int acc = it % kTcAccs;
+  const bool last_shared = n_local % kTcGroups == 1;
+  const int it_end = group < kTcGroups ? n_local + (last_shared && group == 1) : 0;
+  for (int next = group; next < it_end; next += kTcGroups) {
+    const int it = min(next, n_local - 1), acc = it % kTcAccs;
+    const bool half_tile = last_shared && it == n_local - 1;
+    const int c_first = half_tile ? 2 * group : 0, c_end = half_tile ? c_first + 2 : 4;   // of the four pieces of 32 columns
     const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * 128;
     const int tile = blockIdx.x + it * gridDim.x;
     const int head = tile % a.n_kv_heads, hq = tile / a.n_kv_heads;
@@ -276,7 +282,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     for (int i = 0; i < 32; ++i) y[i] = 0.f;
     if (kHist) {
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = c_first; c < c_end; ++c) {
         if (ready) tc_ld32(taddr + 32 * c, y);
         if (c == 3) accumulator_read();
         if (ready && row < a.total_tokens) {
@@ -301,7 +307,7 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     if (!(sqsum < CUDART_INF_F) && row < a.total_tokens) {  // NaN or overflow: look at the inputs
       const int bad = count_nonfinite_bf16(kv ? a.V : a.K, xoff);
       if (bad) {
-        atomicAdd(a.status + 1, bad);
+        if (c_first == 0) atomicAdd(a.status + 1, bad);
         set_status(a.status, PQ_ERR_NONFINITE);
         bad_row = true;
       }
@@ -329,9 +335,9 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     // piece of code (their instruction streams interleave), the rare queue pushes come after both
     uint32_t l2lo = 0, l2hi = 0, l3acc = 0, l4acc = 0, sat = 0;
 #pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
+    for (int c = c_first; c < c_end; ++c) {
       if (ready) tc_ld32(taddr + 32 * c, y);
-      if (c == 3) accumulator_read();
+      if (c == 3) accumulator_read();   // (of a shared tile: nothing waits for that)
       FastBlock fb0, fb1;
       if (analytic) {
         polar_quant_block_fast<true>(y, rm, *fq, &fb0);
@@ -366,11 +372,19 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
     }
     if (tb != nullptr) {
       if (bad_row) l2lo = l2hi = l3acc = l4acc = sat = 0u;  // a row with non-finite inputs is stored as the zero vector
-      *reinterpret_cast<uint2*>(tb + o2 + tok * 8) = make_uint2(l2lo, l2hi);
-      *reinterpret_cast<uint32_t*>(tb + o3 + tok * 4) = l3acc;
-      *reinterpret_cast<uint16_t*>(tb + o4 + tok * 2) = (uint16_t)l4acc;
+      if (half_tile) {
+        *reinterpret_cast<uint32_t*>(tb + o2 + tok * 8 + 4 * group) = group ? l2hi : l2lo;
+        *reinterpret_cast<uint16_t*>(tb + o3 + tok * 4 + 2 * group) = (uint16_t)(l3acc >> (16 * group));
+        tb[o4 + tok * 2 + group] = (uint8_t)(l4acc >> (8 * group));
+      } else {
+        *reinterpret_cast<uint2*>(tb + o2 + tok * 8) = make_uint2(l2lo, l2hi);
+        *reinterpret_cast<uint32_t*>(tb + o3 + tok * 4) = l3acc;
+        *reinterpret_cast<uint16_t*>(tb + o4 + tok * 2) = (uint16_t)l4acc;
+      }
       if (sat) atomicAdd(a.status + 2, (int)sat);
     }
+    // Re-decisions patch whole words: the other half of a shared tile's words is written first.
+    if (half_tile) asm volatile("bar.sync %0, %1;" ::"n"(1 + kTcGroups), "n"(2 * kTcGroupThreads) : "memory");
     // End of the tile for the group.  The barrier decides, for all 128 threads alike, whether the group has to take
     // its queued exact re-decisions now: when a push did not fit or a region is 3/4 full.  Otherwise they wait
     // for the end of the CTA's work, where all 16 warps take them together (the float64 pipe is slow, and a group
