@@ -105,8 +105,8 @@ def test_single_query_kernels(d, g):
 
 # The tensor-core encoder where a group's queue of uncertified decisions fills up again and again (zero rows, rows on the boundaries of an
 # unrotated codebook), at every number of tiles that its three groups of warps can be left with, against the float32 encoder: the same
-# codes and status counts, radii that are neighbours at most.
-@pytest.mark.parametrize("n", [128, 129, 640, 1700, 2500])
+# codes and status counts, radii that are neighbours at most.  One to six tiles per CTA: the last of one or four is shared by two groups.
+@pytest.mark.parametrize("n", [128, 129, 640, 1700, 2500, 4700, 6000])
 @pytest.mark.parametrize("analytic", [True, False])
 def test_tensor_core_encoder_with_many_uncertified_decisions(n, analytic):
     Hkv = 8
