@@ -3,23 +3,23 @@
 // attention kernel, where a CTA needs them for its own 128 rows and repeats them for every range of the blocks, they took 90 us
 // of every CTA's time.
 // A block of 256 threads takes kTile rows.  64 rows: thread = 4 columns x 8 rows (a warp shares its rows, so its reads of them
-// are broadcasts, and reads 512 consecutive bytes of S), bound by the multiply-adds.  8 or 16 rows, while that many blocks do not fill
+// are broadcasts, and reads 512 consecutive bytes of S), bound by the multiply-adds.  8, 16 or 32 rows, while that many blocks do not fill
 // the device: thread = one column x half of the rows; every warp reading all of S takes twice as many shared-memory wavefronts,
 // which bound such a block.  As long as every block can have an SM to itself it asks for more than half of the shared memory: two or
 // three on the SMs that the attention kernel left first took 7 us each for a product of 2.
+// Attention of 32 queries in four sequences of 150 tokens, 32/8 heads, 4096 rows: 34 us with tiles of 32, 39 with 16 or 64 (tcgen05 kernel).
 #pragma once
 
 namespace pq {
 
 constexpr int kRotThreads = 256, kRotSStride = 132;
-constexpr int kRotAlone = 116 * 1024, kRotSms = 148;
+constexpr int kRotAlone = 116 * 1024;
 template <int kTile>
-inline int rot_smem_bytes(int64_t n_rows) {
+inline int rot_smem_bytes(int64_t n_rows, int n_sm) {
   constexpr int need = (128 * kRotSStride + kTile * 128) * 4;
   static_assert(need <= kRotAlone, "the limit that the kernels are configured for");
-  return n_rows <= kRotSms * kTile ? kRotAlone : need;
+  return n_rows <= (int64_t)n_sm * kTile ? kRotAlone : need;
 }
-inline int rot_tile(int64_t n_rows) { return n_rows <= 8 * kRotSms ? 8 : n_rows <= 16 * kRotSms ? 16 : 64; }
 
 // What a thread computes of the tile's product: kRows rows from r0 on, kCols columns from c0 on.
 template <int kTile>
@@ -312,50 +312,42 @@ static int32_t launch_dependent(void (*kernel)(Params...), dim3 grid, int thread
   return launch_status();
 }
 
-template <int kTile>
-static int32_t launch_rotate_as(const float* S, const void* q, int io_dtype, int64_t n_rows, float factor, __half* qrot, cudaStream_t stream) {
-  static DeviceMemo configured;
-  if (configure_for_device(rotate_rows_kernel<kTile>, kRotAlone, configured) == 0) return PQ_ERR_CUDA;
-  return launch_dependent(rotate_rows_kernel<kTile>, dim3((unsigned)((n_rows + kTile - 1) / kTile)), kRotThreads, rot_smem_bytes<kTile>(n_rows),
-                          stream, S, q, io_dtype, n_rows, factor, qrot);
+// `launch` with the tile for the number of rows as a constant, and the device's SMs.
+template <class Launch>
+static int32_t with_rot_tile(int64_t n_rows, Launch launch) {
+  static DeviceMemo sm_count;
+  const int n_sm = sm_count_of_device(sm_count);
+  if (n_sm == 0) return PQ_ERR_CUDA;
+  if (n_rows <= 8 * (int64_t)n_sm) return launch(std::integral_constant<int, 8>{}, n_sm);
+  if (n_rows <= 16 * (int64_t)n_sm) return launch(std::integral_constant<int, 16>{}, n_sm);
+  if (n_rows <= 32 * (int64_t)n_sm) return launch(std::integral_constant<int, 32>{}, n_sm);
+  return launch(std::integral_constant<int, 64>{}, n_sm);
+}
+template <int kTile, typename... Params, typename... Args>
+static int32_t launch_rot_kernel(void (*kernel)(Params...), DeviceMemo& configured, int64_t n_rows, int n_sm, cudaStream_t stream, Args... args) {
+  if (configure_for_device(kernel, kRotAlone, configured) == 0) return PQ_ERR_CUDA;
+  return launch_dependent(kernel, dim3((unsigned)((n_rows + kTile - 1) / kTile)), kRotThreads, rot_smem_bytes<kTile>(n_rows, n_sm), stream, args...);
 }
 static int32_t launch_rotate(const float* S, const void* q, int io_dtype, int64_t n_rows, float factor, __half* qrot, cudaStream_t stream) {
-  switch (rot_tile(n_rows)) {
-    case 8: return launch_rotate_as<8>(S, q, io_dtype, n_rows, factor, qrot, stream);
-    case 16: return launch_rotate_as<16>(S, q, io_dtype, n_rows, factor, qrot, stream);
-    default: return launch_rotate_as<64>(S, q, io_dtype, n_rows, factor, qrot, stream);
-  }
-}
-template <int kTile>
-static int32_t launch_unrotate_as(const float* S, const float* parts, const float* lse, int n_parts, int64_t n_rows, void* out, int out_dtype,
-                                  int32_t* status, cudaStream_t stream) {
-  static DeviceMemo configured;
-  if (configure_for_device(merge_unrotate_kernel<kTile>, kRotAlone, configured) == 0) return PQ_ERR_CUDA;
-  return launch_dependent(merge_unrotate_kernel<kTile>, dim3((unsigned)((n_rows + kTile - 1) / kTile)), kRotThreads, rot_smem_bytes<kTile>(n_rows),
-                          stream, S, parts, lse, n_parts, n_rows, out, out_dtype, status);
+  return with_rot_tile(n_rows, [&](auto tile, int n_sm) {
+    static DeviceMemo configured;
+    return launch_rot_kernel<tile>(rotate_rows_kernel<tile>, configured, n_rows, n_sm, stream, S, q, io_dtype, n_rows, factor, qrot);
+  });
 }
 static int32_t launch_unrotate(const float* S, const float* parts, const float* lse, int n_parts, int64_t n_rows, void* out, int out_dtype,
                                int32_t* status, cudaStream_t stream) {
-  switch (rot_tile(n_rows)) {
-    case 8: return launch_unrotate_as<8>(S, parts, lse, n_parts, n_rows, out, out_dtype, status, stream);
-    case 16: return launch_unrotate_as<16>(S, parts, lse, n_parts, n_rows, out, out_dtype, status, stream);
-    default: return launch_unrotate_as<64>(S, parts, lse, n_parts, n_rows, out, out_dtype, status, stream);
-  }
-}
-
-template <int kTile>
-static int32_t launch_merge_rows_as(const DecodeArgs& a, cudaStream_t stream) {
-  static DeviceMemo configured;
-  if (configure_for_device(merge_rows_kernel<kTile>, kRotAlone, configured) == 0) return PQ_ERR_CUDA;
-  return launch_dependent(merge_rows_kernel<kTile>, dim3((unsigned)(((int64_t)a.batch * a.n_q_heads + kTile - 1) / kTile)), kRotThreads,
-                          rot_smem_bytes<kTile>((int64_t)a.batch * a.n_q_heads), stream, a.S, a);
+  return with_rot_tile(n_rows, [&](auto tile, int n_sm) {
+    static DeviceMemo configured;
+    return launch_rot_kernel<tile>(merge_unrotate_kernel<tile>, configured, n_rows, n_sm, stream, S, parts, lse, n_parts, n_rows, out, out_dtype,
+                                   status);
+  });
 }
 static int32_t launch_merge_rows(const DecodeArgs& a, cudaStream_t stream) {
-  switch (rot_tile((int64_t)a.batch * a.n_q_heads)) {
-    case 8: return launch_merge_rows_as<8>(a, stream);
-    case 16: return launch_merge_rows_as<16>(a, stream);
-    default: return launch_merge_rows_as<64>(a, stream);
-  }
+  const int64_t n_rows = (int64_t)a.batch * a.n_q_heads;
+  return with_rot_tile(n_rows, [&](auto tile, int n_sm) {
+    static DeviceMemo configured;
+    return launch_rot_kernel<tile>(merge_rows_kernel<tile>, configured, n_rows, n_sm, stream, a.S, a);
+  });
 }
 
 }  // namespace pq

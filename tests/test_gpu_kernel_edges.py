@@ -144,6 +144,18 @@ def test_attention_with_codebooks_that_are_not_analytic(g, paged, moved):
             _check_multi(cache, ref, q, lens, kernel)
 
 
+# The rotations around several queries take 8, 16, 32 or 64 rows per block: one sequence of 64 rows on both sides of where each begins,
+# and a number of rows that leaves a remainder of every tile.
+@pytest.mark.parametrize("per_sm,more", [(8, 0), (8, 1), (16, 1), (32, 0), (32, 1)])
+@pytest.mark.parametrize("kernel,n_q", [(ROWS, 16), (TCGEN05, 16), (ROWS, 15)])
+def test_rotations_of_many_rows(kernel, n_q, per_sm, more):
+    B = per_sm * torch.cuda.get_device_properties(0).multi_processor_count // 64 + more
+    lens = [1 + 7 * b % 40 for b in range(B)]
+    cache, ref = _filled(lens, 4, 1, 128, 80)
+    q = torch.randn((B, n_q, 4, 128), generator=torch.Generator(device=DEV).manual_seed(n_q), device=DEV)
+    _check_multi(cache, ref, q, lens, kernel)
+
+
 # Scores of a few hundred: an error of the keys' factors that a softmax over small scores hides moves the log-sum-exp by its share of them.
 # Keys and queries are fp16 values with fp16 residuals, 22 bits of each coordinate: 2^-22 of sum |q_i||k_i| <= |q||k| for each of the
 # two, and the float32 sums of the score take as much again.
