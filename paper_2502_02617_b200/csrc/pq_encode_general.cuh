@@ -159,17 +159,23 @@ __device__ __forceinline__ int64_t ge_destination(const GenEncodeArgs& a, int ro
   return off * kTokenBlock + pos % kTokenBlock;
 }
 
-// Bounds on the error of the product on tensor cores relative to ||x||_2, as rot_err in the kernel and rotation_block_error: products
-// of bf16 values are exact in float32, the three terms represent S to 2^-26, and each of the six accumulating MMAs of a slice is
-// taken to add at most 2 * 2^-24 of the largest of its terms (16 products and the running sum); over the coordinates of a block the
-// squares of those add up to at most the squared norm of the slice of x, as they do for one coordinate; the slices' norms add up to sqrt(slices) ||x|| at most and their sums are added one by one.  Measured against
-// float64 over 2^20 vectors per head dim of 16 to 256 (normal, outlier channels, log-normal, concentrated, positive): at most 0.37
-// of the first bound and 0.42 of the second (head_dim 32; 0.09 and 0.10 at 128).
-__host__ __device__ constexpr float ge_mma_error(int dc) {
-  return 1.1f * (12.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
-}
+// Bounds on the error of the product on tensor cores relative to ||x||_2 (rot_err in the kernel, and as rotation_block_error).  The
+// hardware's sum is not IEEE's: mma.sync m16n8k16 of bf16 truncates its sixteen products, which are exact, and C to multiples of 2^(e - 25),
+// e the largest exponent among them (of a product: the sum of its factors' exponents), adds them exactly and truncates the sum to
+// float32.  An emulation of that agrees with the device on three million sums (normal, wide ranges of exponents, cancelling pairs beside terms
+// at the cut, positive, geometric), bit for bit.  So with M the largest of the terms in magnitude and R the result an MMA is off
+// by at most 16 * 2^-25 M + 2^-23 |R| = 2^-24 (8 M + 2 |R|).
+// Three bf16 terms hold a float32 S exactly (24 bits), the second at most 2^-9 and the third 2^-18 of the first.  A k-step of 16 rows
+// starts from 0 and takes the smallest term first, so M and R are those of the k-step, not of the whole sum:
+//   * a coordinate: M and |R| are at most ||x_k|| ||S_kj|| of the k-step (Cauchy-Schwarz), and these add up to ||x|| ||S_j|| = ||x||: 10.1
+//     with the smaller terms; then a rounding of 2^-24 for each addition of a k-step but the first;
+//   * the coordinates of a block in the 2-norm: the squares of M add up to at most sum_k x_k^2 sum_j S_kj^2 <= ||x_k||^2, those of R too
+//     (spectral norm), and the k-steps' norms to sqrt(k-steps) ||x|| at most.
+// 10 % and 2 % for the rounding of S (its columns are unit vectors to float32) and second order.
+__host__ __device__ constexpr int ge_mma_steps(int dc) { return dc / 16; }
+__host__ __device__ constexpr float ge_mma_error(int dc) { return 1.1f * (10.1f + ge_mma_steps(dc)) * 5.9604644775390625e-08f; }
 __host__ __device__ constexpr float ge_mma_block_error(int dc) {
-  return 1.02f * (12.f * const_sqrt((dc + kGeSlice - 1) / kGeSlice) + (dc + kGeSlice - 1) / kGeSlice + 0.25f) * 5.9604644775390625e-08f;
+  return 1.02f * (10.1f * const_sqrt(ge_mma_steps(dc)) + ge_mma_steps(dc)) * 5.9604644775390625e-08f;
 }
 
 // Three bf16 terms of a pair of float32 values (round to nearest each: together within 2^-26 of the values).
@@ -199,7 +205,7 @@ __device__ __forceinline__ void ge_mma(float* d, const uint32_t (&a)[4], uint32_
 
 // y = x S of a tile of V bf16 vectors (xh [V][dc + 8]) on tensor cores, into y [V][dc / 16][20] over the same memory.  S goes through
 // shared memory in slices of 32 rows, split into three bf16 terms as it arrives; a warp owns eight 16 x 8 tiles of y, smallest terms
-// first, a fresh accumulator per slice.
+// first, a fresh accumulator per k-step (see the bounds).
 __device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, int dc, float* xy, float* Ss, int tid) {
   const int lane = tid & 31, warp = tid >> 5, stride = dc + 8;
   const __nv_bfloat16* xh = reinterpret_cast<const __nv_bfloat16*>(xy);
@@ -233,11 +239,6 @@ __device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, in
         *reinterpret_cast<uint2*>(Sw + ((t * kGeSlice + k) * stride + n) / 2) = make_uint2(lo[t], hi[t]);
     }
     __syncthreads();
-    float acc[8][4];
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[t][e] = 0.f;
 #pragma unroll 1
     for (int ks = 0; ks < nk; ks += 16) {
       uint32_t A[4];
@@ -245,19 +246,21 @@ __device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, in
       for (int p = 0; p < 4; ++p) {
         const int m = m0 + p / pairs, n = n0 + (p % pairs) * 16;
         if (p % pairs == 0) ge_ldmatrix<false>(xh + (m * 16 + lr) * stride + k0 + ks + lc, A);
+        float acc[2][4] = {};
 #pragma unroll
         for (int t = 2; t >= 0; --t) {
           uint32_t B[4];
           ge_ldmatrix<true>(reinterpret_cast<const __nv_bfloat16*>(Sw) + (t * kGeSlice + ks + lr) * stride + n + lc, B);
-          ge_mma(acc[2 * p], A, B[0], B[1]);
-          ge_mma(acc[2 * p + 1], A, B[2], B[3]);
+          ge_mma(acc[0], A, B[0], B[1]);
+          ge_mma(acc[1], A, B[2], B[3]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          tot[2 * p][e] += acc[0][e];
+          tot[2 * p + 1][e] += acc[1][e];
         }
       }
     }
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) tot[t][e] += acc[t][e];
   }
   __syncthreads();   // x has been used: y takes its place
 #pragma unroll

@@ -53,8 +53,8 @@ __device__ __forceinline__ bool radius_unsure(float r, float err) {
 // which is at most that of the slice of x (the rows and columns of an orthogonal S that meet there have spectral norm 1 or less);
 // the slices' norms add up to sqrt(slices) ||x|| at most, and each of the additions moves the block by 2^-24 ||x||.  2 % for the
 // rounding of S and second order.
-__host__ __device__ constexpr float const_sqrt(int n) {   // of 1, 2, 4, 8 exactly enough, rounded up
-  return n <= 1 ? 1.f : n <= 2 ? 1.4143f : n <= 4 ? 2.f : 2.8285f;
+__host__ __device__ constexpr float const_sqrt(int n) {   // of 1, 2, 4, 8, 16 exactly enough, rounded up
+  return n <= 1 ? 1.f : n <= 2 ? 1.4143f : n <= 4 ? 2.f : n <= 8 ? 2.8285f : 4.f;
 }
 __host__ __device__ constexpr float rotation_block_error(int chain, int slices) {
   return 1.02f * (chain * const_sqrt(slices) + slices) * 5.9604644775390625e-08f;

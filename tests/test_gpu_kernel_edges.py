@@ -320,6 +320,27 @@ def test_the_encoder_on_tensor_cores_writes_the_bytes_of_the_float32_one(d, bits
     assert torch.equal(caches[0].cache, caches[1].cache) and caches[0].status[:3].tolist() == caches[1].status[:3].tolist()
 
 
+# The product's sums are truncated, so rows whose products all have one sign are its largest errors: columns of S, scaled, with a little of
+# another row.  The bytes are those of the float32 path all the same.
+@pytest.mark.parametrize("d,bits", [(16, None), (32, None), (64, None), (64, (4, 3, 2)), (128, (3,) * 7), (128, (4, 2, 2, 2)), (256, (4, 2, 2, 2, 2))])
+def test_the_encoder_on_tensor_cores_where_its_sums_have_one_sign(d, bits):
+    Hkv, n = 8, 40960 // d
+    make = lambda: (pq.PolarQuantCache(1, Hkv, Hkv, d, capacity=n, seed=6, device=DEV) if bits is None else
+                    pq.GeneralPolarQuantCache(1, Hkv, Hkv, d, bits, n, seed=6, device=DEV))
+    c = make()
+    K, V = synthetic.kv_like(d + n, n, Hkv, d, torch.bfloat16, DEV, n_outliers=0)
+    columns = c.S.t()[torch.arange(n * Hkv, device=DEV) % d].view(n, Hkv, d)
+    K, V = ((columns * 3 + amount * t.float()).bfloat16() for t, amount in ((K, 2.0 ** -8), (V, 2.0 ** -4)))
+    cu = torch.tensor([0, n], dtype=torch.int32, device=DEV)
+    caches = []
+    for k, v in ((K, V), (K.float(), V.float())):
+        c = make()
+        c.cache.zero_()
+        c.encode(k, v, cu)
+        caches.append(c)
+    assert torch.equal(caches[0].cache, caches[1].cache) and caches[0].status[:3].tolist() == caches[1].status[:3].tolist()
+
+
 # Four coordinates per thread where the pointers allow it, else one.  A weighted mean of three float32 values: 1e-6 is eight
 # roundings of 2^-23.
 @pytest.mark.parametrize("d,shift", [(16, 0), (16, 1), (128, 0), (128, 3)])
