@@ -163,11 +163,9 @@ namespace pq {
 
 // The packed cache for split_attention_kernel.  A tile is part of a token-block: five pieces, one per plane, each a multiple
 // of 16 bytes long and 16-byte aligned in the cache and in the buffer.
-template <int D>
+template <int D, bool kWithPairs = false>
 struct PackedSplit {
-  // pairs of level-1 codes where the loop over the tokens is what takes the time: at head_dim 128 the kernel has short contexts only, and
-  // at 16 a call is mostly its start (256 tokens, one head: 12.2 -> 12.5 us with them)
-  static constexpr bool kEarlyTables = true, kPairs = D == 64 || D == 32;
+  static constexpr bool kEarlyTables = true, kPairs = kWithPairs;   // see kPairTokens
   static constexpr int kTabMax = 32, kDim = D;
   // the planes of a token-block (make_layout for this head_dim)
   static constexpr int kNb = D / 16, kB1 = 4 * kNb, kB2 = kNb, kB3 = kNb >= 2 ? kNb / 2 : 1, kB4 = kNb >= 4 ? kNb / 4 : 1, kBr = 2 * kNb;
@@ -286,10 +284,15 @@ struct PackedSplit {
   }
 };
 
-template <int D>
-static PackedSplit<D> packed_split(const SplitCommon& c, int n_q, const Tables* tables, const uint8_t* cache, const int32_t* lens,
-                                   const Paging& pg) {
-  PackedSplit<D> p;
+// Pairs of level-1 codes in a table of their own (32 KB, filled by every block before its first tile) where the loop over the tokens is what
+// takes the time: head_dim 64 from so many tokens of a block on.  16/8 heads, without and with them: one sequence of 4096 tokens (256
+// a block) 9.35 and 9.19 us, four of 4096 (1024) 13.9 and 13.6; four of 1500 (375) 9.24 and 9.22, of 700 (175) 7.16 and 7.38, one of 300
+// 5.91 and 6.08.  At head_dim 32 nothing is gained at 4096 tokens (10.27 and 10.20 us), at 128 the kernel has short contexts only.
+constexpr int kPairTokens = 256;
+template <int D, bool kWithPairs = false>
+static PackedSplit<D, kWithPairs> packed_split(const SplitCommon& c, int n_q, const Tables* tables, const uint8_t* cache, const int32_t* lens,
+                                               const Paging& pg) {
+  PackedSplit<D, kWithPairs> p;
   p.c = c; p.n_q = n_q; p.tables = tables; p.cache = cache; p.lens = lens; p.pg = pg;
   p.head_bytes = make_layout(D, pg.page_tokens).head_bytes;
   return p;
@@ -957,7 +960,14 @@ static int32_t launch_attention(int32_t head_dim, int32_t n_q_heads, int32_t n_k
   switch (head_dim) {
     case 16: return pq::dispatch_split_attention(pq::packed_split<16>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
     case 32: return pq::dispatch_split_attention(pq::packed_split<32>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
-    case 64: return pq::dispatch_split_attention(pq::packed_split<64>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
+    case 64: {
+      auto split = pq::packed_split<64>(c, n_q, a.tables, a.cache, cache_lens_dev, pg);
+      pq::size_split(split);
+      pq::SplitLoad load = {};
+      if (pq::plan_split(split, pairs, max_len, &load) == 0) return PQ_ERR_CUDA;
+      if (load.waves * load.tokens < pq::kPairTokens) return pq::dispatch_split_attention(split, pairs, max_len, st);
+      return pq::dispatch_split_attention(pq::packed_split<64, true>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
+    }
     default: return pq::dispatch_split_attention(pq::packed_split<128>(c, n_q, a.tables, a.cache, cache_lens_dev, pg), pairs, max_len, st);
   }
 }

@@ -17,7 +17,7 @@
 // whole query by itself instead of meeting the others first, and the merge has one cluster barrier.
 // Measured (32/8 heads; two launches and a workspace before): one sequence of 1000 tokens, head_dim 128 19.8 -> 10.7 us; eight of
 // 4096, head_dim 64 111 -> 32 us; the general layout with three bits and seven levels, eight of 4096, 5330 -> 95 us.
-// Level 1 of the packed layout, head dims 32 and 64: one 16-byte lookup per byte of codes instead of two of 8 bytes, and planes of a staged
+// Level 1 of the packed layout, head_dim 64: one 16-byte lookup per byte of codes instead of two of 8 bytes, and planes of a staged
 // tile at constant distances: 8 sequences of up to 4096 tokens at head_dim 64, four steps with their appends 127.2 -> 123.4 us.
 // kU = 16 for up to four query heads per kv head, 8 for up to eight (the registers of q' and of the accumulators).
 #pragma once
