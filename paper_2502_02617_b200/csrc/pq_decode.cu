@@ -680,10 +680,10 @@ static int32_t launch_persistent(void (*kernel)(DecodeArgs), const DecodeArgs& a
   return launch_status();
 }
 
-template <int kHG>
+template <int kHG, bool kAround>
 static int32_t launch_rows_as(const DecodeArgs& a, bool paged, cudaStream_t stream) {
   static DeviceMemo configured[2];
-  void (*kernel)(DecodeArgs) = paged ? rows_attention_kernel<kHG, true> : rows_attention_kernel<kHG, false>;
+  void (*kernel)(DecodeArgs) = paged ? rows_attention_kernel<kHG, kAround, true> : rows_attention_kernel<kHG, kAround, false>;
   const int n_sm = configure_for_device(kernel, kRowSmTotal, configured[paged ? 1 : 0]);
   return n_sm == 0 ? PQ_ERR_CUDA : launch_persistent(kernel, a, n_sm, kRowThreads, kRowSmTotal, stream);
 }
@@ -700,25 +700,23 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
   // rotation back, and a block that works on two units pays twice (five drafted tokens in four sequences of up to 8192 tokens, encode
   // included: 73.9 -> 58.4 us).  One query has at most eight rows, and its workspace may be the static scratch, which has no room for
   // rotated queries.
-  if (a.n_q > 1) {
-    const int64_t all_rows = (int64_t)a.batch * a.n_q_heads;
-    uint8_t* behind = reinterpret_cast<uint8_t*>(a.ws.elected) + a.ws.bytes;
-    __half* qrot = reinterpret_cast<__half*>(behind);
-    a.qrot = qrot;
-    a.unit_parts = reinterpret_cast<int2*>(qrot + all_rows * 256);
-    const int32_t st = launch_rotate(a.S, a.q, a.io_dtype, all_rows, a.scale * 1.4426950408889634f, qrot, stream);
-    if (st != PQ_OK) return st;
-  }
-  int32_t st;
+  if (a.n_q == 1) return launch_rows_as<2, false>(a, paged, stream);
+  const int64_t all_rows = (int64_t)a.batch * a.n_q_heads;
+  uint8_t* behind = reinterpret_cast<uint8_t*>(a.ws.elected) + a.ws.bytes;
+  __half* qrot = reinterpret_cast<__half*>(behind);
+  a.qrot = qrot;
+  a.unit_parts = reinterpret_cast<int2*>(qrot + all_rows * 256);
+  int32_t st = launch_rotate(a.S, a.q, a.io_dtype, all_rows, a.scale * 1.4426950408889634f, qrot, stream);
+  if (st != PQ_OK) return st;
   switch (rows_groups(cut.rows)) {
-    case 2: st = launch_rows_as<2>(a, paged, stream); break;
-    case 3: st = launch_rows_as<3>(a, paged, stream); break;
-    case 4: st = launch_rows_as<4>(a, paged, stream); break;
-    case 5: st = launch_rows_as<5>(a, paged, stream); break;
-    case 6: st = launch_rows_as<6>(a, paged, stream); break;
-    default: st = launch_rows_as<8>(a, paged, stream); break;
+    case 2: st = launch_rows_as<2, true>(a, paged, stream); break;
+    case 3: st = launch_rows_as<3, true>(a, paged, stream); break;
+    case 4: st = launch_rows_as<4, true>(a, paged, stream); break;
+    case 5: st = launch_rows_as<5, true>(a, paged, stream); break;
+    case 6: st = launch_rows_as<6, true>(a, paged, stream); break;
+    default: st = launch_rows_as<8, true>(a, paged, stream); break;
   }
-  return st != PQ_OK || a.n_q == 1 ? st : launch_merge_rows(a, stream);
+  return st != PQ_OK ? st : launch_merge_rows(a, stream);
 }
 
 // ---- which kernel takes a head_dim-128 call ------------------------------------------------------

@@ -105,33 +105,33 @@ __device__ __forceinline__ void combine_rows(const DecodeArgs& a, const int2* in
   }
   wait_S(bar, phase, abort_flag);
   __syncthreads();
-  // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of four rows at a time
-  const int i_out = tid & 127;
+  // x_hat_i = sum_j y_hat_j S[i][j]: a thread takes output coordinate i of four of the (at most eight) rows
+  const int i_out = tid & 127, r0 = (tid >> 7) * 4;
   const float* srow = S_sm + i_out * kRowSStride;
-#pragma unroll 1
-  for (int r0 = (tid >> 7) * 4; r0 < n_rows; r0 += 8) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-    for (int j = 0; j < 128; j += 4) {
-      const float4 s = *reinterpret_cast<const float4*>(srow + j);
+  for (int j = 0; j < 128; j += 4) {
+    const float4 s = *reinterpret_cast<const float4*>(srow + j);
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float4 y = *reinterpret_cast<const float4*>(y_sm + (r0 + r) * 128 + j);   // rows past n_rows are not stored
-        acc[r] = fmaf(y.w, s.w, fmaf(y.z, s.z, fmaf(y.y, s.y, fmaf(y.x, s.x, acc[r]))));
-      }
+    for (int r = 0; r < 4; ++r) {
+      const float4 y = *reinterpret_cast<const float4*>(y_sm + (r0 + r) * 128 + j);   // rows past n_rows are not stored
+      acc[r] = fmaf(y.w, s.w, fmaf(y.z, s.z, fmaf(y.y, s.y, fmaf(y.x, s.x, acc[r]))));
     }
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      if (r0 + r < n_rows) {
-        const int64_t idx = (int64_t)info[r0 + r].x * 128 + i_out;
-        if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(acc[r]);
-        else reinterpret_cast<float*>(a.out)[idx] = acc[r];
-      }
   }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (r0 + r < n_rows) {
+      const int64_t idx = (int64_t)info[r0 + r].x * 128 + i_out;
+      if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(acc[r]);
+      else reinterpret_cast<float*>(a.out)[idx] = acc[r];
+    }
 }
 
-template <int kHG, bool kPaged>
+// kAround: the rotations are kernels of their own, before and after (several queries, see launch_rows_attention).  Otherwise one query per
+// sequence: the rows are the heads of a group, one row block of at most eight.
+template <int kHG, bool kAround, bool kPaged>
 __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeArgs a) {
+  static_assert(kAround || kHG == 2, "one query has at most eight rows");
   extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((kSmAlign - (smem_u32(smem_raw) & (kSmAlign - 1))) & (kSmAlign - 1));
   const int g_heads = a.n_q_heads / a.n_kv_heads, all_rows = a.n_q * g_heads, R = a.rows_per_block, nrb = a.n_row_blocks;
@@ -155,8 +155,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
   // a programmatic dependent of the kernel before it, like the persistent kernel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();   // the barriers are initialised
-  const bool around = a.qrot != nullptr;   // the rotations are kernels of their own, see launch_rows_attention
-  if (warp == 0 && !around) fetch_S(a.S, sm_base + kRowSmRing, sm_base + kRowSmBarS, lane);   // a constant of the caller, like the tables
+  if (warp == 0 && !kAround) fetch_S(a.S, sm_base + kRowSmRing, sm_base + kRowSmBarS, lane);   // a constant of the caller, like the tables
   build_fast_tables<kRowThreads>(smem, a.tables);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
@@ -176,20 +175,18 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
     return (len_u + kStageTokens - 1) / kStageTokens;
   };
   auto empty_unit = [&](int u) {   // no row sees a token: zeros, and the status says so
-    if (around) {
+    if constexpr (kAround) {
       a.unit_parts[u] = make_int2(0, 0);
-      return;
-    }
-    const int seq = u / (a.n_kv_heads * nrb), rb = u % nrb, hk = (u / nrb) % a.n_kv_heads, n_rows = unit_rows(rb);
+    } else {
 #pragma unroll 1
-    for (int e = 0; e < n_rows * 128; ++e) {
-      const int row = rb * R + (e >> 7), j = row / g_heads;
-      const int64_t idx = (((int64_t)seq * a.n_q + j) * a.n_q_heads + hk * g_heads + (row - j * g_heads)) * 128 + (e & 127);
-      if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
-      else reinterpret_cast<float*>(a.out)[idx] = 0.f;
-      if (a.lse != nullptr && (e & 127) == 0) a.lse[idx >> 7] = -CUDART_INF_F;
+      for (int e = 0; e < g_heads * 128; ++e) {   // u: sequence and kv head
+        const int64_t idx = (int64_t)u * g_heads * 128 + e;
+        if (a.io_dtype == PQ_DTYPE_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[idx] = __float2bfloat16(0.f);
+        else reinterpret_cast<float*>(a.out)[idx] = 0.f;
+        if (a.lse != nullptr && (e & 127) == 0) a.lse[idx >> 7] = -CUDART_INF_F;
+      }
+      if (a.lse == nullptr) set_status(a.status, PQ_ERR_EMPTY);
     }
-    if (a.lse == nullptr) set_status(a.status, PQ_ERR_EMPTY);
   };
 
   const int g = lane >> 2, c = lane & 3;
@@ -238,7 +235,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int li = 0; li < min(kStages - 1, n_li); ++li) issue_copy(li);
       };
-      if (around) {
+      if (kAround) {
         if (tid == 0) first_copies();
       } else if (warp == 0 && batch_no + sg > 0) {
         fetch_S(a.S, ring, bar_S, lane);
@@ -251,9 +248,8 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
       }
       // q' = (q S) * scale * log2(e) of the rows as fp16 value + residual in fragment order: the fragment of
       // (row group, k-step ks, lane) holds, for column n = lane / 4 (row n / 2 of the group; value or residual), coordinates
-      // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.  Read as it is where it was formed before, else formed 16 rows
-      // at a time.
-      if (around) {
+      // 0, 2 | 1, 3 of sub-block ks & 3 of block 2 (lane & 3) + ks / 4.  Read as it is where it was formed before.
+      if constexpr (kAround) {
         __syncthreads();   // info
         static_assert(kRowThreads == 8 * 32, "a thread per fragment of a row group");
         const int ks = tid >> 5, at = (lane >> 2 & 1) * 128 + (2 * (lane & 3) + (ks >> 2)) * 16 + (ks & 3) * 4;
@@ -266,58 +262,55 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         __syncthreads();
       } else {
         float* q_in = reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn);
-        constexpr int kAt = 4 * kHG < 16 ? 4 * kHG : 16, kMine = kAt / 2;   // rows at a time; rows of a thread
+        constexpr int kMine = 4;                                            // rows of a thread
         const int j = tid & 127, r_mine = (tid >> 7) * kMine;               // its rotated coordinate
         const int blk = j >> 4, ks = (blk & 1) * 4 + ((j >> 2) & 3);
         uint8_t* dst = smem + kRowSmQ + ks * 256 + (blk >> 1) * 8 + (j & 1) * 4 + ((j >> 1) & 1) * 2;
-#pragma unroll 1
-        for (int r0 = 0; r0 < 4 * kHG; r0 += kAt) {
-          __syncthreads();
-          for (int i = tid; i < kAt * 16; i += kRowThreads) {   // eight elements of a row (rows past the last repeat it)
-            const int64_t at = (int64_t)info[r0 + (i >> 4)].x * 128 + 8 * (i & 15);
-            float4 lo, hi;
-            if (a.io_dtype == PQ_DTYPE_BF16) {
-              const uint4 w = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.q) + at);
-              lo = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
-                               __uint_as_float(w.y & 0xFFFF0000u));
-              hi = make_float4(__uint_as_float(w.z << 16), __uint_as_float(w.z & 0xFFFF0000u), __uint_as_float(w.w << 16),
-                               __uint_as_float(w.w & 0xFFFF0000u));
-            } else {
-              lo = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at);
-              hi = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at + 4);
-            }
-            *reinterpret_cast<float4*>(q_in + 8 * i) = lo;
-            *reinterpret_cast<float4*>(q_in + 8 * i + 4) = hi;
+        __syncthreads();
+        if (tid < 8 * 16) {   // eight elements of a row (rows past the last repeat it)
+          const int64_t at = (int64_t)info[tid >> 4].x * 128 + 8 * (tid & 15);
+          float4 lo, hi;
+          if (a.io_dtype == PQ_DTYPE_BF16) {
+            const uint4 w = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.q) + at);
+            lo = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                             __uint_as_float(w.y & 0xFFFF0000u));
+            hi = make_float4(__uint_as_float(w.z << 16), __uint_as_float(w.z & 0xFFFF0000u), __uint_as_float(w.w << 16),
+                             __uint_as_float(w.w & 0xFFFF0000u));
+          } else {
+            lo = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at);
+            hi = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + at + 4);
           }
-          if (r0 == 0) wait_S(bar_S, n_S++ & 1, abort_flag);
-          __syncthreads();
-          float acc[kMine];
+          *reinterpret_cast<float4*>(q_in + 8 * tid) = lo;
+          *reinterpret_cast<float4*>(q_in + 8 * tid + 4) = hi;
+        }
+        wait_S(bar_S, n_S++ & 1, abort_flag);
+        __syncthreads();
+        float acc[kMine];
 #pragma unroll
-          for (int r = 0; r < kMine; ++r) acc[r] = 0.f;
+        for (int r = 0; r < kMine; ++r) acc[r] = 0.f;
 #pragma unroll 4
-          for (int k = 0; k < 128; k += 4) {
-            float s_col[4];
+        for (int k = 0; k < 128; k += 4) {
+          float s_col[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) s_col[e] = S_sm[(k + e) * kRowSStride + j];
-#pragma unroll
-            for (int r = 0; r < kMine; ++r) {
-              const float4 q4 = *reinterpret_cast<const float4*>(q_in + (r_mine + r) * 128 + k);
-              acc[r] = fmaf(q4.w, s_col[3], fmaf(q4.z, s_col[2], fmaf(q4.y, s_col[1], fmaf(q4.x, s_col[0], acc[r]))));
-            }
-          }
+          for (int e = 0; e < 4; ++e) s_col[e] = S_sm[(k + e) * kRowSStride + j];
 #pragma unroll
           for (int r = 0; r < kMine; ++r) {
-            const int row = r0 + r_mine + r;
-            const float v = acc[r] * (a.scale * 1.4426950408889634f);
-            const __half qh = __float2half_rn(v);
-            __half* at = reinterpret_cast<__half*>(dst + (row >> 2) * 2048 + 2 * (row & 3) * 32);
-            at[0] = qh;
-            at[16] = __float2half_rn(v - __half2float(qh));
+            const float4 q4 = *reinterpret_cast<const float4*>(q_in + (r_mine + r) * 128 + k);
+            acc[r] = fmaf(q4.w, s_col[3], fmaf(q4.z, s_col[2], fmaf(q4.y, s_col[1], fmaf(q4.x, s_col[0], acc[r]))));
           }
+        }
+#pragma unroll
+        for (int r = 0; r < kMine; ++r) {
+          const int row = r_mine + r;
+          const float v = acc[r] * (a.scale * 1.4426950408889634f);
+          const __half qh = __float2half_rn(v);
+          __half* at = reinterpret_cast<__half*>(dst + (row >> 2) * 2048 + 2 * (row & 3) * 32);
+          at[0] = qh;
+          at[16] = __float2half_rn(v - __half2float(qh));
         }
         __syncthreads();   // S has been used: the ring takes its place
       }
-      if (tid == 0 && !around) first_copies();
+      if (tid == 0 && !kAround) first_copies();
       float o_acc[kHG][4][4];
       float m_run[kHG], l_run[kHG];   // of row c + 4 hg, as in the persistent kernel
       int limit[kHG];                 // tokens the row sees
@@ -522,26 +515,25 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_attention_kernel(DecodeAr
         }
         __stcg(reinterpret_cast<float2*>(a.ws.ml) + (int64_t)slot * R + tid, make_float2(M, l));
       }
-      if (around) {   // merge_rows_kernel does the rest
+      if constexpr (kAround) {   // merge_rows_kernel does the rest
         if (part == 0 && tid == 0) a.unit_parts[u] = make_int2(unit_slot, n_parts);
-        __syncthreads();   // the ring is free again for the next unit
-        continue;
-      }
-      __syncthreads();
-      if (warp == 0) elect_combiner(a, u, unit_slot, part, n_parts, lane, is_last);
-      __syncthreads();
-      if (*is_last) {
-        if (warp == 0) fetch_S(a.S, ring, bar_S, lane);
-        combine_rows(a, info, n_rows, unit_slot, n_parts, reinterpret_cast<float*>(smem + kRowSmQ),
-                     reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn), S_sm, bar_S, n_S++ & 1, abort_flag);
-        if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
+      } else {
+        __syncthreads();
+        if (warp == 0) elect_combiner(a, u, unit_slot, part, n_parts, lane, is_last);
+        __syncthreads();
+        if (*is_last) {
+          if (warp == 0) fetch_S(a.S, ring, bar_S, lane);
+          combine_rows(a, info, n_rows, unit_slot, n_parts, reinterpret_cast<float*>(smem + kRowSmQ),
+                       reinterpret_cast<float*>(smem + kRowSmRing + kRowQIn), S_sm, bar_S, n_S++ & 1, abort_flag);
+          if (tid == 0 && n_parts > 1) *reinterpret_cast<volatile uint32_t*>(a.ws.elected + u) = 0u;
+        }
       }
       __syncthreads();  // the ring is free again for the next unit
     }
   }
   // A block whose range of the work lies between two units has no segment: the copy of S that it started ahead of the split lands
   // before the block ends.
-  if (n_S == 0 && !around) wait_S(bar_S, 0u, abort_flag);
+  if (n_S == 0 && !kAround) wait_S(bar_S, 0u, abort_flag);
   if (tid == 0 && *abort_flag) set_status(a.status, PQ_ERR_TIMEOUT);
 }
 
