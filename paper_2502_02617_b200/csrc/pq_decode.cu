@@ -722,16 +722,18 @@ static int32_t launch_rows_attention(DecodeArgs a, const RowCut& cut, int n_seq,
 // ---- which kernel takes a head_dim-128 call ------------------------------------------------------
 // Four kernels compute the same attention; which is fastest depends on the rows per kv head (queries x heads of the group), on
 // the number of (kv head, sequence) units and on the length.  Each is estimated in us by a formula fitted to measurements on
-// B200 (SM clock 1.9 GHz; 1 to 64 queries, 1 to 32 sequences of 150 to 65536 tokens, 32/8, 28/4, 16/2, 8/8 and 8/1 heads: 2986
-// calls, up to four kernels each), and the shortest estimate wins; over those calls the choice is 0.3 % slower than the best
-// one on average, 28 % at worst (2.5 % and 55 % with the estimates of the kernels before their tables and rotations changed):
+// B200 (SM clock 1.9 GHz; 1 to 64 queries, 1 to 32 sequences of 150 to 65536 tokens, 32/8, 28/4, 16/2, 8/8 and 8/1 heads: 3376
+// calls, up to four kernels each, and the tcgen05 kernel with 1 to 16 ranges in 18 of them), and the shortest estimate wins; over those calls
+// the choice is 0.13 % slower than the best one on average, 20 % at worst (0.5 % and 34 % before the last fit):
 //   * cluster kernel, a unit per (query, kv head, sequence): start and end, then per token of a block and wave;
-//   * persistent kernel, a unit per (query, kv head, sequence) too: start and end, then 215 SM cycles per 16-token tile (256 with
+//   * persistent kernel, a unit per (query, kv head, sequence) too: start and end, then 242 SM cycles per 16-token tile (248 with
 //     more than four heads), more where a block has several units, and the merge of a unit's parts;
-//   * rows kernel, up to 32 rows decoded together: 231 + 58 groups cycles per tile; several queries: start, end and per row the
-//     rotations before and after, which are kernels of their own; one query: 2.8 us per group of four rows inside;
-//   * tcgen05 kernel, up to 256 rows per decoded block, from 32 rows on: 1.09 us per 64-token block of a pair of CTAs; rotating the
-//     queries before and merging and rotating back after grow with the rows and the parts; never below 19.5 us.
+//   * rows kernel, up to 32 rows decoded together: one query 294 + 52 groups cycles per tile and 3.4 us per group of four rows, whose
+//     rotations are inside; several queries 261 + 56 groups, start, end and per row the rotations before and after, which are kernels
+//     of their own;
+//   * tcgen05 kernel, up to 256 rows per decoded block, from 32 rows on: 1.2 us per 64-token block of a pair of CTAs; rotating the
+//     queries before and merging and rotating back after grow with the rows and the parts; never below 19.3 us, and 2.7 us more below
+//     192 rows.
 enum AttentionKernel { kClusterKernel, kPersistentKernel, kRowsKernel, kTensorKernel };
 struct AttentionPlan {
   AttentionKernel kernel, persistent;   // `persistent`: what takes the call if the cluster kernel must not
@@ -779,26 +781,26 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
   auto log_parts = [&](int64_t units) { return std::log2(std::min((double)stages, std::max(1.0, (double)n_sm / units))); };
   double est[4] = {kNever, kNever, kNever, kNever};
   AttentionPlan plan = {kClusterKernel, kClusterKernel, 1};
-  est[kClusterKernel] = g <= 2   ? 8.2 + 0.0136 * load.waves * load.tokens + 6.3 * (load.waves - 1)
-                        : g <= 4 ? 9.5 + 0.0223 * load.waves * load.tokens + 9.0 * (load.waves - 1)
-                                 : 13.5 + 0.0422 * load.waves * load.tokens + 13.4 * (load.waves - 1);
+  est[kClusterKernel] = g <= 2   ? 6.9 + 0.0140 * load.waves * load.tokens + 7.5 * (load.waves - 1)
+                        : g <= 4 ? 9.4 + 0.0223 * load.waves * load.tokens + 7.9 * (load.waves - 1)
+                                 : 14.5 + 0.0408 * load.waves * load.tokens + 13.5 * (load.waves - 1);
   if (kernel_takes(kPersistentKernel, batch, n_q, n_kv_heads, g)) {
     const int64_t units = pairs * n_kv_heads;
     const double full = std::max(0.0, units / (double)n_sm - 1.0);
-    est[kPersistentKernel] = g <= 4 ? 15.3 + units * tiles * 215.0 / sm_hz + 4.2 * more_units(units) + 3.8 * full + 0.5 * log_parts(units) / units
-                                    : 20.0 + units * tiles * 256.0 / sm_hz + 6.0 * more_units(units) + 7.8 * full + 2.8 * log_parts(units) / units;
+    est[kPersistentKernel] = g <= 4 ? 17.0 + units * tiles * 242.0 / sm_hz + 4.0 * more_units(units) + 4.4 * full + 0.7 * log_parts(units) / units
+                                    : 22.0 + units * tiles * 248.0 / sm_hz + 5.1 * more_units(units) + 11.0 * full + 2.75 * log_parts(units) / units;
   }
   if (kernel_takes(kRowsKernel, batch, n_q, n_kv_heads, g)) {
     const RowCut cut = cut_rows(rows);
     const int64_t units = batch * n_kv_heads * cut.blocks;
     if (n_q == 1) {
       const int groups = (cut.rows + 3) / 4;
-      est[kRowsKernel] = 18.2 + units * tiles * (278.0 + 50.0 * groups) / sm_hz + groups * (2.8 + 1.4 * more_units(units) + 0.9 * log_parts(units) / units);
+      est[kRowsKernel] = 19.1 + units * tiles * (294.0 + 52.0 * groups) / sm_hz + groups * (3.4 + 1.5 * more_units(units) + 0.94 * log_parts(units) / units);
     } else {
       const int groups = rows_groups(cut.rows);
       const double full = std::max(0.0, units / (double)n_sm - 1.0), all_rows = (double)pairs * n_kv_heads * g;
-      est[kRowsKernel] = 13.7 + units * tiles * (231.0 + 58.5 * groups) / sm_hz + groups * (0.7 + 0.28 * more_units(units)) + 3.7 * log_parts(units) / units -
-                         1.3 * full + 3.6e-3 * all_rows + 2.9e-3 * std::min(all_rows, 2368.0);
+      est[kRowsKernel] = 13.7 + units * tiles * (261.0 + 56.3 * groups) / sm_hz + groups * (0.71 + 0.24 * more_units(units)) + 3.2 * log_parts(units) / units -
+                         1.3 * full + 3.66e-3 * all_rows + 3.33e-3 * std::min(all_rows, 2368.0);
     }
   }
   if (tensor) {
@@ -808,13 +810,14 @@ static AttentionPlan plan_attention(int64_t batch, int n_q, int n_kv_heads, int 
     for (int s = 1; s <= kMaxSplits && s <= blocks && (s == 1 || (s <= room && batch * s <= 65535)); ++s) {
       const int64_t clusters = (q_blocks + 1) / 2 * n_kv_heads * batch * s, at_once = n_sm / 2;   // two query blocks each
       const double waves = (double)((clusters + at_once - 1) / at_once), work = waves * ((blocks + s - 1) / s);
-      const double t = std::max(19.5, 15.1 + 1.086 * work + 0.72 * std::min(work, 4.0) + 8.8 * (waves - 1.0) +
-                                          2.3e-3 * std::min<int64_t>(all_rows, 2368) + 1.98e-3 * all_rows + 0.08e-3 * s * all_rows);
+      const double t = 13.9 + 1.2 * work + 0.79 * std::min(work, 4.0) + 10.2 * (waves - 1.0) + 2.7e-3 * std::min<int64_t>(all_rows, 2368) +
+                       1.3e-3 * all_rows + 0.165e-3 * s * all_rows;
       if (t < est[kTensorKernel]) {
         est[kTensorKernel] = t;
         plan.n_splits = s;
       }
     }
+    est[kTensorKernel] = std::max(19.3, est[kTensorKernel]) + (all_rows < 192 ? 2.7 : 0.0);
   }
   for (AttentionKernel k : {kPersistentKernel, kRowsKernel, kTensorKernel})
     if (est[k] < est[plan.kernel]) plan.kernel = k;
