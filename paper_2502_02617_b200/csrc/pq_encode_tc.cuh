@@ -51,7 +51,7 @@ constexpr int kTcSmFix = kTcSmMisc + 64;                     // one TcFixQueue p
 constexpr int kTcFixBytes = kTcGroups * (int)sizeof(TcFixQueue) > 4 * PQ_HIST_MAX_BINS * 4 ? kTcGroups * (int)sizeof(TcFixQueue) : 4 * PQ_HIST_MAX_BINS * 4;
 constexpr int kTcSmL1 = kTcSmFix + kTcFixBytes;              // copy of Tables::l1_cells (codebooks other than the analytic ones)
 constexpr int kTcSmTotal = kTcSmL1 + 8 * kL1Cells * 8 + 1024;             // + slack for 1024-byte alignment
-static_assert(kTcTerms == 3, "kRotErrTc is the bound for three terms");
+static_assert(kTcTerms == 3, "kRotErrTc counts on three terms");
 static_assert(sizeof(TcFixQueue) % 16 == 0, "queues are laid out back to back");
 static_assert(kTcSmTotal <= 227 * 1024, "shared memory of one CTA");
 static_assert(8 * (kTcStages + 2 * kTcAccs) <= 128, "barriers");
@@ -223,8 +223,9 @@ encode_tc_kernel(EncodeArgs a, const __grid_constant__ TcMaps maps, int n_row_ti
 #pragma unroll
         for (int q = 0; q < 8 * kTcTerms; ++q) {
           const uint32_t off = ((q >> 2) & 1) * 16384 + (q & 3) * 32;  // k-half, k-step inside the 128-byte swizzled row
-          tc_mma(tmem_u + acc * 128, desc_hi | (adesc_lo + (off >> 4)), desc_hi | (bdesc_lo + (((q >> 3) * kTcSBytes + off) >> 4)),
-                 q ? 1u : 0u);
+          // the smallest term of S first: see kRotErrTc
+          tc_mma(tmem_u + acc * 128, desc_hi | (adesc_lo + (off >> 4)),
+                 desc_hi | (bdesc_lo + (((kTcTerms - 1 - (q >> 3)) * kTcSBytes + off) >> 4)), q ? 1u : 0u);
         }
         tc_commit(bar_acc + 8 * acc);  // the accumulator is complete and the x stage has been read
       }

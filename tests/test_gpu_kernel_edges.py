@@ -231,6 +231,20 @@ def test_encoders_on_both_sides_of_the_few_rows_kernel(dtype, per_sm, Hkv):
         assert torch.all((radii.float() - radii_cut[:, :, :, :n].float()).abs() <= 2.0 ** -10 * radii.float())
 
 
+# The tensor-core encoder's radii are float32 sums rounded to fp16.  An error of e row norms, sqrt(8) radii, brings e sqrt(8) 2^11 of them
+# across a boundary: with the smallest term of S multiplied first e is 0.2 * 2^-24 on average, 0.013 % of the radii are neighbours of
+# the exact norm's rounding; with the largest first 0.089 %.
+def test_radii_of_the_tensor_core_encoder():
+    n, Hkv = 4096, 8
+    K, V = synthetic.kv_like(5, n, Hkv, 128, torch.bfloat16, DEV)
+    c = pq.PolarQuantCache(1, Hkv, Hkv, 128, capacity=n, seed=0, device=DEV)
+    c.encode(K, V, torch.tensor([0, n], dtype=torch.int32, device=DEV))
+    radii = c.unpack(n)[1][0]                                   # [head, K | V, token, block]
+    want = torch.stack([(X.double() @ c.S_host.double().to(DEV)).view(n, Hkv, 8, 16).norm(dim=-1).half() for X in (K, V)], dim=2).permute(1, 2, 0, 3)
+    assert (radii != want).double().mean() < 3e-4
+    assert torch.all((radii.float() - want.float()).abs() <= 2.0 ** -10 * want.float())
+
+
 # What is stored for a row with a non-finite input does not depend on which kernel takes the call: bf16 calls of 128 tokens and more are the
 # tensor-core encoder's or, up to four vectors per SM, the few-rows kernel's, and store the zero vector; tiles of 128 rows (float32, or
 # bf16 rows that are not aligned, above 128 vectors per SM) store what the arithmetic gives, as fewer tokens do.  The other rows are the
