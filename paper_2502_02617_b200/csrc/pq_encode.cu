@@ -520,7 +520,10 @@ int32_t pq_angle_histograms(int32_t head_dim, int32_t n_kv_heads, const float* S
   const int per = 128 / head_dim;
   const int64_t n_vec = (int64_t)total_tokens * 2 * n_kv_heads;
   const int64_t want = (n_vec + per - 1) / per;
-  const int grid = (int)(want < 148 * 8 ? want : 148 * 8);
+  static pq::DeviceMemo sm_count;
+  const int n_sm = pq::sm_count_of_device(sm_count);
+  if (n_sm == 0) return PQ_ERR_CUDA;
+  const int grid = (int)(want < n_sm * 8 ? want : n_sm * 8);
   pq::hist_simple_kernel<<<grid, pq::kHistSimpleThreads, (size_t)4 * n_bins * sizeof(uint32_t), s>>>(a, n_vec, per);
   return pq::launch_status();
 }

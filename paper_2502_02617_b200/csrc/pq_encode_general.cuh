@@ -19,10 +19,10 @@
 // roundings of radii (squares, sums, square root: below 6e-7), table entries and the test itself.
 // A radius is certified by radius_unsure, with the bound of rotation_block_error: 1.4 to 5 % of them are not, according to the slices
 // of S and the blocks of a vector.
-// Bound by the latency of its phases and of the float64 re-decisions (13 of a block's 47 us before the product moved to tensor cores, of
-// which the product on the FMA pipe was 18).  Measured (8 heads; a block per vector in float64 before): 512 tokens, seven
-// levels of three bits 89.7 -> 43.4 us; packed cache, 2048 tokens at head_dim 64 67 -> 40 us.  Product on tensor cores: 8 x 512 tokens,
-// seven levels of three bits, and an attention over 8 x 4096 of 95 us 312 -> 273 us.
+// Bound by the latency of its phases and of the float64 re-decisions, the barriers around them and the fetch of code that a block walks
+// through once.  Measured (8 heads; a block per vector in float64 before): 512 tokens, seven levels of three bits 89.7 -> 43.4 us;
+// packed cache, 2048 tokens at head_dim 64 67 -> 40 us.  Product on tensor cores instead of the FMA pipe: 8 x 512 tokens, seven levels
+// of three bits 206.9 -> 158.9 us.
 #pragma once
 #include <math_constants.h>
 
@@ -760,8 +760,11 @@ static int32_t launch_gen_encode(const GenEncodeArgs& a, cudaStream_t stream) {
   const int64_t n_vec = (int64_t)a.total_tokens * 2 * a.n_kv_heads;
   if (!a.packed && n_vec <= (a.g.d > 128 ? 2048 : a.g.d > 64 ? 3072 : 4096))
     return launch_gen_kernel(gen_encode_vector_kernel, dim3((unsigned)n_vec), a.g.d < 32 ? 32 : a.g.d, 0, a, stream);
+  static DeviceMemo sm_count;
+  const int n_sm = sm_count_of_device(sm_count);
+  if (n_sm == 0) return PQ_ERR_CUDA;
   const GeShape s1 = ge_shape(a.g.d, a.g.row_bytes, 1);
-  const bool few = (int64_t)((a.total_tokens + s1.vecs - 1) / s1.vecs) * 2 * a.n_kv_heads <= 2 * 148;
+  const bool few = (int64_t)((a.total_tokens + s1.vecs - 1) / s1.vecs) * 2 * a.n_kv_heads <= 2 * n_sm;
   switch (a.g.L < 4 ? a.g.L : 4) {
     case 1: return few ? launch_gen_encode_as<1, 1>(a, stream) : launch_gen_encode_as<4, 1>(a, stream);
     case 2: return few ? launch_gen_encode_as<1, 2>(a, stream) : launch_gen_encode_as<4, 2>(a, stream);

@@ -19,9 +19,9 @@ constexpr int kRowMax = 32;                                // rows of a row bloc
 constexpr int kRowSmQ = kSmSegs + 768;                     // q' fragments [row group][k-step][lane], 8 bytes
 constexpr int kRowSmRing = (kRowSmQ + 8 * 8 * 32 * 8 + 127) / 128 * 128;
 // S, rows 528 bytes apart (a thread per row reads it without bank conflicts), lies where the ring is: before the first copies
-// of a segment for the rotation of the queries, and after the merge for the last part's un-rotation; behind it 16 rows of q in
-// float32.  Both products are rolled loops over shared memory: straight-line code that runs once per segment takes longer
-// to fetch (5.7 us for 16 rows) than to run.
+// of a segment for the rotation of the query, and after the merge for the last part's un-rotation; behind it its heads' rows in float32
+// (one query per sequence; several are rotated by kernels of their own).  Both products are rolled loops over shared memory:
+// straight-line code that runs once per segment takes longer to fetch than to run.
 constexpr int kRowSStride = 132, kRowQIn = 128 * kRowSStride * 4;
 constexpr int kRowMergeMl = kRowWarps * 16 * kMrgStride * 4;   // in the merge buffer, behind 16 rows of every warp: (m, l)
 constexpr int kRowMergeBytes = kRowMergeMl + kRowWarps * kRowMax * 8;
