@@ -256,6 +256,31 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
+// A 16 x 16 tile of 16-bit elements as mma.sync fragments: lane l gives the address of row l & 15, 8-column half l >> 4.
+template <bool kTrans>
+__device__ __forceinline__ void ldmatrix_x4(uint32_t at, uint32_t (&v)[4]) {
+  if (kTrans)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
+}
+__device__ __forceinline__ void mma_bf16_16816(float* d, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Three bf16 terms of a pair of float32 values (round to nearest each; a float32 value is their sum exactly), a in the low half.
+__device__ __forceinline__ void bf16_terms(float a, float b, uint32_t* t) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat162 w = __floats2bfloat162_rn(a, b);
+    t[i] = *reinterpret_cast<const uint32_t*>(&w);
+    a -= __uint_as_float(t[i] << 16);
+    b -= __uint_as_float(t[i] & 0xFFFF0000u);
+  }
+}
+
 // Host side: remember the CUDA error behind a PQ_ERR_CUDA return (see pq_last_cuda_error).
 void note_cuda_error(cudaError_t e);
 // Test hook (pq_debug_fail_next_wait): returns true once after the hook was armed for `which`

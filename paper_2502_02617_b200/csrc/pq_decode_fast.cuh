@@ -786,8 +786,8 @@ __global__ void __launch_bounds__(kFastThreads, 1) decode_attention_fast_kernel(
     };
     // Where a paged segment's stages begin is listed in shared memory, kFsPlaceCap of them at a time and the first ones before the second
     // copy is requested (a barrier of the rotation below lies between), so that the copying thread, whose warp has a tile of its own to
-    // work on, needs no division and waits for no table.  Looked up per stage they cost the whole kernel a tenth: 8 x 32768 tokens,
-    // 32/8 heads, pages of 256 131.9 us against 122.6 (contiguous 119.4); 16 x 20000 160.6 -> 148.0, 28/4 heads 88.1 -> 84.5.  Looked up
+    // work on, needs no division and waits for no table.  Looked up per stage they cost the whole kernel a tenth (before the keys' level-1
+    // residuals were back): 8 x 32768 tokens, 32/8 heads, pages of 256 131.9 us against 122.6 (contiguous 119.4; now 132.6 and 129.3); 16 x 20000 160.6 -> 148.0, 28/4 heads 88.1 -> 84.5.  Looked up
     // inside the loop for stages beyond a longer list, the unused branch alone took 125.2: a list is made again instead.
     auto list_places = [&](int first) {
       for (int i = tid; i < min(kFsPlaceCap, st1 - st0 - first); i += kFastThreads)

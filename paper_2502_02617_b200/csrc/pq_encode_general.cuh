@@ -178,31 +178,6 @@ __host__ __device__ constexpr float ge_mma_block_error(int dc) {
   return 1.02f * (10.1f * const_sqrt(ge_mma_steps(dc)) + ge_mma_steps(dc)) * 5.9604644775390625e-08f;
 }
 
-// Three bf16 terms of a pair of float32 values (round to nearest each: together within 2^-26 of the values).
-__device__ __forceinline__ void ge_split(float a, float b, uint32_t* t) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const __nv_bfloat162 w = __floats2bfloat162_rn(a, b);
-    t[i] = *reinterpret_cast<const uint32_t*>(&w);
-    a -= __uint_as_float(t[i] << 16);
-    b -= __uint_as_float(t[i] & 0xFFFF0000u);
-  }
-}
-template <bool kTrans>
-__device__ __forceinline__ void ge_ldmatrix(const __nv_bfloat16* row, uint32_t (&v)[4]) {
-  const uint32_t at = (uint32_t)__cvta_generic_to_shared(row);
-  if (kTrans)
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
-  else
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
-}
-__device__ __forceinline__ void ge_mma(float* d, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // y = x S of a tile of V bf16 vectors (xh [V][dc + 8]) on tensor cores, into y [V][dc / 16][20] over the same memory.  S goes through
 // shared memory in slices of 32 rows, split into three bf16 terms as it arrives; a warp owns eight 16 x 8 tiles of y, smallest terms
 // first, a fresh accumulator per k-step (see the bounds).
@@ -232,8 +207,8 @@ __device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, in
       if (aligned) v = __ldg(reinterpret_cast<const float4*>(src));
       else v = make_float4(__ldg(src), __ldg(src + 1), __ldg(src + 2), __ldg(src + 3));
       uint32_t lo[3], hi[3];
-      ge_split(v.x, v.y, lo);
-      ge_split(v.z, v.w, hi);
+      bf16_terms(v.x, v.y, lo);
+      bf16_terms(v.z, v.w, hi);
 #pragma unroll
       for (int t = 0; t < 3; ++t)
         *reinterpret_cast<uint2*>(Sw + ((t * kGeSlice + k) * stride + n) / 2) = make_uint2(lo[t], hi[t]);
@@ -245,14 +220,14 @@ __device__ __forceinline__ void ge_product_mma(const GenEncodeArgs& a, int V, in
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
         const int m = m0 + p / pairs, n = n0 + (p % pairs) * 16;
-        if (p % pairs == 0) ge_ldmatrix<false>(xh + (m * 16 + lr) * stride + k0 + ks + lc, A);
+        if (p % pairs == 0) ldmatrix_x4<false>((uint32_t)__cvta_generic_to_shared(xh + (m * 16 + lr) * stride + k0 + ks + lc), A);
         float acc[2][4] = {};
 #pragma unroll
         for (int t = 2; t >= 0; --t) {
           uint32_t B[4];
-          ge_ldmatrix<true>(reinterpret_cast<const __nv_bfloat16*>(Sw) + (t * kGeSlice + ks + lr) * stride + n + lc, B);
-          ge_mma(acc[0], A, B[0], B[1]);
-          ge_mma(acc[1], A, B[2], B[3]);
+          ldmatrix_x4<true>((uint32_t)__cvta_generic_to_shared(reinterpret_cast<const __nv_bfloat16*>(Sw) + (t * kGeSlice + ks + lr) * stride + n + lc), B);
+          mma_bf16_16816(acc[0], A, B[0], B[1]);
+          mma_bf16_16816(acc[1], A, B[2], B[3]);
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {

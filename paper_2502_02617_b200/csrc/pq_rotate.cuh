@@ -141,6 +141,19 @@ __global__ void __launch_bounds__(kRotThreads) rotate_rows_kernel(const float* S
   }
 }
 
+// S^T in shared memory.
+__device__ __forceinline__ void load_transposed(const float* S, float* s, int tid) {
+#pragma unroll 4
+  for (int i = tid; i < 128 * 32; i += kRotThreads) {
+    const int n = i & 127, k = 4 * (i >> 7);   // neighbouring threads write neighbouring columns
+    const float4 v = __ldg(reinterpret_cast<const float4*>(S + n * 128 + k));
+    s[k * kRotSStride + n] = v.x;
+    s[(k + 1) * kRotSStride + n] = v.y;
+    s[(k + 2) * kRotSStride + n] = v.z;
+    s[(k + 3) * kRotSStride + n] = v.w;
+  }
+}
+
 // The tile (x) times S^T (s), to the rows from row0 on of out.
 template <int kTile>
 __device__ __forceinline__ void store_unrotated(const float* x, const float* s, int64_t row0, int64_t n_rows, int lane, int warp, void* out,
@@ -179,15 +192,7 @@ __global__ void __launch_bounds__(kRotThreads) merge_unrotate_kernel(const float
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * kTile;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-#pragma unroll 4
-  for (int i = tid; i < 128 * 32; i += kRotThreads) {
-    const int n = i & 127, k = 4 * (i >> 7);   // neighbouring threads write neighbouring columns
-    const float4 v = __ldg(reinterpret_cast<const float4*>(S + n * 128 + k));
-    s[k * kRotSStride + n] = v.x;
-    s[(k + 1) * kRotSStride + n] = v.y;
-    s[(k + 2) * kRotSStride + n] = v.z;
-    s[(k + 3) * kRotSStride + n] = v.w;
-  }
+  load_transposed(S, s, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the parts come from the kernel before this one
 #pragma unroll 2
   for (int i = tid; i < kTile * 32; i += kRotThreads) {   // a warp per row
@@ -234,15 +239,7 @@ __global__ void __launch_bounds__(kRotThreads) merge_rows_kernel(const float* S,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row0 = blockIdx.x * kTile, n_rows = a.batch * a.n_q_heads, g = a.n_q_heads / a.n_kv_heads, R = a.rows_per_block;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-#pragma unroll 4
-  for (int i = tid; i < 128 * 32; i += kRotThreads) {
-    const int n = i & 127, k = 4 * (i >> 7);   // neighbouring threads write neighbouring columns
-    const float4 v = __ldg(reinterpret_cast<const float4*>(S + n * 128 + k));
-    s[k * kRotSStride + n] = v.x;
-    s[(k + 1) * kRotSStride + n] = v.y;
-    s[(k + 2) * kRotSStride + n] = v.z;
-    s[(k + 3) * kRotSStride + n] = v.w;
-  }
+  load_transposed(S, s, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the parts come from the kernel before this one
 #pragma unroll 2
   for (int i = tid; i < kTile * 32; i += kRotThreads) {   // a warp per row

@@ -24,30 +24,11 @@ constexpr int kTmSmRing = kTmSmMl + kTmWarps * 4 * 8;         // the pieces; the
 constexpr int kTmSmTotal = kTmSmRing + kTmWarps * kTmRing * kTmPiece;
 static_assert(kTmSmRing % 128 == 0 && kTmWarps * 4 * 128 * 4 <= kTmWarps * kTmRing * kTmPiece, "map");
 
-__device__ __forceinline__ void tm_ldmatrix(uint32_t at, uint32_t (&v)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
-}
-__device__ __forceinline__ void tm_ldmatrix_trans(uint32_t at, uint32_t (&v)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
-}
-__device__ __forceinline__ void tm_mma(float* d, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 // Term t of the pair (a, b) as bf16, a in the low half.
 __device__ __forceinline__ uint32_t tm_term(float a, float b, int t) {
-  uint32_t w = 0u;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(&h);
-    if (i == t) w = v;
-    a -= __uint_as_float(v << 16);
-    b -= __uint_as_float(v & 0xFFFF0000u);
-  }
-  return w;
+  uint32_t w[3];
+  bf16_terms(a, b, w);
+  return t == 0 ? w[0] : t == 1 ? w[1] : w[2];
 }
 
 __device__ __noinline__ void tail_attention_again(const TailArgs& a, float* sm) { tail_attention<1>(a, sm); }
@@ -115,10 +96,10 @@ __global__ void __launch_bounds__(kTailThreads, 4) tail_mma_kernel(const __grid_
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         uint32_t k4[4];
-        tm_ldmatrix(at + (((2 * ks + (lane >> 4)) ^ (frag_row & 7)) << 4), k4);
+        ldmatrix_x4<false>(at + (((2 * ks + (lane >> 4)) ^ (frag_row & 7)) << 4), k4);
         const uint4 q = *reinterpret_cast<const uint4*>(tm_smem + kTmSmQ + (ks * 32 + lane) * 16);
-        tm_mma(s1, k4, q.z, q.w);
-        tm_mma(s0, k4, q.x, q.y);
+        mma_bf16_16816(s1, k4, q.z, q.w);
+        mma_bf16_16816(s0, k4, q.x, q.y);
       }
     }
     __syncwarp();
@@ -154,9 +135,9 @@ __global__ void __launch_bounds__(kTailThreads, 4) tail_mma_kernel(const __grid_
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         uint32_t v4[4];
-        tm_ldmatrix_trans(at + (((2 * j + (lane >> 4)) ^ (frag_row & 7)) << 4), v4);
-        tm_mma(o[2 * j], pa, v4[0], v4[1]);
-        tm_mma(o[2 * j + 1], pa, v4[2], v4[3]);
+        ldmatrix_x4<true>(at + (((2 * j + (lane >> 4)) ^ (frag_row & 7)) << 4), v4);
+        mma_bf16_16816(o[2 * j], pa, v4[0], v4[1]);
+        mma_bf16_16816(o[2 * j + 1], pa, v4[2], v4[3]);
       }
     }
     __syncwarp();
